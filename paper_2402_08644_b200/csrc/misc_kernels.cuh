@@ -23,7 +23,7 @@ struct LoopState {
                        // [7] sequences still drafting (adaptive block length), [8] router launches since the prompt pass,
                        // [9] CTAs of the running router launch that have finished
     volatile int* host_flags;   // mapped pinned host memory: [0] ticket, [1] live, [2] n_max, [3] n_sum, [4] iterations,
-                                // [5] router ticket, [6] sequences still drafting
+                                // [5] router ticket, [6] sequences still drafting, [7] most tokens any live sequence still wants
     int* block_len;    // [B] adaptive block length: drafts made in the current iteration
     int* drafting;     // [B] adaptive block length: 1 while the router lets the sequence go on drafting
     float* confidence; // [B][gamma_limit] the router's 1 - s for every draft of the current iteration
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restric
     }
 }
 
-// Verify / accept / rollback (Section 3.1), one thread per sequence, one CTA.
+// Verify / accept / rollback (Section 3.1), one warp per sequence, one CTA.
 //   a = longest prefix of drafts equal to the large model's tokens (or forced);
 //   the sequence gains d_1..d_a and g_{a+1}; n advances; g_{a+1} becomes pending.
 // Rolling the caches back is the update of n: positions >= n-1 are rewritten by the next iteration.
@@ -280,74 +280,96 @@ __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restric
 // mode 4 is sampled SPEED: sample_verify_kernel has already written each sequence's accept length and, at that index
 // of its targets, the token drawn after the kept drafts; this kernel only does the bookkeeping.
 // block_len (nullable): per-sequence number of drafts of this iteration when the router chose it.
-// block: 256.
-__global__ void __launch_bounds__(256) verify_kernel(LoopState st, int batch, int gamma, int mode, unsigned long long seed,
+// A lone CTA at the end of the iteration's chain, bound by the latency of dependent loads: 32 warps finish up to 32
+// arg-max rows side by side, a sequence's drafts and targets are fetched by the lanes of its warp in one round trip, and
+// the totals for the host are summed in shared memory.
+// block: VERIFY_THREADS; batch * (gamma + 1) <= 256.
+constexpr int VERIFY_THREADS = 1024;
+__global__ void __launch_bounds__(VERIFY_THREADS) verify_kernel(LoopState st, int batch, int gamma, int mode, unsigned long long seed,
                                                      int max_new, const float* amax_val, const int* amax_idx, int amax_stride,
                                                      int n_tiles, const float* fin_val, const int* fin_idx, const int* block_len) {
+    __shared__ int s_tok[256];                     // the large model's token per block row (mode 3: the last draft per sequence)
+    __shared__ int s_live, s_nmax, s_nsum, s_left;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int WARPS = VERIFY_THREADS / 32;
+    if (threadIdx.x == 0) { s_live = 0; s_nmax = 0; s_nsum = 0; s_left = 0; }
     pdl_wait();
     pdl_launch_dependents();
-    if (mode == 3) {
-        if (fin_val != nullptr && gamma > 0) {
-            for (int b = threadIdx.x >> 5; b < batch; b += 8) {
-                const int tok = argmax_from_tiles(fin_val + (size_t)b * amax_stride, fin_idx + (size_t)b * amax_stride, n_tiles);
-                if ((threadIdx.x & 31) == 0) st.drafts[b * st.gamma_limit + gamma - 1] = tok;
-            }
-        }
-        __syncthreads();
-    } else if (amax_val != nullptr && mode != 4) {   // (mode 4: the sampled decisions are already in place)
-        const int rows = batch * (gamma + 1);
-        for (int m = threadIdx.x >> 5; m < rows; m += 8) {
-            const int tok = argmax_from_tiles(amax_val + (size_t)m * amax_stride, amax_idx + (size_t)m * amax_stride, n_tiles);
-            if ((threadIdx.x & 31) == 0) st.targets[(m / (gamma + 1)) * (st.gamma_limit + 1) + m % (gamma + 1)] = tok;
-        }
-        __syncthreads();
+    const bool finish_last = mode == 3 && fin_val != nullptr && gamma > 0;
+    const bool finish_rows = mode != 3 && mode != 4 && amax_val != nullptr;   // (mode 4: the sampled decisions are already in place)
+    const int rows = finish_last ? batch : (finish_rows ? batch * (gamma + 1) : 0);
+    const float* val = finish_last ? fin_val : amax_val;
+    const int* idx = finish_last ? fin_idx : amax_idx;
+    for (int m = warp; m < rows; m += WARPS) {
+        const int tok = argmax_from_tiles(val + (size_t)m * amax_stride, idx + (size_t)m * amax_stride, n_tiles);
+        if (lane == 0) s_tok[m] = tok;
     }
-    const int b = threadIdx.x;
+    __syncthreads();
     const int iteration = st.counters[0];
     const int live_before = st.counters[1];
-    __syncthreads();
-    if (b < batch && !st.done[b]) {
-        const int* d = st.drafts + b * st.gamma_limit;
-        const int* g = st.targets + b * (st.gamma_limit + 1);
-        int a = 0;
-        if (mode == 1 || mode == 3) a = gamma;
-        else if (mode == 4) a = min(max(st.accept_len[b], 0), gamma);   // sampled SPEED: decided by sample_verify_kernel, with g[a] the token it drew
-        else if (mode == 2) a = (int)(splitmix64(splitmix64(splitmix64(seed) ^ (unsigned long long)b) ^ (unsigned long long)iteration) % (unsigned long long)(gamma + 1));
-        else {   // adaptive block length: only the drafts the sequence really made count (later rows are dead)
-            const int gamma_b = block_len ? min(block_len[b], gamma) : gamma;
-            while (a < gamma_b && d[a] == g[a]) ++a;
+    for (int b = warp; b < batch; b += WARPS) {
+        int* dp = st.drafts + b * st.gamma_limit;
+        int* gp = st.targets + b * (st.gamma_limit + 1);
+        // lane i: draft d_{i+1} and target g_{i+1}, as far as the block goes
+        int d = lane < gamma ? __ldcg(dp + lane) : -1;
+        if (finish_last && lane == gamma - 1) { d = s_tok[b]; dp[lane] = d; }
+        int g = -1;
+        if (lane <= gamma && mode != 3) {
+            if (finish_rows) { g = s_tok[b * (gamma + 1) + lane]; gp[lane] = g; }
+            else g = __ldcg(gp + lane);
         }
-        st.accept_len[b] = a;
-        atomicAdd(st.hist + a, 1ull);
-        const int em = st.emitted[b];
-        const int room = max_new - em;
-        const int take = min(mode == 3 ? a : a + 1, room);
-        int last = st.pending[b];
-        for (int i = 0; i < take; ++i) {
-            last = (i < a) ? d[i] : g[a];
-            if (em + i < st.out_cap) st.out_ids[(size_t)b * st.out_cap + em + i] = last;
+        const int done = st.done[b], em = st.emitted[b], n = st.n[b], pending = st.pending[b];
+        const int gamma_b = block_len ? min(block_len[b], gamma) : gamma;
+        const int sampled_a = mode == 4 ? st.accept_len[b] : 0;
+        int n_new = n, left = 0, live = 0;
+        if (!done) {
+            int a;
+            if (mode == 1 || mode == 3) a = gamma;
+            else if (mode == 4) a = min(max(sampled_a, 0), gamma);   // sampled SPEED: decided by sample_verify_kernel, with g[a] the token it drew
+            else if (mode == 2) a = (int)(splitmix64(splitmix64(splitmix64(seed) ^ (unsigned long long)b) ^ (unsigned long long)iteration) % (unsigned long long)(gamma + 1));
+            else a = __ffs(~__ballot_sync(0xffffffffu, lane < gamma_b && d == g)) - 1;   // adaptive block length: only the drafts really made count
+            const int bonus = __shfl_sync(0xffffffffu, g, a);
+            const int take = min(mode == 3 ? a : a + 1, max_new - em);
+            const int tok = lane < a ? d : bonus;          // the block's token number lane + 1
+            if (lane < take && em + lane < st.out_cap) st.out_ids[(size_t)b * st.out_cap + em + lane] = tok;
+            const int last = __shfl_sync(0xffffffffu, tok, max(take - 1, 0));
+            n_new = n + take;
+            live = em + take < max_new;
+            left = max_new - em - take;
+            if (lane == 0) {
+                st.accept_len[b] = a;
+                atomicAdd(st.hist + a, 1ull);
+                st.emitted[b] = em + take;
+                st.n[b] = n_new;
+                st.pending[b] = take > 0 ? last : pending;
+                if (!live) st.done[b] = 1;
+            }
         }
-        st.emitted[b] = em + take;
-        st.n[b] += take;
-        st.pending[b] = last;
-        if (em + take >= max_new) { st.done[b] = 1; atomicSub(st.counters + 1, 1); }
+        if (lane == 0) {
+            atomicAdd(&s_live, live);
+            atomicMax(&s_nmax, n_new);
+            atomicAdd(&s_nsum, n_new);
+            atomicMax(&s_left, left);
+        }
     }
     __syncthreads();
-    if (b == 0) {
-        if (live_before > 0) { st.counters[0] = iteration + 1; st.counters[5] += 1; }
-        int n_max = 0, n_sum = 0;
-        for (int i = 0; i < batch; ++i) { n_max = max(n_max, st.n[i]); n_sum += st.n[i]; }
-        st.counters[3] = n_max;
-        st.counters[4] = n_sum;
+    if (threadIdx.x == 0) {
+        const int iters = st.counters[5] + (live_before > 0 ? 1 : 0);
         const int ticket = st.counters[6] + 1;
-        st.counters[6] = ticket;
         // publish to the host: data first, then the ticket it polls on
-        st.host_flags[1] = st.counters[1];
-        st.host_flags[2] = n_max;
-        st.host_flags[3] = n_sum;
-        st.host_flags[4] = st.counters[5];
+        st.host_flags[1] = s_live;
+        st.host_flags[2] = s_nmax;
+        st.host_flags[3] = s_nsum;
+        st.host_flags[4] = iters;
+        st.host_flags[7] = s_left;
         __threadfence_system();
         st.host_flags[0] = ticket;
+        if (live_before > 0) st.counters[0] = iteration + 1;
+        st.counters[1] = s_live;
+        st.counters[3] = s_nmax;
+        st.counters[4] = s_nsum;
+        st.counters[5] = iters;
+        st.counters[6] = ticket;
     }
 }
 

@@ -213,8 +213,9 @@ Layout make_layout(const tandem_config& c) {
     L.kv_large = take((size_t)c.large.n_layers * 2 * L.kv_large_layer * esz);
     L.kv_small = take((size_t)c.small.n_layers * 2 * L.kv_small_layer * esz);
     L.st_n = take(B * 4); L.st_pending = take(B * 4); L.st_drafts = take(B * GL * 4);
-    L.st_targets = take(B * (GL + 1) * 4); L.st_accept = take(B * 4); L.st_emitted = take(B * 4);
-    L.st_done = take(B * 4); L.st_out = take(B * T * 4); L.st_counters = take(16 * 4); L.st_hist = take((GL + 1) * 8);
+    L.st_targets = take(B * (GL + 1) * 4); L.st_accept = take(B * 4);
+    L.st_done = take(B * 4); L.st_out = take(B * T * 4);
+    L.st_counters = take(16 * 4); L.st_hist = take((GL + 1) * 8); L.st_emitted = take(B * 4);   // adjacent: read back together
     L.st_block_len = take(B * 4); L.st_drafting = take(B * 4); L.st_confidence = take(B * GL * 4);
     L.row_tok = take(R * 4); L.row_seq = take(R * 4); L.row_pos = take(R * 4);
     L.grp_row0 = take((size_t)L.max_groups * 4); L.grp_cnt = take((size_t)L.max_groups * 4);
@@ -806,7 +807,7 @@ void launch_score_rows(tandem_ctx& c, int gamma) {
 
 void launch_verify(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new, bool from_tiles, bool adaptive = false) {
     ProfScope ps(c, PC_VERIFY, (double)c.batch * (2 * gamma + 8) * 4.0);
-    launch_ex(c, true, 1, verify_kernel, dim3(1), dim3(256), 0, c.st, c.batch, gamma, mode, (unsigned long long)seed, max_new,
+    launch_ex(c, true, 1, verify_kernel, dim3(1), dim3(VERIFY_THREADS), 0, c.st, c.batch, gamma, mode, (unsigned long long)seed, max_new,
               from_tiles ? (const float*)at<float>(c, c.lay.amax_val_large) : (const float*)nullptr,
               from_tiles ? (const int*)at<int>(c, c.lay.amax_idx_large) : (const int*)nullptr, c.lay.vocab_tiles, c.lay.vocab_tiles,
               from_tiles ? (const float*)at<float>(c, c.lay.amax_val_small) : (const float*)nullptr,
@@ -1206,9 +1207,11 @@ tandem_status begin_call(tandem_ctx* c) {
     return TANDEM_OK;
 }
 
-__global__ void reset_call_kernel(LoopState st, int batch) {
+// Start of a generate or step call: nobody has emitted anything; a generate call also clears the histogram.  block: 256.
+__global__ void reset_call_kernel(LoopState st, int batch, bool clear_hist) {
     const int b = threadIdx.x;
     if (b < batch) { st.emitted[b] = 0; st.done[b] = 0; }
+    if (clear_hist && b <= st.gamma_limit) st.hist[b] = 0ull;
     if (b == 0) { st.counters[1] = batch; st.counters[5] = 0; }
 }
 
@@ -1279,7 +1282,8 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->small.d = cfg->small; c->small.wbase = 5 + 10 * cfg->large.n_layers; c->small.kv_off = lay.kv_small; c->small.kv_layer_elems = lay.kv_small_layer;
     c->tbase = c->small.wbase + 5 + 10 * cfg->small.n_layers;
     c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0;
-    c->pinned_ints = (size_t)3 * lay.max_rows + 2 * lay.max_groups + 4 * cfg->max_batch + 64;
+    c->pinned_ints = std::max((size_t)3 * lay.max_rows + 2 * lay.max_groups + 4 * cfg->max_batch + 64,
+                              (size_t)cfg->max_batch * (cfg->max_seq + 1) + 2 * 64 + 64);   // prompt rows going in; tokens, counters, histogram, lengths coming out
     c->pinned = nullptr;
     LoopState& st = c->st;
     st.n = at<int>(*c, lay.st_n); st.pending = at<int>(*c, lay.st_pending); st.drafts = at<int>(*c, lay.st_drafts);
@@ -1529,7 +1533,7 @@ extern "C" tandem_status tandem_block_step(tandem_ctx* c, int32_t gamma, int32_t
     if (accept_mode == TANDEM_ACCEPT_REPRESENTATION_ONLY && gamma < 1) return TANDEM_ERR_INVALID_ARG;
     if (c->batch == 0) return TANDEM_ERR_STATE;
     TRY(capacity_for(c, 0, gamma));
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch);
+    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch, false);
     c->launches++;
     TRY(launch_iteration(*c, 0, gamma, accept_mode, mode_seed, INT_MAX));
     c->n_ub += gamma + 1;
@@ -1565,6 +1569,32 @@ extern "C" tandem_status tandem_block_step(tandem_ctx* c, int32_t gamma, int32_t
 
 namespace {
 
+// End of a generate call: counters, histogram, lengths and tokens come back in two copies behind one wait; the caller's
+// buffers are written only once the call is known to be good.
+tandem_status read_results(tandem_ctx* c, int max_new, int32_t* out_ids, int32_t* out_lens, unsigned long long* hist, int64_t* iters) {
+    const int B = c->batch;
+    int32_t* ids = c->pinned;   // staging is idle outside prefill
+    unsigned char* tail = reinterpret_cast<unsigned char*>(c->pinned + align_up((size_t)B * max_new, 64));
+    const size_t tail_bytes = c->lay.st_emitted + (size_t)B * 4 - c->lay.st_counters;
+    CK(cudaMemcpyAsync(tail, c->arena + c->lay.st_counters, tail_bytes, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpy2DAsync(ids, (size_t)max_new * 4, c->st.out_ids, (size_t)c->st.out_cap * 4, (size_t)max_new * 4, B,
+                         cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    const int32_t* cnt = reinterpret_cast<const int32_t*>(tail);
+    c->n_ub = cnt[3];
+    c->n_sum = cnt[4];
+    if (cnt[2] != 0) {   // a bounded device-side wait gave up somewhere in this call
+        snprintf(g_cuda_err, sizeof(g_cuda_err), "device-side wait expired (code %d)", cnt[2]);
+        CK(cudaMemsetAsync(c->st.counters + 2, 0, 4, c->stream));
+        return TANDEM_ERR_TIMEOUT;
+    }
+    *iters = cnt[5];
+    memcpy(hist, tail + (c->lay.st_hist - c->lay.st_counters), (TANDEM_GAMMA_LIMIT + 1) * 8);
+    memcpy(out_ids, ids, (size_t)B * max_new * 4);
+    if (out_lens) memcpy(out_lens, tail + (c->lay.st_emitted - c->lay.st_counters), (size_t)B * 4);
+    return TANDEM_OK;
+}
+
 // lead_large_step: the call starts with one round of the large model alone over the pending token (a block of one
 // row with projection and output head), which gives the first new token (Figure 2, left).
 tandem_status run_generate(tandem_ctx* c, bool speculative, int gamma, int max_new, int mode, uint64_t seed,
@@ -1575,26 +1605,24 @@ tandem_status run_generate(tandem_ctx* c, bool speculative, int gamma, int max_n
     TRY(capacity_for(c, max_new, gamma));
     const int B = c->batch;
     const int64_t launches0 = c->launches;
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B);
+    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B, true);
     c->launches++;
-    CK(cudaMemsetAsync(c->st.hist, 0, (TANDEM_GAMMA_LIMIT + 1) * 8, c->stream));
-    // Iterations are enqueued ahead of the host's knowledge of their outcome.  None can be the last one before
-    // ceil(max_new / (gamma + 1)); after that at most DEPTH iterations are in flight beyond the last one whose
-    // result the host has seen (surplus iterations find every sequence frozen and change nothing).
-    const int DEPTH = 3;
+    // Iterations are enqueued ahead of the host's knowledge of their outcome, but only those that are certain to be
+    // needed: every iteration gives a sequence at most per_iter tokens, so with `left` tokens still wanted by some
+    // sequence after the last observed iteration, ceil(left / per_iter) more must run whatever is accepted.  Beyond
+    // those the host waits for a result: a launch into an idle GPU costs about 10 us, a surplus iteration, which would find
+    // every sequence frozen and change nothing, a whole pass (two of them at the end of a call were 8 % of a small
+    // 64-token response and 15 % of the decode phase of a 32-token one).
     const int kind = speculative ? 0 : 1;
     const int64_t ticket0 = c->ticket;
     const int per_iter = (mode == TANDEM_ACCEPT_REPRESENTATION_ONLY || mode == 5) ? gamma : gamma + 1;   // most tokens one iteration can emit
     const int lead = lead_large_step ? 1 : 0;
-    const int min_iters = lead + (max_new - lead + per_iter - 1) / per_iter;
     const int n_known0 = c->n_ub;
     int64_t enq = 0, seen = 0;   // iterations of this call enqueued / observed
     int n_known = n_known0;      // max_b n_b after the last observed iteration
-    bool finished = false;
-    while (!finished) {
-        if (enq >= min_iters && enq - seen >= DEPTH) {
-            TRY(wait_ticket(*c, ticket0 + enq - DEPTH + 1));
-        }
+    int64_t certain = lead + (max_new - lead + per_iter - 1) / per_iter;   // iterations that must follow the last observed one
+    for (;;) {
+        if (enq - seen >= certain) TRY(wait_ticket(*c, ticket0 + seen + 1));
         // take whatever has been published so far
         const int64_t pub = (int64_t)((volatile int32_t*)c->hflags)[0] - ticket0;
         if (pub > seen) {
@@ -1602,33 +1630,20 @@ tandem_status run_generate(tandem_ctx* c, bool speculative, int gamma, int max_n
             seen = std::min<int64_t>(pub, enq);
             n_known = c->hflags[2];
             c->n_sum = c->hflags[3];
-            if (seen >= min_iters && c->hflags[1] <= 0) finished = true;
+            if (c->hflags[1] <= 0) break;
+            certain = std::max(1, (c->hflags[7] + per_iter - 1) / per_iter);
         }
-        if (finished) break;
-        if (enq > (int64_t)max_new + DEPTH + 1) return TANDEM_ERR_STATE;   // every live iteration emits a token
+        if (enq - seen >= certain) continue;
+        if (enq > (int64_t)max_new + 1) return TANDEM_ERR_STATE;   // every live iteration emits a token
         c->n_ub = std::min<long long>((long long)n_known + (enq - seen) * (gamma + 1), (long long)n_known0 + max_new);
         if (lead && enq == 0) TRY(launch_iteration(*c, 0, 0, TANDEM_ACCEPT_NATURAL, 0ull, max_new));
         else TRY(launch_iteration(*c, kind, gamma, mode, seed, max_new));
         ++enq;
     }
-    int32_t* cnt = c->pinned;   // staging is idle outside prefill
-    CK(cudaMemcpyAsync(cnt, c->st.counters, 8 * 4, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    c->n_ub = cnt[3];
-    c->n_sum = cnt[4];
-    if (cnt[2] != 0) {   // a bounded device-side wait gave up somewhere in this call
-        snprintf(g_cuda_err, sizeof(g_cuda_err), "device-side wait expired (code %d)", cnt[2]);
-        CK(cudaMemsetAsync(c->st.counters + 2, 0, 4, c->stream));
-        return TANDEM_ERR_TIMEOUT;
-    }
-    const int64_t iters = cnt[5];
-    TRY(check_launch());
-    CK(cudaMemcpy2DAsync(out_ids, (size_t)max_new * 4, c->st.out_ids, (size_t)c->st.out_cap * 4, (size_t)max_new * 4, B,
-                         cudaMemcpyDeviceToHost, c->stream));
+    int64_t iters = 0;
     std::vector<unsigned long long> hist(TANDEM_GAMMA_LIMIT + 1);
-    CK(cudaMemcpyAsync(hist.data(), c->st.hist, hist.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (out_lens) CK(cudaMemcpyAsync(out_lens, c->st.emitted, (size_t)B * 4, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    TRY(read_results(c, max_new, out_ids, out_lens, hist.data(), &iters));
+    TRY(check_launch());
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->iterations = iters;
@@ -1697,7 +1712,7 @@ extern "C" tandem_status tandem_adaptive_step(tandem_ctx* c, int32_t gamma_max, 
     if (gamma_max < 1 || gamma_max > c->cfg.gamma_max) return TANDEM_ERR_INVALID_ARG;
     if (c->batch == 0 || !c->has_router) return TANDEM_ERR_STATE;
     TRY(capacity_for(c, 0, gamma_max));
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch);
+    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch, false);
     c->launches++;
     int block_max = 0;
     TRY(adaptive_iteration(c, gamma_max, INT_MAX, &block_max));
@@ -1736,9 +1751,8 @@ extern "C" tandem_status tandem_adaptive_generate(tandem_ctx* c, int32_t gamma_m
     TRY(capacity_for(c, max_new, gamma_max));
     const int B = c->batch;
     const int64_t launches0 = c->launches;
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B);
+    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B, true);
     c->launches++;
-    CK(cudaMemsetAsync(c->st.hist, 0, (TANDEM_GAMMA_LIMIT + 1) * 8, c->stream));
     int64_t iters = 0, small_runs = 0;
     for (;;) {
         if (iters > max_new) return TANDEM_ERR_STATE;   // every live iteration emits a token
@@ -1748,13 +1762,9 @@ extern "C" tandem_status tandem_adaptive_generate(tandem_ctx* c, int32_t gamma_m
         small_runs += block_max;
         if (c->hflags[1] <= 0) break;
     }
-    TRY(check_error_word(c));
-    CK(cudaMemcpy2DAsync(out_ids, (size_t)max_new * 4, c->st.out_ids, (size_t)c->st.out_cap * 4, (size_t)max_new * 4, B,
-                         cudaMemcpyDeviceToHost, c->stream));
+    int64_t live_iters = 0;
     std::vector<unsigned long long> hist(TANDEM_GAMMA_LIMIT + 1);
-    CK(cudaMemcpyAsync(hist.data(), c->st.hist, hist.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (out_lens) CK(cudaMemcpyAsync(out_lens, c->st.emitted, (size_t)B * 4, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    TRY(read_results(c, max_new, out_ids, out_lens, hist.data(), &live_iters));
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->iterations = iters;
