@@ -31,7 +31,10 @@ struct AttnArgs {
     int split, t_max2;                         //   positions >= split (used when k2 != nullptr)
     void* out; int ldo;                  // T [M][ldo]; float when out_f32 is set (attn_decode_kernel only)
     int out_f32;
-    const int* row_seq; const int* row_pos;
+    const int* row_seq; const int* row_pos;    // attn_decode_kernel: row_seq may be null, then group g is sequence g and every
+    int pos_all;                               //   sequence's first row sits at position pos_all (no row arrays to fill and fetch)
+    int wait_first;                            // attn_decode_kernel: 1 = nothing is read before the wait on the preceding kernel
+                                               //   (a stand-alone call: whatever precedes it may be writing the keys and values)
     const int* grp_row0; const int* grp_cnt;   // nullable: then group g = rows g*nq .. g*nq+nq-1
     int nq;
     int n_heads, t_max;
@@ -326,8 +329,9 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // read before the wait below: a kernel lets its successor start only after its own wait has returned, that is
     // after its predecessor has finished, hence everything older than the immediate predecessor is complete.
     const int nq = a.nq, cnt = gpc * nq, row0 = g * nq;   // cnt: rows of the tile in use
-    const int b = __ldcg(a.row_seq + row0);          // from L2: nothing an earlier kernel on this SM may have cached
-    const int pos_first = __ldcg(a.row_pos + row0);
+    if (a.wait_first) pdl_wait();
+    const int b = a.row_seq ? __ldcg(a.row_seq + row0) : g;          // from L2: nothing an earlier kernel on this SM may have cached
+    const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
     const int pos_last = pos_first + nq - 1;
     const int n_chunks = pos_last / ATT_CH + 1;
     const int n_mine = rank < n_chunks ? (n_chunks - rank + CL - 1) / CL : 0;

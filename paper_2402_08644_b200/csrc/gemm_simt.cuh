@@ -19,7 +19,7 @@ struct EpiArgs {
     int ldo;
     void* kcache;         // QKV / KV: this layer's keys   [B][H][t_max][d_head] (T)
     void* vcache;         //           this layer's values
-    const int* row_seq;   // [M] sequence of each row
+    const int* row_seq;   // [M] sequence of each row (null on the tensor-core decode path: row j is sequence j at position 0)
     const int* row_pos;   // [M] absolute position of each row
     int n_heads, d_head, t_max;   // n_heads: key/value heads of the cache
     int seg0;             // QKV / KV: columns of the first segment (QKV: the queries, d_model; KV: the keys)

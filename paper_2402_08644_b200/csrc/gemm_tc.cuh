@@ -53,6 +53,8 @@ struct TcDecodeArgs {
     int tiles_per_seg;      // ceil(seg_rows / 128)
     int splits;             // K-slices per tile: 1, 2, 4 or 8 = the cluster size; grid = tiles * splits
     int stream_weights;     // 1: weights are read once per pass and should not stay in L2
+    int wait_first;         // 1: nothing is read before the wait on the preceding kernel (a stand-alone call: whatever precedes
+                            // it may be writing the weights)
     int* err_flag;          // nullable
     unsigned poll_limit;    // polls before a wait on an mbarrier gives up; 0 = MBAR_POLL_LIMIT
     int withhold_weights;   // test hook for the give-up path: the TMA thread issues no loads, so the wait for
@@ -177,7 +179,8 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     if (S > 1) cluster_arrive_relaxed();   // opening handshake: waited for just before the first remote store
 
     if (warp == 4) {
-        // ---- weight tiles: independent of every earlier kernel, so no wait on the predecessor here ----
+        // ---- weight tiles: independent of every earlier kernel of a context, so no wait on the predecessor here ----
+        if (a.wait_first) pdl_wait();
         if (PRO == PRO_TMA && lane == 0 && !a.withhold_weights) {
             // Weights of the first ring-ful before the wait on the predecessor, then the wait, then their token rows
             // (two planes, 16-row boxes), then weights and rows together as stages come free.
@@ -261,6 +264,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     } else {
     // ---- warps 0-3: token rows into the B stages (then the epilogue) ----
     float4 gq[C::STAGES], bq[C::STAGES];   // register path: gain / bias of this lane's slot in each of the CTA's K-blocks
+    if (a.wait_first) pdl_wait();
     if (ln_regs) {
 #pragma unroll
         for (int i = 0; i < C::STAGES; ++i) {
@@ -275,7 +279,10 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         // cache index of (row j, head h, element el) = ((seq_j * H + h) * t_max + pos_j) * d_head + el: the row part once
         // per row.  Only the epilogue needs it: the two loads are in flight while the B operand is produced, and the
         // barrier that publishes the offsets sits after that.
-        if (tid < a.rows) { my_seq = a.e.row_seq[tid]; my_pos = a.e.row_pos[tid]; }   // first used ahead of the epilogue
+        if (tid < a.rows) {                                                           // first used ahead of the epilogue
+            if (a.e.row_seq) { my_seq = a.e.row_seq[tid]; my_pos = a.e.row_pos[tid]; }
+            else my_seq = a.x_row0 + tid;                                             // stand-alone: row j is sequence j at position 0
+        }
     }
     if (EPI == EPI_RESID) {
         // the residual-stream values this thread will add to: fetched now, off the critical path

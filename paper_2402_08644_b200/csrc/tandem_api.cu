@@ -353,6 +353,7 @@ struct TcScratch {
     int* err;                  // where a bounded wait that ran out records its code (nullable)
     unsigned poll_limit = 0;   // 0: the kernels' default
     int withhold_weights = 0;  // test hook, see TcDecodeArgs
+    int wait_first = 0;        // the launch may follow kernels that write its weights, see TcDecodeArgs
 };
 
 TcW tcw3(const tandem_ctx& c, int i0, int i1, int i2, int seg_rows0, int seg_rows, int K) {
@@ -437,6 +438,7 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
         const int nr = std::min(64, rows - r0);
         a.rows = nr;
         a.x_row0 = r0; a.x_plane_rows = x_plane_rows;
+        a.wait_first = r0 == 0 ? sc.wait_first : 0;
         a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
         a.x = static_cast<const unsigned char*>(x) + (size_t)r0 * ldx * xsz;
         a.amax_val = amax_val ? amax_val + (size_t)r0 * amax_stride : nullptr;
@@ -1976,24 +1978,25 @@ extern "C" tandem_status tandem_debug_read(tandem_ctx* c, int32_t what, int32_t 
 // stand-alone kernels
 // ---------------------------------------------------------------------------------------------------
 
+// Stand-alone calls: two launches of one call, or of consecutive calls on a stream, are chained by programmatic dependent
+// launch, so that a kernel's set-up runs under its predecessor's end; the first kernel of a call reads nothing before its
+// predecessor has finished (the caller's kernels may be writing the inputs).  Only the stream, the launch counter and
+// the launch options of the context are used by the launch helpers.
 namespace {
-struct AttnScratch { size_t rows, total; };
-// The kernel reads each row's sequence and position from two int arrays; that is all the work space it needs.
-AttnScratch attn_scratch_layout(int batch) {
-    AttnScratch s;
-    s.rows = 0;
-    s.total = align_up((size_t)batch * 2 * 4);
-    return s;
-}
-__global__ void iota_rows_kernel(int* row_seq, int* row_pos, int n, int pos) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) { row_seq[i] = i; row_pos[i] = pos; }
-}
+struct StandaloneCtx : tandem_ctx {
+    explicit StandaloneCtx(void* s) {
+        stream = static_cast<cudaStream_t>(s);
+        n_sms = sm_count();
+    }
+};
+// Work space that the attention entry points ask their callers for: two ints per sequence, kept in the contract (the
+// kernel takes a sequence's number and position from its arguments now, which spared a kernel launch per call).
+size_t attn_scratch_size(int batch) { return align_up((size_t)batch * 2 * 4); }
 }  // namespace
 
 extern "C" size_t tandem_decode_attention_scratch_bytes(int32_t batch, int32_t n_heads, int32_t d_head, int32_t derived_len, int32_t own_len) {
     if (batch < 1 || n_heads < 1 || d_head < 1 || derived_len < 0 || own_len < 0 || derived_len + own_len < 1) return 0;
-    return attn_scratch_layout(batch).total;
+    return attn_scratch_size(batch);
 }
 
 extern "C" tandem_status tandem_decode_attention(const void* q, const void* k_derived, const void* v_derived, const void* k_own,
@@ -2006,23 +2009,14 @@ extern "C" tandem_status tandem_decode_attention(const void* q, const void* k_de
     if ((long long)batch * n_heads > 65535 * 16) return TANDEM_ERR_SHAPE;
     if (((uintptr_t)q | (uintptr_t)k_derived | (uintptr_t)v_derived | (uintptr_t)k_own | (uintptr_t)v_own | (uintptr_t)out | (uintptr_t)scratch) & 15)
         return TANDEM_ERR_INVALID_ARG;
-    const AttnScratch sl = attn_scratch_layout(batch);
-    if (scratch_bytes < sl.total) return TANDEM_ERR_ARENA_TOO_SMALL;
+    if (scratch_bytes < attn_scratch_size(batch)) return TANDEM_ERR_ARENA_TOO_SMALL;
     if (batch > 65535) return TANDEM_ERR_SHAPE;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    unsigned char* sc = static_cast<unsigned char*>(scratch);
-    int* row_seq = reinterpret_cast<int*>(sc + sl.rows);
-    int* row_pos = row_seq + batch;
-    iota_rows_kernel<<<cdiv(batch, 256), 256, 0, s>>>(row_seq, row_pos, batch, derived_len + own_len - 1);
     AttnArgs a; memset(&a, 0, sizeof(a));
     a.q = q; a.ldq = n_heads * d_head; a.kcache = k_derived; a.vcache = v_derived; a.k2 = k_own; a.v2 = v_own;
     a.split = derived_len; a.t_max = derived_len; a.t_max2 = own_len;
-    a.out = out; a.ldo = n_heads * d_head; a.row_seq = row_seq; a.row_pos = row_pos; a.nq = 1; a.n_heads = n_heads;
+    a.out = out; a.ldo = n_heads * d_head; a.pos_all = derived_len + own_len - 1; a.wait_first = 1; a.nq = 1; a.n_heads = n_heads;
     a.scale = 1.0f / sqrtf((float)d_head);
-    tandem_ctx tmp;   // only the stream, the launch counter and the launch options are used by the launch helpers
-    tmp.stream = s;
-    tmp.use_pdl = false;
-    tmp.n_sms = sm_count();
+    StandaloneCtx tmp(stream);
     launch_attn_decode(tmp, d_head, a, batch, 0.0);
     return check_launch();
 }
@@ -2031,46 +2025,21 @@ extern "C" tandem_status tandem_decode_attention(const void* q, const void* k_de
 // Decode attention for callers that cannot allocate device memory
 // ---------------------------------------------------------------------------------------------------
 
-// The per-row index arrays of tandem_decode_attention_static live here instead of in a caller-provided buffer.  Every GPU that loads this library holds these bytes until the process exits.
-static __device__ __align__(256) unsigned char g_static_attn_scratch[TANDEM_STATIC_SCRATCH_BYTES];
-
-namespace {
-// In host code the array's name is only a handle for the runtime, not a device address: the address
-// a kernel may use comes from cudaGetSymbolAddress, asked once per device with that device current.
-void* g_static_scratch_addr[MAX_DEVICES] = {};
-std::mutex g_static_scratch_mutex;
-
-tandem_status static_scratch_for_current_device(void** out) {
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= MAX_DEVICES) return TANDEM_ERR_INVALID_ARG;
-    std::lock_guard<std::mutex> lock(g_static_scratch_mutex);
-    if (!g_static_scratch_addr[dev]) {
-        void* p = nullptr;
-        CK(cudaGetSymbolAddress(&p, g_static_attn_scratch));
-        g_static_scratch_addr[dev] = p;
-    }
-    *out = g_static_scratch_addr[dev];
-    return TANDEM_OK;
-}
-}  // namespace
-
 extern "C" tandem_status tandem_decode_attention_static(const void* q, const void* k_derived, const void* v_derived,
                                                         const void* k_own, const void* v_own, void* out, int32_t batch,
                                                         int32_t n_heads, int32_t d_head, int32_t derived_len, int32_t own_len,
                                                         void* stream) {
     if (batch < 1 || n_heads < 1 || d_head < 1 || derived_len < 0 || own_len < 0 || derived_len + own_len < 1)
         return TANDEM_ERR_INVALID_ARG;
-    const size_t need = attn_scratch_layout(batch).total;
+    const size_t need = attn_scratch_size(batch);
     if (need > (size_t)TANDEM_STATIC_SCRATCH_BYTES) {
         snprintf(g_cuda_err, sizeof(g_cuda_err),
                  "tandem_decode_attention_static: this batch needs %zu bytes of work space, the built-in buffer holds %d; "
                  "use tandem_decode_attention with your own scratch", need, TANDEM_STATIC_SCRATCH_BYTES);
         return TANDEM_ERR_CAPACITY;
     }
-    void* scratch = nullptr;
-    TRY(static_scratch_for_current_device(&scratch));
-    return tandem_decode_attention(q, k_derived, v_derived, k_own, v_own, out, scratch, (size_t)TANDEM_STATIC_SCRATCH_BYTES, batch,
+    // the kernel reads and writes no work space; the call below only wants a non-null, aligned argument
+    return tandem_decode_attention(q, k_derived, v_derived, k_own, v_own, out, out, (size_t)TANDEM_STATIC_SCRATCH_BYTES, batch,
                                    n_heads, d_head, derived_len, own_len, stream);
 }
 
@@ -2096,13 +2065,12 @@ int* standalone_err_word() {
     return g_standalone_err_addr[dev];
 }
 
-struct ProjScratch { size_t yhat, a_s, rows, total; };
+struct ProjScratch { size_t yhat, a_s, total; };
 ProjScratch proj_scratch_layout(int rows, int d_small) {
     ProjScratch p;
     size_t off = 0;
     p.yhat = off; off = align_up(off + (size_t)rows * d_small * 4);
     p.a_s = off; off = align_up(off + (size_t)rows * d_small * 4);
-    p.rows = off; off = align_up(off + (size_t)rows * 8);
     p.total = off;
     return p;
 }
@@ -2137,15 +2105,10 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
     if (((uintptr_t)x | (uintptr_t)w_t | (uintptr_t)wk | (uintptr_t)wv | (uintptr_t)k_out | (uintptr_t)v_out | (uintptr_t)scratch |
          (uintptr_t)ln_g | (uintptr_t)ln_b) & 15)
         return TANDEM_ERR_INVALID_ARG;
-    tandem_ctx tmp;   // only the stream, the launch counter and the launch options are used by the launch helpers
-    tmp.stream = static_cast<cudaStream_t>(stream);
-    tmp.use_pdl = false;
-    tmp.n_sms = sm_count();
+    StandaloneCtx tmp(stream);
     unsigned char* sc = static_cast<unsigned char*>(scratch);
     float* yhat = reinterpret_cast<float*>(sc + pl.yhat);
     float* a_s = reinterpret_cast<float*>(sc + pl.a_s);
-    int* row_seq = reinterpret_cast<int*>(sc + pl.rows);
-    int* row_pos = row_seq + rows;
     TcW wt, wkv;
     if (!make_tmap_bf16(&wt.tm[0], w_t, (uint64_t)d_small, (uint64_t)d_large, (uint64_t)d_large) ||
         !make_tmap_bf16(&wkv.tm[0], wk, (uint64_t)d_small, (uint64_t)d_small, (uint64_t)d_small) ||
@@ -2155,17 +2118,18 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
     }
     wt.tm[1] = wt.tm[2] = wt.tm[0]; wt.n_segs = 1; wt.seg_rows0 = wt.seg_rows = d_small; wt.K = d_large;
     wkv.tm[2] = wkv.tm[0]; wkv.n_segs = 2; wkv.seg_rows0 = wkv.seg_rows = d_small; wkv.K = d_small;
-    iota_rows_kernel<<<cdiv(rows, 256), 256, 0, tmp.stream>>>(row_seq, row_pos, rows, 0);
     EpiArgs e; memset(&e, 0, sizeof(e));
-    e.kcache = k_out; e.vcache = v_out; e.row_seq = row_seq; e.row_pos = row_pos; e.n_heads = 1; e.d_head = d_small; e.t_max = 1; e.seg0 = e.seg = d_small;
+    e.kcache = k_out; e.vcache = v_out; e.n_heads = 1; e.d_head = d_small; e.t_max = 1; e.seg0 = e.seg = d_small;
     // weights streamed once per GEMM and group of 64 rows; for a few short rows the LayerNorm is fused into the
     // second GEMM's operand load
     TcScratch ts; ts.err = standalone_err_word();
+    ts.wait_first = 1;
     launch_tc_decode<PRO_BF16, EPI_STORE_F32>(tmp, ts, x, d_large, nullptr, nullptr, rows, wt, true, epi_plain(yhat, d_small));
+    ts.wait_first = 0;   // the kernels behind it start once everything older than the first GEMM has finished: the weights are final
     if (rows <= 8 && d_small <= 1024) {
         launch_tc_decode<PRO_LN, EPI_KV>(tmp, ts, yhat, d_small, ln_g, ln_b, rows, wkv, true, e);
     } else {
-        launch_ex(tmp, false, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
+        launch_ex(tmp, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
                   static_cast<const float*>(ln_b), a_s, (int)d_small, (bf16*)nullptr);
         launch_tc_decode<PRO_F32, EPI_KV>(tmp, ts, a_s, d_small, nullptr, nullptr, rows, wkv, true, e);
     }
@@ -2178,10 +2142,7 @@ extern "C" tandem_status tandem_block_linear(const void* x, const void* w, void*
     if (rows < 1 || rows > 64 || in_features < 8 || out_features < 1) return TANDEM_ERR_INVALID_ARG;
     if (in_features % 8) return TANDEM_ERR_SHAPE;
     if (((uintptr_t)x | (uintptr_t)w | (uintptr_t)y) & 15) return TANDEM_ERR_INVALID_ARG;
-    tandem_ctx tmp;   // only the stream, the launch counter and the launch options are used by the launch helpers
-    tmp.stream = static_cast<cudaStream_t>(stream);
-    tmp.use_pdl = false;
-    tmp.n_sms = sm_count();
+    StandaloneCtx tmp(stream);
     TcW tw;
     if (!make_tmap_bf16(&tw.tm[0], w, (uint64_t)out_features, (uint64_t)in_features, (uint64_t)in_features)) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled unavailable or failed");
@@ -2189,6 +2150,7 @@ extern "C" tandem_status tandem_block_linear(const void* x, const void* w, void*
     }
     tw.tm[1] = tw.tm[2] = tw.tm[0]; tw.n_segs = 1; tw.seg_rows0 = tw.seg_rows = out_features; tw.K = in_features;
     TcScratch ts; ts.err = standalone_err_word();
+    ts.wait_first = 1;
     launch_tc_decode<PRO_BF16, EPI_STORE>(tmp, ts, x, in_features, nullptr, nullptr, rows, tw, true, epi_plain(y, out_features));
     return check_launch();
 }
