@@ -1,6 +1,6 @@
 // Attention over a KV cache laid out [seq][head][position][d_head].
 //
-// One kernel serves three uses (Eq. 1 and Eq. 2, second line):
+// attn_kernel (fp32 mode; prompt pass at head size 32) serves three uses (Eq. 1 and Eq. 2, second line):
 //   * the small model's decode step: one query per (sequence, head) over the mixed context; positions
 //     the large model has processed hold large-derived keys/values, later ones the small model's own,
 //     in one contiguous cache, so the boundary needs no special handling here;
@@ -22,7 +22,7 @@ namespace tandem {
 
 constexpr int ATT_CH = 128;       // positions per chunk
 constexpr int ATT_NQ = 16;        // most queries per CTA (gamma limit + 1)
-constexpr int ATT_THREADS = 128;
+constexpr int ATT_THREADS = 256;
 
 struct AttnArgs {
     const void* q; int ldq;              // T [M][ldq]; head h at columns h*DH..
@@ -53,20 +53,25 @@ struct AttnArgs {
 
 template <typename T, int DH>
 constexpr size_t attn_smem_bytes() {
-    return (size_t)2 * ATT_CH * (DH + VecN<T>::N) * sizeof(T) + (size_t)ATT_NQ * DH * sizeof(float) +
+    return (size_t)2 * ATT_CH * (DH + 2 * VecN<T>::N) * sizeof(T) + (size_t)ATT_NQ * DH * sizeof(float) +
            (size_t)ATT_NQ * ATT_CH * sizeof(float) + (size_t)2 * ATT_NQ * sizeof(float);
 }
 
-// grid: (chunks, heads, groups) in split mode; (1, heads, groups) in loop mode.
+// grid: (chunks, heads, groups) in split mode; (1, heads, groups) in loop mode; block: ATT_THREADS.
+// Exact-arithmetic kernel, bound by the latency of its phases on short contexts (a draft step of the fp32 mode has one
+// CTA per head): two threads share a key's dot products, and in the value phase ATT_THREADS / DH threads share an output
+// element, each summing its own groups of four positions for all queries at once (four values and one 16-byte load of
+// probabilities per query and step), before their sums are added in a fixed order.  A block of five queries over 100
+// positions of 64-wide heads: 5.3 us, against 11.4 us with one thread per key and a query-by-query walk over the values.
 template <typename T, int DH, bool LOOP>
 __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
     constexpr int VN = VecN<T>::N;
-    constexpr int LD = DH + VN;                 // padded row: keeps 16-byte alignment, spreads banks
+    constexpr int LD = DH + 2 * VN;             // padded row: keeps 16-byte alignment, spreads banks
     constexpr int VPR = DH / VN;                // 16-byte vectors per row
-    constexpr int QS = ATT_THREADS / DH;        // query stride of the value phase
-    constexpr int QPT = (ATT_NQ + QS - 1) / QS; // queries per thread in the value phase
+    constexpr int PARTS = ATT_THREADS / DH;     // threads that share an output element in the value phase
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_last;
+    __shared__ float fo[ATT_NQ];   // LOOP: factor of what the earlier chunks contributed, per query
     pdl_wait();                // queries and keys/values come from earlier kernels
     pdl_launch_dependents();   // the next kernel may start fetching its weights
     T* ks = reinterpret_cast<T*>(smem_raw);
@@ -75,6 +80,8 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
     float* ss = qs + ATT_NQ * DH;
     float* cm = ss + ATT_NQ * ATT_CH;
     float* cl = cm + ATT_NQ;
+    float* red = reinterpret_cast<float*>(smem_raw);   // [PARTS][cnt][DH] where the keys were, once they are done with
+    static_assert((size_t)ATT_THREADS * ATT_NQ * sizeof(float) <= (size_t)2 * ATT_CH * LD * sizeof(T), "the parts' sums fit where the keys and values were");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.z, h = blockIdx.y;
@@ -94,114 +101,143 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
         qs[qi * DH + el] = to_float(qg[(size_t)(row0 + qi) * a.ldq + h * DH + el]);
     }
 
-    const int e = tid % DH, qsub = tid / DH;
-    float racc[QPT], rm[QPT], rl[QPT];
+    const int e = tid % DH, part = tid / DH;
+    float acc[ATT_NQ];
 #pragma unroll
-    for (int i = 0; i < QPT; ++i) { racc[i] = 0.f; rm[i] = -INFINITY; rl[i] = 0.f; }
+    for (int i = 0; i < ATT_NQ; ++i) acc[i] = 0.f;
+    if (LOOP && tid < ATT_NQ) { cm[tid] = -INFINITY; cl[tid] = 0.f; }
 
     const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
     const int kvh = h / (a.n_heads / n_kv);            // grouped-query attention: several query heads share one key/value head
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
-    const size_t head_base2 = ((size_t)b * n_kv + kvh) * a.t_max2;
-    const int split = a.k2 ? a.split : INT_MAX;
     for (int c = c_begin; c < c_end; ++c) {
         const int t0 = c * ATT_CH;
         const int nt = min(ATT_CH, pos_last + 1 - t0);
+        const int nt4 = (nt + 3) & ~3;
         __syncthreads();   // previous chunk fully consumed (and qs written, first time round)
-        for (int i = tid; i < nt * VPR; i += ATT_THREADS) {
+        for (int i = tid; i < nt4 * VPR; i += ATT_THREADS) {
             const int t = i / VPR, v = i - t * VPR;
-            const int ta = t0 + t;
-            const T* kg;
-            const T* vg;
-            if (ta < split) {
-                kg = static_cast<const T*>(a.kcache) + (head_base + ta) * DH;
-                vg = static_cast<const T*>(a.vcache) + (head_base + ta) * DH;
-            } else {
-                kg = static_cast<const T*>(a.k2) + (head_base2 + (ta - split)) * DH;
-                vg = static_cast<const T*>(a.v2) + (head_base2 + (ta - split)) * DH;
+            if (t < nt) {
+                const size_t src = (head_base + t0 + t) * DH + v * VN;
+                cp_async16(ks + t * LD + v * VN, static_cast<const T*>(a.kcache) + src);
+                cp_async16(vs + t * LD + v * VN, static_cast<const T*>(a.vcache) + src);
+            } else {       // up to three rows that fill the last group of four: a zero weight times them stays zero
+                *reinterpret_cast<uint4*>(vs + t * LD + v * VN) = make_uint4(0u, 0u, 0u, 0u);
             }
-            cp_async16(ks + t * LD + v * VN, kg + v * VN);
-            cp_async16(vs + t * LD + v * VN, vg + v * VN);
         }
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
 
-        // scores: thread t owns key t0+t for every query
-        for (int t = tid; t < nt; t += ATT_THREADS) {
+        // scores: threads 2t and 2t+1 own key t0+t for every query (even / odd 16-byte vectors of the row)
+        {
+            const int t = tid >> 1, half = tid & 1;
+            static_assert(ATT_THREADS == 2 * ATT_CH, "two threads per key");
             float dot[ATT_NQ];
 #pragma unroll
             for (int qi = 0; qi < ATT_NQ; ++qi) dot[qi] = 0.f;
+            if (t < nt) {
 #pragma unroll 2
-            for (int v = 0; v < VPR; ++v) {
-                float kv[VN];
-                load_vec(ks + t * LD + v * VN, kv);
+                for (int v = half; v < VPR; v += 2) {
+                    float kv[VN];
+                    load_vec(ks + t * LD + v * VN, kv);
 #pragma unroll
-                for (int qi = 0; qi < ATT_NQ; ++qi) {
-                    if (qi < cnt) {
+                    for (int qi = 0; qi < ATT_NQ; ++qi) {
+                        if (qi >= cnt) break;
 #pragma unroll
-                        for (int i = 0; i < VN; ++i) dot[qi] = fmaf(qs[qi * DH + v * VN + i], kv[i], dot[qi]);
+                        for (int i = 0; i < VN; i += 4) {
+                            const float4 q4 = *reinterpret_cast<const float4*>(qs + qi * DH + v * VN + i);
+                            dot[qi] = fmaf(q4.x, kv[i], dot[qi]); dot[qi] = fmaf(q4.y, kv[i + 1], dot[qi]);
+                            dot[qi] = fmaf(q4.z, kv[i + 2], dot[qi]); dot[qi] = fmaf(q4.w, kv[i + 3], dot[qi]);
+                        }
                     }
                 }
             }
 #pragma unroll
-            for (int qi = 0; qi < ATT_NQ; ++qi)
-                if (qi < cnt) ss[qi * ATT_CH + t] = (t0 + t <= pos_first + qi) ? dot[qi] * a.scale : -INFINITY;
+            for (int qi = 0; qi < ATT_NQ; ++qi) {
+                if (qi >= cnt) break;
+                const float d = dot[qi] + __shfl_xor_sync(0xffffffffu, dot[qi], 1);
+                if (half == 0 && t < nt4) ss[qi * ATT_CH + t] = (t < nt && t0 + t <= pos_first + qi) ? d * a.scale : -INFINITY;
+            }
         }
         __syncthreads();
 
-        // per query: chunk max, exponentials, chunk sum
+        // per query: maximum (LOOP: of everything so far), exponentials, sum
         for (int qi = warp; qi < cnt; qi += ATT_THREADS / 32) {
-            float m = -INFINITY;
+            float m = LOOP ? cm[qi] : -INFINITY;
+            const float m_old = m;
             for (int t = lane; t < nt; t += 32) m = fmaxf(m, ss[qi * ATT_CH + t]);
             m = warp_max(m);
             float l = 0.f;
-            if (m > -INFINITY) {
-                for (int t = lane; t < nt; t += 32) {
-                    const float p = expf(ss[qi * ATT_CH + t] - m);
-                    ss[qi * ATT_CH + t] = p;
-                    l += p;
-                }
-                l = warp_sum(l);
+            for (int t = lane; t < nt4; t += 32) {
+                const float p = m > -INFINITY ? expf(ss[qi * ATT_CH + t] - m) : 0.f;
+                ss[qi * ATT_CH + t] = p;
+                l += p;
             }
-            if (lane == 0) { cm[qi] = m; cl[qi] = l; }
+            l = warp_sum(l);
+            __syncwarp();
+            if (lane == 0) {
+                if (LOOP) {
+                    const float f = m_old > -INFINITY ? expf(m_old - m) : 0.f;
+                    fo[qi] = f;
+                    l = fmaf(cl[qi], f, l);
+                }
+                cm[qi] = m;
+                cl[qi] = l;
+            }
         }
         __syncthreads();
 
-        // weighted values: thread owns element e for queries qsub, qsub+QS, ...
+        // weighted values: this thread's groups of four positions, element e, every query
+        if (LOOP) {
 #pragma unroll
-        for (int i = 0; i < QPT; ++i) {
-            const int qi = qsub + i * QS;
-            if (qi < cnt && cm[qi] > -INFINITY) {
-                float o = 0.f;
-                for (int t = 0; t < nt; ++t) o = fmaf(ss[qi * ATT_CH + t], to_float(vs[t * LD + e]), o);
-                if (LOOP) {
-                    const float m_new = fmaxf(rm[i], cm[qi]);
-                    const float f_old = expf(rm[i] - m_new), f_new = expf(cm[qi] - m_new);
-                    racc[i] = racc[i] * f_old + o * f_new;
-                    rl[i] = rl[i] * f_old + cl[qi] * f_new;
-                    rm[i] = m_new;
-                } else {
-                    const size_t p = ((size_t)(row0 + qi) * a.n_heads + h) * a.n_chunks_max + c;
-                    a.part_acc[p * DH + e] = o;
-                    if (e == 0) { a.part_ml[p * 2] = cm[qi]; a.part_ml[p * 2 + 1] = cl[qi]; }
-                }
+            for (int qi = 0; qi < ATT_NQ; ++qi) {
+                if (qi >= cnt) break;
+                acc[qi] *= fo[qi];
+            }
+        }
+        for (int t = 4 * part; t < nt4; t += 4 * PARTS) {
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = to_float(vs[(t + i) * LD + e]);
+#pragma unroll
+            for (int qi = 0; qi < ATT_NQ; ++qi) {
+                if (qi >= cnt) break;
+                const float4 p = *reinterpret_cast<const float4*>(ss + qi * ATT_CH + t);
+                acc[qi] = fmaf(p.x, v[0], acc[qi]); acc[qi] = fmaf(p.y, v[1], acc[qi]);
+                acc[qi] = fmaf(p.z, v[2], acc[qi]); acc[qi] = fmaf(p.w, v[3], acc[qi]);
             }
         }
     }
-    T* og = static_cast<T*>(a.out);
-    if (LOOP) {
+    // the parts' sums of every (query, element), added in part order
+    __syncthreads();
 #pragma unroll
-        for (int i = 0; i < QPT; ++i) {
-            const int qi = qsub + i * QS;
-            if (qi < cnt) og[(size_t)(row0 + qi) * a.ldo + h * DH + e] = from_float<T>(racc[i] / rl[i]);
+    for (int qi = 0; qi < ATT_NQ; ++qi) {
+        if (qi >= cnt) break;
+        red[((size_t)part * cnt + qi) * DH + e] = acc[qi];
+    }
+    __syncthreads();
+    T* og = static_cast<T*>(a.out);
+    const int n_active = pos_last / ATT_CH + 1;        // CTAs of this (group, head) in split mode
+    for (int i = tid; i < cnt * DH; i += ATT_THREADS) {
+        const int qi = i / DH, el = i - qi * DH;
+        float o = 0.f;
+#pragma unroll
+        for (int p = 0; p < PARTS; ++p) o += red[(size_t)p * cnt * DH + i];
+        if (LOOP || n_active == 1) {
+            og[(size_t)(row0 + qi) * a.ldo + h * DH + el] = from_float<T>(o / cl[qi]);
+        } else if (cm[qi] > -INFINITY) {
+            const size_t p = ((size_t)(row0 + qi) * a.n_heads + h) * a.n_chunks_max + c_begin;
+            a.part_acc[p * DH + el] = o;
+            if (el == 0) { a.part_ml[p * 2] = cm[qi]; a.part_ml[p * 2 + 1] = cl[qi]; }
         }
-    } else {
+    }
+    if (!LOOP && n_active > 1) {
         // The CTA that finishes last for this (group, head) merges every query's chunks in position order.
         __threadfence();
         __syncthreads();
         if (tid == 0) {
-            const int active = min((int)gridDim.x, pos_last / ATT_CH + 1);   // CTAs that got this far
+            const int active = min((int)gridDim.x, n_active);   // CTAs that got this far
             int* counter = a.merge_counters + (size_t)g * a.n_heads + h;
             const int t = atomicAdd(counter, 1);
             s_last = (t == active - 1);
@@ -210,10 +246,8 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-#pragma unroll
-        for (int i = 0; i < QPT; ++i) {
-            const int qi = qsub + i * QS;
-            if (qi >= cnt) continue;
+        for (int i = tid; i < cnt * DH; i += ATT_THREADS) {
+            const int qi = i / DH, el = i - qi * DH;
             const int nc = (pos_first + qi) / ATT_CH + 1;
             const size_t base = ((size_t)(row0 + qi) * a.n_heads + h) * a.n_chunks_max;
             float mx = -INFINITY;
@@ -223,12 +257,12 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
 #pragma unroll 4
             for (int c = 0; c < nc; ++c) {
                 const float2 ml = __ldcg(reinterpret_cast<const float2*>(a.part_ml + (base + c) * 2));
-                const float pa = __ldcg(a.part_acc + (base + c) * DH + e);
+                const float pa = __ldcg(a.part_acc + (base + c) * DH + el);
                 const float f = expf(ml.x - mx);
                 l = fmaf(ml.y, f, l);
                 o = fmaf(pa, f, o);
             }
-            og[(size_t)(row0 + qi) * a.ldo + h * DH + e] = from_float<T>(o / l);
+            og[(size_t)(row0 + qi) * a.ldo + h * DH + el] = from_float<T>(o / l);
         }
     }
 }

@@ -1,7 +1,8 @@
 // SIMT GEMMs  y[m][n] = sum_k x[m][k] * W[n][k]  (weights [out][in]) with fused epilogues.
 //
-//  gemm_smallm_kernel  decode path (few rows): one warp per group of output columns streams the weight
-//                      rows once with 16-byte loads; the rows of x sit in shared memory.  HBM-bound.
+//  gemm_rows_kernel    few rows (the decode passes; prompts of up to 64 rows): one warp per one or four output
+//                      columns streams the weight rows with 16-byte loads; the rows of x sit in shared memory,
+//                      normalised on the way where LayerNorm precedes the map.
 //                      Each output element is reduced in an order that depends only on K, never on the
 //                      number of rows, so a block pass and a one-row pass give identical bits.
 //  gemm_tiled_kernel   prompt path (many rows), classic shared-memory tiling.
@@ -9,6 +10,7 @@
 // Both are the exact-arithmetic (fp32 FMA) paths of the fp32 test mode.
 #pragma once
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace tandem {
 
@@ -73,68 +75,135 @@ __device__ __forceinline__ void epilogue(const EpiArgs& e, int m, int n, float v
 
 constexpr int GS_THREADS = 256;
 constexpr int GS_WARPS = GS_THREADS / 32;
-constexpr int GS_COLS = 4;       // output columns per warp
-constexpr int GS_KC = 2048;      // K elements of x staged in shared memory at a time
+constexpr int GS_KC = 2048;      // K elements of x staged in shared memory at a time; the longest row whose LayerNorm is fused
 
-// grid: (ceil(N / (GS_WARPS*GS_COLS)), ceil(M / MT)); dynamic smem: MT * GS_KC * sizeof(T)
-template <typename T, int MT, int EPI>
-__global__ void __launch_bounds__(GS_THREADS)
-gemm_smallm_kernel(const T* __restrict__ x, int ldx, int M, int K, WSegs ws, int N, EpiArgs e) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* xs = reinterpret_cast<T*>(smem_raw);
-    constexpr int VN = VecN<T>::N;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n0 = (blockIdx.x * GS_WARPS + warp) * GS_COLS;
-    const int m0 = blockIdx.y * MT;
-
-    const T* wrow[GS_COLS];
+// Sums NV values over the warp's lanes, NV a power of two up to 32: halves the number of values a lane carries while it
+// halves the distance, so NV values cost NV - 1 + (5 - log2 NV) shuffles instead of 5 NV.  Lane L returns the sum of value
+// L >> (5 - log2 NV).  The tree of additions is the butterfly 16, 8, 4, 2, 1 for every value and every NV.
+template <int NV>
+__device__ __forceinline__ float warp_sum_many(float (&v)[NV], int lane) {
+    int off = 16;
 #pragma unroll
-    for (int c = 0; c < GS_COLS; ++c) wrow[c] = (n0 + c < N) ? weight_row<T>(ws, n0 + c, K) : nullptr;
-
-    float acc[MT][GS_COLS];
+    for (int n = NV; n > 1; n >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
 #pragma unroll
-    for (int r = 0; r < MT; ++r)
-#pragma unroll
-        for (int c = 0; c < GS_COLS; ++c) acc[r][c] = 0.f;
-
-    for (int k0 = 0; k0 < K; k0 += GS_KC) {
-        const int kc = min(GS_KC, K - k0);
-        const int vec_per_row = kc / VN;
-        __syncthreads();
-        for (int i = threadIdx.x; i < MT * vec_per_row; i += GS_THREADS) {
-            const int r = i / vec_per_row, v = i - r * vec_per_row;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (m0 + r < M) val = *reinterpret_cast<const uint4*>(x + (size_t)(m0 + r) * ldx + k0 + v * VN);
-            *reinterpret_cast<uint4*>(xs + r * GS_KC + v * VN) = val;
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int kk = lane * VN; kk < kc; kk += 32 * VN) {
-            float wv[GS_COLS][VN];
-#pragma unroll
-            for (int c = 0; c < GS_COLS; ++c) {
-                uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-                if (wrow[c] != nullptr) raw = ldg_stream(wrow[c] + k0 + kk);
-                widen(raw, wv[c]);
-            }
-#pragma unroll
-            for (int r = 0; r < MT; ++r) {
-                float xv[VN];
-                load_vec(xs + r * GS_KC + kk, xv);
-#pragma unroll
-                for (int c = 0; c < GS_COLS; ++c)
-#pragma unroll
-                    for (int i = 0; i < VN; ++i) acc[r][c] = fmaf(xv[i], wv[c][i], acc[r][c]);
-            }
+        for (int i = 0; i < n / 2; ++i) {
+            const float keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
 #pragma unroll
-    for (int r = 0; r < MT; ++r)
+    for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    return v[0];
+}
+
+// Few rows, fp32: one warp per NC output columns, the rows of x in shared memory, LayerNorm fused (LN, K <= GS_KC).
+// Bound by latency (the fp32 pair's matrices are 0.06-1 MB): NC = 1 spreads N = 256..1024 over the whole GPU, NC = 4 reads
+// the staged rows once per four columns when there are columns enough; a warp's first weights are fetched before the wait
+// on the preceding kernel; the row sums leave the warp through warp_sum_many and are finished by several lanes side by
+// side.  Five rows, N = 768, K = 256 with LayerNorm: 4.0 us of the stream's time, against 2.1 us for a LayerNorm kernel and
+// 12.4 us for four columns per warp, a butterfly per sum and one writing lane.
+// grid: (ceil(N / (GS_WARPS * NC)), ceil(M / MT)); dynamic smem: MT * min(K, GS_KC) floats.
+template <int MT, int NC, bool LN, int EPI>
+__global__ void __launch_bounds__(GS_THREADS)
+gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, int N, const float* __restrict__ ln_g,
+                 const float* __restrict__ ln_b, EpiArgs e) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float* xs = reinterpret_cast<float*>(smem_raw);
+    constexpr int PF = 8 / NC;    // float4s of each column fetched ahead of the wait
+    constexpr int NV = MT * NC;
+    constexpr int LOG = NV == 1 ? 0 : (NV == 4 ? 2 : (NV == 8 ? 3 : (NV == 16 ? 4 : 5)));
+    static_assert(NV == 1 || NV == 4 || NV == 8 || NV == 16 || NV == 32, "warp_sum_many");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = (blockIdx.x * GS_WARPS + warp) * NC;
+    const int m0 = blockIdx.y * MT, rows = min(MT, M - m0);
+    const int KS = min(K, GS_KC);      // row stride in shared memory
+
+    const float* wrow[NC];
 #pragma unroll
-        for (int c = 0; c < GS_COLS; ++c) {
-            const float v = warp_sum(acc[r][c]);
-            if (lane == 0 && m0 + r < M && n0 + c < N) epilogue<T, EPI>(e, m0 + r, n0 + c, v);
+    for (int c = 0; c < NC; ++c) wrow[c] = (n0 + c < N) ? weight_row<float>(ws, n0 + c, K) : nullptr;
+    float4 wpre[NC][PF];               // weights are parameters: no need to wait for them
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < PF; ++i) {
+            const int kk = (lane + 32 * i) * 4;
+            wpre[c][i] = (wrow[c] != nullptr && kk < K) ? __ldg(reinterpret_cast<const float4*>(wrow[c] + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+    pdl_wait();
+    pdl_launch_dependents();
+
+    float acc[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] = 0.f;
+    auto step = [&](const float4 (&w)[NC], int kk) {
+#pragma unroll
+        for (int r = 0; r < MT; ++r) {
+            if (r >= rows) break;
+            const float4 xv = *reinterpret_cast<const float4*>(xs + r * KS + kk);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                float t = acc[r * NC + c];
+                t = fmaf(xv.x, w[c].x, t); t = fmaf(xv.y, w[c].y, t); t = fmaf(xv.z, w[c].z, t); t = fmaf(xv.w, w[c].w, t);
+                acc[r * NC + c] = t;
+            }
+        }
+    };
+    for (int k0 = 0; k0 < K; k0 += GS_KC) {
+        const int kc = min(GS_KC, K - k0), vec = kc >> 2;
+        __syncthreads();
+        for (int i = threadIdx.x; i < rows * vec; i += GS_THREADS) {
+            const int r = i / vec, v = i - r * vec;
+            *reinterpret_cast<float4*>(xs + r * KS + v * 4) = __ldcg(reinterpret_cast<const float4*>(x + (size_t)(m0 + r) * ldx + k0 + v * 4));
+        }
+        __syncthreads();
+        if (LN) {   // one warp per row, fixed lane-strided order (biased variance, eps 1e-5)
+            for (int r = warp; r < rows; r += GS_WARPS) {
+                float* xr = xs + r * KS;
+                float s = 0.f;
+                for (int k = lane * 4; k < K; k += 128) { const float4 t = *reinterpret_cast<const float4*>(xr + k); s += (t.x + t.y) + (t.z + t.w); }
+                const float mu = warp_sum(s) / (float)K;
+                float q = 0.f;
+                for (int k = lane * 4; k < K; k += 128) {
+                    const float4 t = *reinterpret_cast<const float4*>(xr + k);
+                    const float d0 = t.x - mu, d1 = t.y - mu, d2 = t.z - mu, d3 = t.w - mu;
+                    q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
+                }
+                const float rs = 1.0f / sqrtf(warp_sum(q) / (float)K + 1e-5f);
+                for (int k = lane * 4; k < K; k += 128) {
+                    float4 t = *reinterpret_cast<const float4*>(xr + k);
+                    const float4 g = __ldg(reinterpret_cast<const float4*>(ln_g + k)), b = __ldg(reinterpret_cast<const float4*>(ln_b + k));
+                    t.x = (t.x - mu) * rs * g.x + b.x; t.y = (t.y - mu) * rs * g.y + b.y;
+                    t.z = (t.z - mu) * rs * g.z + b.z; t.w = (t.w - mu) * rs * g.w + b.w;
+                    *reinterpret_cast<float4*>(xr + k) = t;
+                }
+            }
+            __syncthreads();
+        }
+        int i = 0;
+        if (k0 == 0) {
+#pragma unroll
+            for (int p = 0; p < PF; ++p) {
+                const int kk = (lane + 32 * p) * 4;
+                float4 w[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) w[c] = wpre[c][p];
+                if (kk < kc) step(w, kk);
+            }
+            i = PF;
+        }
+#pragma unroll 2
+        for (int kk = (lane + 32 * i) * 4; kk < kc; kk += 128) {
+            float4 w[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                w[c] = wrow[c] != nullptr ? __ldg(reinterpret_cast<const float4*>(wrow[c] + k0 + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            step(w, kk);
+        }
+    }
+    const float v = warp_sum_many<NV>(acc, lane);
+    const int idx = lane >> (5 - LOG), r = idx / NC, n = n0 + idx % NC;
+    if ((lane & ((32 >> LOG) - 1)) == 0 && r < rows && n < N) epilogue<float, EPI>(e, m0 + r, n, v);
 }
 
 // Shared-memory tiled GEMM for many rows.  64x64 output tile, 16-deep K slices, 4x4 outputs per thread.

@@ -32,17 +32,6 @@ struct LoopState {
     int gamma_limit;
 };
 
-// Decode rows: sequence b contributes rows r0 .. r0+nq-1 of its block (row 0 = pending token, row r = draft r).
-// Row m = b*nq + (r - r0):  token, sequence, absolute position n_b - 1 + r.
-__global__ void setup_rows_kernel(LoopState st, int batch, int r0, int nq, int* row_tok, int* row_seq, int* row_pos) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= batch * nq) return;
-    const int b = m / nq, r = r0 + (m - b * nq);
-    row_tok[m] = (r == 0) ? st.pending[b] : st.drafts[b * st.gamma_limit + r - 1];
-    row_seq[m] = b;
-    row_pos[m] = st.n[b] - 1 + r;
-}
-
 // x^(0) = Emb(t) + Pos(index)  (Eq. 1); fp32 residual stream.  grid: rows; block: 128.
 template <typename T>
 __global__ void embed_kernel(const int* __restrict__ row_tok, const int* __restrict__ row_pos, const T* __restrict__ emb,
@@ -244,6 +233,8 @@ __global__ void cast_rows_kernel(const float* __restrict__ x, T* __restrict__ ou
 __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restrict__ logits, int V, int* dst, int nq, int seq_stride, int off) {
     __shared__ float sv[8];
     __shared__ int si[8];
+    pdl_wait();
+    pdl_launch_dependents();
     const float* lr = logits + (size_t)blockIdx.x * V;
     float best = -INFINITY;
     int bi = 0x7fffffff;

@@ -301,17 +301,6 @@ int sm_count() {
     return n;
 }
 
-template <typename T, int MT, int EPI>
-void launch_smallm(tandem_ctx& c, const T* x, int ldx, int M, int K, const WSegs& ws, int N, const EpiArgs& e) {
-    static std::atomic<unsigned long long> attr_done{0};
-    const size_t smem = (size_t)MT * GS_KC * sizeof(T);
-    ensure_dyn_smem(gemm_smallm_kernel<T, MT, EPI>, smem, attr_done);
-    dim3 grid(cdiv(N, GS_WARPS * GS_COLS), cdiv(M, MT));
-    ProfScope ps(c, PC_GEMM_SMALLM, ((double)N * K + (double)M * K + (double)M * N) * sizeof(T));
-    gemm_smallm_kernel<T, MT, EPI><<<grid, GS_THREADS, smem, c.stream>>>(x, ldx, M, K, ws, N, e);
-    c.launches++;
-}
-
 // ---------------------------------------------------------------------------------------------------
 // tensor-core GEMMs: tensor maps and launches
 // ---------------------------------------------------------------------------------------------------
@@ -499,39 +488,56 @@ WSegs segs_of(const tandem_ctx& c, const Lin& l) {
     return s;
 }
 
-// y = x W^T with a fused epilogue.  decode: few rows, streaming kernel; otherwise the prompt-pass kernels
-// (tensor cores for bf16 when the context has tensor maps).
-template <typename T, int EPI>
-void launch_gemm(tandem_ctx& c, bool decode, const T* x, int ldx, int M, const Lin& l, const EpiArgs& e) {
+// fp32, few rows.  ln_g / ln_b non-null: LayerNorm of the rows first (fused; K <= GS_KC, see fp32_few_rows).
+template <int MT, int NC, bool LN, int EPI>
+void launch_rows_as(tandem_ctx& c, const float* x, int ldx, int M, int K, const WSegs& ws, int N, const float* ln_g, const float* ln_b, const EpiArgs& e) {
+    static std::atomic<unsigned long long> attr_done{0};
+    ensure_dyn_smem(gemm_rows_kernel<MT, NC, LN, EPI>, (size_t)MT * GS_KC * sizeof(float), attr_done);
+    launch_ex(c, true, 1, gemm_rows_kernel<MT, NC, LN, EPI>, dim3(cdiv(N, GS_WARPS * NC), cdiv(M, MT)), dim3(GS_THREADS),
+              (size_t)MT * std::min(K, GS_KC) * sizeof(float), x, ldx, M, K, ws, N, ln_g, ln_b, e);
+}
+template <bool LN, int EPI>
+void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, const EpiArgs& e, const void* ln_g = nullptr, const void* ln_b = nullptr) {
     if (M <= 0) return;
     const WSegs ws = segs_of(c, l);
     const int N = lin_n(l), K = l.K;
-    if (decode) {
-        if (M <= 1) launch_smallm<T, 1, EPI>(c, x, ldx, M, K, ws, N, e);
-        else if (M <= 2) launch_smallm<T, 2, EPI>(c, x, ldx, M, K, ws, N, e);
-        else if (M <= 4) launch_smallm<T, 4, EPI>(c, x, ldx, M, K, ws, N, e);
-        else launch_smallm<T, 8, EPI>(c, x, ldx, M, K, ws, N, e);
-    } else if (sizeof(T) == 2 && c.tc) {
-        if (launch_tc_tiled<EPI>(c, reinterpret_cast<const bf16*>(x), ldx, M, tcw3(c, l.i0, l.i1, l.i2, l.seg_rows0, l.seg_rows, l.K), e,
-                                 c.st.counters + 2) != TANDEM_OK)
+    const float *g = static_cast<const float*>(ln_g), *b = static_cast<const float*>(ln_b);
+    ProfScope ps(c, PC_GEMM_SMALLM, ((double)N * K + (double)M * K + (double)M * N) * sizeof(float));
+    // one column per warp until that is two CTAs per multiprocessor, then four (the staged rows are read once for them)
+    const bool wide = N > 2 * GS_WARPS * std::max(1, c.n_sms);
+    if (M <= 1) { if (wide) launch_rows_as<1, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<1, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
+    else if (M <= 4) { if (wide) launch_rows_as<4, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<4, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
+    else { if (wide) launch_rows_as<8, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<8, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
+}
+
+// y = x W^T with a fused epilogue for many rows: the prompt-pass kernels (tensor cores for bf16).
+template <typename T, int EPI>
+void launch_gemm(tandem_ctx& c, const T* x, int ldx, int M, const Lin& l, const EpiArgs& e) {
+    if (M <= 0) return;
+    if constexpr (sizeof(T) == 2) {
+        if (launch_tc_tiled<EPI>(c, x, ldx, M, tcw3(c, l.i0, l.i1, l.i2, l.seg_rows0, l.seg_rows, l.K), e, c.st.counters + 2) != TANDEM_OK)
             c.setup_failed = true;
     } else {
+        const int N = lin_n(l), K = l.K;
         dim3 grid(cdiv(N, GT_BN), cdiv(M, GT_BM));
         ProfScope ps(c, PC_GEMM_TILED, 2.0 * M * (double)N * K);   // flops, not bytes: this one is compute-bound
-        gemm_tiled_kernel<T, EPI><<<grid, GT_THREADS, 0, c.stream>>>(x, ldx, M, K, ws, N, e);
+        gemm_tiled_kernel<T, EPI><<<grid, GT_THREADS, 0, c.stream>>>(x, ldx, M, K, segs_of(c, l), N, e);
         c.launches++;
     }
 }
 
 template <typename T, int DH>
 void launch_attn_dh(tandem_ctx& c, const AttnArgs& a, int groups, bool loop, int n_chunks, double kv_bytes) {
-    static std::atomic<unsigned long long> attr_done_split{0}, attr_done_loop{0};
-    ensure_dyn_smem(attn_kernel<T, DH, false>, attn_smem_bytes<T, DH>(), attr_done_split);
-    ensure_dyn_smem(attn_kernel<T, DH, true>, attn_smem_bytes<T, DH>(), attr_done_loop);
+    static std::atomic<unsigned long long> attr_done_loop{0};
     if (loop) {
+        ensure_dyn_smem(attn_kernel<T, DH, true>, attn_smem_bytes<T, DH>(), attr_done_loop);
         ProfScope ps(c, PC_ATTN_PROMPT, kv_bytes);
-        launch_ex(c, false, 1, attn_kernel<T, DH, true>, dim3(1, a.n_heads, groups), dim3(ATT_THREADS), attn_smem_bytes<T, DH>(), a);
-    } else {
+        launch_ex(c, true, 1, attn_kernel<T, DH, true>, dim3(1, a.n_heads, groups), dim3(ATT_THREADS), attn_smem_bytes<T, DH>(), a);
+        return;
+    }
+    if constexpr (sizeof(T) == 4) {   // (the bf16 decode passes have their own kernel)
+        static std::atomic<unsigned long long> attr_done_split{0};
+        ensure_dyn_smem(attn_kernel<T, DH, false>, attn_smem_bytes<T, DH>(), attr_done_split);
         ProfScope ps(c, PC_ATTN_SPLIT, kv_bytes);
         launch_ex(c, true, 1, attn_kernel<T, DH, false>, dim3(n_chunks, a.n_heads, groups), dim3(ATT_THREADS), attn_smem_bytes<T, DH>(), a);
     }
@@ -674,24 +680,53 @@ void attention_decode(tandem_ctx& c, const Model& m, int l, const bf16* q, float
     launch_attn_decode(c, dh, aa, r.groups, r.kv_positions * 2.0 * d * 2.0);
 }
 
+// The fp32 passes whose maps run on the few-row kernel with LayerNorm fused into it: decode passes and short prompts.
+bool fp32_few_rows(const tandem_ctx& c, const Rows& r) {
+    return c.cfg.dtype == TANDEM_DTYPE_FP32 && (r.decode || r.M <= 64);
+}
+// LayerNorm, then y = a W^T (few rows, fp32): one kernel up to GS_KC elements per row, two beyond.
+template <int EPI>
+void ln_rows(tandem_ctx& c, const float* h, int M, const void* g, const void* b, const Lin& l, const EpiArgs& e) {
+    if (l.K <= GS_KC) { launch_rows<true, EPI>(c, h, l.K, M, l, e, g, b); return; }
+    float* a = at<float>(c, c.lay.a);
+    launch_layernorm<float>(c, M, h, g, b, a, l.K);
+    launch_rows<false, EPI>(c, a, l.K, M, l, e);
+}
+
 // Eq. 2, first line, for small layer j, then that layer's LayerNorm and key/value maps: writes the
 // small model's large-derived keys/values for the rows' positions.
 template <typename T>
 void project_layer(tandem_ctx& c, int j, const Rows& r) {
     const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    T* xb = at<T>(c, c.lay.xb);
+    const Lin t0 = lin1(wi_tandem(c, j, 0), c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR ? dS : c.hidden, dL);
+    const Lin kv = lin3(wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, c.small.d_kv, dS);
     float* yhat = at<float>(c, c.lay.yhat);
+    T* t1 = at<T>(c, c.lay.t1);
+    const EpiArgs ekv = epi_cache<T>(c, c.small, j, nullptr);
+    const void *lg = w_layer(c, c.small, j, W_LN1G), *lb = w_layer(c, c.small, j, W_LN1B);
+    if constexpr (sizeof(T) == 4) {
+        const float* x = at<float>(c, c.lay.h_large);   // fp32: the residual stream itself is the input
+        if (fp32_few_rows(c, r)) {
+            if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
+                launch_rows<false, EPI_STORE_F32>(c, x, dL, r.M, t0, epi_plain(yhat, dS));
+            } else {
+                launch_rows<false, EPI_GELU>(c, x, dL, r.M, t0, epi_plain(t1, c.hidden));
+                launch_rows<false, EPI_STORE_F32>(c, t1, c.hidden, r.M, lin1(wi_tandem(c, j, 1), dS, c.hidden), epi_plain(yhat, dS));
+            }
+            ln_rows<EPI_KV>(c, yhat, r.M, lg, lb, kv, ekv);
+            return;
+        }
+    }
+    const T* x = sizeof(T) == 4 ? reinterpret_cast<const T*>(at<float>(c, c.lay.h_large)) : at<T>(c, c.lay.xb);
     T* a_s = at<T>(c, c.lay.a_s);
     if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
-        launch_gemm<T, EPI_STORE_F32>(c, r.decode, xb, dL, r.M, lin1(wi_tandem(c, j, 0), dS, dL), epi_plain(yhat, dS));
+        launch_gemm<T, EPI_STORE_F32>(c, x, dL, r.M, t0, epi_plain(yhat, dS));
     } else {
-        T* t1 = at<T>(c, c.lay.t1);
-        launch_gemm<T, EPI_GELU>(c, r.decode, xb, dL, r.M, lin1(wi_tandem(c, j, 0), c.hidden, dL), epi_plain(t1, c.hidden));
-        launch_gemm<T, EPI_STORE_F32>(c, r.decode, t1, c.hidden, r.M, lin1(wi_tandem(c, j, 1), dS, c.hidden), epi_plain(yhat, dS));
+        launch_gemm<T, EPI_GELU>(c, x, dL, r.M, t0, epi_plain(t1, c.hidden));
+        launch_gemm<T, EPI_STORE_F32>(c, t1, c.hidden, r.M, lin1(wi_tandem(c, j, 1), dS, c.hidden), epi_plain(yhat, dS));
     }
-    launch_layernorm<T>(c, r.M, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), a_s, dS);
-    launch_gemm<T, EPI_KV>(c, r.decode, a_s, dS, r.M, lin3(wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, c.small.d_kv, dS),
-                           epi_cache<T>(c, c.small, j, nullptr));
+    launch_layernorm<T>(c, r.M, yhat, lg, lb, a_s, dS);
+    launch_gemm<T, EPI_KV>(c, a_s, dS, r.M, kv, ekv);
 }
 
 template <typename T>
@@ -699,8 +734,8 @@ void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
     bool any = false;
     for (int j = 0; j < c.small.d.n_layers; ++j) any |= (c.layer_map[j] == n_large_layers_done);
     if (!any) return;
-    const size_t n = (size_t)r.M * c.large.d.d_model;
-    {
+    if constexpr (sizeof(T) == 2) {
+        const size_t n = (size_t)r.M * c.large.d.d_model;
         ProfScope ps(c, PC_ROWS, (double)n * (4.0 + sizeof(T)));
         cast_rows_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(at<float>(c, c.lay.h_large), at<T>(c, c.lay.xb), n);
         c.launches++;
@@ -717,45 +752,58 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
     T* q = at<T>(c, c.lay.q);
     T* o = at<T>(c, c.lay.o);
     T* f = at<T>(c, c.lay.f);
-    launch_layernorm<T>(c, r.M, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), a, d);
-    launch_gemm<T, EPI_QKV>(c, r.decode, a, d, r.M, lin3(wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d),
-                            epi_cache<T>(c, m, l, q));
+    const Lin qkv = lin3(wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d);
+    const Lin wo = lin1(wi_layer(m, l, W_WO), d, d), w1 = lin1(wi_layer(m, l, W_W1), dff, d), w2 = lin1(wi_layer(m, l, W_W2), d, dff);
+    const void *g1 = w_layer(c, m, l, W_LN1G), *b1 = w_layer(c, m, l, W_LN1B), *g2 = w_layer(c, m, l, W_LN2G), *b2 = w_layer(c, m, l, W_LN2B);
+    if constexpr (sizeof(T) == 4) {
+        if (fp32_few_rows(c, r)) {
+            ln_rows<EPI_QKV>(c, h, r.M, g1, b1, qkv, epi_cache<T>(c, m, l, q));
+            attention<T>(c, m, l, q, o, r);
+            launch_rows<false, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
+            ln_rows<EPI_GELU>(c, h, r.M, g2, b2, w1, epi_plain(f, dff));
+            launch_rows<false, EPI_RESID>(c, f, dff, r.M, w2, epi_plain(h, d));
+            return;
+        }
+    }
+    launch_layernorm<T>(c, r.M, h, g1, b1, a, d);
+    launch_gemm<T, EPI_QKV>(c, a, d, r.M, qkv, epi_cache<T>(c, m, l, q));
     attention<T>(c, m, l, q, o, r);
-    launch_gemm<T, EPI_RESID>(c, r.decode, o, d, r.M, lin1(wi_layer(m, l, W_WO), d, d), epi_plain(h, d));
-    launch_layernorm<T>(c, r.M, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), a, d);
-    launch_gemm<T, EPI_GELU>(c, r.decode, a, d, r.M, lin1(wi_layer(m, l, W_W1), dff, d), epi_plain(f, dff));
-    launch_gemm<T, EPI_RESID>(c, r.decode, f, dff, r.M, lin1(wi_layer(m, l, W_W2), d, dff), epi_plain(h, d));
+    launch_gemm<T, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
+    launch_layernorm<T>(c, r.M, h, g2, b2, a, d);
+    launch_gemm<T, EPI_GELU>(c, a, d, r.M, w1, epi_plain(f, dff));
+    launch_gemm<T, EPI_RESID>(c, f, dff, r.M, w2, epi_plain(h, d));
 }
 
-// Final LayerNorm, output head, arg-max.  dst[(m / nq) * seq_stride + m % nq + off].
-template <typename T>
+// Final LayerNorm, output head, arg-max of a decode pass (fp32).  dst[(m / nq) * seq_stride + m % nq + off].
 void head_argmax(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* logits, int* dst, int seq_stride, int off) {
     const int d = m.d.d_model, V = m.d.vocab;
-    T* a = at<T>(c, c.lay.a);
-    launch_layernorm<T>(c, r.M, h, w_tail(c, m, 0), w_tail(c, m, 1), a, d);
-    launch_gemm<T, EPI_STORE_F32>(c, r.decode, a, d, r.M, lin1(wi_tail(m, 2), V, d), epi_plain(logits, V));
+    ln_rows<EPI_STORE_F32>(c, h, r.M, w_tail(c, m, 0), w_tail(c, m, 1), lin1(wi_tail(m, 2), V, d), epi_plain(logits, V));
     ProfScope ps(c, PC_ARGMAX, (double)r.M * V * 4.0);
-    argmax_rows_kernel<<<r.M, 256, 0, c.stream>>>(logits, V, dst, r.nq, seq_stride, off);
-    c.launches++;
+    launch_ex(c, true, 1, argmax_rows_kernel, dim3(r.M), dim3(256), 0, (const float*)logits, V, dst, r.nq, seq_stride, off);
 }
 
-// The large model over the current rows (block mode in decode, whole prompt otherwise).
+// The large model's layers over the current rows, whose embeddings are in the residual stream (block mode in decode,
+// whole prompt otherwise).
 template <typename T>
-void large_pass(tandem_ctx& c, const Rows& r, bool project, bool head) {
+void large_layers(tandem_ctx& c, const Rows& r, bool project) {
     float* h = at<float>(c, c.lay.h_large);
-    {
-        ProfScope ps(c, PC_ROWS, (double)r.M * c.large.d.d_model * (4.0 + 2 * sizeof(T)));
-        embed_kernel<T><<<r.M, 128, 0, c.stream>>>(at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_pos), (const T*)w_emb(c, c.large),
-                                                   (const T*)w_pos(c, c.large), h, c.large.d.d_model);
-        c.launches++;
-    }
     if (project) project_after<T>(c, 0, r);
     for (int l = 0; l < c.large.d.n_layers; ++l) {
         decoder_layer<T>(c, c.large, l, h, r);
         if (project) project_after<T>(c, l + 1, r);
     }
-    if (head)
-        head_argmax<T>(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.st.targets, TANDEM_GAMMA_LIMIT + 1, 0);
+}
+
+// Prompt pass of the large model.
+template <typename T>
+void large_prompt(tandem_ctx& c, const Rows& r) {
+    {
+        ProfScope ps(c, PC_ROWS, (double)r.M * c.large.d.d_model * (4.0 + 2 * sizeof(T)));
+        embed_kernel<T><<<r.M, 128, 0, c.stream>>>(at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_pos), (const T*)w_emb(c, c.large),
+                                                   (const T*)w_pos(c, c.large), at<float>(c, c.lay.h_large), c.large.d.d_model);
+        c.launches++;
+    }
+    large_layers<T>(c, r, true);
 }
 
 Rows decode_rows(tandem_ctx& c, int r_last, int nq) {
@@ -766,31 +814,36 @@ Rows decode_rows(tandem_ctx& c, int r_last, int nq) {
     return r;
 }
 
-void setup_rows(tandem_ctx& c, int r0, int nq) {
-    const int M = c.batch * nq;
-    ProfScope ps(c, PC_ROWS, (double)M * 12.0);
-    setup_rows_kernel<<<cdiv(M, 128), 128, 0, c.stream>>>(c.st, c.batch, r0, nq, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos));
-    c.launches++;
+// Row set-up + embedding for block rows r0 .. r0+nq-1 of every sequence; fin_r: block row whose token is the
+// arg-max the small model's last head GEMM left as per-tile results (-1: none).
+template <typename T>
+void begin_rows(tandem_ctx& c, const Model& m, float* h, int r0, int nq, int fin_r, float* snap = nullptr) {
+    ProfScope ps(c, PC_ROWS, (double)c.batch * nq * m.d.d_model * 8.0);
+    launch_ex(c, true, 1, step_begin_kernel<T>, dim3(c.batch * nq), dim3(128), 0, c.st, r0, nq, fin_r,
+              (const float*)at<float>(c, c.lay.amax_val_small), (const int*)at<int>(c, c.lay.amax_idx_small), c.lay.vocab_tiles,
+              c.lay.vocab_tiles, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos),
+              (const T*)w_emb(c, m), (const T*)w_pos(c, m), h, m.d.d_model, snap);
 }
 
-// Draft step s: one token per sequence through the small model over the mixed context (Eq. 2, lines 2-3).
-// dst: where the step's arg-max goes (default: draft s of the loop state; a teacher-forced round keeps its given
-// drafts and sends the arg-max to the unused target array).
-template <typename T>
-void small_step(tandem_ctx& c, int s, bool keep_drafts = false) {
-    setup_rows(c, s, 1);
-    Rows r = decode_rows(c, s, 1);
+// fp32 draft step s: one token per sequence through the small model over the mixed context (Eq. 2, lines 2-3).
+// keep_drafts: a teacher-forced round keeps its given drafts and sends the step's arg-max to the unused target array.
+void fp32_small_step(tandem_ctx& c, int s, bool keep_drafts = false) {
     float* y = at<float>(c, c.lay.h_small);
-    {
-        ProfScope ps(c, PC_ROWS, (double)r.M * c.small.d.d_model * (4.0 + 2 * sizeof(T)));
-        embed_kernel<T><<<r.M, 128, 0, c.stream>>>(at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_pos), (const T*)w_emb(c, c.small),
-                                                   (const T*)w_pos(c, c.small), y, c.small.d.d_model);
-        c.launches++;
-    }
-    for (int j = 0; j < c.small.d.n_layers; ++j) decoder_layer<T>(c, c.small, j, y, r);
+    begin_rows<float>(c, c.small, y, s, 1, -1);
+    const Rows r = decode_rows(c, s, 1);
+    for (int j = 0; j < c.small.d.n_layers; ++j) decoder_layer<float>(c, c.small, j, y, r);
     float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
-    if (keep_drafts) head_argmax<T>(c, c.small, y, r, logits, c.st.targets, TANDEM_GAMMA_LIMIT + 1, s);
-    else head_argmax<T>(c, c.small, y, r, logits, c.st.drafts, TANDEM_GAMMA_LIMIT, s);
+    if (keep_drafts) head_argmax(c, c.small, y, r, logits, c.st.targets, TANDEM_GAMMA_LIMIT + 1, s);
+    else head_argmax(c, c.small, y, r, logits, c.st.drafts, TANDEM_GAMMA_LIMIT, s);
+}
+
+// fp32 block pass of the large model over nq rows per sequence; head: final LayerNorm + output head + arg-max.
+void fp32_large_block(tandem_ctx& c, int nq, bool project, bool head) {
+    float* h = at<float>(c, c.lay.h_large);
+    begin_rows<float>(c, c.large, h, 0, nq, -1);
+    const Rows r = decode_rows(c, nq - 1, nq);
+    large_layers<float>(c, r, project);
+    if (head) head_argmax(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.st.targets, TANDEM_GAMMA_LIMIT + 1, 0);
 }
 
 // Teacher-forced round (accept mode 5): the given tokens become the round's drafts; after the draft steps their
@@ -849,30 +902,22 @@ void launch_sample_verify(tandem_ctx& c, int gamma, uint64_t seed) {
               c.temp_large, c.temp_small, (unsigned long long)seed);
 }
 
-template <typename T>
-void iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
+void fp32_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
     if (mode == 5) launch_forced_fill(c, gamma);
     for (int s = 0; s < gamma; ++s) {
-        small_step<T>(c, s, mode == 5);
+        fp32_small_step(c, s, mode == 5);
         if (mode == 4) launch_sample_draft(c, s, seed);   // replaces the arg-max draft of this step
     }
     if (mode == 5) launch_score_rows(c, gamma);
-    if (mode == 3 || mode == 5) {   // stand-alone Tandem without the free token: gamma rows, no output head
-        setup_rows(c, 0, gamma);
-        large_pass<T>(c, decode_rows(c, gamma - 1, gamma), true, false);
-    } else {
-        setup_rows(c, 0, gamma + 1);
-        large_pass<T>(c, decode_rows(c, gamma, gamma + 1), true, true);
-    }
+    if (mode == 3 || mode == 5) fp32_large_block(c, gamma, true, false);   // stand-alone Tandem without the free token: gamma rows, no output head
+    else fp32_large_block(c, gamma + 1, true, true);
     if (mode == 4) launch_sample_verify(c, gamma, seed);
     launch_verify(c, gamma, mode == 5 ? 3 : mode, seed, max_new, false);
     c.last_gamma = gamma;
 }
 
-template <typename T>
-void greedy_iteration(tandem_ctx& c, int max_new) {
-    setup_rows(c, 0, 1);
-    large_pass<T>(c, decode_rows(c, 0, 1), false, true);
+void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
+    fp32_large_block(c, 1, false, true);
     launch_verify(c, 0, 0, 0ull, max_new, false);
     c.last_gamma = 0;
 }
@@ -880,16 +925,6 @@ void greedy_iteration(tandem_ctx& c, int max_new) {
 // ---------------------------------------------------------------------------------------------------
 // bf16 decode on the tensor cores: five kernels per decoder layer, chained by programmatic dependent launch
 // ---------------------------------------------------------------------------------------------------
-
-// Row set-up + embedding for block rows r0 .. r0+nq-1 of every sequence; fin_r: block row whose token is the
-// arg-max the small model's last head GEMM left as per-tile results (-1: none).
-void tc_begin(tandem_ctx& c, const Model& m, float* h, int r0, int nq, int fin_r, float* snap = nullptr) {
-    ProfScope ps(c, PC_ROWS, (double)c.batch * nq * m.d.d_model * 8.0);
-    launch_ex(c, true, 1, step_begin_kernel<bf16>, dim3(c.batch * nq), dim3(128), 0, c.st, r0, nq, fin_r,
-              (const float*)at<float>(c, c.lay.amax_val_small), (const int*)at<int>(c, c.lay.amax_idx_small), c.lay.vocab_tiles,
-              c.lay.vocab_tiles, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos),
-              (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h, m.d.d_model, snap);
-}
 
 // The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = LayerNorm output, 1 = attention
 // output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width for buffer 2).
@@ -988,7 +1023,7 @@ void tc_head(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* logi
 // arg-max results.
 void tc_small_step(tandem_ctx& c, int s, bool sampled) {
     float* y = at<float>(c, c.lay.h_small);
-    tc_begin(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1);
+    begin_rows<bf16>(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1);
     const Rows r = decode_rows(c, s, 1);
     for (int j = 0; j < c.small.d.n_layers; ++j) tc_decoder_layer(c, c.small, j, y, r, false);
     float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
@@ -1048,7 +1083,7 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
         return slot >= 0 ? at<float>(c, c.lay.proj_snap) + (size_t)slot * snap_elems : nullptr;
     };
     bool any_fork = false;
-    tc_begin(c, c.large, h, 0, nq, fin_r, snap_of(0));
+    begin_rows<bf16>(c, c.large, h, 0, nq, fin_r, snap_of(0));
     const Rows r = decode_rows(c, nq - 1, nq);
     if (project && project_slot(c, 0) >= 0) { tc_project_forked(c, 0, project_slot(c, 0), r); any_fork = true; }
     for (int l = 0; l < c.large.d.n_layers; ++l) {
@@ -1107,7 +1142,7 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
     const bool bf = c.cfg.dtype == TANDEM_DTYPE_BF16;   // one bf16 path: the tensor-core kernels (a bf16 context always has tensor maps)
     if (kind == 3) {
         if (gamma == 0) launch_adaptive_begin(c);
-        if (bf) tc_small_step(c, gamma, false); else small_step<float>(c, gamma);
+        if (bf) tc_small_step(c, gamma, false); else fp32_small_step(c, gamma);
         launch_router(c, gamma, mode);
         return;
     }
@@ -1115,8 +1150,7 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
         if (bf) {
             tc_large_block(c, gamma + 1, gamma, true, true);
         } else {
-            setup_rows(c, 0, gamma + 1);
-            large_pass<float>(c, decode_rows(c, gamma, gamma + 1), true, true);
+            fp32_large_block(c, gamma + 1, true, true);
         }
         launch_verify(c, gamma, TANDEM_ACCEPT_NATURAL, 0ull, max_new, bf, true);
         c.last_gamma = gamma;
@@ -1126,8 +1160,8 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
         if (kind == 0) tc_iteration(c, gamma, mode, seed, max_new); else tc_greedy_iteration(c, max_new);
         return;
     }
-    if (kind == 0) iteration<float>(c, gamma, mode, seed, max_new);
-    else greedy_iteration<float>(c, max_new);
+    if (kind == 0) fp32_iteration(c, gamma, mode, seed, max_new);
+    else fp32_greedy_iteration(c, max_new);
 }
 
 // Enqueues one iteration on the context's stream: eagerly the first time a launch shape is seen (and whenever
@@ -1476,8 +1510,8 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     for (int q = 0; q < n_queries; ++q) c->prompt_sq_sum += (double)(prompt_lens[q] - 1) * (prompt_lens[q] - 1);
     if (M > 0) {
         Rows r; r.M = M; r.groups = groups; r.nq = 0; r.decode = false; r.n_chunks = 0; r.kv_positions = (double)rows;
-        if (c->cfg.dtype == TANDEM_DTYPE_BF16) large_pass<bf16>(*c, r, true, false);
-        else large_pass<float>(*c, r, true, false);
+        if (c->cfg.dtype == TANDEM_DTYPE_BF16) large_prompt<bf16>(*c, r);
+        else large_prompt<float>(*c, r);
     }
     TRY(check_launch(*c));
     if (samples > 1) {
