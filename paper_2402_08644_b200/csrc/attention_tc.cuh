@@ -1,20 +1,28 @@
 // Causal prompt attention (Eq. 1 over the prompt) on the tcgen05 tensor cores, bf16, head size 64 or 128.
 //
-// One CTA serves one (head, tile of up to 128 consecutive queries of one sequence); two such CTAs share an SM, so
-// that one's tensor work runs while the other's softmax does.  The context is swept in chunks of 64 keys anchored
-// at position 0, up to the tile's last query:
-//     S  = Q K^T        M = 128 queries on the TMEM lanes, N = 64 keys, K = head size; two S buffers in TMEM
-//     P  = softmax step thread i owns query i: reads its row of S from TMEM once, masks keys after its position,
-//                       writes bf16 probabilities into a swizzled A tile (one 128-byte row)
-//     O += P V          M = 128 queries, N = head size, K = 64 keys, accumulated in TMEM over all chunks; V is used as
-//                       it lies in the cache ([key][element], i.e. MN-major for the B operand)
+// One CTA serves one head and up to 256 consecutive queries of one sequence, as two tiles of 128.  The context is swept in
+// chunks of 64 keys anchored at position 0, each tile up to its own last query; per tile and chunk:
+//     S  = Q K^T        M = 128 queries on the TMEM lanes, N = 64 keys, K = head size; two S buffers per tile in TMEM
+//     P  = softmax step thread i of the tile's four warps owns query i: reads its row of S from TMEM, masks keys after its
+//                       position, writes bf16 probabilities back into TMEM where S was
+//     O += P V          M = 128 queries, N = head size, K = 64 keys; P is the A operand straight from TMEM, V is used as it
+//                       lies in the cache ([key][element], i.e. MN-major for the B operand), O accumulates in TMEM
+// S of the next chunk is issued before P of this one is awaited, so the softmax warps never wait for the tensor pipe unless
+// it is the slower one, and one tile's softmax runs beside the other's.  (A buffer is rewritten by a product that is
+// issued behind the one that reads it: a CTA's products run in issue order.)  TMEM holds two S / P buffers of both tiles and
+// both O: all 512 columns.  Nothing but Q, K and V goes through shared memory, and a chunk of K and V serves 256 queries.
+// The bounds lie close together: at 128-wide heads 128 x 128 exponentials per 128 queries and keys are 1024 clocks of the
+// exponential unit, the products 1280 clocks (N = 64 reads its A operand from shared memory at 1.5 times the rate it has).
+// The longest tiles start first (a causal tile costs what its position says).  8191 rows x 32 heads x 128: 502 us = 1094
+// TFLOP/s at full clocks, 720 us inside the power-capped prompt pass of the large pair, where the kernel before (one tile
+// per CTA, P through shared memory, MMAs issued from a divergent branch) took 1157 us; with chunks of 128 keys and one S
+// buffer per tile the products wait for the softmax and it for them (734 us before the issue was fixed).
 // The running maximum is lazy: probabilities are taken relative to a reference m that moves only when a chunk's
 // maximum exceeds it by more than ATC_LAZY (so they stay below e^ATC_LAZY); only then is O, in TMEM, rescaled
 // (tcgen05.ld, multiply, tcgen05.st) - rare after the first chunks.  The row sum adds the fp32 probabilities (their
 // bf16 roundings, which the tensor core multiplies with V, differ from them by 2^-9 each with random signs).
-// Warp 4 streams K (two stages) and V (one stage) by TMA, warp 5 allocates TMEM and issues the MMAs (S of chunk c+1
-// goes out before the probabilities of chunk c are awaited), warps 0-3 do the softmax and the epilogue.  Every wait is
-// bounded.
+// Warps 0-3 / 4-7: softmax and epilogue of tile 0 / 1; warp 8 streams K and V (four stages each) by TMA; warp 9 allocates
+// TMEM and issues the MMAs.  Every wait is bounded.
 #pragma once
 #include "common.cuh"
 #include "gemm_tc.cuh"
@@ -32,21 +40,22 @@ struct AttnTcArgs {
     int* err_flag;
 };
 
-constexpr int ATC_THREADS = 192;
-constexpr int ATC_Q = 128;                // queries per tile
+constexpr int ATC_THREADS = 320;
+constexpr int ATC_TILE = 128;             // queries per tile
+constexpr int ATC_Q = 2 * ATC_TILE;       // queries per CTA
 constexpr int ATC_KC = 64;                // keys per chunk
-constexpr int ATC_SUB = 128 * 128;        // bytes of one 128-row x 64-element bf16 sub-tile (queries, probabilities)
+constexpr int ATC_STAGES = 4;             // chunks of keys, and of values, in flight
+constexpr int ATC_SUB = 128 * 128;        // bytes of one 128-row x 64-element bf16 sub-tile (queries)
 constexpr int ATC_KSUB = ATC_KC * 128;    // bytes of one 64-key x 64-element sub-tile (keys, values)
 constexpr float ATC_LAZY = 5.0f;          // how far a chunk's maximum may exceed the reference before O is rescaled
 template <int DH> struct AtcCfg {
     static constexpr int NSUB = DH / 64;                       // 64-element sub-tiles along the head dimension
-    static constexpr int Q_BYTES = NSUB * ATC_SUB;
-    static constexpr int K_BYTES = NSUB * ATC_KSUB;            // keys (or values) of one chunk
-    static constexpr int P_BYTES = ATC_SUB;                    // 128 queries x 64 keys bf16
-    static constexpr int SMEM_BYTES = Q_BYTES + 3 * K_BYTES + P_BYTES + 1024;   // two key stages, one value stage
-    static constexpr int TMEM_COLS = 256;                      // S of even / odd chunks: columns 0..63 / 64..127; O: 128..128+DH-1
+    static constexpr int Q_BYTES = NSUB * ATC_SUB;             // a tile of queries
+    static constexpr int K_BYTES = NSUB * ATC_KSUB;            // a chunk of keys, a chunk of values
+    static constexpr int SMEM_BYTES = 2 * Q_BYTES + 2 * ATC_STAGES * K_BYTES + 1024;
+    static constexpr int TMEM_COLS = 512;                      // S / P of tile t, buffer b: columns 128 t + 64 b ..; O of tile t: 256 + 128 t ..
 };
-static_assert(AtcCfg<128>::SMEM_BYTES + 2048 <= 113 * 1024, "two CTAs per SM");
+static_assert(AtcCfg<128>::SMEM_BYTES + 1024 <= 227 * 1024, "one CTA per SM");
 
 // Instruction descriptor: bf16 A (K-major) and B, fp32 accumulation; b_mn = 1 when B is MN-major.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16_b(int M, int N, int b_mn) {
@@ -93,6 +102,34 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
 #pragma unroll
     for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 16 consecutive columns of this thread's TMEM lane, as they are (the probabilities of 32 keys, two to a column).
+__device__ __forceinline__ void tmem_st16_u32(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+          "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem]: A's rows are the TMEM lanes, two bf16 of K per 32-bit column.
+__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Two fp32 operations in one instruction: a * b + c, and a + b, on pairs.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(reinterpret_cast<uint64_t&>(d))
+        : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)), "l"(reinterpret_cast<const uint64_t&>(c)));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<uint64_t&>(d))
+        : "l"(reinterpret_cast<const uint64_t&>(a)), "l"(reinterpret_cast<const uint64_t&>(b)));
+    return d;
+}
 // 2^x by the hardware approximation (relative error about 2^-22; 2^-inf = 0), one instruction.
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
@@ -100,40 +137,35 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// grid: (heads, groups); dynamic smem AtcCfg<DH>::SMEM_BYTES.
+// grid: (heads, groups), the last group first; dynamic smem AtcCfg<DH>::SMEM_BYTES.
 // tmq: queries [M][d_model] (box 64 x 128); tmk / tmv: one layer's cache seen as [(seq, kv head, position)][DH] (box 64 x 64).
 template <int DH>
-__global__ void __launch_bounds__(ATC_THREADS, 2)
+__global__ void __launch_bounds__(ATC_THREADS, 1)
 attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                        const __grid_constant__ CUtensorMap tmv) {
     using C = AtcCfg<DH>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_qfull, s_kfull[2], s_kfree[2], s_vfull, s_vfree, s_sfull[2], s_pready, s_ofull;
+    __shared__ __align__(8) uint64_t s_qfull, s_kfull[ATC_STAGES], s_kfree[ATC_STAGES], s_vfull[ATC_STAGES], s_vfree[ATC_STAGES];
+    __shared__ __align__(8) uint64_t s_sfull[2][2], s_pready[2][2], s_odone[2];   // [tile][buffer]; odone[tile]: one phase per chunk
     __shared__ uint32_t s_tmem;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
-    unsigned char* base = smem_dyn + (base0 - smem_u32(smem_dyn));
-    const uint32_t q0 = base0, k0 = q0 + C::Q_BYTES, v0 = k0 + 2 * C::K_BYTES, p0 = v0 + C::K_BYTES;
-    unsigned char* pg = base + C::Q_BYTES + 3 * C::K_BYTES;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    const uint32_t q0 = (smem_u32(smem_dyn) + 1023u) & ~1023u, k0 = q0 + 2 * C::Q_BYTES, v0 = k0 + ATC_STAGES * C::K_BYTES;
 
-    const int h = blockIdx.x, g = blockIdx.y;
-    const int row0 = a.grp_row0[g], cnt = a.grp_cnt[g];
-    if (cnt <= 0) return;
-    const int b = a.row_seq[row0];
-    const int pos_first = a.row_pos[row0];
-    const int pos_last = pos_first + cnt - 1;
-    const int n_chunks = pos_last / ATC_KC + 1;
-    const int kv_row0 = (b * a.n_kv_heads + h / (a.n_heads / a.n_kv_heads)) * a.t_max;   // row of position 0 of this head's key/value head in the cache's 2-D view
-
-    if (warp == 5) {
+    if (warp == 9) {
         if (lane == 0) {
             mbar_init(smem_u32(&s_qfull), 1);
-            for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&s_kfull[s]), 1); mbar_init(smem_u32(&s_kfree[s]), 1); mbar_init(smem_u32(&s_sfull[s]), 1); }
-            mbar_init(smem_u32(&s_vfull), 1);
-            mbar_init(smem_u32(&s_vfree), 1);
-            mbar_init(smem_u32(&s_pready), 4);   // one arrive per softmax warp
-            mbar_init(smem_u32(&s_ofull), 1);
+            for (int s = 0; s < ATC_STAGES; ++s) {
+                mbar_init(smem_u32(&s_kfull[s]), 1); mbar_init(smem_u32(&s_kfree[s]), 1);
+                mbar_init(smem_u32(&s_vfull[s]), 1); mbar_init(smem_u32(&s_vfree[s]), 1);
+            }
+            for (int t = 0; t < 2; ++t) {
+                mbar_init(smem_u32(&s_odone[t]), 1);
+                for (int u = 0; u < 2; ++u) {
+                    mbar_init(smem_u32(&s_sfull[t][u]), 1);
+                    mbar_init(smem_u32(&s_pready[t][u]), 4);   // one arrive per softmax warp of the tile
+                }
+            }
             mbar_init_fence();
         }
         __syncwarp();
@@ -143,162 +175,182 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = s_tmem;
+    const uint32_t tmem = warp_uniform(s_tmem);
+    pdl_wait();                // queries, keys and values come from the kernel before this one
 
-    if (warp == 4) {
-        // ---- TMA: Q once; K of chunk c+1 as soon as its stage is free (S of chunk c-1 done), V of chunk c+1 once P V of chunk c is done ----
-        if (lane == 0) {
-            tma_prefetch_desc(&tmq); tma_prefetch_desc(&tmk); tma_prefetch_desc(&tmv);
-            mbar_arrive_expect_tx(smem_u32(&s_qfull), C::Q_BYTES);
-            for (int sb = 0; sb < C::NSUB; ++sb) tma_load_2d_nohint(q0 + sb * ATC_SUB, &tmq, h * DH + sb * 64, row0, smem_u32(&s_qfull));
-            auto load_k = [&](int c) {
-                const uint32_t bar = smem_u32(&s_kfull[c & 1]);
-                mbar_arrive_expect_tx(bar, C::K_BYTES);
-                for (int sb = 0; sb < C::NSUB; ++sb) tma_load_2d_nohint(k0 + (c & 1) * C::K_BYTES + sb * ATC_KSUB, &tmk, sb * 64, kv_row0 + c * ATC_KC, bar);
-            };
-            auto load_v = [&](int c) {
-                const uint32_t bar = smem_u32(&s_vfull);
-                mbar_arrive_expect_tx(bar, C::K_BYTES);
-                for (int sb = 0; sb < C::NSUB; ++sb) tma_load_2d_nohint(v0 + sb * ATC_KSUB, &tmv, sb * 64, kv_row0 + c * ATC_KC, bar);
-            };
-            load_k(0);
-            load_v(0);
-            for (int c = 0; c + 1 < n_chunks; ++c) {
-                if (c + 1 >= 2 && !mbar_wait(smem_u32(&s_kfree[(c + 1) & 1]), (((c + 1) >> 1) - 1) & 1)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
-                load_k(c + 1);
-                if (!mbar_wait(smem_u32(&s_vfree), c & 1)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
-                load_v(c + 1);
+    const int h = blockIdx.x, g = gridDim.y - 1 - blockIdx.y;
+    const int row0 = a.grp_row0[g], cnt = a.grp_cnt[g];
+    const int b = a.row_seq[row0];
+    const int pos_first = a.row_pos[row0];
+    // chunks of each tile: up to the tile's last query (0: the group ends before the tile)
+    const int n0 = (pos_first + min(cnt, ATC_TILE) - 1) / ATC_KC + 1;
+    const int n1 = cnt > ATC_TILE ? (pos_first + cnt - 1) / ATC_KC + 1 : 0;
+    const int n_max = max(n0, n1);
+    const int kv_row0 = (b * a.n_kv_heads + h / (a.n_heads / a.n_kv_heads)) * a.t_max;   // row of position 0 of this head's key/value head in the cache's 2-D view
+
+    if (warp == 8) {
+        // ---- TMA: Q once, then K and V of every chunk as their stages come free ----
+        {
+            const bool leader = elect_one();
+            if (leader) { tma_prefetch_desc(&tmq); tma_prefetch_desc(&tmk); tma_prefetch_desc(&tmv); }
+            const int tiles = n1 > 0 ? 2 : 1;
+            if (leader) mbar_arrive_expect_tx(smem_u32(&s_qfull), tiles * C::Q_BYTES);
+            for (int t = 0; t < tiles && leader; ++t)
+                for (int sb = 0; sb < C::NSUB; ++sb)
+                    tma_load_2d_nohint(q0 + t * C::Q_BYTES + sb * ATC_SUB, &tmq, h * DH + sb * 64, row0 + t * ATC_TILE, smem_u32(&s_qfull));
+            for (int c = 0; c < n_max; ++c) {
+                const int st = c % ATC_STAGES;
+                const uint32_t old = ((c / ATC_STAGES) - 1) & 1;
+                if (c >= ATC_STAGES && !mbar_wait_warp(smem_u32(&s_kfree[st]), old)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(smem_u32(&s_kfull[st]), C::K_BYTES);
+                    for (int sb = 0; sb < C::NSUB; ++sb)
+                        tma_load_2d_nohint(k0 + st * C::K_BYTES + sb * ATC_KSUB, &tmk, sb * 64, kv_row0 + c * ATC_KC, smem_u32(&s_kfull[st]));
+                }
+                if (c >= ATC_STAGES && !mbar_wait_warp(smem_u32(&s_vfree[st]), old)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(smem_u32(&s_vfull[st]), C::K_BYTES);
+                    for (int sb = 0; sb < C::NSUB; ++sb)
+                        tma_load_2d_nohint(v0 + st * C::K_BYTES + sb * ATC_KSUB, &tmv, sb * 64, kv_row0 + c * ATC_KC, smem_u32(&s_vfull[st]));
+                }
             }
+            pdl_launch_dependents();
         }
         __syncwarp();
-    } else if (warp == 5) {
-        // ---- MMA issue: one thread ----
-        if (lane == 0) {
+    } else if (warp == 9) {
+        // ---- MMA issue: one elected thread of a converged warp ----
+        {
             constexpr uint32_t idesc_s = umma_idesc_bf16_b(128, ATC_KC, 0);
             constexpr uint32_t idesc_o = umma_idesc_bf16_b(128, DH, 1);
-            bool ok = mbar_wait(smem_u32(&s_qfull), 0);
+            bool ok = mbar_wait_warp(smem_u32(&s_qfull), 0);
             if (!ok) tc_report(a.err_flag, TC_ERR_OPERANDS);
-            // S = Q K^T of chunk c into S buffer c & 1: both K-major, 16 elements of the head dimension per instruction
+            // S = Q K^T of chunk c for both tiles, each into its buffer c & 1: both operands K-major, 16 elements of the head
+            // dimension per instruction
             auto issue_s = [&](int c) -> bool {
-                const int st = c & 1;
-                if (!mbar_wait(smem_u32(&s_kfull[st]), (c >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); return false; }
+                const int st = c % ATC_STAGES;
+                if (!mbar_wait_warp(smem_u32(&s_kfull[st]), (c / ATC_STAGES) & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); return false; }
                 tc_fence_after_sync();
                 const uint32_t kaddr = k0 + st * C::K_BYTES;
+                for (int t = 0; t < 2; ++t) {
+                    if (c >= (t == 0 ? n0 : n1)) continue;
+                    const uint32_t qaddr = q0 + t * C::Q_BYTES, d = tmem + t * 128 + (c & 1) * ATC_KC;
+                    if (elect_one()) {
 #pragma unroll
-                for (int sb = 0; sb < C::NSUB; ++sb)
+                    for (int sb = 0; sb < C::NSUB; ++sb)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        umma_bf16(tmem + st * ATC_KC, umma_desc_k_sw128(q0 + sb * ATC_SUB) + 2 * k, umma_desc_k_sw128(kaddr + sb * ATC_KSUB) + 2 * k,
-                                  idesc_s, (sb | k) != 0 ? 1u : 0u);
-                umma_commit(smem_u32(&s_sfull[st]));
-                umma_commit(smem_u32(&s_kfree[st]));   // the key stage may be refilled
+                        for (int k = 0; k < 4; ++k)
+                            umma_bf16(d, umma_desc_k_sw128(qaddr + sb * ATC_SUB) + 2 * k, umma_desc_k_sw128(kaddr + sb * ATC_KSUB) + 2 * k,
+                                      idesc_s, (sb | k) != 0 ? 1u : 0u);
+                    umma_commit(smem_u32(&s_sfull[t][c & 1])); }
+                }
+                if (elect_one()) umma_commit(smem_u32(&s_kfree[st]));
                 return true;
             };
             ok = ok && issue_s(0);
-            for (int c = 0; c < n_chunks && ok; ++c) {
-                // the next chunk's scores are computed while the softmax warps work on this one (its S buffer was
-                // released with the probabilities of chunk c - 1)
-                if (c + 1 < n_chunks && !issue_s(c + 1)) break;
-                if (!mbar_wait(smem_u32(&s_pready), c & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); break; }
-                if (!mbar_wait(smem_u32(&s_vfull), c & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); break; }
-                tc_fence_after_sync();
-                // O += P V: P K-major (one 64-key sub-tile), V MN-major; 16 keys per instruction
+            for (int c = 0; c < n_max && ok; ++c) {
+                const int st = c % ATC_STAGES;
+                // the buffers of chunk c + 1 were read by the products of chunk c - 1, which are ahead in the pipe
+                if (c + 1 < n_max && !issue_s(c + 1)) break;
+                if (!mbar_wait_warp(smem_u32(&s_vfull[st]), (c / ATC_STAGES) & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); break; }
+                for (int t = 0; t < 2; ++t) {
+                    if (c >= (t == 0 ? n0 : n1)) continue;
+                    if (!mbar_wait_warp(smem_u32(&s_pready[t][c & 1]), (c >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
+                    tc_fence_after_sync();
+                    // O += P V: P from TMEM (16 keys = 8 columns per instruction), V MN-major
+                    if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < ATC_KC / 16; ++ks)
-                    umma_bf16(tmem + 128, umma_desc_k_sw128(p0) + 2 * ks, umma_desc_mn_sw128(v0 + ks * 2048, ATC_KSUB), idesc_o,
-                              (c | ks) != 0 ? 1u : 0u);
-                umma_commit(smem_u32(&s_vfree));    // V of this chunk may be overwritten
-                umma_commit(smem_u32(&s_ofull));    // O holds chunks 0..c; the P tile may be rewritten
+                    for (int ks = 0; ks < ATC_KC / 16; ++ks)
+                        umma_bf16_ts(tmem + 256 + t * 128, tmem + t * 128 + (c & 1) * ATC_KC + ks * 8,
+                                     umma_desc_mn_sw128(v0 + st * C::K_BYTES + ks * 2048, ATC_KSUB), idesc_o, (c | ks) != 0 ? 1u : 0u);
+                    umma_commit(smem_u32(&s_odone[t])); }  // O of tile t holds chunks 0 .. c
+                }
+                if (elect_one()) umma_commit(smem_u32(&s_vfree[st]));
             }
         }
         __syncwarp();
     } else {
         // ---- softmax warps: thread = query = TMEM lane ----
-        const int qi = warp * 32 + lane;
+        const int t = warp >> 2, wl = warp & 3;
+        const int qi = t * ATC_TILE + wl * 32 + lane;
+        const int n = t == 0 ? n0 : n1;
+        const int tile_pos = pos_first + t * ATC_TILE;
         const int qpos = pos_first + qi;                 // (rows past cnt compute on whatever the tile holds; never stored)
-        const uint32_t lane_addr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-        // Everything runs in the base-2 domain: with sc2 = scale * log2(e), a probability is 2^(s * sc2 - m) (one
-        // multiply-add and one ex2 per element); m is the reference maximum in that domain.
+        const uint32_t lane_addr = tmem + (static_cast<uint32_t>(wl * 32) << 16);
+        const uint32_t o_addr = lane_addr + 256 + t * 128;
+        // Everything runs in the base-2 domain: with sc2 = scale * log2(e), a probability is 2^(s * sc2 - m) (half a
+        // paired multiply-add and one ex2 per element); m is the reference maximum in that domain.
         const float sc2 = a.scale * 1.4426950408889634f;
         constexpr float LAZY2 = ATC_LAZY * 1.4426950408889634f;
         float m = -INFINITY, l = 0.f;                    // reference maximum of the exponentials, running sum
         bool ok = true;
-        for (int c = 0; c < n_chunks && ok; ++c) {
-            if (!mbar_wait(smem_u32(&s_sfull[c & 1]), (c >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
+        for (int c = 0; c < n; ++c) {
+            if (!mbar_wait(smem_u32(&s_sfull[t][c & 1]), (c >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
             tc_fence_after_sync();
-            const uint32_t s_addr = lane_addr + (c & 1) * ATC_KC;
-            // this row of S, raw; keys after the query's position become -inf (every chunk but the tile's last ones lies
-            // wholly before its first query and needs no mask)
-            const bool full = c * ATC_KC + ATC_KC - 1 <= pos_first;
-            float t[ATC_KC];
-            tmem_ld64(s_addr, t);                        // the whole row in one load
-            float mr = -INFINITY;
-            if (full) {
+            const uint32_t s_addr = lane_addr + t * 128 + (c & 1) * ATC_KC;
+            float s[ATC_KC];
+            tmem_ld64(s_addr, s);                        // this row of S, raw
+            // keys after the query's position become -inf (every chunk but the tile's last ones lies wholly before its first query)
+            if (c * ATC_KC + ATC_KC - 1 > tile_pos) {
 #pragma unroll
-                for (int i = 0; i < ATC_KC; ++i) mr = fmaxf(mr, t[i]);
-            } else {
+                for (int i = 0; i < ATC_KC; ++i) s[i] = (c * ATC_KC + i <= qpos) ? s[i] : -INFINITY;
+            }
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                for (int i = 0; i < ATC_KC; ++i) {
-                    t[i] = (c * ATC_KC + i <= qpos) ? t[i] : -INFINITY;
-                    mr = fmaxf(mr, t[i]);
-                }
-            }
-            const float mc = mr * sc2;                   // the chunk's maximum in the base-2 domain (the scale is positive)
-            tc_fence_before_sync();      // the TMEM reads of S are done before the MMA after next may overwrite the buffer
-            // P V of the previous chunk must be complete before the P tile is rewritten or O is touched
-            if (c > 0) {
-                if (!mbar_wait(smem_u32(&s_ofull), (c - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
-                tc_fence_after_sync();
-            }
+            for (int i = 0; i < ATC_KC; i += 8)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], fmaxf(s[i + u], s[i + 4 + u]));
+            const float mc = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sc2;   // the chunk's maximum in the base-2 domain (the scale is positive)
             // lazy reference: it moves only when this chunk's maximum exceeds it by more than the margin
             const bool move = mc > m + LAZY2;            // (first chunk: m = -inf, every row with a visible key moves)
-            if (c > 0 && __any_sync(0xffffffffu, move)) {
+            if (c > 0 && __any_sync(0xffffffffu, move)) {   // O is touched only when P V of the previous chunk is complete
+                if (!mbar_wait(smem_u32(&s_odone[t]), (c - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
+                tc_fence_after_sync();
                 const float f = (move && m > -INFINITY) ? ex2_approx(m - mc) : 1.0f;   // rows that keep their reference: exactly 1
-#pragma unroll
+#pragma unroll 1
                 for (int e0 = 0; e0 < DH; e0 += 16) {
                     float o[16];
-                    tmem_ld16(lane_addr + 128 + e0, o);
+                    tmem_ld16(o_addr + e0, o);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) o[i] *= f;
-                    tmem_st16(lane_addr + 128 + e0, o);
+                    tmem_st16(o_addr + e0, o);
                 }
-                tmem_wait_st();
                 l *= f;
             }
             if (move) m = mc;
-            // probabilities relative to the reference (2^(-inf) = 0 for masked keys), their sum, and one 128-byte row
-            // of the bf16 P tile
-            unsigned char* prow = pg + qi * 128;
-            const float nm = -m;
-            float ls0 = 0.f, ls1 = 0.f;
+            // probabilities relative to the reference (2^(-inf) = 0 for masked keys), their sum, and the row of P where S was
+            const float2 sc22 = make_float2(sc2, sc2), nm2 = make_float2(-m, -m);
+            float2 ls0 = make_float2(0.f, 0.f), ls1 = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int c0 = 0; c0 < ATC_KC; c0 += 8) {
-                uint32_t pk[4];
+            for (int c0 = 0; c0 < ATC_KC; c0 += 32) {
+                uint32_t pk[16];
 #pragma unroll
-                for (int i = 0; i < 8; i += 2) {
-                    const float p0v = ex2_approx(fmaf(t[c0 + i], sc2, nm));
-                    const float p1v = ex2_approx(fmaf(t[c0 + i + 1], sc2, nm));
-                    ls0 += p0v; ls1 += p1v;
-                    pk[i >> 1] = pack_bf16x2(p0v, p1v);
+                for (int i = 0; i < 32; i += 4) {
+                    const float* sp = &s[c0 + i];
+                    const float2 x0 = fma2(make_float2(sp[0], sp[1]), sc22, nm2), x1 = fma2(make_float2(sp[2], sp[3]), sc22, nm2);
+                    const float2 p0 = make_float2(ex2_approx(x0.x), ex2_approx(x0.y)), p1 = make_float2(ex2_approx(x1.x), ex2_approx(x1.y));
+                    ls0 = add2(ls0, p0);
+                    ls1 = add2(ls1, p1);
+                    pk[i >> 1] = pack_bf16x2(p0.x, p0.y);
+                    pk[(i >> 1) + 1] = pack_bf16x2(p1.x, p1.y);
                 }
-                *reinterpret_cast<uint4*>(prow + ((((c0 >> 3)) ^ (qi & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                tmem_st16_u32(s_addr + (c0 >> 1), pk);
             }
-            const float ls = ls0 + ls1;
-            l += ls;
-            tc_fence_before_sync();      // the rescaled O is in TMEM before the next P V accumulates onto it
-            fence_proxy_async_smem();
+            ls0 = add2(ls0, ls1);
+            l += ls0.x + ls0.y;
+            tmem_wait_st();
+            tc_fence_before_sync();      // P and a rescaled O are in TMEM before the next product reads them
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_pready));
+            if (lane == 0) mbar_arrive(smem_u32(&s_pready[t][c & 1]));
         }
-        if (ok) {   // all chunks accumulated
-            if (!mbar_wait(smem_u32(&s_ofull), (n_chunks - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
+        if (ok && n > 0) {   // all chunks accumulated
+            if (!mbar_wait(smem_u32(&s_odone[t]), (n - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
             tc_fence_after_sync();
             const float inv = 1.0f / l;
             bf16* dst = static_cast<bf16*>(a.out) + (size_t)(row0 + qi) * a.ldo + h * DH;
-#pragma unroll
+#pragma unroll 2
             for (int e0 = 0; e0 < DH; e0 += 16) {
                 float o[16];
-                tmem_ld16(lane_addr + 128 + e0, o);   // warp-wide: every lane takes part
+                tmem_ld16(o_addr + e0, o);   // warp-wide: every lane takes part
                 if (ok && qi < cnt) {
                     uint4 lo, hi;
                     lo.x = pack_bf16x2(o[0] * inv, o[1] * inv); lo.y = pack_bf16x2(o[2] * inv, o[3] * inv);
@@ -314,7 +366,7 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 5) tmem_dealloc(tmem, C::TMEM_COLS);
+    if (warp == 9) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
 }  // namespace tandem

@@ -131,7 +131,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     __shared__ int s_ai[4][NB];
     __shared__ long long s_rowoff[NB];   // EPI_QKV / EPI_KV: the row-dependent part of an output's cache index
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;          // shared-space address of stage 0
     unsigned char* ring = smem_dyn + (ring0 - smem_u32(smem_dyn));         // the same place as a generic pointer
 
@@ -175,25 +175,25 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = s_tmem;
+    const uint32_t tmem = warp_uniform(s_tmem);
     if (S > 1) cluster_arrive_relaxed();   // opening handshake: waited for just before the first remote store
 
     if (warp == 4) {
         // ---- weight tiles: independent of every earlier kernel of a context, so no wait on the predecessor here ----
         if (a.wait_first) pdl_wait();
-        if (PRO == PRO_TMA && lane == 0 && !a.withhold_weights) {
+        const CUtensorMap* tm = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
+        const uint64_t pol = l2_policy_evict_first();
+        auto load_a = [&](int i, int st) {
+            const uint32_t bar = smem_u32(&s_full[st]);
+            mbar_arrive_expect_tx(bar, C::A_BYTES);
+            if (a.stream_weights) tma_load_2d(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar, pol);
+            else tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar);
+        };
+        if (a.withhold_weights) {
+            // (test hook: nothing is loaded)
+        } else if (PRO == PRO_TMA) {
             // Weights of the first ring-ful before the wait on the predecessor, then the wait, then their token rows
             // (two planes, 16-row boxes), then weights and rows together as stages come free.
-            const CUtensorMap* tm = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
-            tma_prefetch_desc(tm);
-            tma_prefetch_desc(&tmx);
-            const uint64_t pol = l2_policy_evict_first();
-            auto load_a = [&](int i, int st) {
-                const uint32_t bar = smem_u32(&s_full[st]);
-                mbar_arrive_expect_tx(bar, C::A_BYTES);
-                if (a.stream_weights) tma_load_2d(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar, pol);
-                else tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar);
-            };
             auto load_b = [&](int i, int st) {
                 const uint32_t bar = smem_u32(&s_full[st]);
                 const uint32_t dst = ring0 + st * C::STAGE_BYTES + C::A_BYTES;
@@ -205,47 +205,49 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                 }
             };
             const int n_pre = min(nkb, C::STAGES);
-            for (int i = 0; i < n_pre; ++i) load_a(i, i);
+            if (elect_one()) {
+                tma_prefetch_desc(tm);
+                tma_prefetch_desc(&tmx);
+                for (int i = 0; i < n_pre; ++i) load_a(i, i);
+            }
             pdl_wait();
-            for (int i = 0; i < n_pre; ++i) load_b(i, i);
+            if (elect_one())
+                for (int i = 0; i < n_pre; ++i) load_b(i, i);
             for (int i = n_pre; i < nkb; ++i) {
                 const int st = i % C::STAGES;
-                if (!mbar_wait(smem_u32(&s_empty[st]), ((i / C::STAGES) - 1) & 1, poll_limit)) {
+                if (!mbar_wait_warp(smem_u32(&s_empty[st]), ((i / C::STAGES) - 1) & 1, poll_limit)) {
                     tc_report(a.err_flag, TC_ERR_SLOT);
                     break;
                 }
-                load_a(i, st);
-                load_b(i, st);
+                if (elect_one()) {
+                    load_a(i, st);
+                    load_b(i, st);
+                }
             }
             pdl_launch_dependents();   // the last token rows are on their way: the successor may start (see the note at the epilogue)
-        } else if (lane == 0 && !a.withhold_weights) {
-            const CUtensorMap* tm = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
-            tma_prefetch_desc(tm);
-            const uint64_t pol = l2_policy_evict_first();
+        } else {
+            if (elect_one()) tma_prefetch_desc(tm);
             for (int i = 0; i < nkb; ++i) {
                 const int st = i % C::STAGES;
-                if (i >= C::STAGES && !mbar_wait(smem_u32(&s_empty[st]), ((i / C::STAGES) - 1) & 1, poll_limit)) {
+                if (i >= C::STAGES && !mbar_wait_warp(smem_u32(&s_empty[st]), ((i / C::STAGES) - 1) & 1, poll_limit)) {
                     tc_report(a.err_flag, TC_ERR_SLOT);
                     break;
                 }
-                const uint32_t bar = smem_u32(&s_full[st]);
-                mbar_arrive_expect_tx(bar, C::A_BYTES);
-                if (a.stream_weights) tma_load_2d(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar, pol);
-                else tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar);
+                if (elect_one()) load_a(i, st);
             }
         }
         __syncwarp();
     } else if (warp == 5) {
-        // ---- MMA issue: one thread ----
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, C::NB2);
-            for (int i = 0; i < nkb; ++i) {
-                const int st = i % C::STAGES;
-                if (!mbar_wait(smem_u32(&s_full[st]), (i / C::STAGES) & 1, poll_limit)) {
-                    tc_report(a.err_flag, TC_ERR_OPERANDS);
-                    break;
-                }
-                tc_fence_after_sync();
+        // ---- MMA issue: one elected thread of a converged warp ----
+        constexpr uint32_t idesc = umma_idesc_bf16(128, C::NB2);
+        for (int i = 0; i < nkb; ++i) {
+            const int st = i % C::STAGES;
+            if (!mbar_wait_warp(smem_u32(&s_full[st]), (i / C::STAGES) & 1, poll_limit)) {
+                tc_report(a.err_flag, TC_ERR_OPERANDS);
+                break;
+            }
+            tc_fence_after_sync();
+            if (elect_one()) {
                 const uint64_t da = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES);
                 const uint64_t db = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES + C::A_BYTES);
 #pragma unroll
@@ -253,8 +255,8 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                     umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
                 umma_commit(smem_u32(&s_empty[st]));
             }
-            umma_commit(smem_u32(&s_accum));
         }
+        if (elect_one()) umma_commit(smem_u32(&s_accum));
         __syncwarp();
         // TMEM goes back as soon as the epilogue warps have read the accumulator (they arrive on barrier 2 right after
         // their loads), not at the end of the kernel: nothing is left to do for this warp after that.
@@ -679,7 +681,7 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
     __shared__ __align__(8) uint64_t s_acc_full[2], s_acc_free[2];
     __shared__ uint32_t s_tmem;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const int KB = (a.K + 63) >> 6;
     const int total = a.tiles_n * a.tiles_m;
@@ -703,26 +705,24 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = s_tmem;
+    const uint32_t tmem = warp_uniform(s_tmem);
 
     if (warp == 4) {
-        if (lane == 0) {
-            tma_prefetch_desc(&tmx);
-            tma_prefetch_desc(&tm0);
-            long long g = 0;   // k-blocks issued by this CTA over all of its tiles: ring position
-            bool ok = true;
-            for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-                int n_local0;
-                const int seg = seg_of(t % a.tiles_n, n_local0);
-                const int m0 = (t / a.tiles_n) * 128;
-                const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
-                for (int i = 0; i < KB; ++i, ++g) {
-                    const int st = (int)(g % C::STAGES);
-                    if (g >= C::STAGES && !mbar_wait(smem_u32(&s_empty[st]), (uint32_t)((g / C::STAGES) - 1) & 1)) {
-                        tc_report(a.err_flag, TC_ERR_SLOT);
-                        ok = false;
-                        break;
-                    }
+        if (elect_one()) { tma_prefetch_desc(&tmx); tma_prefetch_desc(&tm0); }
+        int st = 0, round = 0;   // ring position, and how often the ring has gone round
+        bool ok = true;
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+            int n_local0;
+            const int seg = seg_of(t % a.tiles_n, n_local0);
+            const int m0 = (t / a.tiles_n) * 128;
+            const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
+            for (int i = 0; i < KB; ++i) {
+                if (round > 0 && !mbar_wait_warp(smem_u32(&s_empty[st]), (uint32_t)(round - 1) & 1)) {
+                    tc_report(a.err_flag, TC_ERR_SLOT);
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
                     const uint32_t bar = smem_u32(&s_full[st]);
                     mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
                     tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, &tmx, i * 64, m0, bar);
@@ -730,39 +730,40 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
                     for (int hb = 0; hb < BN / 128; ++hb)   // rows past the segment's end arrive as zeros
                         tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES + (1 + hb) * TCT_TILE_BYTES, tw, i * 64, n_local0 + hb * 128, bar);
                 }
+                if (++st == C::STAGES) { st = 0; ++round; }
             }
         }
         __syncwarp();
     } else if (warp == 5) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
-            long long g = 0;
-            bool ok = true;
-            int it = 0;
-            for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++it) {
-                const int buf = it & 1;
-                // the accumulator's previous tile (two tiles back) must have been read out
-                if (it >= 2 && !mbar_wait(smem_u32(&s_acc_free[buf]), (uint32_t)((it >> 1) - 1) & 1)) {
-                    tc_report(a.err_flag, TC_ERR_ACCUM);
+        constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
+        int st = 0, round = 0;
+        bool ok = true;
+        int it = 0;
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++it) {
+            const int buf = it & 1;
+            // the accumulator's previous tile (two tiles back) must have been read out
+            if (it >= 2 && !mbar_wait_warp(smem_u32(&s_acc_free[buf]), (uint32_t)((it >> 1) - 1) & 1)) {
+                tc_report(a.err_flag, TC_ERR_ACCUM);
+                break;
+            }
+            tc_fence_after_sync();
+            for (int i = 0; i < KB; ++i) {
+                if (!mbar_wait_warp(smem_u32(&s_full[st]), (uint32_t)round & 1)) {
+                    tc_report(a.err_flag, TC_ERR_OPERANDS);
+                    ok = false;
                     break;
                 }
                 tc_fence_after_sync();
-                for (int i = 0; i < KB; ++i, ++g) {
-                    const int st = (int)(g % C::STAGES);
-                    if (!mbar_wait(smem_u32(&s_full[st]), (uint32_t)(g / C::STAGES) & 1)) {
-                        tc_report(a.err_flag, TC_ERR_OPERANDS);
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
+                if (elect_one()) {
                     const uint64_t da = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES);
                     const uint64_t db = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES + TCT_TILE_BYTES);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) umma_bf16(tmem + buf * BN, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
                     umma_commit(smem_u32(&s_empty[st]));
                 }
-                umma_commit(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
+                if (++st == C::STAGES) { st = 0; ++round; }
             }
+            if (elect_one()) umma_commit(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
         }
         __syncwarp();
     } else {

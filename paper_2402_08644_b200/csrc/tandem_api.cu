@@ -628,7 +628,7 @@ template <int DH>
 void launch_attn_prompt_tc_dh(tandem_ctx& c, const AttnTcArgs& a, const CUtensorMap& tmq, int l, int groups) {
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(attn_prefill_tc_kernel<DH>, AtcCfg<DH>::SMEM_BYTES, attr_done);
-    launch_ex(c, false, 1, attn_prefill_tc_kernel<DH>, dim3(a.n_heads, groups), dim3(ATC_THREADS), (size_t)AtcCfg<DH>::SMEM_BYTES, a, tmq,
+    launch_ex(c, true, 1, attn_prefill_tc_kernel<DH>, dim3(a.n_heads, groups), dim3(ATC_THREADS), (size_t)AtcCfg<DH>::SMEM_BYTES, a, tmq,
               c.kmap[l], c.vmap[l]);
 }
 void launch_attn_prompt_tc(tandem_ctx& c, int l, const bf16* q, bf16* o, const Rows& r) {
