@@ -20,6 +20,8 @@
 //                          prefetch in flight (deeper chains of waiting kernels cost more than they hide).
 //  gemm_tc_tiled_kernel    many rows (prompt pass): 128 x 256 output tiles, both operands by TMA; persistent CTAs with two
 //                          accumulators in TMEM, so that a tile's epilogue runs under the next tile's MMAs.
+//  gemm_tc_split_kernel    prompt passes whose 128 x 256 tiles would leave multiprocessors idle: 128 x 128 tiles, one per
+//                          cluster of one, two or four CTAs that share the tile's K range.
 //
 // An output element's reduction order depends on (N, K) only, never on the number of rows, so a block
 // pass and a one-row pass give identical bits.
@@ -596,28 +598,26 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Many rows: 128 x 256 output tiles, A = token rows, B = weight rows, both by TMA.
+// Many rows: A = token rows, B = weight rows, both by TMA.
 // ---------------------------------------------------------------------------------------------------
 
 struct TcTiledArgs {
     int M, K, N;
-    int seg_rows0, tiles0;   // first segment: output features, tiles of BN
+    int seg_rows0, tiles0;   // first segment: output features, feature tiles
     int seg_rows, tiles_per_seg;
-    int tiles_n, tiles_m;    // BN-wide feature tiles over all segments, 128-row tiles
+    int tiles_n, tiles_m;    // feature tiles over all segments, 128-row tiles
+    int splits, stages;      // gemm_tc_split_kernel: CTAs that share a tile's K range, ring stages
     int* err_flag;
     EpiArgs e;
 };
 
 constexpr int TCT_THREADS = 192;
 constexpr int TCT_TILE_BYTES = 128 * 128;          // one TMA box: 128 rows x 64 bf16
-// BN = output features per tile: 256 when that still fills the GPU (each token-row tile read from shared memory then
-// feeds twice the MMA work of a square tile), else 128.
-template <int BN> struct TctCfg {
-    static constexpr int STAGES = BN == 256 ? 4 : 6;
-    static constexpr int STAGE_BYTES = (1 + BN / 128) * TCT_TILE_BYTES;   // token rows, then the weight rows (one box per 128)
-    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
-    static constexpr int TMEM_COLS = 2 * BN;   // two accumulators
-};
+constexpr int TCT_BN = 256;                        // output features per tile
+constexpr int TCT_STAGES = 4;
+constexpr int TCT_STAGE_BYTES = 3 * TCT_TILE_BYTES;   // token rows, then the weight rows (one box per 128)
+constexpr int TCT_SMEM_BYTES = TCT_STAGES * TCT_STAGE_BYTES + 1024;
+constexpr int TCT_GROUP_M = 16;                    // row tiles that share a sweep over the weights, see tct_tile
 
 // Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.
 template <int EPI>
@@ -666,18 +666,36 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int seg, int
     reinterpret_cast<uint4*>(dst)[1] = hi;
 }
 
-// Persistent: grid = min(tiles, SMs) CTAs, CTA b takes output tiles b, b + grid, ... (tile = (row tile, BN-wide feature
-// tile), feature tiles fastest).  The TMA ring runs on across tile boundaries, and two accumulators in TMEM alternate,
-// so that the epilogue of one tile (TMEM -> registers -> global) overlaps the MMAs of the next.
-// dynamic smem TctCfg<BN>::SMEM_BYTES.
-template <int EPI, int BN>
+// Feature tile -> (segment, first feature within it).
+__device__ __forceinline__ int tct_segment(const TcTiledArgs& a, int tile_n, int width, int& n_local0) {
+    const int seg = tile_n < a.tiles0 ? 0 : 1 + (tile_n - a.tiles0) / a.tiles_per_seg;
+    n_local0 = (seg == 0 ? tile_n : tile_n - a.tiles0 - (seg - 1) * a.tiles_per_seg) * width;
+    return seg;
+}
+// Tile number -> (row tile, feature tile).  Row tiles in groups of TCT_GROUP_M, inside a group row tiles fastest: the CTAs
+// that run at the same time share 16 row tiles and about nine feature tiles, so the weights pass through L2 once per group
+// of row tiles.  With feature tiles fastest over all of them, three row tiles met the whole matrix at a time: at 64 row tiles
+// and 12288 x 4096 weights (100 MB, about the size of L2) that is 21 passes over the weights instead of four.
+__device__ __forceinline__ void tct_tile(const TcTiledArgs& a, int t, int& tile_m, int& tile_n) {
+    const int per_group = TCT_GROUP_M * a.tiles_n;
+    const int g = t / per_group, r = t - g * per_group;
+    const int gm = min(TCT_GROUP_M, a.tiles_m - g * TCT_GROUP_M);
+    tile_n = r / gm;
+    tile_m = g * TCT_GROUP_M + r - tile_n * gm;
+}
+
+// Persistent: grid = min(tiles, SMs) CTAs, CTA b takes output tiles b, b + grid, ... in the order of tct_tile.  The TMA ring
+// runs on across tile boundaries, and two accumulators in TMEM alternate, so that the epilogue of one tile (TMEM ->
+// registers -> global) overlaps the MMAs of the next.
+// dynamic smem TCT_SMEM_BYTES.
+template <int EPI>
 __global__ void __launch_bounds__(TCT_THREADS)
 gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
                      const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2) {
-    using C = TctCfg<BN>;
+    constexpr int BN = TCT_BN;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_full[C::STAGES];
-    __shared__ __align__(8) uint64_t s_empty[C::STAGES];
+    __shared__ __align__(8) uint64_t s_full[TCT_STAGES];
+    __shared__ __align__(8) uint64_t s_empty[TCT_STAGES];
     __shared__ __align__(8) uint64_t s_acc_full[2], s_acc_free[2];
     __shared__ uint32_t s_tmem;
 
@@ -685,21 +703,15 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const int KB = (a.K + 63) >> 6;
     const int total = a.tiles_n * a.tiles_m;
-    // feature tile -> (segment, first feature within it)
-    auto seg_of = [&](int tile_n, int& n_local0) {
-        const int seg = tile_n < a.tiles0 ? 0 : 1 + (tile_n - a.tiles0) / a.tiles_per_seg;
-        n_local0 = (seg == 0 ? tile_n : tile_n - a.tiles0 - (seg - 1) * a.tiles_per_seg) * BN;
-        return seg;
-    };
 
     if (warp == 5) {
         if (lane == 0) {
-            for (int s = 0; s < C::STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            for (int s = 0; s < TCT_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
             for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&s_acc_full[s]), 1); mbar_init(smem_u32(&s_acc_free[s]), 4); }   // free: one arrive per epilogue warp
             mbar_init_fence();
         }
         __syncwarp();
-        tmem_alloc(smem_u32(&s_tmem), C::TMEM_COLS);
+        tmem_alloc(smem_u32(&s_tmem), 2 * BN);
         tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -709,12 +721,14 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
 
     if (warp == 4) {
         if (elect_one()) { tma_prefetch_desc(&tmx); tma_prefetch_desc(&tm0); }
+        pdl_wait();              // the token rows come from the kernel before this one
         int st = 0, round = 0;   // ring position, and how often the ring has gone round
         bool ok = true;
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-            int n_local0;
-            const int seg = seg_of(t % a.tiles_n, n_local0);
-            const int m0 = (t / a.tiles_n) * 128;
+            int tile_m, tile_n, n_local0;
+            tct_tile(a, t, tile_m, tile_n);
+            const int seg = tct_segment(a, tile_n, BN, n_local0);
+            const int m0 = tile_m * 128;
             const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
             for (int i = 0; i < KB; ++i) {
                 if (round > 0 && !mbar_wait_warp(smem_u32(&s_empty[st]), (uint32_t)(round - 1) & 1)) {
@@ -723,16 +737,17 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
                     break;
                 }
                 if (elect_one()) {
-                    const uint32_t bar = smem_u32(&s_full[st]);
-                    mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
-                    tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, &tmx, i * 64, m0, bar);
+                    const uint32_t bar = smem_u32(&s_full[st]), dst = ring0 + st * TCT_STAGE_BYTES;
+                    mbar_arrive_expect_tx(bar, TCT_STAGE_BYTES);
+                    tma_load_2d_nohint(dst, &tmx, i * 64, m0, bar);
 #pragma unroll
                     for (int hb = 0; hb < BN / 128; ++hb)   // rows past the segment's end arrive as zeros
-                        tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES + (1 + hb) * TCT_TILE_BYTES, tw, i * 64, n_local0 + hb * 128, bar);
+                        tma_load_2d_nohint(dst + (1 + hb) * TCT_TILE_BYTES, tw, i * 64, n_local0 + hb * 128, bar);
                 }
-                if (++st == C::STAGES) { st = 0; ++round; }
+                if (++st == TCT_STAGES) { st = 0; ++round; }
             }
         }
+        pdl_launch_dependents();
         __syncwarp();
     } else if (warp == 5) {
         constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
@@ -755,28 +770,30 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
                 }
                 tc_fence_after_sync();
                 if (elect_one()) {
-                    const uint64_t da = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES);
-                    const uint64_t db = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES + TCT_TILE_BYTES);
+                    const uint64_t da = umma_desc_k_sw128(ring0 + st * TCT_STAGE_BYTES);
+                    const uint64_t db = umma_desc_k_sw128(ring0 + st * TCT_STAGE_BYTES + TCT_TILE_BYTES);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) umma_bf16(tmem + buf * BN, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
                     umma_commit(smem_u32(&s_empty[st]));
                 }
-                if (++st == C::STAGES) { st = 0; ++round; }
+                if (++st == TCT_STAGES) { st = 0; ++round; }
             }
             if (elect_one()) umma_commit(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
         }
         __syncwarp();
     } else {
+        pdl_wait();
         int it = 0;
         for (int t = blockIdx.x; t < total; t += gridDim.x, ++it) {
             const int buf = it & 1;
-            int n_local0;
-            const int seg = seg_of(t % a.tiles_n, n_local0);
+            int tile_m, tile_n, n_local0;
+            tct_tile(a, t, tile_m, tile_n);
+            const int seg = tct_segment(a, tile_n, BN, n_local0);
             const int seg_rows = seg == 0 ? a.seg_rows0 : a.seg_rows;
             const int seg_base = seg == 0 ? 0 : a.seg_rows0 + (seg - 1) * a.seg_rows;
             if (!mbar_wait(smem_u32(&s_acc_full[buf]), (uint32_t)(it >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); break; }
             tc_fence_after_sync();
-            const int m = (t / a.tiles_n) * 128 + warp * 32 + lane;   // output row = TMEM lane
+            const int m = tile_m * 128 + warp * 32 + lane;   // output row = TMEM lane
             const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16) + buf * BN;
             if (EPI == EPI_RESID && n_local0 + BN <= seg_rows && (a.e.ldo & 3) == 0 && (seg_base & 3) == 0) {
                 // residual add on whole tiles: the old values of 64 columns are fetched together (sixteen 16-byte loads in
@@ -816,7 +833,163 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 5) tmem_dealloc(tmem, C::TMEM_COLS);
+    if (warp == 5) tmem_dealloc(tmem, 2 * BN);
+}
+
+// Prompt passes of few tiles (the small pair's 511 rows: 32 tiles of 128 x 128 for N = 1024): a tile's time is its
+// operands' way from L2 into one multiprocessor (32 KB per 64 of K at about 64 bytes a clock, twice the MMAs' time), so the
+// tile's K range is dealt to the S = 1, 2 or 4 CTAs of a cluster.  Each sends its partial sums of the columns that another
+// one finishes into that CTA's inbox (16-byte stores that count their bytes on the receiver's barrier, a lane per row, 512
+// contiguous bytes per warp and store), and CTA r finishes columns r * 128 / S ..: sums in slice order, then the
+// epilogue, which is S times shorter per CTA.  Eight epilogue warps, two per 32 rows.  One tile per cluster; with S = 1 two CTAs
+// share a multiprocessor (one's epilogue runs under the other's MMAs).
+// grid: tiles * S; dynamic smem tcs_smem_bytes(S).
+constexpr int TCS_THREADS = 320;   // warps 0-7: epilogue; warp 8: TMA; warp 9: TMEM + MMA issue
+constexpr int TCS_BN = 128;
+constexpr int TCS_STAGE_BYTES = 2 * TCT_TILE_BYTES;
+constexpr int TCS_MAX_STAGES = 4;
+constexpr int tcs_stages(int S) { return S == 1 ? 3 : 4; }
+constexpr int tcs_smem_bytes(int S) { return tcs_stages(S) * TCS_STAGE_BYTES + (S == 1 ? 0 : (S - 1) * (128 * TCS_BN * 4 / S)) + 1024; }
+static_assert(2 * (tcs_smem_bytes(1) + 1024 + 1024) <= 227 * 1024 && tcs_smem_bytes(4) + 1024 <= 227 * 1024, "two CTAs per SM without a split, one with");
+
+template <int EPI>
+__global__ void __launch_bounds__(TCS_THREADS)
+gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
+                     const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2) {
+    extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    __shared__ __align__(8) uint64_t s_full[TCS_MAX_STAGES];
+    __shared__ __align__(8) uint64_t s_empty[TCS_MAX_STAGES];
+    __shared__ __align__(8) uint64_t s_accum, s_inbox;
+    __shared__ uint32_t s_tmem;
+
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const int S = a.splits, stages = a.stages;
+    const int tile = blockIdx.x / S, sp = blockIdx.x - tile * S;           // sp = this CTA's rank in its cluster
+    int n_local0;
+    const int seg = tct_segment(a, tile % a.tiles_n, TCS_BN, n_local0);
+    const int m0 = (tile / a.tiles_n) * 128;
+    const int seg_rows = seg == 0 ? a.seg_rows0 : a.seg_rows;
+    const int seg_base = seg == 0 ? 0 : a.seg_rows0 + (seg - 1) * a.seg_rows;
+    const int KB = (a.K + 63) >> 6;
+    const int kb0 = KB * sp / S, nkb = KB * (sp + 1) / S - kb0;
+
+    if (warp == 9) {
+        if (lane == 0) {
+            for (int s = 0; s < TCS_MAX_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            mbar_init(smem_u32(&s_accum), 1);
+            mbar_init(smem_u32(&s_inbox), 1);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        tmem_alloc(smem_u32(&s_tmem), TCS_BN);
+        tmem_relinquish();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = warp_uniform(s_tmem);
+    if (S > 1) cluster_arrive_relaxed();   // opening handshake: waited for just before the first remote store
+
+    if (warp == 8) {
+        const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
+        const int n_pre = min(nkb, stages);
+        if (elect_one()) {   // weights are parameters: the first ring-ful of them before the wait on the predecessor
+            tma_prefetch_desc(&tmx);
+            tma_prefetch_desc(tw);
+            for (int i = 0; i < n_pre; ++i) {
+                const uint32_t bar = smem_u32(&s_full[i]);
+                mbar_arrive_expect_tx(bar, TCS_STAGE_BYTES);
+                tma_load_2d_nohint(ring0 + i * TCS_STAGE_BYTES + TCT_TILE_BYTES, tw, (kb0 + i) * 64, n_local0, bar);
+            }
+        }
+        pdl_wait();
+        if (elect_one())
+            for (int i = 0; i < n_pre; ++i) tma_load_2d_nohint(ring0 + i * TCS_STAGE_BYTES, &tmx, (kb0 + i) * 64, m0, smem_u32(&s_full[i]));
+        int st = 0, round = 0;
+        for (int i = n_pre; i < nkb; ++i) {
+            if (!mbar_wait_warp(smem_u32(&s_empty[st]), (uint32_t)round & 1)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
+            if (elect_one()) {
+                const uint32_t bar = smem_u32(&s_full[st]), dst = ring0 + st * TCS_STAGE_BYTES;
+                mbar_arrive_expect_tx(bar, TCS_STAGE_BYTES);
+                tma_load_2d_nohint(dst, &tmx, (kb0 + i) * 64, m0, bar);
+                tma_load_2d_nohint(dst + TCT_TILE_BYTES, tw, (kb0 + i) * 64, n_local0, bar);
+            }
+            if (++st == stages) { st = 0; ++round; }
+        }
+        pdl_launch_dependents();
+        if (S > 1) cluster_wait();
+    } else if (warp == 9) {
+        constexpr uint32_t idesc = umma_idesc_bf16(128, TCS_BN);
+        int st = 0, round = 0;
+        for (int i = 0; i < nkb; ++i) {
+            if (!mbar_wait_warp(smem_u32(&s_full[st]), (uint32_t)round & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); break; }
+            tc_fence_after_sync();
+            if (elect_one()) {
+                const uint64_t da = umma_desc_k_sw128(ring0 + st * TCS_STAGE_BYTES);
+                const uint64_t db = umma_desc_k_sw128(ring0 + st * TCS_STAGE_BYTES + TCT_TILE_BYTES);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
+                umma_commit(smem_u32(&s_empty[st]));
+            }
+            if (++st == stages) { st = 0; ++round; }
+        }
+        if (elect_one()) umma_commit(smem_u32(&s_accum));
+        if (S > 1) cluster_wait();
+    } else {
+        pdl_wait();
+        const int quarter = warp & 3, half = warp >> 2;
+        const int row = quarter * 32 + lane, m = m0 + row;   // output row = TMEM lane
+        const uint32_t acc = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+        const int CS = TCS_BN / S;                           // columns that a CTA finishes
+        const uint32_t inbox0 = ring0 + stages * TCS_STAGE_BYTES;   // [S - 1 senders][CS / 4][128 rows] of four floats
+        const uint32_t ibar = smem_u32(&s_inbox);
+        if (!mbar_wait(smem_u32(&s_accum), 0)) tc_report(a.err_flag, TC_ERR_ACCUM);
+        tc_fence_after_sync();
+        if (S > 1) {
+            cluster_wait();   // closes the opening handshake: every CTA of the cluster is running
+            if (tid == 0) mbar_arrive_expect_tx(ibar, (uint32_t)((S - 1) * 128 * CS * 4));
+            for (int q = 0; q < S; ++q) {
+                if (q == sp) continue;
+                const uint32_t slot = inbox0 + (uint32_t)(sp < q ? sp : sp - 1) * (128 * CS * 4);   // the receiver leaves itself out
+#pragma unroll 1
+                for (int c0 = half * (CS / 2); c0 < (half + 1) * (CS / 2); c0 += 16) {
+                    float v[16];
+                    tmem_ld16(acc + q * CS + c0, v);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        st_async_dsmem_f32x4(slot + (uint32_t)(((c0 >> 2) + i) * 128 + row) * 16, ibar, q, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                }
+            }
+            if (!mbar_wait(ibar, 0)) tc_report(a.err_flag, TC_ERR_EXCHANGE);
+        }
+        const float4* inbox = reinterpret_cast<const float4*>(smem_dyn + (inbox0 - smem_u32(smem_dyn)));
+#pragma unroll 1
+        for (int c0 = half * (CS / 2); c0 < (half + 1) * (CS / 2); c0 += 16) {
+            float v[16];
+            tmem_ld16(acc + sp * CS + c0, v);   // warp-wide: every lane takes part
+            if (S > 1) {
+                float t[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) t[i] = 0.f;
+                for (int q = 0; q < S; ++q) {   // slice order
+                    const float4* from = inbox + (size_t)(q < sp ? q : q - 1) * (128 * CS / 4) + (c0 >> 2) * 128 + row;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 p = q == sp ? make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]) : from[i * 128];
+                        t[4 * i] += p.x; t[4 * i + 1] += p.y; t[4 * i + 2] += p.z; t[4 * i + 3] += p.w;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = t[i];
+            }
+            const int n_local = n_local0 + sp * CS + c0;
+            if (m < a.M && n_local < seg_rows) epilogue16<EPI>(a.e, m, seg, seg_base, seg_rows, n_local, v);
+        }
+        tc_fence_before_sync();
+    }
+    __syncthreads();
+    if (warp == 9) { tc_fence_after_sync(); tmem_dealloc(tmem, TCS_BN); }
 }
 
 }  // namespace tandem

@@ -20,7 +20,7 @@ struct LoopState {
     int* counters;     // [0] iteration index since prefill (advances while sequences are live), [1] live sequences,
                        // [2] error flags, [3] max_b n_b, [4] sum_b n_b, [5] live iterations of the current call,
                        // [6] verify kernels executed since the context was created (the host's ticket),
-                       // [7] sequences still drafting (adaptive block length), [8] router launches since the prompt pass,
+                       // [7] sequences still drafting (adaptive block length), [8] router launches since the context was created,
                        // [9] CTAs of the running router launch that have finished
     volatile int* host_flags;   // mapped pinned host memory: [0] ticket, [1] live, [2] n_max, [3] n_sum, [4] iterations,
                                 // [5] router ticket, [6] sequences still drafting, [7] most tokens any live sequence still wants
@@ -32,14 +32,78 @@ struct LoopState {
     int gamma_limit;
 };
 
-// x^(0) = Emb(t) + Pos(index)  (Eq. 1); fp32 residual stream.  grid: rows; block: 128.
+// x^(0) = Emb(t) + Pos(index) of one row (Eq. 1) into the fp32 residual stream, 16 bytes of the tables at a time.
+// d is a multiple of 8.  All threads of a block of BLOCK take part.
+template <typename T, int BLOCK>
+__device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __restrict__ pr, float* __restrict__ hr, float* __restrict__ snap, int d) {
+    constexpr int VN = VecN<T>::N;
+    for (int i = threadIdx.x * VN; i < d; i += BLOCK * VN) {
+        float e[VN], p[VN];
+        load_vec(er + i, e);
+        load_vec(pr + i, p);
+#pragma unroll
+        for (int u = 0; u < VN; u += 4) {
+            const float4 v = make_float4(e[u] + p[u], e[u + 1] + p[u + 1], e[u + 2] + p[u + 2], e[u + 3] + p[u + 3]);
+            *reinterpret_cast<float4*>(hr + i + u) = v;
+            if (snap) *reinterpret_cast<float4*>(snap + i + u) = v;
+        }
+    }
+}
+
+// What a prompt pass needs on the device, staged in one copy: per query its length and its offsets among the token ids,
+// the processed rows and the attention groups ([4][n_queries]), then the ids, query after query.
+struct PromptStage {
+    const int* len; const int* id_off; const int* row_off; const int* grp_off; const int* ids;
+    int n_queries, samples, rows, group;   // sequences per query; processed rows; queries per attention group
+};
+
+// Start of a prompt pass: block m < rows sets up processed row m (token, sequence, position, its attention group if it
+// starts one) and embeds it; the last block sets the loop state of every sequence.  The tickets are the host's counts of
+// the verify and router kernels it has enqueued, which the device's counts equal by then.
+// grid: rows + 1; block: 128.
 template <typename T>
-__global__ void embed_kernel(const int* __restrict__ row_tok, const int* __restrict__ row_pos, const T* __restrict__ emb,
-                             const T* __restrict__ pos, float* __restrict__ h, int d) {
+__global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptStage ps, int* row_tok, int* row_seq, int* row_pos, int* grp_row0, int* grp_cnt,
+                                                           const T* __restrict__ emb, const T* __restrict__ pos, float* __restrict__ h, int d,
+                                                           int ticket, int router_ticket) {
     const int m = blockIdx.x;
-    const T* er = emb + (size_t)row_tok[m] * d;
-    const T* pr = pos + (size_t)row_pos[m] * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) h[(size_t)m * d + i] = to_float(er[i]) + to_float(pr[i]);
+    if (m == ps.rows) {
+        for (int b = threadIdx.x; b < ps.n_queries * ps.samples; b += 128) {
+            const int q = b / ps.samples, len = ps.len[q];
+            st.n[b] = len;
+            st.pending[b] = ps.ids[ps.id_off[q] + len - 1];
+        }
+        if (threadIdx.x == 0) { st.counters[6] = ticket; st.counters[8] = router_ticket; }
+        return;
+    }
+    int lo = 0, hi = ps.n_queries - 1;   // the last query whose rows begin at or before m (queries without rows share a start: the last one has it)
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (ps.row_off[mid] <= m) lo = mid; else hi = mid - 1;
+    }
+    const int p = m - ps.row_off[lo], tok = ps.ids[ps.id_off[lo] + p];
+    if (threadIdx.x == 0) {
+        row_tok[m] = tok; row_seq[m] = lo * ps.samples; row_pos[m] = p;
+        if (p % ps.group == 0) {
+            const int g = ps.grp_off[lo] + p / ps.group;
+            grp_row0[g] = m;
+            grp_cnt[g] = min(ps.group, ps.len[lo] - 1 - p);
+        }
+    }
+    embed_row<T, 128>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d);
+}
+
+// Keys / values of a query's first sequence to its other samples: one block per (layer and K or V, key/value head, query),
+// 16 bytes at a time, read once and written samples - 1 times.  cache: [layers * 2][batch][heads][t_max][row_bytes].
+// grid: (layers * 2, heads, queries); block: 256.
+__global__ void __launch_bounds__(256) copy_samples_kernel(unsigned char* cache, size_t layer_bytes, int samples, int t_max, int row_bytes,
+                                                           const int* __restrict__ len) {
+    const size_t pitch = (size_t)t_max * row_bytes, seq = pitch * gridDim.y;
+    unsigned char* src = cache + blockIdx.x * layer_bytes + (size_t)blockIdx.z * samples * seq + blockIdx.y * pitch;
+    const int n16 = (len[blockIdx.z] - 1) * (row_bytes >> 4);
+    for (int i = threadIdx.x; i < n16; i += 256) {
+        const uint4 v = reinterpret_cast<const uint4*>(src)[i];
+        for (int j = 1; j < samples; ++j) reinterpret_cast<uint4*>(src + j * seq)[i] = v;
+    }
 }
 
 // Arg-max of one row from the per-tile (value, index) pairs an output-head GEMM left behind; lowest index
@@ -97,13 +161,8 @@ __global__ void __launch_bounds__(128) step_begin_kernel(LoopState st, int r0, i
         }
     }
     __syncthreads();
-    const T* er = emb + (size_t)s_tok * d;
-    const T* pr = pos + (size_t)s_pos * d;
-    for (int i = threadIdx.x; i < d; i += 128) {
-        const float v = to_float(er[i]) + to_float(pr[i]);
-        h[(size_t)m * d + i] = v;
-        if (snap) snap[(size_t)m * d + i] = v;   // copy for the FF_Tandem projection of x^(0)
-    }
+    // (snap: copy for the FF_Tandem projection of x^(0))
+    embed_row<T, 128>(emb + (size_t)s_tok * d, pos + (size_t)s_pos * d, h + (size_t)m * d, snap ? snap + (size_t)m * d : nullptr, d);
 }
 
 __device__ __forceinline__ float block_sum_128(float v, float* red) {
@@ -112,22 +171,6 @@ __device__ __forceinline__ float block_sum_128(float v, float* red) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     return red[0] + red[1] + red[2] + red[3];
-}
-
-// LayerNorm of fp32 rows (biased variance, eps 1e-5), output in the storage type.  grid: rows; block: 128.
-template <typename T>
-__global__ void __launch_bounds__(128) layernorm_kernel(const float* __restrict__ x, const float* __restrict__ gain,
-                                                        const float* __restrict__ bias, T* __restrict__ out, int d) {
-    __shared__ float red[4];
-    const float* xr = x + (size_t)blockIdx.x * d;
-    float s = 0.f;
-    for (int i = threadIdx.x; i < d; i += 128) s += xr[i];
-    const float mu = block_sum_128(s, red) / d;
-    float v = 0.f;
-    for (int i = threadIdx.x; i < d; i += 128) { const float c = xr[i] - mu; v = fmaf(c, c, v); }
-    const float rstd = 1.0f / sqrtf(block_sum_128(v, red) / d + 1e-5f);
-    for (int i = threadIdx.x; i < d; i += 128)
-        out[(size_t)blockIdx.x * d + i] = from_float<T>((xr[i] - mu) * rstd * gain[i] + bias[i]);
 }
 
 // Four normalised values to the output row: fp32 as they are, bf16 rounded.
@@ -152,18 +195,18 @@ __device__ __forceinline__ void ln_store4(bf16* orow, bf16* rrow, int k4, float 
     else ln_store4(orow, k4, y0, y1, y2, y3);
 }
 
-// Decode-path LayerNorm of fp32 rows ahead of the tensor-core GEMMs (fp32 out; bf16 out for the stand-alone
-// projection above 64 rows): the row sits in registers between the passes (up to 4096 elements), loads and stores
-// are 16 bytes wide.  grid: rows; block: 128; d % 4 == 0.
+// LayerNorm of fp32 rows (biased variance, eps 1e-5) ahead of the GEMMs, output in the storage type: the row sits in
+// registers between the passes (up to 4096 elements), loads and stores are 16 bytes wide (8191 rows of 4096: 56 us with
+// scalar accesses in three passes).  raw (nullable): bf16 copy of the row as it is, for the FF_Tandem projection that reads
+// the same residual stream (a pass of its own over it took 120 us there).  A block keeps gain and bias in registers over its
+// rows and fetches a row ahead: with one row per block those 32 KB per 16 KB of row made the L2 traffic (51 us at 8191 rows).
+// grid: at most M blocks; block: 128; d % 4 == 0.
 template <typename TO>
 __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __restrict__ x, const float* __restrict__ gain,
                                                              const float* __restrict__ bias, TO* __restrict__ out, int d,
-                                                             bf16* out_lo = nullptr) {
+                                                             int M, bf16* out_lo = nullptr, bf16* raw = nullptr) {
     __shared__ float red[4];
     const int d4 = d >> 2;
-    const float4* xr = reinterpret_cast<const float4*>(x + (size_t)blockIdx.x * d);
-    TO* orow = out + (size_t)blockIdx.x * d;
-    bf16* rrow = out_lo ? out_lo + (size_t)blockIdx.x * d : nullptr;   // TO = bf16 only: the remainder plane's row
     if (d4 <= 8 * 128) {
         // gains and biases are parameters: fetched while the kernel that writes x is still running
         float4 gq[8], bq[8];
@@ -175,57 +218,90 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
         }
         pdl_wait();
         pdl_launch_dependents();
-        float4 t[8];
+        float4 tn[8];
+        auto fetch = [&](int row) {
+            const float4* xr = reinterpret_cast<const float4*>(x + (size_t)row * d);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = (threadIdx.x + 128 * u < d4) ? __ldcg(xr + threadIdx.x + 128 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-        float s = 0.f;
+            for (int u = 0; u < 8; ++u) tn[u] = (threadIdx.x + 128 * u < d4) ? __ldcg(xr + threadIdx.x + 128 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        fetch(blockIdx.x);
+        for (int row = blockIdx.x; row < M; row += gridDim.x) {
+            float4 t[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) s += (t[u].x + t[u].y) + (t[u].z + t[u].w);
-        const float mu = block_sum_128(s, red) / d;
-        float q = 0.f;
+            for (int u = 0; u < 8; ++u) t[u] = tn[u];
+            if (row + gridDim.x < M) fetch(row + gridDim.x);   // under this row's reductions
+            TO* orow = out + (size_t)row * d;
+            bf16* rrow = out_lo ? out_lo + (size_t)row * d : nullptr;   // TO = bf16 only: the remainder plane's row
+            if (raw) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (threadIdx.x + 128 * u < d4) {
-                const float d0 = t[u].x - mu, d1 = t[u].y - mu, d2 = t[u].z - mu, d3 = t[u].w - mu;
-                q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
+                for (int u = 0; u < 8; ++u)
+                    if (threadIdx.x + 128 * u < d4) ln_store4(raw + (size_t)row * d, threadIdx.x + 128 * u, t[u].x, t[u].y, t[u].z, t[u].w);
             }
-        }
-        const float rs = 1.0f / sqrtf(block_sum_128(q, red) / d + 1e-5f);
+            float s = 0.f;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int k4 = threadIdx.x + 128 * u;
-            if (k4 < d4) {
-                const float4 g = gq[u], b = bq[u];
-                ln_store4(orow, rrow, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
-                          (t[u].z - mu) * rs * g.z + b.z, (t[u].w - mu) * rs * g.w + b.w);
+            for (int u = 0; u < 8; ++u) s += (t[u].x + t[u].y) + (t[u].z + t[u].w);
+            const float mu = block_sum_128(s, red) / d;
+            float q = 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (threadIdx.x + 128 * u < d4) {
+                    const float d0 = t[u].x - mu, d1 = t[u].y - mu, d2 = t[u].z - mu, d3 = t[u].w - mu;
+                    q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
+                }
+            }
+            const float rs = 1.0f / sqrtf(block_sum_128(q, red) / d + 1e-5f);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k4 = threadIdx.x + 128 * u;
+                if (k4 < d4) {
+                    const float4 g = gq[u], b = bq[u];
+                    ln_store4(orow, rrow, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
+                              (t[u].z - mu) * rs * g.z + b.z, (t[u].w - mu) * rs * g.w + b.w);
+                }
             }
         }
     } else {
         pdl_wait();
         pdl_launch_dependents();
-        float s = 0.f;
-        for (int k4 = threadIdx.x; k4 < d4; k4 += 128) { const float4 t = __ldcg(xr + k4); s += (t.x + t.y) + (t.z + t.w); }
-        const float mu = block_sum_128(s, red) / d;
-        float q = 0.f;
-        for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
-            const float4 t = __ldcg(xr + k4);
-            const float d0 = t.x - mu, d1 = t.y - mu, d2 = t.z - mu, d3 = t.w - mu;
-            q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
-        }
-        const float rs = 1.0f / sqrtf(block_sum_128(q, red) / d + 1e-5f);
-        for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
-            const float4 t = __ldcg(xr + k4);
-            const float4 g = __ldg(reinterpret_cast<const float4*>(gain) + k4), b = __ldg(reinterpret_cast<const float4*>(bias) + k4);
-            ln_store4(orow, rrow, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
-                      (t.w - mu) * rs * g.w + b.w);
+        for (int row = blockIdx.x; row < M; row += gridDim.x) {
+            const float4* xr = reinterpret_cast<const float4*>(x + (size_t)row * d);
+            TO* orow = out + (size_t)row * d;
+            bf16* rrow = out_lo ? out_lo + (size_t)row * d : nullptr;
+            float s = 0.f;
+            for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
+                const float4 t = __ldcg(xr + k4);
+                s += (t.x + t.y) + (t.z + t.w);
+                if (raw) ln_store4(raw + (size_t)row * d, k4, t.x, t.y, t.z, t.w);
+            }
+            const float mu = block_sum_128(s, red) / d;
+            float q = 0.f;
+            for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
+                const float4 t = __ldcg(xr + k4);
+                const float d0 = t.x - mu, d1 = t.y - mu, d2 = t.z - mu, d3 = t.w - mu;
+                q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
+            }
+            const float rs = 1.0f / sqrtf(block_sum_128(q, red) / d + 1e-5f);
+            for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
+                const float4 t = __ldcg(xr + k4);
+                const float4 g = __ldg(reinterpret_cast<const float4*>(gain) + k4), b = __ldg(reinterpret_cast<const float4*>(bias) + k4);
+                ln_store4(orow, rrow, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
+                          (t.w - mu) * rs * g.w + b.w);
+            }
         }
     }
 }
 
-template <typename T>
-__global__ void cast_rows_kernel(const float* __restrict__ x, T* __restrict__ out, size_t n) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = from_float<T>(x[i]);
+// bf16 copy of the residual stream for a projection that no LayerNorm of the large model follows.  n a multiple of 8.
+// grid: enough blocks of 256 for n / 8.
+__global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ x, bf16* __restrict__ out, size_t n) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 8;
+    if (i >= n) return;
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(x + i)), b = __ldcg(reinterpret_cast<const float4*>(x + i) + 1);
+    const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w), p2 = __floats2bfloat162_rn(b.x, b.y), p3 = __floats2bfloat162_rn(b.z, b.w);
+    *reinterpret_cast<uint4*>(out + i) = make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
+                                                    *reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
 }
 
 // Arg-max of fp32 rows, lowest index on ties.  grid: rows; block: 256.

@@ -51,6 +51,7 @@ struct Layout {   // byte offsets into the arena
     size_t st_block_len, st_drafting, st_confidence;
     size_t forced_ids, forced_len, forced_nll, forced_top;   // teacher-forced forward: given tokens [B][T], lengths [B], scores [B][T]
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
+    size_t stage;                                   // a prompt pass's lengths, offsets and token ids as the host staged them
     size_t attn_counters;   // inside the zero-filled state block
     size_t h_large, h_small, a, q, o, f, xb, t1, yhat, a_s, logits_large, logits_small, part_ml, part_acc, dbg;
     size_t amax_val_large, amax_idx_large, amax_val_small, amax_idx_small;
@@ -116,7 +117,7 @@ struct tandem_ctx {
     bool use_graphs = true;
     int chunks_launch = 1;               // attention grid size along the context for the current iteration
     int32_t* hflags = nullptr;           // mapped pinned host memory the verify kernel publishes to
-    int64_t ticket = 0;                  // verify kernels enqueued since creation
+    int64_t ticket = 0;                  // verify kernels enqueued since creation (the device counts them too)
     // tensor-core path (bf16 only)
     bool tc = false;                     // weights have tensor maps; GEMMs run on tcgen05
     bool use_pdl = true;                 // programmatic dependent launch between the decode kernels
@@ -131,6 +132,7 @@ struct tandem_ctx {
     cudaStream_t side = nullptr;         // the decode-time FF_Tandem projections run here, beside the large model's later layers
     std::vector<cudaEvent_t> ev_fork;    // one per small layer
     cudaEvent_t ev_join = nullptr;
+    cudaEvent_t ev_staged = nullptr;     // the last prompt pass's copy out of the pinned staging buffer
     bool next_launch_plain = false;      // the next launch follows a cross-stream wait: no programmatic dependency on a kernel
     bool setup_failed = false;           // a launch helper could not encode a tensor map: reported by the enclosing call
     bool tc_prompt_attn = false;         // prompt attention on the tensor cores (head size 64 or 128)
@@ -138,7 +140,7 @@ struct tandem_ctx {
     float temp_large = 1.0f, temp_small = 1.0f;   // sampled SPEED (accept mode 4): temperatures of the two models
     RouterArgs router{};                 // adaptive block length: the router's weights (caller-owned, DEVICE) and threshold
     bool has_router = false;
-    int64_t router_ticket = 0;           // router launches since the prompt pass
+    int64_t router_ticket = 0;           // router launches since creation
     double prompt_sq_sum = 0.0;          // sum over the sequences of the current prompt pass of (rows)^2 (accounting of the attention's work)
 };
 
@@ -219,6 +221,7 @@ Layout make_layout(const tandem_config& c) {
     L.st_block_len = take(B * 4); L.st_drafting = take(B * 4); L.st_confidence = take(B * GL * 4);
     L.row_tok = take(R * 4); L.row_seq = take(R * 4); L.row_pos = take(R * 4);
     L.grp_row0 = take((size_t)L.max_groups * 4); L.grp_cnt = take((size_t)L.max_groups * 4);
+    L.stage = take((4 * B + R + B) * 4);
     L.attn_counters = take(B * hmax * 4);
     L.h_large = take(R * c.large.d_model * 4);
     L.h_small = take(B * c.small.d_model * 4);
@@ -446,19 +449,6 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
 }
 
 // y = x W^T for many rows on the tensor cores; x bf16 [M][ldx].
-template <int EPI, int BN>
-void launch_tc_tiled_bn(tandem_ctx& c, TcTiledArgs& a, const CUtensorMap& tmx, const TcW& w, int M) {
-    using C = TctCfg<BN>;
-    static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_tc_tiled_kernel<EPI, BN>, C::SMEM_BYTES, attr_done);
-    a.tiles0 = cdiv(w.seg_rows0, BN);
-    a.tiles_per_seg = cdiv(w.seg_rows, BN);
-    a.tiles_n = a.tiles0 + (w.n_segs - 1) * a.tiles_per_seg;
-    a.tiles_m = cdiv(M, 128);
-    launch_ex(c, false, 1, gemm_tc_tiled_kernel<EPI, BN>, dim3(std::min(a.tiles_n * a.tiles_m, std::max(1, c.n_sms))), dim3(TCT_THREADS), (size_t)C::SMEM_BYTES,
-              a, tmx, w.tm[0], w.tm[1], w.tm[2]);
-}
-
 template <int EPI>
 tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, const TcW& w, const EpiArgs& e, int* err) {
     if (M <= 0) return TANDEM_OK;
@@ -471,10 +461,32 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     memset(&a, 0, sizeof(a));
     a.M = M; a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.seg_rows = w.seg_rows;
     a.err_flag = err; a.e = e;
+    a.tiles_m = cdiv(M, 128);
+    const int n_sms = std::max(1, c.n_sms);
+    auto feature_tiles = [&](int width) {
+        a.tiles0 = cdiv(w.seg_rows0, width);
+        a.tiles_per_seg = cdiv(w.seg_rows, width);
+        a.tiles_n = a.tiles0 + (w.n_segs - 1) * a.tiles_per_seg;
+        return (long long)a.tiles_n * a.tiles_m;
+    };
     ProfScope ps(c, PC_GEMM_TC_TILED, 2.0 * M * (double)a.N * w.K);   // flops
-    // 256-wide tiles when they still give every SM a tile, else square ones
-    if ((long long)(cdiv(w.seg_rows0, 256) + (w.n_segs - 1) * cdiv(w.seg_rows, 256)) * cdiv(M, 128) >= c.n_sms) launch_tc_tiled_bn<EPI, 256>(c, a, tmx, w, M);
-    else launch_tc_tiled_bn<EPI, 128>(c, a, tmx, w, M);
+    const long long wide = feature_tiles(TCT_BN);
+    if (wide >= n_sms) {   // a 256-wide tile for every multiprocessor: each token-row tile read from shared memory feeds twice the MMA work of a square one
+        static std::atomic<unsigned long long> attr_done{0};
+        ensure_dyn_smem(gemm_tc_tiled_kernel<EPI>, TCT_SMEM_BYTES, attr_done);
+        launch_ex(c, true, 1, gemm_tc_tiled_kernel<EPI>, dim3(n_sms), dim3(TCT_THREADS), (size_t)TCT_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
+        return TANDEM_OK;
+    }
+    // Fewer: square tiles, and the K range of each dealt to as many CTAs (1, 2 or 4) as still get a multiprocessor of their
+    // own and four 64-element K-blocks each (fewer would not pay for the exchange).
+    const int tiles = (int)feature_tiles(TCS_BN), KB = cdiv(w.K, 64);
+    int S = 1;
+    while (S < 4 && tiles * S * 2 <= n_sms && KB >= 8 * S) S *= 2;
+    a.splits = S;
+    a.stages = tcs_stages(S);
+    static std::atomic<unsigned long long> attr_done{0};
+    ensure_dyn_smem(gemm_tc_split_kernel<EPI>, std::max(tcs_smem_bytes(2), tcs_smem_bytes(4)), attr_done);
+    launch_ex(c, true, S, gemm_tc_split_kernel<EPI>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)tcs_smem_bytes(S), a, tmx, w.tm[0], w.tm[1], w.tm[2]);
     return TANDEM_OK;
 }
 
@@ -586,11 +598,12 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     else launch_attn_decode_dq<128>(c, a, groups, cl, kv_bytes);
 }
 
+// raw (bf16 only, nullable): also leaves a bf16 copy of the rows as they are.
 template <typename T>
-void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d) {
-    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + sizeof(T)));
-    layernorm_kernel<T><<<M, 128, 0, c.stream>>>(x, static_cast<const float*>(gain), static_cast<const float*>(bias), out, d);
-    c.launches++;
+void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr) {
+    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + sizeof(T) + (raw ? 2.0 : 0.0)));
+    launch_ex(c, true, 1, layernorm_rows_kernel<T>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain), static_cast<const float*>(bias), out, d,
+              M, (bf16*)nullptr, raw);
 }
 
 // Describes the rows of one pass.
@@ -729,24 +742,22 @@ void project_layer(tandem_ctx& c, int j, const Rows& r) {
     launch_gemm<T, EPI_KV>(c, a_s, dS, r.M, kv, ekv);
 }
 
+bool projects_from(const tandem_ctx& c, int n_large_layers_done) {
+    for (int j = 0; j < c.small.d.n_layers; ++j)
+        if (c.layer_map[j] == n_large_layers_done) return true;
+    return false;
+}
 template <typename T>
 void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
-    bool any = false;
-    for (int j = 0; j < c.small.d.n_layers; ++j) any |= (c.layer_map[j] == n_large_layers_done);
-    if (!any) return;
-    if constexpr (sizeof(T) == 2) {
-        const size_t n = (size_t)r.M * c.large.d.d_model;
-        ProfScope ps(c, PC_ROWS, (double)n * (4.0 + sizeof(T)));
-        cast_rows_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(at<float>(c, c.lay.h_large), at<T>(c, c.lay.xb), n);
-        c.launches++;
-    }
     for (int j = 0; j < c.small.d.n_layers; ++j)
         if (c.layer_map[j] == n_large_layers_done) project_layer<T>(c, j, r);
 }
 
-// One decoder layer (Eq. 1; the same form serves the small model's layers in Eq. 2) on residual stream h.
+// One decoder layer (Eq. 1; the same form serves the small model's layers in Eq. 2) on residual stream h.  project: the
+// FF_Tandem projections that read h as it enters the layer (they run behind the first LayerNorm, which leaves them a bf16
+// copy of h on its way).
 template <typename T>
-void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r) {
+void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool project = false) {
     const int d = m.d.d_model, dff = m.d.d_ff;
     T* a = at<T>(c, c.lay.a);
     T* q = at<T>(c, c.lay.q);
@@ -757,6 +768,7 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
     const void *g1 = w_layer(c, m, l, W_LN1G), *b1 = w_layer(c, m, l, W_LN1B), *g2 = w_layer(c, m, l, W_LN2G), *b2 = w_layer(c, m, l, W_LN2B);
     if constexpr (sizeof(T) == 4) {
         if (fp32_few_rows(c, r)) {
+            if (project) project_after<T>(c, l, r);
             ln_rows<EPI_QKV>(c, h, r.M, g1, b1, qkv, epi_cache<T>(c, m, l, q));
             attention<T>(c, m, l, q, o, r);
             launch_rows<false, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
@@ -765,7 +777,8 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
             return;
         }
     }
-    launch_layernorm<T>(c, r.M, h, g1, b1, a, d);
+    launch_layernorm<T>(c, r.M, h, g1, b1, a, d, project && sizeof(T) == 2 ? at<bf16>(c, c.lay.xb) : nullptr);
+    if (project) project_after<T>(c, l, r);
     launch_gemm<T, EPI_QKV>(c, a, d, r.M, qkv, epi_cache<T>(c, m, l, q));
     attention<T>(c, m, l, q, o, r);
     launch_gemm<T, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
@@ -787,23 +800,15 @@ void head_argmax(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* 
 template <typename T>
 void large_layers(tandem_ctx& c, const Rows& r, bool project) {
     float* h = at<float>(c, c.lay.h_large);
-    if (project) project_after<T>(c, 0, r);
-    for (int l = 0; l < c.large.d.n_layers; ++l) {
-        decoder_layer<T>(c, c.large, l, h, r);
-        if (project) project_after<T>(c, l + 1, r);
+    const int n = c.large.d.n_layers;
+    for (int l = 0; l < n; ++l) decoder_layer<T>(c, c.large, l, h, r, project && projects_from(c, l));
+    if (!project || !projects_from(c, n)) return;
+    if constexpr (sizeof(T) == 2) {   // after the last layer no LayerNorm of the large model follows
+        const size_t elems = (size_t)r.M * c.large.d.d_model;
+        ProfScope ps(c, PC_ROWS, (double)elems * 6.0);
+        launch_ex(c, true, 1, cast_rows_kernel, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, at<bf16>(c, c.lay.xb), elems);
     }
-}
-
-// Prompt pass of the large model.
-template <typename T>
-void large_prompt(tandem_ctx& c, const Rows& r) {
-    {
-        ProfScope ps(c, PC_ROWS, (double)r.M * c.large.d.d_model * (4.0 + 2 * sizeof(T)));
-        embed_kernel<T><<<r.M, 128, 0, c.stream>>>(at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_pos), (const T*)w_emb(c, c.large),
-                                                   (const T*)w_pos(c, c.large), at<float>(c, c.lay.h_large), c.large.d.d_model);
-        c.launches++;
-    }
-    large_layers<T>(c, r, true);
+    project_after<T>(c, n, r);
 }
 
 Rows decode_rows(tandem_ctx& c, int r_last, int nq) {
@@ -963,7 +968,7 @@ void tc_ln_gemm(tandem_ctx& c, const float* h, const void* ln_g, const void* ln_
         {
             ProfScope ps(c, PC_LAYERNORM, (double)rows * w.K * 8.0);
             launch_ex(c, true, 1, layernorm_rows_kernel<bf16>, dim3(rows), dim3(128), 0, h, static_cast<const float*>(ln_g),
-                      static_cast<const float*>(ln_b), xp.hi, w.K, xp.lo);
+                      static_cast<const float*>(ln_b), xp.hi, w.K, rows, xp.lo, (bf16*)nullptr);
         }
         launch_tc_decode<PRO_TMA, EPI>(c, sc, xp.hi, w.K, nullptr, nullptr, rows, w, stream_w, e, amax_val, amax_idx, amax_stride, xp.map,
                                        c.lay.dec_rows);
@@ -973,7 +978,7 @@ void tc_ln_gemm(tandem_ctx& c, const float* h, const void* ln_g, const void* ln_
     {
         ProfScope ps(c, PC_LAYERNORM, (double)rows * w.K * 8.0);
         launch_ex(c, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, h, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a, w.K, (bf16*)nullptr);
+                  static_cast<const float*>(ln_b), a, w.K, rows, (bf16*)nullptr, (bf16*)nullptr);
     }
     launch_tc_decode<PRO_F32, EPI>(c, sc, a, w.K, nullptr, nullptr, rows, w, stream_w, e, amax_val, amax_idx, amax_stride);
 }
@@ -1285,6 +1290,7 @@ void release_side(tandem_ctx& c) {
     for (cudaEvent_t ev : c.ev_fork) cudaEventDestroy(ev);
     c.ev_fork.clear();
     if (c.ev_join) { cudaEventDestroy(c.ev_join); c.ev_join = nullptr; }
+    if (c.ev_staged) { cudaEventDestroy(c.ev_staged); c.ev_staged = nullptr; }
     if (c.side) { cudaStreamDestroy(c.side); c.side = nullptr; }
 }
 }  // namespace
@@ -1318,7 +1324,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->small.d = cfg->small; c->small.wbase = 5 + 10 * cfg->large.n_layers; c->small.kv_off = lay.kv_small; c->small.kv_layer_elems = lay.kv_small_layer;
     c->tbase = c->small.wbase + 5 + 10 * cfg->small.n_layers;
     c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0;
-    c->pinned_ints = std::max((size_t)3 * lay.max_rows + 2 * lay.max_groups + 4 * cfg->max_batch + 64,
+    c->pinned_ints = std::max((size_t)lay.max_rows + 5 * cfg->max_batch + 64,
                               (size_t)cfg->max_batch * (cfg->max_seq + 1) + 2 * 64 + 64);   // prompt rows going in; tokens, counters, histogram, lengths coming out
     c->pinned = nullptr;
     LoopState& st = c->st;
@@ -1340,6 +1346,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_staged, cudaEventDisableTiming);
     for (int j = 0; j < cfg->small.n_layers && e == cudaSuccess; ++j) {
         cudaEvent_t ev = nullptr;
         e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
@@ -1465,77 +1472,61 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     for (long long i = 0; i < total_ids; ++i)
         if (prompt_ids[i] < 0 || prompt_ids[i] >= c->cfg.large.vocab) return TANDEM_ERR_INVALID_ARG;
 
-    CK(cudaStreamSynchronize(c->stream));   // staging buffer free again; no verify kernel in flight
-    c->ticket = 0;                          // the device-side tickets are cleared with the rest of the loop state below
-    c->router_ticket = 0;
-    c->hflags[0] = 0;
-    c->hflags[5] = 0;
+    // The pass is enqueued behind whatever the stream still runs; only the staging buffer has to be free again, which it is
+    // as soon as the previous pass's copy has gone.  (Everything else that uses the buffer waits before it returns.)
+    CK(cudaEventSynchronize(c->ev_staged));
     const int M = (int)rows;
-    int32_t* p_tok = c->pinned;
-    int32_t* p_seq = p_tok + c->lay.max_rows;
-    int32_t* p_pos = p_seq + c->lay.max_rows;
-    int32_t* p_g0 = p_pos + c->lay.max_rows;
-    int32_t* p_gc = p_g0 + c->lay.max_groups;
-    int32_t* p_n = p_gc + c->lay.max_groups;
-    int32_t* p_pend = p_n + c->cfg.max_batch;
+    int32_t* p_len = c->pinned;
+    int32_t *p_id = p_len + n_queries, *p_row = p_id + n_queries, *p_grp = p_row + n_queries, *p_ids = p_grp + n_queries;
     int m = 0, groups = 0;
     long long off = 0;
     for (int q = 0; q < n_queries; ++q) {
-        const int len = prompt_lens[q];
-        for (int p = 0; p < len - 1; ++p) {
-            if (p % c->prompt_group == 0) { p_g0[groups] = m; p_gc[groups] = std::min(c->prompt_group, len - 1 - p); ++groups; }
-            p_tok[m] = prompt_ids[off + p]; p_seq[m] = q * samples; p_pos[m] = p; ++m;
-        }
-        for (int j = 0; j < samples; ++j) {
-            p_n[q * samples + j] = len;
-            p_pend[q * samples + j] = prompt_ids[off + len - 1];
-        }
-        off += len;
+        p_len[q] = prompt_lens[q]; p_id[q] = (int)off; p_row[q] = m; p_grp[q] = groups;
+        off += prompt_lens[q];
+        m += prompt_lens[q] - 1;
+        groups += cdiv(prompt_lens[q] - 1, c->prompt_group);
     }
+    memcpy(p_ids, prompt_ids, (size_t)total_ids * 4);
     cudaStream_t s = c->stream;
-    if (M > 0) {
-        CK(cudaMemcpyAsync(c->arena + c->lay.row_tok, p_tok, (size_t)M * 4, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(c->arena + c->lay.row_seq, p_seq, (size_t)M * 4, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(c->arena + c->lay.row_pos, p_pos, (size_t)M * 4, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(c->arena + c->lay.grp_row0, p_g0, (size_t)groups * 4, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(c->arena + c->lay.grp_cnt, p_gc, (size_t)groups * 4, cudaMemcpyHostToDevice, s));
-    }
     CK(cudaMemsetAsync(c->arena + c->lay.st_n, 0, c->lay.row_tok - c->lay.st_n, s));
-    CK(cudaMemcpyAsync(c->st.n, p_n, (size_t)batch * 4, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->st.pending, p_pend, (size_t)batch * 4, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(c->arena + c->lay.stage, c->pinned, ((size_t)4 * n_queries + total_ids) * 4, cudaMemcpyHostToDevice, s));
+    CK(cudaEventRecord(c->ev_staged, s));
     c->batch = batch;
     c->n_ub = n_max;
     c->n_sum = total;
     c->prompt_sq_sum = 0.0;
     for (int q = 0; q < n_queries; ++q) c->prompt_sq_sum += (double)(prompt_lens[q] - 1) * (prompt_lens[q] - 1);
+    PromptStage ps;
+    ps.len = at<int>(*c, c->lay.stage); ps.id_off = ps.len + n_queries; ps.row_off = ps.id_off + n_queries; ps.grp_off = ps.row_off + n_queries;
+    ps.ids = ps.grp_off + n_queries;
+    ps.n_queries = n_queries; ps.samples = samples; ps.rows = M; ps.group = c->prompt_group;
+    const bool bf = c->cfg.dtype == TANDEM_DTYPE_BF16;
+    {
+        ProfScope prof(*c, PC_ROWS, (double)M * c->large.d.d_model * (4.0 + 2 * c->esz));
+        auto begin = [&](auto* emb, auto* pos, auto kernel) {
+            kernel<<<M + 1, 128, 0, s>>>(c->st, ps, at<int>(*c, c->lay.row_tok), at<int>(*c, c->lay.row_seq), at<int>(*c, c->lay.row_pos),
+                                         at<int>(*c, c->lay.grp_row0), at<int>(*c, c->lay.grp_cnt), emb, pos, at<float>(*c, c->lay.h_large),
+                                         c->large.d.d_model, (int)c->ticket, (int)c->router_ticket);
+        };
+        if (bf) begin((const bf16*)w_emb(*c, c->large), (const bf16*)w_pos(*c, c->large), prompt_begin_kernel<bf16>);
+        else begin((const float*)w_emb(*c, c->large), (const float*)w_pos(*c, c->large), prompt_begin_kernel<float>);
+        c->launches++;
+    }
     if (M > 0) {
         Rows r; r.M = M; r.groups = groups; r.nq = 0; r.decode = false; r.n_chunks = 0; r.kv_positions = (double)rows;
-        if (c->cfg.dtype == TANDEM_DTYPE_BF16) large_prompt<bf16>(*c, r);
-        else large_prompt<float>(*c, r);
+        if (bf) large_layers<bf16>(*c, r, true);
+        else large_layers<float>(*c, r, true);
     }
-    TRY(check_launch(*c));
-    if (samples > 1) {
-        // the prompt's keys / values, per (model, layer, K or V, key/value head): positions 0 .. len - 2 of sequence
-        // q * samples go to the query's other sequences (one strided copy per destination)
+    if (samples > 1 && M > 0) {
         for (const Model* mdl : {&c->large, &c->small}) {
-            const int dh = mdl->d.d_model / mdl->d.n_heads;
-            const size_t pitch = (size_t)c->cfg.max_seq * dh * c->esz;            // one head's positions
-            const size_t seq_bytes = pitch * mdl->kv_heads;
-            for (int l = 0; l < mdl->d.n_layers; ++l)
-                for (int which = 0; which < 2; ++which) {
-                    unsigned char* base = c->arena + mdl->kv_off + ((size_t)l * 2 + which) * mdl->kv_layer_elems * c->esz;
-                    for (int q = 0; q < n_queries; ++q) {
-                        const size_t width = (size_t)(prompt_lens[q] - 1) * dh * c->esz;
-                        if (width == 0) continue;
-                        const unsigned char* src = base + (size_t)q * samples * seq_bytes;
-                        for (int j = 1; j < samples; ++j)
-                            CK(cudaMemcpy2DAsync(base + ((size_t)q * samples + j) * seq_bytes, pitch, src, pitch, width, mdl->kv_heads,
-                                                 cudaMemcpyDeviceToDevice, s));
-                    }
-                }
+            const int row_bytes = mdl->d.d_model / mdl->d.n_heads * (int)c->esz;
+            ProfScope prof(*c, PC_ROWS, 0.0);
+            copy_samples_kernel<<<dim3(mdl->d.n_layers * 2, mdl->kv_heads, n_queries), 256, 0, s>>>(c->arena + mdl->kv_off, mdl->kv_layer_elems * c->esz,
+                                                                                                 samples, c->cfg.max_seq, row_bytes, ps.len);
+            c->launches++;
         }
     }
-    return TANDEM_OK;
+    return check_launch(*c);
 }
 
 }  // namespace
@@ -2164,7 +2155,7 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
         launch_tc_decode<PRO_LN, EPI_KV>(tmp, ts, yhat, d_small, ln_g, ln_b, rows, wkv, true, e);
     } else {
         launch_ex(tmp, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a_s, (int)d_small, (bf16*)nullptr);
+                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr, (bf16*)nullptr);
         launch_tc_decode<PRO_F32, EPI_KV>(tmp, ts, a_s, d_small, nullptr, nullptr, rows, wkv, true, e);
     }
     return check_launch();

@@ -188,6 +188,15 @@ __device__ __forceinline__ void st_async_dsmem_f32(uint32_t local_smem_addr, uin
                  ::"r"(ra), "r"(__float_as_uint(v)), "r"(rb) : "memory");
 }
 
+// The same with sixteen bytes (both addresses 16-byte aligned).
+__device__ __forceinline__ void st_async_dsmem_f32x4(uint32_t local_smem_addr, uint32_t local_bar, int rank, float v0, float v1, float v2, float v3) {
+    uint32_t ra, rb;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_smem_addr), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(local_bar), "r"(rank));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(ra), "r"(__float_as_uint(v0)), "r"(__float_as_uint(v1)), "r"(__float_as_uint(v2)), "r"(__float_as_uint(v3)), "r"(rb) : "memory");
+}
+
 // Named barrier among a subset of the CTA's warps.
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 

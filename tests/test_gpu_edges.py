@@ -2,7 +2,7 @@
 import pytest
 
 from paper_2402_08644_b200 import binding, build, synth
-from test_gpu_parity import TOL_FP32, _replay_compare, gpu_toy_shape, prompts_for, toy_weights
+from test_gpu_parity import TOL_BF16, TOL_FP32, _bf16_weights, _replay_compare, gpu_toy_shape, prompts_for, toy_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -22,3 +22,15 @@ def test_fp32_few_row_kernels_at_their_edges(lens, gamma):
     shape = gpu_toy_shape(large=(1, 2080, 65, 2400), small=(1, 64, 1, 136), max_pos=160, layer_map=(1,))
     w = toy_weights(shape, seed=3, std=0.02)
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=4), gamma, 3, TOL_FP32, 1e-6, check_kv=True) == 0
+
+
+@pytest.mark.parametrize("lens", [[129],            # one row tile: K dealt to four CTAs (17 K-blocks: 4, 4, 4, 5)
+                                  [130, 2, 1],      # two row tiles, the second of two rows; a prompt without processed rows
+                                  [900, 385]])      # ten: two CTAs per tile, or one
+def test_bf16_split_k_prompt_gemm_at_its_edges(lens):
+    """Square tiles with one, two and four CTAs per tile: ragged last row tile and feature tile (1088 = 8.5 x 128, 1160),
+    K-blocks that do not divide evenly, grouped-query key / value segments of half a tile, both head sizes' attention tiles
+    (128 and 256 queries) with one row in the last one."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 1088, 17, 1160), small=(1, 128, 2, 256), max_pos=960, layer_map=(1,), kv_heads=(1, 0))
+    w = _bf16_weights(shape, seed=9, std=0.02)
+    assert _replay_compare(shape, w, prompts_for(shape, lens, seed=5), 2, 2, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 4
