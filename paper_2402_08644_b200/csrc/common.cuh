@@ -58,6 +58,17 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// What a kernel that produces rows of the residual stream leaves for the GEMM behind the next LayerNorm (bf16 decode
+// passes): the rows times the LayerNorm's gain as two bf16 planes (values, remainders) that the GEMM loads by TMA, and per row
+// and group of 32 features the group's mean and sum of squared deviations, which the GEMM merges into the row's
+// statistics while its products run.
+struct NextLn {
+    const float* gain;     // null: nothing is left
+    bf16* hi; bf16* lo;    // [rows][d]
+    float2* stats;         // [rows][groups]
+    int groups;            // ceil(d / 32)
+};
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -30,6 +30,7 @@ struct EpiArgs {
                           // the bf16 plane of the remainders (x = value + remainder), both [M][ldo], for a consumer that loads them by TMA
     void* snap;           // EPI_RESID on the tensor-core decode path: optional fp32 copy of the new values [M][snap_ld]
     int snap_ld;
+    NextLn ln;            // EPI_RESID on the tensor-core decode path, see NextLn
 };
 
 struct WSegs {            // up to three weight matrices stacked along N: [seg_rows0][K], then [seg_rows][K] each

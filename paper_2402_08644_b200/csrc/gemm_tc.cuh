@@ -7,9 +7,11 @@
 //                          K-slices of a tile sit in one thread-block cluster: each CTA sends its partial
 //                          sums to the CTA that finishes those token rows (remote shared-memory stores), which
 //                          adds them in slice order.
-//                          The token rows are written into the B stages by the CTA's own threads, which is
-//                          where the LayerNorm of the residual stream is fused.  Activations arrive in fp32 and
-//                          enter the product as the sum of two bf16 numbers (the rounded value and the rounded
+//                          LayerNorm ahead of a map is applied behind it:  LN(x) W^T = r (x.g) W^T - r m (g W^T) + b W^T
+//                          with the row's mean m and reciprocal deviation r.  The producer of x leaves x.g in two bf16
+//                          planes, g and b ride along as four more rows of the B operand (each as value + remainder), and
+//                          the row's statistics are merged while the products run, so nothing but TMA stands between
+//                          the producer and the MMAs (PRO_LNT).  Activations enter the product as the sum of two bf16 numbers (the rounded value and the rounded
 //                          remainder, about 16 significant bits): the B tile holds the NB value rows followed
 //                          by the NB remainder rows, one MMA of N = 2 NB covers both (the weight tile is read
 //                          from shared memory once), and the epilogue adds the two accumulator columns of a
@@ -37,7 +39,10 @@ namespace tandem {
 // LayerNorm, then value + remainder; PRO_F32: fp32 rows as value + remainder; PRO_TMA: the producer of the rows has
 // already written them as two bf16 planes (values, remainders), and TMA brings them into the B stages beside the
 // weights (no registers, no rounds, nothing for warps 0-3 to do before the epilogue).
-enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3 };
+// PRO_LNT: LayerNorm rows, x.g by TMA like PRO_TMA and the rest in the epilogue (see above); the small pair's maps behind a
+// LayerNorm took 4.4 us of the stream's time with the rows normalised in the prologue of every CTA (batch 1, 2), and
+// 4.4 + 1.9 us with a LayerNorm kernel of their own (more sequences).
+enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3, PRO_LNT = 4 };
 constexpr int EPI_ARGMAX = 6;                       // fp32 store plus the (max, index) of each row within the tile
 enum { TC_ERR_SLOT = 1, TC_ERR_OPERANDS = 2, TC_ERR_ACCUM = 3, TC_ERR_EXCHANGE = 4 };   // which bounded wait gave up
 
@@ -49,6 +54,9 @@ struct TcDecodeArgs {
                                 // a chain of dependent steps, nothing to protect) instead of after the last token-row loads
     const float* ln_g;      // PRO_LN: LayerNorm gain / bias [K]
     const float* ln_b;
+    int ln_row;             // PRO_LNT: first of the four rows of this LayerNorm in its tensor map
+    const float2* ln_stats; // PRO_LNT: [rows][ln_groups], see NextLn
+    int ln_groups;
     int rows, K, N;         // N = output features over all segments
     int seg_rows0, tiles0;  // output features and tiles of the first weight segment (one tensor map per segment)
     int seg_rows;           // output features of every further segment
@@ -68,18 +76,21 @@ struct TcDecodeArgs {
 };
 
 constexpr int TCD_THREADS = 192;   // warps 0-3: B operand + epilogue; warp 4: TMA; warp 5: TMEM + MMA issue
-template <int NB> struct TcdCfg {
+template <int NB, bool LNT> struct TcdCfg {
     static constexpr int NB2 = 2 * NB;              // B-operand rows = accumulator columns: values, then remainders
-    static constexpr int STAGES = NB <= 16 ? 5 : 3;   // two CTAs fit on an SM up to NB = 48 (at most 113 KB each with the static part)
+    static constexpr int N = NB2 + (LNT ? 16 : 0);  // ... and the LayerNorm's g, g's remainder, b, b's remainder (of 16 columns four are used)
+    static constexpr int STAGES = NB <= 16 ? (LNT ? 4 : 5) : 3;   // two CTAs fit on an SM up to NB = 48 (at most 113 KB each with the static part)
     static constexpr int A_BYTES = 128 * 128;       // 128 weight rows x 64 bf16
     static constexpr int B_BYTES = NB2 * 128;       // 2 NB rows x 64 bf16
-    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int LN_BYTES = LNT ? 4 * 128 : 0;
+    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + (LNT ? 1024 : 0);   // (the MMA's last twelve B rows are whatever follows: unread columns)
     static constexpr int INBOX_BYTES = NB * 128 * 4;   // the K-slices' partial sums for the token rows this CTA finishes
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + INBOX_BYTES + 1024;   // + slack to align the ring to 1024
-    static constexpr int TMEM_COLS = NB2 <= 32 ? 32 : (NB2 <= 64 ? 64 : 128);
+    static constexpr int TMEM_COLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
-static_assert(TcdCfg<16>::SMEM_BYTES + 3072 <= 113 * 1024 && TcdCfg<32>::SMEM_BYTES + 3072 <= 113 * 1024 &&
-              TcdCfg<48>::SMEM_BYTES + 3072 <= 113 * 1024, "two CTAs per SM: a kernel and its prefetching successor");
+static_assert(TcdCfg<16, true>::SMEM_BYTES + 1024 <= 113 * 1024 && TcdCfg<16, false>::SMEM_BYTES + 1024 <= 113 * 1024 &&
+              TcdCfg<32, true>::SMEM_BYTES + 1024 <= 113 * 1024 && TcdCfg<48, true>::SMEM_BYTES + 1024 <= 113 * 1024,
+              "two CTAs per SM: a kernel and its prefetching successor (static shared memory below 1 KB)");
 
 // x = hi + lo with hi = bf16(x), lo = bf16(x - hi): the pair carries x to about 16 significant bits.
 __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -116,12 +127,14 @@ __device__ __forceinline__ ScatterCol scatter_col(const EpiArgs& e, int seg, int
     return sc;
 }
 
-// grid: tiles * splits CTAs in clusters of `splits` (the K-slices of one tile); dynamic smem TcdCfg<NB>::SMEM_BYTES.
+// grid: tiles * splits CTAs in clusters of `splits` (the K-slices of one tile); dynamic smem TcdCfg::SMEM_BYTES.
 template <int NB, int PRO, int EPI>
 __global__ void __launch_bounds__(TCD_THREADS)
 gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
-                      const __grid_constant__ CUtensorMap tm2, const __grid_constant__ CUtensorMap tmx) {
-    using C = TcdCfg<NB>;
+                      const __grid_constant__ CUtensorMap tm2, const __grid_constant__ CUtensorMap tmx,
+                      const __grid_constant__ CUtensorMap tml) {
+    constexpr bool LNT = PRO == PRO_LNT, BY_TMA = PRO == PRO_TMA || LNT;   // BY_TMA: the token rows are loaded beside the weights
+    using C = TcdCfg<NB, LNT>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     __shared__ __align__(8) uint64_t s_full[C::STAGES];
     __shared__ __align__(8) uint64_t s_empty[C::STAGES];
@@ -129,8 +142,6 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     __shared__ __align__(8) uint64_t s_inbox;   // counts the bytes of the K-slices' partial sums sent to this CTA
     __shared__ uint32_t s_tmem;
     __shared__ float s_mu[NB], s_rstd[NB];
-    __shared__ float s_av[4][NB];
-    __shared__ int s_ai[4][NB];
     __shared__ long long s_rowoff[NB];   // EPI_QKV / EPI_KV: the row-dependent part of an output's cache index
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
@@ -158,12 +169,13 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     const int j_first = S == 1 ? 0 : sp * rpc;
     const int j_count = max(0, min(rpc, a.rows - j_first));
     float hres[EPI == EPI_RESID ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
+    float next_gain = 0.f;                   // EPI_RESID: gain of the LayerNorm that follows, at this thread's feature (a parameter)
     int my_seq = 0, my_pos = 0;              // EPI_QKV / EPI_KV, threads below a.rows: this token row's sequence and position
 
     if (warp == 5) {
         if (lane == 0) {
             for (int s = 0; s < C::STAGES; ++s) {
-                mbar_init(smem_u32(&s_full[s]), PRO == PRO_TMA ? 2 : 5);   // the TMA thread's arrive + one per B-operand warp (PRO_TMA: its second arrive)
+                mbar_init(smem_u32(&s_full[s]), BY_TMA ? 2 : 5);   // the TMA thread's arrive + one per B-operand warp (BY_TMA: its second arrive)
                 mbar_init(smem_u32(&s_empty[s]), 1);   // the MMA thread's commit
             }
             mbar_init(smem_u32(&s_accum), 1);
@@ -187,13 +199,14 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         const uint64_t pol = l2_policy_evict_first();
         auto load_a = [&](int i, int st) {
             const uint32_t bar = smem_u32(&s_full[st]);
-            mbar_arrive_expect_tx(bar, C::A_BYTES);
+            mbar_arrive_expect_tx(bar, C::A_BYTES + C::LN_BYTES);
+            if (LNT) tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES + C::A_BYTES + C::B_BYTES, &tml, (kb0 + i) * 64, a.ln_row, bar);   // parameters too
             if (a.stream_weights) tma_load_2d(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar, pol);
             else tma_load_2d_nohint(ring0 + st * C::STAGE_BYTES, tm, (kb0 + i) * 64, n_local0, bar);
         };
         if (a.withhold_weights) {
             // (test hook: nothing is loaded)
-        } else if (PRO == PRO_TMA) {
+        } else if (BY_TMA) {
             // Weights of the first ring-ful before the wait on the predecessor, then the wait, then their token rows
             // (two planes, 16-row boxes), then weights and rows together as stages come free.
             auto load_b = [&](int i, int st) {
@@ -210,6 +223,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             if (elect_one()) {
                 tma_prefetch_desc(tm);
                 tma_prefetch_desc(&tmx);
+                if (LNT) tma_prefetch_desc(&tml);
                 for (int i = 0; i < n_pre; ++i) load_a(i, i);
             }
             pdl_wait();
@@ -241,7 +255,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         __syncwarp();
     } else if (warp == 5) {
         // ---- MMA issue: one elected thread of a converged warp ----
-        constexpr uint32_t idesc = umma_idesc_bf16(128, C::NB2);
+        constexpr uint32_t idesc = umma_idesc_bf16(128, C::N);
         for (int i = 0; i < nkb; ++i) {
             const int st = i % C::STAGES;
             if (!mbar_wait_warp(smem_u32(&s_full[st]), (i / C::STAGES) & 1, poll_limit)) {
@@ -269,6 +283,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     // ---- warps 0-3: token rows into the B stages (then the epilogue) ----
     float4 gq[C::STAGES], bq[C::STAGES];   // register path: gain / bias of this lane's slot in each of the CTA's K-blocks
     if (a.wait_first) pdl_wait();
+    if (EPI == EPI_RESID && a.e.ln.gain && n_local0 + tid < seg_rows) next_gain = __ldg(a.e.ln.gain + seg_base + n_local0 + tid);
     if (ln_regs) {
 #pragma unroll
         for (int i = 0; i < C::STAGES; ++i) {
@@ -358,7 +373,32 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         __syncwarp();
         if (lane == 0)
             for (int i = 0; i < nkb; ++i) mbar_arrive(smem_u32(&s_full[i]));
-    } else if (PRO != PRO_TMA) {
+    } else if (LNT) {
+        // The rows' statistics from the groups' (mean, sum of squared deviations): eight lanes per row, sums relative to the
+        // first group's mean.  For each row the order of the sums depends on K only.
+        if (nkb <= C::STAGES || a.release_early) pdl_launch_dependents();   // (see the note at the epilogue)
+        for (int r0 = warp * 4; r0 < a.rows; r0 += 16) {
+            const int r = r0 + (lane >> 3), gl = lane & 7;
+            const float2* sp = a.ln_stats + (size_t)min(r, a.rows - 1) * a.ln_groups;
+            const float ref = __ldcg(sp).x;
+            float s = 0.f, q = 0.f;
+#pragma unroll 4
+            for (int g = gl; g < a.ln_groups; g += 8) {
+                const float2 p = __ldcg(sp + g);
+                const float n = (float)min(32, a.K - 32 * g), dm = p.x - ref;
+                s = fmaf(n, dm, s);
+                q += fmaf(n * dm, dm, p.y);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) { s += __shfl_xor_sync(0xffffffffu, s, o); q += __shfl_xor_sync(0xffffffffu, q, o); }
+            const float dmu = s / (float)a.K;
+            if (gl == 0 && r < a.rows) {
+                s_mu[r] = ref + dmu;
+                s_rstd[r] = 1.0f / sqrtf(fmaxf(q - s * dmu, 0.f) / (float)a.K + 1e-5f);
+            }
+        }
+        bar_sync(1, 128);
+    } else if (!BY_TMA) {
         // general case: statistics (LayerNorm), then the K-blocks a ring's worth at a time
         if (PRO == PRO_LN) {
             for (int r = warp; r < a.rows; r += 4) {   // one warp per row, fixed lane-strided order
@@ -474,15 +514,22 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         // else here, after the last round has been written.  Letting it start right after the wait measured 2-3 %
         // slower per iteration (its CTAs' set-up and loads compete with the row loads); later than here (after the
         // accumulator is ready, or after the exchange) slower again (the successor's head start shrinks).
-        // (PRO_TMA with a K-slice longer than the ring and a matrix large enough to be a stream: the TMA thread does it, after
+        // (BY_TMA with a K-slice longer than the ring and a matrix large enough to be a stream: the TMA thread does it, after
         // its last loads; otherwise there is nothing of this kernel's in the successor's way, and it is released at once)
-        if (PRO != PRO_TMA || nkb <= C::STAGES || a.release_early) pdl_launch_dependents();
+        if (!BY_TMA || (!LNT && (nkb <= C::STAGES || a.release_early))) pdl_launch_dependents();
         if (EPI == EPI_QKV || EPI == EPI_KV) {
             if (tid < a.rows) s_rowoff[tid] = ((long long)my_seq * a.e.n_heads * a.e.t_max + my_pos) * a.e.d_head;
             bar_sync(1, 128);
         }
         if (!mbar_wait(smem_u32(&s_accum), 0, poll_limit)) tc_report(a.err_flag, TC_ERR_ACCUM);
         tc_fence_after_sync();
+        float c1 = 0.f, c2 = 0.f;                     // PRO_LNT: this feature's (slice of) g W^T and b W^T
+        if (LNT) {
+            float w[16];
+            tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + C::NB2, w);
+            c1 = w[0] + w[1];
+            c2 = w[2] + w[3];
+        }
 #pragma unroll
         for (int c0 = 0; c0 < NB; c0 += 16) {
             if (c0 >= a.rows) break;                  // columns of absent token rows are never read
@@ -490,7 +537,10 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c0, t);        // x's values times W
             tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + NB + c0, u);   // x's remainders times W
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[c0 + i] = t[i] + u[i];
+            for (int i = 0; i < 16; ++i) {
+                v[c0 + i] = t[i] + u[i];
+                if (LNT) v[c0 + i] = fmaf(s_rstd[c0 + i], fmaf(-s_mu[c0 + i], c1, v[c0 + i]), c2);   // (rows past the last: never used)
+            }
         }
         tc_fence_before_sync();
         asm volatile("bar.arrive 2, 160;" ::: "memory");   // the accumulator has been read: warp 5 may free the TMEM columns
@@ -501,6 +551,8 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     if (EPI == EPI_ARGMAX) {                            // whole tiles only (S == 1)
         if (warp < 4) {
             float* out = static_cast<float*>(a.e.out);
+            float* s_av = reinterpret_cast<float*>(ring + C::STAGES * C::STAGE_BYTES);   // [4 warps][NB], where the inbox would be
+            int* s_ai = reinterpret_cast<int*>(s_av + 4 * NB);
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 if (j >= a.rows) break;
@@ -514,15 +566,15 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
                         if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
                     }
-                    if (lane == 0) { s_av[warp][j] = bv; s_ai[warp][j] = bi; }
+                    if (lane == 0) { s_av[warp * NB + j] = bv; s_ai[warp * NB + j] = bi; }
                 }
             }
             bar_sync(1, 128);
             if (tid < a.rows) {
-                float bv = s_av[0][tid];
-                int bi = s_ai[0][tid];
+                float bv = s_av[tid];
+                int bi = s_ai[tid];
                 for (int w = 1; w < 4; ++w)
-                    if (s_av[w][tid] > bv || (s_av[w][tid] == bv && s_ai[w][tid] < bi)) { bv = s_av[w][tid]; bi = s_ai[w][tid]; }
+                    if (s_av[w * NB + tid] > bv || (s_av[w * NB + tid] == bv && s_ai[w * NB + tid] < bi)) { bv = s_av[w * NB + tid]; bi = s_ai[w * NB + tid]; }
                 a.amax_val[(size_t)tid * a.amax_stride + tile] = bv;
                 a.amax_idx[(size_t)tid * a.amax_stride + tile] = bi;
             }
@@ -565,6 +617,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         if (warp < 4) {
             ScatterCol sc;
             if (EPI == EPI_QKV || EPI == EPI_KV) sc = scatter_col<EPI>(a.e, seg, n_local);
+            const int n_group = max(0, min(32, seg_rows - (n_local0 + warp * 32)));   // features of this warp's group of 32
 #pragma unroll
             for (int s = 0; s < NB; ++s) {
                 if (s >= j_count) break;
@@ -576,6 +629,12 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         if (EPI == EPI_RESID || EPI == EPI_STORE_F32) {
                             static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = hv;
                             if (EPI == EPI_RESID && a.e.snap) static_cast<float*>(a.e.snap)[(size_t)j * a.e.snap_ld + n] = hv;
+                            if (EPI == EPI_RESID && a.e.ln.gain) {
+                                const float x = hv * next_gain;
+                                const bf16 hi = __float2bfloat16_rn(x);
+                                a.e.ln.hi[(size_t)j * a.e.ldo + n] = hi;
+                                a.e.ln.lo[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                            }
                         } else if (EPI == EPI_GELU) {   // activations between the decode kernels stay fp32, or value + remainder planes
                             const float gv = gelu_bf16_out(hv);
                             if (a.e.out_lo) {
@@ -590,6 +649,34 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         } else {
                             epilogue<bf16, EPI>(a.e, j, n, hv);
                         }
+                    }
+                    if (EPI == EPI_RESID) v[s] = hv;   // (for the statistics below)
+                }
+            }
+            if (EPI == EPI_RESID && a.e.ln.gain && n_group > 0) {   // (warp-uniform)
+                // Mean and squared deviations of this warp's 32 features, four rows at a time in one transposing reduction (row by
+                // row, with two five-step sums each, they cost 1.3 us of a 7.4 us launch with four rows per CTA).  Sums are
+                // relative to the group's first feature.
+                const float inv = 1.0f / (float)n_group;
+#pragma unroll
+                for (int s0 = 0; s0 < NB; s0 += 4) {
+                    if (s0 >= j_count) break;
+                    float sums[8], ref[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float hv = s0 + u < j_count ? v[s0 + u] : 0.f;
+                        ref[u] = __shfl_sync(0xffffffffu, hv, 0);
+                        const float dv = valid ? hv - ref[u] : 0.f;
+                        sums[2 * u] = dv;
+                        sums[2 * u + 1] = dv * dv;
+                    }
+                    const float mine = warp_sum_many<8>(sums, lane);                     // lane L: sum number L / 4
+                    const float sd = __shfl_sync(0xffffffffu, mine, lane & ~7), sq = __shfl_sync(0xffffffffu, mine, (lane & ~7) + 4);
+                    const int u = lane >> 3;
+                    if ((lane & 7) == 0 && s0 + u < j_count) {
+                        const float rf = u == 0 ? ref[0] : (u == 1 ? ref[1] : (u == 2 ? ref[2] : ref[3]));
+                        a.e.ln.stats[(size_t)(j_first + s0 + u) * a.e.ln.groups + ((seg_base + n_local0 + warp * 32) >> 5)] =
+                            make_float2(fmaf(sd, inv, rf), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
                     }
                 }
             }

@@ -32,23 +32,71 @@ struct LoopState {
     int gamma_limit;
 };
 
-// x^(0) = Emb(t) + Pos(index) of one row (Eq. 1) into the fp32 residual stream, 16 bytes of the tables at a time.
-// d is a multiple of 8.  All threads of a block of BLOCK take part.
+// x^(0) = Emb(t) + Pos(index) of one row (Eq. 1) into the fp32 residual stream, 16 bytes of the tables at a time, with what
+// the first LayerNorm's GEMM wants of it (bf16; `row` is its row there).  d is a multiple of 8.  All threads of a block of
+// BLOCK take part.
 template <typename T, int BLOCK>
-__device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __restrict__ pr, float* __restrict__ hr, float* __restrict__ snap, int d) {
+__device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __restrict__ pr, float* __restrict__ hr, float* __restrict__ snap, int d,
+                                          const NextLn& ln, int row) {
     constexpr int VN = VecN<T>::N;
-    for (int i = threadIdx.x * VN; i < d; i += BLOCK * VN) {
-        float e[VN], p[VN];
-        load_vec(er + i, e);
-        load_vec(pr + i, p);
+    for (int i0 = 0; i0 < d; i0 += BLOCK * VN) {
+        const int i = i0 + threadIdx.x * VN;
+        float v[VN];
 #pragma unroll
-        for (int u = 0; u < VN; u += 4) {
-            const float4 v = make_float4(e[u] + p[u], e[u + 1] + p[u + 1], e[u + 2] + p[u + 2], e[u + 3] + p[u + 3]);
-            *reinterpret_cast<float4*>(hr + i + u) = v;
-            if (snap) *reinterpret_cast<float4*>(snap + i + u) = v;
+        for (int u = 0; u < VN; ++u) v[u] = 0.f;
+        if (i < d) {
+            float p[VN];
+            load_vec(er + i, v);
+            load_vec(pr + i, p);
+#pragma unroll
+            for (int u = 0; u < VN; ++u) v[u] += p[u];
+#pragma unroll
+            for (int u = 0; u < VN; u += 4) {
+                const float4 t = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
+                *reinterpret_cast<float4*>(hr + i + u) = t;
+                if (snap) *reinterpret_cast<float4*>(snap + i + u) = t;
+            }
+        }
+        if constexpr (sizeof(T) == 2) {
+            if (ln.gain == nullptr) continue;
+            if (i < d) {
+                uint4 hi, lo;
+                uint32_t *ph = &hi.x, *pl = &lo.x;
+#pragma unroll
+                for (int u = 0; u < VN; u += 4) {
+                    const float4 g = __ldg(reinterpret_cast<const float4*>(ln.gain + i + u));
+                    const float x0 = v[u] * g.x, x1 = v[u + 1] * g.y, x2 = v[u + 2] * g.z, x3 = v[u + 3] * g.w;
+                    const __nv_bfloat162 a = __floats2bfloat162_rn(x0, x1), b = __floats2bfloat162_rn(x2, x3);
+                    const __nv_bfloat162 ra = __floats2bfloat162_rn(x0 - __low2float(a), x1 - __high2float(a));
+                    const __nv_bfloat162 rb = __floats2bfloat162_rn(x2 - __low2float(b), x3 - __high2float(b));
+                    ph[u / 2] = *reinterpret_cast<const uint32_t*>(&a); ph[u / 2 + 1] = *reinterpret_cast<const uint32_t*>(&b);
+                    pl[u / 2] = *reinterpret_cast<const uint32_t*>(&ra); pl[u / 2 + 1] = *reinterpret_cast<const uint32_t*>(&rb);
+                }
+                *reinterpret_cast<uint4*>(ln.hi + (size_t)row * d + i) = hi;
+                *reinterpret_cast<uint4*>(ln.lo + (size_t)row * d + i) = lo;
+            }
+            // four neighbouring threads hold a group of 32 features
+            const float n = (float)min(32, d - (i & ~31));
+            float s = 0.f, q = 0.f;
+#pragma unroll
+            for (int u = 0; u < VN; ++u) s += v[u];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            const float mean = s / n;
+            if (i < d) {
+#pragma unroll
+                for (int u = 0; u < VN; ++u) { const float c = v[u] - mean; q = fmaf(c, c, q); }
+            }
+            q += __shfl_xor_sync(0xffffffffu, q, 1);
+            q += __shfl_xor_sync(0xffffffffu, q, 2);
+            if (i < d && (threadIdx.x & 3) == 0) ln.stats[(size_t)row * ln.groups + (i >> 5)] = make_float2(mean, q);
         }
     }
 }
+
+// One LayerNorm's parameters and where its four rows go that ride along in the GEMM behind it: gain, the gain's bf16
+// remainder, bias, its remainder ([4][d]).
+struct LnSource { const float* g; const float* b; bf16* rows; int d; };
 
 // What a prompt pass needs on the device, staged in one copy: per query its length and its offsets among the token ids,
 // the processed rows and the attention groups ([4][n_queries]), then the ids, query after query.
@@ -59,13 +107,26 @@ struct PromptStage {
 
 // Start of a prompt pass: block m < rows sets up processed row m (token, sequence, position, its attention group if it
 // starts one) and embeds it; the last block sets the loop state of every sequence.  The tickets are the host's counts of
-// the verify and router kernels it has enqueued, which the device's counts equal by then.
-// grid: rows + 1; block: 128.
+// the verify and router kernels it has enqueued, which the device's counts equal by then.  Blocks beyond that write the
+// LayerNorms' rows for the decode passes that follow (bf16).
+// grid: rows + 1 + LayerNorms; block: 128.
 template <typename T>
 __global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptStage ps, int* row_tok, int* row_seq, int* row_pos, int* grp_row0, int* grp_cnt,
                                                            const T* __restrict__ emb, const T* __restrict__ pos, float* __restrict__ h, int d,
-                                                           int ticket, int router_ticket) {
+                                                           int ticket, int router_ticket, const LnSource* __restrict__ lns) {
     const int m = blockIdx.x;
+    if (m > ps.rows) {
+        const LnSource l = lns[m - ps.rows - 1];
+        for (int i = threadIdx.x; i < l.d; i += 128) {
+            const float g = l.g[i], b = l.b[i];
+            const bf16 gh = __float2bfloat16_rn(g), bh = __float2bfloat16_rn(b);
+            l.rows[i] = gh;
+            l.rows[l.d + i] = __float2bfloat16_rn(g - __bfloat162float(gh));
+            l.rows[2 * l.d + i] = bh;
+            l.rows[3 * l.d + i] = __float2bfloat16_rn(b - __bfloat162float(bh));
+        }
+        return;
+    }
     if (m == ps.rows) {
         for (int b = threadIdx.x; b < ps.n_queries * ps.samples; b += 128) {
             const int q = b / ps.samples, len = ps.len[q];
@@ -89,7 +150,7 @@ __global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptS
             grp_cnt[g] = min(ps.group, ps.len[lo] - 1 - p);
         }
     }
-    embed_row<T, 128>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d);
+    embed_row<T, 128>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0);
 }
 
 // Keys / values of a query's first sequence to its other samples: one block per (layer and K or V, key/value head, query),
@@ -142,7 +203,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) step_begin_kernel(LoopState st, int r0, int nq, int fin_r, const float* amax_val,
                                                          const int* amax_idx, int amax_stride, int n_tiles, int* row_tok,
                                                          int* row_seq, int* row_pos, const T* __restrict__ emb,
-                                                         const T* __restrict__ pos, float* __restrict__ h, int d, float* snap) {
+                                                         const T* __restrict__ pos, float* __restrict__ h, int d, float* snap, NextLn ln) {
     __shared__ int s_tok, s_pos;
     pdl_wait();
     pdl_launch_dependents();
@@ -162,7 +223,7 @@ __global__ void __launch_bounds__(128) step_begin_kernel(LoopState st, int r0, i
     }
     __syncthreads();
     // (snap: copy for the FF_Tandem projection of x^(0))
-    embed_row<T, 128>(emb + (size_t)s_tok * d, pos + (size_t)s_pos * d, h + (size_t)m * d, snap ? snap + (size_t)m * d : nullptr, d);
+    embed_row<T, 128>(emb + (size_t)s_tok * d, pos + (size_t)s_pos * d, h + (size_t)m * d, snap ? snap + (size_t)m * d : nullptr, d, ln, m);
 }
 
 __device__ __forceinline__ float block_sum_128(float v, float* red) {

@@ -55,7 +55,8 @@ struct Layout {   // byte offsets into the arena
     size_t attn_counters;   // inside the zero-filled state block
     size_t h_large, h_small, a, q, o, f, xb, t1, yhat, a_s, logits_large, logits_small, part_ml, part_acc, dbg;
     size_t amax_val_large, amax_idx_large, amax_val_small, amax_idx_small;
-    size_t a32, o32, f32;                           // fp32 activations between the bf16 decode kernels: LayerNorm / attention / GELU outputs
+    size_t a32, o32, f32;                           // value / remainder planes between the bf16 decode kernels: LayerNorm inputs (x.g) / attention / GELU outputs
+    size_t ln_src, ln_rows_large, ln_rows_small, ln_stats;   // LayerNorms behind the GEMMs (bf16 decode): sources, their rows, the token rows' statistics
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles;
@@ -119,14 +120,15 @@ struct tandem_ctx {
     int32_t* hflags = nullptr;           // mapped pinned host memory the verify kernel publishes to
     int64_t ticket = 0;                  // verify kernels enqueued since creation (the device counts them too)
     // tensor-core path (bf16 only)
+    int n_lns = 0;                       // LayerNorms of both models (bf16), see Layout::ln_src
     bool tc = false;                     // weights have tensor maps; GEMMs run on tcgen05
     bool use_pdl = true;                 // programmatic dependent launch between the decode kernels
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
     // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
-    // TMA: maps of the LayerNorm / attention / GELU buffers, [buffer 0..2][0 large, 1 small], 16-row boxes.
-    CUtensorMap xmap[3][2];
-    bool xmap_ok = false;
+    // TMA: maps of the residual stream (times the next LayerNorm's gain) / attention / GELU buffers, [buffer 0..2][0 large,
+    // 1 small], 16-row boxes; and the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one).
+    CUtensorMap xmap[3][2], lnmap[2];
     std::vector<char> wmap_ok;
     std::vector<CUtensorMap> kmap, vmap; // the large model's key / value cache of each layer as [(seq, head, position)][d_head]
     cudaStream_t side = nullptr;         // the decode-time FF_Tandem projections run here, beside the large model's later layers
@@ -244,6 +246,10 @@ Layout make_layout(const tandem_config& c) {
     L.proj_yhat = take(nS * RD * c.small.d_model * 4);
     L.proj_a = take(nS * RD * c.small.d_model * 4);
     L.proj_t1 = take(nS * RD * hidden * 4);
+    L.ln_src = take((size_t)(2 * c.large.n_layers + 1 + 2 * c.small.n_layers + 1) * sizeof(LnSource));
+    L.ln_rows_large = take((size_t)(2 * c.large.n_layers + 1) * 4 * c.large.d_model * 2);
+    L.ln_rows_small = take((size_t)(2 * c.small.n_layers + 1) * 4 * c.small.d_model * 2);
+    L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
     L.total = off;
     return L;
 }
@@ -390,13 +396,23 @@ void launch_ex(tandem_ctx& c, bool pdl, int cluster, void (*kernel)(KArgs...), d
     c.launches++;
 }
 
+// Token rows that lie in two bf16 planes (PRO_TMA), and the LayerNorm that is applied to them (PRO_LNT).
+struct TcRows {
+    const CUtensorMap* map = nullptr;
+    int plane_rows = 0;                    // rows between the value and the remainder plane
+    const CUtensorMap* ln_map = nullptr;
+    int ln_row = 0;                        // the LayerNorm's first row there
+    const float2* ln_stats = nullptr;      // [rows][ln_groups]
+    int ln_groups = 0;
+};
+
 template <int NB, int PRO, int EPI>
-void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const CUtensorMap* xmap) {
-    using C = TcdCfg<NB>;
+void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const TcRows& x) {
+    using C = TcdCfg<NB, PRO == PRO_LNT>;
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(gemm_tc_decode_kernel<NB, PRO, EPI>, C::SMEM_BYTES, attr_done);
     launch_ex(c, true, a.splits, gemm_tc_decode_kernel<NB, PRO, EPI>, dim3(units), dim3(TCD_THREADS), (size_t)C::SMEM_BYTES, a, w.tm[0], w.tm[1], w.tm[2],
-              xmap ? *xmap : w.tm[0]);
+              x.map ? *x.map : w.tm[0], x.ln_map ? *x.ln_map : w.tm[0]);
 }
 
 // y = prologue(x) W^T for few rows on the tensor cores, streaming W once per group of up to 64 rows (one group in
@@ -404,7 +420,7 @@ void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int
 template <int PRO, int EPI>
 void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx, const void* ln_g, const void* ln_b, int rows,
                       const TcW& w, bool stream_weights, const EpiArgs& e, float* amax_val = nullptr, int* amax_idx = nullptr,
-                      int amax_stride = 0, const CUtensorMap* xmap = nullptr, int x_plane_rows = 0) {
+                      int amax_stride = 0, const TcRows& xr = TcRows()) {
     if (rows <= 0) return;
     TcDecodeArgs a;
     memset(&a, 0, sizeof(a));
@@ -429,7 +445,9 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     for (int r0 = 0; r0 < rows; r0 += 64) {
         const int nr = std::min(64, rows - r0);
         a.rows = nr;
-        a.x_row0 = r0; a.x_plane_rows = x_plane_rows;
+        a.x_row0 = r0; a.x_plane_rows = xr.plane_rows;
+        a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups;
+        a.ln_stats = xr.ln_stats ? xr.ln_stats + (size_t)r0 * xr.ln_groups : nullptr;
         a.wait_first = r0 == 0 ? sc.wait_first : 0;
         a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
         a.x = static_cast<const unsigned char*>(x) + (size_t)r0 * ldx * xsz;
@@ -440,11 +458,12 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
         if (e.out_lo) a.e.out_lo = static_cast<unsigned char*>(e.out_lo) + (size_t)r0 * e.ldo * 2;   // (value / remainder planes are bf16)
         if (e.row_seq) { a.e.row_seq = e.row_seq + r0; a.e.row_pos = e.row_pos + r0; }
         if (e.snap) a.e.snap = static_cast<float*>(e.snap) + (size_t)r0 * e.snap_ld;
+        if (e.ln.gain) { a.e.ln.hi = e.ln.hi + (size_t)r0 * e.ldo; a.e.ln.lo = e.ln.lo + (size_t)r0 * e.ldo; a.e.ln.stats = e.ln.stats + (size_t)r0 * e.ln.groups; }
         ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + (double)nr * w.K * xsz + (double)nr * a.N * (EPI == EPI_QKV || EPI == EPI_KV || EPI == EPI_STORE ? 2.0 : 4.0));
-        if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, a, w, units, xmap);
-        else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, a, w, units, xmap);
-        else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, a, w, units, xmap);
-        else launch_tc_decode_nb<64, PRO, EPI>(c, a, w, units, xmap);
+        if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, a, w, units, xr);
+        else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, a, w, units, xr);
+        else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, a, w, units, xr);
+        else launch_tc_decode_nb<64, PRO, EPI>(c, a, w, units, xr);
     }
 }
 
@@ -822,12 +841,12 @@ Rows decode_rows(tandem_ctx& c, int r_last, int nq) {
 // Row set-up + embedding for block rows r0 .. r0+nq-1 of every sequence; fin_r: block row whose token is the
 // arg-max the small model's last head GEMM left as per-tile results (-1: none).
 template <typename T>
-void begin_rows(tandem_ctx& c, const Model& m, float* h, int r0, int nq, int fin_r, float* snap = nullptr) {
+void begin_rows(tandem_ctx& c, const Model& m, float* h, int r0, int nq, int fin_r, float* snap = nullptr, const NextLn& ln = NextLn{}) {
     ProfScope ps(c, PC_ROWS, (double)c.batch * nq * m.d.d_model * 8.0);
     launch_ex(c, true, 1, step_begin_kernel<T>, dim3(c.batch * nq), dim3(128), 0, c.st, r0, nq, fin_r,
               (const float*)at<float>(c, c.lay.amax_val_small), (const int*)at<int>(c, c.lay.amax_idx_small), c.lay.vocab_tiles,
               c.lay.vocab_tiles, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos),
-              (const T*)w_emb(c, m), (const T*)w_pos(c, m), h, m.d.d_model, snap);
+              (const T*)w_emb(c, m), (const T*)w_pos(c, m), h, m.d.d_model, snap, ln);
 }
 
 // fp32 draft step s: one token per sequence through the small model over the mixed context (Eq. 2, lines 2-3).
@@ -931,108 +950,87 @@ void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
 // bf16 decode on the tensor cores: five kernels per decoder layer, chained by programmatic dependent launch
 // ---------------------------------------------------------------------------------------------------
 
-// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = LayerNorm output, 1 = attention
-// output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width for buffer 2).
-struct XPlanes { bf16* hi; bf16* lo; const CUtensorMap* map; };
+// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = residual stream times the next
+// LayerNorm's gain, 1 = attention output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width
+// for buffer 2).
+struct XPlanes { bf16* hi; bf16* lo; TcRows rows; };
 XPlanes x_planes(tandem_ctx& c, int buf, const Model& m) {
     const size_t off = buf == 0 ? c.lay.a32 : (buf == 1 ? c.lay.o32 : c.lay.f32);
     const size_t K = buf == 2 ? m.d.d_ff : m.d.d_model;
     XPlanes p;
-    p.hi = reinterpret_cast<bf16*>(c.arena + off);
+    p.hi = at<bf16>(c, off);
     p.lo = p.hi + (size_t)c.lay.dec_rows * K;
-    p.map = &c.xmap[buf][&m == &c.large ? 0 : 1];
+    p.rows.map = &c.xmap[buf][&m == &c.large ? 0 : 1];
+    p.rows.plane_rows = c.lay.dec_rows;
     return p;
 }
 
-// Whether LayerNorm is fused into the GEMM's operand load.  Fused, every CTA of the GEMM normalises the rows it
-// needs itself: right for a couple of sequences and short rows, wasteful beyond (eight sequences of 768 elements
-// already measured 2 % slower per iteration than the LayerNorm kernel).  The choice depends on the batch
-// and the model only, never on the number of rows, so a block pass and a one-row pass take the same route.
-bool tc_fused_prologue(const tandem_ctx& c, int K) { return c.batch <= 2 && K <= 1024; }
-
-// y = LayerNorm(h) W^T with the given epilogue; h fp32 [rows][K].  ln_out: where the normalised rows go when the
-// LayerNorm runs as its own kernel (default: the pass's activation buffer).
-template <int EPI>
-void tc_ln_gemm(tandem_ctx& c, const float* h, const void* ln_g, const void* ln_b, int rows, const TcW& w, bool stream_w,
-                const EpiArgs& e, float* amax_val = nullptr, int* amax_idx = nullptr, int amax_stride = 0, float* ln_out = nullptr) {
-    const TcScratch sc = tc_scratch(c);
-    if (tc_fused_prologue(c, w.K)) {
-        launch_tc_decode<PRO_LN, EPI>(c, sc, h, w.K, ln_g, ln_b, rows, w, stream_w, e, amax_val, amax_idx, amax_stride);
-        return;
-    }
-    const Model* hm = h == reinterpret_cast<const float*>(c.arena + c.lay.h_large) ? &c.large :
-                      (h == reinterpret_cast<const float*>(c.arena + c.lay.h_small) ? &c.small : nullptr);
-    if (!ln_out && c.xmap_ok && hm && hm->d.d_model == w.K) {
-        // the LayerNorm kernel leaves value and remainder planes, the GEMM loads them by TMA beside its weights
-        const XPlanes xp = x_planes(c, 0, *hm);
-        {
-            ProfScope ps(c, PC_LAYERNORM, (double)rows * w.K * 8.0);
-            launch_ex(c, true, 1, layernorm_rows_kernel<bf16>, dim3(rows), dim3(128), 0, h, static_cast<const float*>(ln_g),
-                      static_cast<const float*>(ln_b), xp.hi, w.K, rows, xp.lo, (bf16*)nullptr);
-        }
-        launch_tc_decode<PRO_TMA, EPI>(c, sc, xp.hi, w.K, nullptr, nullptr, rows, w, stream_w, e, amax_val, amax_idx, amax_stride, xp.map,
-                                       c.lay.dec_rows);
-        return;
-    }
-    float* a = ln_out ? ln_out : at<float>(c, c.lay.a32);
-    {
-        ProfScope ps(c, PC_LAYERNORM, (double)rows * w.K * 8.0);
-        launch_ex(c, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, h, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a, w.K, rows, (bf16*)nullptr, (bf16*)nullptr);
-    }
-    launch_tc_decode<PRO_F32, EPI>(c, sc, a, w.K, nullptr, nullptr, rows, w, stream_w, e, amax_val, amax_idx, amax_stride);
+// LayerNorm number `idx` of a model (2 l, 2 l + 1 of layer l, 2 n_layers the final one): its gain, what the producer of the
+// residual stream leaves for it, and the operand of the GEMM behind it.
+const void* ln_gain(const tandem_ctx& c, const Model& m, int idx) {
+    return idx == 2 * m.d.n_layers ? w_tail(c, m, 0) : w_layer(c, m, idx / 2, idx % 2 ? W_LN2G : W_LN1G);
+}
+NextLn next_ln(tandem_ctx& c, const Model& m, int idx) {
+    const XPlanes p = x_planes(c, 0, m);
+    return {static_cast<const float*>(ln_gain(c, m, idx)), p.hi, p.lo, at<float2>(c, c.lay.ln_stats), cdiv(m.d.d_model, 32)};
+}
+TcRows ln_rows_of(tandem_ctx& c, const Model& m, int idx) {
+    TcRows r = x_planes(c, 0, m).rows;
+    r.ln_map = &c.lnmap[&m == &c.large ? 0 : 1];
+    r.ln_row = 4 * idx;
+    r.ln_stats = at<float2>(c, c.lay.ln_stats);
+    r.ln_groups = cdiv(m.d.d_model, 32);
+    return r;
 }
 
-// One decoder layer of a decode pass.  Between the kernels the activations are fp32 (attention and GELU outputs,
-// normalised rows); only the queries and the cached keys / values are bf16.
+// Whether the projection's LayerNorm is fused into its GEMM's operand load.  Fused, every CTA of the GEMM normalises the rows
+// it needs itself: right for a couple of sequences and short rows, wasteful beyond.  The choice depends on the batch and the
+// model only, never on the number of rows.
+bool tc_fused_prologue(const tandem_ctx& c, int K) { return c.batch <= 2 && K <= 1024; }
+
+// One decoder layer of a decode pass.  Between the kernels the activations are fp32 (the residual stream) or pairs of bf16
+// planes; only the queries and the cached keys / values are bf16.
 void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool stream_w, float* snap = nullptr) {
     const int d = m.d.d_model, dff = m.d.d_ff;
     bf16* q = at<bf16>(c, c.lay.q);
-    float* o = at<float>(c, c.lay.o32);
-    float* f = at<float>(c, c.lay.f32);
     const TcScratch sc = tc_scratch(c);
-    tc_ln_gemm<EPI_QKV>(c, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), r.M,
-                        tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w, epi_cache<bf16>(c, m, l, q));
+    const XPlanes xo = x_planes(c, 1, m), xf = x_planes(c, 2, m);
+    launch_tc_decode<PRO_LNT, EPI_QKV>(c, sc, nullptr, d, nullptr, nullptr, r.M,
+                                       tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w,
+                                       epi_cache<bf16>(c, m, l, q), nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l));
+    attention_decode(c, m, l, q, reinterpret_cast<float*>(xo.hi), r, xo.lo);
+    EpiArgs eo = epi_plain(h, d);
+    eo.ln = next_ln(c, m, 2 * l + 1);
+    launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w, eo,
+                                         nullptr, nullptr, 0, xo.rows);
+    EpiArgs e1 = epi_plain(xf.hi, dff);
+    e1.out_lo = xf.lo;
+    launch_tc_decode<PRO_LNT, EPI_GELU>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), stream_w, e1,
+                                        nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l + 1));
     EpiArgs e2 = epi_plain(h, d);
     e2.snap = snap; e2.snap_ld = d;   // copy of x^(l+1) when an FF_Tandem projection reads it
-    if (c.xmap_ok) {
-        // attention and GELU outputs as value / remainder planes that the next GEMM loads by TMA
-        const XPlanes xo = x_planes(c, 1, m), xf = x_planes(c, 2, m);
-        attention_decode(c, m, l, q, reinterpret_cast<float*>(xo.hi), r, xo.lo);
-        launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, xo.hi, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w,
-                                             epi_plain(h, d), nullptr, nullptr, 0, xo.map, c.lay.dec_rows);
-        EpiArgs e1 = epi_plain(xf.hi, dff);
-        e1.out_lo = xf.lo;
-        tc_ln_gemm<EPI_GELU>(c, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d),
-                             stream_w, e1);
-        launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, xf.hi, dff, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), stream_w, e2,
-                                             nullptr, nullptr, 0, xf.map, c.lay.dec_rows);
-        return;
-    }
-    attention_decode(c, m, l, q, o, r);
-    launch_tc_decode<PRO_F32, EPI_RESID>(c, sc, o, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w,
-                                         epi_plain(h, d));
-    tc_ln_gemm<EPI_GELU>(c, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d),
-                         stream_w, epi_plain(f, dff));
-    launch_tc_decode<PRO_F32, EPI_RESID>(c, sc, f, dff, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), stream_w, e2);
+    e2.ln = next_ln(c, m, 2 * l + 2);
+    launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, dff, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), stream_w, e2,
+                                         nullptr, nullptr, 0, xf.rows);
 }
 
 // Final LayerNorm + output head; leaves fp32 logits and the per-tile (max, index) pairs that the next kernel
 // (the next pass's row set-up, or the verify kernel) turns into token ids.
-void tc_head(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool stream_w) {
-    tc_ln_gemm<EPI_ARGMAX>(c, h, w_tail(c, m, 0), w_tail(c, m, 1), r.M, tcw(c, wi_tail(m, 2), -1, -1, m.d.vocab, m.d.d_model), stream_w,
-                           epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.lay.vocab_tiles);
+void tc_head(tandem_ctx& c, const Model& m, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool stream_w) {
+    launch_tc_decode<PRO_LNT, EPI_ARGMAX>(c, tc_scratch(c), nullptr, m.d.d_model, nullptr, nullptr, r.M, tcw(c, wi_tail(m, 2), -1, -1, m.d.vocab, m.d.d_model),
+                                          stream_w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.lay.vocab_tiles,
+                                          ln_rows_of(c, m, 2 * m.d.n_layers));
 }
 
 // sampled: the previous draft was drawn by sample_draft_kernel (it is in the loop state already), not left as per-tile
 // arg-max results.
 void tc_small_step(tandem_ctx& c, int s, bool sampled) {
     float* y = at<float>(c, c.lay.h_small);
-    begin_rows<bf16>(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1);
+    begin_rows<bf16>(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1, nullptr, next_ln(c, c.small, 0));
     const Rows r = decode_rows(c, s, 1);
     for (int j = 0; j < c.small.d.n_layers; ++j) tc_decoder_layer(c, c.small, j, y, r, false);
     float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
-    tc_head(c, c.small, y, r, logits, c.lay.amax_val_small, c.lay.amax_idx_small, false);
+    tc_head(c, c.small, r, logits, c.lay.amax_val_small, c.lay.amax_idx_small, false);
 }
 
 // FF_Tandem of the block's rows after n large layers (Eq. 2, first line) for every small layer fed from there, then
@@ -1064,9 +1062,15 @@ void tc_project_forked(tandem_ctx& c, int n_large_layers_done, int slot, const R
             launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, t1, c.hidden, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden),
                                                      true, epi_plain(yhat, dS));
         }
-        tc_ln_gemm<EPI_KV>(c, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), r.M,
-                           tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS), true, epi_cache<bf16>(c, c.small, j, nullptr),
-                           nullptr, nullptr, 0, a_j);
+        const void *lg = w_layer(c, c.small, j, W_LN1G), *lb = w_layer(c, c.small, j, W_LN1B);
+        const TcW wkv = tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS);
+        const EpiArgs ekv = epi_cache<bf16>(c, c.small, j, nullptr);
+        if (tc_fused_prologue(c, dS)) {
+            launch_tc_decode<PRO_LN, EPI_KV>(c, sc, yhat, dS, lg, lb, r.M, wkv, true, ekv);
+        } else {
+            launch_layernorm<float>(c, r.M, yhat, lg, lb, a_j, dS);
+            launch_tc_decode<PRO_F32, EPI_KV>(c, sc, a_j, dS, nullptr, nullptr, r.M, wkv, true, ekv);
+        }
     }
     c.stream = main_stream;
 }
@@ -1088,14 +1092,14 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
         return slot >= 0 ? at<float>(c, c.lay.proj_snap) + (size_t)slot * snap_elems : nullptr;
     };
     bool any_fork = false;
-    begin_rows<bf16>(c, c.large, h, 0, nq, fin_r, snap_of(0));
+    begin_rows<bf16>(c, c.large, h, 0, nq, fin_r, snap_of(0), next_ln(c, c.large, 0));
     const Rows r = decode_rows(c, nq - 1, nq);
     if (project && project_slot(c, 0) >= 0) { tc_project_forked(c, 0, project_slot(c, 0), r); any_fork = true; }
     for (int l = 0; l < c.large.d.n_layers; ++l) {
         tc_decoder_layer(c, c.large, l, h, r, true, snap_of(l + 1));
         if (project && project_slot(c, l + 1) >= 0) { tc_project_forked(c, l + 1, project_slot(c, l + 1), r); any_fork = true; }
     }
-    if (head) tc_head(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.lay.amax_val_large, c.lay.amax_idx_large, true);
+    if (head) tc_head(c, c.large, r, at<float>(c, c.lay.logits_large), c.lay.amax_val_large, c.lay.amax_idx_large, true);
     if (any_fork) {   // the projections join the main stream before the verify kernel
         cudaEventRecord(c.ev_join, c.side);
         cudaStreamWaitEvent(c.stream, c.ev_join, 0);
@@ -1378,6 +1382,28 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             if (cfg->ff_tandem_kind == TANDEM_FF_LINEAR) add(wi_tandem(*c, j, 0), cfg->small.d_model, cfg->large.d_model);
             else { add(wi_tandem(*c, j, 0), c->hidden, cfg->large.d_model); add(wi_tandem(*c, j, 1), cfg->small.d_model, c->hidden); }
         }
+        for (int mi = 0; mi < 2; ++mi) {   // decode activations and the LayerNorms' rows
+            const Model& mm = mi == 0 ? c->large : c->small;
+            for (int buf = 0; buf < 3; ++buf) {
+                const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
+                const size_t at_off = buf == 0 ? lay.a32 : (buf == 1 ? lay.o32 : lay.f32);
+                ok = ok && make_tmap_bf16(&c->xmap[buf][mi], c->arena + at_off, 2 * (uint64_t)lay.dec_rows, K, K, 16);
+            }
+            const uint64_t d = mm.d.d_model, n_ln = 2 * mm.d.n_layers + 1;
+            ok = ok && make_tmap_bf16(&c->lnmap[mi], c->arena + (mi == 0 ? lay.ln_rows_large : lay.ln_rows_small), 4 * n_ln, d, d, 4);
+        }
+        std::vector<LnSource> lns;
+        for (int mi = 0; mi < 2; ++mi) {
+            const Model& mm = mi == 0 ? c->large : c->small;
+            bf16* rows = at<bf16>(*c, mi == 0 ? lay.ln_rows_large : lay.ln_rows_small);
+            for (int i = 0; i <= 2 * mm.d.n_layers; ++i) {
+                const bool last = i == 2 * mm.d.n_layers;
+                const void* b = last ? w_tail(*c, mm, 1) : w_layer(*c, mm, i / 2, i % 2 ? W_LN2B : W_LN1B);
+                lns.push_back({static_cast<const float*>(ln_gain(*c, mm, i)), static_cast<const float*>(b), rows + (size_t)i * 4 * mm.d.d_model, mm.d.d_model});
+            }
+        }
+        c->n_lns = (int)lns.size();
+        e = cudaMemcpy(c->arena + lay.ln_src, lns.data(), lns.size() * sizeof(LnSource), cudaMemcpyHostToDevice);
         if (!ok) {
             snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled unavailable or failed for a weight matrix");
             if (c->pinned) cudaFreeHost(c->pinned);
@@ -1388,18 +1414,6 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             return TANDEM_ERR_CUDA;
         }
         c->tc = true;
-        {
-            bool okx = true;
-            const uint64_t RDx = (uint64_t)lay.dec_rows;
-            for (int buf = 0; buf < 3 && okx; ++buf)
-                for (int mi = 0; mi < 2 && okx; ++mi) {
-                    const Model& mm = mi == 0 ? c->large : c->small;
-                    const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
-                    const size_t off = buf == 0 ? lay.a32 : (buf == 1 ? lay.o32 : lay.f32);
-                    okx = K % 8 == 0 && make_tmap_bf16(&c->xmap[buf][mi], c->arena + off, 2 * RDx, K, K, 16);
-                }
-            c->xmap_ok = okx;
-        }
         const int dhL = cfg->large.d_model / cfg->large.n_heads;
         if (dhL == 64 || dhL == 128) {
             c->kmap.resize(cfg->large.n_layers);
@@ -1504,9 +1518,9 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     {
         ProfScope prof(*c, PC_ROWS, (double)M * c->large.d.d_model * (4.0 + 2 * c->esz));
         auto begin = [&](auto* emb, auto* pos, auto kernel) {
-            kernel<<<M + 1, 128, 0, s>>>(c->st, ps, at<int>(*c, c->lay.row_tok), at<int>(*c, c->lay.row_seq), at<int>(*c, c->lay.row_pos),
+            kernel<<<M + 1 + c->n_lns, 128, 0, s>>>(c->st, ps, at<int>(*c, c->lay.row_tok), at<int>(*c, c->lay.row_seq), at<int>(*c, c->lay.row_pos),
                                          at<int>(*c, c->lay.grp_row0), at<int>(*c, c->lay.grp_cnt), emb, pos, at<float>(*c, c->lay.h_large),
-                                         c->large.d.d_model, (int)c->ticket, (int)c->router_ticket);
+                                         c->large.d.d_model, (int)c->ticket, (int)c->router_ticket, at<LnSource>(*c, c->lay.ln_src));
         };
         if (bf) begin((const bf16*)w_emb(*c, c->large), (const bf16*)w_pos(*c, c->large), prompt_begin_kernel<bf16>);
         else begin((const float*)w_emb(*c, c->large), (const float*)w_pos(*c, c->large), prompt_begin_kernel<float>);

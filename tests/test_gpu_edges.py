@@ -34,3 +34,16 @@ def test_bf16_split_k_prompt_gemm_at_its_edges(lens):
     shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 1088, 17, 1160), small=(1, 128, 2, 256), max_pos=960, layer_map=(1,), kv_heads=(1, 0))
     w = _bf16_weights(shape, seed=9, std=0.02)
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=5), 2, 2, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 4
+
+
+@pytest.mark.parametrize("batch,gamma,offset", [(1, 0, 0.0), (3, 4, 0.5), (4, 3, 0.0), (1, 15, 0.5),      # 1, 15, 16 and 16 block rows
+                                                (3, 5, 0.0), (11, 2, 0.5), (7, 6, 0.0), (4, 15, 0.0)])     # 18, 33, 49 and 64
+def test_bf16_layernorm_behind_the_product(batch, gamma, offset):
+    """LayerNorm applied in the epilogue of the map behind it, at every token-column width, one to sixteen rows per warp of
+    statistics, row lengths that end inside a K-block (96, 160), and rows whose mean is several times their deviation."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 160, 5, 288), small=(2, 96, 3, 136), max_pos=64, layer_map=(0, 2))
+    w = _bf16_weights(shape, seed=gamma + 3, std=0.05)
+    for tag in "LS":
+        w[tag + ".pos"] = synth.round_to_bf16(w[tag + ".pos"] + offset)
+    prompts = prompts_for(shape, [1 + 3 * (b % 5) for b in range(batch)], seed=batch)
+    assert _replay_compare(shape, w, prompts, gamma, 2, TOL_BF16, 2 * TOL_BF16) <= 10
