@@ -590,14 +590,36 @@ void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl,
     launch_ex(c, true, cl, attn_decode_kernel<DH>, dim3(cl, a.n_heads / std::max(1, a.heads_per_cta), groups), dim3(ATD_THREADS),
               attn_decode_smem_bytes<DH>(), a);
 }
-// Cluster size: the largest of 1, 2, 4, 8 that keeps the launch within one wave of resident CTAs (two per SM,
-// one for 128-wide heads).  It depends on the number of sequences and heads only, so every pass of a run
-// (block or one-row) cuts the context the same way.  (Sizes in between, which would fill the wave better, measured
+// Clusters of `cl` decode-attention CTAs that the device can run at the same time (asked once per device and size).  It is
+// less than the multiprocessors would suggest, because a cluster has to fit into one GPC: with 148 multiprocessors and one
+// 128-wide CTA on each, 33 clusters of four and 15 of eight (64-wide, two CTAs each: 71 and 33).
+template <int DH>
+int attn_max_clusters(int cl) {
+    static std::atomic<int> cache[MAX_DEVICES][4];
+    std::atomic<int>& slot = cache[cur_dev()][cl == 8 ? 3 : (cl == 4 ? 2 : (cl == 2 ? 1 : 0))];
+    int n = slot.load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    static std::atomic<unsigned long long> attr_done{0};
+    ensure_dyn_smem(attn_decode_kernel<DH>, attn_decode_smem_bytes<DH>(), attr_done);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(cl); cfg.blockDim = dim3(ATD_THREADS); cfg.dynamicSmemBytes = attn_decode_smem_bytes<DH>();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)cl; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_decode_kernel<DH>, &cfg) != cudaSuccess || n < 1) n = 1;
+    slot.store(n, std::memory_order_relaxed);
+    return n;
+}
+// Cluster size: the largest of 1, 2, 4, 8 with which all clusters run at the same time.  It depends on the number of sequences
+// and key/value heads only, so every pass of a run (block or one-row) cuts the context the same way.  One cluster of eight
+// too many cost a second wave: two sequences x 4000 positions x 8 key/value heads x 128, blocks of six rows, took 35-41 us with
+// eight (16 clusters where 15 fit), 18.6 us with four.  (Sizes in between, which would fill the wave better, measured
 // 3 % slower per iteration at batch 8: a cluster of three merges more states than its extra CTAs save.)
-int attn_cluster_size(int n_sms, int groups, int n_heads, int d_head) {
-    const long long slots = (long long)n_sms * (d_head == 128 ? 1 : 2);
-    int cl = 1;
-    while (cl < ATD_CLUSTER && (long long)groups * n_heads * cl * 2 <= slots) cl *= 2;
+int attn_cluster_size(int clusters, int d_head) {
+    int cl = ATD_CLUSTER;
+    while (cl > 1 && clusters > (d_head == 32 ? attn_max_clusters<32>(cl) : (d_head == 64 ? attn_max_clusters<64>(cl) : attn_max_clusters<128>(cl)))) cl /= 2;
     return cl;
 }
 void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int groups, double kv_bytes) {
@@ -611,7 +633,7 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     int gpc = 1;
     while (gpc * 2 <= group && group % (gpc * 2) == 0 && gpc * 2 * a.nq <= ATT_NQ) gpc *= 2;
     a.heads_per_cta = gpc;
-    const int cl = attn_cluster_size(c.n_sms, groups, n_kv, d_head);
+    const int cl = attn_cluster_size((int)std::min<long long>((long long)groups * n_kv, INT_MAX), d_head);
     if (d_head == 32) launch_attn_decode_dq<32>(c, a, groups, cl, kv_bytes);
     else if (d_head == 64) launch_attn_decode_dq<64>(c, a, groups, cl, kv_bytes);
     else launch_attn_decode_dq<128>(c, a, groups, cl, kv_bytes);
