@@ -5,19 +5,24 @@
 //
 // Every draw uses one uniform variate from a counter-based generator keyed by (seed, sequence, iteration, slot):
 // slots 0..gamma-1 draw the drafts, 16 + r tests draft r, 48 redraws.  A draw from weights w with variate u returns
-// the first index whose running sum exceeds u * sum(w).  The running sums are fp32: each warp of the block owns a
-// contiguous range of the row, the ranges' sums are scanned in warp order, and the warp whose range contains the
-// target walks it again 32 weights at a time.
+// the first index whose running sum exceeds u * sum(w).  The running sums are fp32: each warp owns a contiguous range of
+// the row, the ranges' sums are scanned in range order, and the warp whose range contains the target finds the index by
+// its 32-weight pieces' sums, then inside the piece.
+//
+// A row of logits is dealt to the eight CTAs of a cluster and stays in registers between the maximum, the sums and the
+// search (up to 32768 logits; longer rows are read again for each step).  One CTA per row was bound by the
+// passes over the row following one another: 32000 logits, four sequences, three drafts, a draw 12.1 us and the decisions
+// 45.2 us.  The maxima and sums that the accept tests need come from the draws (small model) and from a launch over all rows
+// of the block (large model) instead of four passes per draft in the deciding CTA.
 #pragma once
 #include <math.h>
 #include "common.cuh"
+#include "gemm_simt.cuh"
 #include "misc_kernels.cuh"
 #include "tc_common.cuh"
 
 namespace tandem {
 
-constexpr int SMP_THREADS = 1024;   // one CTA walks a whole row of logits several times: many loads in flight
-constexpr int SMP_WARPS = SMP_THREADS / 32;
 constexpr int SMP_SLOT_ACCEPT = 16;
 constexpr int SMP_SLOT_REDRAW = 48;
 
@@ -27,164 +32,219 @@ __device__ __forceinline__ float uniform_variate(unsigned long long seed, int se
     return (float)(x >> 40) * (1.0f / 16777216.0f);   // 24 bits: exact in fp32
 }
 
-// Block-wide reductions over SMP_THREADS threads; `red` holds SMP_WARPS floats.  Every thread gets the result.
-__device__ __forceinline__ float smp_block_max(float v, float* red) {
-    v = warp_max(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float r = red[0];
+constexpr int SMC_THREADS = 256, SMC_WARPS = SMC_THREADS / 32, SMC_CLUSTER = 8;
+constexpr int SMC_RANGES = SMC_CLUSTER * SMC_WARPS;          // contiguous ranges of a row, one per warp of the cluster
+constexpr int SMC_REGS = 16;                                 // weights per lane, one of each 32-weight piece of the range
+
+// One draw by a cluster from the weights weight(load(i), m), i in [0, V).  RELMAX: the weights are relative to the maximum m of
+// load(i), exp((x - m) * inv_t), and every warp takes its own range's maximum until the ranges' records meet; otherwise they
+// are absolute (m = 0).  Every CTA gets every range's (m, sum); the one warp whose range contains u * total finds the index and
+// returns it in all of its lanes (all other warps return -1).  *m_out, *total_out (nullable): the row's maximum and the total
+// relative to it.  box: SMC_RANGES float2 of shared memory, written by all CTAs of the cluster, whose opening handshake must
+// be closed.  All threads of the cluster take part.
+template <bool RELMAX, typename L, typename W>
+__device__ __forceinline__ int smc_draw(L load, W weight, int V, int rank, float inv_t, float u, float2* box, float* m_out, float* total_out) {
+    const int lane = threadIdx.x & 31, id = rank * SMC_WARPS + (threadIdx.x >> 5);
+    const int chunk = (((V + SMC_RANGES - 1) / SMC_RANGES) + 31) & ~31;
+    const int i0 = min(V, id * chunk), i1 = min(V, i0 + chunk);
+    const bool in_regs = chunk <= 32 * SMC_REGS;             // (uniform) else the range is read again for each step
+    float m = RELMAX ? -INFINITY : 0.f, local = 0.f;
+    float p[SMC_REGS];
+    if (in_regs) {
+        decltype(load(0)) x[SMC_REGS];
 #pragma unroll
-    for (int w = 1; w < SMP_WARPS; ++w) r = fmaxf(r, red[w]);
-    return r;
-}
-
-// Maximum of row[0..V).
-__device__ __forceinline__ float smp_row_max(const float* row, int V, float* red) {
-    float m = -INFINITY;
-    const bool vec = (V & 3) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0;   // 16 bytes at a time, several loads in flight
-    const int V4 = vec ? V >> 2 : 0;
-#pragma unroll 4
-    for (int i4 = threadIdx.x; i4 < V4; i4 += SMP_THREADS) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(row) + i4);
-        m = fmaxf(fmaxf(m, fmaxf(x.x, x.y)), fmaxf(x.z, x.w));
-    }
-    for (int i = 4 * V4 + threadIdx.x; i < V; i += SMP_THREADS) m = fmaxf(m, __ldcg(row + i));
-    return smp_block_max(m, red);
-}
-
-// Inverse-CDF draw from the non-negative weights w(i), i in [0, V), with variate u in [0, 1).
-// Warp j of the block owns the contiguous range [j * chunk, (j + 1) * chunk).  Pass A: every warp sums its range
-// (lanes stride over it, coalesced), the warps' sums are scanned in warp order.  Pass B: the warp whose range
-// contains the target u * total walks it again, 32 consecutive weights at a time with a warp-wide running sum, and
-// takes the first index whose running sum exceeds the target.
-// wsum: SMP_WARPS floats of shared memory; s_pick: one int.  Every thread returns the drawn index; *total_out
-// (nullable) receives the total of the weights.
-template <typename W>
-__device__ __forceinline__ int smp_draw(W w, int V, float u, float* wsum, int* s_pick, float* total_out) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int chunk = (((V + SMP_WARPS - 1) / SMP_WARPS) + 31) & ~31;
-    const int i0 = min(V, warp * chunk), i1 = min(V, i0 + chunk);
-    float local = 0.f;
-    int last_pos = -1;
-    for (int i = i0 + lane; i < i1; i += 32) {
-        const float x = w(i);
-        local += x;
-        if (x > 0.f) last_pos = i;
+        for (int j = 0; j < SMC_REGS; ++j) x[j] = load(min(i0 + 32 * j + lane, V - 1));
+        if constexpr (RELMAX) {
+#pragma unroll
+            for (int j = 0; j < SMC_REGS; ++j) m = fmaxf(m, i0 + 32 * j + lane < i1 ? x[j] : -INFINITY);
+            m = warp_max(m);
+        }
+#pragma unroll
+        for (int j = 0; j < SMC_REGS; ++j) {
+            p[j] = i0 + 32 * j + lane < i1 ? weight(x[j], m) : 0.f;
+            local += p[j];
+        }
+    } else {
+        if constexpr (RELMAX) {
+#pragma unroll 8
+            for (int i = i0 + lane; i < i1; i += 32) m = fmaxf(m, load(i));
+            m = warp_max(m);
+        }
+#pragma unroll 8
+        for (int i = i0 + lane; i < i1; i += 32) local += weight(load(i), m);
     }
     local = warp_sum(local);
-    __syncthreads();
-    if (lane == 0) wsum[warp] = local;
-    if (tid == 0) *s_pick = -1;
-    __syncthreads();
-    if (tid == 0) {   // inclusive scan of the warps' sums in warp order
-        float run = 0.f;
-        for (int t = 0; t < SMP_WARPS; ++t) { run += wsum[t]; wsum[t] = run; }
+    if (lane < SMC_CLUSTER) {
+        st_dsmem_f32(smem_u32(&box[id].x), lane, m);
+        st_dsmem_f32(smem_u32(&box[id].y), lane, local);
     }
-    __syncthreads();
-    const float total = wsum[SMP_WARPS - 1];
+    cluster_sync_all();
+    // ranges 2 L and 2 L + 1 in lane L: common maximum, sums relative to it, inclusive running sums
+    const float2 a = box[2 * lane], b = box[2 * lane + 1];
+    const float M = warp_max(fmaxf(a.x, b.x));
+    const float sa = a.x > -INFINITY ? a.y * expf((a.x - M) * inv_t) : 0.f, sb = b.x > -INFINITY ? b.y * expf((b.x - M) * inv_t) : 0.f;
+    float incl = sa + sb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float q = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += q;
+    }
+    const float total = __shfl_sync(0xffffffffu, incl, 31);
+    const float prev = __shfl_up_sync(0xffffffffu, incl, 1);
+    const float before = lane > 0 ? prev : 0.f;                   // running sum ahead of this lane's pair
     const float target = u * total;
-    const float incl = wsum[warp], excl = warp > 0 ? wsum[warp - 1] : 0.f;
-    if (incl > target && excl <= target) {   // exactly one warp's range contains the target (warp-uniform condition)
+    if (m_out) *m_out = M;
+    if (total_out) *total_out = total;
+    // the first range whose running sum exceeds the target; rounding may leave none: then the last range with any weight
+    const bool in_a = before + sa > target;
+    const unsigned hit = __ballot_sync(0xffffffffu, in_a || incl > target), some = __ballot_sync(0xffffffffu, sa > 0.f || sb > 0.f);
+    const int from = hit ? __ffs(hit) - 1 : (some ? 31 - __clz(some) : 0);
+    const bool second = hit ? !in_a : sb > 0.f;
+    const bool own_second = __shfl_sync(0xffffffffu, (int)second, from) != 0;
+    const float excl = __shfl_sync(0xffffffffu, second ? before + sa : before, from);
+    if (2 * from + (own_second ? 1 : 0) != id) return -1;
+    const float f = m > -INFINITY ? expf((m - M) * inv_t) : 0.f;
+    int pick = -1, last = -1;                                     // last: the range's last positive weight, where rounding fell short of the target
+    if (in_regs) {
+        // sums of the 32-weight pieces (lanes 2 j and 2 j + 1 get piece j), then the piece that contains the target
+        float q[SMC_REGS];
+#pragma unroll
+        for (int j = 0; j < SMC_REGS; ++j) q[j] = p[j];
+        const float two = warp_sum_many<SMC_REGS>(q, lane) * f;
+        const float piece = __shfl_sync(0xffffffffu, two, (2 * lane) & 31);
+        float run = lane < SMC_REGS ? piece : 0.f;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float t = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += t;
+        }
+        const unsigned ph = __ballot_sync(0xffffffffu, lane < SMC_REGS && excl + run > target);
+        if (hit && ph) {
+            const int j = __ffs(ph) - 1;
+            const float upto = __shfl_sync(0xffffffffu, run, max(j - 1, 0));
+            const float ahead = excl + (j > 0 ? upto : 0.f);
+            float x = 0.f;
+#pragma unroll
+            for (int jj = 0; jj < SMC_REGS; ++jj) if (jj == j) x = p[jj];
+            x *= f;
+            float s = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const float t = __shfl_up_sync(0xffffffffu, s, o);
+                if (lane >= o) s += t;
+            }
+            const unsigned eh = __ballot_sync(0xffffffffu, ahead + s > target), pos = __ballot_sync(0xffffffffu, x > 0.f);
+            if (eh) pick = i0 + 32 * j + __ffs(eh) - 1;
+            else if (pos) pick = i0 + 32 * j + 31 - __clz(pos);
+        }
+#pragma unroll
+        for (int j = 0; j < SMC_REGS; ++j) if (p[j] > 0.f) last = i0 + 32 * j + lane;
+    } else {
         float run = excl;
-        int pick = -1;
         for (int base = i0; base < i1 && pick < 0; base += 32) {
             const int i = base + lane;
-            float p = i < i1 ? w(i) : 0.f;
+            const float x = i < i1 ? weight(load(i), m) * f : 0.f;
+            if (x > 0.f) last = i;
+            float s = x;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {   // inclusive running sum over the 32 lanes
-                const float q = __shfl_up_sync(0xffffffffu, p, o);
-                if (lane >= o) p += q;
+            for (int o = 1; o < 32; o <<= 1) {
+                const float t = __shfl_up_sync(0xffffffffu, s, o);
+                if (lane >= o) s += t;
             }
-            const unsigned hit = __ballot_sync(0xffffffffu, run + p > target);
-            if (hit) pick = base + __ffs(hit) - 1;
-            run += __shfl_sync(0xffffffffu, p, 31);
+            const unsigned eh = __ballot_sync(0xffffffffu, run + s > target);
+            if (hit && eh) pick = base + __ffs(eh) - 1;
+            run += __shfl_sync(0xffffffffu, s, 31);
         }
-        if (pick < 0) {   // rounding: the second walk fell just short of the target: the range's last positive weight
-            int lp = last_pos;
+    }
+    if (pick < 0) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) lp = max(lp, __shfl_xor_sync(0xffffffffu, lp, o));
-            pick = lp;
-        }
-        if (lane == 0) *s_pick = pick;
+        for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+        pick = max(last, 0);   // (all weights zero: index 0)
     }
-    __syncthreads();
-    if (*s_pick < 0) {   // rounding left no range beyond the target: the last index with a positive weight
-        __syncthreads();
-        atomicMax(s_pick, last_pos);
-        __syncthreads();
-    }
-    if (total_out) *total_out = total;
-    return max(*s_pick, 0);   // (all weights zero: index 0)
+    return pick;
 }
 
-// Draft s of every live sequence, drawn from softmax(logits / temp).  logits: [batch][V] of draft step s.
-// grid: batch; block: SMP_THREADS.
-__global__ void __launch_bounds__(SMP_THREADS) sample_draft_kernel(LoopState st, const float* __restrict__ logits, int V, int s,
-                                                                   float temp, unsigned long long seed) {
-    __shared__ float red[SMP_WARPS], scan[SMP_WARPS];
-    __shared__ int s_pick;
+// Draft s of every live sequence, drawn from softmax(logits / temp).  logits: [batch][V] of draft step s; stats[b] receives
+// the row's maximum and the sum of its weights.  grid: (SMC_CLUSTER, batch), a cluster per sequence; block: SMC_THREADS.
+__global__ void __launch_bounds__(SMC_THREADS) sample_draft_kernel(LoopState st, const float* __restrict__ logits, int V, int s,
+                                                                   float temp, unsigned long long seed, float2* __restrict__ stats) {
+    __shared__ float2 box[SMC_RANGES];
+    cluster_arrive_relaxed();   // opening handshake
     pdl_wait();
     pdl_launch_dependents();
-    const int b = blockIdx.x;
+    cluster_wait();
+    const int b = blockIdx.y;
     const float* row = logits + (size_t)b * V;
-    const float m = smp_row_max(row, V, red);
     const float inv_t = 1.0f / temp;
     const float u = uniform_variate(seed, b, st.counters[0], s);
-    const int tok = smp_draw([&](int i) { return expf((__ldcg(row + i) - m) * inv_t); }, V, u, scan, &s_pick, nullptr);
-    if (threadIdx.x == 0) st.drafts[b * st.gamma_limit + s] = tok;
+    float m, z;
+    const int tok = smc_draw<true>([&](int i) { return __ldcg(row + i); }, [&](float x, float mx) { return expf((x - mx) * inv_t); }, V, blockIdx.x,
+                                   inv_t, u, box, &m, &z);
+    if (tok >= 0 && (threadIdx.x & 31) == 0) { st.drafts[b * st.gamma_limit + s] = tok; stats[b] = make_float2(m, z); }
 }
 
-// Accept / redraw decisions of one iteration, one CTA per sequence: writes accept_len[b] and, at index accept_len of
-// the sequence's target array, the token that follows the kept drafts.  The bookkeeping (emit, advance n, publish)
-// is done by verify_kernel in mode 4, which takes these decisions as given.
-// logits_large: [batch][gamma+1][V]; logits_small: [gamma][batch][V].  grid: batch; block: SMP_THREADS.
-__global__ void __launch_bounds__(SMP_THREADS) sample_verify_kernel(LoopState st, int batch, int gamma, const float* __restrict__ logits_large,
-                                                                    const float* __restrict__ logits_small, int V, float temp_large,
-                                                                    float temp_small, unsigned long long seed) {
-    __shared__ float red[SMP_WARPS], scan[SMP_WARPS];
-    __shared__ int s_pick;
+// Maximum and sum of weights of every row of the large model's block.  logits: [rows][V].
+// grid: (SMC_CLUSTER, rows); block: SMC_THREADS.
+__global__ void __launch_bounds__(SMC_THREADS) sample_stats_kernel(const float* __restrict__ logits, int V, float temp, float2* __restrict__ stats) {
+    __shared__ float2 box[SMC_RANGES];
+    cluster_arrive_relaxed();   // opening handshake
     pdl_wait();
     pdl_launch_dependents();
-    const int b = blockIdx.x;
-    if (st.done[b]) return;
+    cluster_wait();
+    const float* row = logits + (size_t)blockIdx.y * V;
+    const float inv_t = 1.0f / temp;
+    float m, z;
+    smc_draw<true>([&](int i) { return __ldcg(row + i); }, [&](float x, float mx) { return expf((x - mx) * inv_t); }, V, blockIdx.x, inv_t, 0.f, box,
+                   &m, &z);
+    if (blockIdx.x == 0 && threadIdx.x == 0) stats[blockIdx.y] = make_float2(m, z);
+}
+
+// Accept / redraw decisions of one iteration, one cluster per sequence: writes accept_len[b] and, at index accept_len of
+// the sequence's target array, the token that follows the kept drafts.  The bookkeeping (emit, advance n, publish)
+// is done by verify_kernel in mode 4, which takes these decisions as given.
+// logits_large: [batch][gamma+1][V] with stats_large per row; logits_small: [gamma][batch][V] with stats_small per row.
+// grid: (SMC_CLUSTER, batch); block: SMC_THREADS.
+__global__ void __launch_bounds__(SMC_THREADS) sample_verify_kernel(LoopState st, int batch, int gamma, const float* __restrict__ logits_large,
+                                                                    const float* __restrict__ logits_small, int V, float temp_large,
+                                                                    float temp_small, unsigned long long seed,
+                                                                    const float2* __restrict__ stats_large, const float2* __restrict__ stats_small) {
+    __shared__ float2 box[SMC_RANGES];
+    cluster_arrive_relaxed();   // opening handshake
+    pdl_wait();
+    pdl_launch_dependents();
+    cluster_wait();
+    const int b = blockIdx.y, lane = threadIdx.x & 31;
+    if (st.done[b]) return;     // (uniform over the cluster)
     const int iteration = st.counters[0];
     const float inv_tl = 1.0f / temp_large, inv_ts = 1.0f / temp_small;
-    const int* d = st.drafts + b * st.gamma_limit;
-    int a = 0;
-    float mL = 0.f, mS = 0.f, zL = 1.f, zS = 1.f;
-    const float* lrow = logits_large + (size_t)b * (gamma + 1) * V;
-    const float* srow = nullptr;
-    for (; a < gamma; ++a) {
-        lrow = logits_large + ((size_t)b * (gamma + 1) + a) * V;
-        srow = logits_small + ((size_t)a * batch + b) * V;
-        mL = smp_row_max(lrow, V, red);
-        mS = smp_row_max(srow, V, red);
-        // the two normalisers, each summed in the draw's own order (segments front to back, then in thread order)
-        smp_draw([&](int i) { return expf((__ldcg(lrow + i) - mL) * inv_tl); }, V, 0.f, scan, &s_pick, &zL);
-        smp_draw([&](int i) { return expf((__ldcg(srow + i) - mS) * inv_ts); }, V, 0.f, scan, &s_pick, &zS);
-        const int tok = d[a];
-        const float pL = expf((__ldcg(lrow + tok) - mL) * inv_tl) / zL;
-        const float pS = expf((__ldcg(srow + tok) - mS) * inv_ts) / zS;
+    // lane a tests draft a (every warp for itself); the first rejection is the accept length
+    bool rejected = false;
+    if (lane < gamma) {
+        const float* lrow = logits_large + ((size_t)b * (gamma + 1) + lane) * V;
+        const float* srow = logits_small + ((size_t)lane * batch + b) * V;
+        const int tok = st.drafts[b * st.gamma_limit + lane];
+        const float2 sl = __ldcg(stats_large + b * (gamma + 1) + lane), ss = __ldcg(stats_small + lane * batch + b);
+        const float pL = expf((__ldcg(lrow + tok) - sl.x) * inv_tl) / sl.y;
+        const float pS = expf((__ldcg(srow + tok) - ss.x) * inv_ts) / ss.y;
         const float ratio = pS > 0.f ? fminf(1.0f, pL / pS) : 1.0f;
-        const float u = uniform_variate(seed, b, iteration, SMP_SLOT_ACCEPT + a);
-        if (!(u < ratio)) break;   // rejected: redraw below from this position's distributions
+        rejected = !(uniform_variate(seed, b, iteration, SMP_SLOT_ACCEPT + lane) < ratio);
     }
+    const unsigned mask = __ballot_sync(0xffffffffu, rejected);
+    const int a = mask ? __ffs(mask) - 1 : gamma;
     const float u = uniform_variate(seed, b, iteration, SMP_SLOT_REDRAW);
-    int tok;
-    if (a < gamma) {
-        const float* lr = lrow;
-        const float* sr = srow;
-        const float cl = 1.0f / zL, cs = 1.0f / zS;
-        tok = smp_draw([&](int i) {
-            return fmaxf(expf((__ldcg(lr + i) - mL) * inv_tl) * cl - expf((__ldcg(sr + i) - mS) * inv_ts) * cs, 0.f);
-        }, V, u, scan, &s_pick, nullptr);
-    } else {
-        const float* lr = logits_large + ((size_t)b * (gamma + 1) + gamma) * V;
-        const float m = smp_row_max(lr, V, red);
-        tok = smp_draw([&](int i) { return expf((__ldcg(lr + i) - m) * inv_tl); }, V, u, scan, &s_pick, nullptr);
-    }
-    if (threadIdx.x == 0) {
+    // the positive part of p - q at the first rejection, or the large model's next distribution
+    const float* lr = logits_large + ((size_t)b * (gamma + 1) + a) * V;
+    const float* sr = logits_small + ((size_t)(a < gamma ? a : 0) * batch + b) * V;
+    const float2 sl = __ldcg(stats_large + b * (gamma + 1) + a);
+    const float2 ss = a < gamma ? __ldcg(stats_small + a * batch + b) : make_float2(0.f, 1.f);
+    const float cl = 1.0f / sl.y, cs = 1.0f / ss.y;
+    int tok = smc_draw<false>([&](int i) { return make_float2(__ldcg(lr + i), a < gamma ? __ldcg(sr + i) : 0.f); },
+                              [&](float2 x, float) {
+                                  const float l = expf((x.x - sl.x) * inv_tl);
+                                  return a < gamma ? fmaxf(l * cl - expf((x.y - ss.x) * inv_ts) * cs, 0.f) : l;
+                              }, V, blockIdx.x, inv_tl, u, box, nullptr, nullptr);
+    if (lane != 0) tok = -1;
+    if (tok >= 0) {
         st.accept_len[b] = a;
         st.targets[b * (st.gamma_limit + 1) + a] = tok;
     }

@@ -54,6 +54,7 @@ struct Layout {   // byte offsets into the arena
     size_t stage;                                   // a prompt pass's lengths, offsets and token ids as the host staged them
     size_t attn_counters;   // inside the zero-filled state block
     size_t h_large, h_small, a, q, o, f, xb, t1, yhat, a_s, logits_large, logits_small, part_ml, part_acc, dbg;
+    size_t smp_large, smp_small;                     // sampled SPEED: (maximum, sum of weights) of every row of logits
     size_t amax_val_large, amax_idx_large, amax_val_small, amax_idx_small;
     size_t a32, o32, f32;                           // value / remainder planes between the bf16 decode kernels: LayerNorm inputs (x.g) / attention / GELU outputs
     size_t ln_src, ln_rows_large, ln_rows_small, ln_stats;   // LayerNorms behind the GEMMs (bf16 decode): sources, their rows, the token rows' statistics
@@ -237,6 +238,7 @@ Layout make_layout(const tandem_config& c) {
     L.part_acc = take(RD * dmax * L.n_chunks_max * 4);
     L.dbg = take(T * dmax * 4);
     L.forced_ids = take(B * T * 4); L.forced_len = take(B * 4); L.forced_nll = take(B * T * 4); L.forced_top = take(B * T * 4);
+    L.smp_large = take(RD * 8); L.smp_small = take((size_t)std::max(1, c.gamma_max) * B * 8);
     L.vocab_tiles = cdiv(c.large.vocab, 128);
     L.amax_val_large = take(RD * L.vocab_tiles * 4); L.amax_idx_large = take(RD * L.vocab_tiles * 4);
     L.amax_val_small = take(B * L.vocab_tiles * 4); L.amax_idx_small = take(B * L.vocab_tiles * 4);
@@ -936,16 +938,19 @@ void launch_adaptive_begin(tandem_ctx& c) {
 // Sampled SPEED: draft s of every sequence drawn from the small model's logits of step s.
 void launch_sample_draft(tandem_ctx& c, int s, uint64_t seed) {
     const float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
-    ProfScope ps(c, PC_ARGMAX, (double)c.batch * c.small.d.vocab * 8.0);
-    launch_ex(c, true, 1, sample_draft_kernel, dim3(c.batch), dim3(SMP_THREADS), 0, c.st, logits, (int)c.small.d.vocab, s, c.temp_small,
-              (unsigned long long)seed);
+    ProfScope ps(c, PC_ARGMAX, (double)c.batch * c.small.d.vocab * 4.0);
+    launch_ex(c, true, SMC_CLUSTER, sample_draft_kernel, dim3(SMC_CLUSTER, c.batch), dim3(SMC_THREADS), 0, c.st, logits, (int)c.small.d.vocab, s,
+              c.temp_small, (unsigned long long)seed, at<float2>(c, c.lay.smp_small) + (size_t)s * c.batch);
 }
 // Sampled SPEED: accept / redraw decisions of the iteration, ahead of the verify kernel's bookkeeping.
 void launch_sample_verify(tandem_ctx& c, int gamma, uint64_t seed) {
-    ProfScope ps(c, PC_ARGMAX, (double)c.batch * (2 * gamma + 1) * c.large.d.vocab * 8.0);
-    launch_ex(c, true, 1, sample_verify_kernel, dim3(c.batch), dim3(SMP_THREADS), 0, c.st, c.batch, gamma,
-              (const float*)at<float>(c, c.lay.logits_large), (const float*)at<float>(c, c.lay.logits_small), (int)c.large.d.vocab,
-              c.temp_large, c.temp_small, (unsigned long long)seed);
+    const int rows = c.batch * (gamma + 1), V = c.large.d.vocab;
+    const float* logits = at<float>(c, c.lay.logits_large);
+    ProfScope ps(c, PC_ARGMAX, (double)(rows + 2 * c.batch) * V * 4.0);
+    launch_ex(c, true, SMC_CLUSTER, sample_stats_kernel, dim3(SMC_CLUSTER, rows), dim3(SMC_THREADS), 0, logits, V, c.temp_large, at<float2>(c, c.lay.smp_large));
+    launch_ex(c, true, SMC_CLUSTER, sample_verify_kernel, dim3(SMC_CLUSTER, c.batch), dim3(SMC_THREADS), 0, c.st, c.batch, gamma, logits,
+              (const float*)at<float>(c, c.lay.logits_small), V, c.temp_large, c.temp_small, (unsigned long long)seed,
+              (const float2*)at<float2>(c, c.lay.smp_large), (const float2*)at<float2>(c, c.lay.smp_small));
 }
 
 void fp32_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
@@ -1196,7 +1201,7 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
 }
 
 // Enqueues one iteration on the context's stream: eagerly the first time a launch shape is seen (and whenever
-// per-launch profiling is on), as a CUDA graph afterwards.  kind 0 = draft + verify, 1 = plain greedy M_L.
+// per-launch profiling is on), as a CUDA graph afterwards.  kind: see enqueue_iteration.
 tandem_status launch_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t seed, int max_new) {
     const int need = (c.n_ub - 1 + gamma) / ATT_CH + 1;
     c.chunks_launch = std::min(c.lay.n_chunks_max, (need + 3) / 4 * 4);
