@@ -923,11 +923,14 @@ void launch_router(tandem_ctx& c, int s, int gamma_max) {
     const float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
     ProfScope ps(c, PC_ARGMAX, (double)c.batch * c.small.d.vocab * 8.0);
     const size_t feat_bytes = sizeof(float) * (size_t)(1 + c.router.k + c.router.k * c.small.d.d_model);   // <= 48 KB, checked by tandem_set_router
+    static std::atomic<unsigned long long> attr_bf16{0}, attr_fp32{0};
+    if (c.cfg.dtype == TANDEM_DTYPE_BF16) ensure_dyn_smem(router_kernel<bf16>, 48 * 1024, attr_bf16);
+    else ensure_dyn_smem(router_kernel<float>, 48 * 1024, attr_fp32);   // (48 KB and the static part are more than the default limit)
     if (c.cfg.dtype == TANDEM_DTYPE_BF16)
-        launch_ex(c, true, 1, router_kernel<bf16>, dim3(c.batch), dim3(RT_THREADS), feat_bytes, c.st, c.batch, logits, (int)c.small.d.vocab, s, gamma_max,
+        launch_ex(c, true, RT_CLUSTER, router_kernel<bf16>, dim3(RT_CLUSTER, c.batch), dim3(RT_THREADS), feat_bytes, c.st, c.batch, logits, (int)c.small.d.vocab, s, gamma_max,
                   (const bf16*)w_emb(c, c.small), (int)c.small.d.d_model, c.router);
     else
-        launch_ex(c, true, 1, router_kernel<float>, dim3(c.batch), dim3(RT_THREADS), feat_bytes, c.st, c.batch, logits, (int)c.small.d.vocab, s, gamma_max,
+        launch_ex(c, true, RT_CLUSTER, router_kernel<float>, dim3(RT_CLUSTER, c.batch), dim3(RT_THREADS), feat_bytes, c.st, c.batch, logits, (int)c.small.d.vocab, s, gamma_max,
                   (const float*)w_emb(c, c.small), (int)c.small.d.d_model, c.router);
 }
 void launch_adaptive_begin(tandem_ctx& c) {
@@ -1209,7 +1212,9 @@ tandem_status launch_iteration(tandem_ctx& c, int kind, int gamma, int mode, uin
         c.chunks_launch = 1;   // the cluster attention's grid does not depend on the context length: one graph serves all
     if (kind == 3) c.router_ticket++; else c.ticket++;   // what the host will wait for: the router's or the verify kernel's publication
     if (kind != 3) c.last_gamma = kind == 1 ? 0 : gamma;   // (set here, not while enqueueing: a replayed graph enqueues nothing on the host)
-    if (c.prof.on || !c.use_graphs) {
+    // (a draft step of the adaptive block length starts when the host has seen the router's answer to the one before: a graph's
+    // launch would add its latency to every step, 12.8 ms against 11.5 ms for 48 tokens of the small pair)
+    if (c.prof.on || !c.use_graphs || kind == 3) {
         enqueue_iteration(c, kind, gamma, mode, seed, max_new);
         return check_launch();
     }

@@ -2,7 +2,7 @@
 import pytest
 
 from paper_2402_08644_b200 import binding, build, synth
-from test_gpu_parity import TOL_BF16, TOL_FP32, _bf16_weights, _replay_compare, gpu_toy_shape, prompts_for, toy_weights
+from test_gpu_parity import TOL_BF16, TOL_FP32, _adaptive_replay, _bf16_weights, _replay_compare, _sampled_replay, gpu_toy_shape, prompts_for, toy_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +47,14 @@ def test_bf16_layernorm_behind_the_product(batch, gamma, offset):
         w[tag + ".pos"] = synth.round_to_bf16(w[tag + ".pos"] + offset)
     prompts = prompts_for(shape, [1 + 3 * (b % 5) for b in range(batch)], seed=batch)
     assert _replay_compare(shape, w, prompts, gamma, 2, TOL_BF16, 2 * TOL_BF16) <= 10
+
+
+@pytest.mark.parametrize("vocab", [31, 2049, 32768, 32801])
+def test_sampling_and_router_over_a_cluster(vocab):
+    """Rows of logits dealt to eight CTAs: fewer logits than ranges, a ragged last range, the longest row that stays in registers
+    and one that does not; draws, accept decisions, router features and block lengths against the checker."""
+    shape = gpu_toy_shape(large=(1, 64, 2, 64), small=(1, 32, 1, 64), vocab=vocab, max_pos=48, layer_map=(1,))
+    w = toy_weights(shape, seed=2, std=0.3)
+    prompts = prompts_for(shape, [5, 9], seed=1)
+    _sampled_replay(shape, w, prompts, 3, 3, 0.7, 0.9, seed=11, tol=TOL_FP32, eps=2e-5)
+    _adaptive_replay(shape, w, prompts, 4, 3, TOL_FP32, 1e-4)
