@@ -20,9 +20,10 @@
 //                          stream (programmatic dependent launch), so they overlap its run; a kernel lets its
 //                          own successor start once the predecessor is done, which keeps one kernel's worth of
 //                          prefetch in flight (deeper chains of waiting kernels cost more than they hide).
-//  gemm_tc_tiled_kernel    many rows (prompt pass): 128 x 256 output tiles, both operands by TMA; persistent CTAs with two
-//                          accumulators in TMEM, so that a tile's epilogue runs under the next tile's MMAs.
-//  gemm_tc_split_kernel    prompt passes whose 128 x 256 tiles would leave multiprocessors idle: 128 x 128 tiles, one per
+//  gemm_tc_pair_kernel     many rows (prompt pass): 256 x 256 output tiles, one per pair of multiprocessors, both operands by
+//                          TMA; persistent, with two accumulators in TMEM, so that a tile's epilogue runs under the next
+//                          tile's MMAs.
+//  gemm_tc_split_kernel    prompt passes whose 256 x 256 tiles would leave multiprocessors idle: 128 x 128 tiles, one per
 //                          cluster of one, two or four CTAs that share the tile's K range.
 //
 // An output element's reduction order depends on (N, K) only, never on the number of rows, so a block
@@ -692,19 +693,20 @@ struct TcTiledArgs {
     int M, K, N;
     int seg_rows0, tiles0;   // first segment: output features, feature tiles
     int seg_rows, tiles_per_seg;
-    int tiles_n, tiles_m;    // feature tiles over all segments, 128-row tiles
+    int tiles_n, tiles_m;    // feature tiles over all segments, row tiles (of 256 in the pair kernel, else 128)
     int splits, stages;      // gemm_tc_split_kernel: CTAs that share a tile's K range, ring stages
+    int whole, parts;        // gemm_tc_pair_kernel: tiles done whole; parts that each of the remaining ones is cut into (1, 2, 4)
     int* err_flag;
     EpiArgs e;
 };
 
-constexpr int TCT_THREADS = 192;
-constexpr int TCT_TILE_BYTES = 128 * 128;          // one TMA box: 128 rows x 64 bf16
-constexpr int TCT_BN = 256;                        // output features per tile
-constexpr int TCT_STAGES = 4;
-constexpr int TCT_STAGE_BYTES = 3 * TCT_TILE_BYTES;   // token rows, then the weight rows (one box per 128)
-constexpr int TCT_SMEM_BYTES = TCT_STAGES * TCT_STAGE_BYTES + 1024;
-constexpr int TCT_GROUP_M = 16;                    // row tiles that share a sweep over the weights, see tct_tile
+constexpr int TCT_TILE_BYTES = 128 * 128;          // 128 rows x 64 bf16
+constexpr int TCP_THREADS = 320;   // warps 0-7: epilogue, two per 32 rows; warp 8: TMA; warp 9: TMEM + MMA issue
+constexpr int TCP_BN = 256;                           // output features per tile
+constexpr int TCP_STAGES = 6;
+constexpr int TCP_STAGE_BYTES = 2 * TCT_TILE_BYTES;   // this CTA's token rows, its half of the weight rows
+constexpr int TCP_SMEM_BYTES = TCP_STAGES * TCP_STAGE_BYTES + 1024;
+constexpr int TCP_GROUP_M = 8;                        // row tiles that share a sweep over the weights, see tcp_item
 
 // Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.
 template <int EPI>
@@ -749,8 +751,12 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int seg, int
             dst = static_cast<bf16*>(s == 0 ? e.kcache : e.vcache) + idx;
         }
     }
-    reinterpret_cast<uint4*>(dst)[0] = lo;
-    reinterpret_cast<uint4*>(dst)[1] = hi;
+    if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {   // (rows of an odd multiple of eight elements alternate)
+        st_global_u32x8(dst, lo, hi);
+    } else {
+        reinterpret_cast<uint4*>(dst)[0] = lo;
+        reinterpret_cast<uint4*>(dst)[1] = hi;
+    }
 }
 
 // Feature tile -> (segment, first feature within it).
@@ -759,64 +765,128 @@ __device__ __forceinline__ int tct_segment(const TcTiledArgs& a, int tile_n, int
     n_local0 = (seg == 0 ? tile_n : tile_n - a.tiles0 - (seg - 1) * a.tiles_per_seg) * width;
     return seg;
 }
-// Tile number -> (row tile, feature tile).  Row tiles in groups of TCT_GROUP_M, inside a group row tiles fastest: the CTAs
-// that run at the same time share 16 row tiles and about nine feature tiles, so the weights pass through L2 once per group
-// of row tiles.  With feature tiles fastest over all of them, three row tiles met the whole matrix at a time: at 64 row tiles
-// and 12288 x 4096 weights (100 MB, about the size of L2) that is 21 passes over the weights instead of four.
-__device__ __forceinline__ void tct_tile(const TcTiledArgs& a, int t, int& tile_m, int& tile_n) {
-    const int per_group = TCT_GROUP_M * a.tiles_n;
+// Work item -> (row tile, feature tile, first feature within the tile, width).  Row tiles go in groups of TCP_GROUP_M, inside
+// a group row tiles fastest: the pairs that run at the same time share eight row tiles and about nine feature tiles, so
+// the weights pass through L2 once per group of row tiles.  (With feature tiles fastest over all of them, few row tiles met
+// the whole matrix at a time: 12288 x 4096 weights are 100 MB, about the size of L2.)  Tiles that do not fill a last
+// round of all pairs are cut into two or four parts along the features, so that round costs a half or a quarter (12280 x
+// 2048: 384 tiles on 74 pairs are 5.2 rounds, 6 without).
+__device__ __forceinline__ void tcp_item(const TcTiledArgs& a, int item, int& tile_m, int& tile_n, int& c0, int& width) {
+    int t = item;
+    c0 = 0;
+    width = TCP_BN;
+    if (item >= a.whole) {
+        const int u = item - a.whole;
+        t = a.whole + u / a.parts;
+        width = TCP_BN / a.parts;
+        c0 = (u - (t - a.whole) * a.parts) * width;
+    }
+    const int per_group = TCP_GROUP_M * a.tiles_n;
     const int g = t / per_group, r = t - g * per_group;
-    const int gm = min(TCT_GROUP_M, a.tiles_m - g * TCT_GROUP_M);
+    const int gm = min(TCP_GROUP_M, a.tiles_m - g * TCP_GROUP_M);
     tile_n = r / gm;
-    tile_m = g * TCT_GROUP_M + r - tile_n * gm;
+    tile_m = g * TCP_GROUP_M + r - tile_n * gm;
 }
 
-// Persistent: grid = min(tiles, SMs) CTAs, CTA b takes output tiles b, b + grid, ... in the order of tct_tile.  The TMA ring
-// runs on across tile boundaries, and two accumulators in TMEM alternate, so that the epilogue of one tile (TMEM ->
-// registers -> global) overlaps the MMAs of the next.
-// dynamic smem TCT_SMEM_BYTES.
+// CW columns of an output row (= TMEM lane), TMEM -> registers -> global; acc: the first of them in this warp's lanes; n_local0:
+// its feature within the segment.  A thread moves whole 32-byte sectors of its row (with 16-byte accesses the residual
+// add fetched every sector of the stream twice).  The residual add has its first 64 old values in flight before the accumulator
+// is awaited, which `wait` does.
+template <int EPI, typename Wait>
+__device__ __forceinline__ void tcp_epilogue(const TcTiledArgs& a, uint32_t acc, int m, int seg, int seg_base, int seg_rows, int n_local0, int CW, Wait wait) {
+    if (EPI == EPI_RESID && n_local0 + CW <= seg_rows && (a.e.ldo & 7) == 0 && (seg_base & 7) == 0) {
+        float* prow = static_cast<float*>(a.e.out) + (size_t)min(m, a.M - 1) * a.e.ldo + seg_base + n_local0;
+        f32x8 cur[4], nxt[4];
+        auto load = [&](f32x8 (&o)[4], int c) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[j] = ld_global_f32x8(prow + c + 8 * j);
+        };
+        load(cur, 0);
+        if (CW > 32) load(nxt, 32);
+        if (!wait()) return;
+#pragma unroll 2
+        for (int c = 0; c < CW; c += 32) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                float v[16];
+                tmem_ld16(acc + c + 16 * q, v);   // warp-wide: every lane takes part
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { cur[2 * q].v[i] += v[i]; cur[2 * q + 1].v[i] += v[8 + i]; }
+                if (m < a.M) {
+                    st_global_f32x8(prow + c + 16 * q, cur[2 * q]);
+                    st_global_f32x8(prow + c + 16 * q + 8, cur[2 * q + 1]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
+            if (c + 64 < CW) load(nxt, c + 64);
+        }
+        return;
+    }
+    if (!wait()) return;
+#pragma unroll 1
+    for (int c = 0; c < CW; c += 16) {
+        float v[16];
+        tmem_ld16(acc + c, v);   // warp-wide: every lane takes part
+        if (m < a.M && n_local0 + c < seg_rows) epilogue16<EPI>(a.e, m, seg, seg_base, seg_rows, n_local0 + c, v);
+    }
+}
+
+// Persistent, on pairs of multiprocessors: a cluster of two CTAs computes a 256 x 256 tile with MMAs that span both (each CTA
+// brings its 128 token rows and one half of the 256 weight rows, and keeps its 128 rows of the accumulator), so a
+// multiprocessor reads a third less from L2 and shared memory per product than with a 128 x 256 tile of its own, and the ring
+// holds six K-blocks instead of four.  The first CTA's warp 9 issues the MMAs; both CTAs' loads count on its barriers; the
+// commits arrive on both CTAs' barriers.  The ring runs on across tile boundaries, and two accumulators in TMEM alternate.
+// Seconds-long loops under the power cap, against 128 x 256 tiles with four epilogue warps: 8191 x 12288 x 4096 656 -> 594 us
+// (1387 TFLOP/s), 8191 x 11008 x 4096 with GELU 585 -> 555 us, 8191 x 4096 x 11008 with the residual add 628 -> 579 us,
+// 12280 x 2048 x 2048 with the residual add 156 -> 108 us.
+// tmh*: the weights in boxes of 32 rows, for the parts of tiles.
+// grid: 2 * min(items, SMs / 2) in clusters of two; dynamic smem TCP_SMEM_BYTES.
 template <int EPI>
-__global__ void __launch_bounds__(TCT_THREADS)
-gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
-                     const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2) {
-    constexpr int BN = TCT_BN;
+__global__ void __launch_bounds__(TCP_THREADS)
+gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
+                    const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2,
+                    const __grid_constant__ CUtensorMap tmh0, const __grid_constant__ CUtensorMap tmh1, const __grid_constant__ CUtensorMap tmh2) {
+    constexpr int BN = TCP_BN;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_full[TCT_STAGES];
-    __shared__ __align__(8) uint64_t s_empty[TCT_STAGES];
+    __shared__ __align__(8) uint64_t s_full[TCP_STAGES];    // first CTA: both CTAs' loads of a stage
+    __shared__ __align__(8) uint64_t s_empty[TCP_STAGES];
     __shared__ __align__(8) uint64_t s_acc_full[2], s_acc_free[2];
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const int KB = (a.K + 63) >> 6;
-    const int total = a.tiles_n * a.tiles_m;
+    const int total = a.whole + (a.tiles_n * a.tiles_m - a.whole) * a.parts;
 
-    if (warp == 5) {
+    if (warp == 9) {
         if (lane == 0) {
-            for (int s = 0; s < TCT_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
-            for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&s_acc_full[s]), 1); mbar_init(smem_u32(&s_acc_free[s]), 4); }   // free: one arrive per epilogue warp
+            for (int s = 0; s < TCP_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&s_acc_full[s]), 1); mbar_init(smem_u32(&s_acc_free[s]), 16); }   // free: one arrive per epilogue warp of the pair
             mbar_init_fence();
         }
         __syncwarp();
-        tmem_alloc(smem_u32(&s_tmem), 2 * BN);
-        tmem_relinquish();
+        tmem_alloc_pair(smem_u32(&s_tmem), 2 * BN);
+        tmem_relinquish_pair();
     }
     tc_fence_before_sync();
-    __syncthreads();
+    cluster_sync_all();          // both CTAs' barriers are initialised
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(s_tmem);
 
-    if (warp == 4) {
+    if (warp == 8) {
         if (elect_one()) { tma_prefetch_desc(&tmx); tma_prefetch_desc(&tm0); }
         pdl_wait();              // the token rows come from the kernel before this one
         int st = 0, round = 0;   // ring position, and how often the ring has gone round
         bool ok = true;
-        for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-            int tile_m, tile_n, n_local0;
-            tct_tile(a, t, tile_m, tile_n);
+        for (int t = pair; t < total && ok; t += n_pairs) {
+            int tile_m, tile_n, c0, width, n_local0;
+            tcp_item(a, t, tile_m, tile_n, c0, width);
             const int seg = tct_segment(a, tile_n, BN, n_local0);
-            const int m0 = tile_m * 128;
+            const int m0 = tile_m * 256 + rank * 128, n0 = n_local0 + c0 + rank * (width / 2);
             const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
+            const CUtensorMap* th = seg == 0 ? &tmh0 : (seg == 1 ? &tmh1 : &tmh2);
             for (int i = 0; i < KB; ++i) {
                 if (round > 0 && !mbar_wait_warp(smem_u32(&s_empty[st]), (uint32_t)(round - 1) & 1)) {
                     tc_report(a.err_flag, TC_ERR_SLOT);
@@ -824,103 +894,83 @@ gemm_tc_tiled_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
                     break;
                 }
                 if (elect_one()) {
-                    const uint32_t bar = smem_u32(&s_full[st]), dst = ring0 + st * TCT_STAGE_BYTES;
-                    mbar_arrive_expect_tx(bar, TCT_STAGE_BYTES);
-                    tma_load_2d_nohint(dst, &tmx, i * 64, m0, bar);
-#pragma unroll
-                    for (int hb = 0; hb < BN / 128; ++hb)   // rows past the segment's end arrive as zeros
-                        tma_load_2d_nohint(dst + (1 + hb) * TCT_TILE_BYTES, tw, i * 64, n_local0 + hb * 128, bar);
+                    const uint32_t bar = cluster_map(smem_u32(&s_full[st]), 0), dst = ring0 + st * TCP_STAGE_BYTES;
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&s_full[st]), 2 * TCT_TILE_BYTES + width * 128);
+                    tma_load_2d_pair(dst, &tmx, i * 64, m0, bar);                     // rows past the end arrive as zeros
+                    if (width == BN) tma_load_2d_pair(dst + TCT_TILE_BYTES, tw, i * 64, n0, bar);
+                    else
+                        for (int q = 0; q < width / 2; q += 32) tma_load_2d_pair(dst + TCT_TILE_BYTES + q * 128, th, i * 64, n0 + q, bar);
                 }
-                if (++st == TCT_STAGES) { st = 0; ++round; }
+                if (++st == TCP_STAGES) { st = 0; ++round; }
             }
         }
         pdl_launch_dependents();
         __syncwarp();
-    } else if (warp == 5) {
-        constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
-        int st = 0, round = 0;
-        bool ok = true;
-        int it = 0;
-        for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++it) {
-            const int buf = it & 1;
-            // the accumulator's previous tile (two tiles back) must have been read out
-            if (it >= 2 && !mbar_wait_warp(smem_u32(&s_acc_free[buf]), (uint32_t)((it >> 1) - 1) & 1)) {
-                tc_report(a.err_flag, TC_ERR_ACCUM);
-                break;
-            }
-            tc_fence_after_sync();
-            for (int i = 0; i < KB; ++i) {
-                if (!mbar_wait_warp(smem_u32(&s_full[st]), (uint32_t)round & 1)) {
-                    tc_report(a.err_flag, TC_ERR_OPERANDS);
-                    ok = false;
+    } else if (warp == 9) {
+        if (rank == 0) {
+            int st = 0, round = 0;
+            bool ok = true;
+            int it = 0;
+            for (int t = pair; t < total && ok; t += n_pairs, ++it) {
+                const int buf = it & 1;
+                const uint32_t idesc = t < a.whole ? umma_idesc_bf16(256, BN) : umma_idesc_bf16(256, BN / a.parts);
+                // the accumulator's previous tile (two tiles back) must have been read out by both CTAs
+                if (it >= 2 && !mbar_wait_warp(smem_u32(&s_acc_free[buf]), (uint32_t)((it >> 1) - 1) & 1)) {
+                    tc_report(a.err_flag, TC_ERR_ACCUM);
                     break;
                 }
                 tc_fence_after_sync();
-                if (elect_one()) {
-                    const uint64_t da = umma_desc_k_sw128(ring0 + st * TCT_STAGE_BYTES);
-                    const uint64_t db = umma_desc_k_sw128(ring0 + st * TCT_STAGE_BYTES + TCT_TILE_BYTES);
+                for (int i = 0; i < KB; ++i) {
+                    if (!mbar_wait_warp(smem_u32(&s_full[st]), (uint32_t)round & 1)) {
+                        tc_report(a.err_flag, TC_ERR_OPERANDS);
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+                        const uint64_t da = umma_desc_k_sw128(ring0 + st * TCP_STAGE_BYTES);
+                        const uint64_t db = umma_desc_k_sw128(ring0 + st * TCP_STAGE_BYTES + TCT_TILE_BYTES);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_bf16(tmem + buf * BN, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
-                    umma_commit(smem_u32(&s_empty[st]));
+                        for (int k = 0; k < 4; ++k) umma_bf16_pair(tmem + buf * BN, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
+                        umma_commit_pair(smem_u32(&s_empty[st]));
+                    }
+                    if (++st == TCP_STAGES) { st = 0; ++round; }
                 }
-                if (++st == TCT_STAGES) { st = 0; ++round; }
+                if (elect_one()) umma_commit_pair(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
             }
-            if (elect_one()) umma_commit(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
         }
         __syncwarp();
     } else {
         pdl_wait();
         int it = 0;
-        for (int t = blockIdx.x; t < total; t += gridDim.x, ++it) {
+        for (int t = pair; t < total; t += n_pairs, ++it) {
             const int buf = it & 1;
-            int tile_m, tile_n, n_local0;
-            tct_tile(a, t, tile_m, tile_n);
+            int tile_m, tile_n, c0, width, n_local0;
+            tcp_item(a, t, tile_m, tile_n, c0, width);
             const int seg = tct_segment(a, tile_n, BN, n_local0);
+            const int col = (warp >> 2) * (width / 2);                    // this warp's half of the columns
             const int seg_rows = seg == 0 ? a.seg_rows0 : a.seg_rows;
             const int seg_base = seg == 0 ? 0 : a.seg_rows0 + (seg - 1) * a.seg_rows;
-            if (!mbar_wait(smem_u32(&s_acc_full[buf]), (uint32_t)(it >> 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); break; }
-            tc_fence_after_sync();
-            const int m = tile_m * 128 + warp * 32 + lane;   // output row = TMEM lane
-            const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16) + buf * BN;
-            if (EPI == EPI_RESID && n_local0 + BN <= seg_rows && (a.e.ldo & 3) == 0 && (seg_base & 3) == 0) {
-                // residual add on whole tiles: the old values of 64 columns are fetched together (sixteen 16-byte loads in
-                // flight) before the accumulator is read, instead of one exposed round trip per 16 columns
-                float* prow = static_cast<float*>(a.e.out) + (size_t)min(m, a.M - 1) * a.e.ldo + seg_base + n_local0;
-#pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 64) {
-                    float4 old[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) old[j] = __ldcg(reinterpret_cast<const float4*>(prow + c0) + j);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float v[16];
-                        tmem_ld16(acc + c0 + 16 * q, v);   // warp-wide: every lane takes part
-                        if (m < a.M) {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const float4 o = old[4 * q + i];
-                                reinterpret_cast<float4*>(prow + c0 + 16 * q)[i] =
-                                    make_float4(v[4 * i] + o.x, v[4 * i + 1] + o.y, v[4 * i + 2] + o.z, v[4 * i + 3] + o.w);
-                            }
-                        }
-                    }
-                }
-            } else {
-#pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(acc + c0, v);   // warp-wide: every lane takes part
-                    if (m < a.M && n_local0 + c0 < seg_rows) epilogue16<EPI>(a.e, m, seg, seg_base, seg_rows, n_local0 + c0, v);
-                }
-            }
+            bool ok = true;
+            auto wait = [&]() {
+                ok = mbar_wait(smem_u32(&s_acc_full[buf]), (uint32_t)(it >> 1) & 1);
+                if (!ok) tc_report(a.err_flag, TC_ERR_ACCUM);
+                tc_fence_after_sync();
+                return ok;
+            };
+            const int m = tile_m * 256 + rank * 128 + (warp & 3) * 32 + lane;   // output row = TMEM lane
+            const uint32_t acc = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + buf * BN + col;
+            tcp_epilogue<EPI>(a, acc, m, seg, seg_base, seg_rows, n_local0 + c0 + col, width / 2, wait);
+            if (!ok) break;
             tc_fence_before_sync();   // this warp's TMEM reads are done: the accumulator may be overwritten
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_acc_free[buf]));
+            if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(&s_acc_free[buf]), 0));
         }
     }
     tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 5) tmem_dealloc(tmem, 2 * BN);
+    cluster_sync_all();           // nobody leaves while the other CTA's operands or accumulators are in use
+    tc_fence_after_sync();
+    if (warp == 9) tmem_dealloc_pair(tmem, 2 * BN);
 }
 
 // Prompt passes of few tiles (the small pair's 511 rows: 32 tiles of 128 x 128 for N = 1024): a tile's time is its

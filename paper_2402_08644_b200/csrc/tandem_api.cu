@@ -126,6 +126,7 @@ struct tandem_ctx {
     bool use_pdl = true;                 // programmatic dependent launch between the decode kernels
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
+    std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
     // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
     // TMA: maps of the residual stream (times the next LayerNorm's gain) / attention / GELU buffers, [buffer 0..2][0 large,
     // 1 small], 16-row boxes; and the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one).
@@ -346,6 +347,7 @@ bool make_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t c
 
 struct TcW {              // up to three weight matrices stacked along the output features
     CUtensorMap tm[3];
+    CUtensorMap part[3];  // the same in boxes of 32 rows (prompt pass)
     int n_segs, seg_rows0, seg_rows, K;   // rows of the first segment, rows of every further one
 };
 inline int tcw_n(const TcW& w) { return w.seg_rows0 + (w.n_segs - 1) * w.seg_rows; }
@@ -361,6 +363,9 @@ TcW tcw3(const tandem_ctx& c, int i0, int i1, int i2, int seg_rows0, int seg_row
     w.tm[0] = c.wmap[i0];
     w.tm[1] = c.wmap[i1 >= 0 ? i1 : i0];
     w.tm[2] = c.wmap[i2 >= 0 ? i2 : i0];
+    w.part[0] = c.wpart[i0];
+    w.part[1] = c.wpart[i1 >= 0 ? i1 : i0];
+    w.part[2] = c.wpart[i2 >= 0 ? i2 : i0];
     w.n_segs = 1 + (i1 >= 0) + (i2 >= 0);
     w.seg_rows0 = seg_rows0; w.seg_rows = seg_rows; w.K = K;
     return w;
@@ -482,7 +487,6 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     memset(&a, 0, sizeof(a));
     a.M = M; a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.seg_rows = w.seg_rows;
     a.err_flag = err; a.e = e;
-    a.tiles_m = cdiv(M, 128);
     const int n_sms = std::max(1, c.n_sms);
     auto feature_tiles = [&](int width) {
         a.tiles0 = cdiv(w.seg_rows0, width);
@@ -491,13 +495,22 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
         return (long long)a.tiles_n * a.tiles_m;
     };
     ProfScope ps(c, PC_GEMM_TC_TILED, 2.0 * M * (double)a.N * w.K);   // flops
-    const long long wide = feature_tiles(TCT_BN);
-    if (wide >= n_sms) {   // a 256-wide tile for every multiprocessor: each token-row tile read from shared memory feeds twice the MMA work of a square one
+    // Where 256 x 256 tiles give every pair of multiprocessors one; the tiles beyond the last full round of all pairs are cut into
+    // as many parts (1, 2 or 4) as still fit one round.
+    a.tiles_m = cdiv(M, 256);
+    const long long pair_tiles = feature_tiles(TCP_BN);
+    const int n_pairs = n_sms / 2;
+    if (n_pairs > 0 && pair_tiles >= n_pairs) {
+        const int rest = (int)(pair_tiles % n_pairs);
+        a.whole = (int)pair_tiles - rest;
+        a.parts = rest * 4 <= n_pairs ? 4 : (rest * 2 <= n_pairs ? 2 : 1);
         static std::atomic<unsigned long long> attr_done{0};
-        ensure_dyn_smem(gemm_tc_tiled_kernel<EPI>, TCT_SMEM_BYTES, attr_done);
-        launch_ex(c, true, 1, gemm_tc_tiled_kernel<EPI>, dim3(n_sms), dim3(TCT_THREADS), (size_t)TCT_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
+        ensure_dyn_smem(gemm_tc_pair_kernel<EPI>, TCP_SMEM_BYTES, attr_done);
+        launch_ex(c, true, 2, gemm_tc_pair_kernel<EPI>, dim3(2 * n_pairs), dim3(TCP_THREADS), (size_t)TCP_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2],
+                  w.part[0], w.part[1], w.part[2]);
         return TANDEM_OK;
     }
+    a.tiles_m = cdiv(M, 128);
     // Fewer: square tiles, and the K range of each dealt to as many CTAs (1, 2 or 4) as still get a multiprocessor of their
     // own and four 64-element K-blocks each (fewer would not pay for the exchange).
     const int tiles = (int)feature_tiles(TCS_BN), KB = cdiv(w.K, 64);
@@ -1396,10 +1409,12 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     if (e == cudaSuccess && cfg->dtype == TANDEM_DTYPE_BF16) {
         // one tensor map per weight matrix: [out_features][in_features], 128 x 64 tiles
         c->wmap.resize(c->w.size());
+        c->wpart.resize(c->w.size());
         c->wmap_ok.assign(c->w.size(), 0);
         bool ok = tmap_encoder() != nullptr;
         auto add = [&](int idx, int rows, int cols) {
-            if (ok && make_tmap_bf16(&c->wmap[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols)) c->wmap_ok[idx] = 1;
+            if (ok && make_tmap_bf16(&c->wmap[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols) &&
+                make_tmap_bf16(&c->wpart[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols, 32)) c->wmap_ok[idx] = 1;
             else ok = false;
         };
         for (const Model* m : {&c->large, &c->small}) {

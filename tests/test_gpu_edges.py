@@ -58,3 +58,12 @@ def test_sampling_and_router_over_a_cluster(vocab):
     prompts = prompts_for(shape, [5, 9], seed=1)
     _sampled_replay(shape, w, prompts, 3, 3, 0.7, 0.9, seed=11, tol=TOL_FP32, eps=2e-5)
     _adaptive_replay(shape, w, prompts, 4, 3, TOL_FP32, 1e-4)
+
+
+def test_bf16_pair_prompt_gemm_with_tiles_in_parts():
+    """256 x 256 tiles on pairs of multiprocessors: 2104 rows are nine row tiles, the last with 56 rows (none for the second CTA);
+    the tiles beyond the last full round of 74 pairs are cut into four parts (9 feature tiles: 81), two (27: 243) and left
+    whole (12.5: 117, ragged features too)."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, 2304, 18, 3200), small=(1, 128, 2, 256), max_pos=2120, layer_map=(1,))
+    w = _bf16_weights(shape, seed=6, std=0.02)
+    assert _replay_compare(shape, w, prompts_for(shape, [2105], seed=7), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 1
