@@ -694,7 +694,7 @@ struct TcTiledArgs {
     int seg_rows0, tiles0;   // first segment: output features, feature tiles
     int seg_rows, tiles_per_seg;
     int tiles_n, tiles_m;    // feature tiles over all segments, row tiles (of 256 in the pair kernel, else 128)
-    int splits, stages;      // gemm_tc_split_kernel: CTAs that share a tile's K range, ring stages
+    int splits;              // gemm_tc_split_kernel: CTAs that share a tile's K range
     int whole, parts;        // gemm_tc_pair_kernel: tiles done whole; parts that each of the remaining ones is cut into (1, 2, 4)
     int* err_flag;
     EpiArgs e;
@@ -978,30 +978,33 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
 // tile's K range is dealt to the S = 1, 2 or 4 CTAs of a cluster.  Each sends its partial sums of the columns that another
 // one finishes into that CTA's inbox (16-byte stores that count their bytes on the receiver's barrier, a lane per row, 512
 // contiguous bytes per warp and store), and CTA r finishes columns r * 128 / S ..: sums in slice order, then the
-// epilogue, which is S times shorter per CTA.  Eight epilogue warps, two per 32 rows.  One tile per cluster; with S = 1 two CTAs
-// share a multiprocessor (one's epilogue runs under the other's MMAs).
-// grid: tiles * S; dynamic smem tcs_smem_bytes(S).
+// epilogue, which is S times shorter per CTA.  Eight epilogue warps, two per 32 rows.  The inbox lies where the ring was: a
+// cluster barrier after the last product says that every ring is free.  That keeps a CTA at 97 KB, so that the next kernel's
+// CTAs sit beside it with their first weights loaded (with an inbox of its own a CTA of four took 176 KB, and every kernel
+// began with a cold start after the one before).  One tile per cluster.
+// grid: tiles * S; dynamic smem TCS_SMEM_BYTES.
 constexpr int TCS_THREADS = 320;   // warps 0-7: epilogue; warp 8: TMA; warp 9: TMEM + MMA issue
 constexpr int TCS_BN = 128;
+constexpr int TCS_STAGES = 3;
 constexpr int TCS_STAGE_BYTES = 2 * TCT_TILE_BYTES;
-constexpr int TCS_MAX_STAGES = 4;
-constexpr int tcs_stages(int S) { return S == 1 ? 3 : 4; }
-constexpr int tcs_smem_bytes(int S) { return tcs_stages(S) * TCS_STAGE_BYTES + (S == 1 ? 0 : (S - 1) * (128 * TCS_BN * 4 / S)) + 1024; }
-static_assert(2 * (tcs_smem_bytes(1) + 1024 + 1024) <= 227 * 1024 && tcs_smem_bytes(4) + 1024 <= 227 * 1024, "two CTAs per SM without a split, one with");
+constexpr int TCS_SMEM_BYTES = TCS_STAGES * TCS_STAGE_BYTES + 1024;
+static_assert(2 * (TCS_SMEM_BYTES + 1024 + 1024) <= 227 * 1024, "two CTAs per SM");
+static_assert(3 * (128 * TCS_BN * 4 / 4) <= TCS_STAGES * TCS_STAGE_BYTES && 128 * TCS_BN * 4 / 2 <= TCS_STAGES * TCS_STAGE_BYTES, "the inbox fits where the ring was");
 
 template <int EPI>
 __global__ void __launch_bounds__(TCS_THREADS)
 gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
                      const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2) {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_full[TCS_MAX_STAGES];
-    __shared__ __align__(8) uint64_t s_empty[TCS_MAX_STAGES];
+    __shared__ __align__(8) uint64_t s_full[TCS_STAGES];
+    __shared__ __align__(8) uint64_t s_empty[TCS_STAGES];
     __shared__ __align__(8) uint64_t s_accum, s_inbox;
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
-    const int S = a.splits, stages = a.stages;
+    const int S = a.splits;
+    constexpr int stages = TCS_STAGES;
     const int tile = blockIdx.x / S, sp = blockIdx.x - tile * S;           // sp = this CTA's rank in its cluster
     int n_local0;
     const int seg = tct_segment(a, tile % a.tiles_n, TCS_BN, n_local0);
@@ -1013,7 +1016,7 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
 
     if (warp == 9) {
         if (lane == 0) {
-            for (int s = 0; s < TCS_MAX_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            for (int s = 0; s < TCS_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
             mbar_init(smem_u32(&s_accum), 1);
             mbar_init(smem_u32(&s_inbox), 1);
             mbar_init_fence();
@@ -1026,8 +1029,6 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(s_tmem);
-    if (S > 1) cluster_arrive_relaxed();   // opening handshake: waited for just before the first remote store
-
     if (warp == 8) {
         const CUtensorMap* tw = seg == 0 ? &tm0 : (seg == 1 ? &tm1 : &tm2);
         const int n_pre = min(nkb, stages);
@@ -1055,7 +1056,8 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             if (++st == stages) { st = 0; ++round; }
         }
         pdl_launch_dependents();
-        if (S > 1) cluster_wait();
+        __syncwarp();
+        if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
     } else if (warp == 9) {
         constexpr uint32_t idesc = umma_idesc_bf16(128, TCS_BN);
         int st = 0, round = 0;
@@ -1072,19 +1074,21 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             if (++st == stages) { st = 0; ++round; }
         }
         if (elect_one()) umma_commit(smem_u32(&s_accum));
-        if (S > 1) cluster_wait();
+        __syncwarp();
+        if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
     } else {
         pdl_wait();
         const int quarter = warp & 3, half = warp >> 2;
         const int row = quarter * 32 + lane, m = m0 + row;   // output row = TMEM lane
         const uint32_t acc = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const int CS = TCS_BN / S;                           // columns that a CTA finishes
-        const uint32_t inbox0 = ring0 + stages * TCS_STAGE_BYTES;   // [S - 1 senders][CS / 4][128 rows] of four floats
+        const uint32_t inbox0 = ring0;                       // [S - 1 senders][CS / 4][128 rows] of four floats
         const uint32_t ibar = smem_u32(&s_inbox);
         if (!mbar_wait(smem_u32(&s_accum), 0)) tc_report(a.err_flag, TC_ERR_ACCUM);
         tc_fence_after_sync();
         if (S > 1) {
-            cluster_wait();   // closes the opening handshake: every CTA of the cluster is running
+            cluster_arrive_relaxed();   // this CTA's products have read its ring ...
+            cluster_wait();             // ... and so have the others'
             if (tid == 0) mbar_arrive_expect_tx(ibar, (uint32_t)((S - 1) * 128 * CS * 4));
             for (int q = 0; q < S; ++q) {
                 if (q == sp) continue;

@@ -517,10 +517,9 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     int S = 1;
     while (S < 4 && tiles * S * 2 <= n_sms && KB >= 8 * S) S *= 2;
     a.splits = S;
-    a.stages = tcs_stages(S);
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_tc_split_kernel<EPI>, std::max(tcs_smem_bytes(2), tcs_smem_bytes(4)), attr_done);
-    launch_ex(c, true, S, gemm_tc_split_kernel<EPI>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)tcs_smem_bytes(S), a, tmx, w.tm[0], w.tm[1], w.tm[2]);
+    ensure_dyn_smem(gemm_tc_split_kernel<EPI>, TCS_SMEM_BYTES, attr_done);
+    launch_ex(c, true, S, gemm_tc_split_kernel<EPI>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)TCS_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
     return TANDEM_OK;
 }
 
