@@ -344,9 +344,26 @@ class Tandem:
         return out
 
 
-# The stand-alone kernels run for a few microseconds, so their wrappers keep the host's share below that: plain integers
-# as arguments (ctypes converts them by the declared types), no query that a given buffer makes unnecessary, and the
-# stream's handle without a Python stream object around it (14 us per short attention call before, 5 us now).
+# The stand-alone kernels run for a few microseconds: their calls go through a native module (csrc/standalone_py.cpp).
+_fast = None
+
+
+def _standalone():
+    global _fast
+    if _fast is None:
+        import importlib.machinery
+        import importlib.util
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        load_library()
+        path = os.path.join(os.path.dirname(_LIB_PATH), "_standalone.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build it first (python -m paper_2402_08644_b200.build)")
+        loader = importlib.machinery.ExtensionFileLoader("_standalone", path)
+        _fast = importlib.util.module_from_spec(importlib.util.spec_from_loader("_standalone", loader))
+        loader.exec_module(_fast)
+    return _fast
+
+
 def _stream_of(t):
     import torch
     return torch._C._cuda_getCurrentRawStream(t.get_device())
@@ -358,20 +375,10 @@ def _ptr_or_null(t):
 
 def tandem_decode_attention(q, k_derived, v_derived, k_own, v_own, out=None, scratch=None):
     """bf16 device tensors: q [B][H][dh]; k/v_derived [B][H][Td][dh]; k/v_own [B][H][To][dh].  Returns out."""
-    lib = _lib or load_library()
-    B, H, dh = q.shape
-    Td, To = k_derived.shape[2], k_own.shape[2]
-    if scratch is None or out is None:
-        import torch
-        if scratch is None:
-            scratch = torch.empty(lib.tandem_decode_attention_scratch_bytes(B, H, dh, Td, To), dtype=torch.uint8, device=q.device)
-        if out is None:
-            out = torch.empty_like(q)
-    status = lib.tandem_decode_attention(q.data_ptr(), _ptr_or_null(k_derived), _ptr_or_null(v_derived), _ptr_or_null(k_own), _ptr_or_null(v_own),
-                                         out.data_ptr(), scratch.data_ptr(), scratch.numel(), B, H, dh, Td, To, _stream_of(q))
-    if status:
-        _check(status, "tandem_decode_attention")
-    return out
+    r = (_fast or _standalone()).decode_attention(q, k_derived, v_derived, k_own, v_own, out, scratch)
+    if type(r) is int:
+        _check(r, "tandem_decode_attention")
+    return r
 
 
 STATIC_SCRATCH_BYTES = 64 * 1024
@@ -394,33 +401,18 @@ def tandem_decode_attention_static(q, k_derived, v_derived, k_own, v_own, out):
 
 def tandem_ff_tandem_project(x, w_t, ln_g, ln_b, wk, wv, scratch=None):
     """x [rows][d_L] bf16, w_t [d_S][d_L], ln_* [d_S] fp32, wk/wv [d_S][d_S] -> (k, v) [rows][d_S] bf16."""
-    import torch
-    lib = _lib or load_library()
-    rows, d_l = x.shape
-    d_s = w_t.shape[0]
-    k = torch.empty((rows, d_s), dtype=torch.bfloat16, device=x.device)
-    v = torch.empty_like(k)
-    if scratch is None:
-        scratch = torch.empty(lib.tandem_ff_tandem_project_scratch_bytes(rows, d_s), dtype=torch.uint8, device=x.device)
-    status = lib.tandem_ff_tandem_project(x.data_ptr(), w_t.data_ptr(), ln_g.data_ptr(), ln_b.data_ptr(), wk.data_ptr(), wv.data_ptr(),
-                                          k.data_ptr(), v.data_ptr(), scratch.data_ptr(), scratch.numel(), rows, d_l, d_s, _stream_of(x))
-    if status:
-        _check(status, "tandem_ff_tandem_project")
-    return k, v
+    r = (_fast or _standalone()).ff_tandem_project(x, w_t, ln_g, ln_b, wk, wv, scratch)
+    if type(r) is int:
+        _check(r, "tandem_ff_tandem_project")
+    return r
 
 
 def tandem_block_linear(x, w, y=None):
     """x [rows][K] bf16, w [N][K] bf16 -> y [rows][N] bf16 (rows <= 64)."""
-    lib = _lib or load_library()
-    rows, k = x.shape
-    n = w.shape[0]
-    if y is None:
-        import torch
-        y = torch.empty((rows, n), dtype=torch.bfloat16, device=x.device)
-    status = lib.tandem_block_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, k, n, _stream_of(x))
-    if status:
-        _check(status, "tandem_block_linear")
-    return y
+    r = (_fast or _standalone()).block_linear(x, w, y)
+    if type(r) is int:
+        _check(r, "tandem_block_linear")
+    return r
 
 
 def tandem_standalone_check(device=None) -> None:

@@ -345,6 +345,23 @@ bool make_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t c
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same, remembered: a tensor map depends on nothing but its arguments, and the stand-alone calls get the same matrices again
+// and again (an encoding costs the host about 0.4 us).  128 maps per thread, 24 KB, the last one to hash to a place stays.
+bool cached_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols) {
+    struct Entry { const void* base; uint64_t rows, cols; CUtensorMap tm; };
+    static thread_local std::vector<Entry> cache;
+    if (cache.empty()) cache.resize(128, Entry{nullptr, 0, 0, {}});
+    const uint64_t h = splitmix64(reinterpret_cast<uintptr_t>(base) ^ (rows << 40) ^ (cols << 20));
+    Entry& e = cache[h & 127];
+    if (e.base != base || e.rows != rows || e.cols != cols) {
+        e.base = nullptr;
+        if (!make_tmap_bf16(&e.tm, base, rows, cols, cols)) return false;
+        e.base = base; e.rows = rows; e.cols = cols;
+    }
+    *tm = e.tm;
+    return true;
+}
+
 struct TcW {              // up to three weight matrices stacked along the output features
     CUtensorMap tm[3];
     CUtensorMap part[3];  // the same in boxes of 32 rows (prompt pass)
@@ -2195,9 +2212,8 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
     float* yhat = reinterpret_cast<float*>(sc + pl.yhat);
     float* a_s = reinterpret_cast<float*>(sc + pl.a_s);
     TcW wt, wkv;
-    if (!make_tmap_bf16(&wt.tm[0], w_t, (uint64_t)d_small, (uint64_t)d_large, (uint64_t)d_large) ||
-        !make_tmap_bf16(&wkv.tm[0], wk, (uint64_t)d_small, (uint64_t)d_small, (uint64_t)d_small) ||
-        !make_tmap_bf16(&wkv.tm[1], wv, (uint64_t)d_small, (uint64_t)d_small, (uint64_t)d_small)) {
+    if (!cached_tmap_bf16(&wt.tm[0], w_t, (uint64_t)d_small, (uint64_t)d_large) || !cached_tmap_bf16(&wkv.tm[0], wk, (uint64_t)d_small, (uint64_t)d_small) ||
+        !cached_tmap_bf16(&wkv.tm[1], wv, (uint64_t)d_small, (uint64_t)d_small)) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled unavailable or failed");
         return TANDEM_ERR_CUDA;
     }
@@ -2229,7 +2245,7 @@ extern "C" tandem_status tandem_block_linear(const void* x, const void* w, void*
     if (((uintptr_t)x | (uintptr_t)w | (uintptr_t)y) & 15) return TANDEM_ERR_INVALID_ARG;
     StandaloneCtx tmp(stream);
     TcW tw;
-    if (!make_tmap_bf16(&tw.tm[0], w, (uint64_t)out_features, (uint64_t)in_features, (uint64_t)in_features)) {
+    if (!cached_tmap_bf16(&tw.tm[0], w, (uint64_t)out_features, (uint64_t)in_features)) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled unavailable or failed");
         return TANDEM_ERR_CUDA;
     }
