@@ -276,13 +276,15 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
 // warps' states in warp order, sends the result to the CTA that finishes the query (remote shared-memory stores),
 // and that CTA merges the CL states in rank order.  No global scratch, no second kernel.
 //
-// The two small products of a 16-position tile, S = Q K^T (16 query rows x 16 keys) and O += P V, run on the tensor
-// cores as warp-level m16n8k16 MMAs: with scalar FMAs and shuffles a block of gamma+1 queries is bound by
-// instruction issue at well under half of the memory bandwidth.  The query rows are the MMA's A rows (absent rows
-// are zero), K and V fragments come straight from the ring with ldmatrix (V transposed on the way), the softmax
-// works on the accumulator fragments (a row's 16 scores sit in the four lanes of a quad), and each probability
-// enters the second product as two bf16 numbers (value and remainder).  An output row depends on its own query row
-// only, so a block pass and a one-row pass give the same bits.  The probabilities use the fast exponential
+// The two small products of a 16-position tile run on the tensor cores as warp-level m16n8k16 MMAs, transposed: S^T = K Q^T with
+// the 16 keys as the MMA's rows and eight queries as its columns, O^T += V^T P^T with 16 elements of the head as rows.  (With
+// the queries as the 16 rows a block of up to eight of them left half of every MMA to absent rows, and these MMAs are slow,
+// about 32 clocks each on a quarter of a multiprocessor: 32 sequences x 16 heads x 64 x 8194 positions took 187-190 us a call, now
+// 169 us, 6.3 TB/s.)  K and V fragments come straight from the ring
+// with ldmatrix (V transposed on the way), the queries stay in registers, the softmax works on the accumulator fragments (a
+// query's 16 scores sit in eight lanes), and the probabilities become the second product's B fragments by an 8 x 8 register
+// transpose, each as two bf16 numbers (value and remainder).  A query's column depends on its own query only, so a block
+// pass and a one-row pass give the same bits.  The probabilities use the fast exponential
 // (2^x hardware approximation), well inside the bf16 tolerance.
 // ---------------------------------------------------------------------------------------------------
 constexpr int ATD_THREADS = 256;
@@ -291,7 +293,7 @@ constexpr int ATD_ERR_EXCHANGE = 5;                                 // error cod
 constexpr int ATD_CLUSTER = 8;                                      // largest cluster; launches use 1, 2, 4 or 8
 constexpr int ATD_SLOTS = ATT_NQ;                                   // inbox states per CTA: cluster size x queries it finishes <= 16
 constexpr int ATD_WROWS = ATT_CH / ATD_WARPS;                       // positions of a chunk per warp (16)
-static_assert(ATD_WROWS == 16 && ATT_NQ == 16, "one m16n8k16 tile per warp and chunk");
+static_assert(ATD_WROWS == 16, "one m16n8k16 tile per warp and chunk");
 
 template <int DH> struct AtdCfg {
     static constexpr int TPK = DH / 8;               // 16-byte units per key
@@ -299,8 +301,7 @@ template <int DH> struct AtdCfg {
     static constexpr int TILE_ELEMS = ATD_WROWS * DH;   // a warp's keys (or values) of one chunk
     static constexpr int STAGE_ELEMS = 2 * TILE_ELEMS;
     static constexpr int UNITS = ATD_WROWS * TPK / 32;  // 16-byte units per lane per tile
-    static constexpr int KSTEPS = DH / 16;           // MMAs along the head dimension for S
-    static constexpr int NTILES = DH / 8;            // 8-wide output tiles of O
+    static constexpr int KSTEPS = DH / 16;           // MMAs along the head dimension for S, 16-row tiles of O^T
 };
 template <int DH>
 constexpr size_t attn_decode_smem_bytes() {
@@ -330,13 +331,20 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// Transpose of an 8 x 8 matrix of 16-bit elements held as a fragment.
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
 __device__ __forceinline__ uint32_t atd_pack_bf16x2(float lo, float hi) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&p);
 }
 
 // grid: (CL, heads, sequences) with the CL CTAs along x forming one cluster, CL in {1, 2, 4, 8}; block: ATD_THREADS.
-template <int DH>
+// NT: groups of eight query columns in use (1 up to eight rows per CTA, 2 up to 16).
+template <int DH, int NT>
 __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     using C = AtdCfg<DH>;
     constexpr int NW = ATD_WARPS;
@@ -440,36 +448,43 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         }
     }
 
-    // The queries as A fragments: this lane holds rows lane/4 and lane/4 + 8, columns 2*(lane%4) (+1) (+8) of each
-    // 16-wide step along the head dimension.
-    const int row_lo = lane >> 2, row_hi = row_lo + 8, kc = 2 * (lane & 3);
-    // tile row -> (query head within the CTA, block row); rows beyond cnt are absent (zero queries, never stored)
-    const int hq_lo = row_lo < cnt ? row_lo / nq : 0, hq_hi = row_hi < cnt ? row_hi / nq : 0;
-    const int i_lo = row_lo < cnt ? row_lo - hq_lo * nq : 0, i_hi = row_hi < cnt ? row_hi - hq_hi * nq : 0;
-    uint32_t qf[C::KSTEPS][4];
-    {
-        const bf16* qg = static_cast<const bf16*>(a.q) + h * DH + kc;
-        const bf16* q_lo = qg + (size_t)(row0 + i_lo) * a.ldq + hq_lo * DH;
-        const bf16* q_hi = qg + (size_t)(row0 + i_hi) * a.ldq + hq_hi * DH;
+    // The queries as B fragments: this lane holds query 8 nt + lane/4, elements 2*(lane%4) (+1) (+8) of each 16-wide step along
+    // the head dimension; queries beyond cnt are absent (zero, never stored)
+    const int kc = 2 * (lane & 3);
+    uint32_t qf[NT][C::KSTEPS][2];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        const int rr = nt * 8 + (lane >> 2);
+        const int hq = rr < cnt ? rr / nq : 0, ib = rr < cnt ? rr - hq * nq : 0;      // query head within the CTA, block row
+        const bf16* qp = static_cast<const bf16*>(a.q) + (size_t)(row0 + ib) * a.ldq + (h + hq) * DH + kc;
 #pragma unroll
         for (int ks = 0; ks < C::KSTEPS; ++ks) {
-            qf[ks][0] = row_lo < cnt ? *reinterpret_cast<const uint32_t*>(q_lo + ks * 16) : 0u;
-            qf[ks][1] = row_hi < cnt ? *reinterpret_cast<const uint32_t*>(q_hi + ks * 16) : 0u;
-            qf[ks][2] = row_lo < cnt ? *reinterpret_cast<const uint32_t*>(q_lo + ks * 16 + 8) : 0u;
-            qf[ks][3] = row_hi < cnt ? *reinterpret_cast<const uint32_t*>(q_hi + ks * 16 + 8) : 0u;
+            qf[nt][ks][0] = rr < cnt ? *reinterpret_cast<const uint32_t*>(qp + ks * 16) : 0u;
+            qf[nt][ks][1] = rr < cnt ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 8) : 0u;
         }
     }
-    float o[C::NTILES][4];
+    // Accumulators: this lane's columns are queries 8 nt + kc + e, e = 0, 1; last position that each of them attends (-1: absent)
+    int q_last[NT][2];
+    float o[NT][C::KSTEPS][4];
+    float m[NT][2], l[NT][2];                            // l: this lane's keys only until the end
 #pragma unroll
-    for (int nt = 0; nt < C::NTILES; ++nt) { o[nt][0] = 0.f; o[nt][1] = 0.f; o[nt][2] = 0.f; o[nt][3] = 0.f; }
-    float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;   // l: this lane's keys only until the end
-    const bool has_hi = cnt > 8;
+    for (int nt = 0; nt < NT; ++nt) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int rr = nt * 8 + kc + e;
+            q_last[nt][e] = rr < cnt ? pos_first + rr % nq : -1;
+            m[nt][e] = -INFINITY;
+            l[nt][e] = 0.f;
+        }
+#pragma unroll
+        for (int mt = 0; mt < C::KSTEPS; ++mt) { o[nt][mt][0] = 0.f; o[nt][mt][1] = 0.f; o[nt][mt][2] = 0.f; o[nt][mt][3] = 0.f; }
+    }
 
     // ldmatrix row addresses of this lane (matrix lane/8, row lane%8), relative to the K (or V) tile of a stage
     const int lm_m = lane >> 3, lm_r = lane & 7;
-    const int lm_sw = DH >= 64 ? lm_r : (lm_r >> 1);
-    const uint32_t k_row = (uint32_t)(lm_r * DH * 2);                           // K: key = 8 * nt + row, unit = 4 * kp + matrix
-    const uint32_t v_row = (uint32_t)((((lm_m & 1) << 3) + lm_r) * DH * 2);     // V: key = 8 * (matrix & 1) + row, unit = 2 * np + matrix / 2
+    const uint32_t k_row = (uint32_t)((((lm_m & 1) << 3) + lm_r) * DH * 2);     // K: key = 8 * (matrix & 1) + row, unit = 2 * ks + matrix / 2
+    const uint32_t v_row = (uint32_t)((((lm_m >> 1) << 3) + lm_r) * DH * 2);    // V: key = 8 * (matrix / 2) + row, unit = 2 * mt + matrix & 1
+    const int k_sw = atd_swz<DH>(((lm_m & 1) << 3) + lm_r, 0), v_sw = atd_swz<DH>(((lm_m >> 1) << 3) + lm_r, 0);
 
     for (int it = 0; it < n_mine; ++it) {
         if (it + C::STAGES - 1 < n_mine) issue(it + C::STAGES - 1);
@@ -480,108 +495,87 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         const uint32_t ks_s = ring_s + (uint32_t)((it % C::STAGES) * C::STAGE_ELEMS * 2);
         const uint32_t vs_s = ks_s + (uint32_t)(C::TILE_ELEMS * 2);
 
-        // S = Q K^T for the tile's 16 keys: two 8-key halves
-        float sc[2][4];
+        // S^T = K Q^T for the tile's 16 keys; even and odd steps in two accumulators (half the dependent chain)
+        float sc[NT][2][4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-            sc[nt][0] = 0.f; sc[nt][1] = 0.f; sc[nt][2] = 0.f; sc[nt][3] = 0.f;
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int kp = 0; kp < C::KSTEPS / 2; ++kp) {
-                uint32_t kf[4];
-                ldmatrix_x4(ks_s + (uint32_t)(nt * 8 * DH * 2) + k_row + (uint32_t)((((kp * 4 + lm_m) ^ lm_sw)) << 4), kf);
-                mma_bf16_16816(sc[nt], qf[2 * kp], kf[0], kf[1]);
-                mma_bf16_16816(sc[nt], qf[2 * kp + 1], kf[2], kf[3]);
-            }
+            for (int b2 = 0; b2 < 2; ++b2) { sc[nt][b2][0] = 0.f; sc[nt][b2][1] = 0.f; sc[nt][b2][2] = 0.f; sc[nt][b2][3] = 0.f; }
+#pragma unroll
+        for (int ks = 0; ks < C::KSTEPS; ++ks) {
+            uint32_t kf[4];
+            ldmatrix_x4(ks_s + k_row + (uint32_t)(((ks * 2 + (lm_m >> 1)) ^ k_sw) << 4), kf);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(sc[nt][ks & 1], kf, qf[nt][ks][0], qf[nt][ks][1]);
         }
-        // scale, causal mask, running maxima (a row's scores sit in the four lanes of a quad).  Rows 8-15 are
-        // skipped when the block has at most eight queries: their state stays (-inf, 0, 0) and is never read.
-        float mc_lo = -INFINITY, mc_hi = -INFINITY;
+        // scale, causal mask, running maxima, probabilities: element (hh, e) is key t0 + lane/4 + 8 hh, query 8 nt + kc + e
+        uint32_t pf[NT][2], pr[NT][2];
+        float f[NT][2];
+        bool moved = false;
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
+        for (int nt = 0; nt < NT; ++nt) {
+            float p[2][2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const int ta = t0 + nt * 8 + kc + e;
-                sc[nt][e] = (row_lo < cnt && ta <= pos_first + i_lo) ? sc[nt][e] * a.scale : -INFINITY;
-                mc_lo = fmaxf(mc_lo, sc[nt][e]);
-                if (has_hi) {
-                    sc[nt][2 + e] = (row_hi < cnt && ta <= pos_first + i_hi) ? sc[nt][2 + e] * a.scale : -INFINITY;
-                    mc_hi = fmaxf(mc_hi, sc[nt][2 + e]);
-                }
+                const int key = t0 + (lane >> 2);
+                float x0 = (sc[nt][0][e] + sc[nt][1][e]) * a.scale, x1 = (sc[nt][0][2 + e] + sc[nt][1][2 + e]) * a.scale;
+                x0 = key <= q_last[nt][e] ? x0 : -INFINITY;
+                x1 = key + 8 <= q_last[nt][e] ? x1 : -INFINITY;
+                float mc = fmaxf(x0, x1);
+                mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 4));
+                mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 8));
+                mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 16));
+                const float mn = fmaxf(m[nt][e], mc);
+                f[nt][e] = m[nt][e] > -INFINITY ? __expf(m[nt][e] - mn) : (mn > -INFINITY ? 0.f : 1.f);
+                m[nt][e] = mn;
+                moved = moved || f[nt][e] != 1.f;
+                p[0][e] = mn > -INFINITY ? __expf(x0 - mn) : 0.f;
+                p[1][e] = mn > -INFINITY ? __expf(x1 - mn) : 0.f;
+                l[nt][e] = l[nt][e] * f[nt][e] + (p[0][e] + p[1][e]);
             }
-        }
-        mc_lo = fmaxf(mc_lo, __shfl_xor_sync(0xffffffffu, mc_lo, 1));
-        mc_lo = fmaxf(mc_lo, __shfl_xor_sync(0xffffffffu, mc_lo, 2));
-        const float mn_lo = fmaxf(m_lo, mc_lo);
-        const float f_lo = m_lo > -INFINITY ? __expf(m_lo - mn_lo) : 0.f;
-        m_lo = mn_lo;
-        float mn_hi = -INFINITY, f_hi = 1.f;
-        if (has_hi) {
-            mc_hi = fmaxf(mc_hi, __shfl_xor_sync(0xffffffffu, mc_hi, 1));
-            mc_hi = fmaxf(mc_hi, __shfl_xor_sync(0xffffffffu, mc_hi, 2));
-            mn_hi = fmaxf(m_hi, mc_hi);
-            f_hi = m_hi > -INFINITY ? __expf(m_hi - mn_hi) : 0.f;
-            m_hi = mn_hi;
-        }
-        // probabilities as the sum of two bf16 numbers (the rounded value and the rounded remainder): the second
-        // product then sees them to about 16 significant bits instead of 8, at the price of a second MMA
-        uint32_t pf[4], pr[4];
-        float ls_lo = 0.f, ls_hi = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-            const float p0 = mn_lo > -INFINITY ? __expf(sc[nt][0] - mn_lo) : 0.f, p1 = mn_lo > -INFINITY ? __expf(sc[nt][1] - mn_lo) : 0.f;
-            ls_lo += p0 + p1;
-            const __nv_bfloat162 h_lo = __floats2bfloat162_rn(p0, p1);
-            pf[2 * nt] = *reinterpret_cast<const uint32_t*>(&h_lo);       // keys 8 nt + kc (+1): A columns of the same numbers
-            pr[2 * nt] = atd_pack_bf16x2(p0 - __low2float(h_lo), p1 - __high2float(h_lo));
-            pf[2 * nt + 1] = 0u; pr[2 * nt + 1] = 0u;
-            if (has_hi) {
-                const float p2 = mn_hi > -INFINITY ? __expf(sc[nt][2] - mn_hi) : 0.f, p3 = mn_hi > -INFINITY ? __expf(sc[nt][3] - mn_hi) : 0.f;
-                ls_hi += p2 + p3;
-                const __nv_bfloat162 h_hi = __floats2bfloat162_rn(p2, p3);
-                pf[2 * nt + 1] = *reinterpret_cast<const uint32_t*>(&h_hi);
-                pr[2 * nt + 1] = atd_pack_bf16x2(p2 - __low2float(h_hi), p3 - __high2float(h_hi));
-            }
-        }
-        l_lo = l_lo * f_lo + ls_lo;
-        l_hi = l_hi * f_hi + ls_hi;
-        // O = O * f + P V; the rescaling is skipped while no row of the warp has a new maximum (a factor of exactly 1)
-        const bool rescale = __any_sync(0xffffffffu, f_lo != 1.f || f_hi != 1.f);
-#pragma unroll
-        for (int np = 0; np < C::NTILES / 2; ++np) {
-            uint32_t vf[4];
-            ldmatrix_x4_trans(vs_s + v_row + (uint32_t)((((2 * np + (lm_m >> 1)) ^ lm_sw)) << 4), vf);
+            // each probability as the sum of two bf16 numbers (the rounded value and the rounded remainder): the second product
+            // then sees them to about 16 significant bits instead of 8, at the price of a second MMA
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-                float (&acc)[4] = o[2 * np + hh];
-                if (rescale) { acc[0] *= f_lo; acc[1] *= f_lo; acc[2] *= f_hi; acc[3] *= f_hi; }
-                mma_bf16_16816(acc, pf, vf[2 * hh], vf[2 * hh + 1]);
-                mma_bf16_16816(acc, pr, vf[2 * hh], vf[2 * hh + 1]);
+                const __nv_bfloat162 hi = __floats2bfloat162_rn(p[hh][0], p[hh][1]);
+                pf[nt][hh] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&hi));
+                pr[nt][hh] = movmatrix_trans(atd_pack_bf16x2(p[hh][0] - __low2float(hi), p[hh][1] - __high2float(hi)));
+            }
+        }
+        // O^T = O^T * f + V^T P^T; the rescaling is skipped while no query of the warp has a new maximum (a factor of exactly 1)
+        const bool rescale = __any_sync(0xffffffffu, moved);
+#pragma unroll
+        for (int mt = 0; mt < C::KSTEPS; ++mt) {
+            uint32_t vf[4];
+            ldmatrix_x4_trans(vs_s + v_row + (uint32_t)(((2 * mt + (lm_m & 1)) ^ v_sw) << 4), vf);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                float (&acc)[4] = o[nt][mt];
+                if (rescale) { acc[0] *= f[nt][0]; acc[1] *= f[nt][1]; acc[2] *= f[nt][0]; acc[3] *= f[nt][1]; }
+                mma_bf16_16816(acc, vf, pf[nt][0], pf[nt][1]);
+                mma_bf16_16816(acc, vf, pr[nt][0], pr[nt][1]);
             }
         }
         __syncwarp();   // the stage may be refilled by this warp's next issue
     }
     pdl_launch_dependents();   // the successor starts behind the merge, not behind this kernel's loads (measured: a little faster)
-    // a row's sum: add the quad's lanes
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();   // every warp is done with its ring: the warps' states go where the rings were
-    {
-        float* st_lo = wst + (size_t)(warp * ATT_NQ + row_lo) * SW;
-        float* st_hi = wst + (size_t)(warp * ATT_NQ + row_hi) * SW;
-        if (row_lo < cnt) {
 #pragma unroll
-            for (int nt = 0; nt < C::NTILES; ++nt) *reinterpret_cast<float2*>(st_lo + nt * 8 + kc) = make_float2(o[nt][0], o[nt][1]);
-            if ((lane & 3) == 0) { st_lo[DH] = m_lo; st_lo[DH + 1] = l_lo; }
-        }
-        if (row_hi < cnt) {
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < C::NTILES; ++nt) *reinterpret_cast<float2*>(st_hi + nt * 8 + kc) = make_float2(o[nt][2], o[nt][3]);
-            if ((lane & 3) == 0) { st_hi[DH] = m_hi; st_hi[DH + 1] = l_hi; }
+        for (int e = 0; e < 2; ++e) {
+            float lr = l[nt][e];                       // a query's sum: add the eight lanes that share its column
+            lr += __shfl_xor_sync(0xffffffffu, lr, 4);
+            lr += __shfl_xor_sync(0xffffffffu, lr, 8);
+            lr += __shfl_xor_sync(0xffffffffu, lr, 16);
+            const int rr = nt * 8 + kc + e;
+            if (rr >= cnt) continue;
+            float* st = wst + (size_t)(warp * ATT_NQ + rr) * SW + (lane >> 2);
+#pragma unroll
+            for (int mt = 0; mt < C::KSTEPS; ++mt) { st[mt * 16] = o[nt][mt][e]; st[mt * 16 + 8] = o[nt][mt][2 + e]; }
+            if (lane < 4) { st[DH] = m[nt][e]; st[DH + 1] = lr; }
         }
-    }
     __syncthreads();
     // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa % CL
     if (CL > 1) cluster_wait();   // closes the opening handshake: every CTA of the cluster is running

@@ -612,14 +612,18 @@ void launch_attn(tandem_ctx& c, int d_head, const AttnArgs& a, int groups, bool 
     else launch_attn_dh<T, 128>(c, a, groups, loop, n_chunks, kv_bytes);
 }
 
-// bf16 decode attention: one cluster of `cl` CTAs per (sequence, head); no scratch.
+// bf16 decode attention: one cluster of `cl` CTAs per (sequence, group of query heads); no scratch.
 template <int DH>
 void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl, double kv_bytes) {
-    static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(attn_decode_kernel<DH>, attn_decode_smem_bytes<DH>(), attr_done);
+    static std::atomic<unsigned long long> attr_done1{0}, attr_done2{0};
+    const int gpc = std::max(1, a.heads_per_cta);
     ProfScope ps(c, PC_ATTN_SPLIT, kv_bytes);
-    launch_ex(c, true, cl, attn_decode_kernel<DH>, dim3(cl, a.n_heads / std::max(1, a.heads_per_cta), groups), dim3(ATD_THREADS),
-              attn_decode_smem_bytes<DH>(), a);
+    auto launch = [&](auto kernel, std::atomic<unsigned long long>& done) {
+        ensure_dyn_smem(kernel, attn_decode_smem_bytes<DH>(), done);
+        launch_ex(c, true, cl, kernel, dim3(cl, a.n_heads / gpc, groups), dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
+    };
+    if (gpc * a.nq <= 8) launch(attn_decode_kernel<DH, 1>, attr_done1);
+    else launch(attn_decode_kernel<DH, 2>, attr_done2);
 }
 // Clusters of `cl` decode-attention CTAs that the device can run at the same time (asked once per device and size).  It is
 // less than the multiprocessors would suggest, because a cluster has to fit into one GPC: with 148 multiprocessors and one
@@ -631,7 +635,7 @@ int attn_max_clusters(int cl) {
     int n = slot.load(std::memory_order_relaxed);
     if (n > 0) return n;
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(attn_decode_kernel<DH>, attn_decode_smem_bytes<DH>(), attr_done);
+    ensure_dyn_smem(attn_decode_kernel<DH, 2>, attn_decode_smem_bytes<DH>(), attr_done);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(cl); cfg.blockDim = dim3(ATD_THREADS); cfg.dynamicSmemBytes = attn_decode_smem_bytes<DH>();
@@ -639,7 +643,7 @@ int attn_max_clusters(int cl) {
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)cl; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_decode_kernel<DH>, &cfg) != cudaSuccess || n < 1) n = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_decode_kernel<DH, 2>, &cfg) != cudaSuccess || n < 1) n = 1;
     slot.store(n, std::memory_order_relaxed);
     return n;
 }
