@@ -647,15 +647,22 @@ int attn_max_clusters(int cl) {
     slot.store(n, std::memory_order_relaxed);
     return n;
 }
-// Cluster size: the largest of 1, 2, 4, 8 with which all clusters run at the same time.  It depends on the number of sequences
-// and key/value heads only, so every pass of a run (block or one-row) cuts the context the same way.  One cluster of eight
-// too many cost a second wave: two sequences x 4000 positions x 8 key/value heads x 128, blocks of six rows, took 35-41 us with
-// eight (16 clusters where 15 fit), 18.6 us with four.  (Sizes in between, which would fill the wave better, measured
-// 3 % slower per iteration at batch 8: a cluster of three merges more states than its extra CTAs save.)
-int attn_cluster_size(int clusters, int d_head) {
-    int cl = ATD_CLUSTER;
-    while (cl > 1 && clusters > (d_head == 32 ? attn_max_clusters<32>(cl) : (d_head == 64 ? attn_max_clusters<64>(cl) : attn_max_clusters<128>(cl)))) cl /= 2;
-    return cl;
+// Cluster size, 1, 2, 4 or 8: the one with the least rounds of resident clusters x (a CTA's share of the context + what a CTA
+// costs apart from it, about two and a half chunks).  It depends on the number of sequences and key/value heads only (the
+// share is taken of 24 chunks, 3072 positions), so every pass of a run (block or one-row) cuts the context the same way.
+// Two sequences x 8 key/value heads x 128, blocks of six rows: 35-41 us with eight (16 clusters where 15 fit), 18.6 us with
+// four.  20 sequences x 16 heads x 64 x 3000 positions, 320 clusters where 296 CTAs fit: 61 us with one, 52 with two, 49 with
+// four; 32 x 16 x 64 x 8194: 160 us with one, 166 with two.  (Sizes in between measured 3 % slower per iteration at batch 8: a
+// cluster of three merges more states than its extra CTAs save.)
+int attn_cluster_size(long long clusters, int d_head) {
+    int best = 1;
+    double least = 0.0;
+    for (int cl = 1; cl <= ATD_CLUSTER; cl *= 2) {
+        const int fit = d_head == 32 ? attn_max_clusters<32>(cl) : (d_head == 64 ? attn_max_clusters<64>(cl) : attn_max_clusters<128>(cl));
+        const double cost = (double)((clusters + fit - 1) / fit) * (24.0 / cl + 2.5);
+        if (cl == 1 || cost < least) { least = cost; best = cl; }
+    }
+    return best;
 }
 void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int groups, double kv_bytes) {
     AttnArgs a = a0;
@@ -668,7 +675,7 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     int gpc = 1;
     while (gpc * 2 <= group && group % (gpc * 2) == 0 && gpc * 2 * a.nq <= ATT_NQ) gpc *= 2;
     a.heads_per_cta = gpc;
-    const int cl = attn_cluster_size((int)std::min<long long>((long long)groups * n_kv, INT_MAX), d_head);
+    const int cl = attn_cluster_size((long long)groups * n_kv, d_head);
     if (d_head == 32) launch_attn_decode_dq<32>(c, a, groups, cl, kv_bytes);
     else if (d_head == 64) launch_attn_decode_dq<64>(c, a, groups, cl, kv_bytes);
     else launch_attn_decode_dq<128>(c, a, groups, cl, kv_bytes);
