@@ -257,24 +257,24 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     } else if (warp == 5) {
         // ---- MMA issue: one elected thread of a converged warp ----
         constexpr uint32_t idesc = umma_idesc_bf16(128, C::N);
-        for (int i = 0; i < nkb; ++i) {
-            const int st = i % C::STAGES;
-            if (!mbar_wait_warp(smem_u32(&s_full[st]), (i / C::STAGES) & 1, poll_limit)) {
+        constexpr uint64_t NEXT = C::STAGE_BYTES / 16;   // a stage further on, in a descriptor's units
+        uint64_t da = umma_desc_k_sw128(ring0), db = umma_desc_k_sw128(ring0 + C::A_BYTES);
+        uint32_t phase = 0, ok = mbar_test(smem_u32(&s_full[0]), 0);
+        for (int i = 0, st = 0; i < nkb; ++i) {
+            if (!mbar_wait_tested(ok, smem_u32(&s_full[st]), phase, poll_limit)) {
                 tc_report(a.err_flag, TC_ERR_OPERANDS);
                 break;
             }
             tc_fence_after_sync();
-            if (elect_one()) {
-                const uint64_t da = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES);
-                const uint64_t db = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES + C::A_BYTES);
-#pragma unroll
-                for (int k = 0; k < 4; ++k)   // 4 x 16 elements of K per stage
-                    umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
-                umma_commit(smem_u32(&s_empty[st]));
-            }
+            const int done = st;
+            const uint64_t ka = da, kb = db;
+            if (++st == C::STAGES) { st = 0; phase ^= 1; da -= (C::STAGES - 1) * NEXT; db -= (C::STAGES - 1) * NEXT; }
+            else { da += NEXT; db += NEXT; }
+            if (i + 1 < nkb) ok = mbar_test(smem_u32(&s_full[st]), phase);
+            umma_bf16_k64(tmem, ka, kb, idesc, i != 0 ? 1u : 0u);
+            umma_commit_one(smem_u32(&s_empty[done]));
         }
-        if (elect_one()) umma_commit(smem_u32(&s_accum));
-        __syncwarp();
+        umma_commit_one(smem_u32(&s_accum));
         // TMEM goes back as soon as the epilogue warps have read the accumulator (they arrive on barrier 2 right after
         // their loads), not at the end of the kernel: nothing is left to do for this warp after that.
         asm volatile("bar.sync 2, 160;" ::: "memory");
@@ -1060,21 +1060,18 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
         if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
     } else if (warp == 9) {
         constexpr uint32_t idesc = umma_idesc_bf16(128, TCS_BN);
-        int st = 0, round = 0;
-        for (int i = 0; i < nkb; ++i) {
-            if (!mbar_wait_warp(smem_u32(&s_full[st]), (uint32_t)round & 1)) { tc_report(a.err_flag, TC_ERR_OPERANDS); break; }
+        uint32_t phase = 0, ok = mbar_test(smem_u32(&s_full[0]), 0);
+        for (int i = 0, st = 0; i < nkb; ++i) {
+            if (!mbar_wait_tested(ok, smem_u32(&s_full[st]), phase)) { tc_report(a.err_flag, TC_ERR_OPERANDS); break; }
             tc_fence_after_sync();
-            if (elect_one()) {
-                const uint64_t da = umma_desc_k_sw128(ring0 + st * TCS_STAGE_BYTES);
-                const uint64_t db = umma_desc_k_sw128(ring0 + st * TCS_STAGE_BYTES + TCT_TILE_BYTES);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
-                umma_commit(smem_u32(&s_empty[st]));
-            }
-            if (++st == stages) { st = 0; ++round; }
+            const int done = st;
+            if (++st == stages) { st = 0; phase ^= 1; }
+            if (i + 1 < nkb) ok = mbar_test(smem_u32(&s_full[st]), phase);
+            umma_bf16_k64(tmem, umma_desc_k_sw128(ring0 + done * TCS_STAGE_BYTES), umma_desc_k_sw128(ring0 + done * TCS_STAGE_BYTES + TCT_TILE_BYTES),
+                          idesc, i != 0 ? 1u : 0u);
+            umma_commit_one(smem_u32(&s_empty[done]));
         }
-        if (elect_one()) umma_commit(smem_u32(&s_accum));
-        __syncwarp();
+        umma_commit_one(smem_u32(&s_accum));
         if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
     } else {
         pdl_wait();

@@ -63,6 +63,21 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t limit = MBAR_POLL_LIMIT) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit)) != 0;
 }
+// Whether the phase with the given parity has completed, without waiting for it: asked before the products of the K-block before are
+// issued and used after, the answer's way (about 115 clocks) runs beside them.
+__device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok;
+}
+// The wait that follows such a question.
+__device__ __forceinline__ bool mbar_wait_tested(uint32_t ok, uint32_t bar, uint32_t parity, uint32_t limit = MBAR_POLL_LIMIT) {
+    return __all_sync(0xffffffffu, ok != 0) || mbar_wait_warp(bar, parity, limit);
+}
 // A value that is the same in all lanes, made known as such.
 __device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
@@ -136,6 +151,29 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint
 // The mbarrier gets one arrival when every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// The four products of 64 elements of K (K-major operands with the 128-byte swizzle), and a commit, issued by one lane of a
+// converged warp: predicated, not branched to.  Inside `if (elect_one())` the compiler forms the operands again for every
+// product and the wait that precedes does not overlap: 317 clocks per K-block of 128 x 32 with its operands present, 205 like
+// this and with the next barrier asked for first, of which 160 are the products (40 clocks each for 32 columns or fewer).
+__device__ __forceinline__ void umma_bf16_k64(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred e, p, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.eq.b32 t, 0, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, t;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, t;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, t;\n\t}"
+        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "l"(desc_a + 2), "l"(desc_b + 2),
+          "l"(desc_a + 4), "l"(desc_b + 4), "l"(desc_a + 6), "l"(desc_b + 6) : "memory");
+}
+__device__ __forceinline__ void umma_commit_one(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 // ---- the same for a pair of CTAs (a cluster of two): one 256-row tile on two multiprocessors -----------------------------
 // Address of the same shared-memory location in the cluster's CTA number `rank`.
