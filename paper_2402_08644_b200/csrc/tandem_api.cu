@@ -453,10 +453,15 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     a.seg_rows = w.seg_rows; a.tiles_per_seg = cdiv(w.seg_rows, 128);
     const int tiles = a.tiles0 + (w.n_segs - 1) * a.tiles_per_seg, KB = cdiv(w.K, 64);
     // K-slices per tile = cluster size: the smallest power of two that puts tiles * S CTAs at or above one per
-    // multiprocessor, at most 8 and at most one per 64-element K-block.  The head GEMM keeps whole tiles.
+    // multiprocessor, at most 8 and at most one per 64-element K-block; four instead of eight where those already reach a
+    // quarter of the multiprocessors with slices of four K-blocks or fewer (they fit the ring, and only 15 clusters of
+    // eight run beside each other before two CTAs share a multiprocessor, but 33 of four).  A layer's four GEMMs with four
+    // slices in both wide ones against eight: 1024 wide, one row 12.5 -> 11.9 us, eight rows 13.9 -> 13.1; 512 wide 9.9 -> 9.5 and
+    // 11.8 -> 11.4.  The residual GEMMs (a quarter of the tiles or a slice beyond the ring) are 2 to 10 % slower with four.
+    // The head GEMM keeps whole tiles.
     int S = 1;
     if (EPI != EPI_ARGMAX)
-        while (S < 8 && 2 * S <= KB && tiles * S < c.n_sms) S *= 2;
+        while (S < 8 && 2 * S <= KB && tiles * S < c.n_sms && !(S == 4 && KB <= 16 && 16 * tiles >= c.n_sms)) S *= 2;
     a.splits = S;
     a.stream_weights = stream_weights ? 1 : 0;
     a.err_flag = sc.err;
