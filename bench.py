@@ -351,10 +351,8 @@ def measure_workload(name, steps, warmup, rank, local_rank, world, extras, keep_
         out, lens, stats = t.tandem_speculative_generate(gamma, new, 0)
     torch.cuda.synchronize()
     r["e2e_step_ms"] = 1e3 * (time.perf_counter() - t0) / steps
-    rows = B * (P - 1)
-    group = 128 if shape.dtype == synth.DTYPE_BF16 else 16       # queries per attention group of the prompt pass
-    r["h2d"] = 4 * (3 * rows + 2 * (rows // group + B) + 2 * B)  # row token/sequence/position, query groups, n, pending
-    r["d2h"] = 4 * (B * new + B + 16) + stats["iterations"] * 20  # tokens, lengths, histogram; 5 counters per iteration
+    r["h2d"] = 4 * (4 * B + B * P)                               # per prompt its length and offsets, then the token ids
+    r["d2h"] = 4 * (B * new + B + 16) + 8 * 16 + stats["iterations"] * 24  # tokens, lengths, counters, histogram; six words per iteration
 
     if extras:
         # context: accept-all timing mode and plain greedy decoding of the large model alone (graphs warmed first)

@@ -299,10 +299,10 @@ TANDEM_API int64_t tandem_launch_count(tandem_ctx* ctx);
  *   q, out           [batch][n_heads][d_head]
  *   k_derived, v_derived  [batch][n_heads][derived_len][d_head]
  *   k_own, v_own     [batch][n_heads][own_len][d_head]
- *   scratch          work space of at least tandem_decode_attention_scratch_bytes(...) bytes (the kernel reads
- *                    every row's sequence and position from two int arrays that the call fills there)
+ *   scratch          work space of at least tandem_decode_attention_scratch_bytes(...) bytes; not read or
+ *                    written by the present kernel
  * d_head in {32, 64, 128}; batch <= 65535.  The context is cut into 128-position chunks by absolute position.
- * A cluster of 1, 2, 4 or 8 CTAs (chosen from batch * n_heads) serves one (sequence, head): CTA r takes every
+ * A cluster of 1, 2, 4 or 8 CTAs (chosen from batch * n_heads and what fits the chip at once) serves one (sequence, head): CTA r takes every
  * cluster-size-th chunk starting at r, each warp keeps an online-softmax state for its share of the positions,
  * and the states are merged in a fixed order through the cluster's shared memory. */
 TANDEM_API size_t tandem_decode_attention_scratch_bytes(int32_t batch, int32_t n_heads, int32_t d_head,
@@ -318,23 +318,14 @@ TANDEM_API tandem_status tandem_decode_attention(const void* q, const void* k_de
  * Who needs it: code that runs where cudaMalloc is off limits - inside a host callback or another
  * library's hook, in a process whose memory pool is owned by a framework that hands out no raw buffers,
  * or in a service that must not touch the allocator after start-up because an allocation can block on,
- * or synchronise with, other work on the device.  Such a caller still passes its inputs and its output,
- * but the kernel's work space (the per-row sequence / position arrays) is a buffer built into the library:
- * a file-scope __device__ array of TANDEM_STATIC_SCRATCH_BYTES that every GPU loading the library holds
- * until the process exits.
+ * or synchronise with, other work on the device.  Such a caller passes its inputs and its output
+ * and nothing else: the kernel keeps its state on the chip.
  *
  * Same arguments, layouts and results as tandem_decode_attention, minus scratch.  Differences:
  *  - Batches whose work space exceeds TANDEM_STATIC_SCRATCH_BYTES (tandem_decode_attention_scratch_bytes
  *    tells; 8 bytes per sequence, so 8192 sequences fit) are refused with TANDEM_ERR_CAPACITY before anything
  *    is launched; tandem_last_cuda_error() then holds a sentence with both sizes.
- *  - The first call on each device looks up the device address of the built-in buffer (with that device
- *    current - make the device that owns the tensors current before calling).  Make that first call before
- *    any stream capture is begun on the device.  Later calls only launch.
- *  - The call itself allocates nothing on host or device and frees nothing.
- *  - All calls on a device share the one buffer, and it keeps whatever the previous call left there.  Each call
- *    rewrites the part it reads, so the caller clears nothing between calls; but two calls that can overlap
- *    on the GPU (different streams, or one stream and a graph) race on it and give wrong results.  Keep calls
- *    to this entry point on one stream, or order them with events. */
+ *  - The call itself allocates nothing on host or device and frees nothing. Calls on different streams may overlap. */
 #define TANDEM_STATIC_SCRATCH_BYTES (64 * 1024)
 TANDEM_API tandem_status tandem_decode_attention_static(const void* q, const void* k_derived, const void* v_derived,
                                                         const void* k_own, const void* v_own, void* out,
@@ -349,7 +340,7 @@ TANDEM_API tandem_status tandem_decode_attention_static(const void* q, const voi
  *   and its normalised fp32 copy).  rows <= 256; d_large, d_small multiples of 8.
  * The two GEMMs stream their weights on the tensor cores (once up to 64 rows, else once per group of 64 rows)
  * with the key/value write as the second one's epilogue; the LayerNorm is fused into the second one's operand
- * load for up to 8 rows of up to 1024 elements and runs as a kernel of its own otherwise.  Asynchronous; a
+ * load for few short rows and runs as a kernel of its own otherwise.  Asynchronous; a
  * bounded device-side wait that ran out is reported by tandem_standalone_check. */
 TANDEM_API size_t tandem_ff_tandem_project_scratch_bytes(int32_t rows, int32_t d_small);
 TANDEM_API tandem_status tandem_ff_tandem_project(const void* x, const void* w_t, const void* ln_g, const void* ln_b,
