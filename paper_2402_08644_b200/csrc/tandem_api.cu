@@ -1498,10 +1498,11 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             c->kmap.resize(cfg->large.n_layers);
             c->vmap.resize(cfg->large.n_layers);
             bool okm = true;
+            const unsigned atc_kc = dhL == 128 ? AtcCfg<128>::KC : AtcCfg<64>::KC;
             const uint64_t kv_rows = (uint64_t)cfg->max_batch * c->large.kv_heads * cfg->max_seq;
             for (int l = 0; l < cfg->large.n_layers && okm; ++l)
-                okm = make_tmap_bf16(&c->kmap[l], kv_ptr<bf16>(*c, c->large, l, 0), kv_rows, (uint64_t)dhL, (uint64_t)dhL, ATC_KC) &&
-                      make_tmap_bf16(&c->vmap[l], kv_ptr<bf16>(*c, c->large, l, 1), kv_rows, (uint64_t)dhL, (uint64_t)dhL, ATC_KC);
+                okm = make_tmap_bf16(&c->kmap[l], kv_ptr<bf16>(*c, c->large, l, 0), kv_rows, (uint64_t)dhL, (uint64_t)dhL, atc_kc) &&
+                      make_tmap_bf16(&c->vmap[l], kv_ptr<bf16>(*c, c->large, l, 1), kv_rows, (uint64_t)dhL, (uint64_t)dhL, atc_kc);
             if (okm) { c->tc_prompt_attn = true; c->prompt_group = ATC_Q; }
         }
     }
