@@ -374,7 +374,10 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
             if (lane == 0) mbar_arrive(smem_u32(&s_pready[t][c % C::BUFS]));
         }
         if (ok && n > 0) {   // all chunks accumulated
-            if (!mbar_wait(smem_u32(&s_odone[t]), (n - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
+            // (one phase after the other: this S being there says no more than that the product BUFS chunks back is done, and a
+            // wait for a parity is also satisfied two phases early)
+            const bool before = n < 2 || mbar_wait(smem_u32(&s_odone[t]), (n - 2) & 1);
+            if (!before || !mbar_wait(smem_u32(&s_odone[t]), (n - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
             tc_fence_after_sync();
             const float inv = 1.0f / l;
             bf16* dst = static_cast<bf16*>(a.out) + (size_t)(row0 + qi) * a.ldo + h * DH;

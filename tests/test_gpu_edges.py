@@ -67,3 +67,20 @@ def test_bf16_pair_prompt_gemm_with_tiles_in_parts():
     shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, 2304, 18, 3200), small=(1, 128, 2, 256), max_pos=2120, layer_map=(1,))
     w = _bf16_weights(shape, seed=6, std=0.02)
     assert _replay_compare(shape, w, prompts_for(shape, [2105], seed=7), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 1
+
+
+@pytest.mark.parametrize("heads", [2, 1])   # head sizes 64 and 128: chunks of 64 and of 128 keys
+def test_bf16_prompt_attention_at_chunk_edges(heads):
+    """Prompts that end one query before, at and behind the end of a chunk, a tile and a group of two tiles, in one batch."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, 128, heads, 128), small=(1, 64, 1, 64), max_pos=640, layer_map=(1,))
+    w = _bf16_weights(shape, seed=12, std=0.1)
+    prompts = prompts_for(shape, [64, 65, 66, 128, 129, 130, 256, 257, 258, 386, 514], seed=13)
+    assert _replay_compare(shape, w, prompts, 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 4
+
+
+@pytest.mark.parametrize("width,ffn", [(512, 1160), (576, 1288), (1088, 2184)])   # 8, 9 and 17 K-blocks; 9 / 10, 11 and 18 feature tiles
+def test_bf16_few_row_gemm_with_four_and_eight_slices(width, ffn):
+    """Around the rule that gives wide matrices of short rows four K-slices instead of eight, ragged last tiles and slices."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, width // 64, ffn), small=(1, 64, 1, 64), max_pos=64, layer_map=(1,))
+    w = _bf16_weights(shape, seed=14, std=0.03)
+    assert _replay_compare(shape, w, prompts_for(shape, [5, 9, 2], seed=15), 3, 2, TOL_BF16, 2 * TOL_BF16) <= 4
