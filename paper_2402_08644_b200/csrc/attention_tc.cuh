@@ -180,7 +180,7 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
     using C = AtcCfg<DH>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     __shared__ __align__(8) uint64_t s_qfull, s_kfull[C::STAGES], s_kfree[C::STAGES], s_vfull[C::STAGES], s_vfree[C::STAGES];
-    __shared__ __align__(8) uint64_t s_sfull[2][C::BUFS], s_pready[2][C::BUFS], s_odone[2];   // [tile][buffer]; odone[tile]: one phase per chunk
+    __shared__ __align__(8) uint64_t s_sfull[2][C::BUFS], s_pready[2][C::BUFS], s_odone[2], s_ofinal[2];   // [tile][buffer]; odone[tile]: one phase per chunk but the last, ofinal[tile]: the last
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
@@ -194,7 +194,7 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
                 mbar_init(smem_u32(&s_vfull[s]), 1); mbar_init(smem_u32(&s_vfree[s]), 1);
             }
             for (int t = 0; t < 2; ++t) {
-                mbar_init(smem_u32(&s_odone[t]), 1);
+                mbar_init(smem_u32(&s_odone[t]), 1); mbar_init(smem_u32(&s_ofinal[t]), 1);
                 for (int u = 0; u < C::BUFS; ++u) {
                     mbar_init(smem_u32(&s_sfull[t][u]), 1);
                     mbar_init(smem_u32(&s_pready[t][u]), 4);   // one arrive per softmax warp of the tile
@@ -292,7 +292,7 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
                 for (int ks = 0; ks < C::KC / 64; ++ks)
                     umma_bf16_ts_k64(tmem + 256 + t * 128, tmem + t * 128 + buf * C::KC + ks * 32, umma_desc_mn_sw128(v0 + st * C::K_BYTES + ks * 8192, C::KSUB),
                                      2048 >> 4, idesc_o, (c | ks) != 0 ? 1u : 0u);
-                umma_commit_one(smem_u32(&s_odone[t]));   // O of tile t holds chunks 0 .. c
+                umma_commit_one(smem_u32(c + 1 < n ? &s_odone[t] : &s_ofinal[t]));   // O of tile t holds chunks 0 .. c
                 if (next < n) issue_s(t, next);
             }
             umma_commit_one(smem_u32(&s_vfree[st]));
@@ -334,6 +334,7 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
             // lazy reference: it moves only when this chunk's maximum exceeds it by more than the margin
             const bool move = mc > m + LAZY2;            // (first chunk: m = -inf, every row with a visible key moves)
             if (c > 0 && __any_sync(0xffffffffu, move)) {   // O is touched only when P V of the previous chunk is complete
+                // (phase c - 1 or c is current: S of chunk c lies behind product c - BUFS, and product c needs this warp's P)
                 if (!mbar_wait(smem_u32(&s_odone[t]), (c - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; break; }
                 tc_fence_after_sync();
                 const float f = (move && m > -INFINITY) ? ex2_approx(m - mc) : 1.0f;   // rows that keep their reference: exactly 1
@@ -374,10 +375,9 @@ attn_prefill_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap t
             if (lane == 0) mbar_arrive(smem_u32(&s_pready[t][c % C::BUFS]));
         }
         if (ok && n > 0) {   // all chunks accumulated
-            // (one phase after the other: this S being there says no more than that the product BUFS chunks back is done, and a
-            // wait for a parity is also satisfied two phases early)
-            const bool before = n < 2 || mbar_wait(smem_u32(&s_odone[t]), (n - 2) & 1);
-            if (!before || !mbar_wait(smem_u32(&s_odone[t]), (n - 1) & 1)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
+            // (a barrier of its own: this S being there says no more than that the product BUFS chunks back is done, and a wait for a
+            // parity cannot tell a phase from the one two before it)
+            if (!mbar_wait(smem_u32(&s_ofinal[t]), 0)) { tc_report(a.err_flag, TC_ERR_ACCUM); ok = false; }
             tc_fence_after_sync();
             const float inv = 1.0f / l;
             bf16* dst = static_cast<bf16*>(a.out) + (size_t)(row0 + qi) * a.ldo + h * DH;
