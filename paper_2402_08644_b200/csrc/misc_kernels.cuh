@@ -518,42 +518,70 @@ __global__ void __launch_bounds__(256) forced_fill_kernel(LoopState st, int batc
 
 // Scores of a teacher-forced round: for draft step s of sequence b, at position p = n_b - 1 + s, the negative
 // log-likelihood of the true token at p + 1 under softmax(logits) and the arg-max (lowest id on ties).
-// logits: [gamma][batch][V].  grid: (gamma, batch); block: 256.
-__global__ void __launch_bounds__(256) score_rows_kernel(LoopState st, int batch, const float* __restrict__ logits, int V,
-                                                         const int* __restrict__ forced, const int* __restrict__ forced_len, int stride,
-                                                         float* __restrict__ nll, int* __restrict__ top1) {
-    __shared__ float sv[8], ss[8];
-    __shared__ int si[8];
+// Bound by the latency of a row's passes: a row is dealt to the 64 warps of a cluster, whose ranges stay in registers between the
+// maximum and the sum (up to 32768 logits, else they are read again); the warps' maxima, positions and sums meet in the first
+// CTA.  32000 logits, 16 rows: 19 us with one CTA per row and two passes over it, about 6 us like this.
+// logits: [gamma][batch][V].  grid: (SCR_CLUSTER, gamma, batch), a cluster per row; block: SCR_THREADS.
+constexpr int SCR_CLUSTER = 8, SCR_THREADS = 256, SCR_RANGES = SCR_CLUSTER * SCR_THREADS / 32, SCR_REGS = 16;
+__global__ void __launch_bounds__(SCR_THREADS) score_rows_kernel(LoopState st, int batch, const float* __restrict__ logits, int V,
+                                                                 const int* __restrict__ forced, const int* __restrict__ forced_len, int stride,
+                                                                 float* __restrict__ nll, int* __restrict__ top1) {
+    __shared__ float s_max[SCR_RANGES], s_sum[SCR_RANGES], s_pos[SCR_RANGES];   // first CTA: one entry per range (s_pos: the bits of an int)
+    cluster_arrive_relaxed();   // opening handshake
     pdl_wait();
     pdl_launch_dependents();
-    const int s = blockIdx.x, b = blockIdx.y;
+    cluster_wait();
+    const int s = blockIdx.y, b = blockIdx.z, lane = threadIdx.x & 31;
     const int p = st.n[b] - 1 + s;
-    if (p + 1 >= forced_len[b]) return;                  // no true next token: nothing to score
+    if (p + 1 >= forced_len[b]) return;                  // no true next token: nothing to score (the same for the whole cluster)
     const float* row = logits + ((size_t)s * batch + b) * V;
-    float best = -INFINITY;
+    const int id = blockIdx.x * (SCR_THREADS / 32) + (threadIdx.x >> 5);
+    const int chunk = (((V + SCR_RANGES - 1) / SCR_RANGES) + 31) & ~31;
+    const int i0 = min(V, id * chunk), i1 = min(V, i0 + chunk);
+    float best = -INFINITY, z = 0.f;
     int bi = INT_MAX;
-    for (int i = threadIdx.x; i < V; i += 256) {
-        const float v = __ldcg(row + i);
+    auto take = [&](float v, int i) {
         if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-    }
+    };
+    auto across = [&]() {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+            take(ov, __shfl_xor_sync(0xffffffffu, bi, o));
+        }
+    };
+    if (chunk <= 32 * SCR_REGS) {
+        float x[SCR_REGS];
+#pragma unroll
+        for (int j = 0; j < SCR_REGS; ++j) x[j] = __ldcg(row + min(i0 + 32 * j + lane, V - 1));
+#pragma unroll
+        for (int j = 0; j < SCR_REGS; ++j) if (i0 + 32 * j + lane < i1) take(x[j], i0 + 32 * j + lane);
+        across();
+#pragma unroll
+        for (int j = 0; j < SCR_REGS; ++j) z += i0 + 32 * j + lane < i1 ? expf(x[j] - best) : 0.f;
+    } else {
+#pragma unroll 8
+        for (int i = i0 + lane; i < i1; i += 32) take(__ldcg(row + i), i);
+        across();
+#pragma unroll 8
+        for (int i = i0 + lane; i < i1; i += 32) z += expf(__ldcg(row + i) - best);
     }
-    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
-    __syncthreads();
-    for (int w = 0; w < 8; ++w)
-        if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
-    float z = 0.f;
-    for (int i = threadIdx.x; i < V; i += 256) z += expf(__ldcg(row + i) - best);
     z = warp_sum(z);
-    if ((threadIdx.x & 31) == 0) ss[threadIdx.x >> 5] = z;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float tot = 0.f;
-        for (int w = 0; w < 8; ++w) tot += ss[w];
+    if (lane == 0) {
+        st_dsmem_f32(smem_u32(&s_max[id]), 0, best);
+        st_dsmem_f32(smem_u32(&s_sum[id]), 0, z);
+        st_dsmem_f32(smem_u32(&s_pos[id]), 0, __int_as_float(bi));
+    }
+    cluster_sync_all();
+    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+    best = -INFINITY;
+    bi = INT_MAX;
+    for (int r = lane; r < SCR_RANGES; r += 32) take(s_max[r], __float_as_int(s_pos[r]));
+    across();
+    float tot = 0.f;
+    for (int r = lane; r < SCR_RANGES; r += 32) tot += s_sum[r] > 0.f ? s_sum[r] * expf(s_max[r] - best) : 0.f;   // (an empty range: 0)
+    tot = warp_sum(tot);
+    if (lane == 0) {
         const int truth = forced[(size_t)b * stride + p + 1];
         nll[(size_t)b * stride + p] = best + logf(tot) - __ldcg(row + truth);
         top1[(size_t)b * stride + p] = bi;

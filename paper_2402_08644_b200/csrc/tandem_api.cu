@@ -948,7 +948,7 @@ void launch_forced_fill(tandem_ctx& c, int gamma) {
 }
 void launch_score_rows(tandem_ctx& c, int gamma) {
     ProfScope ps(c, PC_ARGMAX, (double)c.batch * gamma * c.small.d.vocab * 8.0);
-    launch_ex(c, true, 1, score_rows_kernel, dim3(gamma, c.batch), dim3(256), 0, c.st, c.batch, (const float*)at<float>(c, c.lay.logits_small),
+    launch_ex(c, true, SCR_CLUSTER, score_rows_kernel, dim3(SCR_CLUSTER, gamma, c.batch), dim3(SCR_THREADS), 0, c.st, c.batch, (const float*)at<float>(c, c.lay.logits_small),
               (int)c.small.d.vocab, (const int*)at<int>(c, c.lay.forced_ids), (const int*)at<int>(c, c.lay.forced_len), (int)c.cfg.max_seq,
               at<float>(c, c.lay.forced_nll), at<int>(c, c.lay.forced_top));
 }

@@ -1,6 +1,7 @@
 """Edges of the kernels' dispatch rules and tiles, each against the fp64 checker."""
 import pytest
 
+from oracle import tandem_oracle as O
 from paper_2402_08644_b200 import binding, build, synth
 from test_gpu_parity import TOL_BF16, TOL_FP32, _adaptive_replay, _bf16_weights, _replay_compare, _sampled_replay, gpu_toy_shape, prompts_for, toy_weights
 
@@ -84,3 +85,18 @@ def test_bf16_few_row_gemm_with_four_and_eight_slices(width, ffn):
     shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, width // 64, ffn), small=(1, 64, 1, 64), max_pos=64, layer_map=(1,))
     w = _bf16_weights(shape, seed=14, std=0.03)
     assert _replay_compare(shape, w, prompts_for(shape, [5, 9, 2], seed=15), 3, 2, TOL_BF16, 2 * TOL_BF16) <= 4
+
+
+@pytest.mark.parametrize("vocab", [31, 2049, 32801])
+def test_teacher_forced_scores_over_a_cluster(vocab):
+    """Rows of logits dealt to 64 warps: fewer logits than ranges, a ragged last range, and rows too long for registers."""
+    shape = gpu_toy_shape(large=(1, 64, 2, 64), small=(1, 32, 1, 64), vocab=vocab, max_pos=48, layer_map=(1,))
+    w = toy_weights(shape, seed=5, std=0.3)
+    seqs = prompts_for(shape, [2, 11, 6], seed=6)
+    t = binding.Tandem(shape, w, max_batch=3, max_seq=48, gamma_max=4)
+    nll, top = t.tandem_teacher_forced_forward(seqs, 4)
+    for b, ids in enumerate(seqs):
+        want_nll, want_top = O.next_token_scores(O.teacher_forced_tandem_logits(shape, w, ids, 4), ids)
+        assert abs(nll[b] - want_nll).max() < 2 * TOL_FP32
+        assert top[b].tolist() == list(want_top)
+    t.close()
