@@ -1439,7 +1439,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->use_pdl = getenv("TANDEM_NO_PDL") == nullptr;
     c->n_sms = sm_count();
     if (e == cudaSuccess && cfg->dtype == TANDEM_DTYPE_BF16) {
-        // one tensor map per weight matrix: [out_features][in_features], 128 x 64 tiles
+        // two tensor maps per weight matrix: [out_features][in_features], 128 x 64 tiles and 32 x 64
         c->wmap.resize(c->w.size());
         c->wpart.resize(c->w.size());
         c->wmap_ok.assign(c->w.size(), 0);
@@ -1482,7 +1482,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             }
         }
         c->n_lns = (int)lns.size();
-        e = cudaMemcpy(c->arena + lay.ln_src, lns.data(), lns.size() * sizeof(LnSource), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(c->arena + lay.ln_src, lns.data(), lns.size() * sizeof(LnSource), cudaMemcpyHostToDevice, c->stream);   // (pageable: staged before the call returns)
         if (!ok) {
             snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled unavailable or failed for a weight matrix");
             if (c->pinned) cudaFreeHost(c->pinned);
