@@ -534,10 +534,12 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     }
     a.tiles_m = cdiv(M, 128);
     // Fewer: square tiles, and the K range of each dealt to as many CTAs (1, 2 or 4) as still get a multiprocessor of their
-    // own and four 64-element K-blocks each (fewer would not pay for the exchange).
+    // own and four 64-element K-blocks each (fewer would not pay for the exchange); or as get half a
+    // multiprocessor, where the slices keep sixteen K-blocks: cold weights come with 1.5 us of latency
+    // and a ring holds three K-blocks (329 rows x 4096 x 11008, 96 tiles: 107 -> 64 us).
     const int tiles = (int)feature_tiles(TCS_BN), KB = cdiv(w.K, 64);
     int S = 1;
-    while (S < 4 && tiles * S * 2 <= n_sms && KB >= 8 * S) S *= 2;
+    while (S < 4 && ((tiles * S * 2 <= n_sms && KB >= 8 * S) || (tiles * S <= n_sms && KB >= 32 * S))) S *= 2;
     a.splits = S;
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(gemm_tc_split_kernel<EPI>, TCS_SMEM_BYTES, attr_done);
