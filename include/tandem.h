@@ -25,7 +25,9 @@
  *  - bf16 contexts: weights, queries and both KV caches are bf16; everything else between the kernels of a
  *    decode pass (residual stream, normalised rows, attention and GELU outputs) is fp32, and enters each
  *    tensor-core product as the sum of two bf16 numbers.  The prompt pass keeps bf16 activations.
- *    The LayerNorm gains and biases of those passes are the ones that tandem_prefill found.
+ *  - Weights are read where they lie, in every call.  A change that the context's stream orders between two calls holds
+ *    from the second one on (for the positions that it computes: cached keys and values stay); a weight must not change
+ *    while a call's work runs.
  *  - Two environment variables are read once by tandem_create, for diagnosis only; neither changes a result:
  *    TANDEM_NO_GRAPH (set to anything) launches every kernel of an iteration eagerly instead of replaying a CUDA
  *    graph; TANDEM_NO_PDL orders the kernels by plain stream order instead of programmatic dependent launch.

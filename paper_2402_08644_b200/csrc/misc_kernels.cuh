@@ -98,26 +98,15 @@ __device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __r
 // remainder, bias, its remainder ([4][d]).
 struct LnSource { const float* g; const float* b; bf16* rows; int d; };
 
-// What a prompt pass needs on the device, staged in one copy: per query its length and its offsets among the token ids,
-// the processed rows and the attention groups ([4][n_queries]), then the ids, query after query.
-struct PromptStage {
-    const int* len; const int* id_off; const int* row_off; const int* grp_off; const int* ids;
-    int n_queries, samples, rows, group;   // sequences per query; processed rows; queries per attention group
-};
-
-// Start of a prompt pass: block m < rows sets up processed row m (token, sequence, position, its attention group if it
-// starts one) and embeds it; the last block sets the loop state of every sequence.  The tickets are the host's counts of
-// the verify and router kernels it has enqueued, which the device's counts equal by then.  Blocks beyond that write the
-// LayerNorms' rows for the decode passes that follow (bf16).
-// grid: rows + 1 + LayerNorms; block: 128.
-template <typename T>
-__global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptStage ps, int* row_tok, int* row_seq, int* row_pos, int* grp_row0, int* grp_cnt,
-                                                           const T* __restrict__ emb, const T* __restrict__ pos, float* __restrict__ h, int d,
-                                                           int ticket, int router_ticket, const LnSource* __restrict__ lns) {
-    const int m = blockIdx.x;
-    if (m > ps.rows) {
-        const LnSource l = lns[m - ps.rows - 1];
-        for (int i = threadIdx.x; i < l.d; i += 128) {
+// Start of a generate or step call: the first block says that nobody has emitted anything (a generate call also clears the
+// histogram); the others write the LayerNorms' rows from the parameters as they are now (bf16: the decode GEMMs multiply by the live gain too,
+// so parameters that the caller changed since the prompt pass hold for the whole call).  Not launched behind a running
+// kernel: the GEMMs that read the rows ahead of their wait start two launches later.
+// grid: 1 + LayerNorms; block: 256 (batch <= 256).
+__global__ void __launch_bounds__(256) call_begin_kernel(LoopState st, int batch, bool clear_hist, const LnSource* __restrict__ lns) {
+    if (blockIdx.x > 0) {
+        const LnSource l = lns[blockIdx.x - 1];
+        for (int i = threadIdx.x; i < l.d; i += 256) {
             const float g = l.g[i], b = l.b[i];
             const bf16 gh = __float2bfloat16_rn(g), bh = __float2bfloat16_rn(b);
             l.rows[i] = gh;
@@ -127,6 +116,28 @@ __global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptS
         }
         return;
     }
+    const int b = threadIdx.x;
+    if (b < batch) { st.emitted[b] = 0; st.done[b] = 0; }
+    if (clear_hist && b <= st.gamma_limit) st.hist[b] = 0ull;
+    if (b == 0) { st.counters[1] = batch; st.counters[5] = 0; }
+}
+
+// What a prompt pass needs on the device, staged in one copy: per query its length and its offsets among the token ids,
+// the processed rows and the attention groups ([4][n_queries]), then the ids, query after query.
+struct PromptStage {
+    const int* len; const int* id_off; const int* row_off; const int* grp_off; const int* ids;
+    int n_queries, samples, rows, group;   // sequences per query; processed rows; queries per attention group
+};
+
+// Start of a prompt pass: block m < rows sets up processed row m (token, sequence, position, its attention group if it
+// starts one) and embeds it; the last block sets the loop state of every sequence.  The tickets are the host's counts of
+// the verify and router kernels it has enqueued, which the device's counts equal by then.
+// grid: rows + 1; block: 128.
+template <typename T>
+__global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptStage ps, int* row_tok, int* row_seq, int* row_pos, int* grp_row0, int* grp_cnt,
+                                                           const T* __restrict__ emb, const T* __restrict__ pos, float* __restrict__ h, int d,
+                                                           int ticket, int router_ticket) {
+    const int m = blockIdx.x;
     if (m == ps.rows) {
         for (int b = threadIdx.x; b < ps.n_queries * ps.samples; b += 128) {
             const int q = b / ps.samples, len = ps.len[q];

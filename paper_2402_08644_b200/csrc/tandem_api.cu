@@ -1331,12 +1331,9 @@ tandem_status begin_call(tandem_ctx* c) {
     return TANDEM_OK;
 }
 
-// Start of a generate or step call: nobody has emitted anything; a generate call also clears the histogram.  block: 256.
-__global__ void reset_call_kernel(LoopState st, int batch, bool clear_hist) {
-    const int b = threadIdx.x;
-    if (b < batch) { st.emitted[b] = 0; st.done[b] = 0; }
-    if (clear_hist && b <= st.gamma_limit) st.hist[b] = 0ull;
-    if (b == 0) { st.counters[1] = batch; st.counters[5] = 0; }
+void launch_call_begin(tandem_ctx& c, bool clear_hist) {
+    call_begin_kernel<<<1 + c.n_lns, 256, 0, c.stream>>>(c.st, c.batch, clear_hist, at<LnSource>(c, c.lay.ln_src));
+    c.launches++;
 }
 
 }  // namespace
@@ -1600,9 +1597,9 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     {
         ProfScope prof(*c, PC_ROWS, (double)M * c->large.d.d_model * (4.0 + 2 * c->esz));
         auto begin = [&](auto* emb, auto* pos, auto kernel) {
-            kernel<<<M + 1 + c->n_lns, 128, 0, s>>>(c->st, ps, at<int>(*c, c->lay.row_tok), at<int>(*c, c->lay.row_seq), at<int>(*c, c->lay.row_pos),
+            kernel<<<M + 1, 128, 0, s>>>(c->st, ps, at<int>(*c, c->lay.row_tok), at<int>(*c, c->lay.row_seq), at<int>(*c, c->lay.row_pos),
                                          at<int>(*c, c->lay.grp_row0), at<int>(*c, c->lay.grp_cnt), emb, pos, at<float>(*c, c->lay.h_large),
-                                         c->large.d.d_model, (int)c->ticket, (int)c->router_ticket, at<LnSource>(*c, c->lay.ln_src));
+                                         c->large.d.d_model, (int)c->ticket, (int)c->router_ticket);
         };
         if (bf) begin((const bf16*)w_emb(*c, c->large), (const bf16*)w_pos(*c, c->large), prompt_begin_kernel<bf16>);
         else begin((const float*)w_emb(*c, c->large), (const float*)w_pos(*c, c->large), prompt_begin_kernel<float>);
@@ -1656,8 +1653,7 @@ extern "C" tandem_status tandem_block_step(tandem_ctx* c, int32_t gamma, int32_t
     if (accept_mode == TANDEM_ACCEPT_REPRESENTATION_ONLY && gamma < 1) return TANDEM_ERR_INVALID_ARG;
     if (c->batch == 0) return TANDEM_ERR_STATE;
     TRY(capacity_for(c, 0, gamma));
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch, false);
-    c->launches++;
+    launch_call_begin(*c, false);
     TRY(launch_iteration(*c, 0, gamma, accept_mode, mode_seed, INT_MAX));
     c->n_ub += gamma + 1;
     c->n_sum += (long long)c->batch * (gamma + 1);
@@ -1728,8 +1724,7 @@ tandem_status run_generate(tandem_ctx* c, bool speculative, int gamma, int max_n
     TRY(capacity_for(c, max_new, gamma));
     const int B = c->batch;
     const int64_t launches0 = c->launches;
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B, true);
-    c->launches++;
+    launch_call_begin(*c, true);
     // Iterations are enqueued ahead of the host's knowledge of their outcome, but only those that are certain to be
     // needed: every iteration gives a sequence at most per_iter tokens, so with `left` tokens still wanted by some
     // sequence after the last observed iteration, ceil(left / per_iter) more must run whatever is accepted.  Beyond
@@ -1835,8 +1830,7 @@ extern "C" tandem_status tandem_adaptive_step(tandem_ctx* c, int32_t gamma_max, 
     if (gamma_max < 1 || gamma_max > c->cfg.gamma_max) return TANDEM_ERR_INVALID_ARG;
     if (c->batch == 0 || !c->has_router) return TANDEM_ERR_STATE;
     TRY(capacity_for(c, 0, gamma_max));
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, c->batch, false);
-    c->launches++;
+    launch_call_begin(*c, false);
     int block_max = 0;
     TRY(adaptive_iteration(c, gamma_max, INT_MAX, &block_max));
     TRY(check_error_word(c));
@@ -1874,8 +1868,7 @@ extern "C" tandem_status tandem_adaptive_generate(tandem_ctx* c, int32_t gamma_m
     TRY(capacity_for(c, max_new, gamma_max));
     const int B = c->batch;
     const int64_t launches0 = c->launches;
-    reset_call_kernel<<<1, 256, 0, c->stream>>>(c->st, B, true);
-    c->launches++;
+    launch_call_begin(*c, true);
     int64_t iters = 0, small_runs = 0;
     for (;;) {
         if (iters > max_new) return TANDEM_ERR_STATE;   // every live iteration emits a token

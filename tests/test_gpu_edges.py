@@ -100,3 +100,30 @@ def test_teacher_forced_scores_over_a_cluster(vocab):
         assert abs(nll[b] - want_nll).max() < 2 * TOL_FP32
         assert top[b].tolist() == list(want_top)
     t.close()
+
+
+def test_bf16_layernorm_parameters_changed_between_calls():
+    """Gains and biases that the caller changes after the prompt pass, and again between two steps, hold from the next call on, in
+    every map behind a LayerNorm and in the projection."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 128, 2, 256), small=(2, 64, 1, 136), max_pos=64, layer_map=(0, 2))
+    w = _bf16_weights(shape, seed=17, std=0.08)
+    prompt, gamma = prompts_for(shape, [9], seed=18)[0], 3
+    t = binding.Tandem(shape, w, max_batch=1, max_seq=64, gamma_max=gamma)
+    t.tandem_prefill([prompt])
+    o = O.TandemOracle(shape, w)
+    o.prefill(prompt)
+    for factor, shift in ((1.5, 0.25), (0.5, -0.5)):
+        w = {k: (v * factor + shift).astype("float32") if synth.is_norm_param(k) else v for k, v in w.items()}
+        for name, v in binding.upload_weights(shape, w, t.device).items():
+            if synth.is_norm_param(name):
+                t.weights[name].copy_(v)
+        o.large = O.Decoder(w, "L", shape.large.n_layers, shape.large.n_heads)
+        o.small = O.Decoder(w, "S", shape.small.n_layers, shape.small.n_heads)
+        res = t.tandem_block_step(gamma)
+        drafts, targets = res["drafts"][0].tolist(), res["targets"][0].tolist()
+        _, sl = o.draft(gamma, forced=drafts)
+        _, ll, reps = o.verify(drafts)
+        assert abs(t.tandem_debug_read(binding.READ_SMALL_LOGITS, gamma)[:, 0] - sl).max() < TOL_BF16
+        assert abs(t.tandem_debug_read(binding.READ_LARGE_LOGITS, gamma)[0] - ll).max() < TOL_BF16
+        o.commit(int(res["accept_len"][0]), drafts, targets, reps)
+    t.close()
