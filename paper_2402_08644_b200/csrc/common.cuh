@@ -75,14 +75,17 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 // What a kernel that produces rows of the residual stream leaves for the GEMM behind the next LayerNorm (bf16 decode
-// passes): the rows times the LayerNorm's gain as two bf16 planes (values, remainders) that the GEMM loads by TMA, and per row
-// and group of 32 features the group's mean and sum of squared deviations, which the GEMM merges into the row's
-// statistics while its products run.
+// passes): the rows, less a value c per row, times the LayerNorm's gain as two bf16 planes (values, remainders) that the GEMM
+// loads by TMA, and per row and group of 32 features the group's mean and sum of squared deviations, which the GEMM merges into
+// the row's statistics while its products run.  c stands for the row's mean, which the planes must not spend their 16 bits on: an
+// embedded row has its exact mean taken off, a residual add the mean of the row before the add (its own needs the whole
+// row, which no CTA of the GEMM has), left by the GEMM behind the previous LayerNorm.  The GEMM subtracts the rest, m - c.
 struct NextLn {
     const float* gain;     // null: nothing is left
     bf16* hi; bf16* lo;    // [rows][d]
     float2* stats;         // [rows][groups]
     int groups;            // ceil(d / 32)
+    float* ref;            // [rows] c: written by the embedding, read by a residual add
 };
 
 __device__ __forceinline__ float warp_max(float v) {

@@ -7,9 +7,11 @@
 //                          K-slices of a tile sit in one thread-block cluster: each CTA sends its partial
 //                          sums to the CTA that finishes those token rows (remote shared-memory stores), which
 //                          adds them in slice order.
-//                          LayerNorm ahead of a map is applied behind it:  LN(x) W^T = r (x.g) W^T - r m (g W^T) + b W^T
-//                          with the row's mean m and reciprocal deviation r.  The producer of x leaves x.g in two bf16
-//                          planes, g and b ride along as four more rows of the B operand (each as value + remainder), and
+//                          LayerNorm ahead of a map is applied behind it:
+//                          LN(x) W^T = r ((x - c).g) W^T - r (m - c) (g W^T) + b W^T
+//                          with the row's mean m and reciprocal deviation r.  The producer of x leaves (x - c).g in two bf16
+//                          planes, with c near m (see NextLn: a bit of the planes is lost for every doubling of |m - c| beyond the
+//                          deviation), g and b ride along as four more rows of the B operand (each as value + remainder), and
 //                          the row's statistics are merged while the products run, so nothing but TMA stands between
 //                          the producer and the MMAs (PRO_LNT).  Activations enter the product as the sum of two bf16 numbers (the rounded value and the rounded
 //                          remainder, about 16 significant bits): the B tile holds the NB value rows followed
@@ -40,7 +42,7 @@ namespace tandem {
 // LayerNorm, then value + remainder; PRO_F32: fp32 rows as value + remainder; PRO_TMA: the producer of the rows has
 // already written them as two bf16 planes (values, remainders), and TMA brings them into the B stages beside the
 // weights (no registers, no rounds, nothing for warps 0-3 to do before the epilogue).
-// PRO_LNT: LayerNorm rows, x.g by TMA like PRO_TMA and the rest in the epilogue (see above); the small pair's maps behind a
+// PRO_LNT: LayerNorm rows, (x - c).g by TMA like PRO_TMA and the rest in the epilogue (see above); the small pair's maps behind a
 // LayerNorm took 4.4 us of the stream's time with the rows normalised in the prologue of every CTA (batch 1, 2), and
 // 4.4 + 1.9 us with a LayerNorm kernel of their own (more sequences).
 enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3, PRO_LNT = 4 };
@@ -58,6 +60,8 @@ struct TcDecodeArgs {
     int ln_row;             // PRO_LNT: first of the four rows of this LayerNorm in its tensor map
     const float2* ln_stats; // PRO_LNT: [rows][ln_groups], see NextLn
     int ln_groups;
+    const float* ln_ref;    // PRO_LNT: [rows] c of the planes, see NextLn
+    float* ln_mean;         // PRO_LNT: [rows] the rows' means, which the first CTA leaves for the producer of the next LayerNorm's planes
     int rows, K, N;         // N = output features over all segments
     int seg_rows0, tiles0;  // output features and tiles of the first weight segment (one tensor map per segment)
     int seg_rows;           // output features of every further segment
@@ -142,7 +146,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     __shared__ __align__(8) uint64_t s_accum;
     __shared__ __align__(8) uint64_t s_inbox;   // counts the bytes of the K-slices' partial sums sent to this CTA
     __shared__ uint32_t s_tmem;
-    __shared__ float s_mu[NB], s_rstd[NB];
+    __shared__ float s_mu[NB], s_rstd[NB];   // LayerNorm prologues: the rows' means (PRO_LNT: less c) and reciprocal deviations;  EPI_RESID: s_mu[s] = c of row j_first + s
     __shared__ long long s_rowoff[NB];   // EPI_QKV / EPI_KV: the row-dependent part of an output's cache index
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
@@ -313,6 +317,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             if (s >= j_count) break;   // (every loop over rows leaves at the last row: the unrolled rest is never fetched)
             hres[s] = nl < seg_rows ? __ldcg(hp + (size_t)(j_first + s) * a.e.ldo + seg_base + nl) : 0.f;
         }
+        if (a.e.ln.gain && tid < j_count) s_mu[tid] = __ldcg(a.e.ln.ref + j_first + tid);   // (published by the barrier ahead of the epilogue)
     }
     if (ln_regs) {
         // short LayerNorm rows: one pass over x.  Lane L holds the row's float4 number L + 32u in
@@ -381,7 +386,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         for (int r0 = warp * 4; r0 < a.rows; r0 += 16) {
             const int r = r0 + (lane >> 3), gl = lane & 7;
             const float2* sp = a.ln_stats + (size_t)min(r, a.rows - 1) * a.ln_groups;
-            const float ref = __ldcg(sp).x;
+            const float ref = __ldcg(sp).x, c = __ldcg(a.ln_ref + min(r, a.rows - 1));
             float s = 0.f, q = 0.f;
 #pragma unroll 4
             for (int g = gl; g < a.ln_groups; g += 8) {
@@ -394,7 +399,8 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             for (int o = 4; o > 0; o >>= 1) { s += __shfl_xor_sync(0xffffffffu, s, o); q += __shfl_xor_sync(0xffffffffu, q, o); }
             const float dmu = s / (float)a.K;
             if (gl == 0 && r < a.rows) {
-                s_mu[r] = ref + dmu;
+                s_mu[r] = (ref - c) + dmu;
+                if (unit == 0) a.ln_mean[r] = ref + dmu;
                 s_rstd[r] = 1.0f / sqrtf(fmaxf(q - s * dmu, 0.f) / (float)a.K + 1e-5f);
             }
         }
@@ -522,6 +528,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             if (tid < a.rows) s_rowoff[tid] = ((long long)my_seq * a.e.n_heads * a.e.t_max + my_pos) * a.e.d_head;
             bar_sync(1, 128);
         }
+        if (EPI == EPI_RESID && a.e.ln.gain) bar_sync(1, 128);
         if (!mbar_wait(smem_u32(&s_accum), 0, poll_limit)) tc_report(a.err_flag, TC_ERR_ACCUM);
         tc_fence_after_sync();
         float c1 = 0.f, c2 = 0.f;                     // PRO_LNT: this feature's (slice of) g W^T and b W^T
@@ -631,7 +638,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                             static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = hv;
                             if (EPI == EPI_RESID && a.e.snap) static_cast<float*>(a.e.snap)[(size_t)j * a.e.snap_ld + n] = hv;
                             if (EPI == EPI_RESID && a.e.ln.gain) {
-                                const float x = hv * next_gain;
+                                const float x = (hv - s_mu[s]) * next_gain;
                                 const bf16 hi = __float2bfloat16_rn(x);
                                 a.e.ln.hi[(size_t)j * a.e.ldo + n] = hi;
                                 a.e.ln.lo[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(x - __bfloat162float(hi));

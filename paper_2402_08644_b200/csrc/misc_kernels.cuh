@@ -33,23 +33,37 @@ struct LoopState {
 };
 
 // x^(0) = Emb(t) + Pos(index) of one row (Eq. 1) into the fp32 residual stream, 16 bytes of the tables at a time, with what
-// the first LayerNorm's GEMM wants of it (bf16; `row` is its row there).  d is a multiple of 8.  All threads of a block of
-// BLOCK take part.
-template <typename T, int BLOCK>
+// the first LayerNorm's GEMM wants of it (LN, bf16; `row` is its row there; red: one float per warp).  d is a multiple of 8.
+// All threads of a block of BLOCK take part.
+template <typename T, int BLOCK, bool LN>
 __device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __restrict__ pr, float* __restrict__ hr, float* __restrict__ snap, int d,
-                                          const NextLn& ln, int row) {
+                                          const NextLn& ln, int row, float* red) {
     constexpr int VN = VecN<T>::N;
+    const bool once = d <= BLOCK * VN;   // the row stays in registers
+    float v[VN], gain[LN ? VN : 1], sum = 0.f;
+    auto fetch = [&](int i) {
+        float p[VN];
+        load_vec(er + i, v);
+        load_vec(pr + i, p);
+#pragma unroll
+        for (int u = 0; u < VN; ++u) v[u] += p[u];
+    };
+    auto fetch_gain = [&](int i) {
+        if constexpr (LN) {
+#pragma unroll
+            for (int u = 0; u < VN; u += 4) {
+                const float4 g = __ldg(reinterpret_cast<const float4*>(ln.gain + i + u));
+                gain[u] = g.x; gain[u + 1] = g.y; gain[u + 2] = g.z; gain[u + 3] = g.w;
+            }
+        }
+    };
     for (int i0 = 0; i0 < d; i0 += BLOCK * VN) {
         const int i = i0 + threadIdx.x * VN;
-        float v[VN];
 #pragma unroll
         for (int u = 0; u < VN; ++u) v[u] = 0.f;
         if (i < d) {
-            float p[VN];
-            load_vec(er + i, v);
-            load_vec(pr + i, p);
-#pragma unroll
-            for (int u = 0; u < VN; ++u) v[u] += p[u];
+            fetch(i);
+            if (once) fetch_gain(i);
 #pragma unroll
             for (int u = 0; u < VN; u += 4) {
                 const float4 t = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
@@ -57,29 +71,12 @@ __device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __r
                 if (snap) *reinterpret_cast<float4*>(snap + i + u) = t;
             }
         }
-        if constexpr (sizeof(T) == 2) {
-            if (ln.gain == nullptr) continue;
-            if (i < d) {
-                uint4 hi, lo;
-                uint32_t *ph = &hi.x, *pl = &lo.x;
-#pragma unroll
-                for (int u = 0; u < VN; u += 4) {
-                    const float4 g = __ldg(reinterpret_cast<const float4*>(ln.gain + i + u));
-                    const float x0 = v[u] * g.x, x1 = v[u + 1] * g.y, x2 = v[u + 2] * g.z, x3 = v[u + 3] * g.w;
-                    const __nv_bfloat162 a = __floats2bfloat162_rn(x0, x1), b = __floats2bfloat162_rn(x2, x3);
-                    const __nv_bfloat162 ra = __floats2bfloat162_rn(x0 - __low2float(a), x1 - __high2float(a));
-                    const __nv_bfloat162 rb = __floats2bfloat162_rn(x2 - __low2float(b), x3 - __high2float(b));
-                    ph[u / 2] = *reinterpret_cast<const uint32_t*>(&a); ph[u / 2 + 1] = *reinterpret_cast<const uint32_t*>(&b);
-                    pl[u / 2] = *reinterpret_cast<const uint32_t*>(&ra); pl[u / 2 + 1] = *reinterpret_cast<const uint32_t*>(&rb);
-                }
-                *reinterpret_cast<uint4*>(ln.hi + (size_t)row * d + i) = hi;
-                *reinterpret_cast<uint4*>(ln.lo + (size_t)row * d + i) = lo;
-            }
-            // four neighbouring threads hold a group of 32 features
+        if constexpr (LN) {   // four neighbouring threads hold a group of 32 features
             const float n = (float)min(32, d - (i & ~31));
             float s = 0.f, q = 0.f;
 #pragma unroll
             for (int u = 0; u < VN; ++u) s += v[u];
+            sum += s;
             s += __shfl_xor_sync(0xffffffffu, s, 1);
             s += __shfl_xor_sync(0xffffffffu, s, 2);
             const float mean = s / n;
@@ -90,6 +87,31 @@ __device__ __forceinline__ void embed_row(const T* __restrict__ er, const T* __r
             q += __shfl_xor_sync(0xffffffffu, q, 1);
             q += __shfl_xor_sync(0xffffffffu, q, 2);
             if (i < d && (threadIdx.x & 3) == 0) ln.stats[(size_t)row * ln.groups + (i >> 5)] = make_float2(mean, q);
+        }
+    }
+    if constexpr (LN) {
+        sum = warp_sum(sum);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+        __syncthreads();
+        float c = 0.f;
+#pragma unroll
+        for (int w = 0; w < BLOCK / 32; ++w) c += red[w];
+        c /= (float)d;
+        if (threadIdx.x == 0) ln.ref[row] = c;
+        for (int i = threadIdx.x * VN; i < d; i += BLOCK * VN) {
+            if (!once) { fetch(i); fetch_gain(i); }
+            uint4 hi, lo;
+            uint32_t *ph = &hi.x, *pl = &lo.x;
+#pragma unroll
+            for (int u = 0; u < VN; u += 2) {
+                const float x0 = (v[u] - c) * gain[u], x1 = (v[u + 1] - c) * gain[u + 1];
+                const __nv_bfloat162 a = __floats2bfloat162_rn(x0, x1);
+                const __nv_bfloat162 r = __floats2bfloat162_rn(x0 - __low2float(a), x1 - __high2float(a));
+                ph[u / 2] = *reinterpret_cast<const uint32_t*>(&a);
+                pl[u / 2] = *reinterpret_cast<const uint32_t*>(&r);
+            }
+            *reinterpret_cast<uint4*>(ln.hi + (size_t)row * d + i) = hi;
+            *reinterpret_cast<uint4*>(ln.lo + (size_t)row * d + i) = lo;
         }
     }
 }
@@ -161,7 +183,7 @@ __global__ void __launch_bounds__(128) prompt_begin_kernel(LoopState st, PromptS
             grp_cnt[g] = min(ps.group, ps.len[lo] - 1 - p);
         }
     }
-    embed_row<T, 128>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0);
+    embed_row<T, 128, false>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0, nullptr);
 }
 
 // Keys / values of a query's first sequence to its other samples: one block per (layer and K or V, key/value head, query),
@@ -216,6 +238,7 @@ __global__ void __launch_bounds__(128) step_begin_kernel(LoopState st, int r0, i
                                                          int* row_seq, int* row_pos, const T* __restrict__ emb,
                                                          const T* __restrict__ pos, float* __restrict__ h, int d, float* snap, NextLn ln) {
     __shared__ int s_tok, s_pos;
+    __shared__ float s_red[4];
     pdl_wait();
     pdl_launch_dependents();
     const int m = blockIdx.x;
@@ -234,7 +257,7 @@ __global__ void __launch_bounds__(128) step_begin_kernel(LoopState st, int r0, i
     }
     __syncthreads();
     // (snap: copy for the FF_Tandem projection of x^(0))
-    embed_row<T, 128>(emb + (size_t)s_tok * d, pos + (size_t)s_pos * d, h + (size_t)m * d, snap ? snap + (size_t)m * d : nullptr, d, ln, m);
+    embed_row<T, 128, sizeof(T) == 2>(emb + (size_t)s_tok * d, pos + (size_t)s_pos * d, h + (size_t)m * d, snap ? snap + (size_t)m * d : nullptr, d, ln, m, s_red);
 }
 
 __device__ __forceinline__ float block_sum_128(float v, float* red) {

@@ -56,8 +56,8 @@ struct Layout {   // byte offsets into the arena
     size_t h_large, h_small, a, q, o, f, xb, t1, yhat, a_s, logits_large, logits_small, part_ml, part_acc, dbg;
     size_t smp_large, smp_small;                     // sampled SPEED: (maximum, sum of weights) of every row of logits
     size_t amax_val_large, amax_idx_large, amax_val_small, amax_idx_small;
-    size_t a32, o32, f32;                           // value / remainder planes between the bf16 decode kernels: LayerNorm inputs (x.g) / attention / GELU outputs
-    size_t ln_src, ln_rows_large, ln_rows_small, ln_stats;   // LayerNorms behind the GEMMs (bf16 decode): sources, their rows, the token rows' statistics
+    size_t a32, o32, f32;                           // value / remainder planes between the bf16 decode kernels: LayerNorm inputs ((x - c).g) / attention / GELU outputs
+    size_t ln_src, ln_rows_large, ln_rows_small, ln_stats, ln_ref;   // LayerNorms behind the GEMMs (bf16 decode): sources, their rows, the token rows' statistics, reference values (see ln_ref_of)
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles;
@@ -128,7 +128,7 @@ struct tandem_ctx {
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
     std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
     // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
-    // TMA: maps of the residual stream (times the next LayerNorm's gain) / attention / GELU buffers, [buffer 0..2][0 large,
+    // TMA: maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
     // 1 small], 16-row boxes; and the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one).
     CUtensorMap xmap[3][2], lnmap[2];
     std::vector<char> wmap_ok;
@@ -253,6 +253,7 @@ Layout make_layout(const tandem_config& c) {
     L.ln_rows_large = take((size_t)(2 * c.large.n_layers + 1) * 4 * c.large.d_model * 2);
     L.ln_rows_small = take((size_t)(2 * c.small.n_layers + 1) * 4 * c.small.d_model * 2);
     L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
+    L.ln_ref = take(2 * RD * 4);
     L.total = off;
     return L;
 }
@@ -428,6 +429,8 @@ struct TcRows {
     int ln_row = 0;                        // the LayerNorm's first row there
     const float2* ln_stats = nullptr;      // [rows][ln_groups]
     int ln_groups = 0;
+    const float* ln_ref = nullptr;         // [rows] each
+    float* ln_mean = nullptr;
 };
 
 template <int NB, int PRO, int EPI>
@@ -477,6 +480,8 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
         a.x_row0 = r0; a.x_plane_rows = xr.plane_rows;
         a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups;
         a.ln_stats = xr.ln_stats ? xr.ln_stats + (size_t)r0 * xr.ln_groups : nullptr;
+        a.ln_ref = xr.ln_ref ? xr.ln_ref + r0 : nullptr;
+        a.ln_mean = xr.ln_mean ? xr.ln_mean + r0 : nullptr;
         a.wait_first = r0 == 0 ? sc.wait_first : 0;
         a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
         a.x = static_cast<const unsigned char*>(x) + (size_t)r0 * ldx * xsz;
@@ -487,7 +492,7 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
         if (e.out_lo) a.e.out_lo = static_cast<unsigned char*>(e.out_lo) + (size_t)r0 * e.ldo * 2;   // (value / remainder planes are bf16)
         if (e.row_seq) { a.e.row_seq = e.row_seq + r0; a.e.row_pos = e.row_pos + r0; }
         if (e.snap) a.e.snap = static_cast<float*>(e.snap) + (size_t)r0 * e.snap_ld;
-        if (e.ln.gain) { a.e.ln.hi = e.ln.hi + (size_t)r0 * e.ldo; a.e.ln.lo = e.ln.lo + (size_t)r0 * e.ldo; a.e.ln.stats = e.ln.stats + (size_t)r0 * e.ln.groups; }
+        if (e.ln.gain) { a.e.ln.hi = e.ln.hi + (size_t)r0 * e.ldo; a.e.ln.lo = e.ln.lo + (size_t)r0 * e.ldo; a.e.ln.stats = e.ln.stats + (size_t)r0 * e.ln.groups; a.e.ln.ref = e.ln.ref + r0; }
         ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + (double)nr * w.K * xsz + (double)nr * a.N * (EPI == EPI_QKV || EPI == EPI_KV || EPI == EPI_STORE ? 2.0 : 4.0));
         if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, a, w, units, xr);
         else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, a, w, units, xr);
@@ -1027,7 +1032,7 @@ void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
 // bf16 decode on the tensor cores: five kernels per decoder layer, chained by programmatic dependent launch
 // ---------------------------------------------------------------------------------------------------
 
-// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = residual stream times the next
+// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = residual stream, less c, times the next
 // LayerNorm's gain, 1 = attention output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width
 // for buffer 2).
 struct XPlanes { bf16* hi; bf16* lo; TcRows rows; };
@@ -1047,9 +1052,12 @@ XPlanes x_planes(tandem_ctx& c, int buf, const Model& m) {
 const void* ln_gain(const tandem_ctx& c, const Model& m, int idx) {
     return idx == 2 * m.d.n_layers ? w_tail(c, m, 0) : w_layer(c, m, idx / 2, idx % 2 ? W_LN2G : W_LN1G);
 }
+// The value taken off each row before LayerNorm `idx` (NextLn::ref).  Two arrays in turn: the GEMM behind a LayerNorm reads its
+// own from one and leaves the rows' means, the next LayerNorm's, in the other.
+float* ln_ref_of(tandem_ctx& c, int idx) { return at<float>(c, c.lay.ln_ref) + (size_t)(idx & 1) * c.lay.dec_rows; }
 NextLn next_ln(tandem_ctx& c, const Model& m, int idx) {
     const XPlanes p = x_planes(c, 0, m);
-    return {static_cast<const float*>(ln_gain(c, m, idx)), p.hi, p.lo, at<float2>(c, c.lay.ln_stats), cdiv(m.d.d_model, 32)};
+    return {static_cast<const float*>(ln_gain(c, m, idx)), p.hi, p.lo, at<float2>(c, c.lay.ln_stats), cdiv(m.d.d_model, 32), ln_ref_of(c, idx)};
 }
 TcRows ln_rows_of(tandem_ctx& c, const Model& m, int idx) {
     TcRows r = x_planes(c, 0, m).rows;
@@ -1057,6 +1065,8 @@ TcRows ln_rows_of(tandem_ctx& c, const Model& m, int idx) {
     r.ln_row = 4 * idx;
     r.ln_stats = at<float2>(c, c.lay.ln_stats);
     r.ln_groups = cdiv(m.d.d_model, 32);
+    r.ln_ref = ln_ref_of(c, idx);
+    r.ln_mean = ln_ref_of(c, idx + 1);
     return r;
 }
 

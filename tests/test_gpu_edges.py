@@ -1,4 +1,5 @@
 """Edges of the kernels' dispatch rules and tiles, each against the fp64 checker."""
+import numpy as np
 import pytest
 
 from oracle import tandem_oracle as O
@@ -127,3 +128,38 @@ def test_bf16_layernorm_parameters_changed_between_calls():
         assert abs(t.tandem_debug_read(binding.READ_LARGE_LOGITS, gamma)[0] - ll).max() < TOL_BF16
         o.commit(int(res["accept_len"][0]), drafts, targets, reps)
     t.close()
+
+
+@pytest.mark.parametrize("batch,gamma", [(1, 3), (7, 15)])     # 4 block rows, and 112: two groups of 64
+@pytest.mark.parametrize("offset", [0.0, 40.0])
+def test_bf16_layernorm_of_rows_far_from_zero(batch, gamma, offset):
+    """Rows whose mean is 200 times their deviation lose nothing to the 16 bits of the planes.  The layers add zero (output and second
+    FFN maps of zeros), so the heads see LayerNorm(Emb + Pos) itself: embedded rows beyond and within one block's registers,
+    and rows that every residual add has written anew.  Entries are multiples of 2^-8: all sums of x are exact.
+    Bound: each term of a logit carries its operand's 16 bits (at most 2^-16 of the term; independent roundings, four deviations are
+    less than 4 / sqrt(3) of the terms' norm), the bias its own, and the row's fp32 mean half a unit in its last place."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 1088, 17, 128), small=(2, 96, 3, 136), max_pos=64, layer_map=(0, 2))
+    w = _bf16_weights(shape, seed=19, std=0.05)
+    for tag, m in (("L", shape.large), ("S", shape.small)):
+        w[tag + ".emb"] = np.round(w[tag + ".emb"] * 4 * 256).astype(np.float32) / 256
+        w[tag + ".pos"] = np.full_like(w[tag + ".pos"], offset)
+        for l in range(m.n_layers):
+            w[f"{tag}.{l}.wo"] = np.zeros_like(w[f"{tag}.{l}.wo"])
+            w[f"{tag}.{l}.w2"] = np.zeros_like(w[f"{tag}.{l}.w2"])
+    prompts = prompts_for(shape, [1 + b for b in range(batch)], seed=20)
+    t = binding.Tandem(shape, w, max_batch=batch, max_seq=64, gamma_max=gamma)
+    t.tandem_prefill(prompts)
+    drafts = t.tandem_block_step(gamma)["drafts"]
+    small, large = t.tandem_debug_read(binding.READ_SMALL_LOGITS, gamma), t.tandem_debug_read(binding.READ_LARGE_LOGITS, gamma)
+    t.close()
+    for b in range(batch):
+        tokens = [prompts[b][-1]] + drafts[b].tolist()
+        for tag, got in (("S", small[:, b]), ("L", large[b])):
+            g, bias, head = (w[tag + n].astype(np.float64) for n in (".lnf_g", ".lnf_b", ".w_out"))
+            for r, row in enumerate(got):
+                x = w[tag + ".emb"][tokens[r]].astype(np.float64) + offset
+                z = (x - x.mean()) / np.sqrt(x.var() + 1e-5)
+                want = (z * g + bias) @ head.T
+                bound = 4 / np.sqrt(3) * 2.0 ** -16 * (np.linalg.norm(z * g * head, axis=1) + np.linalg.norm(bias * head, axis=1))
+                bound += 2.0 ** -24 * (abs(x.mean()) / x.std() * abs(head @ g) + 8 * abs(z * g * head).sum(1))
+                assert (abs(row - want) <= bound).all()
