@@ -369,6 +369,15 @@ def _stream_of(t):
     return torch._C._cuda_getCurrentRawStream(t.get_device())
 
 
+def _check_device(first, *others):
+    """The kernel takes plain addresses: what it would read or write lies on the first tensor's GPU."""
+    if not first.is_cuda:
+        raise ValueError(f"expected a tensor on a CUDA device, got one on {first.device}")
+    for t in others:
+        if t.numel() and t.device != first.device:
+            raise ValueError(f"an argument is on {t.device}, the first one on {first.device}")
+
+
 def _ptr_or_null(t):
     return t.data_ptr() if t.numel() else None
 
@@ -391,6 +400,7 @@ def tandem_decode_attention_static(q, k_derived, v_derived, k_own, v_own, out):
     share that buffer: keep them on one stream.  Make the first call on a device outside any stream capture."""
     lib = _lib or load_library()
     B, H, dh = q.shape
+    _check_device(q, k_derived, v_derived, k_own, v_own, out)
     Td, To = k_derived.shape[2], k_own.shape[2]
     status = lib.tandem_decode_attention_static(q.data_ptr(), _ptr_or_null(k_derived), _ptr_or_null(v_derived), _ptr_or_null(k_own),
                                                 _ptr_or_null(v_own), out.data_ptr(), B, H, dh, Td, To, _stream_of(q))

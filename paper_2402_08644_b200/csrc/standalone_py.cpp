@@ -8,6 +8,8 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <string>
+
 #include "../../include/tandem.h"
 
 namespace {
@@ -16,6 +18,17 @@ const at::Tensor* tensor_arg(PyObject* o) {
     if (THPVariable_Check(o)) return &THPVariable_Unpack(o);
     PyErr_SetString(PyExc_TypeError, "a torch.Tensor is expected");
     return nullptr;
+}
+// The kernels take plain addresses: whatever they would read or write lies on the first argument's GPU (t: null where an optional
+// argument is absent; an empty tensor is never touched).  Ranks of the first argument as documented.
+void check_arguments(const at::Tensor* const* t, int n, int rank) {
+    const at::Tensor& first = *t[0];
+    TORCH_CHECK_VALUE(first.dim() == rank, "the first argument must have " + std::to_string(rank) + " dimensions, it has " + std::to_string(first.dim()));
+    TORCH_CHECK_VALUE(first.is_cuda(), "expected a tensor on a CUDA device, got one on " + first.device().str());
+    for (int i = 1; i < n; ++i)
+        if (t[i] && t[i]->numel())
+            TORCH_CHECK_VALUE(t[i]->device() == first.device(),
+                              "argument " + std::to_string(i + 1) + " is on " + t[i]->device().str() + ", the first one on " + first.device().str());
 }
 const void* ptr_of(const at::Tensor& t) { return t.numel() ? t.const_data_ptr() : nullptr; }
 void* stream_of(const at::Tensor& t) { return c10::cuda::getCurrentCUDAStream(t.get_device()).stream(); }
@@ -32,6 +45,7 @@ PyObject* decode_attention(PyObject*, PyObject* const* args, Py_ssize_t n) {
     for (int i = 0; i < 7; ++i)
         if (i < 5 || args[i] != Py_None)
             if (!(t[i] = tensor_arg(args[i]))) return nullptr;
+    check_arguments(t, 7, 3);
     const at::Tensor& q = *t[0];
     const int B = (int)q.size(0), H = (int)q.size(1), dh = (int)q.size(2), Td = (int)t[1]->size(2), To = (int)t[3]->size(2);
     const at::Tensor out = t[5] ? *t[5] : empty_like_device(q.sizes(), q.scalar_type(), q);
@@ -50,6 +64,7 @@ PyObject* ff_tandem_project(PyObject*, PyObject* const* args, Py_ssize_t n) {
     for (int i = 0; i < 7; ++i)
         if (i < 6 || args[i] != Py_None)
             if (!(t[i] = tensor_arg(args[i]))) return nullptr;
+    check_arguments(t, 7, 2);
     const at::Tensor& x = *t[0];
     const int rows = (int)x.size(0), d_l = (int)x.size(1), d_s = (int)t[1]->size(0);
     const at::Tensor k = empty_like_device({rows, d_s}, at::kBFloat16, x), v = empty_like_device({rows, d_s}, at::kBFloat16, x);
@@ -70,13 +85,15 @@ PyObject* ff_tandem_project(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyObject* block_linear(PyObject*, PyObject* const* args, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (n != 3) { PyErr_SetString(PyExc_TypeError, "three arguments are expected"); return nullptr; }
-    const at::Tensor *x = tensor_arg(args[0]), *w = x ? tensor_arg(args[1]) : nullptr;
-    if (!w) return nullptr;
-    const at::Tensor* given = nullptr;
-    if (args[2] != Py_None && !(given = tensor_arg(args[2]))) return nullptr;
-    const int rows = (int)x->size(0), k = (int)x->size(1), nf = (int)w->size(0);
-    const at::Tensor y = given ? *given : empty_like_device({rows, nf}, at::kBFloat16, *x);
-    return result(tandem_block_linear(x->const_data_ptr(), w->const_data_ptr(), y.mutable_data_ptr(), rows, k, nf, stream_of(*x)), y);
+    const at::Tensor* t[3] = {};
+    for (int i = 0; i < 3; ++i)
+        if (i < 2 || args[i] != Py_None)
+            if (!(t[i] = tensor_arg(args[i]))) return nullptr;
+    check_arguments(t, 3, 2);
+    const at::Tensor &x = *t[0], &w = *t[1];
+    const int rows = (int)x.size(0), k = (int)x.size(1), nf = (int)w.size(0);
+    const at::Tensor y = t[2] ? *t[2] : empty_like_device({rows, nf}, at::kBFloat16, x);
+    return result(tandem_block_linear(x.const_data_ptr(), w.const_data_ptr(), y.mutable_data_ptr(), rows, k, nf, stream_of(x)), y);
     END_HANDLE_TH_ERRORS
 }
 

@@ -61,3 +61,20 @@ def test_null_context_calls_fail_cleanly(lib):
     assert lib.tandem_block_step(None, 1, 0, 0, None) == 1
     assert lib.tandem_decode_attention_scratch_bytes(0, 1, 64, 1, 1) == 0
     assert lib.tandem_decode_attention_scratch_bytes(2, 16, 64, 1000, 4) >= 2 * 2 * 4
+
+
+@pytest.mark.parametrize("lead", [0, 1])   # an extra leading dimension: refused too
+def test_standalone_calls_refuse_tensors_that_no_kernel_may_touch(lib, lead):
+    """Host tensors, and a first argument of another rank, are refused before anything is launched or allocated."""
+    import torch
+    z = lambda *n, dtype=torch.bfloat16: torch.zeros(n, dtype=dtype)  # noqa: E731
+    first = lambda *n: z(*[1] * lead, *n)  # noqa: E731
+    kv, scratch = z(1, 2, 4, 64), z(64, dtype=torch.uint8)
+    with pytest.raises(ValueError):
+        binding.tandem_decode_attention(first(1, 2, 64), kv, kv, kv, kv, z(1, 2, 64), scratch)
+    with pytest.raises(ValueError):
+        binding.tandem_decode_attention_static(first(1, 2, 64), kv, kv, kv, kv, z(1, 2, 64))
+    with pytest.raises(ValueError):
+        binding.tandem_ff_tandem_project(first(1, 64), z(64, 64), z(64), z(64), z(64, 64), z(64, 64), scratch)
+    with pytest.raises(ValueError):
+        binding.tandem_block_linear(first(1, 64), z(64, 64), z(1, 64))

@@ -163,3 +163,22 @@ def test_bf16_layernorm_of_rows_far_from_zero(batch, gamma, offset):
                 bound = 4 / np.sqrt(3) * 2.0 ** -16 * (np.linalg.norm(z * g * head, axis=1) + np.linalg.norm(bias * head, axis=1))
                 bound += 2.0 ** -24 * (abs(x.mean()) / x.std() * abs(head @ g) + 8 * abs(z * g * head).sum(1))
                 assert (abs(row - want) <= bound).all()
+
+
+def test_standalone_calls_refuse_arguments_on_another_device():
+    """Any one argument left on the host is refused (an empty segment, which no kernel touches, is not)."""
+    import torch
+    on = lambda *n, dtype=torch.bfloat16: torch.zeros(n, dtype=dtype, device="cuda")  # noqa: E731
+    f32 = torch.float32
+    kv, scratch = [on(1, 2, 4, 64) for _ in range(4)], on(1 << 16, dtype=torch.uint8)
+    calls = [(binding.tandem_decode_attention, [on(1, 2, 64), *kv, on(1, 2, 64), scratch]),
+             (binding.tandem_decode_attention_static, [on(1, 2, 64), *kv, on(1, 2, 64)]),
+             (binding.tandem_ff_tandem_project, [on(1, 64), on(64, 64), on(64, dtype=f32), on(64, dtype=f32), on(64, 64), on(64, 64), scratch]),
+             (binding.tandem_block_linear, [on(1, 64), on(64, 64), on(1, 64)])]
+    for call, args in calls:
+        call(*args)
+        for i in range(len(args)):
+            with pytest.raises(ValueError):
+                call(*[a.cpu() if j == i else a for j, a in enumerate(args)])
+    none = torch.zeros(1, 2, 0, 64, dtype=torch.bfloat16)
+    assert binding.tandem_decode_attention(on(1, 2, 64), none, none, kv[0], kv[1]).shape == (1, 2, 64)
