@@ -1071,7 +1071,7 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
         }
         pdl_launch_dependents();
         __syncwarp();
-        if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
+        if (S > 1) cluster_sync_all();
     } else if (warp == 9) {
         constexpr uint32_t idesc = umma_idesc_bf16(128, TCS_BN);
         uint32_t phase = 0, ok = mbar_test(smem_u32(&s_full[0]), 0);
@@ -1086,7 +1086,7 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             umma_commit_one(smem_u32(&s_empty[done]));
         }
         umma_commit_one(smem_u32(&s_accum));
-        if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }
+        if (S > 1) cluster_sync_all();
     } else {
         pdl_wait();
         const int quarter = warp & 3, half = warp >> 2;
@@ -1113,8 +1113,9 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
         if (!mbar_wait(smem_u32(&s_accum), 0)) tc_report(a.err_flag, TC_ERR_ACCUM);
         tc_fence_after_sync();
         if (S > 1) {
-            cluster_arrive_relaxed();   // this CTA's products have read its ring ...
-            cluster_wait();             // ... and so have the others'
+            // This CTA's products have read its ring, and so have the others'.  With release: the reads, known to be done by
+            // the wait above, come before the peers' stores to the same bytes.
+            cluster_sync_all();
             if (tid == 0) mbar_arrive_expect_tx(ibar, (uint32_t)((S - 1) * 128 * CS * 4));
             for (int q = 0; q < S; ++q) {
                 if (q == sp) continue;
