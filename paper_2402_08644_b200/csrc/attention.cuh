@@ -29,8 +29,7 @@ struct AttnArgs {
     const void* kcache; const void* vcache;   // [seq][head][t_max][DH]
     const void* k2; const void* v2;            // optional second segment [seq][head][t_max2][DH] holding
     int split, t_max2;                         //   positions >= split (used when k2 != nullptr)
-    void* out; int ldo;                  // T [M][ldo]; float when out_f32 is set (attn_decode_kernel only)
-    int out_f32;
+    void* out; int ldo;                  // T [M][ldo]
     const int* row_seq; const int* row_pos;    // attn_decode_kernel: row_seq may be null, then group g is sequence g and every
     int pos_all;                               //   sequence's first row sits at position pos_all (no row arrays to fill and fetch)
     int wait_first;                            // attn_decode_kernel: 1 = nothing is read before the wait on the preceding kernel
@@ -647,8 +646,9 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
                 const bf16 hi = __float2bfloat16_rn(res);
                 static_cast<bf16*>(a.out)[oi] = hi;
                 static_cast<bf16*>(a.out_lo)[oi] = __float2bfloat16_rn(res - __bfloat162float(hi));
-            } else if (a.out_f32) static_cast<float*>(a.out)[oi] = res;
-            else static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
+            } else {
+                static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
+            }
         }
     }
 }

@@ -38,8 +38,8 @@
 
 namespace tandem {
 
-// How the token rows become the B operand: PRO_BF16: bf16 rows as they are (remainder rows zero); PRO_LN: fp32 rows,
-// LayerNorm, then value + remainder; PRO_F32: fp32 rows as value + remainder; PRO_TMA: the producer of the rows has
+// How the token rows become the B operand: PRO_BF16: bf16 rows as they are (remainder rows zero); PRO_LN: fp32 rows
+// of at most 1024 elements, LayerNorm, then value + remainder; PRO_F32: fp32 rows as value + remainder; PRO_TMA: the producer of the rows has
 // already written them as two bf16 planes (values, remainders), and TMA brings them into the B stages beside the
 // weights (no registers, no rounds, nothing for warps 0-3 to do before the epilogue).
 // PRO_LNT: LayerNorm rows, (x - c).g by TMA like PRO_TMA and the rest in the epilogue (see above); the small pair's maps behind a
@@ -166,9 +166,9 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     const int kb0 = sp * kb_base + min(sp, kb_rem);
     const int nkb = kb_base + (sp < kb_rem ? 1 : 0);
     const int K4 = a.K >> 2;
-    // LayerNorm rows short enough to sit in registers (8 float4 per lane) and a K-slice that fits the ring
-    // without reuse: the B operand is then written straight from the registers that gave the statistics.
-    const bool ln_regs = PRO == PRO_LN && K4 <= 256 && nkb <= C::STAGES;
+    // LayerNorm rows (they sit in registers, 8 float4 per lane) and a K-slice that fits the ring without reuse: the B
+    // operand is then written straight from the registers that gave the statistics.
+    const bool ln_regs = PRO == PRO_LN && nkb <= C::STAGES;
     // Token rows whose outputs this CTA finishes: all of them without split-K, else a contiguous share of ceil(rows / S).
     const int rpc = S == 1 ? a.rows : (a.rows + S - 1) / S;
     const int j_first = S == 1 ? 0 : sp * rpc;
@@ -410,38 +410,22 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         if (PRO == PRO_LN) {
             for (int r = warp; r < a.rows; r += 4) {   // one warp per row, fixed lane-strided order
                 const float4* xr = reinterpret_cast<const float4*>(static_cast<const float*>(a.x) + (size_t)r * a.ldx);
-                float mu, var;
-                if (K4 <= 256) {   // the same arithmetic as the register path above
-                    float4 t[8];
+                float4 t[8];           // the same arithmetic as the register path above
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) t[u] = (lane + 32 * u < K4) ? __ldcg(xr + lane + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    float s = 0.f;
+                for (int u = 0; u < 8; ++u) t[u] = (lane + 32 * u < K4) ? __ldcg(xr + lane + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+                float s = 0.f;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) s += (t[u].x + t[u].y) + (t[u].z + t[u].w);
-                    mu = warp_sum(s) / (float)a.K;
-                    float q = 0.f;
+                for (int u = 0; u < 8; ++u) s += (t[u].x + t[u].y) + (t[u].z + t[u].w);
+                const float mu = warp_sum(s) / (float)a.K;
+                float q = 0.f;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (lane + 32 * u < K4) {
-                            const float d0 = t[u].x - mu, d1 = t[u].y - mu, d2 = t[u].z - mu, d3 = t[u].w - mu;
-                            q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
-                        }
-                    }
-                    var = warp_sum(q) / (float)a.K;
-                } else {
-                    float s = 0.f;
-#pragma unroll 8
-                    for (int k4 = lane; k4 < K4; k4 += 32) { const float4 t = __ldcg(xr + k4); s += (t.x + t.y) + (t.z + t.w); }
-                    mu = warp_sum(s) / (float)a.K;
-                    float q = 0.f;
-#pragma unroll 8
-                    for (int k4 = lane; k4 < K4; k4 += 32) {
-                        const float4 t = __ldcg(xr + k4);
-                        const float d0 = t.x - mu, d1 = t.y - mu, d2 = t.z - mu, d3 = t.w - mu;
+                for (int u = 0; u < 8; ++u) {
+                    if (lane + 32 * u < K4) {
+                        const float d0 = t[u].x - mu, d1 = t[u].y - mu, d2 = t[u].z - mu, d3 = t[u].w - mu;
                         q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
                     }
-                    var = warp_sum(q) / (float)a.K;
                 }
+                const float var = warp_sum(q) / (float)a.K;
                 if (lane == 0) { s_mu[r] = mu; s_rstd[r] = 1.0f / sqrtf(var + 1e-5f); }
             }
             bar_sync(1, 128);

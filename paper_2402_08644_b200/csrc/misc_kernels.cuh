@@ -276,20 +276,6 @@ __device__ __forceinline__ void ln_store4(bf16* orow, int k4, float y0, float y1
     const __nv_bfloat162 lo = __floats2bfloat162_rn(y0, y1), hi = __floats2bfloat162_rn(y2, y3);
     reinterpret_cast<uint2*>(orow)[k4] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
-// value plane + remainder plane (x = bf16(x) + bf16(x - bf16(x))), for a GEMM that loads its token rows by TMA
-__device__ __forceinline__ void ln_store4_split(bf16* vrow, bf16* rrow, int k4, float y0, float y1, float y2, float y3) {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(y0, y1), b = __floats2bfloat162_rn(y2, y3);
-    const __nv_bfloat162 ra = __floats2bfloat162_rn(y0 - __low2float(a), y1 - __high2float(a));
-    const __nv_bfloat162 rb = __floats2bfloat162_rn(y2 - __low2float(b), y3 - __high2float(b));
-    reinterpret_cast<uint2*>(vrow)[k4] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-    reinterpret_cast<uint2*>(rrow)[k4] = make_uint2(*reinterpret_cast<const uint32_t*>(&ra), *reinterpret_cast<const uint32_t*>(&rb));
-}
-__device__ __forceinline__ void ln_store4(float* orow, bf16*, int k4, float y0, float y1, float y2, float y3) { ln_store4(orow, k4, y0, y1, y2, y3); }
-__device__ __forceinline__ void ln_store4(bf16* orow, bf16* rrow, int k4, float y0, float y1, float y2, float y3) {
-    if (rrow) ln_store4_split(orow, rrow, k4, y0, y1, y2, y3);
-    else ln_store4(orow, k4, y0, y1, y2, y3);
-}
-
 // LayerNorm of fp32 rows (biased variance, eps 1e-5) ahead of the GEMMs, output in the storage type: the row sits in
 // registers between the passes (up to 4096 elements), loads and stores are 16 bytes wide (8191 rows of 4096: 56 us with
 // scalar accesses in three passes).  raw (nullable): bf16 copy of the row as it is, for the FF_Tandem projection that reads
@@ -299,7 +285,7 @@ __device__ __forceinline__ void ln_store4(bf16* orow, bf16* rrow, int k4, float 
 template <typename TO>
 __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __restrict__ x, const float* __restrict__ gain,
                                                              const float* __restrict__ bias, TO* __restrict__ out, int d,
-                                                             int M, bf16* out_lo = nullptr, bf16* raw = nullptr) {
+                                                             int M, bf16* raw) {
     __shared__ float red[4];
     const int d4 = d >> 2;
     if (d4 <= 8 * 128) {
@@ -326,7 +312,6 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
             for (int u = 0; u < 8; ++u) t[u] = tn[u];
             if (row + gridDim.x < M) fetch(row + gridDim.x);   // under this row's reductions
             TO* orow = out + (size_t)row * d;
-            bf16* rrow = out_lo ? out_lo + (size_t)row * d : nullptr;   // TO = bf16 only: the remainder plane's row
             if (raw) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
@@ -350,7 +335,7 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
                 const int k4 = threadIdx.x + 128 * u;
                 if (k4 < d4) {
                     const float4 g = gq[u], b = bq[u];
-                    ln_store4(orow, rrow, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
+                    ln_store4(orow, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
                               (t[u].z - mu) * rs * g.z + b.z, (t[u].w - mu) * rs * g.w + b.w);
                 }
             }
@@ -361,7 +346,6 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
         for (int row = blockIdx.x; row < M; row += gridDim.x) {
             const float4* xr = reinterpret_cast<const float4*>(x + (size_t)row * d);
             TO* orow = out + (size_t)row * d;
-            bf16* rrow = out_lo ? out_lo + (size_t)row * d : nullptr;
             float s = 0.f;
             for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
                 const float4 t = __ldcg(xr + k4);
@@ -379,7 +363,7 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
             for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
                 const float4 t = __ldcg(xr + k4);
                 const float4 g = __ldg(reinterpret_cast<const float4*>(gain) + k4), b = __ldg(reinterpret_cast<const float4*>(bias) + k4);
-                ln_store4(orow, rrow, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
+                ln_store4(orow, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
                           (t.w - mu) * rs * g.w + b.w);
             }
         }

@@ -122,7 +122,6 @@ struct tandem_ctx {
     int64_t ticket = 0;                  // verify kernels enqueued since creation (the device counts them too)
     // tensor-core path (bf16 only)
     int n_lns = 0;                       // LayerNorms of both models (bf16), see Layout::ln_src
-    bool tc = false;                     // weights have tensor maps; GEMMs run on tcgen05
     bool use_pdl = true;                 // programmatic dependent launch between the decode kernels
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
@@ -131,7 +130,6 @@ struct tandem_ctx {
     // TMA: maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
     // 1 small], 16-row boxes; and the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one).
     CUtensorMap xmap[3][2], lnmap[2];
-    std::vector<char> wmap_ok;
     std::vector<CUtensorMap> kmap, vmap; // the large model's key / value cache of each layer as [(seq, head, position)][d_head]
     cudaStream_t side = nullptr;         // the decode-time FF_Tandem projections run here, beside the large model's later layers
     std::vector<cudaEvent_t> ev_fork;    // one per small layer
@@ -698,7 +696,7 @@ template <typename T>
 void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr) {
     ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + sizeof(T) + (raw ? 2.0 : 0.0)));
     launch_ex(c, true, 1, layernorm_rows_kernel<T>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain), static_cast<const float*>(bias), out, d,
-              M, (bf16*)nullptr, raw);
+              M, raw);
 }
 
 // Describes the rows of one pass.
@@ -776,15 +774,14 @@ void attention(tandem_ctx& c, const Model& m, int l, const T* q, T* o, const Row
     launch_attn<T>(c, dh, aa, r.groups, !r.decode, r.n_chunks, r.kv_positions * 2.0 * d * sizeof(T));
 }
 
-// bf16 decode / block attention over the cache of layer l: bf16 queries, fp32 output rows.
-void attention_decode(tandem_ctx& c, const Model& m, int l, const bf16* q, float* o, const Rows& r, bf16* o_lo = nullptr) {
+// bf16 decode / block attention over the cache of layer l: bf16 queries, output rows as a value and a remainder plane.
+void attention_decode(tandem_ctx& c, const Model& m, int l, const bf16* q, bf16* o, bf16* o_lo, const Rows& r) {
     const int d = m.d.d_model, H = m.d.n_heads, dh = d / H;
     AttnArgs aa; memset(&aa, 0, sizeof(aa));
     aa.q = q; aa.ldq = d; aa.kcache = kv_ptr<bf16>(c, m, l, 0); aa.vcache = kv_ptr<bf16>(c, m, l, 1);
-    aa.out = o; aa.ldo = d; aa.out_f32 = 1; aa.row_seq = at<int>(c, c.lay.row_seq); aa.row_pos = at<int>(c, c.lay.row_pos);
+    aa.out = o; aa.out_lo = o_lo; aa.ldo = d; aa.row_seq = at<int>(c, c.lay.row_seq); aa.row_pos = at<int>(c, c.lay.row_pos);
     aa.nq = r.nq; aa.n_heads = H; aa.n_kv_heads = m.kv_heads; aa.t_max = c.cfg.max_seq; aa.scale = 1.0f / sqrtf((float)dh);
     aa.err_flag = tc_scratch(c).err;
-    aa.out_lo = o_lo;   // non-null: o is the bf16 value plane, o_lo the remainder plane
     launch_attn_decode(c, dh, aa, r.groups, r.kv_positions * 2.0 * d * 2.0);
 }
 
@@ -1085,7 +1082,7 @@ void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows
     launch_tc_decode<PRO_LNT, EPI_QKV>(c, sc, nullptr, d, nullptr, nullptr, r.M,
                                        tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w,
                                        epi_cache<bf16>(c, m, l, q), nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l));
-    attention_decode(c, m, l, q, reinterpret_cast<float*>(xo.hi), r, xo.lo);
+    attention_decode(c, m, l, q, xo.hi, xo.lo, r);
     EpiArgs eo = epi_plain(h, d);
     eo.ln = next_ln(c, m, 2 * l + 1);
     launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w, eo,
@@ -1451,12 +1448,10 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
         // two tensor maps per weight matrix: [out_features][in_features], 128 x 64 tiles and 32 x 64
         c->wmap.resize(c->w.size());
         c->wpart.resize(c->w.size());
-        c->wmap_ok.assign(c->w.size(), 0);
         bool ok = tmap_encoder() != nullptr;
         auto add = [&](int idx, int rows, int cols) {
-            if (ok && make_tmap_bf16(&c->wmap[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols) &&
-                make_tmap_bf16(&c->wpart[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols, 32)) c->wmap_ok[idx] = 1;
-            else ok = false;
+            ok = ok && make_tmap_bf16(&c->wmap[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols) &&
+                 make_tmap_bf16(&c->wpart[idx], c->w[idx], (uint64_t)rows, (uint64_t)cols, (uint64_t)cols, 32);
         };
         for (const Model* m : {&c->large, &c->small}) {
             const int d = m->d.d_model, dff = m->d.d_ff;
@@ -1501,7 +1496,6 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             delete c;
             return TANDEM_ERR_CUDA;
         }
-        c->tc = true;
         const int dhL = cfg->large.d_model / cfg->large.n_heads;
         if (dhL == 64 || dhL == 128) {
             c->kmap.resize(cfg->large.n_layers);
@@ -1825,9 +1819,7 @@ extern "C" tandem_status tandem_set_router(tandem_ctx* c, int32_t top_k, int32_t
     if (!w1 || !b1 || !w2 || top_k < 1 || top_k > RT_MAX_K || hidden < 1 || top_k > c->cfg.small.vocab) return TANDEM_ERR_INVALID_ARG;
     if (((uintptr_t)w1 | (uintptr_t)b1 | (uintptr_t)w2) & 3) return TANDEM_ERR_INVALID_ARG;
     if (sizeof(float) * (size_t)(1 + top_k + (size_t)top_k * c->cfg.small.d_model) > 48 * 1024) return TANDEM_ERR_SHAPE;   // the feature vector sits in shared memory
-    CK(cudaStreamSynchronize(c->stream));
-    for (auto& g : c->graphs)   // the router's arguments are baked into the captured draft steps
-        if (g.kind == 3 && g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
+    CK(cudaStreamSynchronize(c->stream));   // the caller may release the former router's weights
     c->router.w1 = static_cast<const float*>(w1); c->router.b1 = static_cast<const float*>(b1); c->router.w2 = static_cast<const float*>(w2);
     c->router.b2 = b2; c->router.tau = tau; c->router.k = top_k; c->router.hidden = hidden;
     c->has_router = true;
@@ -2253,7 +2245,7 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
         launch_tc_decode<PRO_LN, EPI_KV>(tmp, ts, yhat, d_small, ln_g, ln_b, rows, wkv, true, e);
     } else {
         launch_ex(tmp, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr, (bf16*)nullptr);
+                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr);
         launch_tc_decode<PRO_F32, EPI_KV>(tmp, ts, a_s, d_small, nullptr, nullptr, rows, wkv, true, e);
     }
     return check_launch();

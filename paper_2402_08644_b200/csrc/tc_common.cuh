@@ -87,11 +87,6 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-__device__ __forceinline__ uint64_t l2_policy_evict_last() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tm) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
 }
@@ -140,19 +135,7 @@ __device__ __forceinline__ uint64_t umma_desc_k_sw128(uint32_t smem_addr) {
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]^T; issued by one thread.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate) : "memory");
-}
-// The mbarrier gets one arrival when every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// The four products of 64 elements of K (K-major operands with the 128-byte swizzle), and a commit, issued by one lane of a
+// D[tmem] (+)= A[smem] * B[smem]^T: the four products of 64 elements of K (K-major operands with the 128-byte swizzle), and a commit, issued by one lane of a
 // converged warp: predicated, not branched to.  Inside `if (elect_one())` the compiler forms the operands again for every
 // product and the wait that precedes does not overlap: 317 clocks per K-block of 128 x 32 with its operands present, 205 like
 // this and with the next barrier asked for first, of which 160 are the products (40 clocks each for 32 columns or fewer).
@@ -169,6 +152,7 @@ __device__ __forceinline__ void umma_bf16_k64(uint32_t tmem_d, uint64_t desc_a, 
         ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "l"(desc_a + 2), "l"(desc_b + 2),
           "l"(desc_a + 4), "l"(desc_b + 4), "l"(desc_a + 6), "l"(desc_b + 6) : "memory");
 }
+// The mbarrier gets one arrival when every MMA issued so far by the elected lane has completed.
 __device__ __forceinline__ void umma_commit_one(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred e;\n\t"
@@ -237,15 +221,6 @@ __device__ __forceinline__ void cluster_sync_all() {
 // before that).  No memory ordering is needed for it.
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-// Reads a float at the same shared-memory offset in the cluster's CTA number `rank`.
-__device__ __forceinline__ float ld_dsmem_f32(uint32_t local_smem_addr, int rank) {
-    uint32_t remote;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_smem_addr), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-    return v;
-}
-
 // Writes a float to the same shared-memory offset in the cluster's CTA number `rank`.
 __device__ __forceinline__ void st_dsmem_f32(uint32_t local_smem_addr, int rank, float v) {
     uint32_t remote;
