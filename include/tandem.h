@@ -22,9 +22,11 @@
  *  - A context is bound to one device and one stream and is not thread-safe.  All GPU work is enqueued
  *    on that stream.
  *  - Greedy decisions: arg-max over fp32 logits, lowest token id on ties.
- *  - bf16 contexts: weights, queries and both KV caches are bf16; everything else between the kernels of a
- *    decode pass (residual stream, normalised rows, attention and GELU outputs) is fp32, and enters each
- *    tensor-core product as the sum of two bf16 numbers.  The prompt pass keeps bf16 activations.
+ *  - bf16 contexts: weights, queries and both KV caches are bf16.  Between the kernels of a decode pass the residual
+ *    stream is fp32; attention and GELU outputs, and the residual stream less a value near its mean times the next
+ *    LayerNorm's gain, are sums of two bf16 numbers (about 16 significant bits), as they enter the tensor-core
+ *    products.  The prompt pass keeps bf16 activations; which GEMM it takes depends on the rows of the whole pass, so
+ *    the last bits of a prompt's keys and values can depend on the prompts that it is batched with.
  *  - Weights are read where they lie, in every call.  A change that the context's stream orders between two calls holds
  *    from the second one on (for the positions that it computes: cached keys and values stay); a weight must not change
  *    while a call's work runs.

@@ -394,10 +394,10 @@ STATIC_SCRATCH_BYTES = 64 * 1024
 
 
 def tandem_decode_attention_static(q, k_derived, v_derived, k_own, v_own, out):
-    """tandem_decode_attention without a scratch argument, for callers that may not allocate device memory:
-    the kernel's work space (8 bytes per sequence) is a buffer built into the library (at most STATIC_SCRATCH_BYTES
-    are needed, else TandemError with status CAPACITY).  `out` is required, so this wrapper allocates nothing either.  Calls
-    share that buffer: keep them on one stream.  Make the first call on a device outside any stream capture."""
+    """tandem_decode_attention without a scratch argument, for callers that may not allocate device memory: `out` is
+    required, so this wrapper allocates nothing either.  Batches whose declared work space (8 bytes per sequence) exceeds
+    STATIC_SCRATCH_BYTES are refused (TandemError with status CAPACITY).  Calls share no state: they may overlap on
+    several streams."""
     lib = _lib or load_library()
     B, H, dh = q.shape
     _check_device(q, k_derived, v_derived, k_own, v_own, out)

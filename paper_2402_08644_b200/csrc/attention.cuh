@@ -277,9 +277,8 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
 //
 // The two small products of a 16-position tile run on the tensor cores as warp-level m16n8k16 MMAs, transposed: S^T = K Q^T with
 // the 16 keys as the MMA's rows and eight queries as its columns, O^T += V^T P^T with 16 elements of the head as rows.  (With
-// the queries as the 16 rows a block of up to eight of them left half of every MMA to absent rows, and these MMAs are slow,
-// about 32 clocks each on a quarter of a multiprocessor: 32 sequences x 16 heads x 64 x 8194 positions took 187-190 us a call, now
-// 169 us, 6.3 TB/s.)  K and V fragments come straight from the ring
+// the queries as the 16 rows a block of up to eight of them left half of every MMA to absent rows: 32 sequences x 16 heads x 64
+// x 8194 positions took 187-190 us a call, now 169 us, 6.3 TB/s.)  K and V fragments come straight from the ring
 // with ldmatrix (V transposed on the way), the queries stay in registers, the softmax works on the accumulator fragments (a
 // query's 16 scores sit in eight lanes), and the probabilities become the second product's B fragments by an 8 x 8 register
 // transpose, each as two bf16 numbers (value and remainder).  A query's column depends on its own query only, so a block

@@ -10,13 +10,12 @@
 // The S that takes the place of a chunk's P is issued right behind the product that reads P (a CTA's products run in issue
 // order), and one tile's softmax runs beside the other's products.  TMEM holds S / P and O of both tiles: all 512 columns.
 // Nothing but Q, K and V goes through shared memory, and a chunk of K and V serves 256 queries.
-// The bounds lie close together: at 128-wide heads 128 x 128 exponentials per 128 queries and keys are 1024 clocks of the
-// exponential unit, the products 768 (64 clocks for 128 x 128 x 16 out of shared memory, 32 with A in TMEM), and in
-// between a softmax warp's chain from S to P is about 1700 clocks with its barriers.  Chunks of 128 keys halve those fixed
-// parts and the products' share of reading Q; with 64-wide heads, whose prompts are short, the coarser diagonal costs as much.
-// The longest tiles start first (a causal tile costs what its position says).  8191 rows x 32 heads x 128: 448 us = 1228
-// TFLOP/s at full clocks, 488 us with chunks of 64 keys in two buffers.  Taking the chunk's maximum beside the exponentials
-// instead of before them was slower (470 us).
+// What bounds it (128-wide heads): per 128 queries and keys 128 x 128 exponentials, products whose A operand comes from TMEM for
+// half of them, and the softmax warps' own chain from S to P with its barriers; under ncu the tensor pipe and the
+// exponential unit are both 63 % busy.  Chunks of 128 keys halve the chain's fixed parts and the products' share of reading Q;
+// with 64-wide heads, whose prompts are short, the coarser diagonal costs as much.  The longest tiles start first (a causal
+// tile costs what its position says).  8191 rows x 32 heads x 128: 448 us = 1228 TFLOP/s at full clocks, 488 us with chunks of
+// 64 keys in two buffers.  Taking the chunk's maximum beside the exponentials instead of before them was slower (470 us).
 // The running maximum is lazy: probabilities are taken relative to a reference m that moves only when a chunk's
 // maximum exceeds it by more than ATC_LAZY (so they stay below e^ATC_LAZY); only then is O, in TMEM, rescaled
 // (tcgen05.ld, multiply, tcgen05.st) - rare after the first chunks.  The row sum adds the fp32 probabilities (their

@@ -28,8 +28,9 @@
 //  gemm_tc_split_kernel    prompt passes whose 256 x 256 tiles would leave multiprocessors idle: 128 x 128 tiles, one per
 //                          cluster of one, two or four CTAs that share the tile's K range.
 //
-// An output element's reduction order depends on (N, K) only, never on the number of rows, so a block
-// pass and a one-row pass give identical bits.
+// Decode kernel: an output element's reduction order depends on (N, K) only, never on the number of rows, so a block
+// pass and a one-row pass give identical bits.  Prompt kernels: the kernel and the K-slices are chosen from the pass's rows too, so
+// the last bits of a prompt's keys and values can depend on what it is batched with.
 #pragma once
 #include <limits.h>
 #include "common.cuh"
@@ -972,7 +973,7 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
 }
 
 // Prompt passes of few tiles (the small pair's 511 rows: 32 tiles of 128 x 128 for N = 1024): a tile's time is its
-// operands' way from L2 into one multiprocessor (32 KB per 64 of K at about 64 bytes a clock, twice the MMAs' time), so the
+// operands' way from L2 into one multiprocessor (32 KB per 64 of K; the tensor pipe is 7-26 % busy under ncu), so the
 // tile's K range is dealt to the S = 1, 2 or 4 CTAs of a cluster.  Each sends its partial sums of the columns that another
 // one finishes into that CTA's inbox (16-byte stores that count their bytes on the receiver's barrier, a lane per row, 512
 // contiguous bytes per warp and store), and CTA r finishes columns r * 128 / S ..: sums in slice order, then the

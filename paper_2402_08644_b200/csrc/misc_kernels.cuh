@@ -537,7 +537,8 @@ __global__ void __launch_bounds__(256) forced_fill_kernel(LoopState st, int batc
 // Scores of a teacher-forced round: for draft step s of sequence b, at position p = n_b - 1 + s, the negative
 // log-likelihood of the true token at p + 1 under softmax(logits) and the arg-max (lowest id on ties).
 // Bound by the latency of a row's passes: a row is dealt to the 64 warps of a cluster, whose ranges stay in registers between the
-// maximum and the sum (up to 32768 logits, else they are read again); the warps' maxima, positions and sums meet in the first
+// maximum and the sum (up to 32768 logits, else they are read again: 9.7 us a launch at 32768 and 32776 logits, 11.3 at 65536,
+// 13.8 at 131072); the warps' maxima, positions and sums meet in the first
 // CTA.  32000 logits, 16 rows: 19 us with one CTA per row and two passes over it, about 6 us like this.
 // logits: [gamma][batch][V].  grid: (SCR_CLUSTER, gamma, batch), a cluster per row; block: SCR_THREADS.
 constexpr int SCR_CLUSTER = 8, SCR_THREADS = 256, SCR_RANGES = SCR_CLUSTER * SCR_THREADS / 32, SCR_REGS = 16;

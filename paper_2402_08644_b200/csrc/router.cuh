@@ -7,8 +7,7 @@
 // model disagrees; drafting continues while 1 - s >= tau and fewer than gamma_max drafts exist.
 //
 // A sequence's row of logits and the hidden units are dealt to the CTAs of one cluster (a lone CTA took 43 us for 32000
-// logits and 64 x 2053 weights: one multiprocessor pulls about 64 bytes a clock, and every pass over the row follows the
-// one before): each CTA finds the maximum, the exponential sums and the k best of its slice and sends them to the others;
+// logits and 64 x 2053 weights: one multiprocessor's reads, and every pass over the row follows the one before): each CTA finds the maximum, the exponential sums and the k best of its slice and sends them to the others;
 // all of them merge the eight records, gather the feature vector and compute every eighth hidden unit; CTA 0 adds the
 // eight shares of w2 . hidden and decides.  A warp's first weights are fetched before the wait on the preceding kernel.
 // All sums run in a fixed order, fp32.  What is left (16 us for a launch alone, 8.7 of them in the kernel) is two cluster barriers
@@ -121,7 +120,7 @@ __global__ void __launch_bounds__(RT_THREADS) router_kernel(LoopState st, int ba
     if (st.drafting[b]) {   // (uniform over the cluster)
         const float* row = logits + (size_t)b * V;
         // Up to RT_REGS of the slice's logits per thread stay in registers (32768 in the row); longer rows are read again for
-        // each step.  `each` visits this thread's logits.
+        // each step (a launch 18.8 us at 32768 logits, 34.9 at 32776, 49.7 at 65536, 82 at 131072).  `each` visits this thread's logits.
         const bool in_regs = slice <= RT_THREADS * RT_REGS;
         float x[RT_REGS];
         if (in_regs) {

@@ -344,8 +344,8 @@ bool make_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t c
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The same, remembered: a tensor map depends on nothing but its arguments, and the stand-alone calls get the same matrices again
-// and again (an encoding costs the host about 0.4 us).  128 maps per thread, 24 KB, the last one to hash to a place stays.
+// The same, remembered: a tensor map depends on nothing but its arguments, and the stand-alone calls get the same weight matrices again
+// and again (an encoding costs the host about 0.4 us, which the first call on a matrix pays).  128 maps per thread, 24 KB, the last one to hash to a place stays.
 bool cached_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols) {
     struct Entry { const void* base; uint64_t rows, cols; CUtensorMap tm; };
     static thread_local std::vector<Entry> cache;
@@ -659,7 +659,8 @@ int attn_max_clusters(int cl) {
 }
 // Cluster size, 1, 2, 4 or 8: the one with the least rounds of resident clusters x (a CTA's share of the context + what a CTA
 // costs apart from it, about two and a half chunks).  It depends on the number of sequences and key/value heads only (the
-// share is taken of 24 chunks, 3072 positions), so every pass of a run (block or one-row) cuts the context the same way.
+// share is taken of 24 chunks, 3072 positions), so every pass of a run (block or one-row) cuts the context the same way.  The
+// stand-alone call takes the same rule; its length is not looked at.
 // Two sequences x 8 key/value heads x 128, blocks of six rows: 35-41 us with eight (16 clusters where 15 fit), 18.6 us with
 // four.  20 sequences x 16 heads x 64 x 3000 positions, 320 clusters where 296 CTAs fit: 61 us with one, 52 with two, 49 with
 // four; 32 x 16 x 64 x 8194: 160 us with one, 166 with two.  (Sizes in between measured 3 % slower per iteration at batch 8: a

@@ -49,11 +49,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 }
 
 // ---- one thread of a converged warp -------------------------------------------------------------
-// The warps that issue TMA copies and MMAs run their loops with all lanes and let one elected lane issue.  Written as
-// `if (lane == 0)` around the loop, the code is divergent for the compiler: every operand of an MMA (two 64-bit
-// descriptors, the TMEM address) is moved from vector to uniform registers one by one, about 66 clocks per instruction,
-// twice the 32 clocks that a 128 x 64 x 16 product runs.  Converged, with warp-wide votes on the waits, they are
-// computed in uniform registers (prompt attention, 8191 rows x 32 heads x 128: 752 -> 502 us from this alone).
+// The warps that issue TMA copies and MMAs run their loops with all lanes, vote on their waits and let one elected lane issue:
+// operands known to be the same in the whole warp are cheap to form.  With `if (lane == 0)` around the loop the issue of a
+// product took longer than the product (prompt attention, 8191 rows x 32 heads x 128: 752 us, 502 us like this).
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
@@ -64,7 +62,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, ui
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit)) != 0;
 }
 // Whether the phase with the given parity has completed, without waiting for it: asked before the products of the K-block before are
-// issued and used after, the answer's way (about 115 clocks) runs beside them.
+// issued and used after, the answer's way runs beside them.
 __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -135,10 +133,9 @@ __device__ __forceinline__ uint64_t umma_desc_k_sw128(uint32_t smem_addr) {
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]^T: the four products of 64 elements of K (K-major operands with the 128-byte swizzle), and a commit, issued by one lane of a
-// converged warp: predicated, not branched to.  Inside `if (elect_one())` the compiler forms the operands again for every
-// product and the wait that precedes does not overlap: 317 clocks per K-block of 128 x 32 with its operands present, 205 like
-// this and with the next barrier asked for first, of which 160 are the products (40 clocks each for 32 columns or fewer).
+// D[tmem] (+)= A[smem] * B[smem]^T: the four products of 64 elements of K (K-major operands with the 128-byte swizzle), issued by one
+// lane of a converged warp: predicated, not branched to, so that the operands are formed once and the wait for the next
+// K-block overlaps.
 __device__ __forceinline__ void umma_bf16_k64(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred e, p, t;\n\t"
@@ -215,10 +212,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// The same barrier in two halves.  cluster_arrive_relaxed + cluster_wait is the opening handshake of a kernel that
-// writes into its peers' shared memory: a CTA arrives right after its set-up and waits just before its first
-// remote store, by which time every CTA of the cluster has started (remote shared memory may not be touched
-// before that).  No memory ordering is needed for it.
+// The same barrier in two halves, for the opening handshake of a kernel that writes into its peers' shared memory and for nothing
+// else: a CTA arrives right after its set-up and waits just before its first remote store, by which time every CTA of the cluster
+// has started (remote shared memory may not be touched before that).  It orders no memory but the mbarriers' initialisation,
+// which mbar_init_fence releases.
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // Writes a float to the same shared-memory offset in the cluster's CTA number `rank`.

@@ -1,7 +1,7 @@
 """Seeded synthetic inputs for Tandem + SPEED: model shapes, random-init weights, random prompts.
 
 This module holds no arithmetic of the method.  It only produces the arrays that both the CUDA path
-and the CPU checker consume: weight tensors drawn from N(0, std^2), LayerNorm gains of one and
+and the CPU oracle consume: weight tensors drawn from N(0, std^2), LayerNorm gains of one and
 biases of zero, and prompts of i.i.d. uniform token ids.  The fixed-length random prompts stand in
 for the paper's CNN/DailyMail, Reddit Posts and LM1B prompts (Section 4.2), and the random-init
 weights for its PaLM2 checkpoints (Section 4, "Further Training Details"), none of which are
@@ -205,7 +205,7 @@ def make_self_tandem_weights(shape: TandemShape, seed: int, std: float = 0.02) -
 def device_weights(shape: TandemShape, seed: int, device) -> Dict[str, "torch.Tensor"]:
     """Random-init weights of the same distribution drawn directly on a CUDA device as torch tensors (bf16
     matrices, fp32 LayerNorm parameters), for shapes too large to draw on the host in reasonable time.  No CPU
-    checker run can use them: they serve timing and GPU-internal invariants only."""
+    oracle run can use them: they serve timing and GPU-internal invariants only."""
     import torch
     g = torch.Generator(device=device).manual_seed(seed)
     out = {}
