@@ -15,7 +15,7 @@ of the medium (batch 8) and large (batch 1) configurations.
 With N > 1 (under torchrun) every rank runs an independent replica (sequences are independent units; there
 is no collective on the path); the value is all ranks' tokens over the slowest rank's time.
 
-`--impl reference` times the CPU checker (oracle/) on the host cores on a bounded sample of the same workload.
+`--impl reference` times the CPU oracle (oracle/) on the host cores on a bounded sample of the same workload.
 """
 from __future__ import annotations
 
@@ -60,7 +60,7 @@ def workload_desc(name):
 
 # DRAM bytes (read + write) of one decode iteration from one ncu capture of every kernel of an iteration, valid only
 # while the kernel sources are the ones that were profiled (else the line reports null).
-NCU_TRAFFIC = {"workload": "small", "bytes_per_iteration": 599.35e6, "sources_sha256_16": "2379be2240073bf1"}
+NCU_TRAFFIC = {"workload": "small", "bytes_per_iteration": 597.4e6, "sources_sha256_16": "492e6301ef66ee0a"}
 
 
 def kernel_sources_hash():
@@ -144,7 +144,7 @@ def algorithmic_bytes_per_iteration(shape, B, gamma, T):
 
 
 def run_reference(args):
-    """The CPU checker as it stands, on the host cores, on a bounded sample of the workload."""
+    """The CPU oracle as it stands, on the host cores, on a bounded sample of the workload."""
     rank = int(os.environ.get("RANK", "0"))
     if rank != 0:
         return
