@@ -1,4 +1,4 @@
-"""CPU checker for greedy Tandem + SPEED decoding (Tandem Transformers, arXiv 2402.08644).
+"""CPU oracle for greedy Tandem + SPEED decoding (Tandem Transformers, arXiv 2402.08644).
 
 THIS IS TEST INFRASTRUCTURE, NOT A PRODUCT PATH.  It is a plain, slow, fp64 numpy restatement of the
 paper's equations, used by the tests, by the smoke check and by the benchmark's CPU-baseline leg to
