@@ -342,7 +342,11 @@ __device__ __forceinline__ uint32_t atd_pack_bf16x2(float lo, float hi) {
 
 // grid: (CL, heads, sequences) with the CL CTAs along x forming one cluster, CL in {1, 2, 4, 8}; block: ATD_THREADS.
 // NT: groups of eight query columns in use (1 up to eight rows per CTA, 2 up to 16).
-template <int DH, int NT>
+// MODE: ATD_CLUSTERED, CL in {2, 4, 8}; ATD_ALONE, CL = 1, results straight from the fold of the warps' states (32 x 16 x 64 x 8194:
+// 171 -> 165 us, without the trip through the inbox).  (The same code with this choice made at run time costs the stand-alone call on
+// 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
+enum { ATD_CLUSTERED = 0, ATD_ALONE = 1 };
+template <int DH, int NT, int MODE>
 __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     using C = AtdCfg<DH>;
     constexpr int NW = ATD_WARPS;
@@ -358,7 +362,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // key/value head (row = head * nq + block row), so their keys and values are streamed once for all of them.
     const int gpc = a.heads_per_cta > 0 ? a.heads_per_cta : 1;
     const int h = blockIdx.y * gpc;                // first query head of this CTA
-    const int CL = gridDim.x;                      // cluster size
+    const int CL = MODE == ATD_CLUSTERED ? gridDim.x : 1;   // cluster size
     const int QPC = (ATT_NQ + CL - 1) / CL;        // queries a CTA finishes at most
     __shared__ __align__(8) uint64_t s_inbox_bar;  // counts the bytes of the states sent to this CTA by the cluster's CTAs
     if (CL > 1 && tid == 0) { mbar_init(smem_u32(&s_inbox_bar), 1); mbar_init_fence(); }
@@ -577,8 +581,20 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     __syncthreads();
     // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa % CL
     if (CL > 1) cluster_wait();   // closes the opening handshake: every CTA of the cluster is running
+    auto store = [&](int qi, int e, float res) {   // tile row qi = query head hq of this CTA, block row qi - hq * nq
+        const int hq = qi / nq;
+        const size_t oi = (size_t)(row0 + qi - hq * nq) * a.ldo + (h + hq) * DH + e;
+        if (a.out_lo) {
+            const bf16 hi = __float2bfloat16_rn(res);
+            static_cast<bf16*>(a.out)[oi] = hi;
+            static_cast<bf16*>(a.out_lo)[oi] = __float2bfloat16_rn(res - __bfloat162float(hi));
+        } else {
+            static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
+        }
+    };
     // One thread per (query, output element); the thread of element 0 also folds the query's running sum and sends its
-    // maximum (with 4 queries of 64 elements that is one pass over the block's 256 threads).
+    // maximum (with 4 queries of 64 elements that is one pass over the block's 256 threads).  A CTA on its own has the result
+    // right here (every thread folds the sum then).
     for (int i = tid; i < cnt * DH; i += ATD_THREADS) {
         const int qa = i / DH, e = i - qa * DH;
         float mx = -INFINITY;
@@ -590,21 +606,18 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             const float* st = wst + (size_t)(w * ATT_NQ + qa) * SW;
             const float f = st[DH] > -INFINITY ? __expf(st[DH] - mx) : 0.f;
             val = fmaf(st[e], f, val);
-            if (e == 0) lsum = fmaf(st[DH + 1], f, lsum);
+            if (e == 0 || MODE != ATD_CLUSTERED) lsum = fmaf(st[DH + 1], f, lsum);
         }
+        if (MODE != ATD_CLUSTERED) { store(qa, e, val / lsum); continue; }
         float* slot = inbox + ((size_t)rank * QPC + qa / CL) * SW;
-        if (CL > 1) {   // counted on the receiver's barrier
-            st_async_dsmem_f32(smem_u32(slot + e), smem_u32(&s_inbox_bar), qa % CL, val);
-            if (e == 0) {
-                st_async_dsmem_f32(smem_u32(slot + DH), smem_u32(&s_inbox_bar), qa % CL, mx);
-                st_async_dsmem_f32(smem_u32(slot + DH + 1), smem_u32(&s_inbox_bar), qa % CL, lsum);
-            }
-        } else {
-            slot[e] = val;
-            if (e == 0) { slot[DH] = mx; slot[DH + 1] = lsum; }
+        st_async_dsmem_f32(smem_u32(slot + e), smem_u32(&s_inbox_bar), qa % CL, val);   // counted on the receiver's barrier
+        if (e == 0) {
+            st_async_dsmem_f32(smem_u32(slot + DH), smem_u32(&s_inbox_bar), qa % CL, mx);
+            st_async_dsmem_f32(smem_u32(slot + DH + 1), smem_u32(&s_inbox_bar), qa % CL, lsum);
         }
     }
-    if (CL > 1) {
+    if (MODE != ATD_CLUSTERED) return;
+    {
         // This CTA finishes queries rank, rank + CL, ...: it waits (bounded) until every CTA's state of each of them
         // has arrived.  No cluster-wide barrier: a CTA without queries of its own leaves right after sending.
         const int n_fin = rank < cnt ? (cnt - rank + CL - 1) / CL : 0;
@@ -612,8 +625,6 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             if (tid == 0) mbar_arrive_expect_tx(smem_u32(&s_inbox_bar), (uint32_t)(CL * n_fin * SW * 4));
             if (!mbar_wait(smem_u32(&s_inbox_bar), 0) && a.err_flag) atomicExch(a.err_flag, ATD_ERR_EXCHANGE);
         }
-    } else {
-        __syncthreads();
     }
     for (int u = 0; u < QPC; ++u) {
         const int qi = rank + u * CL;
@@ -638,16 +649,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
                     ov = fmaf(orr[r], f, ov);
                 }
             }
-            const int hq = qi / nq;                  // tile row qi = query head hq of this CTA, block row qi - hq * nq
-            const size_t oi = (size_t)(row0 + qi - hq * nq) * a.ldo + (h + hq) * DH + tid;
-            const float res = ov / l;
-            if (a.out_lo) {
-                const bf16 hi = __float2bfloat16_rn(res);
-                static_cast<bf16*>(a.out)[oi] = hi;
-                static_cast<bf16*>(a.out_lo)[oi] = __float2bfloat16_rn(res - __bfloat162float(hi));
-            } else {
-                static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
-            }
+            store(qi, tid, ov / l);
         }
     }
 }

@@ -623,17 +623,21 @@ void launch_attn(tandem_ctx& c, int d_head, const AttnArgs& a, int groups, bool 
 }
 
 // bf16 decode attention: one cluster of `cl` CTAs per (sequence, group of query heads); no scratch.
+template <int DH, int NT, int MODE>
+void launch_attn_decode_as(tandem_ctx& c, const AttnArgs& a, dim3 grid) {
+    static std::atomic<unsigned long long> attr_done{0};
+    ensure_dyn_smem(attn_decode_kernel<DH, NT, MODE>, attn_decode_smem_bytes<DH>(), attr_done);
+    launch_ex(c, true, (int)grid.x, attn_decode_kernel<DH, NT, MODE>, grid, dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
+}
 template <int DH>
 void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl, double kv_bytes) {
-    static std::atomic<unsigned long long> attr_done1{0}, attr_done2{0};
     const int gpc = std::max(1, a.heads_per_cta);
+    const bool narrow = gpc * a.nq <= 8;
+    const dim3 grid(cl, a.n_heads / gpc, groups);
     ProfScope ps(c, PC_ATTN_SPLIT, kv_bytes);
-    auto launch = [&](auto kernel, std::atomic<unsigned long long>& done) {
-        ensure_dyn_smem(kernel, attn_decode_smem_bytes<DH>(), done);
-        launch_ex(c, true, cl, kernel, dim3(cl, a.n_heads / gpc, groups), dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
-    };
-    if (gpc * a.nq <= 8) launch(attn_decode_kernel<DH, 1>, attr_done1);
-    else launch(attn_decode_kernel<DH, 2>, attr_done2);
+    if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid); }
+    else if (narrow) launch_attn_decode_as<DH, 1, ATD_CLUSTERED>(c, a, grid);
+    else launch_attn_decode_as<DH, 2, ATD_CLUSTERED>(c, a, grid);
 }
 // Clusters of `cl` decode-attention CTAs that the device can run at the same time (asked once per device and size).  It is
 // less than the multiprocessors would suggest, because a cluster has to fit into one GPC: with 148 multiprocessors and one
@@ -645,7 +649,7 @@ int attn_max_clusters(int cl) {
     int n = slot.load(std::memory_order_relaxed);
     if (n > 0) return n;
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(attn_decode_kernel<DH, 2>, attn_decode_smem_bytes<DH>(), attr_done);
+    ensure_dyn_smem(attn_decode_kernel<DH, 2, ATD_CLUSTERED>, attn_decode_smem_bytes<DH>(), attr_done);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(cl); cfg.blockDim = dim3(ATD_THREADS); cfg.dynamicSmemBytes = attn_decode_smem_bytes<DH>();
@@ -653,7 +657,7 @@ int attn_max_clusters(int cl) {
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)cl; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_decode_kernel<DH, 2>, &cfg) != cudaSuccess || n < 1) n = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_decode_kernel<DH, 2, ATD_CLUSTERED>, &cfg) != cudaSuccess || n < 1) n = 1;
     slot.store(n, std::memory_order_relaxed);
     return n;
 }

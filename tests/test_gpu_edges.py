@@ -103,6 +103,20 @@ def test_teacher_forced_scores_over_a_cluster(vocab):
     t.close()
 
 
+@pytest.mark.parametrize("batch,heads,dh,derived,own", [(160, 2, 64, 130, 3), (301, 1, 128, 127, 1), (300, 2, 32, 0, 1)])
+def test_decode_attention_by_lone_ctas(batch, heads, dh, derived, own):
+    """More (sequence, head) pairs than clusters would fit: one CTA for each, whose result leaves with the fold of its warps' states
+    (contexts of one and two chunks, and of one key)."""
+    import torch
+    g = torch.Generator().manual_seed(batch)
+    mk = lambda *s: torch.randn(*s, generator=g).to(torch.bfloat16)
+    q, kd, vd, ko, vo = mk(batch, heads, dh), mk(batch, heads, derived, dh), mk(batch, heads, derived, dh), mk(batch, heads, own, dh), mk(batch, heads, own, dh)
+    out = binding.tandem_decode_attention(*(x.cuda() for x in (q, kd, vd, ko, vo))).double().cpu()
+    K, V = torch.cat([kd, ko], 2).double(), torch.cat([vd, vo], 2).double()
+    want = (torch.softmax((K @ q.double()[..., None])[..., 0] / dh ** 0.5, -1)[..., None, :] @ V)[..., 0, :]
+    assert (out - want).abs().max() < TOL_BF16
+
+
 def test_bf16_layernorm_parameters_changed_between_calls():
     """Gains and biases that the caller changes after the prompt pass, and again between two steps, hold from the next call on, in
     every map behind a LayerNorm and in the projection."""
