@@ -29,6 +29,8 @@ struct AttnArgs {
     const void* kcache; const void* vcache;   // [seq][head][t_max][DH]
     const void* k2; const void* v2;            // optional second segment [seq][head][t_max2][DH] holding
     int split, t_max2;                         //   positions >= split (used when k2 != nullptr)
+    //   (attn_decode_kernel, ATD_PASS: the second segment is a cache like the first, indexed by absolute position, and holds the
+    //   positions from the group's first row on; split and t_max2 unused)
     void* out; int ldo;                  // T [M][ldo]
     const int* row_seq; const int* row_pos;    // attn_decode_kernel: row_seq may be null, then group g is sequence g and every
     int pos_all;                               //   sequence's first row sits at position pos_all (no row arrays to fill and fetch)
@@ -340,12 +342,12 @@ __device__ __forceinline__ uint32_t atd_pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&p);
 }
 
-// grid: (CL, heads, sequences) with the CL CTAs along x forming one cluster, CL in {1, 2, 4, 8}; block: ATD_THREADS.
+// grid: (CL, heads, sequences or groups) with the CL CTAs along x forming one cluster, CL in {1, 2, 4, 8}; block: ATD_THREADS.
 // NT: groups of eight query columns in use (1 up to eight rows per CTA, 2 up to 16).
 // MODE: ATD_CLUSTERED, CL in {2, 4, 8}; ATD_ALONE, CL = 1, results straight from the fold of the warps' states (32 x 16 x 64 x 8194:
-// 171 -> 165 us, without the trip through the inbox).  (The same code with this choice made at run time costs the stand-alone call on
-// 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
-enum { ATD_CLUSTERED = 0, ATD_ALONE = 1 };
+// 171 -> 165 us, without the trip through the inbox); ATD_PASS, CL = 1 in a teacher-forced pass: groups of unequal length, the second segment of a block's own keys.  (The
+// same code with these choices made at run time costs the stand-alone call on 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
+enum { ATD_CLUSTERED = 0, ATD_ALONE = 1, ATD_PASS = 2 };
 template <int DH, int NT, int MODE>
 __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     using C = AtdCfg<DH>;
@@ -372,8 +374,10 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // The row arrays were written at the start of the pass, at least two kernels back in the stream, so they may be
     // read before the wait below: a kernel lets its successor start only after its own wait has returned, that is
     // after its predecessor has finished, hence everything older than the immediate predecessor is complete.
-    const int nq = a.nq, cnt = gpc * nq, row0 = g * nq;   // cnt: rows of the tile in use
     if (a.wait_first) pdl_wait();
+    int nq = a.nq, row0 = g * nq;
+    if (MODE == ATD_PASS && a.grp_cnt) { nq = __ldcg(a.grp_cnt + g); row0 = __ldcg(a.grp_row0 + g); }
+    const int cnt = gpc * nq;                      // rows of the tile in use
     const int b = a.row_seq ? __ldcg(a.row_seq + row0) : g;          // from L2: nothing an earlier kernel on this SM may have cached
     const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
     const int pos_last = pos_first + nq - 1;
@@ -382,8 +386,9 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
     const int kvh = h / (a.n_heads / n_kv);            // grouped-query attention: several query heads share one key/value head
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
-    const size_t head_base2 = ((size_t)b * n_kv + kvh) * a.t_max2;
-    const int split = a.k2 ? a.split : INT_MAX;
+    const size_t head_base2 = ((size_t)b * n_kv + kvh) * (MODE == ATD_PASS ? a.t_max : a.t_max2);
+    const int split = a.k2 ? (MODE == ATD_PASS ? pos_first : a.split) : INT_MAX;
+    const int base2 = MODE == ATD_PASS ? 0 : split;    // position of the second segment's first key
 
     // this warp's rows of its CTA's it-th chunk into stage it % STAGES.  Lane L moves unit L % TPK of rows
     // L / TPK + (32 / TPK) * u; a tile that lies wholly in one cache and before the last query (all but a
@@ -396,7 +401,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         bf16* vs = ks + C::TILE_ELEMS;
         const bool first = t0 + ATD_WROWS <= split, second = t0 >= split;
         if (t0 + ATD_WROWS - 1 <= pos_last && (first || second)) {
-            const size_t src = first ? (head_base + t0 + i_row) * DH : (head_base2 + (t0 - split) + i_row) * DH;
+            const size_t src = first ? (head_base + t0 + i_row) * DH : (head_base2 + (t0 - base2) + i_row) * DH;
             const bf16* kg = static_cast<const bf16*>(first ? a.kcache : a.k2) + src + i_unit * 8;
             const bf16* vg = static_cast<const bf16*>(first ? a.vcache : a.v2) + src + i_unit * 8;
 #pragma unroll
@@ -419,8 +424,8 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
                     kg = static_cast<const bf16*>(a.kcache) + (head_base + ta) * DH;
                     vg = static_cast<const bf16*>(a.vcache) + (head_base + ta) * DH;
                 } else {
-                    kg = static_cast<const bf16*>(a.k2) + (head_base2 + (ta - split)) * DH;
-                    vg = static_cast<const bf16*>(a.v2) + (head_base2 + (ta - split)) * DH;
+                    kg = static_cast<const bf16*>(a.k2) + (head_base2 + (ta - base2)) * DH;
+                    vg = static_cast<const bf16*>(a.v2) + (head_base2 + (ta - base2)) * DH;
                 }
                 cp_async16(ks + dst, kg + v * 8);
                 cp_async16(vs + dst, vg + v * 8);

@@ -48,6 +48,7 @@ namespace tandem {
 // 4.4 + 1.9 us with a LayerNorm kernel of their own (more sequences).
 enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3, PRO_LNT = 4 };
 constexpr int EPI_ARGMAX = 6;                       // fp32 store plus the (max, index) of each row within the tile
+constexpr int EPI_SCORE = 7;                        // no store: per row the tile's (max, index, sum of exp(y - max)), and y at a given feature
 enum { TC_ERR_SLOT = 1, TC_ERR_OPERANDS = 2, TC_ERR_ACCUM = 3, TC_ERR_EXCHANGE = 4 };   // which bounded wait gave up
 
 struct TcDecodeArgs {
@@ -75,11 +76,31 @@ struct TcDecodeArgs {
     unsigned poll_limit;    // polls before a wait on an mbarrier gives up; 0 = MBAR_POLL_LIMIT
     int withhold_weights;   // test hook for the give-up path: the TMA thread issues no loads, so the wait for
                             // operands must run out (nothing is in flight when the kernel leaves)
-    float* amax_val;        // EPI_ARGMAX: [rows][amax_stride] best value per tile
+    float* amax_val;        // EPI_ARGMAX, EPI_SCORE: [rows][amax_stride] best value per tile
     int* amax_idx;          //             and its output feature
     int amax_stride;
+    float* score_sum;       // EPI_SCORE: [rows][amax_stride] sum over the tile's features of exp(y - the tile's best value)
+    const int* truth;       // EPI_SCORE: [rows] the feature whose value goes to truth_val [rows]
+    float* truth_val;
     EpiArgs e;
 };
+
+// The same pass from its row r0 on (nr rows): everything that is indexed by token row moves along.
+template <int PRO, int EPI>
+__host__ __device__ __forceinline__ void tcd_shift_rows(TcDecodeArgs& a, int r0, int nr) {
+    a.rows = nr;
+    a.x_row0 += r0;
+    if (a.x) a.x = static_cast<const unsigned char*>(a.x) + (size_t)r0 * a.ldx * (PRO == PRO_BF16 ? 2 : 4);
+    if (PRO == PRO_LNT) { a.ln_stats += (size_t)r0 * a.ln_groups; a.ln_ref += r0; a.ln_mean += r0; }
+    if (EPI == EPI_ARGMAX || EPI == EPI_SCORE) { a.amax_val += (size_t)r0 * a.amax_stride; a.amax_idx += (size_t)r0 * a.amax_stride; }
+    if (EPI == EPI_SCORE) { a.score_sum += (size_t)r0 * a.amax_stride; a.truth += r0; a.truth_val += r0; }
+    EpiArgs& e = a.e;
+    if (e.out) e.out = static_cast<unsigned char*>(e.out) + (size_t)r0 * e.ldo * ((EPI == EPI_QKV || EPI == EPI_STORE || e.out_lo) ? 2 : 4);
+    if (e.out_lo) e.out_lo = static_cast<unsigned char*>(e.out_lo) + (size_t)r0 * e.ldo * 2;   // (value / remainder planes are bf16)
+    if (e.row_seq) { e.row_seq += r0; e.row_pos += r0; }
+    if (e.snap) e.snap = static_cast<float*>(e.snap) + (size_t)r0 * e.snap_ld;
+    if (e.ln.gain) { e.ln.hi += (size_t)r0 * e.ldo; e.ln.lo += (size_t)r0 * e.ldo; e.ln.stats += (size_t)r0 * e.ln.groups; e.ln.ref += r0; }
+}
 
 constexpr int TCD_THREADS = 192;   // warps 0-3: B operand + epilogue; warp 4: TMA; warp 5: TMEM + MMA issue
 template <int NB, bool LNT> struct TcdCfg {
@@ -92,6 +113,7 @@ template <int NB, bool LNT> struct TcdCfg {
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + (LNT ? 1024 : 0);   // (the MMA's last twelve B rows are whatever follows: unread columns)
     static constexpr int INBOX_BYTES = NB * 128 * 4;   // the K-slices' partial sums for the token rows this CTA finishes
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + INBOX_BYTES + 1024;   // + slack to align the ring to 1024
+    static constexpr int SMEM_BYTES_WHOLE = STAGES * STAGE_BYTES + 1024 + (LNT ? 1024 : 0);   // whole K, nothing exchanged: no inbox (LNT: the unread B rows of the last stage)
     static constexpr int TMEM_COLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
 static_assert(TcdCfg<16, true>::SMEM_BYTES + 1024 <= 113 * 1024 && TcdCfg<16, false>::SMEM_BYTES + 1024 <= 113 * 1024 &&
@@ -133,15 +155,152 @@ __device__ __forceinline__ ScatterCol scatter_col(const EpiArgs& e, int seg, int
     return sc;
 }
 
-// grid: tiles * splits CTAs in clusters of `splits` (the K-slices of one tile); dynamic smem TcdCfg::SMEM_BYTES.
+// The epilogue of a whole pass (PASS): sixteen rows at a time, from TMEM to their places, in a loop that stays in the instruction cache
+// (the decode passes' epilogue, unrolled over its rows, is fetched once per CTA: 32 us for 384 rows x 4096 x 1024 with GELU
+// under ncu, 34 us for 772 rows like this).  Warps 0-3; thread = output feature.
 template <int NB, int PRO, int EPI>
+__device__ __forceinline__ void tcd_pass_epilogue(const TcDecodeArgs& a, uint32_t tmem, int seg, int seg_rows, int seg_base, int n_local0, int tile, unsigned char* ring,
+                                                  float* s_mu, const float* s_rstd, long long* s_rowoff, uint64_t* s_accum, float next_gain, int my_seq, int my_pos,
+                                                  uint32_t poll_limit, bool long_slice) {
+    constexpr bool LNT = PRO == PRO_LNT, BY_TMA = PRO == PRO_TMA || LNT;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    if (warp >= 4) return;
+    if (!BY_TMA || (!LNT && (!long_slice || a.release_early))) pdl_launch_dependents();
+    if (EPI == EPI_QKV || EPI == EPI_KV) {
+        if (tid < a.rows) s_rowoff[tid] = ((long long)my_seq * a.e.n_heads * a.e.t_max + my_pos) * a.e.d_head;
+        bar_sync(1, 128);
+    }
+    const bool with_ln = EPI == EPI_RESID && a.e.ln.gain;
+    if (with_ln) bar_sync(1, 128);
+    const int n_local = n_local0 + tid, n = seg_base + n_local;
+    const bool valid = n_local < seg_rows;
+    float hres[EPI == EPI_RESID ? 16 : 1];   // residual values, sixteen rows ahead
+    auto fetch = [&](int j0) {
+        const float* hp = static_cast<const float*>(a.e.out) + n;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) hres[EPI == EPI_RESID ? i : 0] = valid && j0 + i < a.rows ? __ldcg(hp + (size_t)(j0 + i) * a.e.ldo) : 0.f;
+    };
+    if (EPI == EPI_RESID) fetch(0);
+    ScatterCol sc;
+    if (EPI == EPI_QKV || EPI == EPI_KV) sc = scatter_col<EPI>(a.e, seg, n_local);
+    const int n_group = max(0, min(32, seg_rows - (n_local0 + warp * 32)));   // features of this warp's group of 32
+    const float inv = 1.0f / (float)max(1, n_group);
+    if (!mbar_wait(smem_u32(s_accum), 0, poll_limit)) tc_report(a.err_flag, TC_ERR_ACCUM);
+    tc_fence_after_sync();
+    const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+    float c1 = 0.f, c2 = 0.f;                // PRO_LNT: this feature's g W^T and b W^T
+    if (LNT) {
+        float w[16];
+        tmem_ld16(acc + 2 * NB, w);
+        c1 = w[0] + w[1];
+        c2 = w[2] + w[3];
+    }
+    constexpr int LD = 130;                  // EPI_SCORE: the tile in shared memory, [row][feature]: 16 rows x 2 threads of a warp meet 32 banks
+    float* tile_v = reinterpret_cast<float*>(ring);   // (where the ring was: every product has read it)
+#pragma unroll 1
+    for (int c0 = 0; c0 < a.rows; c0 += 16) {
+        float v[16], u[16];
+        tmem_ld16(acc + c0, v);              // x's values times W
+        tmem_ld16(acc + NB + c0, u);         // x's remainders times W
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            v[i] += u[i];
+            if (LNT) v[i] = fmaf(s_rstd[c0 + i], fmaf(-s_mu[c0 + i], c1, v[i]), c2);   // (rows past the last: never used)
+            if (EPI == EPI_RESID) v[i] += hres[EPI == EPI_RESID ? i : 0];
+        }
+        if (EPI == EPI_RESID && c0 + 16 < a.rows) fetch(c0 + 16);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int j = c0 + i;
+            if (j >= a.rows) break;
+            if (EPI == EPI_SCORE) { tile_v[j * LD + tid] = valid ? v[i] : -INFINITY; continue; }
+            if (!valid) continue;
+            if (EPI == EPI_RESID || EPI == EPI_STORE_F32) {
+                static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = v[i];
+                if (with_ln) {
+                    const float x = (v[i] - s_mu[j]) * next_gain;
+                    const bf16 hi = __float2bfloat16_rn(x);
+                    a.e.ln.hi[(size_t)j * a.e.ldo + n] = hi;
+                    a.e.ln.lo[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                }
+            } else if (EPI == EPI_GELU) {
+                const float gv = gelu_bf16_out(v[i]);
+                if (a.e.out_lo) {
+                    const bf16 hi = __float2bfloat16_rn(gv);
+                    static_cast<bf16*>(a.e.out)[(size_t)j * a.e.ldo + n] = hi;
+                    static_cast<bf16*>(a.e.out_lo)[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(gv - __bfloat162float(hi));
+                } else {
+                    static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = gv;
+                }
+            } else {
+                sc.base[(sc.is_q ? (long long)j * a.e.ldo : s_rowoff[j]) + sc.col] = __float2bfloat16_rn(v[i]);
+            }
+        }
+        if (with_ln && n_group > 0) {        // (warp-uniform) statistics for the next LayerNorm, as in the decode passes' epilogue
+#pragma unroll
+            for (int s0 = 0; s0 < 16; s0 += 4) {
+                if (c0 + s0 >= a.rows) break;
+                float sums[8], ref[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    ref[k] = __shfl_sync(0xffffffffu, v[s0 + k], 0);
+                    const float dv = valid ? v[s0 + k] - ref[k] : 0.f;
+                    sums[2 * k] = dv;
+                    sums[2 * k + 1] = dv * dv;
+                }
+                const float mine = warp_sum_many<8>(sums, lane);
+                const float sd = __shfl_sync(0xffffffffu, mine, lane & ~7), sq = __shfl_sync(0xffffffffu, mine, (lane & ~7) + 4);
+                const int k = lane >> 3, j = c0 + s0 + k;
+                if ((lane & 7) == 0 && j < a.rows) {
+                    const float rf = k == 0 ? ref[0] : (k == 1 ? ref[1] : (k == 2 ? ref[2] : ref[3]));
+                    a.e.ln.stats[(size_t)j * a.e.ln.groups + ((seg_base + n_local0 + warp * 32) >> 5)] = make_float2(fmaf(sd, inv, rf), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
+                }
+            }
+        }
+    }
+    tc_fence_before_sync();
+    asm volatile("bar.arrive 2, 160;" ::: "memory");   // the accumulator has been read: warp 5 may free the TMEM columns
+    if (EPI == EPI_SCORE) {                  // two threads share a row
+        bar_sync(1, 128);
+        const int half = tid & 1, r = tid >> 1;
+        if (r >= a.rows) return;             // (the pair of a row's threads leaves together)
+        const float* row = tile_v + r * LD + half;
+        const int t_loc = a.truth[r] - (seg_base + n_local0);
+        float bv = -INFINITY, z = 0.f;
+        int bi = INT_MAX;
+#pragma unroll 8
+        for (int i = 0; i < 64; ++i) if (row[2 * i] > bv) { bv = row[2 * i]; bi = 2 * i + half; }
+        const uint32_t both = 3u << (lane & ~1);
+        const float ov = __shfl_xor_sync(both, bv, 1);
+        const int oi = __shfl_xor_sync(both, bi, 1);
+        if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+#pragma unroll 8
+        for (int i = 0; i < 64; ++i) z += expf(row[2 * i] - bv);
+        z += __shfl_xor_sync(both, z, 1);
+        if (half == 0) {
+            a.amax_val[(size_t)r * a.amax_stride + tile] = bv;
+            a.amax_idx[(size_t)r * a.amax_stride + tile] = bi == INT_MAX ? INT_MAX : seg_base + n_local0 + bi;
+            a.score_sum[(size_t)r * a.amax_stride + tile] = z;
+            if (t_loc >= 0 && t_loc < 128 && n_local0 + t_loc < seg_rows) a.truth_val[r] = tile_v[r * LD + t_loc];
+        }
+    }
+}
+
+// grid: (tiles * splits CTAs in clusters of `splits` (the K-slices of one tile), groups of NB token rows); dynamic smem
+// TcdCfg::SMEM_BYTES.  PASS (all rows of a teacher-forced pass, splits == 1): a.rows counts the rows of all groups; the groups behind
+// the first find the weights in L2.  Bound by the operands' way from L2 into the multiprocessors (33 KB per 64 of K and group of
+// 64 rows), two CTAs on each, one of them in its epilogue.
+template <int NB, int PRO, int EPI, bool PASS = false>
 __global__ void __launch_bounds__(TCD_THREADS)
-gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
+gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
                       const __grid_constant__ CUtensorMap tm2, const __grid_constant__ CUtensorMap tmx,
                       const __grid_constant__ CUtensorMap tml) {
     constexpr bool LNT = PRO == PRO_LNT, BY_TMA = PRO == PRO_TMA || LNT;   // BY_TMA: the token rows are loaded beside the weights
     using C = TcdCfg<NB, LNT>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    TcDecodeArgs group = a0;
+    if (PASS) tcd_shift_rows<PRO, EPI>(group, blockIdx.y * NB, min(NB, a0.rows - (int)blockIdx.y * NB));
+    const TcDecodeArgs& a = PASS ? group : a0;
     __shared__ __align__(8) uint64_t s_full[C::STAGES];
     __shared__ __align__(8) uint64_t s_empty[C::STAGES];
     __shared__ __align__(8) uint64_t s_accum;
@@ -174,7 +333,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     const int rpc = S == 1 ? a.rows : (a.rows + S - 1) / S;
     const int j_first = S == 1 ? 0 : sp * rpc;
     const int j_count = max(0, min(rpc, a.rows - j_first));
-    float hres[EPI == EPI_RESID ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
+    float hres[EPI == EPI_RESID && !PASS ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
     float next_gain = 0.f;                   // EPI_RESID: gain of the LayerNorm that follows, at this thread's feature (a parameter)
     int my_seq = 0, my_pos = 0;              // EPI_QKV / EPI_KV, threads below a.rows: this token row's sequence and position
 
@@ -315,7 +474,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         const int nl = n_local0 + tid;
 #pragma unroll
         for (int s = 0; s < NB; ++s) {
-            if (s >= j_count) break;   // (every loop over rows leaves at the last row: the unrolled rest is never fetched)
+            if (PASS || s >= j_count) break;   // (every loop over rows leaves at the last row: the unrolled rest is never fetched)
             hres[s] = nl < seg_rows ? __ldcg(hp + (size_t)(j_first + s) * a.e.ldo + seg_base + nl) : 0.f;
         }
         if (a.e.ln.gain && tid < j_count) s_mu[tid] = __ldcg(a.e.ln.ref + j_first + tid);   // (published by the barrier ahead of the epilogue)
@@ -498,6 +657,10 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     }
 
     // ---- epilogue: warps 0-3 own TMEM lanes 32 * warp .. +31 = output features of the tile ----
+    if constexpr (PASS) {
+        tcd_pass_epilogue<NB, PRO, EPI>(a, tmem, seg, seg_rows, seg_base, n_local0, tile, ring, s_mu, s_rstd, s_rowoff, &s_accum, next_gain, my_seq, my_pos, poll_limit, nkb > C::STAGES);
+        return;
+    }
     float v[NB];
     const int tl = warp * 32 + lane;
     if (warp < 4) {

@@ -519,7 +519,92 @@ __global__ void __launch_bounds__(VERIFY_THREADS) verify_kernel(LoopState st, in
     }
 }
 
-// Teacher-forced Tandem forward (Eq. 2 over a given sequence): the next gamma tokens of every sequence become the
+// Teacher-forced Tandem forward, bf16: all given tokens are rows of one pass (or of a few, where the work space is short).  The
+// rows lie sequence after sequence, each padded to whole blocks of gamma positions.
+struct ForcedRows {
+    const int* ids;      // the sequences, one after the other
+    const int* off;      // [batch] where each begins in ids
+    const int* len;      // [batch]
+    const int* vstart;   // [batch + 1] first row of each sequence, over all passes
+    int batch, v0, rows; // this pass: rows v0 .. v0 + rows - 1
+    int group;           // queries per attention group of the large model
+    int* row_tok; int* row_seq; int* row_pos;
+    int* truth;          // [rows] the next token (-1: none)
+    int* out;            // [rows] where the row's scores go (-1: nowhere)
+    int* grp_row0; int* grp_cnt;
+};
+
+// Start of one model's part of such a pass: row set-up and embedding (a row past its sequence's end reads token 0; it is
+// computed and ignored), and, with one block more than rows, the attention groups and the sequences' loop state.
+// grid: rows (+ 1); block: 128.
+__global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRows f, const bf16* __restrict__ emb, const bf16* __restrict__ pos,
+                                                          float* __restrict__ h, int d, NextLn ln, int ticket, int router_ticket) {
+    __shared__ float s_red[4];
+    __shared__ int s_cnt[128];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int m = blockIdx.x;
+    if (m == f.rows) {
+        const int b = threadIdx.x;   // (batch <= 128: at least two rows per sequence in every context)
+        int first = 0, n = 0;
+        if (b < f.batch) {
+            first = max(f.vstart[b], f.v0);
+            n = max(0, min(f.vstart[b + 1], f.v0 + f.rows) - first);
+            st.n[b] = f.len[b];
+            st.pending[b] = f.ids[f.off[b] + f.len[b] - 1];
+        }
+        s_cnt[b] = (n + f.group - 1) / f.group;
+        __syncthreads();
+        int g = 0;
+        for (int i = 0; i < b; ++i) g += s_cnt[i];
+        for (int r = 0; r < n; r += f.group, ++g) { f.grp_row0[g] = first - f.v0 + r; f.grp_cnt[g] = min(f.group, n - r); }
+        if (b == 0) { st.counters[6] = ticket; st.counters[8] = router_ticket; }
+        return;
+    }
+    const int v = f.v0 + m;
+    int lo = 0, hi = f.batch - 1;   // the last sequence that begins at or before row v
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (f.vstart[mid] <= v) lo = mid; else hi = mid - 1;
+    }
+    const int p = v - f.vstart[lo], len = f.len[lo], o = f.off[lo];
+    const int tok = p < len ? f.ids[o + p] : 0;
+    if (threadIdx.x == 0) {
+        f.row_tok[m] = tok; f.row_seq[m] = lo; f.row_pos[m] = p;
+        f.truth[m] = p + 1 < len ? f.ids[o + p + 1] : -1;
+        f.out[m] = p + 1 < len ? o - lo + p : -1;
+    }
+    embed_row<bf16, 128, true>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, ln, m, s_red);
+}
+
+// Scores of rows whose output head left (maximum, its index, sum of exponentials) per tile of features and the true token's
+// logit: negative log-likelihood and arg-max (lowest index on ties).  One warp per row; n_tiles values each, 250 at 32000 logits.
+// grid: ceil(rows / 8); block: 256.
+__global__ void __launch_bounds__(256) score_tiles_kernel(int rows, int n_tiles, const float* __restrict__ tile_max, const int* __restrict__ tile_idx,
+                                                          const float* __restrict__ tile_sum, const float* __restrict__ truth_val,
+                                                          const int* __restrict__ out, float* __restrict__ nll, int* __restrict__ top1) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (m >= rows || out[m] < 0) return;
+    const size_t base = (size_t)m * n_tiles;
+    const int top = argmax_from_tiles(tile_max + base, tile_idx + base, n_tiles);
+    float best = -INFINITY;
+    for (int t = lane; t < n_tiles; t += 32) best = fmaxf(best, __ldcg(tile_max + base + t));
+    best = warp_max(best);
+    float tot = 0.f;
+    for (int t = lane; t < n_tiles; t += 32) {
+        const float z = __ldcg(tile_sum + base + t);
+        tot += z > 0.f ? z * expf(__ldcg(tile_max + base + t) - best) : 0.f;
+    }
+    tot = warp_sum(tot);
+    if (lane == 0) {
+        nll[out[m]] = best + logf(tot) - truth_val[m];
+        top1[out[m]] = top;
+    }
+}
+
+// Teacher-forced Tandem forward in rounds (fp32): the next gamma tokens of every sequence become the
 // "drafts" of the round, so that draft step s reads the true token of its position.  forced: [batch][stride] token
 // ids; positions at or beyond forced_len[b] read as token 0 (rows past a sequence's end are computed and ignored).
 // grid: 1; block: 256.

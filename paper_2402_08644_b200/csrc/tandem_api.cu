@@ -50,6 +50,9 @@ struct Layout {   // byte offsets into the arena
     size_t st_n, st_pending, st_drafts, st_targets, st_accept, st_emitted, st_done, st_out, st_counters, st_hist;
     size_t st_block_len, st_drafting, st_confidence;
     size_t forced_ids, forced_len, forced_nll, forced_top;   // teacher-forced forward: given tokens [B][T], lengths [B], scores [B][T]
+    size_t fr_x, fr_o, fr_f, fr_q, fr_yhat, fr_a, fr_t1;
+    size_t fr_seq, fr_truth, fr_out, fr_truth_val, fr_grp, fr_tiles, fr_kv;   // ... in one pass (bf16), see ForcedRows: offsets / lengths / first rows, next tokens, score places,
+                                                                              // true logits, attention groups, the head's per-tile results, the small model's own keys / values of one layer
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
     size_t stage;                                   // a prompt pass's lengths, offsets and token ids as the host staged them
     size_t attn_counters;   // inside the zero-filled state block
@@ -61,6 +64,7 @@ struct Layout {   // byte offsets into the arena
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles;
+    int fr_rows, fr_head_rows;               // rows of a teacher-forced pass, and of one run of its output head
     size_t kv_large_layer, kv_small_layer;   // elements per (layer, k-or-v)
 };
 
@@ -126,10 +130,12 @@ struct tandem_ctx {
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
     std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
-    // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
-    // TMA: maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
-    // 1 small], 16-row boxes; and the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one).
-    CUtensorMap xmap[3][2], lnmap[2];
+    // Activations as two bf16 planes (values, then remainders, `rows` rows each) that the consuming GEMM loads by
+    // TMA: places and maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
+    // 1 small], 16-row boxes; and the place of the queries.  One set for the decode passes, one for teacher-forced passes (in the prompt pass's buffers).
+    struct PlaneSet { size_t at[3], q; int rows; CUtensorMap xmap[3][2]; } dec_planes, fr_planes;
+    const PlaneSet* planes = &dec_planes;   // of the pass that is being enqueued
+    CUtensorMap lnmap[2];                // the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one)
     std::vector<CUtensorMap> kmap, vmap; // the large model's key / value cache of each layer as [(seq, head, position)][d_head]
     cudaStream_t side = nullptr;         // the decode-time FF_Tandem projections run here, beside the large model's later layers
     std::vector<cudaEvent_t> ev_fork;    // one per small layer
@@ -209,7 +215,12 @@ Layout make_layout(const tandem_config& c) {
     const size_t dmax = std::max(std::max(c.large.d_model, c.small.d_model), hidden);
     const size_t fmax = std::max(c.large.d_ff, c.small.d_ff);
     const size_t hmax = std::max(c.large.n_heads, c.small.n_heads);
+    const bool bf = c.dtype == TANDEM_DTYPE_BF16;
     const size_t R = L.max_rows, RD = L.dec_rows, V = c.large.vocab;
+    // Rows of a teacher-forced pass: as many as a prompt pass takes, and the rows that fill its sequences' last blocks.
+    const size_t RF = bf ? std::min<size_t>(R + (size_t)c.max_batch * c.gamma_max, 32768) : 0;
+    L.fr_rows = (int)RF;
+    L.fr_head_rows = (int)std::min<size_t>(RF, 1024);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     L.kv_large_layer = B * T * d_kv_of(c.large);
@@ -221,16 +232,27 @@ Layout make_layout(const tandem_config& c) {
     L.st_done = take(B * 4); L.st_out = take(B * T * 4);
     L.st_counters = take(16 * 4); L.st_hist = take((GL + 1) * 8); L.st_emitted = take(B * 4);   // adjacent: read back together
     L.st_block_len = take(B * 4); L.st_drafting = take(B * 4); L.st_confidence = take(B * GL * 4);
-    L.row_tok = take(R * 4); L.row_seq = take(R * 4); L.row_pos = take(R * 4);
+    const size_t RR = std::max(R, RF);
+    L.row_tok = take(RR * 4); L.row_seq = take(RR * 4); L.row_pos = take(RR * 4);
     L.grp_row0 = take((size_t)L.max_groups * 4); L.grp_cnt = take((size_t)L.max_groups * 4);
     L.stage = take((4 * B + R + B) * 4);
     L.attn_counters = take(B * hmax * 4);
-    L.h_large = take(R * c.large.d_model * 4);
+    L.h_large = take(std::max(R * c.large.d_model, RF * std::max(c.large.d_model, c.small.d_model)) * 4);
     L.h_small = take(B * c.small.d_model * 4);
+    const size_t ws = off;
     L.a = take(R * dmax * esz); L.q = take(R * dmax * esz); L.o = take(R * dmax * esz);
     L.f = take(R * fmax * esz);
     L.xb = take(R * c.large.d_model * esz); L.t1 = take(R * hidden * esz);
     L.yhat = take(R * c.small.d_model * 4); L.a_s = take(R * c.small.d_model * esz);
+    // The same space in a teacher-forced pass, whose rows are fp32 or two bf16 planes.  The queries and the projections' buffers
+    // share the place of the GELU outputs, which are dead from the end of a layer to the first product of the next one's FFN.
+    const size_t ws_end = off;
+    off = ws;
+    L.fr_x = take(RF * dmax * 4); L.fr_o = take(RF * dmax * 4); L.fr_f = off;
+    L.fr_q = take(RF * dmax * 2);
+    off = L.fr_f;
+    L.fr_yhat = take(RF * c.small.d_model * 4); L.fr_a = take(RF * c.small.d_model * 4); L.fr_t1 = take(RF * hidden * 4);
+    off = std::max(std::max(off, align_up(L.fr_f + std::max(RF * dmax * 2, RF * fmax * 4))), ws_end);
     L.logits_large = take(RD * V * 4);
     L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.part_ml = take(RD * hmax * L.n_chunks_max * 2 * 4);
@@ -250,8 +272,12 @@ Layout make_layout(const tandem_config& c) {
     L.ln_src = take((size_t)(2 * c.large.n_layers + 1 + 2 * c.small.n_layers + 1) * sizeof(LnSource));
     L.ln_rows_large = take((size_t)(2 * c.large.n_layers + 1) * 4 * c.large.d_model * 2);
     L.ln_rows_small = take((size_t)(2 * c.small.n_layers + 1) * 4 * c.small.d_model * 2);
-    L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
-    L.ln_ref = take(2 * RD * 4);
+    L.ln_stats = take(std::max(RD, RF) * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
+    L.ln_ref = take(2 * std::max(RD, RF) * 4);
+    L.fr_seq = take((3 * B + 1) * 4); L.fr_truth = take(RF * 4); L.fr_out = take(RF * 4); L.fr_truth_val = take(RF * 4);
+    L.fr_grp = take(2 * (RF / ATT_NQ + B + 1) * 4);
+    L.fr_tiles = take((size_t)L.fr_head_rows * L.vocab_tiles * 12);
+    L.fr_kv = take(bf ? 2 * L.kv_small_layer * esz : 0);
     L.total = off;
     return L;
 }
@@ -372,6 +398,7 @@ struct TcScratch {
     unsigned poll_limit = 0;   // 0: the kernels' default
     int withhold_weights = 0;  // test hook, see TcDecodeArgs
     int wait_first = 0;        // the launch may follow kernels that write its weights, see TcDecodeArgs
+    bool whole_pass = false;   // all rows of a pass at once, not a block that has to give the bits of its rows alone: K-slices by the number of rows
 };
 
 TcW tcw3(const tandem_ctx& c, int i0, int i1, int i2, int seg_rows0, int seg_rows, int K) {
@@ -423,6 +450,7 @@ void launch_ex(tandem_ctx& c, bool pdl, int cluster, void (*kernel)(KArgs...), d
 struct TcRows {
     const CUtensorMap* map = nullptr;
     int plane_rows = 0;                    // rows between the value and the remainder plane
+    int row0 = 0;                          // the pass's first row there
     const CUtensorMap* ln_map = nullptr;
     int ln_row = 0;                        // the LayerNorm's first row there
     const float2* ln_stats = nullptr;      // [rows][ln_groups]
@@ -431,71 +459,82 @@ struct TcRows {
     float* ln_mean = nullptr;
 };
 
-template <int NB, int PRO, int EPI>
-void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const TcRows& x) {
+template <int NB, int PRO, int EPI, bool PASS = false>
+void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const TcRows& x, int groups = 1) {
     using C = TcdCfg<NB, PRO == PRO_LNT>;
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_tc_decode_kernel<NB, PRO, EPI>, C::SMEM_BYTES, attr_done);
-    launch_ex(c, true, a.splits, gemm_tc_decode_kernel<NB, PRO, EPI>, dim3(units), dim3(TCD_THREADS), (size_t)C::SMEM_BYTES, a, w.tm[0], w.tm[1], w.tm[2],
+    ensure_dyn_smem(gemm_tc_decode_kernel<NB, PRO, EPI, PASS>, C::SMEM_BYTES, attr_done);
+    const size_t smem = PASS ? C::SMEM_BYTES_WHOLE : C::SMEM_BYTES;
+    launch_ex(c, true, a.splits, gemm_tc_decode_kernel<NB, PRO, EPI, PASS>, dim3(units, groups), dim3(TCD_THREADS), smem, a, w.tm[0], w.tm[1], w.tm[2],
               x.map ? *x.map : w.tm[0], x.ln_map ? *x.ln_map : w.tm[0]);
 }
 
+// What the output head leaves per row and tile instead of (or beside) the logits, and the teacher-forced scores' part of it.
+struct TcTiles {
+    float* val = nullptr;
+    int* idx = nullptr;
+    int stride = 0;
+    float* sum = nullptr;          // EPI_SCORE
+    const int* truth = nullptr;
+    float* truth_val = nullptr;
+};
+
 // y = prologue(x) W^T for few rows on the tensor cores, streaming W once per group of up to 64 rows (one group in
-// every benchmark configuration; more rows than that re-read the weights per group, with unchanged arithmetic).
+// every benchmark configuration; more rows than that re-read the weights per group, from L2, with unchanged arithmetic).
 template <int PRO, int EPI>
 void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx, const void* ln_g, const void* ln_b, int rows,
-                      const TcW& w, bool stream_weights, const EpiArgs& e, float* amax_val = nullptr, int* amax_idx = nullptr,
-                      int amax_stride = 0, const TcRows& xr = TcRows()) {
+                      const TcW& w, bool stream_weights, const EpiArgs& e, const TcTiles& t = TcTiles(), const TcRows& xr = TcRows()) {
     if (rows <= 0) return;
     TcDecodeArgs a;
     memset(&a, 0, sizeof(a));
-    a.ldx = ldx; a.ln_g = static_cast<const float*>(ln_g); a.ln_b = static_cast<const float*>(ln_b);
+    a.x = x; a.ldx = ldx; a.ln_g = static_cast<const float*>(ln_g); a.ln_b = static_cast<const float*>(ln_b);
+    a.rows = rows; a.x_row0 = xr.row0; a.x_plane_rows = xr.plane_rows;
+    a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups; a.ln_stats = xr.ln_stats; a.ln_ref = xr.ln_ref; a.ln_mean = xr.ln_mean;
     a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.tiles0 = cdiv(w.seg_rows0, 128);
     a.seg_rows = w.seg_rows; a.tiles_per_seg = cdiv(w.seg_rows, 128);
     const int tiles = a.tiles0 + (w.n_segs - 1) * a.tiles_per_seg, KB = cdiv(w.K, 64);
+    const bool whole = EPI == EPI_SCORE || (sc.whole_pass && rows > 64);
     // K-slices per tile = cluster size: the smallest power of two that puts tiles * S CTAs at or above one per
     // multiprocessor, at most 8 and at most one per 64-element K-block; four instead of eight where those already reach a
     // quarter of the multiprocessors with slices of four K-blocks or fewer (they fit the ring, and only 15 clusters of
     // eight run beside each other before two CTAs share a multiprocessor, but 33 of four).  A layer's four GEMMs with four
     // slices in both wide ones against eight: 1024 wide, one row 12.5 -> 11.9 us, eight rows 13.9 -> 13.1; 512 wide 9.9 -> 9.5 and
     // 11.8 -> 11.4.  The residual GEMMs (a quarter of the tiles or a slice beyond the ring) are 2 to 10 % slower with four.
-    // The head GEMM keeps whole tiles.
+    // The head GEMM keeps whole tiles, and so does a whole pass, which has a CTA per tile and 64 rows.
     int S = 1;
-    if (EPI != EPI_ARGMAX)
+    if (EPI != EPI_ARGMAX && !whole)
         while (S < 8 && 2 * S <= KB && tiles * S < c.n_sms && !(S == 4 && KB <= 16 && 16 * tiles >= c.n_sms)) S *= 2;
     a.splits = S;
-    a.stream_weights = stream_weights ? 1 : 0;
+    a.stream_weights = stream_weights && !whole ? 1 : 0;
     a.err_flag = sc.err;
     a.poll_limit = sc.poll_limit;
     a.withhold_weights = sc.withhold_weights;
-    a.amax_stride = amax_stride;
-    const size_t xsz = PRO == PRO_BF16 ? 2 : 4;
-    const size_t osz = EPI == EPI_STORE ? 2 : 4;       // EPI_QKV: the query buffer is bf16 too (below)
+    a.wait_first = sc.wait_first;
+    a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
+    a.amax_val = t.val; a.amax_idx = t.idx; a.amax_stride = t.stride;
+    a.score_sum = t.sum; a.truth = t.truth; a.truth_val = t.truth_val;
+    a.e = e;
+    const double xsz = PRO == PRO_BF16 ? 2 : 4, osz = EPI == EPI_QKV || EPI == EPI_KV || EPI == EPI_STORE ? 2.0 : 4.0;
     const int units = tiles * S;
-    for (int r0 = 0; r0 < rows; r0 += 64) {
-        const int nr = std::min(64, rows - r0);
-        a.rows = nr;
-        a.x_row0 = r0; a.x_plane_rows = xr.plane_rows;
-        a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups;
-        a.ln_stats = xr.ln_stats ? xr.ln_stats + (size_t)r0 * xr.ln_groups : nullptr;
-        a.ln_ref = xr.ln_ref ? xr.ln_ref + r0 : nullptr;
-        a.ln_mean = xr.ln_mean ? xr.ln_mean + r0 : nullptr;
-        a.wait_first = r0 == 0 ? sc.wait_first : 0;
-        a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
-        a.x = static_cast<const unsigned char*>(x) + (size_t)r0 * ldx * xsz;
-        a.amax_val = amax_val ? amax_val + (size_t)r0 * amax_stride : nullptr;
-        a.amax_idx = amax_idx ? amax_idx + (size_t)r0 * amax_stride : nullptr;
-        a.e = e;
-        if (e.out) a.e.out = static_cast<unsigned char*>(e.out) + (size_t)r0 * e.ldo * ((EPI == EPI_QKV || e.out_lo) ? 2 : osz);
-        if (e.out_lo) a.e.out_lo = static_cast<unsigned char*>(e.out_lo) + (size_t)r0 * e.ldo * 2;   // (value / remainder planes are bf16)
-        if (e.row_seq) { a.e.row_seq = e.row_seq + r0; a.e.row_pos = e.row_pos + r0; }
-        if (e.snap) a.e.snap = static_cast<float*>(e.snap) + (size_t)r0 * e.snap_ld;
-        if (e.ln.gain) { a.e.ln.hi = e.ln.hi + (size_t)r0 * e.ldo; a.e.ln.lo = e.ln.lo + (size_t)r0 * e.ldo; a.e.ln.stats = e.ln.stats + (size_t)r0 * e.ln.groups; a.e.ln.ref = e.ln.ref + r0; }
-        ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + (double)nr * w.K * xsz + (double)nr * a.N * (EPI == EPI_QKV || EPI == EPI_KV || EPI == EPI_STORE ? 2.0 : 4.0));
-        if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, a, w, units, xr);
-        else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, a, w, units, xr);
-        else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, a, w, units, xr);
-        else launch_tc_decode_nb<64, PRO, EPI>(c, a, w, units, xr);
+    if constexpr (EPI == EPI_SCORE || (PRO != PRO_BF16 && PRO != PRO_LN && EPI != EPI_ARGMAX)) {
+        if (whole) {
+            ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K * cdiv(rows, 64) + rows * (w.K * xsz + a.N * osz));
+            launch_tc_decode_nb<64, PRO, EPI, true>(c, a, w, units, xr, cdiv(rows, 64));
+            return;
+        }
+    }
+    if constexpr (EPI != EPI_SCORE) {
+        for (int r0 = 0; r0 < rows; r0 += 64) {
+            const int nr = std::min(64, rows - r0);
+            TcDecodeArgs g = a;
+            tcd_shift_rows<PRO, EPI>(g, r0, nr);
+            if (r0 > 0) g.wait_first = 0;
+            ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + nr * (w.K * xsz + a.N * osz));
+            if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, g, w, units, xr);
+            else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, g, w, units, xr);
+            else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, g, w, units, xr);
+            else launch_tc_decode_nb<64, PRO, EPI>(c, g, w, units, xr);
+        }
     }
 }
 
@@ -630,12 +669,13 @@ void launch_attn_decode_as(tandem_ctx& c, const AttnArgs& a, dim3 grid) {
     launch_ex(c, true, (int)grid.x, attn_decode_kernel<DH, NT, MODE>, grid, dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
 }
 template <int DH>
-void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl, double kv_bytes) {
+void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl, bool pass, double kv_bytes) {
     const int gpc = std::max(1, a.heads_per_cta);
     const bool narrow = gpc * a.nq <= 8;
     const dim3 grid(cl, a.n_heads / gpc, groups);
     ProfScope ps(c, PC_ATTN_SPLIT, kv_bytes);
-    if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid); }
+    if (pass) { if (narrow) launch_attn_decode_as<DH, 1, ATD_PASS>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_PASS>(c, a, grid); }
+    else if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid); }
     else if (narrow) launch_attn_decode_as<DH, 1, ATD_CLUSTERED>(c, a, grid);
     else launch_attn_decode_as<DH, 2, ATD_CLUSTERED>(c, a, grid);
 }
@@ -679,7 +719,8 @@ int attn_cluster_size(long long clusters, int d_head) {
     }
     return best;
 }
-void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int groups, double kv_bytes) {
+// pass: a teacher-forced pass, which has a CTA per group of rows and head.
+void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int groups, double kv_bytes, bool pass = false) {
     AttnArgs a = a0;
     // Grouped-query attention: the query heads of one key/value head ride in one CTA as far as the 16-row tile has
     // room (heads * queries per block <= 16; a power of two that divides the group).  The cluster size is taken
@@ -690,10 +731,10 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     int gpc = 1;
     while (gpc * 2 <= group && group % (gpc * 2) == 0 && gpc * 2 * a.nq <= ATT_NQ) gpc *= 2;
     a.heads_per_cta = gpc;
-    const int cl = attn_cluster_size((long long)groups * n_kv, d_head);
-    if (d_head == 32) launch_attn_decode_dq<32>(c, a, groups, cl, kv_bytes);
-    else if (d_head == 64) launch_attn_decode_dq<64>(c, a, groups, cl, kv_bytes);
-    else launch_attn_decode_dq<128>(c, a, groups, cl, kv_bytes);
+    const int cl = pass ? 1 : attn_cluster_size((long long)groups * n_kv, d_head);
+    if (d_head == 32) launch_attn_decode_dq<32>(c, a, groups, cl, pass, kv_bytes);
+    else if (d_head == 64) launch_attn_decode_dq<64>(c, a, groups, cl, pass, kv_bytes);
+    else launch_attn_decode_dq<128>(c, a, groups, cl, pass, kv_bytes);
 }
 
 // raw (bf16 only, nullable): also leaves a bf16 copy of the rows as they are.
@@ -712,6 +753,9 @@ struct Rows {
     bool decode;      // decode kernels (split attention, streaming GEMM) or prompt kernels
     int n_chunks;     // split attention grid size along the context
     double kv_positions;   // context positions read by one attention launch, summed over sequences (accounting only)
+    bool whole_pass = false;            // a teacher-forced pass (see forced_pass)
+    const int *grp_row0 = nullptr, *grp_cnt = nullptr;   // ... its attention groups of unequal length, else groups of nq rows
+    bf16 *own_k = nullptr, *own_v = nullptr;             // ... the small model's keys / values of its own, beside the large-derived ones in the cache
 };
 
 template <typename T>
@@ -787,7 +831,9 @@ void attention_decode(tandem_ctx& c, const Model& m, int l, const bf16* q, bf16*
     aa.out = o; aa.out_lo = o_lo; aa.ldo = d; aa.row_seq = at<int>(c, c.lay.row_seq); aa.row_pos = at<int>(c, c.lay.row_pos);
     aa.nq = r.nq; aa.n_heads = H; aa.n_kv_heads = m.kv_heads; aa.t_max = c.cfg.max_seq; aa.scale = 1.0f / sqrtf((float)dh);
     aa.err_flag = tc_scratch(c).err;
-    launch_attn_decode(c, dh, aa, r.groups, r.kv_positions * 2.0 * d * 2.0);
+    if (r.grp_cnt) { aa.grp_row0 = r.grp_row0; aa.grp_cnt = r.grp_cnt; aa.wait_first = 1; }   // (a group's earlier positions may be rows of this very pass)
+    if (r.own_k) { aa.k2 = r.own_k; aa.v2 = r.own_v; }
+    launch_attn_decode(c, dh, aa, r.groups, r.kv_positions * 2.0 * d * 2.0, r.whole_pass);
 }
 
 // The fp32 passes whose maps run on the few-row kernel with LayerNorm fused into it: decode passes and short prompts.
@@ -948,7 +994,7 @@ void fp32_large_block(tandem_ctx& c, int nq, bool project, bool head) {
     if (head) head_argmax(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.st.targets, TANDEM_GAMMA_LIMIT + 1, 0);
 }
 
-// Teacher-forced round (accept mode 5): the given tokens become the round's drafts; after the draft steps their
+// Teacher-forced round (accept mode 5, fp32): the given tokens become the round's drafts; after the draft steps their
 // logits are scored against the given next tokens.
 void launch_forced_fill(tandem_ctx& c, int gamma) {
     ProfScope ps(c, PC_ROWS, (double)c.batch * gamma * 8.0);
@@ -1034,18 +1080,18 @@ void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
 // bf16 decode on the tensor cores: five kernels per decoder layer, chained by programmatic dependent launch
 // ---------------------------------------------------------------------------------------------------
 
-// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = residual stream, less c, times the next
+// The decode activations' value / remainder planes (see tandem_ctx::PlaneSet): buffer 0 = residual stream, less c, times the next
 // LayerNorm's gain, 1 = attention output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width
 // for buffer 2).
 struct XPlanes { bf16* hi; bf16* lo; TcRows rows; };
 XPlanes x_planes(tandem_ctx& c, int buf, const Model& m) {
-    const size_t off = buf == 0 ? c.lay.a32 : (buf == 1 ? c.lay.o32 : c.lay.f32);
+    const tandem_ctx::PlaneSet& ps = *c.planes;
     const size_t K = buf == 2 ? m.d.d_ff : m.d.d_model;
     XPlanes p;
-    p.hi = at<bf16>(c, off);
-    p.lo = p.hi + (size_t)c.lay.dec_rows * K;
-    p.rows.map = &c.xmap[buf][&m == &c.large ? 0 : 1];
-    p.rows.plane_rows = c.lay.dec_rows;
+    p.hi = at<bf16>(c, ps.at[buf]);
+    p.lo = p.hi + (size_t)ps.rows * K;
+    p.rows.map = &ps.xmap[buf][&m == &c.large ? 0 : 1];
+    p.rows.plane_rows = ps.rows;
     return p;
 }
 
@@ -1056,7 +1102,7 @@ const void* ln_gain(const tandem_ctx& c, const Model& m, int idx) {
 }
 // The value taken off each row before LayerNorm `idx` (NextLn::ref).  Two arrays in turn: the GEMM behind a LayerNorm reads its
 // own from one and leaves the rows' means, the next LayerNorm's, in the other.
-float* ln_ref_of(tandem_ctx& c, int idx) { return at<float>(c, c.lay.ln_ref) + (size_t)(idx & 1) * c.lay.dec_rows; }
+float* ln_ref_of(tandem_ctx& c, int idx) { return at<float>(c, c.lay.ln_ref) + (size_t)(idx & 1) * c.planes->rows; }
 NextLn next_ln(tandem_ctx& c, const Model& m, int idx) {
     const XPlanes p = x_planes(c, 0, m);
     return {static_cast<const float*>(ln_gain(c, m, idx)), p.hi, p.lo, at<float2>(c, c.lay.ln_stats), cdiv(m.d.d_model, 32), ln_ref_of(c, idx)};
@@ -1081,34 +1127,38 @@ bool tc_fused_prologue(const tandem_ctx& c, int K) { return c.batch <= 2 && K <=
 // planes; only the queries and the cached keys / values are bf16.
 void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool stream_w, float* snap = nullptr) {
     const int d = m.d.d_model, dff = m.d.d_ff;
-    bf16* q = at<bf16>(c, c.lay.q);
-    const TcScratch sc = tc_scratch(c);
+    bf16* q = at<bf16>(c, c.planes->q);
+    TcScratch sc = tc_scratch(c);
+    sc.whole_pass = r.whole_pass;
     const XPlanes xo = x_planes(c, 1, m), xf = x_planes(c, 2, m);
+    EpiArgs eq = epi_cache<bf16>(c, m, l, q);
+    if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; }
     launch_tc_decode<PRO_LNT, EPI_QKV>(c, sc, nullptr, d, nullptr, nullptr, r.M,
                                        tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w,
-                                       epi_cache<bf16>(c, m, l, q), nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l));
+                                       eq, TcTiles(), ln_rows_of(c, m, 2 * l));
     attention_decode(c, m, l, q, xo.hi, xo.lo, r);
     EpiArgs eo = epi_plain(h, d);
     eo.ln = next_ln(c, m, 2 * l + 1);
     launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w, eo,
-                                         nullptr, nullptr, 0, xo.rows);
+                                         TcTiles(), xo.rows);
     EpiArgs e1 = epi_plain(xf.hi, dff);
     e1.out_lo = xf.lo;
     launch_tc_decode<PRO_LNT, EPI_GELU>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), stream_w, e1,
-                                        nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l + 1));
+                                        TcTiles(), ln_rows_of(c, m, 2 * l + 1));
     EpiArgs e2 = epi_plain(h, d);
     e2.snap = snap; e2.snap_ld = d;   // copy of x^(l+1) when an FF_Tandem projection reads it
     e2.ln = next_ln(c, m, 2 * l + 2);
     launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, dff, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), stream_w, e2,
-                                         nullptr, nullptr, 0, xf.rows);
+                                         TcTiles(), xf.rows);
 }
 
 // Final LayerNorm + output head; leaves fp32 logits and the per-tile (max, index) pairs that the next kernel
 // (the next pass's row set-up, or the verify kernel) turns into token ids.
 void tc_head(tandem_ctx& c, const Model& m, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool stream_w) {
+    TcTiles t;
+    t.val = at<float>(c, amax_val_off); t.idx = at<int>(c, amax_idx_off); t.stride = c.lay.vocab_tiles;
     launch_tc_decode<PRO_LNT, EPI_ARGMAX>(c, tc_scratch(c), nullptr, m.d.d_model, nullptr, nullptr, r.M, tcw(c, wi_tail(m, 2), -1, -1, m.d.vocab, m.d.d_model),
-                                          stream_w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.lay.vocab_tiles,
-                                          ln_rows_of(c, m, 2 * m.d.n_layers));
+                                          stream_w, epi_plain(logits, m.d.vocab), t, ln_rows_of(c, m, 2 * m.d.n_layers));
 }
 
 // sampled: the previous draft was drawn by sample_draft_kernel (it is in the loop state already), not left as per-tile
@@ -1122,45 +1172,48 @@ void tc_small_step(tandem_ctx& c, int s, bool sampled) {
     tc_head(c, c.small, r, logits, c.lay.amax_val_small, c.lay.amax_idx_small, false);
 }
 
-// FF_Tandem of the block's rows after n large layers (Eq. 2, first line) for every small layer fed from there, then
-// that layer's LayerNorm and key/value maps with the cache write as the GEMM epilogue.  It runs on the side stream,
-// from the copy `snap` of x^(l(j)) that the producing kernel left: it depends on nothing the large model does
-// afterwards (and nothing in the iteration depends on it before the next draft), so it runs beside the large model's
+// FF_Tandem of decode rows x (fp32, [r.M][d_large], the residual stream after layer_map[j] large layers; Eq. 2, first line) for small layer
+// j, then that layer's LayerNorm and key/value maps with the cache write as the GEMM epilogue.  yhat, a_j, t1: fp32 rows.
+void tc_project(tandem_ctx& c, int j, const float* x, const Rows& r, float* yhat, float* a_j, float* t1) {
+    const int dL = c.large.d.d_model, dS = c.small.d.d_model;
+    TcScratch sc = tc_scratch(c);
+    sc.whole_pass = r.whole_pass;
+    if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
+        launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, x, dL, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), true,
+                                                 epi_plain(yhat, dS));
+    } else {
+        launch_tc_decode<PRO_F32, EPI_GELU>(c, sc, x, dL, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), true,
+                                            epi_plain(t1, c.hidden));
+        launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, t1, c.hidden, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden),
+                                                 true, epi_plain(yhat, dS));
+    }
+    const void *lg = w_layer(c, c.small, j, W_LN1G), *lb = w_layer(c, c.small, j, W_LN1B);
+    const TcW wkv = tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS);
+    const EpiArgs ekv = epi_cache<bf16>(c, c.small, j, nullptr);
+    if (!r.whole_pass && tc_fused_prologue(c, dS)) {
+        launch_tc_decode<PRO_LN, EPI_KV>(c, sc, yhat, dS, lg, lb, r.M, wkv, true, ekv);
+    } else {
+        launch_layernorm<float>(c, r.M, yhat, lg, lb, a_j, dS);
+        launch_tc_decode<PRO_F32, EPI_KV>(c, sc, a_j, dS, nullptr, nullptr, r.M, wkv, true, ekv);
+    }
+}
+
+// The projections of a decode pass after n large layers.  They run on the side stream,
+// from the copy `snap` of x^(l(j)) that the producing kernel left: they depend on nothing the large model does
+// afterwards (and nothing in the iteration depends on them before the next draft), so they run beside the large model's
 // later layers instead of in their chain.
 void tc_project_forked(tandem_ctx& c, int n_large_layers_done, int slot, const Rows& r) {
-    const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    const TcScratch sc = tc_scratch(c);
-    const size_t RD = (size_t)c.lay.dec_rows;
-    const float* snap = at<float>(c, c.lay.proj_snap) + (size_t)slot * RD * dL;
+    const size_t RD = (size_t)c.lay.dec_rows, dS = c.small.d.d_model;
+    const float* snap = at<float>(c, c.lay.proj_snap) + (size_t)slot * RD * c.large.d.d_model;
     cudaStream_t main_stream = c.stream;
     cudaEventRecord(c.ev_fork[slot], main_stream);
     cudaStreamWaitEvent(c.side, c.ev_fork[slot], 0);
     c.stream = c.side;
     c.next_launch_plain = true;   // first kernel after a cross-stream wait
-    for (int j = 0; j < c.small.d.n_layers; ++j) {
-        if (c.layer_map[j] != n_large_layers_done) continue;
-        float* yhat = at<float>(c, c.lay.proj_yhat) + (size_t)j * RD * dS;
-        float* a_j = at<float>(c, c.lay.proj_a) + (size_t)j * RD * dS;
-        if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
-            launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, snap, dL, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), true,
-                                                     epi_plain(yhat, dS));
-        } else {
-            float* t1 = at<float>(c, c.lay.proj_t1) + (size_t)j * RD * c.hidden;
-            launch_tc_decode<PRO_F32, EPI_GELU>(c, sc, snap, dL, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), true,
-                                                epi_plain(t1, c.hidden));
-            launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, t1, c.hidden, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden),
-                                                     true, epi_plain(yhat, dS));
-        }
-        const void *lg = w_layer(c, c.small, j, W_LN1G), *lb = w_layer(c, c.small, j, W_LN1B);
-        const TcW wkv = tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS);
-        const EpiArgs ekv = epi_cache<bf16>(c, c.small, j, nullptr);
-        if (tc_fused_prologue(c, dS)) {
-            launch_tc_decode<PRO_LN, EPI_KV>(c, sc, yhat, dS, lg, lb, r.M, wkv, true, ekv);
-        } else {
-            launch_layernorm<float>(c, r.M, yhat, lg, lb, a_j, dS);
-            launch_tc_decode<PRO_F32, EPI_KV>(c, sc, a_j, dS, nullptr, nullptr, r.M, wkv, true, ekv);
-        }
-    }
+    for (int j = 0; j < c.small.d.n_layers; ++j)
+        if (c.layer_map[j] == n_large_layers_done)
+            tc_project(c, j, snap, r, at<float>(c, c.lay.proj_yhat) + (size_t)j * RD * dS, at<float>(c, c.lay.proj_a) + (size_t)j * RD * dS,
+                       at<float>(c, c.lay.proj_t1) + (size_t)j * RD * c.hidden);
     c.stream = main_stream;
 }
 
@@ -1196,19 +1249,58 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
     }
 }
 
-void tc_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
-    const bool sampled = mode == 4, forced = mode == 5;
-    if (forced) launch_forced_fill(c, gamma);
-    for (int s = 0; s < gamma; ++s) {
-        tc_small_step(c, s, sampled || forced);   // (both find their drafts in the loop state, not in per-tile arg-max results)
-        if (sampled) launch_sample_draft(c, s, seed);
+// The rows f of a teacher-forced forward (all of whole blocks) through both models.  The large model reads them as one causal pass
+// and its projections go to the small model's cache; then the small model reads all blocks at once, since the tokens it would draft
+// are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie in
+// a cache of their own for the time of one layer.  Every row has the arithmetic of the decode passes (activations as value + remainder).
+// Four sequences of 129-257 tokens through the small pair took one round per block, gamma small passes and one large each, 35.8 ms;
+// 2.0 ms like this.
+void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large, double kv_positions) {
+    const Model &L = c.large, &S = c.small;
+    c.planes = &c.fr_planes;
+    Rows r;
+    r.M = f.rows; r.decode = true; r.whole_pass = true; r.n_chunks = 1; r.kv_positions = kv_positions;
+    auto begin = [&](const Model& m, float* h, bool setup) {
+        ProfScope ps(c, PC_ROWS, (double)f.rows * m.d.d_model * 8.0);
+        launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + (setup ? 1 : 0)), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
+                  (int)m.d.d_model, next_ln(c, m, 0), (int)c.ticket, (int)c.router_ticket);
+    };
+    float* h = at<float>(c, c.lay.h_large);
+    float *yhat = at<float>(c, c.lay.fr_yhat), *a_j = at<float>(c, c.lay.fr_a), *t1 = at<float>(c, c.lay.fr_t1);
+    r.nq = ATT_NQ; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
+    begin(L, h, true);
+    for (int l = 0; l <= L.d.n_layers; ++l) {
+        for (int j = 0; j < S.d.n_layers; ++j)
+            if (c.layer_map[j] == l) tc_project(c, j, h, r, yhat, a_j, t1);
+        if (l < L.d.n_layers) tc_decoder_layer(c, L, l, h, r, true);
     }
-    if (forced) {   // teacher-forced round: score the logits, then a representation-only block whose drafts are the given tokens
-        launch_score_rows(c, gamma);
-        tc_large_block(c, gamma, -1, true, false);
-        launch_verify(c, gamma, 3, seed, max_new, false);
-        c.last_gamma = gamma;
-        return;
+    float* y = h;   // (the large model's residual stream has been read for the last time)
+    r.nq = gamma; r.groups = f.rows / gamma; r.grp_row0 = r.grp_cnt = nullptr;
+    r.own_k = at<bf16>(c, c.lay.fr_kv); r.own_v = r.own_k + c.lay.kv_small_layer;
+    begin(S, y, false);
+    for (int j = 0; j < S.d.n_layers; ++j) tc_decoder_layer(c, S, j, y, r, true);
+    for (int r0 = 0; r0 < f.rows; r0 += c.lay.fr_head_rows) {
+        const int rows = std::min(c.lay.fr_head_rows, f.rows - r0), tiles = c.lay.vocab_tiles;
+        TcTiles t;
+        t.val = at<float>(c, c.lay.fr_tiles); t.idx = reinterpret_cast<int*>(t.val + (size_t)rows * tiles); t.stride = tiles;
+        t.sum = t.val + (size_t)2 * rows * tiles;
+        t.truth = f.truth + r0; t.truth_val = at<float>(c, c.lay.fr_truth_val);
+        TcRows x = ln_rows_of(c, S, 2 * S.d.n_layers);
+        x.row0 = r0; x.ln_stats += (size_t)r0 * x.ln_groups; x.ln_ref += r0; x.ln_mean += r0;
+        launch_tc_decode<PRO_LNT, EPI_SCORE>(c, tc_scratch(c), nullptr, S.d.d_model, nullptr, nullptr, rows, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, S.d.d_model),
+                                             false, epi_plain(nullptr, S.d.vocab), t, x);
+        ProfScope ps(c, PC_ARGMAX, 12.0 * rows * tiles);
+        launch_ex(c, true, 1, score_tiles_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, rows, tiles, (const float*)t.val, (const int*)t.idx, (const float*)t.sum,
+                  (const float*)t.truth_val, (const int*)(f.out + r0), at<float>(c, c.lay.forced_nll), at<int>(c, c.lay.forced_top));
+    }
+    c.planes = &c.dec_planes;
+}
+
+void tc_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
+    const bool sampled = mode == 4;
+    for (int s = 0; s < gamma; ++s) {
+        tc_small_step(c, s, sampled);   // (the sampled drafts are found in the loop state, not in per-tile arg-max results)
+        if (sampled) launch_sample_draft(c, s, seed);
     }
     if (mode == 3) tc_large_block(c, gamma, -1, true, false);   // gamma rows, no head: the last draft is finished by the verify kernel
     else tc_large_block(c, gamma + 1, (gamma > 0 && !sampled) ? gamma : -1, true, true);
@@ -1414,10 +1506,12 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->small.kv_heads = kv_heads_of(cfg->small); c->small.d_kv = d_kv_of(cfg->small);
     c->large.d = cfg->large; c->large.wbase = 0; c->large.kv_off = lay.kv_large; c->large.kv_layer_elems = lay.kv_large_layer;
     c->small.d = cfg->small; c->small.wbase = 5 + 10 * cfg->large.n_layers; c->small.kv_off = lay.kv_small; c->small.kv_layer_elems = lay.kv_small_layer;
+    c->dec_planes.at[0] = lay.a32; c->dec_planes.at[1] = lay.o32; c->dec_planes.at[2] = lay.f32; c->dec_planes.q = lay.q; c->dec_planes.rows = lay.dec_rows;
+    c->fr_planes.at[0] = lay.fr_x; c->fr_planes.at[1] = lay.fr_o; c->fr_planes.at[2] = lay.fr_f; c->fr_planes.q = lay.fr_q; c->fr_planes.rows = lay.fr_rows;
     c->tbase = c->small.wbase + 5 + 10 * cfg->small.n_layers;
     c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0;
     c->pinned_ints = std::max((size_t)lay.max_rows + 5 * cfg->max_batch + 64,
-                              (size_t)cfg->max_batch * (cfg->max_seq + 1) + 2 * 64 + 64);   // prompt rows going in; tokens, counters, histogram, lengths coming out
+                              (size_t)cfg->max_batch * (2 * cfg->max_seq + 4) + 2 * 64 + 64);   // prompt rows going in; tokens, counters, histogram, lengths, scores coming out
     c->pinned = nullptr;
     LoopState& st = c->st;
     st.n = at<int>(*c, lay.st_n); st.pending = at<int>(*c, lay.st_pending); st.drafts = at<int>(*c, lay.st_drafts);
@@ -1472,11 +1566,11 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
         }
         for (int mi = 0; mi < 2; ++mi) {   // decode activations and the LayerNorms' rows
             const Model& mm = mi == 0 ? c->large : c->small;
-            for (int buf = 0; buf < 3; ++buf) {
-                const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
-                const size_t at_off = buf == 0 ? lay.a32 : (buf == 1 ? lay.o32 : lay.f32);
-                ok = ok && make_tmap_bf16(&c->xmap[buf][mi], c->arena + at_off, 2 * (uint64_t)lay.dec_rows, K, K, 16);
-            }
+            for (tandem_ctx::PlaneSet* ps : {&c->dec_planes, &c->fr_planes})
+                for (int buf = 0; buf < 3; ++buf) {
+                    const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
+                    ok = ok && make_tmap_bf16(&ps->xmap[buf][mi], c->arena + ps->at[buf], 2 * (uint64_t)ps->rows, K, K, 16);
+                }
             const uint64_t d = mm.d.d_model, n_ln = 2 * mm.d.n_layers + 1;
             ok = ok && make_tmap_bf16(&c->lnmap[mi], c->arena + (mi == 0 ? lay.ln_rows_large : lay.ln_rows_small), 4 * n_ln, d, d, 4);
         }
@@ -1908,6 +2002,64 @@ extern "C" tandem_status tandem_speculative_generate(tandem_ctx* c, int32_t gamm
     return run_generate(c, true, gamma, max_new_tokens, accept_mode, mode_seed, out_ids, out_lens, stats);
 }
 
+namespace {
+
+// The bf16 form of the call below: passes of as many whole blocks as the work space holds.
+tandem_status forced_forward(tandem_ctx* c, int gamma, int batch, const int32_t* ids, const int32_t* lens, long long total, float* nll, int32_t* top1) {
+    CK(cudaEventSynchronize(c->ev_staged));   // (the staging buffer may still be read by a prompt pass's copy)
+    int32_t *p_ids = c->pinned, *p_off = p_ids + total, *p_len = p_off + batch, *p_start = p_len + batch;
+    memcpy(p_ids, ids, (size_t)total * 4);
+    int off = 0, rows = 0, max_len = 0;
+    for (int b = 0; b < batch; ++b) {
+        p_off[b] = off; p_len[b] = lens[b]; p_start[b] = rows;
+        off += lens[b];
+        rows += cdiv(lens[b] - 1, gamma) * gamma;
+        max_len = std::max(max_len, lens[b]);
+    }
+    p_start[batch] = rows;
+    CK(cudaMemsetAsync(c->arena + c->lay.st_n, 0, c->lay.row_tok - c->lay.st_n, c->stream));
+    CK(cudaMemcpyAsync(c->arena + c->lay.forced_ids, p_ids, (size_t)total * 4, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(c->arena + c->lay.fr_seq, p_off, (size_t)(3 * batch + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaEventRecord(c->ev_staged, c->stream));
+    c->batch = batch; c->n_ub = max_len; c->n_sum = total; c->last_gamma = gamma;
+    launch_call_begin(*c, true);
+    ForcedRows f;
+    f.ids = at<int>(*c, c->lay.forced_ids); f.off = at<int>(*c, c->lay.fr_seq); f.len = f.off + batch; f.vstart = f.len + batch;
+    f.batch = batch; f.group = ATT_NQ;
+    f.row_tok = at<int>(*c, c->lay.row_tok); f.row_seq = at<int>(*c, c->lay.row_seq); f.row_pos = at<int>(*c, c->lay.row_pos);
+    f.truth = at<int>(*c, c->lay.fr_truth); f.out = at<int>(*c, c->lay.fr_out);
+    f.grp_row0 = at<int>(*c, c->lay.fr_grp); f.grp_cnt = f.grp_row0 + c->lay.fr_rows / ATT_NQ + c->cfg.max_batch + 1;
+    const int step = c->lay.fr_rows / gamma * gamma;
+    for (f.v0 = 0; f.v0 < rows; f.v0 += step) {
+        f.rows = std::min(step, rows - f.v0);
+        int groups = 0;
+        double kv = 0.0;
+        for (int b = 0; b < batch; ++b) {
+            const int n = std::min(p_start[b + 1], f.v0 + f.rows) - std::max(p_start[b], f.v0);
+            if (n > 0) { groups += cdiv(n, f.group); kv += (double)n / f.group * lens[b]; }
+        }
+        forced_pass(*c, f, gamma, groups, kv);
+    }
+    TRY(check_launch(*c));
+    // scores and the error word come back behind one wait (the ids have long been copied out of the staging buffer)
+    const size_t n = (size_t)(total - batch);
+    int32_t* cnt = c->pinned + 2 * n;
+    CK(cudaMemcpyAsync(c->pinned, c->arena + c->lay.forced_nll, n * 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(c->pinned + n, c->arena + c->lay.forced_top, n * 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(cnt, c->st.counters, 8 * 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    if (cnt[2] != 0) {
+        snprintf(g_cuda_err, sizeof(g_cuda_err), "device-side wait expired (code %d)", cnt[2]);
+        CK(cudaMemsetAsync(c->st.counters + 2, 0, 4, c->stream));
+        return TANDEM_ERR_TIMEOUT;
+    }
+    memcpy(nll, c->pinned, n * 4);
+    if (top1) memcpy(top1, c->pinned + n, n * 4);
+    return TANDEM_OK;
+}
+
+}  // namespace
+
 extern "C" tandem_status tandem_teacher_forced_forward(tandem_ctx* c, int32_t gamma, int32_t batch, const int32_t* ids, const int32_t* lens,
                                                        float* nll, int32_t* top1) {
     TRY(begin_call(c));
@@ -1924,6 +2076,7 @@ extern "C" tandem_status tandem_teacher_forced_forward(tandem_ctx* c, int32_t ga
     if ((long long)max_len + gamma > pos_cap) return TANDEM_ERR_CAPACITY;
     for (long long i = 0; i < total; ++i)
         if (ids[i] < 0 || ids[i] >= c->cfg.large.vocab) return TANDEM_ERR_INVALID_ARG;
+    if (c->cfg.dtype == TANDEM_DTYPE_BF16) return forced_forward(c, gamma, batch, ids, lens, total, nll, top1);
     // an empty prompt pass: the first token of every sequence is its pending token
     std::vector<int32_t> first((size_t)batch), ones((size_t)batch, 1), padded((size_t)batch * c->cfg.max_seq, 0);
     long long off = 0;

@@ -117,6 +117,33 @@ def test_decode_attention_by_lone_ctas(batch, heads, dh, derived, own):
     assert (out - want).abs().max() < TOL_BF16
 
 
+@pytest.mark.parametrize("lens,gamma,prefill_rows,kw", [
+    ([2, 140, 23], 4, 0, dict(layer_map=(1, 3), vocab=129)),                     # one pass of 168 rows: three groups, the last of 40; a head tile of one feature
+    ([131, 7, 66], 3, 20, dict(layer_map=(0, 2))),                               # passes of 12 rows: a sequence over many of them
+    ([47], 15, 0, dict(large=(2, 256, 2, 264), small=(1, 256, 2, 136), kv_heads=(1, 1), layer_map=(2,))),   # blocks of 15, 128-wide heads, shared keys / values
+    ([66, 2], 1, 0, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3), small=(2, 192, 6, 136)))])  # 66 blocks of one row; a small model wider than the large one
+def test_bf16_teacher_forced_pass(lens, gamma, prefill_rows, kw):
+    """All blocks of a teacher-forced forward in one pass or a few: ragged sequences padded to whole blocks, groups of 64 rows, blocks
+    that attend large-derived keys up to their start and their own from there."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, **kw)
+    w = _bf16_weights(shape, seed=23, std=0.06)
+    seqs = prompts_for(shape, lens, seed=24)
+    t = binding.Tandem(shape, w, max_batch=len(lens), max_seq=200, gamma_max=gamma, max_prefill_rows=prefill_rows)
+    for _ in range(2):   # (the second call finds the first one's keys and values in the caches)
+        nll, top = t.tandem_teacher_forced_forward(seqs, gamma)
+        differ = 0
+        for b, ids in enumerate(seqs):
+            logits = O.teacher_forced_tandem_logits(shape, w, ids, gamma)
+            want_nll, want_top = O.next_token_scores(logits, ids)
+            assert nll[b].shape == (len(ids) - 1,)
+            assert np.abs(nll[b] - want_nll).max() < 2 * TOL_BF16
+            for i in np.nonzero(top[b] != want_top)[0]:
+                assert np.max(logits[i]) - logits[i][top[b][i]] < 2 * TOL_BF16
+            differ += int((top[b] != want_top).sum())
+        assert differ <= 4
+    t.close()
+
+
 def test_bf16_layernorm_parameters_changed_between_calls():
     """Gains and biases that the caller changes after the prompt pass, and again between two steps, hold from the next call on, in
     every map behind a LayerNorm and in the projection."""
