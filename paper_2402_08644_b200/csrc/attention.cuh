@@ -308,9 +308,10 @@ constexpr size_t attn_decode_smem_bytes() {
     // the warps' rings (reused for the warps' final states) + the inbox of states sent by the cluster's CTAs
     return (size_t)ATD_WARPS * AtdCfg<DH>::STAGES * AtdCfg<DH>::STAGE_ELEMS * sizeof(bf16) + sizeof(float) * (size_t)ATD_SLOTS * (DH + 2);
 }
-static_assert((size_t)ATD_WARPS * ATT_NQ * (128 + 2) * sizeof(float) <= (size_t)ATD_WARPS * AtdCfg<128>::STAGES * AtdCfg<128>::STAGE_ELEMS * sizeof(bf16) &&
-              (size_t)ATD_WARPS * ATT_NQ * (32 + 2) * sizeof(float) <= (size_t)ATD_WARPS * AtdCfg<32>::STAGES * AtdCfg<32>::STAGE_ELEMS * sizeof(bf16),
-              "the warps' states fit in the ring");
+static_assert((size_t)ATT_NQ * (128 + 2) * sizeof(float) <= (size_t)AtdCfg<128>::STAGES * AtdCfg<128>::STAGE_ELEMS * sizeof(bf16) &&
+              (size_t)ATT_NQ * (64 + 2) * sizeof(float) <= (size_t)AtdCfg<64>::STAGES * AtdCfg<64>::STAGE_ELEMS * sizeof(bf16) &&
+              (size_t)ATT_NQ * (32 + 2) * sizeof(float) <= (size_t)AtdCfg<32>::STAGES * AtdCfg<32>::STAGE_ELEMS * sizeof(bf16),
+              "a warp's states fit in its ring");
 
 // Where the 16-byte unit u of ring row r lives within the row: XOR-swizzled so that the eight row addresses of
 // one ldmatrix fall into different banks (rows are DH * 2 bytes apart).
@@ -355,7 +356,8 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     constexpr int SW = DH + 2;                     // a state: DH output sums, the running maximum, the running sum
     extern __shared__ __align__(128) unsigned char smem_raw[];
     bf16* ring_all = reinterpret_cast<bf16*>(smem_raw);
-    float* wst = reinterpret_cast<float*>(smem_raw);                                            // [NW][16][SW], after the main loop
+    constexpr int WST = C::STAGES * C::STAGE_ELEMS / 2;      // floats between two warps' states: each where the warp's ring was
+    float* wst = reinterpret_cast<float*>(smem_raw);         // [NW][16][SW], after the main loop
     float* inbox = reinterpret_cast<float*>(ring_all + (size_t)NW * C::STAGES * C::STAGE_ELEMS);   // [CL][QPC][SW]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -365,7 +367,8 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     const int gpc = a.heads_per_cta > 0 ? a.heads_per_cta : 1;
     const int h = blockIdx.y * gpc;                // first query head of this CTA
     const int CL = MODE == ATD_CLUSTERED ? gridDim.x : 1;   // cluster size
-    const int QPC = (ATT_NQ + CL - 1) / CL;        // queries a CTA finishes at most
+    const int log_cl = MODE == ATD_CLUSTERED ? __ffs(CL) - 1 : 0;   // (a division by a number known at run time costs the chain about 0.05 us)
+    const int QPC = ATT_NQ >> log_cl;              // queries a CTA finishes at most
     __shared__ __align__(8) uint64_t s_inbox_bar;  // counts the bytes of the states sent to this CTA by the cluster's CTAs
     if (CL > 1 && tid == 0) { mbar_init(smem_u32(&s_inbox_bar), 1); mbar_init_fence(); }
     if (CL > 1) cluster_arrive_relaxed();          // opening handshake: waited for just before the first remote store
@@ -374,6 +377,8 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // The row arrays were written at the start of the pass, at least two kernels back in the stream, so they may be
     // read before the wait below: a kernel lets its successor start only after its own wait has returned, that is
     // after its predecessor has finished, hence everything older than the immediate predecessor is complete.
+    const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
+    const int kvh = n_kv == a.n_heads ? h : h / (a.n_heads / n_kv);   // grouped-query attention: several query heads share one key/value head
     if (a.wait_first) pdl_wait();
     int nq = a.nq, row0 = g * nq;
     if (MODE == ATD_PASS && a.grp_cnt) { nq = __ldcg(a.grp_cnt + g); row0 = __ldcg(a.grp_row0 + g); }
@@ -382,9 +387,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
     const int pos_last = pos_first + nq - 1;
     const int n_chunks = pos_last / ATT_CH + 1;
-    const int n_mine = rank < n_chunks ? (n_chunks - rank + CL - 1) / CL : 0;
-    const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
-    const int kvh = h / (a.n_heads / n_kv);            // grouped-query attention: several query heads share one key/value head
+    const int n_mine = rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
     const size_t head_base2 = ((size_t)b * n_kv + kvh) * (MODE == ATD_PASS ? a.t_max : a.t_max2);
     const int split = a.k2 ? (MODE == ATD_PASS ? pos_first : a.split) : INT_MAX;
@@ -462,7 +465,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
         const int rr = nt * 8 + (lane >> 2);
-        const int hq = rr < cnt ? rr / nq : 0, ib = rr < cnt ? rr - hq * nq : 0;      // query head within the CTA, block row
+        const int hq = gpc > 1 && rr < cnt ? rr / nq : 0, ib = rr < cnt ? rr - hq * nq : 0;      // query head within the CTA, block row
         const bf16* qp = static_cast<const bf16*>(a.q) + (size_t)(row0 + ib) * a.ldq + (h + hq) * DH + kc;
 #pragma unroll
         for (int ks = 0; ks < C::KSTEPS; ++ks) {
@@ -479,7 +482,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int rr = nt * 8 + kc + e;
-            q_last[nt][e] = rr < cnt ? pos_first + rr % nq : -1;
+            q_last[nt][e] = rr < cnt ? pos_first + (gpc > 1 ? rr % nq : rr) : -1;
             m[nt][e] = -INFINITY;
             l[nt][e] = 0.f;
         }
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     }
     pdl_launch_dependents();   // the successor starts behind the merge, not behind this kernel's loads (measured: a little faster)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();   // every warp is done with its ring: the warps' states go where the rings were
+    __syncwarp();   // this warp is done with its ring: its states go there
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -578,16 +581,16 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             lr += __shfl_xor_sync(0xffffffffu, lr, 16);
             const int rr = nt * 8 + kc + e;
             if (rr >= cnt) continue;
-            float* st = wst + (size_t)(warp * ATT_NQ + rr) * SW + (lane >> 2);
+            float* st = wst + warp * WST + rr * SW + (lane >> 2);
 #pragma unroll
             for (int mt = 0; mt < C::KSTEPS; ++mt) { st[mt * 16] = o[nt][mt][e]; st[mt * 16 + 8] = o[nt][mt][2 + e]; }
             if (lane < 4) { st[DH] = m[nt][e]; st[DH + 1] = lr; }
         }
     __syncthreads();
-    // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa % CL
+    // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa & (CL - 1)
     if (CL > 1) cluster_wait();   // closes the opening handshake: every CTA of the cluster is running
     auto store = [&](int qi, int e, float res) {   // tile row qi = query head hq of this CTA, block row qi - hq * nq
-        const int hq = qi / nq;
+        const int hq = gpc > 1 ? qi / nq : 0;
         const size_t oi = (size_t)(row0 + qi - hq * nq) * a.ldo + (h + hq) * DH + e;
         if (a.out_lo) {
             const bf16 hi = __float2bfloat16_rn(res);
@@ -604,28 +607,28 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         const int qa = i / DH, e = i - qa * DH;
         float mx = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) mx = fmaxf(mx, wst[(size_t)(w * ATT_NQ + qa) * SW + DH]);
+        for (int w = 0; w < NW; ++w) mx = fmaxf(mx, wst[w * WST + qa * SW + DH]);
         float val = 0.f, lsum = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
-            const float* st = wst + (size_t)(w * ATT_NQ + qa) * SW;
+            const float* st = wst + w * WST + qa * SW;
             const float f = st[DH] > -INFINITY ? __expf(st[DH] - mx) : 0.f;
             val = fmaf(st[e], f, val);
             if (e == 0 || MODE != ATD_CLUSTERED) lsum = fmaf(st[DH + 1], f, lsum);
         }
         if (MODE != ATD_CLUSTERED) { store(qa, e, val / lsum); continue; }
-        float* slot = inbox + ((size_t)rank * QPC + qa / CL) * SW;
-        st_async_dsmem_f32(smem_u32(slot + e), smem_u32(&s_inbox_bar), qa % CL, val);   // counted on the receiver's barrier
+        float* slot = inbox + ((size_t)rank * QPC + (qa >> log_cl)) * SW;
+        st_async_dsmem_f32(smem_u32(slot + e), smem_u32(&s_inbox_bar), qa & (CL - 1), val);   // counted on the receiver's barrier
         if (e == 0) {
-            st_async_dsmem_f32(smem_u32(slot + DH), smem_u32(&s_inbox_bar), qa % CL, mx);
-            st_async_dsmem_f32(smem_u32(slot + DH + 1), smem_u32(&s_inbox_bar), qa % CL, lsum);
+            st_async_dsmem_f32(smem_u32(slot + DH), smem_u32(&s_inbox_bar), qa & (CL - 1), mx);
+            st_async_dsmem_f32(smem_u32(slot + DH + 1), smem_u32(&s_inbox_bar), qa & (CL - 1), lsum);
         }
     }
     if (MODE != ATD_CLUSTERED) return;
     {
         // This CTA finishes queries rank, rank + CL, ...: it waits (bounded) until every CTA's state of each of them
         // has arrived.  No cluster-wide barrier: a CTA without queries of its own leaves right after sending.
-        const int n_fin = rank < cnt ? (cnt - rank + CL - 1) / CL : 0;
+        const int n_fin = rank < cnt ? (cnt - rank + CL - 1) >> log_cl : 0;
         if (n_fin > 0) {
             if (tid == 0) mbar_arrive_expect_tx(smem_u32(&s_inbox_bar), (uint32_t)(CL * n_fin * SW * 4));
             if (!mbar_wait(smem_u32(&s_inbox_bar), 0) && a.err_flag) atomicExch(a.err_flag, ATD_ERR_EXCHANGE);

@@ -663,6 +663,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
     }
     float v[NB];
     const int tl = warp * 32 + lane;
+    ScatterCol sc;
     if (warp < 4) {
         // The successor may start (set up, fetch its first weight tiles) once this kernel's token-row loads are out of
         // its way: right after they have been issued when the K-slice fits the ring (one round of loads; see above),
@@ -677,24 +678,27 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
             bar_sync(1, 128);
         }
         if (EPI == EPI_RESID && a.e.ln.gain) bar_sync(1, 128);
+        if (EPI == EPI_QKV || EPI == EPI_KV) sc = scatter_col<EPI>(a.e, seg, n_local0 + tl);   // (a division: ahead of the wait)
         if (!mbar_wait(smem_u32(&s_accum), 0, poll_limit)) tc_report(a.err_flag, TC_ERR_ACCUM);
         tc_fence_after_sync();
         float c1 = 0.f, c2 = 0.f;                     // PRO_LNT: this feature's (slice of) g W^T and b W^T
-        if (LNT) {
-            float w[16];
-            tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + C::NB2, w);
-            c1 = w[0] + w[1];
-            c2 = w[2] + w[3];
-        }
+        const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if (LNT) tmem_issue4(acc + C::NB2, w);
 #pragma unroll
         for (int c0 = 0; c0 < NB; c0 += 16) {
             if (c0 >= a.rows) break;                  // columns of absent token rows are never read
-            float t[16], u[16];
-            tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c0, t);        // x's values times W
-            tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + NB + c0, u);   // x's remainders times W
+            uint32_t t[16], u[16];
+            tmem_issue16(acc + c0, t);                // x's values times W
+            tmem_issue16(acc + NB + c0, u);           // x's remainders times W
+            tmem_wait_ld(t, u, w);
+            if (LNT && c0 == 0) {
+                c1 = __uint_as_float(w[0]) + __uint_as_float(w[1]);
+                c2 = __uint_as_float(w[2]) + __uint_as_float(w[3]);
+            }
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                v[c0 + i] = t[i] + u[i];
+                v[c0 + i] = __uint_as_float(t[i]) + __uint_as_float(u[i]);
                 if (LNT) v[c0 + i] = fmaf(s_rstd[c0 + i], fmaf(-s_mu[c0 + i], c1, v[c0 + i]), c2);   // (rows past the last: never used)
             }
         }
@@ -771,8 +775,6 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
         }
         // v[s] is now the finished product of token row j_first + s and this thread's feature
         if (warp < 4) {
-            ScatterCol sc;
-            if (EPI == EPI_QKV || EPI == EPI_KV) sc = scatter_col<EPI>(a.e, seg, n_local);
             const int n_group = max(0, min(32, seg_rows - (n_local0 + warp * 32)));   // features of this warp's group of 32
 #pragma unroll
             for (int s = 0; s < NB; ++s) {
@@ -814,6 +816,14 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
                 // row, with two five-step sums each, they cost 1.3 us of a 7.4 us launch with four rows per CTA).  Sums are
                 // relative to the group's first feature.
                 const float inv = 1.0f / (float)n_group;
+                float2* stats = a.e.ln.stats + (size_t)j_first * a.e.ln.groups + ((seg_base + n_local0 + warp * 32) >> 5);
+                if (j_count == 1) {   // one row (a step's, or a row of a block dealt to its own CTA): five shuffles instead of nine, the same tree
+                    const float ref = __shfl_sync(0xffffffffu, v[0], 0), dv = valid ? v[0] - ref : 0.f;
+                    float sums[2] = {dv, dv * dv};
+                    const float mine = warp_sum_many<2>(sums, lane);                     // lanes 0-15: the sum, 16-31: the sum of squares
+                    const float sd = mine, sq = __shfl_sync(0xffffffffu, mine, 16);
+                    if (lane == 0) *stats = make_float2(fmaf(sd, inv, ref), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
+                } else
 #pragma unroll
                 for (int s0 = 0; s0 < NB; s0 += 4) {
                     if (s0 >= j_count) break;
@@ -831,8 +841,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
                     const int u = lane >> 3;
                     if ((lane & 7) == 0 && s0 + u < j_count) {
                         const float rf = u == 0 ? ref[0] : (u == 1 ? ref[1] : (u == 2 ? ref[2] : ref[3]));
-                        a.e.ln.stats[(size_t)(j_first + s0 + u) * a.e.ln.groups + ((seg_base + n_local0 + warp * 32) >> 5)] =
-                            make_float2(fmaf(sd, inv, rf), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
+                        stats[(size_t)(s0 + u) * a.e.ln.groups] = make_float2(fmaf(sd, inv, rf), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
                     }
                 }
             }
