@@ -38,6 +38,7 @@ struct AttnArgs {
                                                //   (a stand-alone call: whatever precedes it may be writing the keys and values)
     const int* grp_row0; const int* grp_cnt;   // nullable: then group g = rows g*nq .. g*nq+nq-1
     int nq;
+    int units;                           // ATD_PASS: groups * head groups = warps
     int n_heads, t_max;
     int n_kv_heads;                      // key/value heads of the caches; 0 = n_heads.  Query head h reads kv head h / (n_heads / n_kv_heads)
     int* err_flag;                       // attn_decode_kernel: where a bounded wait that ran out records its code (nullable)
@@ -346,8 +347,9 @@ __device__ __forceinline__ uint32_t atd_pack_bf16x2(float lo, float hi) {
 // grid: (CL, heads, sequences or groups) with the CL CTAs along x forming one cluster, CL in {1, 2, 4, 8}; block: ATD_THREADS.
 // NT: groups of eight query columns in use (1 up to eight rows per CTA, 2 up to 16).
 // MODE: ATD_CLUSTERED, CL in {2, 4, 8}; ATD_ALONE, CL = 1, results straight from the fold of the warps' states (32 x 16 x 64 x 8194:
-// 171 -> 165 us, without the trip through the inbox); ATD_PASS, CL = 1 in a teacher-forced pass: groups of unequal length, the second segment of a block's own keys.  (The
-// same code with these choices made at run time costs the stand-alone call on 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
+// 171 -> 165 us, without the trip through the inbox); ATD_PASS, a teacher-forced pass: groups of unequal length, the second segment of a block's own keys,
+// and a warp on its own per group and head, since there are hundreds of them over short contexts (grid: warps in all / 8; 49 groups x 16
+// heads x 64 over up to 257 positions: 25 -> 20 us under ncu, 193 blocks of four rows x 8 heads 26 -> 17 us).  (The same code with these choices made at run time costs the stand-alone call on 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
 enum { ATD_CLUSTERED = 0, ATD_ALONE = 1, ATD_PASS = 2 };
 template <int DH, int NT, int MODE>
 __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
@@ -361,11 +363,14 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     float* inbox = reinterpret_cast<float*>(ring_all + (size_t)NW * C::STAGES * C::STAGE_ELEMS);   // [CL][QPC][SW]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = blockIdx.x, g = blockIdx.z;
+    const int rank = MODE == ATD_PASS ? 0 : blockIdx.x;
     // Grouped-query attention: the tile's 16 rows hold the block's queries of `gpc` query heads that share one
     // key/value head (row = head * nq + block row), so their keys and values are streamed once for all of them.
     const int gpc = a.heads_per_cta > 0 ? a.heads_per_cta : 1;
-    const int h = blockIdx.y * gpc;                // first query head of this CTA
+    const int head_groups = a.n_heads / gpc, unit = MODE == ATD_PASS ? blockIdx.x * NW + warp : 0;   // ATD_PASS: this warp's number
+    if (MODE == ATD_PASS && unit >= a.units) return;
+    const int g = MODE == ATD_PASS ? unit / head_groups : blockIdx.z;
+    const int h = (MODE == ATD_PASS ? unit - g * head_groups : blockIdx.y) * gpc;   // first query head of this CTA (warp)
     const int CL = MODE == ATD_CLUSTERED ? gridDim.x : 1;   // cluster size
     const int log_cl = MODE == ATD_CLUSTERED ? __ffs(CL) - 1 : 0;   // (a division by a number known at run time costs the chain about 0.05 us)
     const int QPC = ATT_NQ >> log_cl;              // queries a CTA finishes at most
@@ -379,7 +384,10 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // after its predecessor has finished, hence everything older than the immediate predecessor is complete.
     const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
     const int kvh = n_kv == a.n_heads ? h : h / (a.n_heads / n_kv);   // grouped-query attention: several query heads share one key/value head
-    if (a.wait_first) pdl_wait();
+    if (a.wait_first) {   // (a successor has nothing to fetch that would be in this kernel's way)
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     int nq = a.nq, row0 = g * nq;
     if (MODE == ATD_PASS && a.grp_cnt) { nq = __ldcg(a.grp_cnt + g); row0 = __ldcg(a.grp_row0 + g); }
     const int cnt = gpc * nq;                      // rows of the tile in use
@@ -387,7 +395,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
     const int pos_last = pos_first + nq - 1;
     const int n_chunks = pos_last / ATT_CH + 1;
-    const int n_mine = rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
+    const int n_mine = MODE == ATD_PASS ? pos_last / ATD_WROWS + 1 : rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
     const size_t head_base2 = ((size_t)b * n_kv + kvh) * (MODE == ATD_PASS ? a.t_max : a.t_max2);
     const int split = a.k2 ? (MODE == ATD_PASS ? pos_first : a.split) : INT_MAX;
@@ -398,8 +406,9 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // boundary tile or two) takes the short way: one base address, constant steps.
     constexpr int RSTEP = 32 / C::TPK;             // rows between a lane's consecutive units
     const int i_row = lane / C::TPK, i_unit = lane - i_row * C::TPK;
+    auto tile_start = [&](int it) { return MODE == ATD_PASS ? it * ATD_WROWS : (rank + it * CL) * ATT_CH + warp * ATD_WROWS; };
     auto issue = [&](int it) {
-        const int t0 = (rank + it * CL) * ATT_CH + warp * ATD_WROWS;
+        const int t0 = tile_start(it);
         bf16* ks = ring + (size_t)(it % C::STAGES) * C::STAGE_ELEMS;
         bf16* vs = ks + C::TILE_ELEMS;
         const bool first = t0 + ATD_WROWS <= split, second = t0 >= split;
@@ -443,7 +452,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     int pre = 0;
 #pragma unroll
     for (int it = 0; it < C::STAGES - 1; ++it) {
-        if (it == pre && it < n_mine && (rank + it * CL) * ATT_CH + (warp + 1) * ATD_WROWS <= pos_first) {
+        if (it == pre && it < n_mine && tile_start(it) + ATD_WROWS <= pos_first) {
             issue(it);
             cp_async_commit();
             ++pre;
@@ -501,7 +510,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         cp_async_commit();
         asm volatile("cp.async.wait_group %0;" ::"n"(C::STAGES - 1) : "memory");
         __syncwarp();
-        const int t0 = (rank + it * CL) * ATT_CH + warp * ATD_WROWS;
+        const int t0 = tile_start(it);
         const uint32_t ks_s = ring_s + (uint32_t)((it % C::STAGES) * C::STAGE_ELEMS * 2);
         const uint32_t vs_s = ks_s + (uint32_t)(C::TILE_ELEMS * 2);
 
@@ -569,6 +578,36 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         __syncwarp();   // the stage may be refilled by this warp's next issue
     }
     pdl_launch_dependents();   // the successor starts behind the merge, not behind this kernel's loads (measured: a little faster)
+    auto store = [&](int qi, int e, float res) {   // tile row qi = query head hq of this CTA (warp), block row qi - hq * nq
+        const int hq = gpc > 1 ? qi / nq : 0;
+        const size_t oi = (size_t)(row0 + qi - hq * nq) * a.ldo + (h + hq) * DH + e;
+        if (a.out_lo) {
+            const bf16 hi = __float2bfloat16_rn(res);
+            static_cast<bf16*>(a.out)[oi] = hi;
+            static_cast<bf16*>(a.out_lo)[oi] = __float2bfloat16_rn(res - __bfloat162float(hi));
+        } else {
+            static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
+        }
+    };
+    if constexpr (MODE == ATD_PASS) {   // the warp has met all keys: results straight from its registers
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float lr = l[nt][e];
+                lr += __shfl_xor_sync(0xffffffffu, lr, 4);
+                lr += __shfl_xor_sync(0xffffffffu, lr, 8);
+                lr += __shfl_xor_sync(0xffffffffu, lr, 16);
+                const int rr = nt * 8 + kc + e;
+                if (rr >= cnt) continue;
+#pragma unroll
+                for (int mt = 0; mt < C::KSTEPS; ++mt) {
+                    store(rr, mt * 16 + (lane >> 2), o[nt][mt][e] / lr);
+                    store(rr, mt * 16 + 8 + (lane >> 2), o[nt][mt][2 + e] / lr);
+                }
+            }
+        return;
+    }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();   // this warp is done with its ring: its states go there
 #pragma unroll
@@ -589,17 +628,6 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     __syncthreads();
     // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa & (CL - 1)
     if (CL > 1) cluster_wait();   // closes the opening handshake: every CTA of the cluster is running
-    auto store = [&](int qi, int e, float res) {   // tile row qi = query head hq of this CTA, block row qi - hq * nq
-        const int hq = gpc > 1 ? qi / nq : 0;
-        const size_t oi = (size_t)(row0 + qi - hq * nq) * a.ldo + (h + hq) * DH + e;
-        if (a.out_lo) {
-            const bf16 hi = __float2bfloat16_rn(res);
-            static_cast<bf16*>(a.out)[oi] = hi;
-            static_cast<bf16*>(a.out_lo)[oi] = __float2bfloat16_rn(res - __bfloat162float(hi));
-        } else {
-            static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
-        }
-    };
     // One thread per (query, output element); the thread of element 0 also folds the query's running sum and sends its
     // maximum (with 4 queries of 64 elements that is one pass over the block's 256 threads).  A CTA on its own has the result
     // right here (every thread folds the sum then).
@@ -614,9 +642,9 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             const float* st = wst + w * WST + qa * SW;
             const float f = st[DH] > -INFINITY ? __expf(st[DH] - mx) : 0.f;
             val = fmaf(st[e], f, val);
-            if (e == 0 || MODE != ATD_CLUSTERED) lsum = fmaf(st[DH + 1], f, lsum);
+            if (e == 0 || MODE == ATD_ALONE) lsum = fmaf(st[DH + 1], f, lsum);
         }
-        if (MODE != ATD_CLUSTERED) { store(qa, e, val / lsum); continue; }
+        if (MODE == ATD_ALONE) { store(qa, e, val / lsum); continue; }
         float* slot = inbox + ((size_t)rank * QPC + (qa >> log_cl)) * SW;
         st_async_dsmem_f32(smem_u32(slot + e), smem_u32(&s_inbox_bar), qa & (CL - 1), val);   // counted on the receiver's barrier
         if (e == 0) {
@@ -624,7 +652,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             st_async_dsmem_f32(smem_u32(slot + DH + 1), smem_u32(&s_inbox_bar), qa & (CL - 1), lsum);
         }
     }
-    if (MODE != ATD_CLUSTERED) return;
+    if (MODE == ATD_ALONE) return;
     {
         // This CTA finishes queries rank, rank + CL, ...: it waits (bounded) until every CTA's state of each of them
         // has arrived.  No cluster-wide barrier: a CTA without queries of its own leaves right after sending.

@@ -663,10 +663,10 @@ void launch_attn(tandem_ctx& c, int d_head, const AttnArgs& a, int groups, bool 
 
 // bf16 decode attention: one cluster of `cl` CTAs per (sequence, group of query heads); no scratch.
 template <int DH, int NT, int MODE>
-void launch_attn_decode_as(tandem_ctx& c, const AttnArgs& a, dim3 grid) {
+void launch_attn_decode_as(tandem_ctx& c, const AttnArgs& a, dim3 grid, int cl) {
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(attn_decode_kernel<DH, NT, MODE>, attn_decode_smem_bytes<DH>(), attr_done);
-    launch_ex(c, true, (int)grid.x, attn_decode_kernel<DH, NT, MODE>, grid, dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
+    launch_ex(c, true, cl, attn_decode_kernel<DH, NT, MODE>, grid, dim3(ATD_THREADS), attn_decode_smem_bytes<DH>(), a);
 }
 template <int DH>
 void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl, bool pass, double kv_bytes) {
@@ -674,10 +674,15 @@ void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl,
     const bool narrow = gpc * a.nq <= 8;
     const dim3 grid(cl, a.n_heads / gpc, groups);
     ProfScope ps(c, PC_ATTN_SPLIT, kv_bytes);
-    if (pass) { if (narrow) launch_attn_decode_as<DH, 1, ATD_PASS>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_PASS>(c, a, grid); }
-    else if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid); }
-    else if (narrow) launch_attn_decode_as<DH, 1, ATD_CLUSTERED>(c, a, grid);
-    else launch_attn_decode_as<DH, 2, ATD_CLUSTERED>(c, a, grid);
+    if (pass) {
+        AttnArgs w = a;
+        w.units = groups * (a.n_heads / gpc);
+        const dim3 warps(cdiv(w.units, ATD_WARPS));
+        if (narrow) launch_attn_decode_as<DH, 1, ATD_PASS>(c, w, warps, 1); else launch_attn_decode_as<DH, 2, ATD_PASS>(c, w, warps, 1);
+    }
+    else if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid, cl); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid, cl); }
+    else if (narrow) launch_attn_decode_as<DH, 1, ATD_CLUSTERED>(c, a, grid, cl);
+    else launch_attn_decode_as<DH, 2, ATD_CLUSTERED>(c, a, grid, cl);
 }
 // Clusters of `cl` decode-attention CTAs that the device can run at the same time (asked once per device and size).  It is
 // less than the multiprocessors would suggest, because a cluster has to fit into one GPC: with 148 multiprocessors and one
@@ -719,7 +724,7 @@ int attn_cluster_size(long long clusters, int d_head) {
     }
     return best;
 }
-// pass: a teacher-forced pass, which has a CTA per group of rows and head.
+// pass: a teacher-forced pass, which has a warp per group of rows and head.
 void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int groups, double kv_bytes, bool pass = false) {
     AttnArgs a = a0;
     // Grouped-query attention: the query heads of one key/value head ride in one CTA as far as the 16-row tile has
