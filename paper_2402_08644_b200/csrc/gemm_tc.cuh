@@ -48,7 +48,8 @@ namespace tandem {
 // 4.4 + 1.9 us with a LayerNorm kernel of their own (more sequences).
 enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3, PRO_LNT = 4 };
 constexpr int EPI_ARGMAX = 6;                       // fp32 store plus the (max, index) of each row within the tile
-constexpr int EPI_SCORE = 7;                        // no store: per row the tile's (max, index, sum of exp(y - max)), and y at a given feature
+constexpr int EPI_SCORE = 7;                        // many rows: no store, per row and SCORE_TILE features (max, index, sum of exp(y - max)), and y at a given feature
+constexpr int SCORE_TILE = 64;
 enum { TC_ERR_SLOT = 1, TC_ERR_OPERANDS = 2, TC_ERR_ACCUM = 3, TC_ERR_EXCHANGE = 4 };   // which bounded wait gave up
 
 struct TcDecodeArgs {
@@ -76,24 +77,20 @@ struct TcDecodeArgs {
     unsigned poll_limit;    // polls before a wait on an mbarrier gives up; 0 = MBAR_POLL_LIMIT
     int withhold_weights;   // test hook for the give-up path: the TMA thread issues no loads, so the wait for
                             // operands must run out (nothing is in flight when the kernel leaves)
-    float* amax_val;        // EPI_ARGMAX, EPI_SCORE: [rows][amax_stride] best value per tile
+    float* amax_val;        // EPI_ARGMAX: [rows][amax_stride] best value per tile
     int* amax_idx;          //             and its output feature
     int amax_stride;
-    float* score_sum;       // EPI_SCORE: [rows][amax_stride] sum over the tile's features of exp(y - the tile's best value)
-    const int* truth;       // EPI_SCORE: [rows] the feature whose value goes to truth_val [rows]
-    float* truth_val;
     EpiArgs e;
 };
 
 // The same pass from its row r0 on (nr rows): everything that is indexed by token row moves along.
 template <int PRO, int EPI>
-__host__ __device__ __forceinline__ void tcd_shift_rows(TcDecodeArgs& a, int r0, int nr) {
+inline void tcd_shift_rows(TcDecodeArgs& a, int r0, int nr) {
     a.rows = nr;
     a.x_row0 += r0;
     if (a.x) a.x = static_cast<const unsigned char*>(a.x) + (size_t)r0 * a.ldx * (PRO == PRO_BF16 ? 2 : 4);
     if (PRO == PRO_LNT) { a.ln_stats += (size_t)r0 * a.ln_groups; a.ln_ref += r0; a.ln_mean += r0; }
-    if (EPI == EPI_ARGMAX || EPI == EPI_SCORE) { a.amax_val += (size_t)r0 * a.amax_stride; a.amax_idx += (size_t)r0 * a.amax_stride; }
-    if (EPI == EPI_SCORE) { a.score_sum += (size_t)r0 * a.amax_stride; a.truth += r0; a.truth_val += r0; }
+    if (EPI == EPI_ARGMAX) { a.amax_val += (size_t)r0 * a.amax_stride; a.amax_idx += (size_t)r0 * a.amax_stride; }
     EpiArgs& e = a.e;
     if (e.out) e.out = static_cast<unsigned char*>(e.out) + (size_t)r0 * e.ldo * ((EPI == EPI_QKV || EPI == EPI_STORE || e.out_lo) ? 2 : 4);
     if (e.out_lo) e.out_lo = static_cast<unsigned char*>(e.out_lo) + (size_t)r0 * e.ldo * 2;   // (value / remainder planes are bf16)
@@ -113,7 +110,6 @@ template <int NB, bool LNT> struct TcdCfg {
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + (LNT ? 1024 : 0);   // (the MMA's last twelve B rows are whatever follows: unread columns)
     static constexpr int INBOX_BYTES = NB * 128 * 4;   // the K-slices' partial sums for the token rows this CTA finishes
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + INBOX_BYTES + 1024;   // + slack to align the ring to 1024
-    static constexpr int SMEM_BYTES_WHOLE = STAGES * STAGE_BYTES + 1024 + (LNT ? 1024 : 0);   // whole K, nothing exchanged: no inbox (LNT: the unread B rows of the last stage)
     static constexpr int TMEM_COLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
 static_assert(TcdCfg<16, true>::SMEM_BYTES + 1024 <= 113 * 1024 && TcdCfg<16, false>::SMEM_BYTES + 1024 <= 113 * 1024 &&
@@ -155,152 +151,15 @@ __device__ __forceinline__ ScatterCol scatter_col(const EpiArgs& e, int seg, int
     return sc;
 }
 
-// The epilogue of a whole pass (PASS): sixteen rows at a time, from TMEM to their places, in a loop that stays in the instruction cache
-// (the decode passes' epilogue, unrolled over its rows, is fetched once per CTA: 32 us for 384 rows x 4096 x 1024 with GELU
-// under ncu, 34 us for 772 rows like this).  Warps 0-3; thread = output feature.
+// grid: tiles * splits CTAs in clusters of `splits` (the K-slices of one tile); dynamic smem TcdCfg::SMEM_BYTES.
 template <int NB, int PRO, int EPI>
-__device__ __forceinline__ void tcd_pass_epilogue(const TcDecodeArgs& a, uint32_t tmem, int seg, int seg_rows, int seg_base, int n_local0, int tile, unsigned char* ring,
-                                                  float* s_mu, const float* s_rstd, long long* s_rowoff, uint64_t* s_accum, float next_gain, int my_seq, int my_pos,
-                                                  uint32_t poll_limit, bool long_slice) {
-    constexpr bool LNT = PRO == PRO_LNT, BY_TMA = PRO == PRO_TMA || LNT;
-    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
-    if (warp >= 4) return;
-    if (!BY_TMA || (!LNT && (!long_slice || a.release_early))) pdl_launch_dependents();
-    if (EPI == EPI_QKV || EPI == EPI_KV) {
-        if (tid < a.rows) s_rowoff[tid] = ((long long)my_seq * a.e.n_heads * a.e.t_max + my_pos) * a.e.d_head;
-        bar_sync(1, 128);
-    }
-    const bool with_ln = EPI == EPI_RESID && a.e.ln.gain;
-    if (with_ln) bar_sync(1, 128);
-    const int n_local = n_local0 + tid, n = seg_base + n_local;
-    const bool valid = n_local < seg_rows;
-    float hres[EPI == EPI_RESID ? 16 : 1];   // residual values, sixteen rows ahead
-    auto fetch = [&](int j0) {
-        const float* hp = static_cast<const float*>(a.e.out) + n;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) hres[EPI == EPI_RESID ? i : 0] = valid && j0 + i < a.rows ? __ldcg(hp + (size_t)(j0 + i) * a.e.ldo) : 0.f;
-    };
-    if (EPI == EPI_RESID) fetch(0);
-    ScatterCol sc;
-    if (EPI == EPI_QKV || EPI == EPI_KV) sc = scatter_col<EPI>(a.e, seg, n_local);
-    const int n_group = max(0, min(32, seg_rows - (n_local0 + warp * 32)));   // features of this warp's group of 32
-    const float inv = 1.0f / (float)max(1, n_group);
-    if (!mbar_wait(smem_u32(s_accum), 0, poll_limit)) tc_report(a.err_flag, TC_ERR_ACCUM);
-    tc_fence_after_sync();
-    const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-    float c1 = 0.f, c2 = 0.f;                // PRO_LNT: this feature's g W^T and b W^T
-    if (LNT) {
-        float w[16];
-        tmem_ld16(acc + 2 * NB, w);
-        c1 = w[0] + w[1];
-        c2 = w[2] + w[3];
-    }
-    constexpr int LD = 130;                  // EPI_SCORE: the tile in shared memory, [row][feature]: 16 rows x 2 threads of a warp meet 32 banks
-    float* tile_v = reinterpret_cast<float*>(ring);   // (where the ring was: every product has read it)
-#pragma unroll 1
-    for (int c0 = 0; c0 < a.rows; c0 += 16) {
-        float v[16], u[16];
-        tmem_ld16(acc + c0, v);              // x's values times W
-        tmem_ld16(acc + NB + c0, u);         // x's remainders times W
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            v[i] += u[i];
-            if (LNT) v[i] = fmaf(s_rstd[c0 + i], fmaf(-s_mu[c0 + i], c1, v[i]), c2);   // (rows past the last: never used)
-            if (EPI == EPI_RESID) v[i] += hres[EPI == EPI_RESID ? i : 0];
-        }
-        if (EPI == EPI_RESID && c0 + 16 < a.rows) fetch(c0 + 16);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int j = c0 + i;
-            if (j >= a.rows) break;
-            if (EPI == EPI_SCORE) { tile_v[j * LD + tid] = valid ? v[i] : -INFINITY; continue; }
-            if (!valid) continue;
-            if (EPI == EPI_RESID || EPI == EPI_STORE_F32) {
-                static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = v[i];
-                if (with_ln) {
-                    const float x = (v[i] - s_mu[j]) * next_gain;
-                    const bf16 hi = __float2bfloat16_rn(x);
-                    a.e.ln.hi[(size_t)j * a.e.ldo + n] = hi;
-                    a.e.ln.lo[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
-                }
-            } else if (EPI == EPI_GELU) {
-                const float gv = gelu_bf16_out(v[i]);
-                if (a.e.out_lo) {
-                    const bf16 hi = __float2bfloat16_rn(gv);
-                    static_cast<bf16*>(a.e.out)[(size_t)j * a.e.ldo + n] = hi;
-                    static_cast<bf16*>(a.e.out_lo)[(size_t)j * a.e.ldo + n] = __float2bfloat16_rn(gv - __bfloat162float(hi));
-                } else {
-                    static_cast<float*>(a.e.out)[(size_t)j * a.e.ldo + n] = gv;
-                }
-            } else {
-                sc.base[(sc.is_q ? (long long)j * a.e.ldo : s_rowoff[j]) + sc.col] = __float2bfloat16_rn(v[i]);
-            }
-        }
-        if (with_ln && n_group > 0) {        // (warp-uniform) statistics for the next LayerNorm, as in the decode passes' epilogue
-#pragma unroll
-            for (int s0 = 0; s0 < 16; s0 += 4) {
-                if (c0 + s0 >= a.rows) break;
-                float sums[8], ref[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    ref[k] = __shfl_sync(0xffffffffu, v[s0 + k], 0);
-                    const float dv = valid ? v[s0 + k] - ref[k] : 0.f;
-                    sums[2 * k] = dv;
-                    sums[2 * k + 1] = dv * dv;
-                }
-                const float mine = warp_sum_many<8>(sums, lane);
-                const float sd = __shfl_sync(0xffffffffu, mine, lane & ~7), sq = __shfl_sync(0xffffffffu, mine, (lane & ~7) + 4);
-                const int k = lane >> 3, j = c0 + s0 + k;
-                if ((lane & 7) == 0 && j < a.rows) {
-                    const float rf = k == 0 ? ref[0] : (k == 1 ? ref[1] : (k == 2 ? ref[2] : ref[3]));
-                    a.e.ln.stats[(size_t)j * a.e.ln.groups + ((seg_base + n_local0 + warp * 32) >> 5)] = make_float2(fmaf(sd, inv, rf), fmaxf(fmaf(-sd * inv, sd, sq), 0.f));
-                }
-            }
-        }
-    }
-    tc_fence_before_sync();
-    asm volatile("bar.arrive 2, 160;" ::: "memory");   // the accumulator has been read: warp 5 may free the TMEM columns
-    if (EPI == EPI_SCORE) {                  // two threads share a row
-        bar_sync(1, 128);
-        const int half = tid & 1, r = tid >> 1;
-        if (r >= a.rows) return;             // (the pair of a row's threads leaves together)
-        const float* row = tile_v + r * LD + half;
-        const int t_loc = a.truth[r] - (seg_base + n_local0);
-        float bv = -INFINITY, z = 0.f;
-        int bi = INT_MAX;
-#pragma unroll 8
-        for (int i = 0; i < 64; ++i) if (row[2 * i] > bv) { bv = row[2 * i]; bi = 2 * i + half; }
-        const uint32_t both = 3u << (lane & ~1);
-        const float ov = __shfl_xor_sync(both, bv, 1);
-        const int oi = __shfl_xor_sync(both, bi, 1);
-        if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-#pragma unroll 8
-        for (int i = 0; i < 64; ++i) z += expf(row[2 * i] - bv);
-        z += __shfl_xor_sync(both, z, 1);
-        if (half == 0) {
-            a.amax_val[(size_t)r * a.amax_stride + tile] = bv;
-            a.amax_idx[(size_t)r * a.amax_stride + tile] = bi == INT_MAX ? INT_MAX : seg_base + n_local0 + bi;
-            a.score_sum[(size_t)r * a.amax_stride + tile] = z;
-            if (t_loc >= 0 && t_loc < 128 && n_local0 + t_loc < seg_rows) a.truth_val[r] = tile_v[r * LD + t_loc];
-        }
-    }
-}
-
-// grid: (tiles * splits CTAs in clusters of `splits` (the K-slices of one tile), groups of NB token rows); dynamic smem
-// TcdCfg::SMEM_BYTES.  PASS (all rows of a teacher-forced pass, splits == 1): a.rows counts the rows of all groups; the groups behind
-// the first find the weights in L2.  Bound by the operands' way from L2 into the multiprocessors (33 KB per 64 of K and group of
-// 64 rows), two CTAs on each, one of them in its epilogue.
-template <int NB, int PRO, int EPI, bool PASS = false>
 __global__ void __launch_bounds__(TCD_THREADS)
-gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
+gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
                       const __grid_constant__ CUtensorMap tm2, const __grid_constant__ CUtensorMap tmx,
                       const __grid_constant__ CUtensorMap tml) {
     constexpr bool LNT = PRO == PRO_LNT, BY_TMA = PRO == PRO_TMA || LNT;   // BY_TMA: the token rows are loaded beside the weights
     using C = TcdCfg<NB, LNT>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    TcDecodeArgs group = a0;
-    if (PASS) tcd_shift_rows<PRO, EPI>(group, blockIdx.y * NB, min(NB, a0.rows - (int)blockIdx.y * NB));
-    const TcDecodeArgs& a = PASS ? group : a0;
     __shared__ __align__(8) uint64_t s_full[C::STAGES];
     __shared__ __align__(8) uint64_t s_empty[C::STAGES];
     __shared__ __align__(8) uint64_t s_accum;
@@ -333,7 +192,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
     const int rpc = S == 1 ? a.rows : (a.rows + S - 1) / S;
     const int j_first = S == 1 ? 0 : sp * rpc;
     const int j_count = max(0, min(rpc, a.rows - j_first));
-    float hres[EPI == EPI_RESID && !PASS ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
+    float hres[EPI == EPI_RESID ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
     float next_gain = 0.f;                   // EPI_RESID: gain of the LayerNorm that follows, at this thread's feature (a parameter)
     int my_seq = 0, my_pos = 0;              // EPI_QKV / EPI_KV, threads below a.rows: this token row's sequence and position
 
@@ -474,7 +333,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
         const int nl = n_local0 + tid;
 #pragma unroll
         for (int s = 0; s < NB; ++s) {
-            if (PASS || s >= j_count) break;   // (every loop over rows leaves at the last row: the unrolled rest is never fetched)
+            if (s >= j_count) break;   // (every loop over rows leaves at the last row: the unrolled rest is never fetched)
             hres[s] = nl < seg_rows ? __ldcg(hp + (size_t)(j_first + s) * a.e.ldo + seg_base + nl) : 0.f;
         }
         if (a.e.ln.gain && tid < j_count) s_mu[tid] = __ldcg(a.e.ln.ref + j_first + tid);   // (published by the barrier ahead of the epilogue)
@@ -657,10 +516,6 @@ gemm_tc_decode_kernel(const TcDecodeArgs a0, const __grid_constant__ CUtensorMap
     }
 
     // ---- epilogue: warps 0-3 own TMEM lanes 32 * warp .. +31 = output features of the tile ----
-    if constexpr (PASS) {
-        tcd_pass_epilogue<NB, PRO, EPI>(a, tmem, seg, seg_rows, seg_base, n_local0, tile, ring, s_mu, s_rstd, s_rowoff, &s_accum, next_gain, my_seq, my_pos, poll_limit, nkb > C::STAGES);
-        return;
-    }
     float v[NB];
     const int tl = warp * 32 + lane;
     ScatterCol sc;
@@ -860,25 +715,68 @@ struct TcTiledArgs {
     int tiles_n, tiles_m;    // feature tiles over all segments, row tiles (of 256 in the pair kernel, else 128)
     int splits;              // gemm_tc_split_kernel: CTAs that share a tile's K range
     int whole, parts;        // gemm_tc_pair_kernel: tiles done whole; parts that each of the remaining ones is cut into (1, 2, 4)
+    int lo_row;              // PL: row of the remainder plane's first row in the token rows' tensor map
     int* err_flag;
+    float* tile_max; int* tile_idx; float* tile_sum;   // EPI_SCORE: [M][tile_stride]
+    int tile_stride;
+    const int* truth; float* truth_val;                // EPI_SCORE: [M] the feature whose value goes to truth_val
     EpiArgs e;
 };
 
 constexpr int TCT_TILE_BYTES = 128 * 128;          // 128 rows x 64 bf16
 constexpr int TCP_THREADS = 320;   // warps 0-7: epilogue, two per 32 rows; warp 8: TMA; warp 9: TMEM + MMA issue
 constexpr int TCP_BN = 256;                           // output features per tile
-constexpr int TCP_STAGES = 6;
-constexpr int TCP_STAGE_BYTES = 2 * TCT_TILE_BYTES;   // this CTA's token rows, its half of the weight rows
-constexpr int TCP_SMEM_BYTES = TCP_STAGES * TCP_STAGE_BYTES + 1024;
+// PL: the token rows are two bf16 planes (values, remainders; fp32 rows to about 16 bits), both multiplied with the same weight tile into
+// the same accumulator: a K-block brings 48 KB for twice the products.
+template <bool PL> struct TcpCfg {
+    static constexpr int STAGES = PL ? 4 : 6;
+    static constexpr int W_AT = (PL ? 2 : 1) * TCT_TILE_BYTES;          // this CTA's token rows, then its half of the weight rows
+    static constexpr int STAGE_BYTES = W_AT + TCT_TILE_BYTES;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+};
 constexpr int TCP_GROUP_M = 8;                        // row tiles that share a sweep over the weights, see tcp_item
 
-// Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.
-template <int EPI>
+// EPI_SCORE: SCORE_TILE features of one row from its TMEM lane; n0: the first of them, valid: how many exist.  Warp-wide loads.
+__device__ __forceinline__ void score_tile(const TcTiledArgs& a, uint32_t acc, int m, int n0, int valid) {
+    float v[SCORE_TILE];
+#pragma unroll
+    for (int i = 0; i < SCORE_TILE; i += 16) {
+        float t[16];
+        tmem_ld16(acc + i, t);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[i + u] = i + u < valid ? t[u] : -INFINITY;
+    }
+    if (m >= a.M || valid <= 0) return;
+    float best = -INFINITY, z = 0.f, true_v = 0.f;
+    int bi = -1;
+    const int truth = a.truth[m] - n0;
+#pragma unroll
+    for (int i = 0; i < SCORE_TILE; ++i) {
+        if (v[i] > best) { best = v[i]; bi = i; }
+        if (i == truth) true_v = v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < SCORE_TILE; ++i) z += expf(v[i] - best);
+    const size_t o = (size_t)m * a.tile_stride + n0 / SCORE_TILE;
+    a.tile_max[o] = best;
+    a.tile_idx[o] = bi < 0 ? INT_MAX : n0 + bi;
+    a.tile_sum[o] = z;
+    if (truth >= 0 && truth < valid && truth < SCORE_TILE) a.truth_val[m] = true_v;
+}
+
+// Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.  PL with EPI_GELU: to two planes.
+template <int EPI, bool PL>
 __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int seg, int seg_base, int seg_rows, int n_local0, size_t row_off, const float (&v)[16]) {
     const int n0 = seg_base + n_local0;
     if (n_local0 + 16 > seg_rows || (e.ldo & 7) || (seg_rows & 7)) {
         for (int i = 0; i < 16; ++i)
-            if (n_local0 + i < seg_rows) epilogue<bf16, EPI>(e, m, n0 + i, v[i]);
+            if (n_local0 + i < seg_rows) {
+                epilogue<bf16, EPI>(e, m, n0 + i, v[i]);
+                if (EPI == EPI_GELU && PL) {
+                    const float g = gelu_bf16_out(v[i]);
+                    static_cast<bf16*>(e.out_lo)[(size_t)m * e.ldo + n0 + i] = __float2bfloat16_rn(g - __bfloat162float(__float2bfloat16_rn(g)));
+                }
+            }
         return;
     }
     if (EPI == EPI_STORE_F32 || EPI == EPI_RESID) {
@@ -892,7 +790,16 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int seg, int
         return;
     }
     uint4 lo, hi;
-    if (EPI == EPI_GELU) {
+    if (EPI == EPI_GELU && PL) {
+        uint4 rlo, rhi;
+        split_bf16x2(gelu_bf16_out(v[0]), gelu_bf16_out(v[1]), lo.x, rlo.x); split_bf16x2(gelu_bf16_out(v[2]), gelu_bf16_out(v[3]), lo.y, rlo.y);
+        split_bf16x2(gelu_bf16_out(v[4]), gelu_bf16_out(v[5]), lo.z, rlo.z); split_bf16x2(gelu_bf16_out(v[6]), gelu_bf16_out(v[7]), lo.w, rlo.w);
+        split_bf16x2(gelu_bf16_out(v[8]), gelu_bf16_out(v[9]), hi.x, rhi.x); split_bf16x2(gelu_bf16_out(v[10]), gelu_bf16_out(v[11]), hi.y, rhi.y);
+        split_bf16x2(gelu_bf16_out(v[12]), gelu_bf16_out(v[13]), hi.z, rhi.z); split_bf16x2(gelu_bf16_out(v[14]), gelu_bf16_out(v[15]), hi.w, rhi.w);
+        uint4* r = reinterpret_cast<uint4*>(static_cast<bf16*>(e.out_lo) + (size_t)m * e.ldo + n0);
+        r[0] = rlo;
+        r[1] = rhi;
+    } else if (EPI == EPI_GELU) {
         lo.x = pack_bf16x2(gelu_bf16_out(v[0]), gelu_bf16_out(v[1])); lo.y = pack_bf16x2(gelu_bf16_out(v[2]), gelu_bf16_out(v[3]));
         lo.z = pack_bf16x2(gelu_bf16_out(v[4]), gelu_bf16_out(v[5])); lo.w = pack_bf16x2(gelu_bf16_out(v[6]), gelu_bf16_out(v[7]));
         hi.x = pack_bf16x2(gelu_bf16_out(v[8]), gelu_bf16_out(v[9])); hi.y = pack_bf16x2(gelu_bf16_out(v[10]), gelu_bf16_out(v[11]));
@@ -962,7 +869,7 @@ __device__ __forceinline__ void tcp_item(const TcTiledArgs& a, int item, int& ti
 // its feature within the segment.  A thread moves whole 32-byte sectors of its row (with 16-byte accesses the residual
 // add fetched every sector of the stream twice).  The residual add has its first 64 old values in flight before the accumulator
 // is awaited, which `wait` does.
-template <int EPI, typename Wait>
+template <int EPI, bool PL, typename Wait>
 __device__ __forceinline__ void tcp_epilogue(const TcTiledArgs& a, uint32_t acc, int m, int seg, int seg_base, int seg_rows, int n_local0, int CW, Wait wait) {
     if (EPI == EPI_RESID && n_local0 + CW <= seg_rows && (a.e.ldo & 7) == 0 && (seg_base & 7) == 0) {
         float* prow = static_cast<float*>(a.e.out) + (size_t)min(m, a.M - 1) * a.e.ldo + seg_base + n_local0;
@@ -995,11 +902,16 @@ __device__ __forceinline__ void tcp_epilogue(const TcTiledArgs& a, uint32_t acc,
     }
     const size_t row_off = cache_row_offset<EPI>(a.e, m, a.M);
     if (!wait()) return;
+    if constexpr (EPI == EPI_SCORE) {   // (one segment, whole tiles)
+#pragma unroll 1
+        for (int c = 0; c < CW; c += SCORE_TILE) score_tile(a, acc + c, m, n_local0 + c, seg_rows - (n_local0 + c));
+        return;
+    }
 #pragma unroll 1
     for (int c = 0; c < CW; c += 16) {
         float v[16];
         tmem_ld16(acc + c, v);   // warp-wide: every lane takes part
-        if (m < a.M && n_local0 + c < seg_rows) epilogue16<EPI>(a.e, m, seg, seg_base, seg_rows, n_local0 + c, row_off, v);
+        if (m < a.M && n_local0 + c < seg_rows) epilogue16<EPI, PL>(a.e, m, seg, seg_base, seg_rows, n_local0 + c, row_off, v);
     }
 }
 
@@ -1012,16 +924,17 @@ __device__ __forceinline__ void tcp_epilogue(const TcTiledArgs& a, uint32_t acc,
 // (1387 TFLOP/s), 8191 x 11008 x 4096 with GELU 585 -> 555 us, 8191 x 4096 x 11008 with the residual add 628 -> 579 us,
 // 12280 x 2048 x 2048 with the residual add 156 -> 108 us.
 // tmh*: the weights in boxes of 32 rows, for the parts of tiles.
-// grid: 2 * min(items, SMs / 2) in clusters of two; dynamic smem TCP_SMEM_BYTES.
-template <int EPI>
+// grid: 2 * min(items, SMs / 2) in clusters of two; dynamic smem TcpCfg::SMEM_BYTES.
+template <int EPI, bool PL>
 __global__ void __launch_bounds__(TCP_THREADS)
 gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
                     const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2,
                     const __grid_constant__ CUtensorMap tmh0, const __grid_constant__ CUtensorMap tmh1, const __grid_constant__ CUtensorMap tmh2) {
+    using C = TcpCfg<PL>;
     constexpr int BN = TCP_BN;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_full[TCP_STAGES];    // first CTA: both CTAs' loads of a stage
-    __shared__ __align__(8) uint64_t s_empty[TCP_STAGES];
+    __shared__ __align__(8) uint64_t s_full[C::STAGES];    // first CTA: both CTAs' loads of a stage
+    __shared__ __align__(8) uint64_t s_empty[C::STAGES];
     __shared__ __align__(8) uint64_t s_acc_full[2], s_acc_free[2];
     __shared__ uint32_t s_tmem;
 
@@ -1033,7 +946,7 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
 
     if (warp == 9) {
         if (lane == 0) {
-            for (int s = 0; s < TCP_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            for (int s = 0; s < C::STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
             for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&s_acc_full[s]), 1); mbar_init(smem_u32(&s_acc_free[s]), 16); }   // free: one arrive per epilogue warp of the pair
             mbar_init_fence();
         }
@@ -1065,14 +978,15 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
                     break;
                 }
                 if (elect_one()) {
-                    const uint32_t bar = cluster_map(smem_u32(&s_full[st]), 0), dst = ring0 + st * TCP_STAGE_BYTES;
-                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&s_full[st]), 2 * TCT_TILE_BYTES + width * 128);
-                    tma_load_2d_pair(dst, &tmx, i * 64, m0, bar);                     // rows past the end arrive as zeros
-                    if (width == BN) tma_load_2d_pair(dst + TCT_TILE_BYTES, tw, i * 64, n0, bar);
+                    const uint32_t bar = cluster_map(smem_u32(&s_full[st]), 0), dst = ring0 + st * C::STAGE_BYTES;
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&s_full[st]), 2 * C::W_AT + width * 128);
+                    tma_load_2d_pair(dst, &tmx, i * 64, m0, bar);                     // rows past the end arrive as zeros (PL: or as another plane's, and are not used)
+                    if (PL) tma_load_2d_pair(dst + TCT_TILE_BYTES, &tmx, i * 64, a.lo_row + m0, bar);
+                    if (width == BN) tma_load_2d_pair(dst + C::W_AT, tw, i * 64, n0, bar);
                     else
-                        for (int q = 0; q < width / 2; q += 32) tma_load_2d_pair(dst + TCT_TILE_BYTES + q * 128, th, i * 64, n0 + q, bar);
+                        for (int q = 0; q < width / 2; q += 32) tma_load_2d_pair(dst + C::W_AT + q * 128, th, i * 64, n0 + q, bar);
                 }
-                if (++st == TCP_STAGES) { st = 0; ++round; }
+                if (++st == C::STAGES) { st = 0; ++round; }
             }
         }
         pdl_launch_dependents();
@@ -1099,13 +1013,17 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
                     }
                     tc_fence_after_sync();
                     if (elect_one()) {
-                        const uint64_t da = umma_desc_k_sw128(ring0 + st * TCP_STAGE_BYTES);
-                        const uint64_t db = umma_desc_k_sw128(ring0 + st * TCP_STAGE_BYTES + TCT_TILE_BYTES);
+                        const uint64_t da = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES);
+                        const uint64_t db = umma_desc_k_sw128(ring0 + st * C::STAGE_BYTES + C::W_AT);
 #pragma unroll
                         for (int k = 0; k < 4; ++k) umma_bf16_pair(tmem + buf * BN, da + 2 * k, db + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
+                        if (PL) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) umma_bf16_pair(tmem + buf * BN, da + TCT_TILE_BYTES / 16 + 2 * k, db + 2 * k, idesc, 1u);
+                        }
                         umma_commit_pair(smem_u32(&s_empty[st]));
                     }
-                    if (++st == TCP_STAGES) { st = 0; ++round; }
+                    if (++st == C::STAGES) { st = 0; ++round; }
                 }
                 if (elect_one()) umma_commit_pair(smem_u32(&s_acc_full[buf]));   // (also after a failed wait: the epilogue warps must not be left waiting)
             }
@@ -1131,7 +1049,7 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
             };
             const int m = tile_m * 256 + rank * 128 + (warp & 3) * 32 + lane;   // output row = TMEM lane
             const uint32_t acc = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + buf * BN + col;
-            tcp_epilogue<EPI>(a, acc, m, seg, seg_base, seg_rows, n_local0 + c0 + col, width / 2, wait);
+            tcp_epilogue<EPI, PL>(a, acc, m, seg, seg_base, seg_rows, n_local0 + c0 + col, width / 2, wait);
             if (!ok) break;
             tc_fence_before_sync();   // this warp's TMEM reads are done: the accumulator may be overwritten
             __syncwarp();
@@ -1153,29 +1071,33 @@ gemm_tc_pair_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx
 // cluster barrier after the last product says that every ring is free.  That keeps a CTA at 97 KB, so that the next kernel's
 // CTAs sit beside it with their first weights loaded (with an inbox of its own a CTA of four took 176 KB, and every kernel
 // began with a cold start after the one before).  One tile per cluster.
-// grid: tiles * S; dynamic smem TCS_SMEM_BYTES.
+// grid: tiles * S; dynamic smem TcsCfg::SMEM_BYTES.
 constexpr int TCS_THREADS = 320;   // warps 0-7: epilogue; warp 8: TMA; warp 9: TMEM + MMA issue
 constexpr int TCS_BN = 128;
-constexpr int TCS_STAGES = 3;
-constexpr int TCS_STAGE_BYTES = 2 * TCT_TILE_BYTES;
-constexpr int TCS_SMEM_BYTES = TCS_STAGES * TCS_STAGE_BYTES + 1024;
-static_assert(2 * (TCS_SMEM_BYTES + 1024 + 1024) <= 227 * 1024, "two CTAs per SM");
-static_assert(3 * (128 * TCS_BN * 4 / 4) <= TCS_STAGES * TCS_STAGE_BYTES && 128 * TCS_BN * 4 / 2 <= TCS_STAGES * TCS_STAGE_BYTES, "the inbox fits where the ring was");
+template <bool PL> struct TcsCfg {
+    static constexpr int STAGES = PL ? 2 : 3;
+    static constexpr int W_AT = (PL ? 2 : 1) * TCT_TILE_BYTES;
+    static constexpr int STAGE_BYTES = W_AT + TCT_TILE_BYTES;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+    static_assert(2 * (SMEM_BYTES + 1024 + 1024) <= 227 * 1024, "two CTAs per SM");
+    static_assert(3 * (128 * TCS_BN * 4 / 4) <= STAGES * STAGE_BYTES && 128 * TCS_BN * 4 / 2 <= STAGES * STAGE_BYTES, "the inbox fits where the ring was");
+};
 
-template <int EPI>
+template <int EPI, bool PL>
 __global__ void __launch_bounds__(TCS_THREADS)
 gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tm0,
                      const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2) {
+    using C = TcsCfg<PL>;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t s_full[TCS_STAGES];
-    __shared__ __align__(8) uint64_t s_empty[TCS_STAGES];
+    __shared__ __align__(8) uint64_t s_full[C::STAGES];
+    __shared__ __align__(8) uint64_t s_empty[C::STAGES];
     __shared__ __align__(8) uint64_t s_accum, s_inbox;
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t ring0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const int S = a.splits;
-    constexpr int stages = TCS_STAGES;
+    constexpr int stages = C::STAGES;
     const int tile = blockIdx.x / S, sp = blockIdx.x - tile * S;           // sp = this CTA's rank in its cluster
     int n_local0;
     const int seg = tct_segment(a, tile % a.tiles_n, TCS_BN, n_local0);
@@ -1187,7 +1109,7 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
 
     if (warp == 9) {
         if (lane == 0) {
-            for (int s = 0; s < TCS_STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+            for (int s = 0; s < C::STAGES; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
             mbar_init(smem_u32(&s_accum), 1);
             mbar_init(smem_u32(&s_inbox), 1);
             mbar_init_fence();
@@ -1208,21 +1130,25 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             tma_prefetch_desc(tw);
             for (int i = 0; i < n_pre; ++i) {
                 const uint32_t bar = smem_u32(&s_full[i]);
-                mbar_arrive_expect_tx(bar, TCS_STAGE_BYTES);
-                tma_load_2d_nohint(ring0 + i * TCS_STAGE_BYTES + TCT_TILE_BYTES, tw, (kb0 + i) * 64, n_local0, bar);
+                mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
+                tma_load_2d_nohint(ring0 + i * C::STAGE_BYTES + C::W_AT, tw, (kb0 + i) * 64, n_local0, bar);
             }
         }
         pdl_wait();
         if (elect_one())
-            for (int i = 0; i < n_pre; ++i) tma_load_2d_nohint(ring0 + i * TCS_STAGE_BYTES, &tmx, (kb0 + i) * 64, m0, smem_u32(&s_full[i]));
+            for (int i = 0; i < n_pre; ++i) {
+                tma_load_2d_nohint(ring0 + i * C::STAGE_BYTES, &tmx, (kb0 + i) * 64, m0, smem_u32(&s_full[i]));
+                if (PL) tma_load_2d_nohint(ring0 + i * C::STAGE_BYTES + TCT_TILE_BYTES, &tmx, (kb0 + i) * 64, a.lo_row + m0, smem_u32(&s_full[i]));
+            }
         int st = 0, round = 0;
         for (int i = n_pre; i < nkb; ++i) {
             if (!mbar_wait_warp(smem_u32(&s_empty[st]), (uint32_t)round & 1)) { tc_report(a.err_flag, TC_ERR_SLOT); break; }
             if (elect_one()) {
-                const uint32_t bar = smem_u32(&s_full[st]), dst = ring0 + st * TCS_STAGE_BYTES;
-                mbar_arrive_expect_tx(bar, TCS_STAGE_BYTES);
+                const uint32_t bar = smem_u32(&s_full[st]), dst = ring0 + st * C::STAGE_BYTES;
+                mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
                 tma_load_2d_nohint(dst, &tmx, (kb0 + i) * 64, m0, bar);
-                tma_load_2d_nohint(dst + TCT_TILE_BYTES, tw, (kb0 + i) * 64, n_local0, bar);
+                if (PL) tma_load_2d_nohint(dst + TCT_TILE_BYTES, &tmx, (kb0 + i) * 64, a.lo_row + m0, bar);
+                tma_load_2d_nohint(dst + C::W_AT, tw, (kb0 + i) * 64, n_local0, bar);
             }
             if (++st == stages) { st = 0; ++round; }
         }
@@ -1238,8 +1164,9 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             const int done = st;
             if (++st == stages) { st = 0; phase ^= 1; }
             if (i + 1 < nkb) ok = mbar_test(smem_u32(&s_full[st]), phase);
-            umma_bf16_k64(tmem, umma_desc_k_sw128(ring0 + done * TCS_STAGE_BYTES), umma_desc_k_sw128(ring0 + done * TCS_STAGE_BYTES + TCT_TILE_BYTES),
-                          idesc, i != 0 ? 1u : 0u);
+            const uint64_t dx = umma_desc_k_sw128(ring0 + done * C::STAGE_BYTES), dw = umma_desc_k_sw128(ring0 + done * C::STAGE_BYTES + C::W_AT);
+            umma_bf16_k64(tmem, dx, dw, idesc, i != 0 ? 1u : 0u);
+            if (PL) umma_bf16_k64(tmem, dx + TCT_TILE_BYTES / 16, dw, idesc, 1u);
             umma_commit_one(smem_u32(&s_empty[done]));
         }
         umma_commit_one(smem_u32(&s_accum));
@@ -1289,6 +1216,9 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
             if (!mbar_wait(ibar, 0)) tc_report(a.err_flag, TC_ERR_EXCHANGE);
         }
         const float4* inbox = reinterpret_cast<const float4*>(smem_dyn + (inbox0 - smem_u32(smem_dyn)));
+        if constexpr (EPI == EPI_SCORE) {   // (one segment, S == 1)
+            score_tile(a, acc + c_first, m, n_local0 + c_first, seg_rows - (n_local0 + c_first));
+        } else
 #pragma unroll 1
         for (int c0 = c_first; c0 < c_end; c0 += 16) {
             float v[16];
@@ -1322,7 +1252,7 @@ gemm_tc_split_kernel(const TcTiledArgs a, const __grid_constant__ CUtensorMap tm
                     continue;
                 }
             }
-            if (m < a.M && n_local < seg_rows) epilogue16<EPI>(a.e, m, seg, seg_base, seg_rows, n_local, row_off, v);
+            if (m < a.M && n_local < seg_rows) epilogue16<EPI, PL>(a.e, m, seg, seg_base, seg_rows, n_local, row_off, v);
         }
         tc_fence_before_sync();
     }

@@ -276,16 +276,28 @@ __device__ __forceinline__ void ln_store4(bf16* orow, int k4, float y0, float y1
     const __nv_bfloat162 lo = __floats2bfloat162_rn(y0, y1), hi = __floats2bfloat162_rn(y2, y3);
     reinterpret_cast<uint2*>(orow)[k4] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
+// The same as value + remainder, the remainder `lo` elements behind the value (lo == 0: the value alone).
+template <bool PL, typename TO>
+__device__ __forceinline__ void ln_put4(TO* orow, size_t lo, int k4, float y0, float y1, float y2, float y3) {
+    if constexpr (PL) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(y0, y1), b = __floats2bfloat162_rn(y2, y3);
+        reinterpret_cast<uint2*>(orow)[k4] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+        ln_store4(orow + lo, k4, y0 - __low2float(a), y1 - __high2float(a), y2 - __low2float(b), y3 - __high2float(b));
+    } else {
+        ln_store4(orow, k4, y0, y1, y2, y3);
+    }
+}
 // LayerNorm of fp32 rows (biased variance, eps 1e-5) ahead of the GEMMs, output in the storage type: the row sits in
 // registers between the passes (up to 4096 elements), loads and stores are 16 bytes wide (8191 rows of 4096: 56 us with
 // scalar accesses in three passes).  raw (nullable): bf16 copy of the row as it is, for the FF_Tandem projection that reads
 // the same residual stream (a pass of its own over it took 120 us there).  A block keeps gain and bias in registers over its
 // rows and fetches a row ahead: with one row per block those 32 KB per 16 KB of row made the L2 traffic (51 us at 8191 rows).
+// PL (TO = bf16): output and raw copy as two planes, values and, `lo` elements behind them, remainders.
 // grid: at most M blocks; block: 128; d % 4 == 0.
-template <typename TO>
+template <typename TO, bool PL = false>
 __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __restrict__ x, const float* __restrict__ gain,
                                                              const float* __restrict__ bias, TO* __restrict__ out, int d,
-                                                             int M, bf16* raw) {
+                                                             int M, bf16* raw, size_t lo = 0) {
     __shared__ float red[4];
     const int d4 = d >> 2;
     if (d4 <= 8 * 128) {
@@ -315,7 +327,7 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
             if (raw) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
-                    if (threadIdx.x + 128 * u < d4) ln_store4(raw + (size_t)row * d, threadIdx.x + 128 * u, t[u].x, t[u].y, t[u].z, t[u].w);
+                    if (threadIdx.x + 128 * u < d4) ln_put4<PL>(raw + (size_t)row * d, lo, threadIdx.x + 128 * u, t[u].x, t[u].y, t[u].z, t[u].w);
             }
             float s = 0.f;
 #pragma unroll
@@ -335,7 +347,7 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
                 const int k4 = threadIdx.x + 128 * u;
                 if (k4 < d4) {
                     const float4 g = gq[u], b = bq[u];
-                    ln_store4(orow, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
+                    ln_put4<PL>(orow, lo, k4, (t[u].x - mu) * rs * g.x + b.x, (t[u].y - mu) * rs * g.y + b.y,
                               (t[u].z - mu) * rs * g.z + b.z, (t[u].w - mu) * rs * g.w + b.w);
                 }
             }
@@ -350,7 +362,7 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
             for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
                 const float4 t = __ldcg(xr + k4);
                 s += (t.x + t.y) + (t.z + t.w);
-                if (raw) ln_store4(raw + (size_t)row * d, k4, t.x, t.y, t.z, t.w);
+                if (raw) ln_put4<PL>(raw + (size_t)row * d, lo, k4, t.x, t.y, t.z, t.w);
             }
             const float mu = block_sum_128(s, red) / d;
             float q = 0.f;
@@ -363,24 +375,25 @@ __global__ void __launch_bounds__(128) layernorm_rows_kernel(const float* __rest
             for (int k4 = threadIdx.x; k4 < d4; k4 += 128) {
                 const float4 t = __ldcg(xr + k4);
                 const float4 g = __ldg(reinterpret_cast<const float4*>(gain) + k4), b = __ldg(reinterpret_cast<const float4*>(bias) + k4);
-                ln_store4(orow, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
+                ln_put4<PL>(orow, lo, k4, (t.x - mu) * rs * g.x + b.x, (t.y - mu) * rs * g.y + b.y, (t.z - mu) * rs * g.z + b.z,
                           (t.w - mu) * rs * g.w + b.w);
             }
         }
     }
 }
 
-// bf16 copy of the residual stream for a projection that no LayerNorm of the large model follows.  n a multiple of 8.
+// bf16 copy of the residual stream for a projection that no LayerNorm of the large model follows.  n a multiple of 8.  PL: two planes,
+// the remainders `lo` elements behind the values.
 // grid: enough blocks of 256 for n / 8.
-__global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ x, bf16* __restrict__ out, size_t n) {
+template <bool PL>
+__global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ x, bf16* __restrict__ out, size_t n, size_t lo) {
     pdl_wait();
     pdl_launch_dependents();
     const size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 8;
     if (i >= n) return;
     const float4 a = __ldcg(reinterpret_cast<const float4*>(x + i)), b = __ldcg(reinterpret_cast<const float4*>(x + i) + 1);
-    const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w), p2 = __floats2bfloat162_rn(b.x, b.y), p3 = __floats2bfloat162_rn(b.z, b.w);
-    *reinterpret_cast<uint4*>(out + i) = make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
-                                                    *reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
+    ln_put4<PL>(out + i, lo, 0, a.x, a.y, a.z, a.w);
+    ln_put4<PL>(out + i, lo, 1, b.x, b.y, b.z, b.w);
 }
 
 // Arg-max of fp32 rows, lowest index on ties.  grid: rows; block: 256.
@@ -538,8 +551,7 @@ struct ForcedRows {
 // computed and ignored), and, with one block more than rows, the attention groups and the sequences' loop state.
 // grid: rows (+ 1); block: 128.
 __global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRows f, const bf16* __restrict__ emb, const bf16* __restrict__ pos,
-                                                          float* __restrict__ h, int d, NextLn ln, int ticket, int router_ticket) {
-    __shared__ float s_red[4];
+                                                          float* __restrict__ h, int d, int ticket, int router_ticket) {
     __shared__ int s_cnt[128];
     pdl_wait();
     pdl_launch_dependents();
@@ -574,11 +586,11 @@ __global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRo
         f.truth[m] = p + 1 < len ? f.ids[o + p + 1] : -1;
         f.out[m] = p + 1 < len ? o - lo + p : -1;
     }
-    embed_row<bf16, 128, true>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, ln, m, s_red);
+    embed_row<bf16, 128, false>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0, nullptr);
 }
 
 // Scores of rows whose output head left (maximum, its index, sum of exponentials) per tile of features and the true token's
-// logit: negative log-likelihood and arg-max (lowest index on ties).  One warp per row; n_tiles values each, 250 at 32000 logits.
+// logit: negative log-likelihood and arg-max (lowest index on ties).  One warp per row; n_tiles values each, 500 at 32000 logits.
 // grid: ceil(rows / 8); block: 256.
 __global__ void __launch_bounds__(256) score_tiles_kernel(int rows, int n_tiles, const float* __restrict__ tile_max, const int* __restrict__ tile_idx,
                                                           const float* __restrict__ tile_sum, const float* __restrict__ truth_val,

@@ -50,7 +50,7 @@ struct Layout {   // byte offsets into the arena
     size_t st_n, st_pending, st_drafts, st_targets, st_accept, st_emitted, st_done, st_out, st_counters, st_hist;
     size_t st_block_len, st_drafting, st_confidence;
     size_t forced_ids, forced_len, forced_nll, forced_top;   // teacher-forced forward: given tokens [B][T], lengths [B], scores [B][T]
-    size_t fr_x, fr_o, fr_f, fr_q, fr_yhat, fr_a, fr_t1;
+    size_t fr_x, fr_o, fr_f, fr_q, fr_raw, fr_yhat, fr_a, fr_t1;
     size_t fr_seq, fr_truth, fr_out, fr_truth_val, fr_grp, fr_tiles, fr_kv;   // ... in one pass (bf16), see ForcedRows: offsets / lengths / first rows, next tokens, score places,
                                                                               // true logits, attention groups, the head's per-tile results, the small model's own keys / values of one layer
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
@@ -63,7 +63,7 @@ struct Layout {   // byte offsets into the arena
     size_t ln_src, ln_rows_large, ln_rows_small, ln_stats, ln_ref;   // LayerNorms behind the GEMMs (bf16 decode): sources, their rows, the token rows' statistics, reference values (see ln_ref_of)
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
-    int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles;
+    int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles, score_tiles;
     int fr_rows, fr_head_rows;               // rows of a teacher-forced pass, and of one run of its output head
     size_t kv_large_layer, kv_small_layer;   // elements per (layer, k-or-v)
 };
@@ -130,11 +130,10 @@ struct tandem_ctx {
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
     std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
-    // Activations as two bf16 planes (values, then remainders, `rows` rows each) that the consuming GEMM loads by
-    // TMA: places and maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
-    // 1 small], 16-row boxes; and the place of the queries.  One set for the decode passes, one for teacher-forced passes (in the prompt pass's buffers).
-    struct PlaneSet { size_t at[3], q; int rows; CUtensorMap xmap[3][2]; } dec_planes, fr_planes;
-    const PlaneSet* planes = &dec_planes;   // of the pass that is being enqueued
+    // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
+    // TMA: maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
+    // 1 small], 16-row boxes.
+    CUtensorMap xmap[3][2];
     CUtensorMap lnmap[2];                // the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one)
     std::vector<CUtensorMap> kmap, vmap; // the large model's key / value cache of each layer as [(seq, head, position)][d_head]
     cudaStream_t side = nullptr;         // the decode-time FF_Tandem projections run here, beside the large model's later layers
@@ -248,11 +247,14 @@ Layout make_layout(const tandem_config& c) {
     // share the place of the GELU outputs, which are dead from the end of a layer to the first product of the next one's FFN.
     const size_t ws_end = off;
     off = ws;
-    L.fr_x = take(RF * dmax * 4); L.fr_o = take(RF * dmax * 4); L.fr_f = off;
-    L.fr_q = take(RF * dmax * 2);
+    L.fr_x = take(RF * dmax * 4); L.fr_o = take(RF * dmax * 4); L.fr_f = take(RF * fmax * 4);
+    const size_t fr_end = off;
     off = L.fr_f;
-    L.fr_yhat = take(RF * c.small.d_model * 4); L.fr_a = take(RF * c.small.d_model * 4); L.fr_t1 = take(RF * hidden * 4);
-    off = std::max(std::max(off, align_up(L.fr_f + std::max(RF * dmax * 2, RF * fmax * 4))), ws_end);
+    L.fr_raw = take(RF * c.large.d_model * 4); L.fr_t1 = take(RF * hidden * 4); L.fr_yhat = take(RF * c.small.d_model * 4); L.fr_a = take(RF * c.small.d_model * 4);
+    const size_t fr_proj_end = off;
+    off = L.fr_f;
+    L.fr_q = take(RF * dmax * 2);
+    off = std::max(std::max(off, fr_proj_end), std::max(fr_end, ws_end));
     L.logits_large = take(RD * V * 4);
     L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.part_ml = take(RD * hmax * L.n_chunks_max * 2 * 4);
@@ -272,11 +274,12 @@ Layout make_layout(const tandem_config& c) {
     L.ln_src = take((size_t)(2 * c.large.n_layers + 1 + 2 * c.small.n_layers + 1) * sizeof(LnSource));
     L.ln_rows_large = take((size_t)(2 * c.large.n_layers + 1) * 4 * c.large.d_model * 2);
     L.ln_rows_small = take((size_t)(2 * c.small.n_layers + 1) * 4 * c.small.d_model * 2);
-    L.ln_stats = take(std::max(RD, RF) * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
-    L.ln_ref = take(2 * std::max(RD, RF) * 4);
+    L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
+    L.ln_ref = take(2 * RD * 4);
     L.fr_seq = take((3 * B + 1) * 4); L.fr_truth = take(RF * 4); L.fr_out = take(RF * 4); L.fr_truth_val = take(RF * 4);
     L.fr_grp = take(2 * (RF / ATT_NQ + B + 1) * 4);
-    L.fr_tiles = take((size_t)L.fr_head_rows * L.vocab_tiles * 12);
+    L.score_tiles = cdiv(c.large.vocab, SCORE_TILE);
+    L.fr_tiles = take((size_t)L.fr_head_rows * L.score_tiles * 12);
     L.fr_kv = take(bf ? 2 * L.kv_small_layer * esz : 0);
     L.total = off;
     return L;
@@ -398,7 +401,6 @@ struct TcScratch {
     unsigned poll_limit = 0;   // 0: the kernels' default
     int withhold_weights = 0;  // test hook, see TcDecodeArgs
     int wait_first = 0;        // the launch may follow kernels that write its weights, see TcDecodeArgs
-    bool whole_pass = false;   // all rows of a pass at once, not a block that has to give the bits of its rows alone: K-slices by the number of rows
 };
 
 TcW tcw3(const tandem_ctx& c, int i0, int i1, int i2, int seg_rows0, int seg_rows, int K) {
@@ -450,7 +452,6 @@ void launch_ex(tandem_ctx& c, bool pdl, int cluster, void (*kernel)(KArgs...), d
 struct TcRows {
     const CUtensorMap* map = nullptr;
     int plane_rows = 0;                    // rows between the value and the remainder plane
-    int row0 = 0;                          // the pass's first row there
     const CUtensorMap* ln_map = nullptr;
     int ln_row = 0;                        // the LayerNorm's first row there
     const float2* ln_stats = nullptr;      // [rows][ln_groups]
@@ -459,98 +460,81 @@ struct TcRows {
     float* ln_mean = nullptr;
 };
 
-template <int NB, int PRO, int EPI, bool PASS = false>
-void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const TcRows& x, int groups = 1) {
+template <int NB, int PRO, int EPI>
+void launch_tc_decode_nb(tandem_ctx& c, const TcDecodeArgs& a, const TcW& w, int units, const TcRows& x) {
     using C = TcdCfg<NB, PRO == PRO_LNT>;
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_tc_decode_kernel<NB, PRO, EPI, PASS>, C::SMEM_BYTES, attr_done);
-    const size_t smem = PASS ? C::SMEM_BYTES_WHOLE : C::SMEM_BYTES;
-    launch_ex(c, true, a.splits, gemm_tc_decode_kernel<NB, PRO, EPI, PASS>, dim3(units, groups), dim3(TCD_THREADS), smem, a, w.tm[0], w.tm[1], w.tm[2],
+    ensure_dyn_smem(gemm_tc_decode_kernel<NB, PRO, EPI>, C::SMEM_BYTES, attr_done);
+    launch_ex(c, true, a.splits, gemm_tc_decode_kernel<NB, PRO, EPI>, dim3(units), dim3(TCD_THREADS), (size_t)C::SMEM_BYTES, a, w.tm[0], w.tm[1], w.tm[2],
               x.map ? *x.map : w.tm[0], x.ln_map ? *x.ln_map : w.tm[0]);
 }
 
-// What the output head leaves per row and tile instead of (or beside) the logits, and the teacher-forced scores' part of it.
-struct TcTiles {
-    float* val = nullptr;
-    int* idx = nullptr;
-    int stride = 0;
-    float* sum = nullptr;          // EPI_SCORE
-    const int* truth = nullptr;
-    float* truth_val = nullptr;
-};
-
 // y = prologue(x) W^T for few rows on the tensor cores, streaming W once per group of up to 64 rows (one group in
-// every benchmark configuration; more rows than that re-read the weights per group, from L2, with unchanged arithmetic).
+// every benchmark configuration; more rows than that re-read the weights per group, with unchanged arithmetic).
 template <int PRO, int EPI>
 void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx, const void* ln_g, const void* ln_b, int rows,
-                      const TcW& w, bool stream_weights, const EpiArgs& e, const TcTiles& t = TcTiles(), const TcRows& xr = TcRows()) {
+                      const TcW& w, bool stream_weights, const EpiArgs& e, float* amax_val = nullptr, int* amax_idx = nullptr,
+                      int amax_stride = 0, const TcRows& xr = TcRows()) {
     if (rows <= 0) return;
     TcDecodeArgs a;
     memset(&a, 0, sizeof(a));
     a.x = x; a.ldx = ldx; a.ln_g = static_cast<const float*>(ln_g); a.ln_b = static_cast<const float*>(ln_b);
-    a.rows = rows; a.x_row0 = xr.row0; a.x_plane_rows = xr.plane_rows;
+    a.rows = rows; a.x_plane_rows = xr.plane_rows;
     a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups; a.ln_stats = xr.ln_stats; a.ln_ref = xr.ln_ref; a.ln_mean = xr.ln_mean;
     a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.tiles0 = cdiv(w.seg_rows0, 128);
     a.seg_rows = w.seg_rows; a.tiles_per_seg = cdiv(w.seg_rows, 128);
     const int tiles = a.tiles0 + (w.n_segs - 1) * a.tiles_per_seg, KB = cdiv(w.K, 64);
-    const bool whole = EPI == EPI_SCORE || (sc.whole_pass && rows > 64);
     // K-slices per tile = cluster size: the smallest power of two that puts tiles * S CTAs at or above one per
     // multiprocessor, at most 8 and at most one per 64-element K-block; four instead of eight where those already reach a
     // quarter of the multiprocessors with slices of four K-blocks or fewer (they fit the ring, and only 15 clusters of
     // eight run beside each other before two CTAs share a multiprocessor, but 33 of four).  A layer's four GEMMs with four
     // slices in both wide ones against eight: 1024 wide, one row 12.5 -> 11.9 us, eight rows 13.9 -> 13.1; 512 wide 9.9 -> 9.5 and
     // 11.8 -> 11.4.  The residual GEMMs (a quarter of the tiles or a slice beyond the ring) are 2 to 10 % slower with four.
-    // The head GEMM keeps whole tiles, and so does a whole pass, which has a CTA per tile and 64 rows.
+    // The head GEMM keeps whole tiles.
     int S = 1;
-    if (EPI != EPI_ARGMAX && !whole)
+    if (EPI != EPI_ARGMAX)
         while (S < 8 && 2 * S <= KB && tiles * S < c.n_sms && !(S == 4 && KB <= 16 && 16 * tiles >= c.n_sms)) S *= 2;
     a.splits = S;
-    a.stream_weights = stream_weights && !whole ? 1 : 0;
+    a.stream_weights = stream_weights ? 1 : 0;
     a.err_flag = sc.err;
     a.poll_limit = sc.poll_limit;
     a.withhold_weights = sc.withhold_weights;
     a.wait_first = sc.wait_first;
     a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
-    a.amax_val = t.val; a.amax_idx = t.idx; a.amax_stride = t.stride;
-    a.score_sum = t.sum; a.truth = t.truth; a.truth_val = t.truth_val;
+    a.amax_val = amax_val; a.amax_idx = amax_idx; a.amax_stride = amax_stride;
     a.e = e;
     const double xsz = PRO == PRO_BF16 ? 2 : 4, osz = EPI == EPI_QKV || EPI == EPI_KV || EPI == EPI_STORE ? 2.0 : 4.0;
     const int units = tiles * S;
-    if constexpr (EPI == EPI_SCORE || (PRO != PRO_BF16 && PRO != PRO_LN && EPI != EPI_ARGMAX)) {
-        if (whole) {
-            ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K * cdiv(rows, 64) + rows * (w.K * xsz + a.N * osz));
-            launch_tc_decode_nb<64, PRO, EPI, true>(c, a, w, units, xr, cdiv(rows, 64));
-            return;
-        }
-    }
-    if constexpr (EPI != EPI_SCORE) {
-        for (int r0 = 0; r0 < rows; r0 += 64) {
-            const int nr = std::min(64, rows - r0);
-            TcDecodeArgs g = a;
-            tcd_shift_rows<PRO, EPI>(g, r0, nr);
-            if (r0 > 0) g.wait_first = 0;
-            ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + nr * (w.K * xsz + a.N * osz));
-            if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, g, w, units, xr);
-            else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, g, w, units, xr);
-            else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, g, w, units, xr);
-            else launch_tc_decode_nb<64, PRO, EPI>(c, g, w, units, xr);
-        }
+    for (int r0 = 0; r0 < rows; r0 += 64) {
+        const int nr = std::min(64, rows - r0);
+        TcDecodeArgs g = a;
+        tcd_shift_rows<PRO, EPI>(g, r0, nr);
+        if (r0 > 0) g.wait_first = 0;
+        ProfScope ps(c, PC_GEMM_TC_DECODE, 2.0 * a.N * w.K + nr * (w.K * xsz + a.N * osz));
+        if (nr <= 16) launch_tc_decode_nb<16, PRO, EPI>(c, g, w, units, xr);
+        else if (nr <= 32) launch_tc_decode_nb<32, PRO, EPI>(c, g, w, units, xr);
+        else if (nr <= 48) launch_tc_decode_nb<48, PRO, EPI>(c, g, w, units, xr);
+        else launch_tc_decode_nb<64, PRO, EPI>(c, g, w, units, xr);
     }
 }
 
-// y = x W^T for many rows on the tensor cores; x bf16 [M][ldx].
-template <int EPI>
-tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, const TcW& w, const EpiArgs& e, int* err) {
+// What the output head of a teacher-forced pass leaves per row and SCORE_TILE features instead of the logits.
+struct TcScore { float* val; int* idx; float* sum; int stride; const int* truth; float* truth_val; };
+
+// y = x W^T for many rows on the tensor cores; x bf16 [M][ldx].  PL: x as two planes, the remainders lo_row rows behind the values.
+template <int EPI, bool PL>
+tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, const TcW& w, const EpiArgs& e, int* err, int lo_row = 0, const TcScore& sc = TcScore()) {
     if (M <= 0) return TANDEM_OK;
     CUtensorMap tmx;
-    if (!make_tmap_bf16(&tmx, x, (uint64_t)M, (uint64_t)w.K, (uint64_t)ldx)) {
+    if (!make_tmap_bf16(&tmx, x, PL ? (uint64_t)lo_row + M : (uint64_t)M, (uint64_t)w.K, (uint64_t)ldx)) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation buffer");
         return TANDEM_ERR_CUDA;
     }
     TcTiledArgs a;
     memset(&a, 0, sizeof(a));
     a.M = M; a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.seg_rows = w.seg_rows;
-    a.err_flag = err; a.e = e;
+    a.err_flag = err; a.e = e; a.lo_row = lo_row;
+    if (EPI == EPI_SCORE) { a.tile_max = sc.val; a.tile_idx = sc.idx; a.tile_sum = sc.sum; a.tile_stride = sc.stride; a.truth = sc.truth; a.truth_val = sc.truth_val; }
     const int n_sms = std::max(1, c.n_sms);
     auto feature_tiles = [&](int width) {
         a.tiles0 = cdiv(w.seg_rows0, width);
@@ -567,10 +551,10 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     if (n_pairs > 0 && pair_tiles >= n_pairs) {
         const int rest = (int)(pair_tiles % n_pairs);
         a.whole = (int)pair_tiles - rest;
-        a.parts = rest * 4 <= n_pairs ? 4 : (rest * 2 <= n_pairs ? 2 : 1);
+        a.parts = EPI == EPI_SCORE ? 1 : (rest * 4 <= n_pairs ? 4 : (rest * 2 <= n_pairs ? 2 : 1));
         static std::atomic<unsigned long long> attr_done{0};
-        ensure_dyn_smem(gemm_tc_pair_kernel<EPI>, TCP_SMEM_BYTES, attr_done);
-        launch_ex(c, true, 2, gemm_tc_pair_kernel<EPI>, dim3(2 * n_pairs), dim3(TCP_THREADS), (size_t)TCP_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2],
+        ensure_dyn_smem(gemm_tc_pair_kernel<EPI, PL>, TcpCfg<PL>::SMEM_BYTES, attr_done);
+        launch_ex(c, true, 2, gemm_tc_pair_kernel<EPI, PL>, dim3(2 * n_pairs), dim3(TCP_THREADS), (size_t)TcpCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2],
                   w.part[0], w.part[1], w.part[2]);
         return TANDEM_OK;
     }
@@ -581,11 +565,11 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     // and a ring holds three K-blocks (329 rows x 4096 x 11008, 96 tiles: 107 -> 64 us).
     const int tiles = (int)feature_tiles(TCS_BN), KB = cdiv(w.K, 64);
     int S = 1;
-    while (S < 4 && ((tiles * S * 2 <= n_sms && KB >= 8 * S) || (tiles * S <= n_sms && KB >= 32 * S))) S *= 2;
+    while (EPI != EPI_SCORE && S < 4 && ((tiles * S * 2 <= n_sms && KB >= 8 * S) || (tiles * S <= n_sms && KB >= 32 * S))) S *= 2;
     a.splits = S;
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_tc_split_kernel<EPI>, TCS_SMEM_BYTES, attr_done);
-    launch_ex(c, true, S, gemm_tc_split_kernel<EPI>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)TCS_SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
+    ensure_dyn_smem(gemm_tc_split_kernel<EPI, PL>, TcsCfg<PL>::SMEM_BYTES, attr_done);
+    launch_ex(c, true, S, gemm_tc_split_kernel<EPI, PL>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)TcsCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
     return TANDEM_OK;
 }
 
@@ -626,7 +610,7 @@ template <typename T, int EPI>
 void launch_gemm(tandem_ctx& c, const T* x, int ldx, int M, const Lin& l, const EpiArgs& e) {
     if (M <= 0) return;
     if constexpr (sizeof(T) == 2) {
-        if (launch_tc_tiled<EPI>(c, x, ldx, M, tcw3(c, l.i0, l.i1, l.i2, l.seg_rows0, l.seg_rows, l.K), e, c.st.counters + 2) != TANDEM_OK)
+        if (launch_tc_tiled<EPI, false>(c, x, ldx, M, tcw3(c, l.i0, l.i1, l.i2, l.seg_rows0, l.seg_rows, l.K), e, c.st.counters + 2) != TANDEM_OK)
             c.setup_failed = true;
     } else {
         const int N = lin_n(l), K = l.K;
@@ -747,7 +731,7 @@ template <typename T>
 void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr) {
     ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + sizeof(T) + (raw ? 2.0 : 0.0)));
     launch_ex(c, true, 1, layernorm_rows_kernel<T>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain), static_cast<const float*>(bias), out, d,
-              M, raw);
+              M, raw, (size_t)0);
 }
 
 // Describes the rows of one pass.
@@ -954,7 +938,7 @@ void large_layers(tandem_ctx& c, const Rows& r, bool project) {
     if constexpr (sizeof(T) == 2) {   // after the last layer no LayerNorm of the large model follows
         const size_t elems = (size_t)r.M * c.large.d.d_model;
         ProfScope ps(c, PC_ROWS, (double)elems * 6.0);
-        launch_ex(c, true, 1, cast_rows_kernel, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, at<bf16>(c, c.lay.xb), elems);
+        launch_ex(c, true, 1, cast_rows_kernel<false>, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, at<bf16>(c, c.lay.xb), elems, (size_t)0);
     }
     project_after<T>(c, n, r);
 }
@@ -1085,18 +1069,18 @@ void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
 // bf16 decode on the tensor cores: five kernels per decoder layer, chained by programmatic dependent launch
 // ---------------------------------------------------------------------------------------------------
 
-// The decode activations' value / remainder planes (see tandem_ctx::PlaneSet): buffer 0 = residual stream, less c, times the next
+// The decode activations' value / remainder planes (see tandem_ctx::xmap): buffer 0 = residual stream, less c, times the next
 // LayerNorm's gain, 1 = attention output, 2 = GELU output; K = the row length in use (the model's width, or its FFN width
 // for buffer 2).
 struct XPlanes { bf16* hi; bf16* lo; TcRows rows; };
 XPlanes x_planes(tandem_ctx& c, int buf, const Model& m) {
-    const tandem_ctx::PlaneSet& ps = *c.planes;
+    const size_t off = buf == 0 ? c.lay.a32 : (buf == 1 ? c.lay.o32 : c.lay.f32);
     const size_t K = buf == 2 ? m.d.d_ff : m.d.d_model;
     XPlanes p;
-    p.hi = at<bf16>(c, ps.at[buf]);
-    p.lo = p.hi + (size_t)ps.rows * K;
-    p.rows.map = &ps.xmap[buf][&m == &c.large ? 0 : 1];
-    p.rows.plane_rows = ps.rows;
+    p.hi = at<bf16>(c, off);
+    p.lo = p.hi + (size_t)c.lay.dec_rows * K;
+    p.rows.map = &c.xmap[buf][&m == &c.large ? 0 : 1];
+    p.rows.plane_rows = c.lay.dec_rows;
     return p;
 }
 
@@ -1107,7 +1091,7 @@ const void* ln_gain(const tandem_ctx& c, const Model& m, int idx) {
 }
 // The value taken off each row before LayerNorm `idx` (NextLn::ref).  Two arrays in turn: the GEMM behind a LayerNorm reads its
 // own from one and leaves the rows' means, the next LayerNorm's, in the other.
-float* ln_ref_of(tandem_ctx& c, int idx) { return at<float>(c, c.lay.ln_ref) + (size_t)(idx & 1) * c.planes->rows; }
+float* ln_ref_of(tandem_ctx& c, int idx) { return at<float>(c, c.lay.ln_ref) + (size_t)(idx & 1) * c.lay.dec_rows; }
 NextLn next_ln(tandem_ctx& c, const Model& m, int idx) {
     const XPlanes p = x_planes(c, 0, m);
     return {static_cast<const float*>(ln_gain(c, m, idx)), p.hi, p.lo, at<float2>(c, c.lay.ln_stats), cdiv(m.d.d_model, 32), ln_ref_of(c, idx)};
@@ -1132,38 +1116,34 @@ bool tc_fused_prologue(const tandem_ctx& c, int K) { return c.batch <= 2 && K <=
 // planes; only the queries and the cached keys / values are bf16.
 void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool stream_w, float* snap = nullptr) {
     const int d = m.d.d_model, dff = m.d.d_ff;
-    bf16* q = at<bf16>(c, c.planes->q);
-    TcScratch sc = tc_scratch(c);
-    sc.whole_pass = r.whole_pass;
+    bf16* q = at<bf16>(c, c.lay.q);
+    const TcScratch sc = tc_scratch(c);
     const XPlanes xo = x_planes(c, 1, m), xf = x_planes(c, 2, m);
-    EpiArgs eq = epi_cache<bf16>(c, m, l, q);
-    if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; }
     launch_tc_decode<PRO_LNT, EPI_QKV>(c, sc, nullptr, d, nullptr, nullptr, r.M,
                                        tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w,
-                                       eq, TcTiles(), ln_rows_of(c, m, 2 * l));
+                                       epi_cache<bf16>(c, m, l, q), nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l));
     attention_decode(c, m, l, q, xo.hi, xo.lo, r);
     EpiArgs eo = epi_plain(h, d);
     eo.ln = next_ln(c, m, 2 * l + 1);
     launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), stream_w, eo,
-                                         TcTiles(), xo.rows);
+                                         nullptr, nullptr, 0, xo.rows);
     EpiArgs e1 = epi_plain(xf.hi, dff);
     e1.out_lo = xf.lo;
     launch_tc_decode<PRO_LNT, EPI_GELU>(c, sc, nullptr, d, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), stream_w, e1,
-                                        TcTiles(), ln_rows_of(c, m, 2 * l + 1));
+                                        nullptr, nullptr, 0, ln_rows_of(c, m, 2 * l + 1));
     EpiArgs e2 = epi_plain(h, d);
     e2.snap = snap; e2.snap_ld = d;   // copy of x^(l+1) when an FF_Tandem projection reads it
     e2.ln = next_ln(c, m, 2 * l + 2);
     launch_tc_decode<PRO_TMA, EPI_RESID>(c, sc, nullptr, dff, nullptr, nullptr, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), stream_w, e2,
-                                         TcTiles(), xf.rows);
+                                         nullptr, nullptr, 0, xf.rows);
 }
 
 // Final LayerNorm + output head; leaves fp32 logits and the per-tile (max, index) pairs that the next kernel
 // (the next pass's row set-up, or the verify kernel) turns into token ids.
 void tc_head(tandem_ctx& c, const Model& m, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool stream_w) {
-    TcTiles t;
-    t.val = at<float>(c, amax_val_off); t.idx = at<int>(c, amax_idx_off); t.stride = c.lay.vocab_tiles;
     launch_tc_decode<PRO_LNT, EPI_ARGMAX>(c, tc_scratch(c), nullptr, m.d.d_model, nullptr, nullptr, r.M, tcw(c, wi_tail(m, 2), -1, -1, m.d.vocab, m.d.d_model),
-                                          stream_w, epi_plain(logits, m.d.vocab), t, ln_rows_of(c, m, 2 * m.d.n_layers));
+                                          stream_w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.lay.vocab_tiles,
+                                          ln_rows_of(c, m, 2 * m.d.n_layers));
 }
 
 // sampled: the previous draft was drawn by sample_draft_kernel (it is in the loop state already), not left as per-tile
@@ -1181,8 +1161,7 @@ void tc_small_step(tandem_ctx& c, int s, bool sampled) {
 // j, then that layer's LayerNorm and key/value maps with the cache write as the GEMM epilogue.  yhat, a_j, t1: fp32 rows.
 void tc_project(tandem_ctx& c, int j, const float* x, const Rows& r, float* yhat, float* a_j, float* t1) {
     const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    TcScratch sc = tc_scratch(c);
-    sc.whole_pass = r.whole_pass;
+    const TcScratch sc = tc_scratch(c);
     if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
         launch_tc_decode<PRO_F32, EPI_STORE_F32>(c, sc, x, dL, nullptr, nullptr, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), true,
                                                  epi_plain(yhat, dS));
@@ -1195,7 +1174,7 @@ void tc_project(tandem_ctx& c, int j, const float* x, const Rows& r, float* yhat
     const void *lg = w_layer(c, c.small, j, W_LN1G), *lb = w_layer(c, c.small, j, W_LN1B);
     const TcW wkv = tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS);
     const EpiArgs ekv = epi_cache<bf16>(c, c.small, j, nullptr);
-    if (!r.whole_pass && tc_fused_prologue(c, dS)) {
+    if (tc_fused_prologue(c, dS)) {
         launch_tc_decode<PRO_LN, EPI_KV>(c, sc, yhat, dS, lg, lb, r.M, wkv, true, ekv);
     } else {
         launch_layernorm<float>(c, r.M, yhat, lg, lb, a_j, dS);
@@ -1254,51 +1233,103 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
     }
 }
 
+// ---- teacher-forced pass (bf16): the prompt pass's kernels with activations as two planes ----------------------------
+
+// What a pass's maps read: two planes of fr_rows rows of K elements.
+template <int EPI>
+void pass_gemm(tandem_ctx& c, const bf16* x, int M, const TcW& w, EpiArgs e, const TcScore& sc = TcScore()) {
+    if (EPI == EPI_GELU) e.out_lo = static_cast<bf16*>(e.out) + (size_t)c.lay.fr_rows * e.ldo;
+    if (launch_tc_tiled<EPI, true>(c, x, w.K, M, w, e, c.st.counters + 2, c.lay.fr_rows, sc) != TANDEM_OK) c.setup_failed = true;
+}
+void pass_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, bf16* out, int d, bf16* raw = nullptr) {
+    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (raw ? 12.0 : 8.0));
+    launch_ex(c, true, 1, layernorm_rows_kernel<bf16, true>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain),
+              static_cast<const float*>(bias), out, d, M, raw, (size_t)c.lay.fr_rows * d);
+}
+
+// FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.
+void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r) {
+    const int dL = c.large.d.d_model, dS = c.small.d.d_model;
+    float* yhat = at<float>(c, c.lay.fr_yhat);
+    bf16 *a_j = at<bf16>(c, c.lay.fr_a), *t1 = at<bf16>(c, c.lay.fr_t1);
+    if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
+        pass_gemm<EPI_STORE_F32>(c, x, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), epi_plain(yhat, dS));
+    } else {
+        pass_gemm<EPI_GELU>(c, x, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), epi_plain(t1, c.hidden));
+        pass_gemm<EPI_STORE_F32>(c, t1, r.M, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden), epi_plain(yhat, dS));
+    }
+    pass_layernorm(c, r.M, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), a_j, dS);
+    pass_gemm<EPI_KV>(c, a_j, r.M, tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS), epi_cache<bf16>(c, c.small, j, nullptr));
+}
+
+// One model's layers over a pass's rows in the residual stream h (and the large model's projections between them).
+void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
+    const int d = m.d.d_model, dff = m.d.d_ff, n = m.d.n_layers;
+    bf16 *x = at<bf16>(c, c.lay.fr_x), *o = at<bf16>(c, c.lay.fr_o), *f = at<bf16>(c, c.lay.fr_f), *q = at<bf16>(c, c.lay.fr_q), *raw = at<bf16>(c, c.lay.fr_raw);
+    const bool large = &m == &c.large;
+    auto project = [&](int l) {
+        for (int j = 0; j < c.small.d.n_layers; ++j)
+            if (c.layer_map[j] == l) pass_project(c, j, raw, r);
+    };
+    for (int l = 0; l < n; ++l) {
+        const bool from_here = large && projects_from(c, l);
+        pass_layernorm(c, r.M, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), x, d, from_here ? raw : nullptr);
+        if (from_here) project(l);
+        EpiArgs eq = epi_cache<bf16>(c, m, l, q);
+        if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; }
+        pass_gemm<EPI_QKV>(c, x, r.M, tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), eq);
+        attention_decode(c, m, l, q, o, o + (size_t)c.lay.fr_rows * d, r);
+        pass_gemm<EPI_RESID>(c, o, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), epi_plain(h, d));
+        pass_layernorm(c, r.M, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), x, d);
+        pass_gemm<EPI_GELU>(c, x, r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), epi_plain(f, dff));
+        pass_gemm<EPI_RESID>(c, f, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), epi_plain(h, d));
+    }
+    if (!large || !projects_from(c, n)) return;
+    const size_t elems = (size_t)r.M * d;   // after the last layer no LayerNorm of the large model follows
+    {
+        ProfScope ps(c, PC_ROWS, (double)elems * 8.0);
+        launch_ex(c, true, 1, cast_rows_kernel<true>, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, raw, elems, (size_t)c.lay.fr_rows * d);
+    }
+    project(n);
+}
+
 // The rows f of a teacher-forced forward (all of whole blocks) through both models.  The large model reads them as one causal pass
 // and its projections go to the small model's cache; then the small model reads all blocks at once, since the tokens it would draft
 // are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie in
-// a cache of their own for the time of one layer.  Every row has the arithmetic of the decode passes (activations as value + remainder).
-// Four sequences of 129-257 tokens through the small pair took one round per block, gamma small passes and one large each, 35.8 ms;
-// 2.0 ms like this.
+// a cache of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
+// is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
+// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.66 ms like this.
 void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large, double kv_positions) {
     const Model &L = c.large, &S = c.small;
-    c.planes = &c.fr_planes;
     Rows r;
     r.M = f.rows; r.decode = true; r.whole_pass = true; r.n_chunks = 1; r.kv_positions = kv_positions;
-    auto begin = [&](const Model& m, float* h, bool setup) {
+    float* h = at<float>(c, c.lay.h_large);
+    auto begin = [&](const Model& m, bool setup) {
         ProfScope ps(c, PC_ROWS, (double)f.rows * m.d.d_model * 8.0);
         launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + (setup ? 1 : 0)), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
-                  (int)m.d.d_model, next_ln(c, m, 0), (int)c.ticket, (int)c.router_ticket);
+                  (int)m.d.d_model, (int)c.ticket, (int)c.router_ticket);
     };
-    float* h = at<float>(c, c.lay.h_large);
-    float *yhat = at<float>(c, c.lay.fr_yhat), *a_j = at<float>(c, c.lay.fr_a), *t1 = at<float>(c, c.lay.fr_t1);
     r.nq = ATT_NQ; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
-    begin(L, h, true);
-    for (int l = 0; l <= L.d.n_layers; ++l) {
-        for (int j = 0; j < S.d.n_layers; ++j)
-            if (c.layer_map[j] == l) tc_project(c, j, h, r, yhat, a_j, t1);
-        if (l < L.d.n_layers) tc_decoder_layer(c, L, l, h, r, true);
-    }
-    float* y = h;   // (the large model's residual stream has been read for the last time)
+    begin(L, true);
+    pass_layers(c, L, h, r);
     r.nq = gamma; r.groups = f.rows / gamma; r.grp_row0 = r.grp_cnt = nullptr;
     r.own_k = at<bf16>(c, c.lay.fr_kv); r.own_v = r.own_k + c.lay.kv_small_layer;
-    begin(S, y, false);
-    for (int j = 0; j < S.d.n_layers; ++j) tc_decoder_layer(c, S, j, y, r, true);
+    begin(S, false);   // (the large model's residual stream has been read for the last time)
+    pass_layers(c, S, h, r);
+    const int d = S.d.d_model, tiles = c.lay.score_tiles;
+    bf16* x = at<bf16>(c, c.lay.fr_x);
+    pass_layernorm(c, f.rows, h, w_tail(c, S, 0), w_tail(c, S, 1), x, d);
     for (int r0 = 0; r0 < f.rows; r0 += c.lay.fr_head_rows) {
-        const int rows = std::min(c.lay.fr_head_rows, f.rows - r0), tiles = c.lay.vocab_tiles;
-        TcTiles t;
-        t.val = at<float>(c, c.lay.fr_tiles); t.idx = reinterpret_cast<int*>(t.val + (size_t)rows * tiles); t.stride = tiles;
-        t.sum = t.val + (size_t)2 * rows * tiles;
+        const int rows = std::min(c.lay.fr_head_rows, f.rows - r0);
+        float* val = at<float>(c, c.lay.fr_tiles);
+        TcScore t;
+        t.val = val; t.idx = reinterpret_cast<int*>(val + (size_t)rows * tiles); t.sum = val + (size_t)2 * rows * tiles; t.stride = tiles;
         t.truth = f.truth + r0; t.truth_val = at<float>(c, c.lay.fr_truth_val);
-        TcRows x = ln_rows_of(c, S, 2 * S.d.n_layers);
-        x.row0 = r0; x.ln_stats += (size_t)r0 * x.ln_groups; x.ln_ref += r0; x.ln_mean += r0;
-        launch_tc_decode<PRO_LNT, EPI_SCORE>(c, tc_scratch(c), nullptr, S.d.d_model, nullptr, nullptr, rows, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, S.d.d_model),
-                                             false, epi_plain(nullptr, S.d.vocab), t, x);
+        pass_gemm<EPI_SCORE>(c, x + (size_t)r0 * d, rows, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, d), epi_plain(nullptr, S.d.vocab), t);
         ProfScope ps(c, PC_ARGMAX, 12.0 * rows * tiles);
         launch_ex(c, true, 1, score_tiles_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, rows, tiles, (const float*)t.val, (const int*)t.idx, (const float*)t.sum,
                   (const float*)t.truth_val, (const int*)(f.out + r0), at<float>(c, c.lay.forced_nll), at<int>(c, c.lay.forced_top));
     }
-    c.planes = &c.dec_planes;
 }
 
 void tc_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
@@ -1511,8 +1542,6 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->small.kv_heads = kv_heads_of(cfg->small); c->small.d_kv = d_kv_of(cfg->small);
     c->large.d = cfg->large; c->large.wbase = 0; c->large.kv_off = lay.kv_large; c->large.kv_layer_elems = lay.kv_large_layer;
     c->small.d = cfg->small; c->small.wbase = 5 + 10 * cfg->large.n_layers; c->small.kv_off = lay.kv_small; c->small.kv_layer_elems = lay.kv_small_layer;
-    c->dec_planes.at[0] = lay.a32; c->dec_planes.at[1] = lay.o32; c->dec_planes.at[2] = lay.f32; c->dec_planes.q = lay.q; c->dec_planes.rows = lay.dec_rows;
-    c->fr_planes.at[0] = lay.fr_x; c->fr_planes.at[1] = lay.fr_o; c->fr_planes.at[2] = lay.fr_f; c->fr_planes.q = lay.fr_q; c->fr_planes.rows = lay.fr_rows;
     c->tbase = c->small.wbase + 5 + 10 * cfg->small.n_layers;
     c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0;
     c->pinned_ints = std::max((size_t)lay.max_rows + 5 * cfg->max_batch + 64,
@@ -1571,11 +1600,11 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
         }
         for (int mi = 0; mi < 2; ++mi) {   // decode activations and the LayerNorms' rows
             const Model& mm = mi == 0 ? c->large : c->small;
-            for (tandem_ctx::PlaneSet* ps : {&c->dec_planes, &c->fr_planes})
-                for (int buf = 0; buf < 3; ++buf) {
-                    const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
-                    ok = ok && make_tmap_bf16(&ps->xmap[buf][mi], c->arena + ps->at[buf], 2 * (uint64_t)ps->rows, K, K, 16);
-                }
+            for (int buf = 0; buf < 3; ++buf) {
+                const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
+                const size_t at_off = buf == 0 ? lay.a32 : (buf == 1 ? lay.o32 : lay.f32);
+                ok = ok && make_tmap_bf16(&c->xmap[buf][mi], c->arena + at_off, 2 * (uint64_t)lay.dec_rows, K, K, 16);
+            }
             const uint64_t d = mm.d.d_model, n_ln = 2 * mm.d.n_layers + 1;
             ok = ok && make_tmap_bf16(&c->lnmap[mi], c->arena + (mi == 0 ? lay.ln_rows_large : lay.ln_rows_small), 4 * n_ln, d, d, 4);
         }
@@ -2408,7 +2437,7 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
         launch_tc_decode<PRO_LN, EPI_KV>(tmp, ts, yhat, d_small, ln_g, ln_b, rows, wkv, true, e);
     } else {
         launch_ex(tmp, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr);
+                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr, (size_t)0);
         launch_tc_decode<PRO_F32, EPI_KV>(tmp, ts, a_s, d_small, nullptr, nullptr, rows, wkv, true, e);
     }
     return check_launch();
