@@ -45,6 +45,10 @@ thread_local char g_cuda_err[256] = "";
 size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 int cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// Queries per attention group of the large model in a teacher-forced pass: one group of the MMA's eight columns (a warp meets all
+// keys of its group on its own, so more and lighter warps: 20.5 -> 17.5 us a layer for 772 rows x 16 heads x 64 under ncu).
+constexpr int PASS_GROUP = 8;
+
 struct Layout {   // byte offsets into the arena
     size_t kv_large, kv_small;
     size_t st_n, st_pending, st_drafts, st_targets, st_accept, st_emitted, st_done, st_out, st_counters, st_hist;
@@ -277,7 +281,7 @@ Layout make_layout(const tandem_config& c) {
     L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
     L.ln_ref = take(2 * RD * 4);
     L.fr_seq = take((3 * B + 1) * 4); L.fr_truth = take(RF * 4); L.fr_out = take(RF * 4); L.fr_truth_val = take(RF * 4);
-    L.fr_grp = take(2 * (RF / ATT_NQ + B + 1) * 4);
+    L.fr_grp = take(2 * (RF / PASS_GROUP + B + 1) * 4);
     L.score_tiles = cdiv(c.large.vocab, SCORE_TILE);
     L.fr_tiles = take((size_t)L.fr_head_rows * L.score_tiles * 12);
     L.fr_kv = take(bf ? 2 * L.kv_small_layer * esz : 0);
@@ -518,6 +522,45 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     }
 }
 
+// Which kernel a prompt pass's product takes, from estimated times in us.  Both are bound by their operands' way from L2 into the
+// multiprocessors, so the estimates are a start-up time, plus per K-block what a CTA's share of it takes, plus what an epilogue
+// leaves uncovered; fitted to measurements at 64-3000 rows and the widths of the three bf16 pairs, which the choice reproduces but
+// for cases within a tenth of each other.  us measured, split kernel with 1 / 2 / 4 K-slices | pair kernel:
+//    511 x 3072 x 1024         7.8  8.3 16.1 |  8.1       511 x 1024 x 4096, residual  32.1 17.5 11.3 | 17.4
+//   1023 x 1024 x 1024, resid. 17.5 10.3 11.8 |  7.2      1500 x 1024 x 4096, residual  37.3 32.1 27.7 | 20.5
+//   1023 x 4096 x 1024, GELU   12.3 20.0  -   | 16.5       511 x 4096 x 4096, residual  42.4 38.9 33.1 | 20.2
+//    255 x 12288 x 4096        32.3 37.0  -   | 28.3      2047 x 2048 x 2048, residual  40.9 56.1  -   | 18.9
+struct TiledPlan { bool pair; int slices, whole, parts; };
+TiledPlan tiled_plan(int n_sms, int epi, bool planes, int tiles128, int tiles256, int KB) {
+    TiledPlan best = {false, 1, 0, 1};
+    double least = 0.0;
+    // Split kernel: the K range of a tile dealt to S CTAs (four K-blocks each at least: fewer would not pay for the exchange); one CTA per
+    // multiprocessor waits for its operands' latency, two share the bandwidth, and slices that do not all run at the same time
+    // wait for each other.
+    for (int S = 1; S <= 4; S *= 2) {
+        const int n = tiles128 * S;
+        if (S > 1 && (epi == EPI_SCORE || KB < 4 * S)) break;
+        const double per_kb = n <= n_sms ? (planes ? 0.60 : 0.33) : (planes ? 0.85 : 0.46) * cdiv(n, 2 * n_sms);
+        double us = 3.0 + per_kb * cdiv(KB, S);
+        if (S > 1) us += 1.2 + (n > 2 * n_sms ? 12.0 : (n > n_sms ? 4.0 : 0.0));
+        if (epi == EPI_RESID) us += S == 1 ? 7.0 : (S == 2 ? 4.0 : 1.5);   // (the stream's old values, a row per thread: more columns to a CTA)
+        if (epi == EPI_GELU) us += 2.0;
+        if (S == 1 || us < least) { least = us; best.slices = S; }
+    }
+    // Pair kernel: full rounds of all pairs, then the rest in parts (1, 2 or 4) as far as one round holds them.
+    const int n_pairs = n_sms / 2;
+    if (n_pairs > 0) {
+        const int rest = tiles256 % n_pairs, rounds = tiles256 / n_pairs;
+        const int parts = epi == EPI_SCORE ? 1 : (rest * 4 <= n_pairs ? 4 : (rest * 2 <= n_pairs ? 2 : 1));
+        const double whole_kb = planes ? 0.75 : 0.42, part_kb = parts == 4 ? (planes ? 0.32 : 0.24) : (parts == 2 ? (planes ? 0.42 : 0.27) : whole_kb);
+        double us = 4.2 + KB * (rounds * whole_kb + (rest > 0 ? part_kb : 0.0));
+        if (epi == EPI_RESID) us += 0.5;
+        if (epi == EPI_GELU) us += 5.0;
+        if (us < least || tiles256 >= 2 * n_pairs) { best.pair = true; best.whole = tiles256 - rest; best.parts = parts; }
+    }
+    return best;
+}
+
 // What the output head of a teacher-forced pass leaves per row and SCORE_TILE features instead of the logits.
 struct TcScore { float* val; int* idx; float* sum; int stride; const int* truth; float* truth_val; };
 
@@ -543,33 +586,26 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
         return (long long)a.tiles_n * a.tiles_m;
     };
     ProfScope ps(c, PC_GEMM_TC_TILED, 2.0 * M * (double)a.N * w.K);   // flops
-    // Where 256 x 256 tiles give every pair of multiprocessors one; the tiles beyond the last full round of all pairs are cut into
-    // as many parts (1, 2 or 4) as still fit one round.
+    a.tiles_m = cdiv(M, 128);
+    const int tiles128 = (int)feature_tiles(TCS_BN);
     a.tiles_m = cdiv(M, 256);
-    const long long pair_tiles = feature_tiles(TCP_BN);
-    const int n_pairs = n_sms / 2;
-    if (n_pairs > 0 && pair_tiles >= n_pairs) {
-        const int rest = (int)(pair_tiles % n_pairs);
-        a.whole = (int)pair_tiles - rest;
-        a.parts = EPI == EPI_SCORE ? 1 : (rest * 4 <= n_pairs ? 4 : (rest * 2 <= n_pairs ? 2 : 1));
+    const int tiles256 = (int)feature_tiles(TCP_BN);
+    const TiledPlan plan = tiled_plan(n_sms, EPI, PL, tiles128, tiles256, cdiv(w.K, 64));
+    if (plan.pair) {
+        a.whole = plan.whole; a.parts = plan.parts;
         static std::atomic<unsigned long long> attr_done{0};
         ensure_dyn_smem(gemm_tc_pair_kernel<EPI, PL>, TcpCfg<PL>::SMEM_BYTES, attr_done);
-        launch_ex(c, true, 2, gemm_tc_pair_kernel<EPI, PL>, dim3(2 * n_pairs), dim3(TCP_THREADS), (size_t)TcpCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2],
+        const int items = plan.whole + (tiles256 - plan.whole) * plan.parts;
+        launch_ex(c, true, 2, gemm_tc_pair_kernel<EPI, PL>, dim3(2 * std::min(items, n_sms / 2)), dim3(TCP_THREADS), (size_t)TcpCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2],
                   w.part[0], w.part[1], w.part[2]);
         return TANDEM_OK;
     }
     a.tiles_m = cdiv(M, 128);
-    // Fewer: square tiles, and the K range of each dealt to as many CTAs (1, 2 or 4) as still get a multiprocessor of their
-    // own and four 64-element K-blocks each (fewer would not pay for the exchange); or as get half a
-    // multiprocessor, where the slices keep sixteen K-blocks: cold weights come with 1.5 us of latency
-    // and a ring holds three K-blocks (329 rows x 4096 x 11008, 96 tiles: 107 -> 64 us).
-    const int tiles = (int)feature_tiles(TCS_BN), KB = cdiv(w.K, 64);
-    int S = 1;
-    while (EPI != EPI_SCORE && S < 4 && ((tiles * S * 2 <= n_sms && KB >= 8 * S) || (tiles * S <= n_sms && KB >= 32 * S))) S *= 2;
-    a.splits = S;
+    feature_tiles(TCS_BN);
+    a.splits = plan.slices;
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(gemm_tc_split_kernel<EPI, PL>, TcsCfg<PL>::SMEM_BYTES, attr_done);
-    launch_ex(c, true, S, gemm_tc_split_kernel<EPI, PL>, dim3(tiles * S), dim3(TCS_THREADS), (size_t)TcsCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
+    launch_ex(c, true, plan.slices, gemm_tc_split_kernel<EPI, PL>, dim3(tiles128 * plan.slices), dim3(TCS_THREADS), (size_t)TcsCfg<PL>::SMEM_BYTES, a, tmx, w.tm[0], w.tm[1], w.tm[2]);
     return TANDEM_OK;
 }
 
@@ -1298,7 +1334,7 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
 // are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie in
 // a cache of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
 // is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
-// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.66 ms like this.
+// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.58 ms like this.
 void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large, double kv_positions) {
     const Model &L = c.large, &S = c.small;
     Rows r;
@@ -1309,7 +1345,7 @@ void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large
         launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + (setup ? 1 : 0)), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
                   (int)m.d.d_model, (int)c.ticket, (int)c.router_ticket);
     };
-    r.nq = ATT_NQ; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
+    r.nq = PASS_GROUP; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
     begin(L, true);
     pass_layers(c, L, h, r);
     r.nq = gamma; r.groups = f.rows / gamma; r.grp_row0 = r.grp_cnt = nullptr;
@@ -2059,10 +2095,10 @@ tandem_status forced_forward(tandem_ctx* c, int gamma, int batch, const int32_t*
     launch_call_begin(*c, true);
     ForcedRows f;
     f.ids = at<int>(*c, c->lay.forced_ids); f.off = at<int>(*c, c->lay.fr_seq); f.len = f.off + batch; f.vstart = f.len + batch;
-    f.batch = batch; f.group = ATT_NQ;
+    f.batch = batch; f.group = PASS_GROUP;
     f.row_tok = at<int>(*c, c->lay.row_tok); f.row_seq = at<int>(*c, c->lay.row_seq); f.row_pos = at<int>(*c, c->lay.row_pos);
     f.truth = at<int>(*c, c->lay.fr_truth); f.out = at<int>(*c, c->lay.fr_out);
-    f.grp_row0 = at<int>(*c, c->lay.fr_grp); f.grp_cnt = f.grp_row0 + c->lay.fr_rows / ATT_NQ + c->cfg.max_batch + 1;
+    f.grp_row0 = at<int>(*c, c->lay.fr_grp); f.grp_cnt = f.grp_row0 + c->lay.fr_rows / PASS_GROUP + c->cfg.max_batch + 1;
     const int step = c->lay.fr_rows / gamma * gamma;
     for (f.v0 = 0; f.v0 < rows; f.v0 += step) {
         f.rows = std::min(step, rows - f.v0);

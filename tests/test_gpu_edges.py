@@ -71,6 +71,16 @@ def test_bf16_pair_prompt_gemm_with_tiles_in_parts():
     assert _replay_compare(shape, w, prompts_for(shape, [2105], seed=7), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 1
 
 
+@pytest.mark.parametrize("lens", [[300], [641, 60], [1100, 31], [1900]])
+def test_bf16_prompt_gemm_between_the_two_kernels(lens):
+    """Prompts of a few hundred rows, where the choice between slices of K and pairs of multiprocessors changes from map to map: pairs
+    with fewer tiles than there are, tiles in four, two and one part, key / value segments of 128 features in tiles of 256, ragged
+    row and feature tiles."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(2, 2176, 17, 2312), small=(1, 128, 2, 256), max_pos=1920, layer_map=(1,), kv_heads=(1, 0))
+    w = _bf16_weights(shape, seed=19, std=0.015)
+    assert _replay_compare(shape, w, prompts_for(shape, lens, seed=20), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 2
+
+
 @pytest.mark.parametrize("heads", [2, 1])   # head sizes 64 and 128: chunks of 64 and of 128 keys
 def test_bf16_prompt_attention_at_chunk_edges(heads):
     """Prompts that end one query before, at and behind the end of a chunk, a tile and a group of two tiles, in one batch."""
