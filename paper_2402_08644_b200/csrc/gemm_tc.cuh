@@ -75,6 +75,7 @@ struct TcDecodeArgs {
                             // it may be writing the weights)
     int* err_flag;          // nullable
     unsigned poll_limit;    // polls before a wait on an mbarrier gives up; 0 = MBAR_POLL_LIMIT
+    int rows_early;         // EPI_QKV / EPI_KV: the row arrays are older than the preceding kernel, and fetched ahead of the wait on it
     int withhold_weights;   // test hook for the give-up path: the TMA thread issues no loads, so the wait for
                             // operands must run out (nothing is in flight when the kernel leaves)
     float* amax_val;        // EPI_ARGMAX: [rows][amax_stride] best value per tile
@@ -194,6 +195,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     const int j_count = max(0, min(rpc, a.rows - j_first));
     float hres[EPI == EPI_RESID ? NB : 1];   // EPI_RESID: the residual values this thread's outputs are added to
     float next_gain = 0.f;                   // EPI_RESID: gain of the LayerNorm that follows, at this thread's feature (a parameter)
+    const float inv_k = LNT ? 1.0f / (float)a.K : 0.f;
     int my_seq = 0, my_pos = 0;              // EPI_QKV / EPI_KV, threads below a.rows: this token row's sequence and position
 
     if (warp == 5) {
@@ -307,6 +309,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
     // ---- warps 0-3: token rows into the B stages (then the epilogue) ----
     float4 gq[C::STAGES], bq[C::STAGES];   // register path: gain / bias of this lane's slot in each of the CTA's K-blocks
     if (a.wait_first) pdl_wait();
+    if ((EPI == EPI_QKV || EPI == EPI_KV) && a.rows_early && tid < a.rows) { my_seq = __ldcg(a.e.row_seq + tid); my_pos = __ldcg(a.e.row_pos + tid); }
     if (EPI == EPI_RESID && a.e.ln.gain && n_local0 + tid < seg_rows) next_gain = __ldg(a.e.ln.gain + seg_base + n_local0 + tid);
     if (ln_regs) {
 #pragma unroll
@@ -322,7 +325,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         // cache index of (row j, head h, element el) = ((seq_j * H + h) * t_max + pos_j) * d_head + el: the row part once
         // per row.  Only the epilogue needs it: the two loads are in flight while the B operand is produced, and the
         // barrier that publishes the offsets sits after that.
-        if (tid < a.rows) {                                                           // first used ahead of the epilogue
+        if (tid < a.rows && !a.rows_early) {                                          // first used ahead of the epilogue
             if (a.e.row_seq) { my_seq = a.e.row_seq[tid]; my_pos = a.e.row_pos[tid]; }
             else my_seq = a.x_row0 + tid;                                             // stand-alone: row j is sequence j at position 0
         }
@@ -399,28 +402,35 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         if (lane == 0)
             for (int i = 0; i < nkb; ++i) mbar_arrive(smem_u32(&s_full[i]));
     } else if (LNT) {
-        // The rows' statistics from the groups' (mean, sum of squared deviations): eight lanes per row, sums relative to the
-        // first group's mean.  For each row the order of the sums depends on K only.
+        // The rows' statistics from the groups' (mean, sum of squared deviations): eight lanes per row, four of a lane's groups
+        // fetched at once, sums relative to the first group's mean.  For each row the order of the sums depends on K only.
+        // (Fetched one after the other where a row has fewer than 32 groups, and with divisions behind the sums, they held the
+        // products up: a one-row pass through a 512-wide map 2.79 us of the chain, 2.31 us like this, a layer of that width 13.1 -> 12.2 us.)
         if (nkb <= C::STAGES || a.release_early) pdl_launch_dependents();   // (see the note at the epilogue)
         for (int r0 = warp * 4; r0 < a.rows; r0 += 16) {
             const int r = r0 + (lane >> 3), gl = lane & 7;
             const float2* sp = a.ln_stats + (size_t)min(r, a.rows - 1) * a.ln_groups;
             const float ref = __ldcg(sp).x, c = __ldcg(a.ln_ref + min(r, a.rows - 1));
             float s = 0.f, q = 0.f;
-#pragma unroll 4
-            for (int g = gl; g < a.ln_groups; g += 8) {
-                const float2 p = __ldcg(sp + g);
-                const float n = (float)min(32, a.K - 32 * g), dm = p.x - ref;
-                s = fmaf(n, dm, s);
-                q += fmaf(n * dm, dm, p.y);
+#pragma unroll 1
+            for (int g0 = gl; g0 < a.ln_groups; g0 += 32) {
+                float2 p[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) p[u] = g0 + 8 * u < a.ln_groups ? __ldcg(sp + g0 + 8 * u) : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float n = (float)max(0, min(32, a.K - 32 * (g0 + 8 * u))), dm = p[u].x - ref;   // (0 past the last group)
+                    s = fmaf(n, dm, s);
+                    q += fmaf(n * dm, dm, p[u].y);
+                }
             }
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) { s += __shfl_xor_sync(0xffffffffu, s, o); q += __shfl_xor_sync(0xffffffffu, q, o); }
-            const float dmu = s / (float)a.K;
+            const float dmu = s * inv_k;
             if (gl == 0 && r < a.rows) {
                 s_mu[r] = (ref - c) + dmu;
                 if (unit == 0) a.ln_mean[r] = ref + dmu;
-                s_rstd[r] = 1.0f / sqrtf(fmaxf(q - s * dmu, 0.f) / (float)a.K + 1e-5f);
+                s_rstd[r] = __frsqrt_rn(fmaf(fmaxf(q - s * dmu, 0.f), inv_k, 1e-5f));
             }
         }
         bar_sync(1, 128);

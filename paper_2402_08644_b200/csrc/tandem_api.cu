@@ -405,6 +405,7 @@ struct TcScratch {
     unsigned poll_limit = 0;   // 0: the kernels' default
     int withhold_weights = 0;  // test hook, see TcDecodeArgs
     int wait_first = 0;        // the launch may follow kernels that write its weights, see TcDecodeArgs
+    int rows_early = 0;        // the row arrays are older than the preceding kernel, see TcDecodeArgs
 };
 
 TcW tcw3(const tandem_ctx& c, int i0, int i1, int i2, int seg_rows0, int seg_rows, int K) {
@@ -504,6 +505,7 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     a.poll_limit = sc.poll_limit;
     a.withhold_weights = sc.withhold_weights;
     a.wait_first = sc.wait_first;
+    a.rows_early = sc.rows_early && e.row_seq ? 1 : 0;
     a.release_early = (size_t)a.N * (size_t)w.K * 2 <= ((size_t)16 << 20) ? 1 : 0;
     a.amax_val = amax_val; a.amax_idx = amax_idx; a.amax_stride = amax_stride;
     a.e = e;
@@ -1153,7 +1155,8 @@ bool tc_fused_prologue(const tandem_ctx& c, int K) { return c.batch <= 2 && K <=
 void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool stream_w, float* snap = nullptr) {
     const int d = m.d.d_model, dff = m.d.d_ff;
     bf16* q = at<bf16>(c, c.lay.q);
-    const TcScratch sc = tc_scratch(c);
+    TcScratch sc = tc_scratch(c);
+    sc.rows_early = l > 0;   // (the first layer's maps follow the kernel that writes them)
     const XPlanes xo = x_planes(c, 1, m), xf = x_planes(c, 2, m);
     launch_tc_decode<PRO_LNT, EPI_QKV>(c, sc, nullptr, d, nullptr, nullptr, r.M,
                                        tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), stream_w,
