@@ -14,8 +14,8 @@
 //                          deviation), g and b ride along as four more rows of the B operand (each as value + remainder), and
 //                          the row's statistics are merged while the products run, so nothing but TMA stands between
 //                          the producer and the MMAs (PRO_LNT).  Activations enter the product as the sum of two bf16 numbers (the rounded value and the rounded
-//                          remainder, about 16 significant bits): the B tile holds the NB value rows followed
-//                          by the NB remainder rows, one MMA of N = 2 NB covers both (the weight tile is read
+//                          remainder, about 16 significant bits): the B tile holds, for every 16 token rows, their values followed
+//                          by their remainders, one MMA of N = 2 NB covers both (the weight tile is read
 //                          from shared memory once), and the epilogue adds the two accumulator columns of a
 //                          token row.  The kernel streams weights, so the wider B operand costs no bandwidth.
 //                          The weight loads are issued before the kernel waits for its predecessor in the
@@ -55,7 +55,7 @@ enum { TC_ERR_SLOT = 1, TC_ERR_OPERANDS = 2, TC_ERR_ACCUM = 3, TC_ERR_EXCHANGE =
 struct TcDecodeArgs {
     const void* x;          // PRO_BF16: bf16 [rows][ldx];  PRO_LN / PRO_F32: float [rows][ldx];  PRO_TMA: unused (tensor map)
     int ldx;
-    int x_row0, x_plane_rows;   // PRO_TMA: first token row of this launch; rows between the value and the remainder plane
+    int x_row0;                 // PRO_TMA: first token row of this launch
     int release_early;          // PRO_TMA: the successor is released right after the wait on the predecessor (a small matrix:
                                 // a chain of dependent steps, nothing to protect) instead of after the last token-row loads
     const float* ln_g;      // PRO_LN: LayerNorm gain / bias [K]
@@ -102,7 +102,7 @@ inline void tcd_shift_rows(TcDecodeArgs& a, int r0, int nr) {
 
 constexpr int TCD_THREADS = 192;   // warps 0-3: B operand + epilogue; warp 4: TMA; warp 5: TMEM + MMA issue
 template <int NB, bool LNT> struct TcdCfg {
-    static constexpr int NB2 = 2 * NB;              // B-operand rows = accumulator columns: values, then remainders
+    static constexpr int NB2 = 2 * NB;              // B-operand rows = accumulator columns: for every 16 token rows their values, then their remainders
     static constexpr int N = NB2 + (LNT ? 16 : 0);  // ... and the LayerNorm's g, g's remainder, b, b's remainder (of 16 columns four are used)
     static constexpr int STAGES = NB <= 16 ? (LNT ? 4 : 5) : 3;   // two CTAs fit on an SM up to NB = 48 (at most 113 KB each with the static part)
     static constexpr int A_BYTES = 128 * 128;       // 128 weight rows x 64 bf16
@@ -234,16 +234,13 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
             // (test hook: nothing is loaded)
         } else if (BY_TMA) {
             // Weights of the first ring-ful before the wait on the predecessor, then the wait, then their token rows
-            // (two planes, 16-row boxes), then weights and rows together as stages come free.
+            // (boxes of 16 rows in both planes; a copy for each plane instead: the small model's output head 5.41 us, 4.80 like this), then weights and rows together as stages come free.
             auto load_b = [&](int i, int st) {
                 const uint32_t bar = smem_u32(&s_full[st]);
                 const uint32_t dst = ring0 + st * C::STAGE_BYTES + C::A_BYTES;
                 mbar_arrive_expect_tx(bar, C::B_BYTES);
 #pragma unroll
-                for (int r16 = 0; r16 < NB; r16 += 16) {
-                    tma_load_2d_nohint(dst + r16 * 128, &tmx, (kb0 + i) * 64, a.x_row0 + r16, bar);                          // values
-                    tma_load_2d_nohint(dst + (NB + r16) * 128, &tmx, (kb0 + i) * 64, a.x_plane_rows + a.x_row0 + r16, bar);   // remainders
-                }
+                for (int r16 = 0; r16 < NB; r16 += 16) tma_load_3d_nohint(dst + r16 * 256, &tmx, (kb0 + i) * 64, a.x_row0 + r16, 0, bar);   // values, remainders
             };
             const int n_pre = min(nkb, C::STAGES);
             if (elect_one()) {
@@ -390,9 +387,9 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         split_bf16x2(y.z, y.w, val.y, rem.y);
                     }
                     const int c = (lane & 15) >> 1;
-                    unsigned char* bt = ring + i * C::STAGE_BYTES + C::A_BYTES + r * 128 + ((c ^ (r & 7)) << 4) + ((lane & 1) << 3);
+                    unsigned char* bt = ring + i * C::STAGE_BYTES + C::A_BYTES + ((r & ~15) + r) * 128 + ((c ^ (r & 7)) << 4) + ((lane & 1) << 3);
                     *reinterpret_cast<uint2*>(bt) = val;
-                    *reinterpret_cast<uint2*>(bt + NB * 128) = rem;   // NB is a multiple of 8: the same swizzle phase
+                    *reinterpret_cast<uint2*>(bt + 16 * 128) = rem;   // (the same swizzle phase)
                 }
             }
         }
@@ -513,9 +510,9 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         }
                     }
                     // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8
-                    unsigned char* dst = bt + r * 128 + ((c ^ (r & 7)) << 4);
+                    unsigned char* dst = bt + ((r & ~15) + r) * 128 + ((c ^ (r & 7)) << 4);
                     *reinterpret_cast<uint4*>(dst) = val;
-                    *reinterpret_cast<uint4*>(dst + NB * 128) = rem;   // the remainder row of token row r (same swizzle phase)
+                    *reinterpret_cast<uint4*>(dst + 16 * 128) = rem;   // the remainder row of token row r (same swizzle phase)
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
@@ -554,8 +551,8 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
         for (int c0 = 0; c0 < NB; c0 += 16) {
             if (c0 >= a.rows) break;                  // columns of absent token rows are never read
             uint32_t t[16], u[16];
-            tmem_issue16(acc + c0, t);                // x's values times W
-            tmem_issue16(acc + NB + c0, u);           // x's remainders times W
+            tmem_issue16(acc + 2 * c0, t);            // x's values times W
+            tmem_issue16(acc + 2 * c0 + 16, u);       // x's remainders times W
             tmem_wait_ld(t, u, w);
             if (LNT && c0 == 0) {
                 c1 = __uint_as_float(w[0]) + __uint_as_float(w[1]);

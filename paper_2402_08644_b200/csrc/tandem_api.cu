@@ -136,7 +136,7 @@ struct tandem_ctx {
     std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
     // Decode activations as two bf16 planes (values, then remainders, dec_rows rows each) that the consuming GEMM loads by
     // TMA: maps of the residual stream (less c, times the next LayerNorm's gain: see NextLn) / attention / GELU buffers, [buffer 0..2][0 large,
-    // 1 small], 16-row boxes.
+    // 1 small], boxes of 16 rows of both planes.
     CUtensorMap xmap[3][2];
     CUtensorMap lnmap[2];                // the LayerNorms' own rows, four per LayerNorm (2 l, 2 l + 1 of layer l, then the final one)
     std::vector<CUtensorMap> kmap, vmap; // the large model's key / value cache of each layer as [(seq, head, position)][d_head]
@@ -377,7 +377,19 @@ bool make_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t c
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The same, remembered: a tensor map depends on nothing but its arguments, and the stand-alone calls get the same weight matrices again
+// Two planes [rows][cols], one behind the other, tiles of 16 rows x 64 columns of both.
+bool make_tmap_planes(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols) {
+    EncodeTiledFn enc = tmap_encoder();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {cols, rows, 2};
+    const cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
+    const cuuint32_t box[3] = {64, 16, 2};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// make_tmap_bf16, remembered: a tensor map depends on nothing but its arguments, and the stand-alone calls get the same weight matrices again
 // and again (an encoding costs the host about 0.4 us, which the first call on a matrix pays).  128 maps per thread, 24 KB, the last one to hash to a place stays.
 bool cached_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols) {
     struct Entry { const void* base; uint64_t rows, cols; CUtensorMap tm; };
@@ -456,7 +468,6 @@ void launch_ex(tandem_ctx& c, bool pdl, int cluster, void (*kernel)(KArgs...), d
 // Token rows that lie in two bf16 planes (PRO_TMA), and the LayerNorm that is applied to them (PRO_LNT).
 struct TcRows {
     const CUtensorMap* map = nullptr;
-    int plane_rows = 0;                    // rows between the value and the remainder plane
     const CUtensorMap* ln_map = nullptr;
     int ln_row = 0;                        // the LayerNorm's first row there
     const float2* ln_stats = nullptr;      // [rows][ln_groups]
@@ -484,7 +495,7 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     TcDecodeArgs a;
     memset(&a, 0, sizeof(a));
     a.x = x; a.ldx = ldx; a.ln_g = static_cast<const float*>(ln_g); a.ln_b = static_cast<const float*>(ln_b);
-    a.rows = rows; a.x_plane_rows = xr.plane_rows;
+    a.rows = rows;
     a.ln_row = xr.ln_row; a.ln_groups = xr.ln_groups; a.ln_stats = xr.ln_stats; a.ln_ref = xr.ln_ref; a.ln_mean = xr.ln_mean;
     a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.tiles0 = cdiv(w.seg_rows0, 128);
     a.seg_rows = w.seg_rows; a.tiles_per_seg = cdiv(w.seg_rows, 128);
@@ -1118,7 +1129,6 @@ XPlanes x_planes(tandem_ctx& c, int buf, const Model& m) {
     p.hi = at<bf16>(c, off);
     p.lo = p.hi + (size_t)c.lay.dec_rows * K;
     p.rows.map = &c.xmap[buf][&m == &c.large ? 0 : 1];
-    p.rows.plane_rows = c.lay.dec_rows;
     return p;
 }
 
@@ -1642,7 +1652,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
             for (int buf = 0; buf < 3; ++buf) {
                 const uint64_t K = buf == 2 ? mm.d.d_ff : mm.d.d_model;
                 const size_t at_off = buf == 0 ? lay.a32 : (buf == 1 ? lay.o32 : lay.f32);
-                ok = ok && make_tmap_bf16(&c->xmap[buf][mi], c->arena + at_off, 2 * (uint64_t)lay.dec_rows, K, K, 16);
+                ok = ok && make_tmap_planes(&c->xmap[buf][mi], c->arena + at_off, (uint64_t)lay.dec_rows, K);
             }
             const uint64_t d = mm.d.d_model, n_ln = 2 * mm.d.n_layers + 1;
             ok = ok && make_tmap_bf16(&c->lnmap[mi], c->arena + (mi == 0 ? lay.ln_rows_large : lay.ln_rows_small), 4 * n_ln, d, d, 4);
