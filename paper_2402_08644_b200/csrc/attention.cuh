@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // Tiles that end before the block's first position hold committed keys and values from earlier iterations (or
     // earlier steps of this one): they are fetched before the wait; what the predecessor may have written, after it.
     int pre = 0;
-#pragma unroll
+#pragma unroll 1   // (less code to fetch)
     for (int it = 0; it < C::STAGES - 1; ++it) {
         if (it == pre && it < n_mine && tile_start(it) + ATD_WROWS <= pos_first) {
             issue(it);
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         }
     }
     pdl_wait();   // queries and the newest keys/values come from the kernel before this one
-#pragma unroll
+#pragma unroll 1
     for (int it = 0; it < C::STAGES - 1; ++it) {
         if (it >= pre) {
             if (it < n_mine) issue(it);

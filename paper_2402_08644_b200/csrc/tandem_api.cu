@@ -747,11 +747,14 @@ int attn_max_clusters(int cl) {
 // four.  20 sequences x 16 heads x 64 x 3000 positions, 320 clusters where 296 CTAs fit: 61 us with one, 52 with two, 49 with
 // four; 32 x 16 x 64 x 8194: 160 us with one, 166 with two.  (Sizes in between measured 3 % slower per iteration at batch 8: a
 // cluster of three merges more states than its extra CTAs save.)
-int attn_cluster_size(long long clusters, int d_head) {
+// In a decode pass (beside others) a cluster of eight, which needs eight places in one GPC, finds about half of them taken by
+// the kernels before and behind it: four sequences x 8 heads x 64, 32 clusters where 33 fit on an empty GPU, a layer of the 512-wide model 14.5 us with eight, 13.1 with four.
+int attn_cluster_size(long long clusters, int d_head, bool alone) {
     int best = 1;
     double least = 0.0;
     for (int cl = 1; cl <= ATD_CLUSTER; cl *= 2) {
-        const int fit = d_head == 32 ? attn_max_clusters<32>(cl) : (d_head == 64 ? attn_max_clusters<64>(cl) : attn_max_clusters<128>(cl));
+        int fit = d_head == 32 ? attn_max_clusters<32>(cl) : (d_head == 64 ? attn_max_clusters<64>(cl) : attn_max_clusters<128>(cl));
+        if (cl == 8 && !alone) fit = std::max(1, fit / 2);
         const double cost = (double)((clusters + fit - 1) / fit) * (24.0 / cl + 2.5);
         if (cl == 1 || cost < least) { least = cost; best = cl; }
     }
@@ -769,7 +772,7 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     int gpc = 1;
     while (gpc * 2 <= group && group % (gpc * 2) == 0 && gpc * 2 * a.nq <= ATT_NQ) gpc *= 2;
     a.heads_per_cta = gpc;
-    const int cl = pass ? 1 : attn_cluster_size((long long)groups * n_kv, d_head);
+    const int cl = pass ? 1 : attn_cluster_size((long long)groups * n_kv, d_head, a.wait_first != 0);
     if (d_head == 32) launch_attn_decode_dq<32>(c, a, groups, cl, pass, kv_bytes);
     else if (d_head == 64) launch_attn_decode_dq<64>(c, a, groups, cl, pass, kv_bytes);
     else launch_attn_decode_dq<128>(c, a, groups, cl, pass, kv_bytes);
