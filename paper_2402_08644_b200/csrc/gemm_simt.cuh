@@ -102,8 +102,9 @@ __device__ __forceinline__ float warp_sum_many(float (&v)[NV], int lane) {
 // Bound by latency (the fp32 pair's matrices are 0.06-1 MB): NC = 1 spreads N = 256..1024 over the whole GPU, NC = 4 reads
 // the staged rows once per four columns when there are columns enough; a warp's first weights are fetched before the wait
 // on the preceding kernel; the row sums leave the warp through warp_sum_many and are finished by several lanes side by
-// side.  Five rows, N = 768, K = 256 with LayerNorm: 4.0 us of the stream's time, against 2.1 us for a LayerNorm kernel and
-// 12.4 us for four columns per warp, a butterfly per sum and one writing lane.
+// side.  One short row goes from L2 straight into the registers of every warp; more rows are staged with all of a thread's loads
+// in flight.  Up to 512 elements a row is normalised in a warp's registers on its way, with gain and bias fetched ahead of the wait.  (Staging
+// loads one after the other, statistics from shared memory and rows read and written back for LayerNorm: a layer of the 128-wide model, one row, 11.9 us of the chain, 9.4 like this; of the 256-wide one, five rows, 18.7 and 17.3.)
 // grid: (ceil(N / (GS_WARPS * NC)), ceil(M / MT)); dynamic smem: MT * min(K, GS_KC) floats.
 template <int MT, int NC, bool LN, int EPI>
 __global__ void __launch_bounds__(GS_THREADS)
@@ -131,6 +132,31 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
             const int kk = (lane + 32 * i) * 4;
             wpre[c][i] = (wrow[c] != nullptr && kk < K) ? __ldg(reinterpret_cast<const float4*>(wrow[c] + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+    constexpr int LV = PF < 4 ? PF : 4;            // float4s per lane of a row that is normalised in registers
+    const bool ln_regs = LN && K <= 128 * LV;
+    const bool direct = MT == 1 && (LN ? ln_regs : K <= 128 * PF);
+    float4 g[LN ? LV : 1], b[LN ? LV : 1];
+    if (ln_regs) {
+#pragma unroll
+        for (int v = 0; v < (LN ? LV : 1); ++v) {
+            const int kk = (lane + 32 * v) * 4;
+            g[v] = kk < K ? __ldg(reinterpret_cast<const float4*>(ln_g + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            b[v] = kk < K ? __ldg(reinterpret_cast<const float4*>(ln_b + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    // where this thread's float4s of the first staging pass come from and go (a division per load ahead of the wait, none behind it)
+    constexpr int ST = MT == 1 ? 2 : 8;
+    int off_x[ST], off_s[ST];
+    {
+        const int vec = KS >> 2;
+        int r = threadIdx.x / vec, v = threadIdx.x - r * vec;
+#pragma unroll
+        for (int u = 0; u < ST; ++u) {
+            off_x[u] = r * ldx + v * 4;
+            off_s[u] = r < rows ? r * KS + v * 4 : -1;
+            for (v += GS_THREADS; v >= vec; v -= vec) ++r;
+        }
+    }
     pdl_wait();
     pdl_launch_dependents();
 
@@ -150,15 +176,68 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
             }
         }
     };
+    // A row of up to 128 * V elements into a warp's registers, normalised where LayerNorm precedes the map (biased variance, eps 1e-5)
+    auto load_row = [&](auto& t, int m) {
+        constexpr int V = sizeof(t) / sizeof(t[0]);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int kk = (lane + 32 * v) * 4;
+            t[v] = kk < K ? __ldcg(reinterpret_cast<const float4*>(x + (size_t)m * ldx + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if constexpr (LN) {
+            float sum = 0.f, q = 0.f;
+#pragma unroll
+            for (int v = 0; v < V; ++v) if ((lane + 32 * v) * 4 < K) sum += (t[v].x + t[v].y) + (t[v].z + t[v].w);
+            const float mu = warp_sum(sum) / (float)K;
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                if ((lane + 32 * v) * 4 < K) {
+                    const float d0 = t[v].x - mu, d1 = t[v].y - mu, d2 = t[v].z - mu, d3 = t[v].w - mu;
+                    q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
+                }
+            const float rs = 1.0f / sqrtf(warp_sum(q) / (float)K + 1e-5f);
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                t[v].x = (t[v].x - mu) * rs * g[v].x + b[v].x; t[v].y = (t[v].y - mu) * rs * g[v].y + b[v].y;
+                t[v].z = (t[v].z - mu) * rs * g[v].z + b[v].z; t[v].w = (t[v].w - mu) * rs * g[v].w + b[v].w;
+            }
+        }
+    };
+    auto dot = [&](float& a, const float4& xv, const float4& w) { a = fmaf(xv.x, w.x, a); a = fmaf(xv.y, w.y, a); a = fmaf(xv.z, w.z, a); a = fmaf(xv.w, w.w, a); };
+    if (direct) {
+        constexpr int V = LN ? LV : PF;
+        float4 t[V];
+        load_row(t, m0);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) if ((lane + 32 * v) * 4 < K) dot(acc[c], t[v], wpre[c][v]);
+    } else
     for (int k0 = 0; k0 < K; k0 += GS_KC) {
         const int kc = min(GS_KC, K - k0), vec = kc >> 2;
         __syncthreads();
-        for (int i = threadIdx.x; i < rows * vec; i += GS_THREADS) {
-            const int r = i / vec, v = i - r * vec;
-            *reinterpret_cast<float4*>(xs + r * KS + v * 4) = __ldcg(reinterpret_cast<const float4*>(x + (size_t)(m0 + r) * ldx + k0 + v * 4));
+        if (ln_regs) {   // (K <= 512: the only staging pass) a warp per row
+            for (int r = warp; r < rows; r += GS_WARPS) {
+                float4 t[LV];
+                load_row(t, m0 + r);
+#pragma unroll
+                for (int v = 0; v < LV; ++v)
+                    if ((lane + 32 * v) * 4 < K) *reinterpret_cast<float4*>(xs + r * KS + (lane + 32 * v) * 4) = t[v];
+            }
+        } else if (k0 == 0 && rows * vec <= ST * GS_THREADS) {   // all of this thread's loads in flight
+            float4 t[ST];
+#pragma unroll
+            for (int u = 0; u < ST; ++u) if (off_s[u] >= 0) t[u] = __ldcg(reinterpret_cast<const float4*>(x + (size_t)m0 * ldx + off_x[u]));
+#pragma unroll
+            for (int u = 0; u < ST; ++u) if (off_s[u] >= 0) *reinterpret_cast<float4*>(xs + off_s[u]) = t[u];
+        } else {
+            for (int i = threadIdx.x; i < rows * vec; i += GS_THREADS) {
+                const int r = i / vec, v = i - r * vec;
+                *reinterpret_cast<float4*>(xs + r * KS + v * 4) = __ldcg(reinterpret_cast<const float4*>(x + (size_t)(m0 + r) * ldx + k0 + v * 4));
+            }
         }
         __syncthreads();
-        if (LN) {   // one warp per row, fixed lane-strided order (biased variance, eps 1e-5)
+        if (LN && !ln_regs) {   // one warp per row, fixed lane-strided order (biased variance, eps 1e-5)
             for (int r = warp; r < rows; r += GS_WARPS) {
                 float* xr = xs + r * KS;
                 float s = 0.f;
