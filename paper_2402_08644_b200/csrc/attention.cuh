@@ -74,8 +74,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_last;
     __shared__ float fo[ATT_NQ];   // LOOP: factor of what the earlier chunks contributed, per query
-    pdl_wait();                // queries and keys/values come from earlier kernels
-    pdl_launch_dependents();   // the next kernel may start fetching its weights
+    if (LOOP) pdl_wait();      // queries and keys/values come from earlier kernels
     T* ks = reinterpret_cast<T*>(smem_raw);
     T* vs = ks + ATT_CH * LD;
     float* qs = reinterpret_cast<float*>(vs + ATT_CH * LD);
@@ -87,15 +86,37 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.z, h = blockIdx.y;
-    const int row0 = a.grp_row0 ? a.grp_row0[g] : g * a.nq;
-    const int cnt = a.grp_cnt ? a.grp_cnt[g] : a.nq;
+    // A decode pass has written its row arrays at least two kernels back: they, and the keys and values of the positions before the
+    // block, are fetched ahead of the wait (one query, 32-wide heads, 60 positions: 2.85 -> 2.24 us of the chain; five, 64-wide: 5.0 -> 4.3).
+    const int row0 = LOOP && a.grp_row0 ? a.grp_row0[g] : g * a.nq;
+    const int cnt = LOOP && a.grp_cnt ? a.grp_cnt[g] : a.nq;
     if (cnt <= 0) return;
-    const int b = a.row_seq[row0];
-    const int pos_first = a.row_pos[row0];
+    const int b = __ldcg(a.row_seq + row0);
+    const int pos_first = __ldcg(a.row_pos + row0);
     const int pos_last = pos_first + cnt - 1;
     const int c_begin = LOOP ? 0 : blockIdx.x;
     const int c_end = LOOP ? pos_last / ATT_CH + 1 : blockIdx.x + 1;
-    if (c_begin * ATT_CH > pos_last) return;
+    if (c_begin * ATT_CH > pos_last) {
+        if (!LOOP) { pdl_wait(); pdl_launch_dependents(); }
+        return;
+    }
+    const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
+    const int kvh = h / (a.n_heads / n_kv);            // grouped-query attention: several query heads share one key/value head
+    const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
+    auto fetch = [&](int t0, int t_lo, int t_hi) {     // positions t0 + t_lo .. t0 + t_hi - 1 into the chunk's rows
+        for (int i = t_lo * VPR + tid; i < t_hi * VPR; i += ATT_THREADS) {
+            const int t = i / VPR, v = i - t * VPR;
+            const size_t src = (head_base + t0 + t) * DH + v * VN;
+            cp_async16(ks + t * LD + v * VN, static_cast<const T*>(a.kcache) + src);
+            cp_async16(vs + t * LD + v * VN, static_cast<const T*>(a.vcache) + src);
+        }
+    };
+    const int n_old = LOOP ? 0 : max(0, min(ATT_CH, pos_first - c_begin * ATT_CH));   // of the (one) chunk's positions
+    if (!LOOP) {
+        fetch(c_begin * ATT_CH, 0, n_old);
+        pdl_wait();
+    }
+    pdl_launch_dependents();   // the next kernel may start fetching its weights
 
     const T* qg = static_cast<const T*>(a.q);
     for (int i = tid; i < cnt * DH; i += ATT_THREADS) {
@@ -109,23 +130,15 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_kernel(AttnArgs a) {
     for (int i = 0; i < ATT_NQ; ++i) acc[i] = 0.f;
     if (LOOP && tid < ATT_NQ) { cm[tid] = -INFINITY; cl[tid] = 0.f; }
 
-    const int n_kv = a.n_kv_heads > 0 ? a.n_kv_heads : a.n_heads;
-    const int kvh = h / (a.n_heads / n_kv);            // grouped-query attention: several query heads share one key/value head
-    const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
     for (int c = c_begin; c < c_end; ++c) {
         const int t0 = c * ATT_CH;
         const int nt = min(ATT_CH, pos_last + 1 - t0);
         const int nt4 = (nt + 3) & ~3;
         __syncthreads();   // previous chunk fully consumed (and qs written, first time round)
-        for (int i = tid; i < nt4 * VPR; i += ATT_THREADS) {
+        fetch(t0, n_old, nt);
+        for (int i = nt * VPR + tid; i < nt4 * VPR; i += ATT_THREADS) {   // up to three rows that fill the last group of four: a zero weight times them stays zero
             const int t = i / VPR, v = i - t * VPR;
-            if (t < nt) {
-                const size_t src = (head_base + t0 + t) * DH + v * VN;
-                cp_async16(ks + t * LD + v * VN, static_cast<const T*>(a.kcache) + src);
-                cp_async16(vs + t * LD + v * VN, static_cast<const T*>(a.vcache) + src);
-            } else {       // up to three rows that fill the last group of four: a zero weight times them stays zero
-                *reinterpret_cast<uint4*>(vs + t * LD + v * VN) = make_uint4(0u, 0u, 0u, 0u);
-            }
+            *reinterpret_cast<uint4*>(vs + t * LD + v * VN) = make_uint4(0u, 0u, 0u, 0u);
         }
         cp_async_commit();
         cp_async_wait_all();
