@@ -9,12 +9,15 @@
 //
 // Both are the exact-arithmetic (fp32 FMA) paths of the fp32 test mode.
 #pragma once
+#include <limits.h>
+#include <math.h>
 #include "common.cuh"
 #include "tc_common.cuh"
 
 namespace tandem {
 
 enum { EPI_STORE = 0, EPI_STORE_F32 = 1, EPI_GELU = 2, EPI_RESID = 3, EPI_QKV = 4, EPI_KV = 5 };
+constexpr int EPI_ARGMAX = 6;   // few rows: fp32 store plus the (max, index) of each row within a tile of features (fp32 mode: a block's columns)
 
 struct EpiArgs {
     void* out;            // EPI_STORE/GELU: T [M][ldo] (GELU on the tensor-core decode path: float);  STORE_F32/RESID: float [M][ldo];  QKV: q as T [M][ldo]
@@ -28,7 +31,7 @@ struct EpiArgs {
     int seg;              //           columns of every further segment (keys / values: kv heads * d_head)
     void* out_lo;         // EPI_GELU on the tensor-core decode path, optional: `out` is then the bf16 plane of the values and this
                           // the bf16 plane of the remainders (x = value + remainder), both [M][ldo], for a consumer that loads them by TMA
-    void* snap;           // EPI_RESID on the tensor-core decode path: optional fp32 copy of the new values [M][snap_ld]
+    void* snap;           // EPI_RESID in decode passes: optional fp32 copy of the new values [M][snap_ld]
     int snap_ld;
     NextLn ln;            // EPI_RESID on the tensor-core decode path, see NextLn
 };
@@ -56,7 +59,9 @@ __device__ __forceinline__ void epilogue(const EpiArgs& e, int m, int n, float v
         static_cast<T*>(e.out)[(size_t)m * e.ldo + n] = from_float<T>(sizeof(T) == 2 ? gelu_bf16_out(v) : gelu_exact(v));
     } else if (EPI == EPI_RESID) {
         float* p = static_cast<float*>(e.out) + (size_t)m * e.ldo + n;
-        *p = *p + v;
+        const float h = *p + v;
+        *p = h;
+        if (sizeof(T) == 4 && e.snap) static_cast<float*>(e.snap)[(size_t)m * e.snap_ld + n] = h;   // (bf16: the few-row kernel has its own epilogue)
     } else {
         int s = 0, c = n;
         if (n >= e.seg0) { s = 1 + (n - e.seg0) / e.seg; c = (n - e.seg0) - (s - 1) * e.seg; }
@@ -109,7 +114,7 @@ __device__ __forceinline__ float warp_sum_many(float (&v)[NV], int lane) {
 template <int MT, int NC, bool LN, int EPI>
 __global__ void __launch_bounds__(GS_THREADS)
 gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, int N, const float* __restrict__ ln_g,
-                 const float* __restrict__ ln_b, EpiArgs e) {
+                 const float* __restrict__ ln_b, EpiArgs e, float* amax_val, int* amax_idx, int amax_stride) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float* xs = reinterpret_cast<float*>(smem_raw);
     constexpr int PF = 8 / NC;    // float4s of each column fetched ahead of the wait
@@ -283,7 +288,28 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
     }
     const float v = warp_sum_many<NV>(acc, lane);
     const int idx = lane >> (5 - LOG), r = idx / NC, n = n0 + idx % NC;
-    if ((lane & ((32 >> LOG) - 1)) == 0 && r < rows && n < N) epilogue<float, EPI>(e, m0 + r, n, v);
+    const bool mine = (lane & ((32 >> LOG) - 1)) == 0 && r < rows;
+    if constexpr (EPI == EPI_ARGMAX) {   // the block's columns, lowest feature on ties; the consumer finishes the row from the blocks' results
+        __shared__ float s_v[GS_WARPS * NC][MT];
+        if (mine) {
+            if (n < N) static_cast<float*>(e.out)[(size_t)(m0 + r) * e.ldo + n] = v;
+            s_v[warp * NC + idx % NC][r] = n < N ? v : -INFINITY;
+        }
+        __syncthreads();
+        if (threadIdx.x < rows) {
+            float best = -INFINITY;
+            int bi = INT_MAX;
+#pragma unroll
+            for (int c = 0; c < GS_WARPS * NC; ++c) {
+                const float t = s_v[c][threadIdx.x];
+                if (t > best) { best = t; bi = blockIdx.x * GS_WARPS * NC + c; }
+            }
+            amax_val[(size_t)(m0 + threadIdx.x) * amax_stride + blockIdx.x] = best;
+            amax_idx[(size_t)(m0 + threadIdx.x) * amax_stride + blockIdx.x] = bi;
+        }
+        return;
+    }
+    if (mine && n < N) epilogue<float, EPI>(e, m0 + r, n, v);
 }
 
 // Shared-memory tiled GEMM for many rows.  64x64 output tile, 16-deep K slices, 4x4 outputs per thread.

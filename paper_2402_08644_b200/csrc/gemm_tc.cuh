@@ -47,7 +47,6 @@ namespace tandem {
 // LayerNorm took 4.4 us of the stream's time with the rows normalised in the prologue of every CTA (batch 1, 2), and
 // 4.4 + 1.9 us with a LayerNorm kernel of their own (more sequences).
 enum { PRO_BF16 = 0, PRO_LN = 1, PRO_F32 = 2, PRO_TMA = 3, PRO_LNT = 4 };
-constexpr int EPI_ARGMAX = 6;                       // fp32 store plus the (max, index) of each row within the tile
 constexpr int EPI_SCORE = 7;                        // many rows: no store, per row and SCORE_TILE features (max, index, sum of exp(y - max)), and y at a given feature
 constexpr int SCORE_TILE = 64;
 enum { TC_ERR_SLOT = 1, TC_ERR_OPERANDS = 2, TC_ERR_ACCUM = 3, TC_ERR_EXCHANGE = 4 };   // which bounded wait gave up

@@ -396,36 +396,6 @@ __global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict_
     ln_put4<PL>(out + i, lo, 1, b.x, b.y, b.z, b.w);
 }
 
-// Arg-max of fp32 rows, lowest index on ties.  grid: rows; block: 256.
-// Row m belongs to sequence m / nq; the result goes to dst[(m / nq) * seq_stride + m % nq + off].
-__global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restrict__ logits, int V, int* dst, int nq, int seq_stride, int off) {
-    __shared__ float sv[8];
-    __shared__ int si[8];
-    pdl_wait();
-    pdl_launch_dependents();
-    const float* lr = logits + (size_t)blockIdx.x * V;
-    float best = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int i = threadIdx.x; i < V; i += 256) {
-        const float v = lr[i];
-        if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
-    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w)
-            if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
-        const int m = blockIdx.x;
-        dst[(size_t)(m / nq) * seq_stride + (m % nq) + off] = bi;
-    }
-}
-
 // Verify / accept / rollback (Section 3.1), one warp per sequence, one CTA.
 //   a = longest prefix of drafts equal to the large model's tokens (or forced);
 //   the sequence gains d_1..d_a and g_{a+1}; n advances; g_{a+1} becomes pending.

@@ -131,6 +131,7 @@ struct tandem_ctx {
     // tensor-core path (bf16 only)
     int n_lns = 0;                       // LayerNorms of both models (bf16), see Layout::ln_src
     bool use_pdl = true;                 // programmatic dependent launch between the decode kernels
+    int amax_tiles = 0;                  // tiles of the output heads' arg-max results per row
     int n_sms = 0;                       // multiprocessors of the context's device: split-K decode GEMMs aim for about one CTA each
     std::vector<CUtensorMap> wmap;       // one per weight pointer (matrices only), box 128 rows x 64 columns
     std::vector<CUtensorMap> wpart;      // the same in boxes of 32 rows
@@ -266,7 +267,7 @@ Layout make_layout(const tandem_config& c) {
     L.dbg = take(T * dmax * 4);
     L.forced_ids = take(B * T * 4); L.forced_len = take(B * 4); L.forced_nll = take(B * T * 4); L.forced_top = take(B * T * 4);
     L.smp_large = take(RD * 8); L.smp_small = take((size_t)std::max(1, c.gamma_max) * B * 8);
-    L.vocab_tiles = cdiv(c.large.vocab, 128);
+    L.vocab_tiles = cdiv(c.large.vocab, bf ? 128 : GS_WARPS);   // (fp32: at most; a block of the head has GS_WARPS columns or four times as many)
     L.amax_val_large = take(RD * L.vocab_tiles * 4); L.amax_idx_large = take(RD * L.vocab_tiles * 4);
     L.amax_val_small = take(B * L.vocab_tiles * 4); L.amax_idx_small = take(B * L.vocab_tiles * 4);
     const size_t nS = c.small.n_layers;
@@ -634,24 +635,27 @@ WSegs segs_of(const tandem_ctx& c, const Lin& l) {
 
 // fp32, few rows.  ln_g / ln_b non-null: LayerNorm of the rows first (fused; K <= GS_KC, see fp32_few_rows).
 template <int MT, int NC, bool LN, int EPI>
-void launch_rows_as(tandem_ctx& c, const float* x, int ldx, int M, int K, const WSegs& ws, int N, const float* ln_g, const float* ln_b, const EpiArgs& e) {
+void launch_rows_as(tandem_ctx& c, const float* x, int ldx, int M, int K, const WSegs& ws, int N, const float* ln_g, const float* ln_b, const EpiArgs& e,
+                    float* amax_val, int* amax_idx) {
     static std::atomic<unsigned long long> attr_done{0};
     ensure_dyn_smem(gemm_rows_kernel<MT, NC, LN, EPI>, (size_t)MT * GS_KC * sizeof(float), attr_done);
     launch_ex(c, true, 1, gemm_rows_kernel<MT, NC, LN, EPI>, dim3(cdiv(N, GS_WARPS * NC), cdiv(M, MT)), dim3(GS_THREADS),
-              (size_t)MT * std::min(K, GS_KC) * sizeof(float), x, ldx, M, K, ws, N, ln_g, ln_b, e);
+              (size_t)MT * std::min(K, GS_KC) * sizeof(float), x, ldx, M, K, ws, N, ln_g, ln_b, e, amax_val, amax_idx, c.amax_tiles);
 }
+// One column per warp until that is two CTAs per multiprocessor, then four (the staged rows are read once for them).
+bool rows_wide(const tandem_ctx& c, int N) { return N > 2 * GS_WARPS * std::max(1, c.n_sms); }
 template <bool LN, int EPI>
-void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, const EpiArgs& e, const void* ln_g = nullptr, const void* ln_b = nullptr) {
+void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, const EpiArgs& e, const void* ln_g = nullptr, const void* ln_b = nullptr,
+                 float* av = nullptr, int* ai = nullptr) {
     if (M <= 0) return;
     const WSegs ws = segs_of(c, l);
     const int N = lin_n(l), K = l.K;
     const float *g = static_cast<const float*>(ln_g), *b = static_cast<const float*>(ln_b);
     ProfScope ps(c, PC_GEMM_SMALLM, ((double)N * K + (double)M * K + (double)M * N) * sizeof(float));
-    // one column per warp until that is two CTAs per multiprocessor, then four (the staged rows are read once for them)
-    const bool wide = N > 2 * GS_WARPS * std::max(1, c.n_sms);
-    if (M <= 1) { if (wide) launch_rows_as<1, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<1, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
-    else if (M <= 4) { if (wide) launch_rows_as<4, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<4, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
-    else { if (wide) launch_rows_as<8, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); else launch_rows_as<8, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e); }
+    const bool wide = rows_wide(c, N);
+    if (M <= 1) { if (wide) launch_rows_as<1, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<1, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
+    else if (M <= 4) { if (wide) launch_rows_as<4, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<4, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
+    else { if (wide) launch_rows_as<8, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<8, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
 }
 
 // y = x W^T with a fused epilogue for many rows: the prompt-pass kernels (tensor cores for bf16).
@@ -883,11 +887,11 @@ bool fp32_few_rows(const tandem_ctx& c, const Rows& r) {
 }
 // LayerNorm, then y = a W^T (few rows, fp32): one kernel up to GS_KC elements per row, two beyond.
 template <int EPI>
-void ln_rows(tandem_ctx& c, const float* h, int M, const void* g, const void* b, const Lin& l, const EpiArgs& e) {
-    if (l.K <= GS_KC) { launch_rows<true, EPI>(c, h, l.K, M, l, e, g, b); return; }
+void ln_rows(tandem_ctx& c, const float* h, int M, const void* g, const void* b, const Lin& l, const EpiArgs& e, float* av = nullptr, int* ai = nullptr) {
+    if (l.K <= GS_KC) { launch_rows<true, EPI>(c, h, l.K, M, l, e, g, b, av, ai); return; }
     float* a = at<float>(c, c.lay.a);
     launch_layernorm<float>(c, M, h, g, b, a, l.K);
-    launch_rows<false, EPI>(c, a, l.K, M, l, e);
+    launch_rows<false, EPI>(c, a, l.K, M, l, e, nullptr, nullptr, av, ai);
 }
 
 // Eq. 2, first line, for small layer j, then that layer's LayerNorm and key/value maps: writes the
@@ -939,9 +943,9 @@ void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
 
 // One decoder layer (Eq. 1; the same form serves the small model's layers in Eq. 2) on residual stream h.  project: the
 // FF_Tandem projections that read h as it enters the layer (they run behind the first LayerNorm, which leaves them a bf16
-// copy of h on its way).
+// copy of h on its way).  snap (fp32 decode passes): copy of x^(l+1) when an FF_Tandem projection reads it.
 template <typename T>
-void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool project = false) {
+void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool project = false, float* snap = nullptr) {
     const int d = m.d.d_model, dff = m.d.d_ff;
     T* a = at<T>(c, c.lay.a);
     T* q = at<T>(c, c.lay.q);
@@ -957,7 +961,9 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
             attention<T>(c, m, l, q, o, r);
             launch_rows<false, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
             ln_rows<EPI_GELU>(c, h, r.M, g2, b2, w1, epi_plain(f, dff));
-            launch_rows<false, EPI_RESID>(c, f, dff, r.M, w2, epi_plain(h, d));
+            EpiArgs e2 = epi_plain(h, d);
+            e2.snap = snap; e2.snap_ld = d;
+            launch_rows<false, EPI_RESID>(c, f, dff, r.M, w2, e2);
             return;
         }
     }
@@ -971,12 +977,12 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
     launch_gemm<T, EPI_RESID>(c, f, dff, r.M, w2, epi_plain(h, d));
 }
 
-// Final LayerNorm, output head, arg-max of a decode pass (fp32).  dst[(m / nq) * seq_stride + m % nq + off].
-void head_argmax(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* logits, int* dst, int seq_stride, int off) {
-    const int d = m.d.d_model, V = m.d.vocab;
-    ln_rows<EPI_STORE_F32>(c, h, r.M, w_tail(c, m, 0), w_tail(c, m, 1), lin1(wi_tail(m, 2), V, d), epi_plain(logits, V));
-    ProfScope ps(c, PC_ARGMAX, (double)r.M * V * 4.0);
-    launch_ex(c, true, 1, argmax_rows_kernel, dim3(r.M), dim3(256), 0, (const float*)logits, V, dst, r.nq, seq_stride, off);
+// Final LayerNorm, output head of a decode pass (fp32): logits, and (argmax) the blocks' maxima that the next pass's row set-up or the
+// verify kernel turns into token ids.
+void fp32_head(tandem_ctx& c, const Model& m, float* h, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool argmax = true) {
+    const Lin w = lin1(wi_tail(m, 2), m.d.vocab, m.d.d_model);
+    if (argmax) ln_rows<EPI_ARGMAX>(c, h, r.M, w_tail(c, m, 0), w_tail(c, m, 1), w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off));
+    else ln_rows<EPI_STORE_F32>(c, h, r.M, w_tail(c, m, 0), w_tail(c, m, 1), w, epi_plain(logits, m.d.vocab));
 }
 
 // The large model's layers over the current rows, whose embeddings are in the residual stream (block mode in decode,
@@ -1009,30 +1015,90 @@ template <typename T>
 void begin_rows(tandem_ctx& c, const Model& m, float* h, int r0, int nq, int fin_r, float* snap = nullptr, const NextLn& ln = NextLn{}) {
     ProfScope ps(c, PC_ROWS, (double)c.batch * nq * m.d.d_model * 8.0);
     launch_ex(c, true, 1, step_begin_kernel<T>, dim3(c.batch * nq), dim3(128), 0, c.st, r0, nq, fin_r,
-              (const float*)at<float>(c, c.lay.amax_val_small), (const int*)at<int>(c, c.lay.amax_idx_small), c.lay.vocab_tiles,
-              c.lay.vocab_tiles, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos),
+              (const float*)at<float>(c, c.lay.amax_val_small), (const int*)at<int>(c, c.lay.amax_idx_small), c.amax_tiles,
+              c.amax_tiles, at<int>(c, c.lay.row_tok), at<int>(c, c.lay.row_seq), at<int>(c, c.lay.row_pos),
               (const T*)w_emb(c, m), (const T*)w_pos(c, m), h, m.d.d_model, snap, ln);
 }
 
-// fp32 draft step s: one token per sequence through the small model over the mixed context (Eq. 2, lines 2-3).
-// keep_drafts: a teacher-forced round keeps its given drafts and sends the step's arg-max to the unused target array.
-void fp32_small_step(tandem_ctx& c, int s, bool keep_drafts = false) {
+// fp32 draft step s: one token per sequence through the small model over the mixed context (Eq. 2, lines 2-3).  drafts_known: the
+// previous draft is in the loop state (drawn, or given), not left as the blocks' maxima.
+void fp32_small_step(tandem_ctx& c, int s, bool drafts_known, bool argmax = true) {
     float* y = at<float>(c, c.lay.h_small);
-    begin_rows<float>(c, c.small, y, s, 1, -1);
+    begin_rows<float>(c, c.small, y, s, 1, (s > 0 && !drafts_known) ? s : -1);
     const Rows r = decode_rows(c, s, 1);
     for (int j = 0; j < c.small.d.n_layers; ++j) decoder_layer<float>(c, c.small, j, y, r);
-    float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
-    if (keep_drafts) head_argmax(c, c.small, y, r, logits, c.st.targets, TANDEM_GAMMA_LIMIT + 1, s);
-    else head_argmax(c, c.small, y, r, logits, c.st.drafts, TANDEM_GAMMA_LIMIT, s);
+    fp32_head(c, c.small, y, r, at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab, c.lay.amax_val_small, c.lay.amax_idx_small, argmax);
 }
 
-// fp32 block pass of the large model over nq rows per sequence; head: final LayerNorm + output head + arg-max.
-void fp32_large_block(tandem_ctx& c, int nq, bool project, bool head) {
+// FF_Tandem of the block's rows x (the residual stream after layer_map[j] large layers) for small layer j, as in the bf16 decode passes.
+void fp32_project(tandem_ctx& c, int j, const float* x, const Rows& r, float* yhat, float* t1) {
+    const int dL = c.large.d.d_model, dS = c.small.d.d_model;
+    if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
+        launch_rows<false, EPI_STORE_F32>(c, x, dL, r.M, lin1(wi_tandem(c, j, 0), dS, dL), epi_plain(yhat, dS));
+    } else {
+        launch_rows<false, EPI_GELU>(c, x, dL, r.M, lin1(wi_tandem(c, j, 0), c.hidden, dL), epi_plain(t1, c.hidden));
+        launch_rows<false, EPI_STORE_F32>(c, t1, c.hidden, r.M, lin1(wi_tandem(c, j, 1), dS, c.hidden), epi_plain(yhat, dS));
+    }
+    const Lin kv = lin3(wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, c.small.d_kv, dS);
+    ln_rows<EPI_KV>(c, yhat, r.M, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), kv, epi_cache<float>(c, c.small, j, nullptr), nullptr, nullptr);
+}
+
+// The projections of a decode pass after n large layers.  They run on the side stream,
+// from the copy of x^(l(j)) that the producing kernel left: they depend on nothing the large model does
+// afterwards (and nothing in the iteration depends on them before the next draft), so they run beside the large model's
+// later layers instead of in their chain.  (fp32, small layers wider than GS_KC: LayerNorm kernel and maps share the large pass's
+// buffer, so those stay in its chain.)
+template <typename P>
+void project_forked(tandem_ctx& c, int n_large_layers_done, int slot, P project) {
+    const size_t RD = (size_t)c.lay.dec_rows, dS = c.small.d.d_model;
+    const float* snap = at<float>(c, c.lay.proj_snap) + (size_t)slot * RD * c.large.d.d_model;
+    cudaStream_t main_stream = c.stream;
+    cudaEventRecord(c.ev_fork[slot], main_stream);
+    cudaStreamWaitEvent(c.side, c.ev_fork[slot], 0);
+    c.stream = c.side;
+    c.next_launch_plain = true;   // first kernel after a cross-stream wait
+    for (int j = 0; j < c.small.d.n_layers; ++j)
+        if (c.layer_map[j] == n_large_layers_done)
+            project(j, snap, at<float>(c, c.lay.proj_yhat) + (size_t)j * RD * dS, at<float>(c, c.lay.proj_a) + (size_t)j * RD * dS,
+                    at<float>(c, c.lay.proj_t1) + (size_t)j * RD * c.hidden);
+    c.stream = main_stream;
+}
+// They join the main stream before the verify kernel.
+void project_join(tandem_ctx& c) {
+    cudaEventRecord(c.ev_join, c.side);
+    cudaStreamWaitEvent(c.stream, c.ev_join, 0);
+    c.next_launch_plain = true;
+}
+
+// Slot of the projection buffers for the residual stream after `n` large layers: the first small layer fed from there, or -1.
+int project_slot(const tandem_ctx& c, int n) {
+    for (int j = 0; j < c.small.d.n_layers; ++j)
+        if (c.layer_map[j] == n) return j;
+    return -1;
+}
+
+// fp32 block pass of the large model over nq rows per sequence; fin_r: see begin_rows; head: final LayerNorm + output head.
+void fp32_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
     float* h = at<float>(c, c.lay.h_large);
-    begin_rows<float>(c, c.large, h, 0, nq, -1);
+    const size_t snap_elems = (size_t)c.lay.dec_rows * c.large.d.d_model;
+    const bool fork = project && c.small.d.d_model <= GS_KC;
+    auto snap_of = [&](int n) -> float* {
+        const int slot = fork ? project_slot(c, n) : -1;
+        return slot >= 0 ? at<float>(c, c.lay.proj_snap) + (size_t)slot * snap_elems : nullptr;
+    };
+    begin_rows<float>(c, c.large, h, 0, nq, fin_r, snap_of(0));
     const Rows r = decode_rows(c, nq - 1, nq);
-    large_layers<float>(c, r, project);
-    if (head) head_argmax(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.st.targets, TANDEM_GAMMA_LIMIT + 1, 0);
+    auto run = [&](int j, const float* snap, float* yhat, float*, float* t1) { fp32_project(c, j, snap, r, yhat, t1); };
+    if (!fork) {
+        large_layers<float>(c, r, project);
+    } else {
+        for (int l = 0; l <= c.large.d.n_layers; ++l) {
+            if (project_slot(c, l) >= 0) project_forked(c, l, project_slot(c, l), run);
+            if (l < c.large.d.n_layers) decoder_layer<float>(c, c.large, l, h, r, false, snap_of(l + 1));
+        }
+    }
+    if (head) fp32_head(c, c.large, h, r, at<float>(c, c.lay.logits_large), c.lay.amax_val_large, c.lay.amax_idx_large);
+    if (fork) project_join(c);   // (every small layer is fed from somewhere)
 }
 
 // Teacher-forced round (accept mode 5, fp32): the given tokens become the round's drafts; after the draft steps their
@@ -1053,7 +1119,7 @@ void launch_verify(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_ne
     ProfScope ps(c, PC_VERIFY, (double)c.batch * (2 * gamma + 8) * 4.0);
     launch_ex(c, true, 1, verify_kernel, dim3(1), dim3(VERIFY_THREADS), 0, c.st, c.batch, gamma, mode, (unsigned long long)seed, max_new,
               from_tiles ? (const float*)at<float>(c, c.lay.amax_val_large) : (const float*)nullptr,
-              from_tiles ? (const int*)at<int>(c, c.lay.amax_idx_large) : (const int*)nullptr, c.lay.vocab_tiles, c.lay.vocab_tiles,
+              from_tiles ? (const int*)at<int>(c, c.lay.amax_idx_large) : (const int*)nullptr, c.amax_tiles, c.amax_tiles,
               from_tiles ? (const float*)at<float>(c, c.lay.amax_val_small) : (const float*)nullptr,
               from_tiles ? (const int*)at<int>(c, c.lay.amax_idx_small) : (const int*)nullptr,
               adaptive ? (const int*)c.st.block_len : (const int*)nullptr);
@@ -1098,22 +1164,23 @@ void launch_sample_verify(tandem_ctx& c, int gamma, uint64_t seed) {
 }
 
 void fp32_iteration(tandem_ctx& c, int gamma, int mode, uint64_t seed, int max_new) {
+    const bool known = mode == 4 || mode == 5;        // drafts drawn, or given
     if (mode == 5) launch_forced_fill(c, gamma);
     for (int s = 0; s < gamma; ++s) {
-        fp32_small_step(c, s, mode == 5);
-        if (mode == 4) launch_sample_draft(c, s, seed);   // replaces the arg-max draft of this step
+        fp32_small_step(c, s, known, !known);
+        if (mode == 4) launch_sample_draft(c, s, seed);
     }
     if (mode == 5) launch_score_rows(c, gamma);
-    if (mode == 3 || mode == 5) fp32_large_block(c, gamma, true, false);   // stand-alone Tandem without the free token: gamma rows, no output head
-    else fp32_large_block(c, gamma + 1, true, true);
+    if (mode == 3 || mode == 5) fp32_large_block(c, gamma, -1, true, false);   // stand-alone Tandem without the free token: gamma rows, no output head
+    else fp32_large_block(c, gamma + 1, (gamma > 0 && !known) ? gamma : -1, true, true);
     if (mode == 4) launch_sample_verify(c, gamma, seed);
-    launch_verify(c, gamma, mode == 5 ? 3 : mode, seed, max_new, false);
+    launch_verify(c, gamma, mode == 5 ? 3 : mode, seed, max_new, mode != 5);
     c.last_gamma = gamma;
 }
 
 void fp32_greedy_iteration(tandem_ctx& c, int max_new) {
-    fp32_large_block(c, 1, false, true);
-    launch_verify(c, 0, 0, 0ull, max_new, false);
+    fp32_large_block(c, 1, -1, false, true);
+    launch_verify(c, 0, 0, 0ull, max_new, true);
     c.last_gamma = 0;
 }
 
@@ -1194,7 +1261,7 @@ void tc_decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows
 // (the next pass's row set-up, or the verify kernel) turns into token ids.
 void tc_head(tandem_ctx& c, const Model& m, const Rows& r, float* logits, size_t amax_val_off, size_t amax_idx_off, bool stream_w) {
     launch_tc_decode<PRO_LNT, EPI_ARGMAX>(c, tc_scratch(c), nullptr, m.d.d_model, nullptr, nullptr, r.M, tcw(c, wi_tail(m, 2), -1, -1, m.d.vocab, m.d.d_model),
-                                          stream_w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.lay.vocab_tiles,
+                                          stream_w, epi_plain(logits, m.d.vocab), at<float>(c, amax_val_off), at<int>(c, amax_idx_off), c.amax_tiles,
                                           ln_rows_of(c, m, 2 * m.d.n_layers));
 }
 
@@ -1234,32 +1301,6 @@ void tc_project(tandem_ctx& c, int j, const float* x, const Rows& r, float* yhat
     }
 }
 
-// The projections of a decode pass after n large layers.  They run on the side stream,
-// from the copy `snap` of x^(l(j)) that the producing kernel left: they depend on nothing the large model does
-// afterwards (and nothing in the iteration depends on them before the next draft), so they run beside the large model's
-// later layers instead of in their chain.
-void tc_project_forked(tandem_ctx& c, int n_large_layers_done, int slot, const Rows& r) {
-    const size_t RD = (size_t)c.lay.dec_rows, dS = c.small.d.d_model;
-    const float* snap = at<float>(c, c.lay.proj_snap) + (size_t)slot * RD * c.large.d.d_model;
-    cudaStream_t main_stream = c.stream;
-    cudaEventRecord(c.ev_fork[slot], main_stream);
-    cudaStreamWaitEvent(c.side, c.ev_fork[slot], 0);
-    c.stream = c.side;
-    c.next_launch_plain = true;   // first kernel after a cross-stream wait
-    for (int j = 0; j < c.small.d.n_layers; ++j)
-        if (c.layer_map[j] == n_large_layers_done)
-            tc_project(c, j, snap, r, at<float>(c, c.lay.proj_yhat) + (size_t)j * RD * dS, at<float>(c, c.lay.proj_a) + (size_t)j * RD * dS,
-                       at<float>(c, c.lay.proj_t1) + (size_t)j * RD * c.hidden);
-    c.stream = main_stream;
-}
-
-// Slot of the projection buffers for the residual stream after `n` large layers: the first small layer fed from there, or -1.
-int project_slot(const tandem_ctx& c, int n) {
-    for (int j = 0; j < c.small.d.n_layers; ++j)
-        if (c.layer_map[j] == n) return j;
-    return -1;
-}
-
 // The large model over nq block rows per sequence (row 0 = pending token, row r = draft r); fin_r: block row whose
 // token the small model's last head GEMM left as per-tile results (-1: none); head: final LayerNorm + output head.
 void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
@@ -1272,17 +1313,14 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
     bool any_fork = false;
     begin_rows<bf16>(c, c.large, h, 0, nq, fin_r, snap_of(0), next_ln(c, c.large, 0));
     const Rows r = decode_rows(c, nq - 1, nq);
-    if (project && project_slot(c, 0) >= 0) { tc_project_forked(c, 0, project_slot(c, 0), r); any_fork = true; }
+    auto run = [&](int j, const float* snap, float* yhat, float* a_j, float* t1) { tc_project(c, j, snap, r, yhat, a_j, t1); };
+    if (project && project_slot(c, 0) >= 0) { project_forked(c, 0, project_slot(c, 0), run); any_fork = true; }
     for (int l = 0; l < c.large.d.n_layers; ++l) {
         tc_decoder_layer(c, c.large, l, h, r, true, snap_of(l + 1));
-        if (project && project_slot(c, l + 1) >= 0) { tc_project_forked(c, l + 1, project_slot(c, l + 1), r); any_fork = true; }
+        if (project && project_slot(c, l + 1) >= 0) { project_forked(c, l + 1, project_slot(c, l + 1), run); any_fork = true; }
     }
     if (head) tc_head(c, c.large, r, at<float>(c, c.lay.logits_large), c.lay.amax_val_large, c.lay.amax_idx_large, true);
-    if (any_fork) {   // the projections join the main stream before the verify kernel
-        cudaEventRecord(c.ev_join, c.side);
-        cudaStreamWaitEvent(c.stream, c.ev_join, 0);
-        c.next_launch_plain = true;
-    }
+    if (any_fork) project_join(c);
 }
 
 // ---- teacher-forced pass (bf16): the prompt pass's kernels with activations as two planes ----------------------------
@@ -1420,7 +1458,7 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
     const bool bf = c.cfg.dtype == TANDEM_DTYPE_BF16;   // one bf16 path: the tensor-core kernels (a bf16 context always has tensor maps)
     if (kind == 3) {
         if (gamma == 0) launch_adaptive_begin(c);
-        if (bf) tc_small_step(c, gamma, false); else fp32_small_step(c, gamma);
+        if (bf) tc_small_step(c, gamma, false); else fp32_small_step(c, gamma, false);
         launch_router(c, gamma, mode);
         return;
     }
@@ -1428,9 +1466,9 @@ void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t se
         if (bf) {
             tc_large_block(c, gamma + 1, gamma, true, true);
         } else {
-            fp32_large_block(c, gamma + 1, true, true);
+            fp32_large_block(c, gamma + 1, gamma, true, true);
         }
-        launch_verify(c, gamma, TANDEM_ACCEPT_NATURAL, 0ull, max_new, bf, true);
+        launch_verify(c, gamma, TANDEM_ACCEPT_NATURAL, 0ull, max_new, true, true);
         c.last_gamma = gamma;
         return;
     }
@@ -1629,6 +1667,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->use_graphs = getenv("TANDEM_NO_GRAPH") == nullptr;
     c->use_pdl = getenv("TANDEM_NO_PDL") == nullptr;
     c->n_sms = sm_count();
+    c->amax_tiles = cfg->dtype == TANDEM_DTYPE_BF16 ? lay.vocab_tiles : cdiv(cfg->large.vocab, GS_WARPS * (rows_wide(*c, cfg->large.vocab) ? 4 : 1));
     if (e == cudaSuccess && cfg->dtype == TANDEM_DTYPE_BF16) {
         // two tensor maps per weight matrix: [out_features][in_features], 128 x 64 tiles and 32 x 64
         c->wmap.resize(c->w.size());
