@@ -386,7 +386,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         split_bf16x2(y.z, y.w, val.y, rem.y);
                     }
                     const int c = (lane & 15) >> 1;
-                    unsigned char* bt = ring + i * C::STAGE_BYTES + C::A_BYTES + ((r & ~15) + r) * 128 + ((c ^ (r & 7)) << 4) + ((lane & 1) << 3);
+                    unsigned char* bt = ring + i * C::STAGE_BYTES + C::A_BYTES + (NB > 16 ? (r & ~15) + r : r) * 128 + ((c ^ (r & 7)) << 4) + ((lane & 1) << 3);
                     *reinterpret_cast<uint2*>(bt) = val;
                     *reinterpret_cast<uint2*>(bt + 16 * 128) = rem;   // (the same swizzle phase)
                 }
@@ -509,7 +509,7 @@ gemm_tc_decode_kernel(const TcDecodeArgs a, const __grid_constant__ CUtensorMap 
                         }
                     }
                     // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8
-                    unsigned char* dst = bt + ((r & ~15) + r) * 128 + ((c ^ (r & 7)) << 4);
+                    unsigned char* dst = bt + (NB > 16 ? (r & ~15) + r : r) * 128 + ((c ^ (r & 7)) << 4);
                     *reinterpret_cast<uint4*>(dst) = val;
                     *reinterpret_cast<uint4*>(dst + 16 * 128) = rem;   // the remainder row of token row r (same swizzle phase)
                 }
