@@ -48,6 +48,8 @@ int cdiv(int a, int b) { return (a + b - 1) / b; }
 // Queries per attention group of the large model in a teacher-forced pass: one group of the MMA's eight columns (a warp meets all
 // keys of its group on its own, so more and lighter warps: 20.5 -> 17.5 us a layer for 772 rows x 16 heads x 64 under ncu).
 constexpr int PASS_GROUP = 8;
+// Most rows of a prompt pass whose projections run beside the large model's layers, see prompt_project_forked.
+constexpr int PROMPT_FORK_ROWS = 2048;
 
 struct Layout {   // byte offsets into the arena
     size_t kv_large, kv_small;
@@ -941,11 +943,31 @@ void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
         if (c.layer_map[j] == n_large_layers_done) project_layer<T>(c, j, r);
 }
 
+// bf16 prompt passes of few rows leave multiprocessors idle: their projections run on the side stream, beside the large model's next
+// layers.  They share the buffers of one projection (and the copy of the residual stream that they read), so the main stream
+// waits for the last ones before the next copy is made, and for all of them at the end of the pass.  (Small pair, 99 / 511 / 1499 rows: 602 -> 567, 759 -> 731, 1279 -> 1235 us;
+// large pair, 899 rows: 1 %.)
+void prompt_project_forked(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
+    cudaStream_t main_stream = c.stream;
+    cudaEvent_t fork = c.ev_fork[0];
+    cudaEventRecord(fork, main_stream);
+    cudaStreamWaitEvent(c.side, fork, 0);
+    c.stream = c.side;
+    c.next_launch_plain = true;   // first kernel after a cross-stream wait
+    project_after<bf16>(c, n_large_layers_done, r);
+    cudaEventRecord(c.ev_join, c.side);
+    c.stream = main_stream;
+}
+void prompt_project_join(tandem_ctx& c) {
+    cudaStreamWaitEvent(c.stream, c.ev_join, 0);
+    c.next_launch_plain = true;
+}
+
 // One decoder layer (Eq. 1; the same form serves the small model's layers in Eq. 2) on residual stream h.  project: the
 // FF_Tandem projections that read h as it enters the layer (they run behind the first LayerNorm, which leaves them a bf16
 // copy of h on its way).  snap (fp32 decode passes): copy of x^(l+1) when an FF_Tandem projection reads it.
 template <typename T>
-void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool project = false, float* snap = nullptr) {
+void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r, bool project = false, float* snap = nullptr, bool fork = false) {
     const int d = m.d.d_model, dff = m.d.d_ff;
     T* a = at<T>(c, c.lay.a);
     T* q = at<T>(c, c.lay.q);
@@ -968,7 +990,7 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
         }
     }
     launch_layernorm<T>(c, r.M, h, g1, b1, a, d, project && sizeof(T) == 2 ? at<bf16>(c, c.lay.xb) : nullptr);
-    if (project) project_after<T>(c, l, r);
+    if (project) { if (fork) prompt_project_forked(c, l, r); else project_after<T>(c, l, r); }
     launch_gemm<T, EPI_QKV>(c, a, d, r.M, qkv, epi_cache<T>(c, m, l, q));
     attention<T>(c, m, l, q, o, r);
     launch_gemm<T, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
@@ -991,7 +1013,15 @@ template <typename T>
 void large_layers(tandem_ctx& c, const Rows& r, bool project) {
     float* h = at<float>(c, c.lay.h_large);
     const int n = c.large.d.n_layers;
-    for (int l = 0; l < n; ++l) decoder_layer<T>(c, c.large, l, h, r, project && projects_from(c, l));
+    const bool fork = sizeof(T) == 2 && project && r.M <= PROMPT_FORK_ROWS;
+    bool forked = false;
+    for (int l = 0; l < n; ++l) {
+        const bool here = project && projects_from(c, l);
+        if (here && forked) prompt_project_join(c);
+        decoder_layer<T>(c, c.large, l, h, r, here, nullptr, fork);
+        forked = forked || (here && fork);
+    }
+    if (forked) prompt_project_join(c);
     if (!project || !projects_from(c, n)) return;
     if constexpr (sizeof(T) == 2) {   // after the last layer no LayerNorm of the large model follows
         const size_t elems = (size_t)r.M * c.large.d.d_model;
