@@ -784,12 +784,18 @@ void launch_attn_decode(tandem_ctx& c, int d_head, const AttnArgs& a0, int group
     else launch_attn_decode_dq<128>(c, a, groups, cl, pass, kv_bytes);
 }
 
-// raw (bf16 only, nullable): also leaves a bf16 copy of the rows as they are.
-template <typename T>
-void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr) {
-    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + sizeof(T) + (raw ? 2.0 : 0.0)));
-    launch_ex(c, true, 1, layernorm_rows_kernel<T>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain), static_cast<const float*>(bias), out, d,
-              M, raw, (size_t)0);
+// raw (bf16 only, nullable): also leaves a bf16 copy of the rows as they are.  PL: both as two planes, the remainders `lo` elements behind.
+template <typename T, bool PL = false>
+void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr, size_t lo = 0) {
+    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + (PL ? 2 : 1) * (sizeof(T) + (raw ? 2.0 : 0.0))));
+    const float *g = static_cast<const float*>(gain), *b = static_cast<const float*>(bias);
+    // a warp per row where there are more rows than multiprocessors (a block per row is a shorter chain for a few: 40 rows of 768
+    // beside the two products of a stand-alone projection 11.7 us, 11.9 with a warp each)
+    auto by_warps = [&](auto kernel) { launch_ex(c, true, 1, kernel, dim3(std::min(cdiv(M, 4), 4 * c.n_sms)), dim3(128), 0, x, g, b, out, d, M, raw, lo); };
+    if (M > c.n_sms && d <= 1024) by_warps(layernorm_warp_kernel<T, PL, 8>);
+    else if (M > c.n_sms && d <= LNW_MAX) by_warps(layernorm_warp_kernel<T, PL, 16>);
+    else
+        launch_ex(c, true, 1, layernorm_rows_kernel<T, PL>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, g, b, out, d, M, raw, lo);
 }
 
 // Describes the rows of one pass.
@@ -1362,9 +1368,7 @@ void pass_gemm(tandem_ctx& c, const bf16* x, int M, const TcW& w, EpiArgs e, con
     if (launch_tc_tiled<EPI, true>(c, x, w.K, M, w, e, c.st.counters + 2, c.lay.fr_rows, sc) != TANDEM_OK) c.setup_failed = true;
 }
 void pass_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, bf16* out, int d, bf16* raw = nullptr) {
-    ProfScope ps(c, PC_LAYERNORM, (double)M * d * (raw ? 12.0 : 8.0));
-    launch_ex(c, true, 1, layernorm_rows_kernel<bf16, true>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, static_cast<const float*>(gain),
-              static_cast<const float*>(bias), out, d, M, raw, (size_t)c.lay.fr_rows * d);
+    launch_layernorm<bf16, true>(c, M, x, gain, bias, out, d, raw, (size_t)c.lay.fr_rows * d);
 }
 
 // FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.
@@ -2557,8 +2561,7 @@ extern "C" tandem_status tandem_ff_tandem_project(const void* x, const void* w_t
     if (rows <= 8 && d_small <= 1024) {
         launch_tc_decode<PRO_LN, EPI_KV>(tmp, ts, yhat, d_small, ln_g, ln_b, rows, wkv, true, e);
     } else {
-        launch_ex(tmp, true, 1, layernorm_rows_kernel<float>, dim3(rows), dim3(128), 0, (const float*)yhat, static_cast<const float*>(ln_g),
-                  static_cast<const float*>(ln_b), a_s, (int)d_small, (int)rows, (bf16*)nullptr, (size_t)0);
+        launch_layernorm<float>(tmp, rows, yhat, ln_g, ln_b, a_s, d_small);
         launch_tc_decode<PRO_F32, EPI_KV>(tmp, ts, a_s, d_small, nullptr, nullptr, rows, wkv, true, e);
     }
     return check_launch();

@@ -81,6 +81,15 @@ def test_bf16_prompt_gemm_between_the_two_kernels(lens):
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=20), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 2
 
 
+@pytest.mark.parametrize("width,heads,lens", [(992, 31, [160]), (1024, 16, [151]), (1056, 33, [150, 2]), (2048, 32, [150]), (2080, 65, [151])])
+def test_bf16_prompt_layernorm_by_warps_and_blocks(width, heads, lens):
+    """Around the rules that give a row of a prompt pass a warp (more rows than multiprocessors, up to 1024 and 2048 elements) or a
+    block: 149 to 159 rows, lanes without a last float4, and the copy of the rows that a projection reads."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, heads, 64), small=(1, 64, 1, 64), max_pos=192, layer_map=(0,))
+    w = _bf16_weights(shape, seed=27, std=0.02)
+    assert _replay_compare(shape, w, prompts_for(shape, lens, seed=28), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 2
+
+
 @pytest.mark.parametrize("heads", [2, 1])   # head sizes 64 and 128: chunks of 64 and of 128 keys
 def test_bf16_prompt_attention_at_chunk_edges(heads):
     """Prompts that end one query before, at and behind the end of a chunk, a tile and a group of two tiles, in one batch."""
