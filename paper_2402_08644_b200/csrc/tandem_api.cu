@@ -1827,6 +1827,10 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     for (long long i = 0; i < total_ids; ++i)
         if (prompt_ids[i] < 0 || prompt_ids[i] >= c->cfg.large.vocab) return TANDEM_ERR_INVALID_ARG;
 
+    // Queries per attention group: two tiles of 128 for a CTA of the tensor-core kernel, one where that leaves more than half of the
+    // multiprocessors without a CTA (small pair's prompt passes of 512 / 900 tokens, 16 heads: 696 -> 685, 884 -> 848 us).
+    int group = c->prompt_group;
+    if (c->tc_prompt_attn && (rows / ATC_Q + n_queries) * c->cfg.large.n_heads * 2 <= c->n_sms) group = ATC_TILE;
     // The pass is enqueued behind whatever the stream still runs; only the staging buffer has to be free again, which it is
     // as soon as the previous pass's copy has gone.  (Everything else that uses the buffer waits before it returns.)
     CK(cudaEventSynchronize(c->ev_staged));
@@ -1839,7 +1843,7 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
         p_len[q] = prompt_lens[q]; p_id[q] = (int)off; p_row[q] = m; p_grp[q] = groups;
         off += prompt_lens[q];
         m += prompt_lens[q] - 1;
-        groups += cdiv(prompt_lens[q] - 1, c->prompt_group);
+        groups += cdiv(prompt_lens[q] - 1, group);
     }
     memcpy(p_ids, prompt_ids, (size_t)total_ids * 4);
     cudaStream_t s = c->stream;
@@ -1854,7 +1858,7 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     PromptStage ps;
     ps.len = at<int>(*c, c->lay.stage); ps.id_off = ps.len + n_queries; ps.row_off = ps.id_off + n_queries; ps.grp_off = ps.row_off + n_queries;
     ps.ids = ps.grp_off + n_queries;
-    ps.n_queries = n_queries; ps.samples = samples; ps.rows = M; ps.group = c->prompt_group;
+    ps.n_queries = n_queries; ps.samples = samples; ps.rows = M; ps.group = group;
     const bool bf = c->cfg.dtype == TANDEM_DTYPE_BF16;
     {
         ProfScope prof(*c, PC_ROWS, (double)M * c->large.d.d_model * (4.0 + 2 * c->esz));
