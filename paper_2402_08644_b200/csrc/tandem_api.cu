@@ -789,11 +789,11 @@ template <typename T, bool PL = false>
 void launch_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, T* out, int d, bf16* raw = nullptr, size_t lo = 0) {
     ProfScope ps(c, PC_LAYERNORM, (double)M * d * (4.0 + (PL ? 2 : 1) * (sizeof(T) + (raw ? 2.0 : 0.0))));
     const float *g = static_cast<const float*>(gain), *b = static_cast<const float*>(bias);
-    // a warp per row where there are more rows than multiprocessors (a block per row is a shorter chain for a few: 40 rows of 768
-    // beside the two products of a stand-alone projection 11.7 us, 11.9 with a warp each)
+    // A warp per row beyond 256 rows, which no decode pass has (those keep one order of the sums whatever their rows); for a few rows
+    // a block each is the shorter chain (40 rows of 768 between the two products of a stand-alone projection 11.7 us, 11.9 with a warp each).
     auto by_warps = [&](auto kernel) { launch_ex(c, true, 1, kernel, dim3(std::min(cdiv(M, 4), 4 * c.n_sms)), dim3(128), 0, x, g, b, out, d, M, raw, lo); };
-    if (M > c.n_sms && d <= 1024) by_warps(layernorm_warp_kernel<T, PL, 8>);
-    else if (M > c.n_sms && d <= LNW_MAX) by_warps(layernorm_warp_kernel<T, PL, 16>);
+    if (M > 256 && d <= 1024) by_warps(layernorm_warp_kernel<T, PL, 8>);
+    else if (M > 256 && d <= LNW_MAX) by_warps(layernorm_warp_kernel<T, PL, 16>);
     else
         launch_ex(c, true, 1, layernorm_rows_kernel<T, PL>, dim3(std::min(M, 4 * std::max(1, c.n_sms))), dim3(128), 0, x, g, b, out, d, M, raw, lo);
 }

@@ -81,11 +81,11 @@ def test_bf16_prompt_gemm_between_the_two_kernels(lens):
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=20), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 2
 
 
-@pytest.mark.parametrize("width,heads,lens", [(992, 31, [160]), (1024, 16, [151]), (1056, 33, [150, 2]), (2048, 32, [150]), (2080, 65, [151])])
+@pytest.mark.parametrize("width,heads,lens", [(992, 31, [258]), (1024, 16, [257]), (1056, 33, [250, 9]), (2048, 32, [262]), (2080, 65, [259])])
 def test_bf16_prompt_layernorm_by_warps_and_blocks(width, heads, lens):
-    """Around the rules that give a row of a prompt pass a warp (more rows than multiprocessors, up to 1024 and 2048 elements) or a
-    block: 149 to 159 rows, lanes without a last float4, and the copy of the rows that a projection reads."""
-    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, heads, 64), small=(1, 64, 1, 64), max_pos=192, layer_map=(0,))
+    """Around the rules that give a row of a prompt pass a warp (more than 256 rows, up to 1024 and 2048 elements) or a
+    block: 256 to 261 rows, lanes without a last float4, and the copy of the rows that a projection reads."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, heads, 64), small=(1, 64, 1, 64), max_pos=288, layer_map=(0,))
     w = _bf16_weights(shape, seed=27, std=0.02)
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=28), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 2
 
