@@ -1303,11 +1303,13 @@ void tc_head(tandem_ctx& c, const Model& m, const Rows& r, float* logits, size_t
 
 // sampled: the previous draft was drawn by sample_draft_kernel (it is in the loop state already), not left as per-tile
 // arg-max results.
-void tc_small_step(tandem_ctx& c, int s, bool sampled) {
+enum StepPart { STEP_WHOLE, STEP_HEAD, STEP_TAIL };   // all of a draft step; its row set-up and first layer; the rest
+void tc_small_step(tandem_ctx& c, int s, bool sampled, StepPart part = STEP_WHOLE) {
     float* y = at<float>(c, c.lay.h_small);
-    begin_rows<bf16>(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1, nullptr, next_ln(c, c.small, 0));
+    if (part != STEP_TAIL) begin_rows<bf16>(c, c.small, y, s, 1, (s > 0 && !sampled) ? s : -1, nullptr, next_ln(c, c.small, 0));
     const Rows r = decode_rows(c, s, 1);
-    for (int j = 0; j < c.small.d.n_layers; ++j) tc_decoder_layer(c, c.small, j, y, r, false);
+    for (int j = part == STEP_TAIL ? 1 : 0; j < (part == STEP_HEAD ? 1 : c.small.d.n_layers); ++j) tc_decoder_layer(c, c.small, j, y, r, false);
+    if (part == STEP_HEAD) return;
     float* logits = at<float>(c, c.lay.logits_small) + (size_t)s * c.batch * c.small.d.vocab;
     tc_head(c, c.small, r, logits, c.lay.amax_val_small, c.lay.amax_idx_small, false);
 }
@@ -1488,12 +1490,14 @@ tandem_status check_launch(tandem_ctx& c) {
 // kind 0: draft + verify (gamma drafts, accept mode);  1: plain greedy M_L;
 // kind 3: one draft step of the adaptive block length (gamma = step index, mode = gamma_max) followed by the router;
 // kind 4: the verify half of an adaptive iteration (gamma = longest block of the batch).
+// bf16: kind 3 is the step's row set-up and first layer, kind 5 (same arguments) the rest of it and the router.
 void enqueue_iteration(tandem_ctx& c, int kind, int gamma, int mode, uint64_t seed, int max_new) {
     const bool bf = c.cfg.dtype == TANDEM_DTYPE_BF16;   // one bf16 path: the tensor-core kernels (a bf16 context always has tensor maps)
-    if (kind == 3) {
-        if (gamma == 0) launch_adaptive_begin(c);
-        if (bf) tc_small_step(c, gamma, false); else fp32_small_step(c, gamma, false);
-        launch_router(c, gamma, mode);
+    if (kind == 3 || kind == 5) {
+        if (kind == 3 && gamma == 0) launch_adaptive_begin(c);
+        if (!bf) fp32_small_step(c, gamma, false);
+        else tc_small_step(c, gamma, false, kind == 3 ? STEP_HEAD : STEP_TAIL);
+        if (!bf || kind == 5) launch_router(c, gamma, mode);
         return;
     }
     if (kind == 4) {
@@ -1521,10 +1525,12 @@ tandem_status launch_iteration(tandem_ctx& c, int kind, int gamma, int mode, uin
     c.chunks_launch = std::min(c.lay.n_chunks_max, (need + 3) / 4 * 4);
     if (c.cfg.dtype == TANDEM_DTYPE_BF16)
         c.chunks_launch = 1;   // the cluster attention's grid does not depend on the context length: one graph serves all
-    if (kind == 3) c.router_ticket++; else c.ticket++;   // what the host will wait for: the router's or the verify kernel's publication
-    if (kind != 3) c.last_gamma = kind == 1 ? 0 : gamma;   // (set here, not while enqueueing: a replayed graph enqueues nothing on the host)
-    // (a draft step of the adaptive block length starts when the host has seen the router's answer to the one before: a graph's
-    // launch would add its latency to every step, 12.8 ms against 11.5 ms for 48 tokens of the small pair)
+    if (kind == 3) c.router_ticket++; else if (kind != 5) c.ticket++;   // what the host will wait for: the router's or the verify kernel's publication
+    if (kind != 3 && kind != 5) c.last_gamma = kind == 1 ? 0 : gamma;   // (set here, not while enqueueing: a replayed graph enqueues nothing on the host)
+    // (A draft step of the adaptive block length starts when the host has seen the router's answer to the one before: a graph of all of
+    // it would add its launch's latency to every step, 12.8 ms against 11.5 ms for 48 tokens of the small pair, and launched one by one
+    // its kernels come slower than the GPU runs them.  So the first layer's kernels go out by themselves, the rest as a graph
+    // behind them: 10.40 -> 10.16 ms.)
     if (c.prof.on || !c.use_graphs || kind == 3) {
         enqueue_iteration(c, kind, gamma, mode, seed, max_new);
         return check_launch();
@@ -2050,6 +2056,7 @@ tandem_status adaptive_iteration(tandem_ctx* c, int gamma_max, int max_new, int*
     int s = 0;
     for (; s < gamma_max; ++s) {
         TRY(launch_iteration(*c, 3, s, gamma_max, 0ull, max_new));
+        if (c->cfg.dtype == TANDEM_DTYPE_BF16) TRY(launch_iteration(*c, 5, s, gamma_max, 0ull, max_new));
         TRY(wait_ticket(*c, c->router_ticket, 5));
         if (c->hflags[6] <= 0) { ++s; break; }
     }
@@ -2082,6 +2089,8 @@ extern "C" tandem_status tandem_set_router(tandem_ctx* c, int32_t top_k, int32_t
     if (((uintptr_t)w1 | (uintptr_t)b1 | (uintptr_t)w2) & 3) return TANDEM_ERR_INVALID_ARG;
     if (sizeof(float) * (size_t)(1 + top_k + (size_t)top_k * c->cfg.small.d_model) > 48 * 1024) return TANDEM_ERR_SHAPE;   // the feature vector sits in shared memory
     CK(cudaStreamSynchronize(c->stream));   // the caller may release the former router's weights
+    for (auto& g : c->graphs)               // (they are arguments of the captured draft steps)
+        if (g.kind == 5 && g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
     c->router.w1 = static_cast<const float*>(w1); c->router.b1 = static_cast<const float*>(b1); c->router.w2 = static_cast<const float*>(w2);
     c->router.b2 = b2; c->router.tau = tau; c->router.k = top_k; c->router.hidden = hidden;
     c->has_router = true;
