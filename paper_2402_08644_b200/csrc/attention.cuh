@@ -38,7 +38,7 @@ struct AttnArgs {
                                                //   (a stand-alone call: whatever precedes it may be writing the keys and values)
     const int* grp_row0; const int* grp_cnt;   // nullable: then group g = rows g*nq .. g*nq+nq-1
     int nq;
-    int units;                           // ATD_PASS: groups * head groups = warps
+    int units, log_parts;                // ATD_PASS: groups * head groups; 2^log_parts warps (1, 2 or 4) share the keys of each
     int n_heads, t_max;
     int n_kv_heads;                      // key/value heads of the caches; 0 = n_heads.  Query head h reads kv head h / (n_heads / n_kv_heads)
     int* err_flag;                       // attn_decode_kernel: where a bounded wait that ran out records its code (nullable)
@@ -361,7 +361,8 @@ __device__ __forceinline__ uint32_t atd_pack_bf16x2(float lo, float hi) {
 // NT: groups of eight query columns in use (1 up to eight rows per CTA, 2 up to 16).
 // MODE: ATD_CLUSTERED, CL in {2, 4, 8}; ATD_ALONE, CL = 1, results straight from the fold of the warps' states (32 x 16 x 64 x 8194:
 // 171 -> 165 us, without the trip through the inbox); ATD_PASS, a teacher-forced pass: groups of unequal length, the second segment of a block's own keys,
-// and a warp on its own per group and head, since there are hundreds of them over short contexts (grid: warps in all / 8; 49 groups x 16
+// and a warp on its own per group and head, since there are hundreds of them over short contexts, or two or four that deal its tiles and merge
+// their states through shared memory where fewer units leave the chip a long chain each (grid: warps in all / 8; one warp each: 49 groups x 16
 // heads x 64 over up to 257 positions: 25 -> 20 us under ncu, 193 blocks of four rows x 8 heads 26 -> 17 us).  (The same code with these choices made at run time costs the stand-alone call on 1 x 16 x 64 x 1028 3.5 %: 5.58 -> 5.78 us.)
 enum { ATD_CLUSTERED = 0, ATD_ALONE = 1, ATD_PASS = 2 };
 template <int DH, int NT, int MODE>
@@ -380,7 +381,8 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // Grouped-query attention: the tile's 16 rows hold the block's queries of `gpc` query heads that share one
     // key/value head (row = head * nq + block row), so their keys and values are streamed once for all of them.
     const int gpc = a.heads_per_cta > 0 ? a.heads_per_cta : 1;
-    const int head_groups = a.n_heads / gpc, unit = MODE == ATD_PASS ? blockIdx.x * NW + warp : 0;   // ATD_PASS: this warp's number
+    const int log_parts = MODE == ATD_PASS ? a.log_parts : 0, part = warp & ((1 << log_parts) - 1);   // ATD_PASS: this warp's share of its unit's tiles
+    const int head_groups = a.n_heads / gpc, unit = MODE == ATD_PASS ? (blockIdx.x * NW + warp) >> log_parts : 0;
     if (MODE == ATD_PASS && unit >= a.units) return;
     const int g = MODE == ATD_PASS ? unit / head_groups : blockIdx.z;
     const int h = (MODE == ATD_PASS ? unit - g * head_groups : blockIdx.y) * gpc;   // first query head of this CTA (warp)
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
     const int pos_last = pos_first + nq - 1;
     const int n_chunks = pos_last / ATT_CH + 1;
-    const int n_mine = MODE == ATD_PASS ? pos_last / ATD_WROWS + 1 : rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
+    const int n_mine = MODE == ATD_PASS ? (pos_last / ATD_WROWS + (1 << log_parts) - part) >> log_parts : rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
     const size_t head_base2 = ((size_t)b * n_kv + kvh) * (MODE == ATD_PASS ? a.t_max : a.t_max2);
     const int split = a.k2 ? (MODE == ATD_PASS ? pos_first : a.split) : INT_MAX;
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
     // boundary tile or two) takes the short way: one base address, constant steps.
     constexpr int RSTEP = 32 / C::TPK;             // rows between a lane's consecutive units
     const int i_row = lane / C::TPK, i_unit = lane - i_row * C::TPK;
-    auto tile_start = [&](int it) { return MODE == ATD_PASS ? it * ATD_WROWS : (rank + it * CL) * ATT_CH + warp * ATD_WROWS; };
+    auto tile_start = [&](int it) { return MODE == ATD_PASS ? ((it << log_parts) + part) * ATD_WROWS : (rank + it * CL) * ATT_CH + warp * ATD_WROWS; };
     auto issue = [&](int it) {
         const int t0 = tile_start(it);
         bf16* ks = ring + (size_t)(it % C::STAGES) * C::STAGE_ELEMS;
@@ -602,7 +604,7 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             static_cast<bf16*>(a.out)[oi] = __float2bfloat16_rn(res);
         }
     };
-    if constexpr (MODE == ATD_PASS) {   // the warp has met all keys: results straight from its registers
+    if (MODE == ATD_PASS && log_parts == 0) {   // the warp has met all keys: results straight from its registers
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -638,6 +640,23 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
             for (int mt = 0; mt < C::KSTEPS; ++mt) { st[mt * 16] = o[nt][mt][e]; st[mt * 16 + 8] = o[nt][mt][2 + e]; }
             if (lane < 4) { st[DH] = m[nt][e]; st[DH + 1] = lr; }
         }
+    if constexpr (MODE == ATD_PASS) {   // the unit's warps fold their states (all of them are here: units end with their last warp)
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (warp >> log_parts)), "r"(32 << log_parts) : "memory");
+        const float* st = wst + (warp - part) * WST;
+        for (int i = part * 32 + lane; i < cnt * DH; i += 32 << log_parts) {
+            const int qa = i / DH, e = i - qa * DH;
+            float mx = -INFINITY, val = 0.f, lsum = 0.f;
+            for (int w = 0; w < 1 << log_parts; ++w) mx = fmaxf(mx, st[w * WST + qa * SW + DH]);
+            for (int w = 0; w < 1 << log_parts; ++w) {
+                const float* sw = st + w * WST + qa * SW;
+                const float f = sw[DH] > -INFINITY ? __expf(sw[DH] - mx) : 0.f;
+                val = fmaf(sw[e], f, val);
+                lsum = fmaf(sw[DH + 1], f, lsum);
+            }
+            store(qa, e, val / lsum);
+        }
+        return;
+    }
     __syncthreads();
     // fold the warps' states in warp order and send the CTA's state of query qa to CTA qa & (CL - 1)
     if (CL > 1) cluster_wait();   // closes the opening handshake: every CTA of the cluster is running

@@ -716,7 +716,11 @@ void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl,
     if (pass) {
         AttnArgs w = a;
         w.units = groups * (a.n_heads / gpc);
-        const dim3 warps(cdiv(w.units, ATD_WARPS));
+        // Up to four warps share a unit's keys as long as all warps run at the same time (two CTAs per multiprocessor): one sequence of 257 tokens
+        // through the small pair 1226 -> 1165 us with four (1185 with two), of 64 tokens 988 -> 967.  Beyond that the merge only
+        // adds work: eight of 400 tokens 3325 us with one, 3530 with two, 3655 with four.
+        while (w.log_parts < 2 && w.units * 2 << w.log_parts <= 2 * ATD_WARPS * c.n_sms) ++w.log_parts;
+        const dim3 warps(cdiv(w.units << w.log_parts, ATD_WARPS));
         if (narrow) launch_attn_decode_as<DH, 1, ATD_PASS>(c, w, warps, 1); else launch_attn_decode_as<DH, 2, ATD_PASS>(c, w, warps, 1);
     }
     else if (cl == 1) { if (narrow) launch_attn_decode_as<DH, 1, ATD_ALONE>(c, a, grid, cl); else launch_attn_decode_as<DH, 2, ATD_ALONE>(c, a, grid, cl); }

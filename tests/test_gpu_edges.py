@@ -140,7 +140,9 @@ def test_decode_attention_by_lone_ctas(batch, heads, dh, derived, own):
     ([2, 140, 23], 4, 0, dict(layer_map=(1, 3), vocab=129)),                     # one pass of 168 rows: three groups, the last of 40; a head tile of one feature
     ([131, 7, 66], 3, 20, dict(layer_map=(0, 2))),                               # passes of 12 rows: a sequence over many of them
     ([47], 15, 0, dict(large=(2, 256, 2, 264), small=(1, 256, 2, 136), kv_heads=(1, 1), layer_map=(2,))),   # blocks of 15, 128-wide heads, shared keys / values
-    ([66, 2], 1, 0, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3), small=(2, 192, 6, 136)))])  # 66 blocks of one row; a small model wider than the large one
+    ([66, 2], 1, 0, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3), small=(2, 192, 6, 136))),  # 66 blocks of one row; a small model wider than the large one
+    ([141], 1, 0, dict(layer_map=(0, 3), small=(2, 192, 6, 136))),               # 840 block heads: two warps share the keys of each (four up to 592)
+    ([130, 70], 1, 0, dict(layer_map=(0, 3), small=(2, 192, 6, 136)))])          # 1188: one warp each (two up to 1184)
 def test_bf16_teacher_forced_pass(lens, gamma, prefill_rows, kw):
     """All blocks of a teacher-forced forward in one pass or a few: ragged sequences padded to whole blocks, groups of 64 rows, blocks
     that attend large-derived keys up to their start and their own from there."""
