@@ -57,6 +57,7 @@ struct Layout {   // byte offsets into the arena
     size_t st_block_len, st_drafting, st_confidence;
     size_t forced_ids, forced_len, forced_nll, forced_top;   // teacher-forced forward: given tokens [B][T], lengths [B], scores [B][T]
     size_t fr_x, fr_o, fr_f, fr_q, fr_raw, fr_yhat, fr_a, fr_t1;
+    size_t fk_raw, fk_yhat, fk_a, fk_t1;            // the projections' buffers in a pass of at most fk_rows rows, whose projections run beside M_L's layers
     size_t fr_seq, fr_truth, fr_out, fr_truth_val, fr_grp, fr_tiles, fr_kv;   // ... in one pass (bf16), see ForcedRows: offsets / lengths / first rows, next tokens, score places,
                                                                               // true logits, attention groups, the head's per-tile results, the small model's own keys / values of one layer
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
@@ -70,7 +71,7 @@ struct Layout {   // byte offsets into the arena
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles, score_tiles;
-    int fr_rows, fr_head_rows;               // rows of a teacher-forced pass, and of one run of its output head
+    int fr_rows, fk_rows, fr_head_rows;      // rows of a teacher-forced pass, of one whose projections are forked, and of one run of its output head
     size_t kv_large_layer, kv_small_layer;   // elements per (layer, k-or-v)
 };
 
@@ -262,6 +263,9 @@ Layout make_layout(const tandem_config& c) {
     off = L.fr_f;
     L.fr_q = take(RF * dmax * 2);
     off = std::max(std::max(off, fr_proj_end), std::max(fr_end, ws_end));
+    const size_t RK = std::min<size_t>(RF, PROMPT_FORK_ROWS);
+    L.fk_rows = (int)RK;
+    L.fk_raw = take(RK * c.large.d_model * 4); L.fk_t1 = take(RK * hidden * 4); L.fk_yhat = take(RK * c.small.d_model * 4); L.fk_a = take(RK * c.small.d_model * 4);
     L.logits_large = take(RD * V * 4);
     L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.part_ml = take(RD * hmax * L.n_chunks_max * 2 * 4);
@@ -811,6 +815,7 @@ struct Rows {
     int n_chunks;     // split attention grid size along the context
     double kv_positions;   // context positions read by one attention launch, summed over sequences (accounting only)
     bool whole_pass = false;            // a teacher-forced pass (see forced_pass)
+    int plane = 0;                      // ... rows between its planes of values and of remainders
     const int *grp_row0 = nullptr, *grp_cnt = nullptr;   // ... its attention groups of unequal length, else groups of nq rows
     bf16 *own_k = nullptr, *own_v = nullptr;             // ... the small model's keys / values of its own, beside the large-derived ones in the cache
 };
@@ -957,14 +962,15 @@ void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
 // layers.  They share the buffers of one projection (and the copy of the residual stream that they read), so the main stream
 // waits for the last ones before the next copy is made, and for all of them at the end of the pass.  (Small pair, 99 / 511 / 1499 rows: 602 -> 567, 759 -> 731, 1279 -> 1235 us;
 // large pair, 899 rows: 1 %.)
-void prompt_project_forked(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
+template <typename P>
+void prompt_project_forked(tandem_ctx& c, P project) {
     cudaStream_t main_stream = c.stream;
     cudaEvent_t fork = c.ev_fork[0];
     cudaEventRecord(fork, main_stream);
     cudaStreamWaitEvent(c.side, fork, 0);
     c.stream = c.side;
     c.next_launch_plain = true;   // first kernel after a cross-stream wait
-    project_after<bf16>(c, n_large_layers_done, r);
+    project();
     cudaEventRecord(c.ev_join, c.side);
     c.stream = main_stream;
 }
@@ -1000,7 +1006,7 @@ void decoder_layer(tandem_ctx& c, const Model& m, int l, float* h, const Rows& r
         }
     }
     launch_layernorm<T>(c, r.M, h, g1, b1, a, d, project && sizeof(T) == 2 ? at<bf16>(c, c.lay.xb) : nullptr);
-    if (project) { if (fork) prompt_project_forked(c, l, r); else project_after<T>(c, l, r); }
+    if (project) { if (fork) prompt_project_forked(c, [&] { project_after<T>(c, l, r); }); else project_after<T>(c, l, r); }
     launch_gemm<T, EPI_QKV>(c, a, d, r.M, qkv, epi_cache<T>(c, m, l, q));
     attention<T>(c, m, l, q, o, r);
     launch_gemm<T, EPI_RESID>(c, o, d, r.M, wo, epi_plain(h, d));
@@ -1367,58 +1373,67 @@ void tc_large_block(tandem_ctx& c, int nq, int fin_r, bool project, bool head) {
 
 // ---- teacher-forced pass (bf16): the prompt pass's kernels with activations as two planes ----------------------------
 
-// What a pass's maps read: two planes of fr_rows rows of K elements.
+// What a pass's maps read: two planes of `plane` rows of K elements.
 template <int EPI>
-void pass_gemm(tandem_ctx& c, const bf16* x, int M, const TcW& w, EpiArgs e, const TcScore& sc = TcScore()) {
-    if (EPI == EPI_GELU) e.out_lo = static_cast<bf16*>(e.out) + (size_t)c.lay.fr_rows * e.ldo;
-    if (launch_tc_tiled<EPI, true>(c, x, w.K, M, w, e, c.st.counters + 2, c.lay.fr_rows, sc) != TANDEM_OK) c.setup_failed = true;
+void pass_gemm(tandem_ctx& c, const bf16* x, int M, int plane, const TcW& w, EpiArgs e, const TcScore& sc = TcScore()) {
+    if (EPI == EPI_GELU) e.out_lo = static_cast<bf16*>(e.out) + (size_t)plane * e.ldo;
+    if (launch_tc_tiled<EPI, true>(c, x, w.K, M, w, e, c.st.counters + 2, plane, sc) != TANDEM_OK) c.setup_failed = true;
 }
-void pass_layernorm(tandem_ctx& c, int M, const float* x, const void* gain, const void* bias, bf16* out, int d, bf16* raw = nullptr) {
-    launch_layernorm<bf16, true>(c, M, x, gain, bias, out, d, raw, (size_t)c.lay.fr_rows * d);
+void pass_layernorm(tandem_ctx& c, int M, int plane, const float* x, const void* gain, const void* bias, bf16* out, int d, bf16* raw = nullptr) {
+    launch_layernorm<bf16, true>(c, M, x, gain, bias, out, d, raw, (size_t)plane * d);
 }
+
+// Whether a pass's projections run on the side stream, beside the large model's next layers (see prompt_project_forked; 772 rows of the small
+// pair 1548 -> 1515 us, 256 rows 1164 -> 1111, 600 rows 1984 -> 1921).
+bool pass_forks(const tandem_ctx& c, const Rows& r) { return r.M <= c.lay.fk_rows; }
 
 // FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.
 void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r) {
     const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    float* yhat = at<float>(c, c.lay.fr_yhat);
-    bf16 *a_j = at<bf16>(c, c.lay.fr_a), *t1 = at<bf16>(c, c.lay.fr_t1);
+    const bool fork = pass_forks(c, r);
+    float* yhat = at<float>(c, fork ? c.lay.fk_yhat : c.lay.fr_yhat);
+    bf16 *a_j = at<bf16>(c, fork ? c.lay.fk_a : c.lay.fr_a), *t1 = at<bf16>(c, fork ? c.lay.fk_t1 : c.lay.fr_t1);
     if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
-        pass_gemm<EPI_STORE_F32>(c, x, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), epi_plain(yhat, dS));
+        pass_gemm<EPI_STORE_F32>(c, x, r.M, r.plane, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), epi_plain(yhat, dS));
     } else {
-        pass_gemm<EPI_GELU>(c, x, r.M, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), epi_plain(t1, c.hidden));
-        pass_gemm<EPI_STORE_F32>(c, t1, r.M, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden), epi_plain(yhat, dS));
+        pass_gemm<EPI_GELU>(c, x, r.M, r.plane, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), epi_plain(t1, c.hidden));
+        pass_gemm<EPI_STORE_F32>(c, t1, r.M, r.plane, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden), epi_plain(yhat, dS));
     }
-    pass_layernorm(c, r.M, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), a_j, dS);
-    pass_gemm<EPI_KV>(c, a_j, r.M, tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS), epi_cache<bf16>(c, c.small, j, nullptr));
+    pass_layernorm(c, r.M, r.plane, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), a_j, dS);
+    pass_gemm<EPI_KV>(c, a_j, r.M, r.plane, tcw(c, wi_layer(c.small, j, W_WK), wi_layer(c.small, j, W_WV), -1, c.small.d_kv, dS), epi_cache<bf16>(c, c.small, j, nullptr));
 }
 
 // One model's layers over a pass's rows in the residual stream h (and the large model's projections between them).
 void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
     const int d = m.d.d_model, dff = m.d.d_ff, n = m.d.n_layers;
-    bf16 *x = at<bf16>(c, c.lay.fr_x), *o = at<bf16>(c, c.lay.fr_o), *f = at<bf16>(c, c.lay.fr_f), *q = at<bf16>(c, c.lay.fr_q), *raw = at<bf16>(c, c.lay.fr_raw);
-    const bool large = &m == &c.large;
+    bf16 *x = at<bf16>(c, c.lay.fr_x), *o = at<bf16>(c, c.lay.fr_o), *f = at<bf16>(c, c.lay.fr_f), *q = at<bf16>(c, c.lay.fr_q), *raw = at<bf16>(c, pass_forks(c, r) ? c.lay.fk_raw : c.lay.fr_raw);
+    const bool large = &m == &c.large, fork = large && pass_forks(c, r);
+    bool forked = false;
     auto project = [&](int l) {
         for (int j = 0; j < c.small.d.n_layers; ++j)
             if (c.layer_map[j] == l) pass_project(c, j, raw, r);
     };
     for (int l = 0; l < n; ++l) {
         const bool from_here = large && projects_from(c, l);
-        pass_layernorm(c, r.M, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), x, d, from_here ? raw : nullptr);
-        if (from_here) project(l);
+        if (from_here && forked) prompt_project_join(c);   // (raw is written again)
+        pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), x, d, from_here ? raw : nullptr);
+        if (from_here) { if (fork) prompt_project_forked(c, [&] { project(l); }); else project(l); }
+        forked = forked || (from_here && fork);
         EpiArgs eq = epi_cache<bf16>(c, m, l, q);
         if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; }
-        pass_gemm<EPI_QKV>(c, x, r.M, tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), eq);
-        attention_decode(c, m, l, q, o, o + (size_t)c.lay.fr_rows * d, r);
-        pass_gemm<EPI_RESID>(c, o, r.M, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), epi_plain(h, d));
-        pass_layernorm(c, r.M, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), x, d);
-        pass_gemm<EPI_GELU>(c, x, r.M, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), epi_plain(f, dff));
-        pass_gemm<EPI_RESID>(c, f, r.M, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), epi_plain(h, d));
+        pass_gemm<EPI_QKV>(c, x, r.M, r.plane, tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), eq);
+        attention_decode(c, m, l, q, o, o + (size_t)r.plane * d, r);
+        pass_gemm<EPI_RESID>(c, o, r.M, r.plane, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), epi_plain(h, d));
+        pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), x, d);
+        pass_gemm<EPI_GELU>(c, x, r.M, r.plane, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), epi_plain(f, dff));
+        pass_gemm<EPI_RESID>(c, f, r.M, r.plane, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), epi_plain(h, d));
     }
+    if (forked) prompt_project_join(c);
     if (!large || !projects_from(c, n)) return;
     const size_t elems = (size_t)r.M * d;   // after the last layer no LayerNorm of the large model follows
     {
         ProfScope ps(c, PC_ROWS, (double)elems * 8.0);
-        launch_ex(c, true, 1, cast_rows_kernel<true>, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, raw, elems, (size_t)c.lay.fr_rows * d);
+        launch_ex(c, true, 1, cast_rows_kernel<true>, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, raw, elems, (size_t)r.plane * d);
     }
     project(n);
 }
@@ -1428,11 +1443,11 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
 // are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie in
 // a cache of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
 // is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
-// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.58 ms like this.
+// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.51 ms like this.
 void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large, double kv_positions) {
     const Model &L = c.large, &S = c.small;
     Rows r;
-    r.M = f.rows; r.decode = true; r.whole_pass = true; r.n_chunks = 1; r.kv_positions = kv_positions;
+    r.M = f.rows; r.decode = true; r.whole_pass = true; r.plane = f.rows <= c.lay.fk_rows ? c.lay.fk_rows : c.lay.fr_rows; r.n_chunks = 1; r.kv_positions = kv_positions;
     float* h = at<float>(c, c.lay.h_large);
     auto begin = [&](const Model& m, bool setup) {
         ProfScope ps(c, PC_ROWS, (double)f.rows * m.d.d_model * 8.0);
@@ -1448,14 +1463,14 @@ void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large
     pass_layers(c, S, h, r);
     const int d = S.d.d_model, tiles = c.lay.score_tiles;
     bf16* x = at<bf16>(c, c.lay.fr_x);
-    pass_layernorm(c, f.rows, h, w_tail(c, S, 0), w_tail(c, S, 1), x, d);
+    pass_layernorm(c, f.rows, r.plane, h, w_tail(c, S, 0), w_tail(c, S, 1), x, d);
     for (int r0 = 0; r0 < f.rows; r0 += c.lay.fr_head_rows) {
         const int rows = std::min(c.lay.fr_head_rows, f.rows - r0);
         float* val = at<float>(c, c.lay.fr_tiles);
         TcScore t;
         t.val = val; t.idx = reinterpret_cast<int*>(val + (size_t)rows * tiles); t.sum = val + (size_t)2 * rows * tiles; t.stride = tiles;
         t.truth = f.truth + r0; t.truth_val = at<float>(c, c.lay.fr_truth_val);
-        pass_gemm<EPI_SCORE>(c, x + (size_t)r0 * d, rows, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, d), epi_plain(nullptr, S.d.vocab), t);
+        pass_gemm<EPI_SCORE>(c, x + (size_t)r0 * d, rows, r.plane, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, d), epi_plain(nullptr, S.d.vocab), t);
         ProfScope ps(c, PC_ARGMAX, 12.0 * rows * tiles);
         launch_ex(c, true, 1, score_tiles_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, rows, tiles, (const float*)t.val, (const int*)t.idx, (const float*)t.sum,
                   (const float*)t.truth_val, (const int*)(f.out + r0), at<float>(c, c.lay.forced_nll), at<int>(c, c.lay.forced_top));
