@@ -48,7 +48,7 @@ int cdiv(int a, int b) { return (a + b - 1) / b; }
 // Queries per attention group of the large model in a teacher-forced pass: one group of the MMA's eight columns (a warp meets all
 // keys of its group on its own, so more and lighter warps: 20.5 -> 17.5 us a layer for 772 rows x 16 heads x 64 under ncu).
 constexpr int PASS_GROUP = 8;
-// Most rows of a prompt pass whose projections run beside the large model's layers, see prompt_project_forked.
+// Most rows of a prompt or teacher-forced pass whose projections run beside the large model's layers, see prompt_project_forked.
 constexpr int PROMPT_FORK_ROWS = 2048;
 
 struct Layout {   // byte offsets into the arena
@@ -1384,7 +1384,7 @@ void pass_layernorm(tandem_ctx& c, int M, int plane, const float* x, const void*
 }
 
 // Whether a pass's projections run on the side stream, beside the large model's next layers (see prompt_project_forked; 772 rows of the small
-// pair 1548 -> 1515 us, 256 rows 1164 -> 1111, 600 rows 1984 -> 1921).
+// pair 1548 -> 1515 us, 256 rows 1164 -> 1111, 1200 rows 1984 -> 1921).
 bool pass_forks(const tandem_ctx& c, const Rows& r) { return r.M <= c.lay.fk_rows; }
 
 // FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.

@@ -165,6 +165,19 @@ def test_bf16_teacher_forced_pass(lens, gamma, prefill_rows, kw):
     t.close()
 
 
+def test_bf16_teacher_forced_pass_beyond_the_forked_rows():
+    """2100 rows keep the projections in the large model's stream and in buffers that other steps share; up to 2048 rows they run
+    beside it.  Both give a position's score within the tolerance that each has against the oracle."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, layer_map=(1, 3))
+    seqs = prompts_for(shape, [141] * 15, seed=25)
+    t = binding.Tandem(shape, _bf16_weights(shape, seed=26, std=0.06), max_batch=15, max_seq=200, gamma_max=14)
+    whole, _ = t.tandem_teacher_forced_forward(seqs, 14)
+    parts = t.tandem_teacher_forced_forward(seqs[:8], 14)[0] + t.tandem_teacher_forced_forward(seqs[8:], 14)[0]
+    for got, want in zip(whole, parts):
+        assert np.abs(got - want).max() < 2 * TOL_BF16
+    t.close()
+
+
 def test_bf16_layernorm_parameters_changed_between_calls():
     """Gains and biases that the caller changes after the prompt pass, and again between two steps, hold from the next call on, in
     every map behind a LayerNorm and in the projection."""
