@@ -726,6 +726,7 @@ struct TcTiledArgs {
     float* tile_max; int* tile_idx; float* tile_sum;   // EPI_SCORE: [M][tile_stride]
     int tile_stride;
     const int* truth; float* truth_val;                // EPI_SCORE: [M] the feature whose value goes to truth_val
+    const int* keep; float* kept;                      // EPI_SCORE: [M] the row of kept [][N] that takes all of the row's values (-1: none)
     EpiArgs e;
 };
 
@@ -768,6 +769,11 @@ __device__ __forceinline__ void score_tile(const TcTiledArgs& a, uint32_t acc, i
     a.tile_idx[o] = bi < 0 ? INT_MAX : n0 + bi;
     a.tile_sum[o] = z;
     if (truth >= 0 && truth < valid && truth < SCORE_TILE) a.truth_val[m] = true_v;
+    const int k = a.keep[m];
+    if (k < 0) return;                       // (all but the last block's rows)
+    float* row = a.kept + (size_t)k * a.N + n0;
+#pragma unroll
+    for (int i = 0; i < SCORE_TILE; ++i) if (i < valid) row[i] = v[i];
 }
 
 // Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.  PL with EPI_GELU: to two planes.

@@ -563,8 +563,10 @@ struct ForcedRows {
     const int* len;      // [batch]
     const int* vstart;   // [batch + 1] first row of each sequence, over all passes
     int batch, v0, rows; // this pass: rows v0 .. v0 + rows - 1
+    int gamma;           // positions per block
     int group;           // queries per attention group of the large model
-    int* row_tok; int* row_seq; int* row_pos;
+    int* row_seq; int* row_pos;
+    int* keep;           // [rows] where the row's logits stay readable: step within the block * batch + sequence for a sequence's last block, else -1
     int* truth;          // [rows] the next token (-1: none)
     int* out;            // [rows] where the row's scores go (-1: nowhere)
     int* grp_row0; int* grp_cnt;
@@ -605,11 +607,24 @@ __global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRo
     const int p = v - f.vstart[lo], len = f.len[lo], o = f.off[lo];
     const int tok = p < len ? f.ids[o + p] : 0;
     if (threadIdx.x == 0) {
-        f.row_tok[m] = tok; f.row_seq[m] = lo; f.row_pos[m] = p;
+        const int s = p - (f.vstart[lo + 1] - f.vstart[lo] - f.gamma);
+        f.row_seq[m] = lo; f.row_pos[m] = p;
+        f.keep[m] = s >= 0 ? s * f.batch + lo : -1;
         f.truth[m] = p + 1 < len ? f.ids[o + p + 1] : -1;
         f.out[m] = p + 1 < len ? o - lo + p : -1;
     }
     embed_row<bf16, 128, false>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0, nullptr);
+}
+
+// The large model's final residual stream of every sequence's last block, as far as it lies in this pass, to where it stays readable
+// (h's place is the small model's next): row b * gamma + s of dst.  grid: batch * gamma; block: 128; d % 4 == 0.
+__global__ void __launch_bounds__(128) forced_hidden_kernel(ForcedRows f, const float* __restrict__ h, float* __restrict__ dst, int d) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int b = blockIdx.x / f.gamma, m = f.vstart[b + 1] - f.gamma + (blockIdx.x - b * f.gamma) - f.v0;
+    if (m < 0 || m >= f.rows) return;
+    for (int k = threadIdx.x; k < d >> 2; k += 128)
+        reinterpret_cast<float4*>(dst + (size_t)blockIdx.x * d)[k] = __ldcg(reinterpret_cast<const float4*>(h + (size_t)m * d) + k);
 }
 
 // Scores of rows whose output head left (maximum, its index, sum of exponentials) per tile of features and the true token's

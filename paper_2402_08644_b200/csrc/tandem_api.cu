@@ -116,6 +116,7 @@ struct tandem_ctx {
     size_t pinned_ints;
     int64_t launches = 0;
     int last_gamma = 0;
+    size_t hidden_at = 0;                // where the large model's final residual stream of the last decode rows lies
     LoopState st{};
     // CUDA graphs of one iteration, keyed by everything baked into the captured launches
     struct GraphEntry {
@@ -582,7 +583,7 @@ TiledPlan tiled_plan(int n_sms, int epi, bool planes, int tiles128, int tiles256
 }
 
 // What the output head of a teacher-forced pass leaves per row and SCORE_TILE features instead of the logits.
-struct TcScore { float* val; int* idx; float* sum; int stride; const int* truth; float* truth_val; };
+struct TcScore { float* val; int* idx; float* sum; int stride; const int* truth; float* truth_val; const int* keep; float* kept; };
 
 // y = x W^T for many rows on the tensor cores; x bf16 [M][ldx].  PL: x as two planes, the remainders lo_row rows behind the values.
 template <int EPI, bool PL>
@@ -597,7 +598,7 @@ tandem_status launch_tc_tiled(tandem_ctx& c, const bf16* x, int ldx, int M, cons
     memset(&a, 0, sizeof(a));
     a.M = M; a.K = w.K; a.N = tcw_n(w); a.seg_rows0 = w.seg_rows0; a.seg_rows = w.seg_rows;
     a.err_flag = err; a.e = e; a.lo_row = lo_row;
-    if (EPI == EPI_SCORE) { a.tile_max = sc.val; a.tile_idx = sc.idx; a.tile_sum = sc.sum; a.tile_stride = sc.stride; a.truth = sc.truth; a.truth_val = sc.truth_val; }
+    if (EPI == EPI_SCORE) { a.tile_max = sc.val; a.tile_idx = sc.idx; a.tile_sum = sc.sum; a.tile_stride = sc.stride; a.truth = sc.truth; a.truth_val = sc.truth_val; a.keep = sc.keep; a.kept = sc.kept; }
     const int n_sms = std::max(1, c.n_sms);
     auto feature_tiles = [&](int width) {
         a.tiles0 = cdiv(w.seg_rows0, width);
@@ -1457,6 +1458,10 @@ void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large
     r.nq = PASS_GROUP; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
     begin(L, true);
     pass_layers(c, L, h, r);
+    {
+        ProfScope ps(c, PC_ROWS, (double)f.batch * gamma * L.d.d_model * 8.0);
+        launch_ex(c, true, 1, forced_hidden_kernel, dim3(f.batch * gamma), dim3(128), 0, f, (const float*)h, at<float>(c, c.lay.proj_snap), (int)L.d.d_model);
+    }
     r.nq = gamma; r.groups = f.rows / gamma; r.grp_row0 = r.grp_cnt = nullptr;
     r.own_k = at<bf16>(c, c.lay.fr_kv); r.own_v = r.own_k + c.lay.kv_small_layer;
     begin(S, false);   // (the large model's residual stream has been read for the last time)
@@ -1470,6 +1475,7 @@ void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large
         TcScore t;
         t.val = val; t.idx = reinterpret_cast<int*>(val + (size_t)rows * tiles); t.sum = val + (size_t)2 * rows * tiles; t.stride = tiles;
         t.truth = f.truth + r0; t.truth_val = at<float>(c, c.lay.fr_truth_val);
+        t.keep = f.keep + r0; t.kept = at<float>(c, c.lay.logits_small);
         pass_gemm<EPI_SCORE>(c, x + (size_t)r0 * d, rows, r.plane, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, d), epi_plain(nullptr, S.d.vocab), t);
         ProfScope ps(c, PC_ARGMAX, 12.0 * rows * tiles);
         launch_ex(c, true, 1, score_tiles_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, rows, tiles, (const float*)t.val, (const int*)t.idx, (const float*)t.sum,
@@ -1545,7 +1551,7 @@ tandem_status launch_iteration(tandem_ctx& c, int kind, int gamma, int mode, uin
     if (c.cfg.dtype == TANDEM_DTYPE_BF16)
         c.chunks_launch = 1;   // the cluster attention's grid does not depend on the context length: one graph serves all
     if (kind == 3) c.router_ticket++; else if (kind != 5) c.ticket++;   // what the host will wait for: the router's or the verify kernel's publication
-    if (kind != 3 && kind != 5) c.last_gamma = kind == 1 ? 0 : gamma;   // (set here, not while enqueueing: a replayed graph enqueues nothing on the host)
+    if (kind != 3 && kind != 5) { c.last_gamma = kind == 1 ? 0 : gamma; c.hidden_at = c.lay.h_large; }   // (set here, not while enqueueing: a replayed graph enqueues nothing on the host)
     // (A draft step of the adaptive block length starts when the host has seen the router's answer to the one before: a graph of all of
     // it would add its launch's latency to every step, 12.8 ms against 11.5 ms for 48 tokens of the small pair, and launched one by one
     // its kernels come slower than the GPU runs them.  So the first layer's kernels go out by themselves, the rest as a graph
@@ -1692,7 +1698,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->large.d = cfg->large; c->large.wbase = 0; c->large.kv_off = lay.kv_large; c->large.kv_layer_elems = lay.kv_large_layer;
     c->small.d = cfg->small; c->small.wbase = 5 + 10 * cfg->large.n_layers; c->small.kv_off = lay.kv_small; c->small.kv_layer_elems = lay.kv_small_layer;
     c->tbase = c->small.wbase + 5 + 10 * cfg->small.n_layers;
-    c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0;
+    c->batch = 0; c->n_ub = 0; c->launches = 0; c->last_gamma = 0; c->hidden_at = lay.h_large;
     c->pinned_ints = std::max((size_t)lay.max_rows + 5 * cfg->max_batch + 64,
                               (size_t)cfg->max_batch * (2 * cfg->max_seq + 4) + 2 * 64 + 64);   // prompt rows going in; tokens, counters, histogram, lengths, scores coming out
     c->pinned = nullptr;
@@ -1877,6 +1883,7 @@ tandem_status prefill_impl(tandem_ctx* c, int n_queries, int samples, const int3
     CK(cudaEventRecord(c->ev_staged, s));
     c->batch = batch;
     c->n_ub = n_max;
+    c->hidden_at = c->lay.h_large;
     c->n_sum = total;
     c->prompt_sq_sum = 0.0;
     for (int q = 0; q < n_queries; ++q) c->prompt_sq_sum += (double)(prompt_lens[q] - 1) * (prompt_lens[q] - 1);
@@ -2213,11 +2220,12 @@ tandem_status forced_forward(tandem_ctx* c, int gamma, int batch, const int32_t*
     CK(cudaMemcpyAsync(c->arena + c->lay.fr_seq, p_off, (size_t)(3 * batch + 1) * 4, cudaMemcpyHostToDevice, c->stream));
     CK(cudaEventRecord(c->ev_staged, c->stream));
     c->batch = batch; c->n_ub = max_len; c->n_sum = total; c->last_gamma = gamma;
+    c->hidden_at = c->lay.proj_snap;
     launch_call_begin(*c, true);
     ForcedRows f;
     f.ids = at<int>(*c, c->lay.forced_ids); f.off = at<int>(*c, c->lay.fr_seq); f.len = f.off + batch; f.vstart = f.len + batch;
-    f.batch = batch; f.group = PASS_GROUP;
-    f.row_tok = at<int>(*c, c->lay.row_tok); f.row_seq = at<int>(*c, c->lay.row_seq); f.row_pos = at<int>(*c, c->lay.row_pos);
+    f.batch = batch; f.gamma = gamma; f.group = PASS_GROUP;
+    f.keep = at<int>(*c, c->lay.row_tok); f.row_seq = at<int>(*c, c->lay.row_seq); f.row_pos = at<int>(*c, c->lay.row_pos);
     f.truth = at<int>(*c, c->lay.fr_truth); f.out = at<int>(*c, c->lay.fr_out);
     f.grp_row0 = at<int>(*c, c->lay.fr_grp); f.grp_cnt = f.grp_row0 + c->lay.fr_rows / PASS_GROUP + c->cfg.max_batch + 1;
     const int step = c->lay.fr_rows / gamma * gamma;
@@ -2405,7 +2413,7 @@ extern "C" tandem_status tandem_debug_read(tandem_ctx* c, int32_t what, int32_t 
         const void* src;
         if (what == 0) { n = (size_t)B * (g + 1) * V; src = c->arena + c->lay.logits_large; }
         else if (what == 1) { n = (size_t)g * B * V; src = c->arena + c->lay.logits_small; }
-        else { n = (size_t)B * (g + 1) * c->cfg.large.d_model; src = c->arena + c->lay.h_large; }
+        else { n = (size_t)B * (g + 1) * c->cfg.large.d_model; src = c->arena + c->hidden_at; }
         if (bytes != n * 4) return TANDEM_ERR_INVALID_ARG;
         if (n) CK(cudaMemcpy(host_dst, src, bytes, cudaMemcpyDeviceToHost));
         return TANDEM_OK;

@@ -165,6 +165,38 @@ def test_bf16_teacher_forced_pass(lens, gamma, prefill_rows, kw):
     t.close()
 
 
+@pytest.mark.parametrize("lens,gamma,prefill_rows,vocab", [([141, 23, 6], 4, 0, 129), ([33, 47], 5, 12, 50)])   # one pass; several
+def test_bf16_logits_and_representations_of_the_last_blocks(lens, gamma, prefill_rows, vocab):
+    """What a teacher-forced forward leaves to read: the small model's logits and the large model's representations of every
+    sequence's last block, not those of the steps before the call."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, layer_map=(1, 3), vocab=vocab)
+    w = _bf16_weights(shape, seed=31, std=0.06)
+    seqs = prompts_for(shape, lens, seed=32)
+    t = binding.Tandem(shape, w, max_batch=len(lens), max_seq=200, gamma_max=gamma, max_prefill_rows=prefill_rows)
+    t.tandem_prefill([s[:3] for s in seqs])
+    t.tandem_block_step(gamma)
+    t.tandem_teacher_forced_forward(seqs, gamma)
+    logits = t.tandem_debug_read(binding.READ_SMALL_LOGITS, gamma)
+    hidden = t.tandem_debug_read(binding.READ_LARGE_HIDDEN, gamma).reshape(-1, shape.large.d_model)
+    for b, ids in enumerate(seqs):
+        o = O.TandemOracle(shape, w)
+        reps, _ = O.large_block_pass(o.large, o.large_cache, ids, 0)
+        want = O.teacher_forced_tandem_logits(shape, w, ids, gamma)
+        first = (len(ids) - 2) // gamma * gamma
+        for p in range(first, len(ids) - 1):
+            assert np.abs(logits[p - first, b] - want[p]).max() < TOL_BF16
+            assert np.abs(hidden[b * gamma + p - first] - reps[-1][p]).max() < 2 * TOL_BF16
+    t.tandem_prefill([s[:3] for s in seqs])       # and a decode iteration's own again
+    res = t.tandem_block_step(gamma)
+    hidden = t.tandem_debug_read(binding.READ_LARGE_HIDDEN, gamma)
+    for b, ids in enumerate(seqs):
+        o = O.TandemOracle(shape, w)
+        o.prefill(ids[:3])
+        _, _, reps = o.verify(res["drafts"][b].tolist())
+        assert np.abs(hidden[b] - np.stack(reps[-1])).max() < 2 * TOL_BF16
+    t.close()
+
+
 def test_bf16_teacher_forced_pass_beyond_the_forked_rows():
     """2100 rows keep the projections in the large model's stream and in buffers that other steps share; up to 2048 rows they run
     beside it.  Both give a position's score within the tolerance that each has against the oracle."""
