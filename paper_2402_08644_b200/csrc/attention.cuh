@@ -29,14 +29,15 @@ struct AttnArgs {
     const void* kcache; const void* vcache;   // [seq][head][t_max][DH]
     const void* k2; const void* v2;            // optional second segment [seq][head][t_max2][DH] holding
     int split, t_max2;                         //   positions >= split (used when k2 != nullptr)
-    //   (attn_decode_kernel, ATD_PASS: the second segment is a cache like the first, indexed by absolute position, and holds the
-    //   positions from the group's first row on; split and t_max2 unused)
+    //   (attn_decode_kernel, ATD_PASS: the second segment is [head][t_max2][DH], indexed by the rows of the pass, and holds the
+    //   positions from the group's first row on; split unused)
     void* out; int ldo;                  // T [M][ldo]
     const int* row_seq; const int* row_pos;    // attn_decode_kernel: row_seq may be null, then group g is sequence g and every
     int pos_all;                               //   sequence's first row sits at position pos_all (no row arrays to fill and fetch)
     int wait_first;                            // attn_decode_kernel: 1 = nothing is read before the wait on the preceding kernel
                                                //   (a stand-alone call: whatever precedes it may be writing the keys and values)
     const int* grp_row0; const int* grp_cnt;   // nullable: then group g = rows g*nq .. g*nq+nq-1
+    const int* pass_grp; const int* pass_pos;  // ATD_PASS: per group first row | rows << 16 | sequence << 20, and the first row's position
     int nq;
     int units, log_parts;                // ATD_PASS: groups * head groups; 2^log_parts warps (1, 2 or 4) share the keys of each
     int n_heads, t_max;
@@ -403,16 +404,16 @@ __global__ void __launch_bounds__(ATD_THREADS) attn_decode_kernel(AttnArgs a) {
         pdl_wait();
         pdl_launch_dependents();
     }
-    int nq = a.nq, row0 = g * nq;
-    if (MODE == ATD_PASS && a.grp_cnt) { nq = __ldcg(a.grp_cnt + g); row0 = __ldcg(a.grp_row0 + g); }
+    const int pg = MODE == ATD_PASS ? __ldcg(a.pass_grp + g) : 0;
+    const int nq = MODE == ATD_PASS ? (pg >> 16) & 15 : a.nq, row0 = MODE == ATD_PASS ? pg & 0xffff : g * nq;
     const int cnt = gpc * nq;                      // rows of the tile in use
-    const int b = a.row_seq ? __ldcg(a.row_seq + row0) : g;          // from L2: nothing an earlier kernel on this SM may have cached
-    const int pos_first = a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all;
+    const int b = MODE == ATD_PASS ? pg >> 20 : (a.row_seq ? __ldcg(a.row_seq + row0) : g);          // from L2: nothing an earlier kernel on this SM may have cached
+    const int pos_first = MODE == ATD_PASS ? __ldcg(a.pass_pos + g) : (a.row_seq ? __ldcg(a.row_pos + row0) : a.pos_all);
     const int pos_last = pos_first + nq - 1;
     const int n_chunks = pos_last / ATT_CH + 1;
     const int n_mine = MODE == ATD_PASS ? (pos_last / ATD_WROWS + (1 << log_parts) - part) >> log_parts : rank < n_chunks ? (n_chunks - rank + CL - 1) >> log_cl : 0;
     const size_t head_base = ((size_t)b * n_kv + kvh) * a.t_max;
-    const size_t head_base2 = ((size_t)b * n_kv + kvh) * (MODE == ATD_PASS ? a.t_max : a.t_max2);
+    const size_t head_base2 = MODE == ATD_PASS ? (size_t)kvh * a.t_max2 + row0 - pos_first : ((size_t)b * n_kv + kvh) * a.t_max2;   // (ATD_PASS: to be added to a position)
     const int split = a.k2 ? (MODE == ATD_PASS ? pos_first : a.split) : INT_MAX;
     const int base2 = MODE == ATD_PASS ? 0 : split;    // position of the second segment's first key
 

@@ -24,7 +24,7 @@ struct EpiArgs {
     int ldo;
     void* kcache;         // QKV / KV: this layer's keys   [B][H][t_max][d_head] (T)
     void* vcache;         //           this layer's values
-    const int* row_seq;   // [M] sequence of each row (null on the tensor-core decode path: row j is sequence j at position 0)
+    const int* row_seq;   // [M] sequence of each row (null: row j is sequence j at position 0 on the tensor-core decode path, position j of one sequence elsewhere)
     const int* row_pos;   // [M] absolute position of each row
     int n_heads, d_head, t_max;   // n_heads: key/value heads of the cache
     int seg0;             // QKV / KV: columns of the first segment (QKV: the queries, d_model; KV: the keys)
@@ -73,7 +73,9 @@ __device__ __forceinline__ void epilogue(const EpiArgs& e, int m, int n, float v
             s -= 1;
         }
         const int h = c / e.d_head, el = c - h * e.d_head;
-        const size_t idx = (((size_t)e.row_seq[m] * e.n_heads + h) * e.t_max + e.row_pos[m]) * e.d_head + el;
+        const bool rows = sizeof(T) == 4 || e.row_seq;
+        const size_t seq = rows ? e.row_seq[m] : 0, pos = rows ? e.row_pos[m] : m;
+        const size_t idx = ((seq * e.n_heads + h) * e.t_max + pos) * e.d_head + el;
         T* base = static_cast<T*>(s == 0 ? e.kcache : e.vcache);
         base[idx] = from_float<T>(v);
     }

@@ -745,35 +745,50 @@ constexpr int TCP_GROUP_M = 8;                        // row tiles that share a 
 
 // EPI_SCORE: SCORE_TILE features of one row from its TMEM lane; n0: the first of them, valid: how many exist.  Warp-wide loads.
 __device__ __forceinline__ void score_tile(const TcTiledArgs& a, uint32_t acc, int m, int n0, int valid) {
-    float v[SCORE_TILE];
+    const bool mine = m < a.M && valid > 0;
+    const int keep = mine ? a.keep[m] : -1;
+    {
+        float v[SCORE_TILE];
 #pragma unroll
+        for (int i = 0; i < SCORE_TILE; i += 16) {
+            float t[16];
+            tmem_ld16(acc + i, t);
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[i + u] = i + u < valid ? t[u] : -INFINITY;
+        }
+        if (mine) {
+            float best = -INFINITY, z = 0.f, true_v = 0.f;
+            int bi = -1;
+            const int truth = a.truth[m] - n0;
+#pragma unroll
+            for (int i = 0; i < SCORE_TILE; ++i) {
+                if (v[i] > best) { best = v[i]; bi = i; }
+                if (i == truth) true_v = v[i];
+            }
+#pragma unroll
+            for (int i = 0; i < SCORE_TILE; ++i) z += expf(v[i] - best);
+            const size_t o = (size_t)m * a.tile_stride + n0 / SCORE_TILE;
+            a.tile_max[o] = best;
+            a.tile_idx[o] = bi < 0 ? INT_MAX : n0 + bi;
+            a.tile_sum[o] = z;
+            if (truth >= 0 && truth < valid && truth < SCORE_TILE) a.truth_val[m] = true_v;
+        }
+    }
+    if (!__any_sync(0xffffffffu, keep >= 0)) return;   // (all but the sequences' last blocks)
+#pragma unroll 1
     for (int i = 0; i < SCORE_TILE; i += 16) {
         float t[16];
         tmem_ld16(acc + i, t);
+        if (keep < 0) continue;
+        float* row = a.kept + (size_t)keep * a.N + n0 + i;
+        if ((a.N & 3) == 0 && i + 16 <= valid) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[i + u] = i + u < valid ? t[u] : -INFINITY;
+            for (int u = 0; u < 16; u += 4) *reinterpret_cast<float4*>(row + u) = make_float4(t[u], t[u + 1], t[u + 2], t[u + 3]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 16; ++u) if (i + u < valid) row[u] = t[u];
+        }
     }
-    if (m >= a.M || valid <= 0) return;
-    float best = -INFINITY, z = 0.f, true_v = 0.f;
-    int bi = -1;
-    const int truth = a.truth[m] - n0;
-#pragma unroll
-    for (int i = 0; i < SCORE_TILE; ++i) {
-        if (v[i] > best) { best = v[i]; bi = i; }
-        if (i == truth) true_v = v[i];
-    }
-#pragma unroll
-    for (int i = 0; i < SCORE_TILE; ++i) z += expf(v[i] - best);
-    const size_t o = (size_t)m * a.tile_stride + n0 / SCORE_TILE;
-    a.tile_max[o] = best;
-    a.tile_idx[o] = bi < 0 ? INT_MAX : n0 + bi;
-    a.tile_sum[o] = z;
-    if (truth >= 0 && truth < valid && truth < SCORE_TILE) a.truth_val[m] = true_v;
-    const int k = a.keep[m];
-    if (k < 0) return;                       // (all but the last block's rows)
-    float* row = a.kept + (size_t)k * a.N + n0;
-#pragma unroll
-    for (int i = 0; i < SCORE_TILE; ++i) if (i < valid) row[i] = v[i];
 }
 
 // Sixteen consecutive output features of one row.  n_local0 is a multiple of 16.  PL with EPI_GELU: to two planes.
@@ -845,6 +860,7 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int seg, int
 template <int EPI>
 __device__ __forceinline__ size_t cache_row_offset(const EpiArgs& e, int m, int M) {
     if ((EPI != EPI_QKV && EPI != EPI_KV) || m >= M) return 0;
+    if (!e.row_seq) return (size_t)m * e.d_head;
     return ((size_t)e.row_seq[m] * e.n_heads * e.t_max + e.row_pos[m]) * e.d_head;
 }
 

@@ -555,46 +555,67 @@ __global__ void __launch_bounds__(VERIFY_THREADS) verify_kernel(LoopState st, in
     }
 }
 
-// Teacher-forced Tandem forward, bf16: all given tokens are rows of one pass (or of a few, where the work space is short).  The
-// rows lie sequence after sequence, each padded to whole blocks of gamma positions.
+// Teacher-forced Tandem forward, bf16: all given tokens that have a next one are rows of one pass (or of a few, where the work space is
+// short), sequence after sequence.
 struct ForcedRows {
-    const int* ids;      // the sequences, one after the other
-    const int* off;      // [batch] where each begins in ids
-    const int* len;      // [batch]
-    const int* vstart;   // [batch + 1] first row of each sequence, over all passes
-    int batch, v0, rows; // this pass: rows v0 .. v0 + rows - 1
-    int gamma;           // positions per block
-    int group;           // queries per attention group of the large model
+    const int* ids;      // the sequences, one after the other: row v of sequence b is ids[v + b], its next token ids[v + b + 1]
+    const int* start;    // [batch + 1] first row of each sequence, over all passes
+    int batch, v0, rows; // this pass: rows v0 .. v0 + rows - 1, whole blocks
+    int gamma, vocab;    // positions per block (a sequence's last one may be shorter)
+    int group;           // queries per attention group: of the large model, or a block of the small model's
     int* row_seq; int* row_pos;
     int* keep;           // [rows] where the row's logits stay readable: step within the block * batch + sequence for a sequence's last block, else -1
-    int* truth;          // [rows] the next token (-1: none)
-    int* out;            // [rows] where the row's scores go (-1: nowhere)
-    int* grp_row0; int* grp_cnt;
+    int* truth;          // [rows] the next token
+    int* grp; int* grp_pos;                      // attention groups, see AttnArgs::pass_grp
+    float* nll; int* top;                        // [rows of all passes] scores
+    const float* hidden; int d_large;            // the large model's final residual stream [rows][d_large]
+    float* last_hidden; float* last_logits;      // readable afterwards, of the sequences' last blocks: [batch][gamma][d_large], [gamma][batch][vocab]
 };
 
-// Start of one model's part of such a pass: row set-up and embedding (a row past its sequence's end reads token 0; it is
-// computed and ignored), and, with one block more than rows, the attention groups and the sequences' loop state.
-// grid: rows (+ 1); block: 128.
+// Start of one model's part of such a pass: row set-up and embedding, and in one more block the attention groups and the sequences' loop
+// state.  The small model's part has batch * gamma blocks more: the large model's final stream of the sequences' last blocks, and
+// zeros where a block ends before gamma positions.
+// grid: rows + 1 (+ batch * gamma); block: 128.
 __global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRows f, const bf16* __restrict__ emb, const bf16* __restrict__ pos,
                                                           float* __restrict__ h, int d, int ticket, int router_ticket) {
-    __shared__ int s_cnt[128];
+    __shared__ int s_first[128], s_n[128];
     pdl_wait();
     pdl_launch_dependents();
     const int m = blockIdx.x;
+    if (m > f.rows) {
+        const int i = m - f.rows - 1, b = i / f.gamma, s = i - b * f.gamma, n = f.start[b + 1] - f.start[b];
+        const int last = (n - 1) / f.gamma * f.gamma, row = f.start[b] + last + s - f.v0;   // the last block's first position
+        float* dst = f.last_hidden + (size_t)i * f.d_large;
+        if (last + s >= n) {
+            for (int k = threadIdx.x; k < f.d_large; k += 128) dst[k] = 0.f;
+            float* row = f.last_logits + (size_t)(s * f.batch + b) * f.vocab;
+            if ((f.vocab & 3) == 0) { for (int k = threadIdx.x; k < f.vocab >> 2; k += 128) reinterpret_cast<float4*>(row)[k] = make_float4(0.f, 0.f, 0.f, 0.f); }
+            else for (int k = threadIdx.x; k < f.vocab; k += 128) row[k] = 0.f;
+        } else if (row >= 0 && row < f.rows) {
+            const float4* src = reinterpret_cast<const float4*>(f.hidden + (size_t)row * f.d_large);
+            for (int k = threadIdx.x; k < f.d_large >> 2; k += 128) reinterpret_cast<float4*>(dst)[k] = __ldcg(src + k);
+        }
+        return;
+    }
     if (m == f.rows) {
         const int b = threadIdx.x;   // (batch <= 128: at least two rows per sequence in every context)
-        int first = 0, n = 0;
+        s_first[b] = s_n[b] = 0;
         if (b < f.batch) {
-            first = max(f.vstart[b], f.v0);
-            n = max(0, min(f.vstart[b + 1], f.v0 + f.rows) - first);
-            st.n[b] = f.len[b];
-            st.pending[b] = f.ids[f.off[b] + f.len[b] - 1];
+            const int first = max(f.start[b], f.v0);
+            s_first[b] = first - f.v0;
+            s_n[b] = max(0, min(f.start[b + 1], f.v0 + f.rows) - first);
+            st.n[b] = f.start[b + 1] - f.start[b] + 1;
+            st.pending[b] = f.ids[f.start[b + 1] + b];
         }
-        s_cnt[b] = (n + f.group - 1) / f.group;
         __syncthreads();
-        int g = 0;
-        for (int i = 0; i < b; ++i) g += s_cnt[i];
-        for (int r = 0; r < n; r += f.group, ++g) { f.grp_row0[g] = first - f.v0 + r; f.grp_cnt[g] = min(f.group, n - r); }
+        for (int i = 0, g = 0; i < f.batch; ++i) {
+            const int n = s_n[i], groups = (n + f.group - 1) / f.group;
+            for (int j = threadIdx.x; j < groups; j += 128) {
+                f.grp[g + j] = (s_first[i] + j * f.group) | min(f.group, n - j * f.group) << 16 | i << 20;
+                f.grp_pos[g + j] = f.v0 + s_first[i] - f.start[i] + j * f.group;
+            }
+            g += groups;
+        }
         if (b == 0) { st.counters[6] = ticket; st.counters[8] = router_ticket; }
         return;
     }
@@ -602,41 +623,27 @@ __global__ void __launch_bounds__(128) forced_rows_kernel(LoopState st, ForcedRo
     int lo = 0, hi = f.batch - 1;   // the last sequence that begins at or before row v
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (f.vstart[mid] <= v) lo = mid; else hi = mid - 1;
+        if (f.start[mid] <= v) lo = mid; else hi = mid - 1;
     }
-    const int p = v - f.vstart[lo], len = f.len[lo], o = f.off[lo];
-    const int tok = p < len ? f.ids[o + p] : 0;
+    const int p = v - f.start[lo], tok = f.ids[v + lo];
     if (threadIdx.x == 0) {
-        const int s = p - (f.vstart[lo + 1] - f.vstart[lo] - f.gamma);
+        const int s = p - (f.start[lo + 1] - f.start[lo] - 1) / f.gamma * f.gamma;
         f.row_seq[m] = lo; f.row_pos[m] = p;
         f.keep[m] = s >= 0 ? s * f.batch + lo : -1;
-        f.truth[m] = p + 1 < len ? f.ids[o + p + 1] : -1;
-        f.out[m] = p + 1 < len ? o - lo + p : -1;
+        f.truth[m] = f.ids[v + lo + 1];
     }
     embed_row<bf16, 128, false>(emb + (size_t)tok * d, pos + (size_t)p * d, h + (size_t)m * d, nullptr, d, NextLn{}, 0, nullptr);
 }
 
-// The large model's final residual stream of every sequence's last block, as far as it lies in this pass, to where it stays readable
-// (h's place is the small model's next): row b * gamma + s of dst.  grid: batch * gamma; block: 128; d % 4 == 0.
-__global__ void __launch_bounds__(128) forced_hidden_kernel(ForcedRows f, const float* __restrict__ h, float* __restrict__ dst, int d) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int b = blockIdx.x / f.gamma, m = f.vstart[b + 1] - f.gamma + (blockIdx.x - b * f.gamma) - f.v0;
-    if (m < 0 || m >= f.rows) return;
-    for (int k = threadIdx.x; k < d >> 2; k += 128)
-        reinterpret_cast<float4*>(dst + (size_t)blockIdx.x * d)[k] = __ldcg(reinterpret_cast<const float4*>(h + (size_t)m * d) + k);
-}
-
 // Scores of rows whose output head left (maximum, its index, sum of exponentials) per tile of features and the true token's
-// logit: negative log-likelihood and arg-max (lowest index on ties).  One warp per row; n_tiles values each, 500 at 32000 logits.
+// logit (in nll): negative log-likelihood and arg-max (lowest index on ties).  One warp per row; n_tiles values each, 500 at 32000 logits.
 // grid: ceil(rows / 8); block: 256.
 __global__ void __launch_bounds__(256) score_tiles_kernel(int rows, int n_tiles, const float* __restrict__ tile_max, const int* __restrict__ tile_idx,
-                                                          const float* __restrict__ tile_sum, const float* __restrict__ truth_val,
-                                                          const int* __restrict__ out, float* __restrict__ nll, int* __restrict__ top1) {
+                                                          const float* __restrict__ tile_sum, float* __restrict__ nll, int* __restrict__ top1) {
     pdl_wait();
     pdl_launch_dependents();
     const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (m >= rows || out[m] < 0) return;
+    if (m >= rows) return;
     const size_t base = (size_t)m * n_tiles;
     const int top = argmax_from_tiles(tile_max + base, tile_idx + base, n_tiles);
     float best = -INFINITY;
@@ -649,8 +656,8 @@ __global__ void __launch_bounds__(256) score_tiles_kernel(int rows, int n_tiles,
     }
     tot = warp_sum(tot);
     if (lane == 0) {
-        nll[out[m]] = best + logf(tot) - truth_val[m];
-        top1[out[m]] = top;
+        nll[m] = best + logf(tot) - nll[m];
+        top1[m] = top;
     }
 }
 

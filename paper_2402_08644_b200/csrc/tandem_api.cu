@@ -56,10 +56,10 @@ struct Layout {   // byte offsets into the arena
     size_t st_n, st_pending, st_drafts, st_targets, st_accept, st_emitted, st_done, st_out, st_counters, st_hist;
     size_t st_block_len, st_drafting, st_confidence;
     size_t forced_ids, forced_len, forced_nll, forced_top;   // teacher-forced forward: given tokens [B][T], lengths [B], scores [B][T]
-    size_t fr_x, fr_o, fr_f, fr_q, fr_raw, fr_yhat, fr_a, fr_t1;
-    size_t fk_raw, fk_yhat, fk_a, fk_t1;            // the projections' buffers in a pass of at most fk_rows rows, whose projections run beside M_L's layers
-    size_t fr_seq, fr_truth, fr_out, fr_truth_val, fr_grp, fr_tiles, fr_kv;   // ... in one pass (bf16), see ForcedRows: offsets / lengths / first rows, next tokens, score places,
-                                                                              // true logits, attention groups, the head's per-tile results, the small model's own keys / values of one layer
+    // ... in one pass (bf16), see place_pass: rows in front of the products, GELU outputs, queries and the projections' buffers of the
+    // large model's part; stream, rows, own keys / values, GELU outputs, queries of the small model's; the head's per-tile results
+    size_t fr_x, fr_f, fr_q, fr_raw, fr_yhat, fr_a, fr_t1, fr_hs, fr_xs, fr_kv, fr_fs, fr_tiles;
+    size_t fr_start, fr_truth;              // ... the sequences' first rows, the rows' next tokens (where a prompt pass has its staged inputs)
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
     size_t stage;                                   // a prompt pass's lengths, offsets and token ids as the host staged them
     size_t attn_counters;   // inside the zero-filled state block
@@ -71,7 +71,7 @@ struct Layout {   // byte offsets into the arena
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles, score_tiles;
-    int fr_rows, fk_rows, fr_head_rows;      // rows of a teacher-forced pass, of one whose projections are forked, and of one run of its output head
+    int fr_rows, fr_head_rows;               // most rows of a teacher-forced pass, and of one run of its output head
     size_t kv_large_layer, kv_small_layer;   // elements per (layer, k-or-v)
 };
 
@@ -209,6 +209,32 @@ tandem_status validate(const tandem_config* c) {
     return TANDEM_OK;
 }
 
+// A teacher-forced pass of `rows` rows in the prompt pass's space from `at` on, as fp32 rows or two bf16 planes; returns where it ends.
+// What two steps of a layer never hold together shares a place: the large model's attention writes where the rows of its QKV map
+// were, and the GELU outputs lie over the queries and the projections' buffers (the projections are done before the
+// FFN's first product).  The small model's part begins when the large model's is over.
+size_t place_pass(const tandem_config& c, Layout& L, size_t at, size_t rows) {
+    const size_t dL = c.large.d_model, dS = c.small.d_model;
+    const size_t hidden = c.ff_tandem_kind == TANDEM_FF_LINEAR ? 0 : (c.ff_tandem_hidden > 0 ? c.ff_tandem_hidden : c.small.d_model);
+    size_t off = at;
+    auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
+    L.fr_x = take(rows * dL * 4);
+    L.fr_f = off;
+    L.fr_raw = take(rows * dL * 4); L.fr_t1 = take(rows * hidden * 4); L.fr_yhat = take(rows * dS * 4); L.fr_a = take(rows * dS * 4);
+    L.fr_q = take(rows * dL * 2);
+    size_t end = std::max(off, align_up(L.fr_f + rows * c.large.d_ff * 4));
+    off = at;
+    L.fr_hs = take(rows * dS * 4); L.fr_xs = take(rows * dS * 4);
+    L.fr_tiles = off;                       // (the layers behind it)
+    L.fr_kv = take(2 * rows * d_kv_of(c.small) * 2);
+    L.fr_fs = take(rows * std::max<size_t>(c.small.d_ff * 4, dS * 2));   // GELU outputs, queries
+    return std::max(end, off);
+}
+
+// Columns per warp of the fp32 few-row kernel: one until that is two CTAs on each of 148 multiprocessors, then four (the staged rows are
+// read once for them).  The output head's arg-max results are laid out by it.
+int rows_columns(int N) { return N > 2 * GS_WARPS * 148 ? 4 : 1; }
+
 Layout make_layout(const tandem_config& c) {
     Layout L;
     memset(&L, 0, sizeof(L));
@@ -225,10 +251,6 @@ Layout make_layout(const tandem_config& c) {
     const size_t hmax = std::max(c.large.n_heads, c.small.n_heads);
     const bool bf = c.dtype == TANDEM_DTYPE_BF16;
     const size_t R = L.max_rows, RD = L.dec_rows, V = c.large.vocab;
-    // Rows of a teacher-forced pass: as many as a prompt pass takes, and the rows that fill its sequences' last blocks.
-    const size_t RF = bf ? std::min<size_t>(R + (size_t)c.max_batch * c.gamma_max, 32768) : 0;
-    L.fr_rows = (int)RF;
-    L.fr_head_rows = (int)std::min<size_t>(RF, 1024);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     L.kv_large_layer = B * T * d_kv_of(c.large);
@@ -240,45 +262,58 @@ Layout make_layout(const tandem_config& c) {
     L.st_done = take(B * 4); L.st_out = take(B * T * 4);
     L.st_counters = take(16 * 4); L.st_hist = take((GL + 1) * 8); L.st_emitted = take(B * 4);   // adjacent: read back together
     L.st_block_len = take(B * 4); L.st_drafting = take(B * 4); L.st_confidence = take(B * GL * 4);
-    const size_t RR = std::max(R, RF);
-    L.row_tok = take(RR * 4); L.row_seq = take(RR * 4); L.row_pos = take(RR * 4);
+    L.row_tok = take(R * 4); L.row_seq = take(R * 4); L.row_pos = take(R * 4);
     L.grp_row0 = take((size_t)L.max_groups * 4); L.grp_cnt = take((size_t)L.max_groups * 4);
     L.stage = take((4 * B + R + B) * 4);
+    L.fr_start = L.stage; L.fr_truth = L.stage + 5 * B * 4;   // (B + 1, R)
     L.attn_counters = take(B * hmax * 4);
-    L.h_large = take(std::max(R * c.large.d_model, RF * std::max(c.large.d_model, c.small.d_model)) * 4);
+    L.h_large = take(R * c.large.d_model * 4);
     L.h_small = take(B * c.small.d_model * 4);
     const size_t ws = off;
     L.a = take(R * dmax * esz); L.q = take(R * dmax * esz); L.o = take(R * dmax * esz);
     L.f = take(R * fmax * esz);
     L.xb = take(R * c.large.d_model * esz); L.t1 = take(R * hidden * esz);
     L.yhat = take(R * c.small.d_model * 4); L.a_s = take(R * c.small.d_model * esz);
-    // The same space in a teacher-forced pass, whose rows are fp32 or two bf16 planes.  The queries and the projections' buffers
-    // share the place of the GELU outputs, which are dead from the end of a layer to the first product of the next one's FFN.
-    const size_t ws_end = off;
-    off = ws;
-    L.fr_x = take(RF * dmax * 4); L.fr_o = take(RF * dmax * 4); L.fr_f = take(RF * fmax * 4);
-    const size_t fr_end = off;
-    off = L.fr_f;
-    L.fr_raw = take(RF * c.large.d_model * 4); L.fr_t1 = take(RF * hidden * 4); L.fr_yhat = take(RF * c.small.d_model * 4); L.fr_a = take(RF * c.small.d_model * 4);
-    const size_t fr_proj_end = off;
-    off = L.fr_f;
-    L.fr_q = take(RF * dmax * 2);
-    off = std::max(std::max(off, fr_proj_end), std::max(fr_end, ws_end));
-    const size_t RK = std::min<size_t>(RF, PROMPT_FORK_ROWS);
-    L.fk_rows = (int)RK;
-    L.fk_raw = take(RK * c.large.d_model * 4); L.fk_t1 = take(RK * hidden * 4); L.fk_yhat = take(RK * c.small.d_model * 4); L.fk_a = take(RK * c.small.d_model * 4);
-    L.logits_large = take(RD * V * 4);
-    L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.part_ml = take(RD * hmax * L.n_chunks_max * 2 * 4);
     L.part_acc = take(RD * dmax * L.n_chunks_max * 4);
+    if (bf) {
+        // A teacher-forced pass takes what it finds here (the attention's parts are fp32 contexts' only): a context asks for no more memory
+        // than its prompt pass needs, and a forward over more rows goes in several passes.  Where feed-forward layers are four times
+        // as wide as the models (or less), a pass has room for a prompt pass's rows.  Only a work space that cannot hold one
+        // block, or sixteen rows' results of the head, grows.
+        const size_t ws_end = off, least = std::min<size_t>(R, std::max(1, c.gamma_max));
+        size_t rows = std::min<size_t>(R, 32768);
+        while (rows > least && place_pass(c, L, ws, rows) > ws_end) {
+            const size_t fit = (size_t)((double)rows * (double)(ws_end - ws) / (double)(place_pass(c, L, ws, rows) - ws));
+            rows = std::max(least, std::min(rows - 1, fit));
+        }
+        const size_t pass_end = std::max(ws_end, place_pass(c, L, ws, rows));
+        L.fr_rows = (int)rows;
+        L.score_tiles = cdiv(c.large.vocab, SCORE_TILE);
+        const size_t tile_bytes = (size_t)L.score_tiles * 12, few = std::min<size_t>(rows, 16);
+        L.fr_head_rows = (int)std::max(few, std::min(std::min<size_t>(rows, 1024), (pass_end - L.fr_tiles) / tile_bytes));
+        off = std::max(pass_end, align_up(L.fr_tiles + few * tile_bytes));
+    }
+    L.logits_large = take(RD * V * 4);
+    L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.dbg = take(T * dmax * 4);
     L.forced_ids = take(B * T * 4); L.forced_len = take(B * 4); L.forced_nll = take(B * T * 4); L.forced_top = take(B * T * 4);
     L.smp_large = take(RD * 8); L.smp_small = take((size_t)std::max(1, c.gamma_max) * B * 8);
-    L.vocab_tiles = cdiv(c.large.vocab, bf ? 128 : GS_WARPS);   // (fp32: at most; a block of the head has GS_WARPS columns or four times as many)
-    L.amax_val_large = take(RD * L.vocab_tiles * 4); L.amax_idx_large = take(RD * L.vocab_tiles * 4);
-    L.amax_val_small = take(B * L.vocab_tiles * 4); L.amax_idx_small = take(B * L.vocab_tiles * 4);
+    auto take_amax = [&](int columns) {
+        L.vocab_tiles = cdiv(c.large.vocab, columns);
+        L.amax_val_large = take(RD * L.vocab_tiles * 4); L.amax_idx_large = take(RD * L.vocab_tiles * 4);
+        L.amax_val_small = take(B * L.vocab_tiles * 4); L.amax_idx_small = take(B * L.vocab_tiles * 4);
+    };
+    const size_t amax = off;
+    take_amax(128);
     const size_t nS = c.small.n_layers;
     L.a32 = take(RD * dmax * 4); L.o32 = take(RD * dmax * 4); L.f32 = take(RD * fmax * 4);
+    if (!bf) {   // blocks of fewer columns, which reach over the planes that fp32 contexts have no use for
+        const size_t end = off;
+        off = amax;
+        take_amax(GS_WARPS * rows_columns(c.large.vocab));
+        off = std::max(off, end);
+    }
     L.proj_snap = take(nS * RD * c.large.d_model * 4);
     L.proj_yhat = take(nS * RD * c.small.d_model * 4);
     L.proj_a = take(nS * RD * c.small.d_model * 4);
@@ -288,11 +323,6 @@ Layout make_layout(const tandem_config& c) {
     L.ln_rows_small = take((size_t)(2 * c.small.n_layers + 1) * 4 * c.small.d_model * 2);
     L.ln_stats = take(RD * ((std::max(c.large.d_model, c.small.d_model) + 31) / 32) * 8);
     L.ln_ref = take(2 * RD * 4);
-    L.fr_seq = take((3 * B + 1) * 4); L.fr_truth = take(RF * 4); L.fr_out = take(RF * 4); L.fr_truth_val = take(RF * 4);
-    L.fr_grp = take(2 * (RF / PASS_GROUP + B + 1) * 4);
-    L.score_tiles = cdiv(c.large.vocab, SCORE_TILE);
-    L.fr_tiles = take((size_t)L.fr_head_rows * L.score_tiles * 12);
-    L.fr_kv = take(bf ? 2 * L.kv_small_layer * esz : 0);
     L.total = off;
     return L;
 }
@@ -649,8 +679,6 @@ void launch_rows_as(tandem_ctx& c, const float* x, int ldx, int M, int K, const 
     launch_ex(c, true, 1, gemm_rows_kernel<MT, NC, LN, EPI>, dim3(cdiv(N, GS_WARPS * NC), cdiv(M, MT)), dim3(GS_THREADS),
               (size_t)MT * std::min(K, GS_KC) * sizeof(float), x, ldx, M, K, ws, N, ln_g, ln_b, e, amax_val, amax_idx, c.amax_tiles);
 }
-// One column per warp until that is two CTAs per multiprocessor, then four (the staged rows are read once for them).
-bool rows_wide(const tandem_ctx& c, int N) { return N > 2 * GS_WARPS * std::max(1, c.n_sms); }
 template <bool LN, int EPI>
 void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, const EpiArgs& e, const void* ln_g = nullptr, const void* ln_b = nullptr,
                  float* av = nullptr, int* ai = nullptr) {
@@ -659,7 +687,7 @@ void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, co
     const int N = lin_n(l), K = l.K;
     const float *g = static_cast<const float*>(ln_g), *b = static_cast<const float*>(ln_b);
     ProfScope ps(c, PC_GEMM_SMALLM, ((double)N * K + (double)M * K + (double)M * N) * sizeof(float));
-    const bool wide = rows_wide(c, N);
+    const bool wide = rows_columns(N) == 4;
     if (M <= 1) { if (wide) launch_rows_as<1, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<1, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
     else if (M <= 4) { if (wide) launch_rows_as<4, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<4, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
     else { if (wide) launch_rows_as<8, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<8, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
@@ -817,8 +845,8 @@ struct Rows {
     double kv_positions;   // context positions read by one attention launch, summed over sequences (accounting only)
     bool whole_pass = false;            // a teacher-forced pass (see forced_pass)
     int plane = 0;                      // ... rows between its planes of values and of remainders
-    const int *grp_row0 = nullptr, *grp_cnt = nullptr;   // ... its attention groups of unequal length, else groups of nq rows
-    bf16 *own_k = nullptr, *own_v = nullptr;             // ... the small model's keys / values of its own, beside the large-derived ones in the cache
+    const int *grp = nullptr, *grp_pos = nullptr;        // ... its attention groups, see AttnArgs::pass_grp
+    bf16 *own_k = nullptr, *own_v = nullptr;             // ... the small model's keys / values of its own [kv head][row of the pass][d_head], beside the large-derived ones in the cache
 };
 
 template <typename T>
@@ -894,8 +922,9 @@ void attention_decode(tandem_ctx& c, const Model& m, int l, const bf16* q, bf16*
     aa.out = o; aa.out_lo = o_lo; aa.ldo = d; aa.row_seq = at<int>(c, c.lay.row_seq); aa.row_pos = at<int>(c, c.lay.row_pos);
     aa.nq = r.nq; aa.n_heads = H; aa.n_kv_heads = m.kv_heads; aa.t_max = c.cfg.max_seq; aa.scale = 1.0f / sqrtf((float)dh);
     aa.err_flag = tc_scratch(c).err;
-    if (r.grp_cnt) { aa.grp_row0 = r.grp_row0; aa.grp_cnt = r.grp_cnt; aa.wait_first = 1; }   // (a group's earlier positions may be rows of this very pass)
-    if (r.own_k) { aa.k2 = r.own_k; aa.v2 = r.own_v; }
+    aa.pass_grp = r.grp; aa.pass_pos = r.grp_pos;
+    if (r.own_k) { aa.k2 = r.own_k; aa.v2 = r.own_v; aa.t_max2 = c.lay.fr_rows; }
+    else if (r.whole_pass) aa.wait_first = 1;   // (a group's earlier positions may be rows of this very pass)
     launch_attn_decode(c, dh, aa, r.groups, r.kv_positions * 2.0 * d * 2.0, r.whole_pass);
 }
 
@@ -1384,16 +1413,11 @@ void pass_layernorm(tandem_ctx& c, int M, int plane, const float* x, const void*
     launch_layernorm<bf16, true>(c, M, x, gain, bias, out, d, raw, (size_t)plane * d);
 }
 
-// Whether a pass's projections run on the side stream, beside the large model's next layers (see prompt_project_forked; 772 rows of the small
-// pair 1548 -> 1515 us, 256 rows 1164 -> 1111, 1200 rows 1984 -> 1921).
-bool pass_forks(const tandem_ctx& c, const Rows& r) { return r.M <= c.lay.fk_rows; }
-
 // FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.
 void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r) {
     const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    const bool fork = pass_forks(c, r);
-    float* yhat = at<float>(c, fork ? c.lay.fk_yhat : c.lay.fr_yhat);
-    bf16 *a_j = at<bf16>(c, fork ? c.lay.fk_a : c.lay.fr_a), *t1 = at<bf16>(c, fork ? c.lay.fk_t1 : c.lay.fr_t1);
+    float* yhat = at<float>(c, c.lay.fr_yhat);
+    bf16 *a_j = at<bf16>(c, c.lay.fr_a), *t1 = at<bf16>(c, c.lay.fr_t1);
     if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
         pass_gemm<EPI_STORE_F32>(c, x, r.M, r.plane, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), epi_plain(yhat, dS));
     } else {
@@ -1407,29 +1431,27 @@ void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r) {
 // One model's layers over a pass's rows in the residual stream h (and the large model's projections between them).
 void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
     const int d = m.d.d_model, dff = m.d.d_ff, n = m.d.n_layers;
-    bf16 *x = at<bf16>(c, c.lay.fr_x), *o = at<bf16>(c, c.lay.fr_o), *f = at<bf16>(c, c.lay.fr_f), *q = at<bf16>(c, c.lay.fr_q), *raw = at<bf16>(c, pass_forks(c, r) ? c.lay.fk_raw : c.lay.fr_raw);
-    const bool large = &m == &c.large, fork = large && pass_forks(c, r);
-    bool forked = false;
+    const bool large = &m == &c.large, fork = large && r.M <= PROMPT_FORK_ROWS;
+    bf16 *x = at<bf16>(c, large ? c.lay.fr_x : c.lay.fr_xs), *f = at<bf16>(c, large ? c.lay.fr_f : c.lay.fr_fs), *q = at<bf16>(c, large ? c.lay.fr_q : c.lay.fr_fs);
+    bf16 *o = x, *raw = at<bf16>(c, c.lay.fr_raw);
     auto project = [&](int l) {
         for (int j = 0; j < c.small.d.n_layers; ++j)
             if (c.layer_map[j] == l) pass_project(c, j, raw, r);
     };
     for (int l = 0; l < n; ++l) {
         const bool from_here = large && projects_from(c, l);
-        if (from_here && forked) prompt_project_join(c);   // (raw is written again)
         pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), x, d, from_here ? raw : nullptr);
         if (from_here) { if (fork) prompt_project_forked(c, [&] { project(l); }); else project(l); }
-        forked = forked || (from_here && fork);
         EpiArgs eq = epi_cache<bf16>(c, m, l, q);
-        if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; }
+        if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; eq.row_seq = eq.row_pos = nullptr; eq.t_max = c.lay.fr_rows; }
         pass_gemm<EPI_QKV>(c, x, r.M, r.plane, tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), eq);
         attention_decode(c, m, l, q, o, o + (size_t)r.plane * d, r);
         pass_gemm<EPI_RESID>(c, o, r.M, r.plane, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), epi_plain(h, d));
+        if (from_here && fork) prompt_project_join(c);   // (the GELU outputs lie over the projections' buffers)
         pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), x, d);
         pass_gemm<EPI_GELU>(c, x, r.M, r.plane, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), epi_plain(f, dff));
         pass_gemm<EPI_RESID>(c, f, r.M, r.plane, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), epi_plain(h, d));
     }
-    if (forked) prompt_project_join(c);
     if (!large || !projects_from(c, n)) return;
     const size_t elems = (size_t)r.M * d;   // after the last layer no LayerNorm of the large model follows
     {
@@ -1439,47 +1461,46 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
     project(n);
 }
 
-// The rows f of a teacher-forced forward (all of whole blocks) through both models.  The large model reads them as one causal pass
+// The rows f of a teacher-forced forward (whole blocks) through both models.  The large model reads them as one causal pass
 // and its projections go to the small model's cache; then the small model reads all blocks at once, since the tokens it would draft
-// are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie in
-// a cache of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
+// are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie
+// row by row in a place of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
 // is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
 // 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.51 ms like this.
-void forced_pass(tandem_ctx& c, const ForcedRows& f, int gamma, int groups_large, double kv_positions) {
+void forced_pass(tandem_ctx& c, ForcedRows f, int groups_large, int groups_small, double kv_positions) {
     const Model &L = c.large, &S = c.small;
     Rows r;
-    r.M = f.rows; r.decode = true; r.whole_pass = true; r.plane = f.rows <= c.lay.fk_rows ? c.lay.fk_rows : c.lay.fr_rows; r.n_chunks = 1; r.kv_positions = kv_positions;
-    float* h = at<float>(c, c.lay.h_large);
-    auto begin = [&](const Model& m, bool setup) {
+    r.M = f.rows; r.decode = true; r.whole_pass = true; r.plane = c.lay.fr_rows; r.n_chunks = 1; r.kv_positions = kv_positions;
+    r.grp = f.grp; r.grp_pos = f.grp_pos;
+    auto begin = [&](const Model& m, float* h, int last_rows) {
         ProfScope ps(c, PC_ROWS, (double)f.rows * m.d.d_model * 8.0);
-        launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + (setup ? 1 : 0)), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
+        launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + 1 + last_rows), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
                   (int)m.d.d_model, (int)c.ticket, (int)c.router_ticket);
     };
-    r.nq = PASS_GROUP; r.groups = groups_large; r.grp_row0 = f.grp_row0; r.grp_cnt = f.grp_cnt;
-    begin(L, true);
+    float *h = at<float>(c, c.lay.h_large), *hs = at<float>(c, c.lay.fr_hs);
+    f.group = PASS_GROUP;
+    r.nq = PASS_GROUP; r.groups = groups_large;
+    begin(L, h, 0);
     pass_layers(c, L, h, r);
-    {
-        ProfScope ps(c, PC_ROWS, (double)f.batch * gamma * L.d.d_model * 8.0);
-        launch_ex(c, true, 1, forced_hidden_kernel, dim3(f.batch * gamma), dim3(128), 0, f, (const float*)h, at<float>(c, c.lay.proj_snap), (int)L.d.d_model);
-    }
-    r.nq = gamma; r.groups = f.rows / gamma; r.grp_row0 = r.grp_cnt = nullptr;
-    r.own_k = at<bf16>(c, c.lay.fr_kv); r.own_v = r.own_k + c.lay.kv_small_layer;
-    begin(S, false);   // (the large model's residual stream has been read for the last time)
-    pass_layers(c, S, h, r);
+    f.group = f.gamma;
+    r.nq = f.gamma; r.groups = groups_small;
+    r.own_k = at<bf16>(c, c.lay.fr_kv); r.own_v = r.own_k + (size_t)c.lay.fr_rows * S.d_kv;
+    begin(S, hs, f.batch * f.gamma);
+    pass_layers(c, S, hs, r);
     const int d = S.d.d_model, tiles = c.lay.score_tiles;
-    bf16* x = at<bf16>(c, c.lay.fr_x);
-    pass_layernorm(c, f.rows, r.plane, h, w_tail(c, S, 0), w_tail(c, S, 1), x, d);
+    bf16* x = at<bf16>(c, c.lay.fr_xs);
+    pass_layernorm(c, f.rows, r.plane, hs, w_tail(c, S, 0), w_tail(c, S, 1), x, d);
     for (int r0 = 0; r0 < f.rows; r0 += c.lay.fr_head_rows) {
         const int rows = std::min(c.lay.fr_head_rows, f.rows - r0);
         float* val = at<float>(c, c.lay.fr_tiles);
         TcScore t;
         t.val = val; t.idx = reinterpret_cast<int*>(val + (size_t)rows * tiles); t.sum = val + (size_t)2 * rows * tiles; t.stride = tiles;
-        t.truth = f.truth + r0; t.truth_val = at<float>(c, c.lay.fr_truth_val);
-        t.keep = f.keep + r0; t.kept = at<float>(c, c.lay.logits_small);
+        t.truth = f.truth + r0; t.truth_val = f.nll + f.v0 + r0;
+        t.keep = f.keep + r0; t.kept = f.last_logits;
         pass_gemm<EPI_SCORE>(c, x + (size_t)r0 * d, rows, r.plane, tcw(c, wi_tail(S, 2), -1, -1, S.d.vocab, d), epi_plain(nullptr, S.d.vocab), t);
         ProfScope ps(c, PC_ARGMAX, 12.0 * rows * tiles);
         launch_ex(c, true, 1, score_tiles_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, rows, tiles, (const float*)t.val, (const int*)t.idx, (const float*)t.sum,
-                  (const float*)t.truth_val, (const int*)(f.out + r0), at<float>(c, c.lay.forced_nll), at<int>(c, c.lay.forced_top));
+                  f.nll + f.v0 + r0, f.top + f.v0 + r0);
     }
 }
 
@@ -1732,7 +1753,7 @@ extern "C" tandem_status tandem_create(const tandem_config* cfg, const tandem_we
     c->use_graphs = getenv("TANDEM_NO_GRAPH") == nullptr;
     c->use_pdl = getenv("TANDEM_NO_PDL") == nullptr;
     c->n_sms = sm_count();
-    c->amax_tiles = cfg->dtype == TANDEM_DTYPE_BF16 ? lay.vocab_tiles : cdiv(cfg->large.vocab, GS_WARPS * (rows_wide(*c, cfg->large.vocab) ? 4 : 1));
+    c->amax_tiles = lay.vocab_tiles;
     if (e == cudaSuccess && cfg->dtype == TANDEM_DTYPE_BF16) {
         // two tensor maps per weight matrix: [out_features][in_features], 128 x 64 tiles and 32 x 64
         c->wmap.resize(c->w.size());
@@ -2202,42 +2223,48 @@ extern "C" tandem_status tandem_speculative_generate(tandem_ctx* c, int32_t gamm
 
 namespace {
 
-// The bf16 form of the call below: passes of as many whole blocks as the work space holds.
+// The bf16 form of the call below: one row per token that has a next one, in passes of as many as the work space holds.
 tandem_status forced_forward(tandem_ctx* c, int gamma, int batch, const int32_t* ids, const int32_t* lens, long long total, float* nll, int32_t* top1) {
     CK(cudaEventSynchronize(c->ev_staged));   // (the staging buffer may still be read by a prompt pass's copy)
-    int32_t *p_ids = c->pinned, *p_off = p_ids + total, *p_len = p_off + batch, *p_start = p_len + batch;
+    int32_t *p_ids = c->pinned, *p_start = p_ids + total;
     memcpy(p_ids, ids, (size_t)total * 4);
-    int off = 0, rows = 0, max_len = 0;
+    int rows = 0, max_len = 0;
     for (int b = 0; b < batch; ++b) {
-        p_off[b] = off; p_len[b] = lens[b]; p_start[b] = rows;
-        off += lens[b];
-        rows += cdiv(lens[b] - 1, gamma) * gamma;
+        p_start[b] = rows;
+        rows += lens[b] - 1;
         max_len = std::max(max_len, lens[b]);
     }
     p_start[batch] = rows;
     CK(cudaMemsetAsync(c->arena + c->lay.st_n, 0, c->lay.row_tok - c->lay.st_n, c->stream));
     CK(cudaMemcpyAsync(c->arena + c->lay.forced_ids, p_ids, (size_t)total * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->arena + c->lay.fr_seq, p_off, (size_t)(3 * batch + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(c->arena + c->lay.fr_start, p_start, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, c->stream));
     CK(cudaEventRecord(c->ev_staged, c->stream));
     c->batch = batch; c->n_ub = max_len; c->n_sum = total; c->last_gamma = gamma;
     c->hidden_at = c->lay.proj_snap;
     launch_call_begin(*c, true);
     ForcedRows f;
-    f.ids = at<int>(*c, c->lay.forced_ids); f.off = at<int>(*c, c->lay.fr_seq); f.len = f.off + batch; f.vstart = f.len + batch;
-    f.batch = batch; f.gamma = gamma; f.group = PASS_GROUP;
+    f.ids = at<int>(*c, c->lay.forced_ids); f.start = at<int>(*c, c->lay.fr_start); f.truth = at<int>(*c, c->lay.fr_truth);
+    f.batch = batch; f.gamma = gamma; f.vocab = c->cfg.large.vocab;
     f.keep = at<int>(*c, c->lay.row_tok); f.row_seq = at<int>(*c, c->lay.row_seq); f.row_pos = at<int>(*c, c->lay.row_pos);
-    f.truth = at<int>(*c, c->lay.fr_truth); f.out = at<int>(*c, c->lay.fr_out);
-    f.grp_row0 = at<int>(*c, c->lay.fr_grp); f.grp_cnt = f.grp_row0 + c->lay.fr_rows / PASS_GROUP + c->cfg.max_batch + 1;
-    const int step = c->lay.fr_rows / gamma * gamma;
-    for (f.v0 = 0; f.v0 < rows; f.v0 += step) {
-        f.rows = std::min(step, rows - f.v0);
-        int groups = 0;
+    f.nll = at<float>(*c, c->lay.forced_nll); f.top = at<int>(*c, c->lay.forced_top);
+    f.hidden = at<float>(*c, c->lay.h_large); f.d_large = c->cfg.large.d_model;
+    f.last_hidden = at<float>(*c, c->lay.proj_snap); f.last_logits = at<float>(*c, c->lay.logits_small);
+    int b0 = 0;
+    for (f.v0 = 0; f.v0 < rows; f.v0 += f.rows) {
+        int end = std::min(rows, f.v0 + c->lay.fr_rows);
+        while (p_start[b0 + 1] <= f.v0) ++b0;
+        int groups_large = 0, groups_small = 0;
         double kv = 0.0;
-        for (int b = 0; b < batch; ++b) {
-            const int n = std::min(p_start[b + 1], f.v0 + f.rows) - std::max(p_start[b], f.v0);
-            if (n > 0) { groups += cdiv(n, f.group); kv += (double)n / f.group * lens[b]; }
+        for (int b = b0; b < batch && p_start[b] < end; ++b) {
+            const int first = std::max(p_start[b], f.v0);
+            if (p_start[b + 1] > end) end -= (end - p_start[b]) % gamma;   // (a block is not cut)
+            const int n = std::min(p_start[b + 1], end) - first;
+            groups_large += cdiv(n, PASS_GROUP); groups_small += cdiv(n, gamma);
+            kv += (double)n / PASS_GROUP * lens[b];
         }
-        forced_pass(*c, f, gamma, groups, kv);
+        f.rows = end - f.v0;
+        f.grp = f.top + f.v0; f.grp_pos = reinterpret_cast<int*>(f.nll) + f.v0;   // (read before the scores are written)
+        forced_pass(*c, f, groups_large, groups_small, kv);
     }
     TRY(check_launch(*c));
     // scores and the error word come back behind one wait (the ids have long been copied out of the staging buffer)

@@ -56,6 +56,26 @@ def test_query_arena_validates_and_sizes(lib):
     assert lib.tandem_query_arena(C.byref(cfg), None) == 1
 
 
+def _pair(large, small, vocab, max_pos, kind=synth.FF_TANDEM_LINEAR, hidden=0, dtype=synth.DTYPE_BF16):
+    return synth.make_shape(synth.ModelDims(*large, vocab, max_pos), synth.ModelDims(*small, vocab, max_pos), kind, hidden, None, dtype)
+
+
+@pytest.mark.parametrize("shape,limits,most", [
+    (synth.named_config("tiny"), (1, 101, 4, 32), 1595904),
+    (synth.named_config("small"), (4, 262, 4, 771), 86630400),
+    (synth.named_config("small"), (1, 33, 4, 28), 4482048),
+    (synth.named_config("medium", 8192), (16, 8192, 3, 0), 35298047744),
+    (synth.named_config("large"), (1, 8448, 5, 0), 5666430976),
+    (_pair((2, 128, 2, 136), (2, 192, 6, 136), 50, 200, synth.FF_TANDEM_MLP, 40), (2, 200, 3, 0), 2650880),      # a small model wider than the large one
+    (_pair((2, 128, 2, 136), (2, 192, 6, 136), 50, 200, synth.FF_TANDEM_MLP, 40), (1, 200, 15, 1), 882688),      # prompts of one token, long blocks
+    (synth.with_dtype(synth.named_config("small"), synth.DTYPE_FP32), (2, 512, 4, 512), 144989952)])
+def test_contexts_fit_the_memory_that_prompt_and_decode_passes_need(lib, shape, limits, most):
+    """Teacher-forced passes and the heads' arg-max results live in space that other passes have anyway.  `most`: caches, loop state,
+    work space of the prompt pass and buffers of the decode passes of these limits, added up without either of the two."""
+    cfg, keep = binding.make_config(shape, *limits[:3], max_prefill_rows=limits[3])
+    assert binding.tandem_query_arena(cfg) <= most
+
+
 def test_null_context_calls_fail_cleanly(lib):
     assert lib.tandem_destroy(None) == 1
     assert lib.tandem_block_step(None, 1, 0, 0, None) == 1

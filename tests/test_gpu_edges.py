@@ -137,16 +137,17 @@ def test_decode_attention_by_lone_ctas(batch, heads, dh, derived, own):
 
 
 @pytest.mark.parametrize("lens,gamma,prefill_rows,kw", [
-    ([2, 140, 23], 4, 0, dict(layer_map=(1, 3), vocab=129)),                     # one pass of 168 rows: three groups, the last of 40; a head tile of one feature
-    ([131, 7, 66], 3, 20, dict(layer_map=(0, 2))),                               # passes of 12 rows: a sequence over many of them
+    ([2, 140, 23], 4, 0, dict(layer_map=(1, 3), vocab=129)),                     # one pass of 162 rows, last blocks of one to three; a head tile of one feature
+    ([131, 7, 66], 3, 20, dict(layer_map=(0, 2))),                               # passes of at most 20 rows, whole blocks: a sequence over many of them
+    ([190, 180], 4, 0, dict(large=(2, 128, 2, 2048), layer_map=(0, 2), max_pos=200)),   # a work space that holds fewer rows than a prompt pass's
     ([47], 15, 0, dict(large=(2, 256, 2, 264), small=(1, 256, 2, 136), kv_heads=(1, 1), layer_map=(2,))),   # blocks of 15, 128-wide heads, shared keys / values
     ([66, 2], 1, 0, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3), small=(2, 192, 6, 136))),  # 66 blocks of one row; a small model wider than the large one
     ([141], 1, 0, dict(layer_map=(0, 3), small=(2, 192, 6, 136))),               # 840 block heads: two warps share the keys of each (four up to 592)
     ([130, 70], 1, 0, dict(layer_map=(0, 3), small=(2, 192, 6, 136)))])          # 1188: one warp each (two up to 1184)
 def test_bf16_teacher_forced_pass(lens, gamma, prefill_rows, kw):
-    """All blocks of a teacher-forced forward in one pass or a few: ragged sequences padded to whole blocks, groups of 64 rows, blocks
-    that attend large-derived keys up to their start and their own from there."""
-    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, **kw)
+    """All blocks of a teacher-forced forward in one pass or a few: ragged sequences, short last blocks, groups of eight rows of the large
+    model, blocks that attend large-derived keys up to their start and their own from there."""
+    shape = gpu_toy_shape(**{**dict(dtype=synth.DTYPE_BF16, max_pos=200), **kw})
     w = _bf16_weights(shape, seed=23, std=0.06)
     seqs = prompts_for(shape, lens, seed=24)
     t = binding.Tandem(shape, w, max_batch=len(lens), max_seq=200, gamma_max=gamma, max_prefill_rows=prefill_rows)
@@ -186,6 +187,8 @@ def test_bf16_logits_and_representations_of_the_last_blocks(lens, gamma, prefill
         for p in range(first, len(ids) - 1):
             assert np.abs(logits[p - first, b] - want[p]).max() < TOL_BF16
             assert np.abs(hidden[b * gamma + p - first] - reps[-1][p]).max() < 2 * TOL_BF16
+        past = (len(ids) - 2) % gamma + 1
+        assert not logits[past:, b].any() and not hidden[b * gamma + past:(b + 1) * gamma].any()
     t.tandem_prefill([s[:3] for s in seqs])       # and a decode iteration's own again
     res = t.tandem_block_step(gamma)
     hidden = t.tandem_debug_read(binding.READ_LARGE_HIDDEN, gamma)
