@@ -2103,7 +2103,7 @@ tandem_status adaptive_iteration(tandem_ctx* c, int gamma_max, int max_new, int*
     int s = 0;
     for (; s < gamma_max; ++s) {
         TRY(launch_iteration(*c, 3, s, gamma_max, 0ull, max_new));
-        if (c->cfg.dtype == TANDEM_DTYPE_BF16) TRY(launch_iteration(*c, 5, s, gamma_max, 0ull, max_new));
+        if (c->cfg.dtype == TANDEM_DTYPE_BF16) TRY(launch_iteration(*c, 5, s, gamma_max, 0ull, 0));   // (no step depends on the tokens asked for: one graph for every length of response)
         TRY(wait_ticket(*c, c->router_ticket, 5));
         if (c->hflags[6] <= 0) { ++s; break; }
     }

@@ -1,4 +1,8 @@
 """Edges of the kernels' dispatch rules and tiles, each against the fp64 checker."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -211,6 +215,38 @@ def test_bf16_teacher_forced_pass_beyond_the_forked_rows():
     for got, want in zip(whole, parts):
         assert np.abs(got - want).max() < 2 * TOL_BF16
     t.close()
+
+
+_CAPTURES = """
+import sys
+sys.path[:0] = [{root!r}, {root!r} + "/tests"]
+import torch
+from paper_2402_08644_b200 import binding, synth
+from test_gpu_parity import _bf16_weights, gpu_toy_shape, prompts_for
+shape = gpu_toy_shape(dtype=synth.DTYPE_BF16)
+t = binding.Tandem(shape, _bf16_weights(shape, seed=1, std=0.05), max_batch=1, max_seq=128, gamma_max=4)
+t.tandem_set_router(synth.make_router(shape, 2, 8, 1), 0.0)    # tau 0: every block has four drafts
+def respond(new):
+    t.tandem_prefill(prompts_for(shape, [7], seed=3))
+    return t.tandem_adaptive_generate(4, new)[0].tolist()
+respond(24)
+with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as p:
+    got = respond(31)
+    torch.cuda.synchronize()
+names = [e.name for e in p.events()]
+print(names.count("cudaStreamBeginCapture"), sum("GraphLaunch" in n for n in names), got == respond(31))
+"""
+
+
+def test_bf16_adaptive_response_of_another_length_finds_its_graphs():
+    """The draft steps do not depend on the number of tokens asked for: a longer response captures the verify half (whose kernel
+    does) and none of the four steps again."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", _CAPTURES.format(root=root)], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    captures, launches, same = out.stdout.split()[-3:]
+    assert same == "True" and int(launches) >= 8
+    assert int(captures) <= 1
 
 
 def test_bf16_layernorm_parameters_changed_between_calls():
