@@ -109,19 +109,28 @@ __device__ __forceinline__ float warp_sum_many(float (&v)[NV], int lane) {
 // Bound by latency (the fp32 pair's matrices are 0.06-1 MB): NC = 1 spreads N = 256..1024 over the whole GPU, NC = 4 reads
 // the staged rows once per four columns when there are columns enough; a warp's first weights are fetched before the wait
 // on the preceding kernel; the row sums leave the warp through warp_sum_many and are finished by several lanes side by
-// side.  One short row goes from L2 straight into the registers of every warp; more rows are staged with all of a thread's loads
-// in flight.  Up to 512 elements a row is normalised in a warp's registers on its way, with gain and bias fetched ahead of the wait.  (Staging
-// loads one after the other, statistics from shared memory and rows read and written back for LayerNorm: a layer of the 128-wide model, one row, 11.9 us of the chain, 9.4 like this; of the 256-wide one, five rows, 18.7 and 17.3.)
+// side.  One short row goes from L2 straight into the registers of every warp; more rows are staged by copies that pass no register.  Short
+// rows are normalised in a warp's registers on their way, with gain and bias fetched ahead of the wait.
+// At most 128 registers (FORM keeps apart what a launch never needs together), so that two CTAs fit a multiprocessor and a successor can
+// set up beside its predecessor.  Requests of the 256 / 128-wide pair, 48 tokens at gamma 4, 1 / 4 / 8 / 16 sequences: 4.61 / 5.80 / 8.04 /
+// 11.2 ms with staged rows in registers (up to 236: one CTA), 4.37 / 4.70 / 5.99 / 7.56 like this (1: 64 tokens), 4.45 / 4.85 / 6.15 / 7.03 squeezed
+// into 80 registers for three CTAs.  1024 / 512-wide, 24 tokens at gamma 3, 4 sequences: 16.7, 13.7, 14.3.
 // grid: (ceil(N / (GS_WARPS * NC)), ceil(M / MT)); dynamic smem: MT * min(K, GS_KC) floats.
-template <int MT, int NC, bool LN, int EPI>
-__global__ void __launch_bounds__(GS_THREADS)
+enum { ROWS_PLAIN = 0, ROWS_LN_REGS = 1, ROWS_LN_SMEM = 2 };
+// Longest row that a warp normalises in its registers: 512 elements with one column per warp, 256 with four.
+__host__ __device__ constexpr int rows_ln_regs_max(int nc) { return 128 * (8 / nc < 4 ? 8 / nc : 4); }
+template <int MT, int NC, int FORM, int EPI>
+__global__ void __launch_bounds__(GS_THREADS, 2)
 gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, int N, const float* __restrict__ ln_g,
                  const float* __restrict__ ln_b, EpiArgs e, float* amax_val, int* amax_idx, int amax_stride) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float* xs = reinterpret_cast<float*>(smem_raw);
-    constexpr int PF = 8 / NC;    // float4s of each column fetched ahead of the wait
+    constexpr bool LN_REGS = FORM == ROWS_LN_REGS;
+    constexpr int LV = rows_ln_regs_max(NC) / 128;   // float4s per lane of a row that is normalised in registers
+    constexpr int PF = LN_REGS ? LV : 8 / NC;        // float4s of each column fetched ahead of the wait
     constexpr int NV = MT * NC;
     constexpr int LOG = NV == 1 ? 0 : (NV == 4 ? 2 : (NV == 8 ? 3 : (NV == 16 ? 4 : 5)));
+    static_assert(MT <= GS_WARPS, "a warp per row where rows are normalised");
     static_assert(NV == 1 || NV == 4 || NV == 8 || NV == 16 || NV == 32, "warp_sum_many");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n0 = (blockIdx.x * GS_WARPS + warp) * NC;
@@ -139,31 +148,18 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
             const int kk = (lane + 32 * i) * 4;
             wpre[c][i] = (wrow[c] != nullptr && kk < K) ? __ldg(reinterpret_cast<const float4*>(wrow[c] + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-    constexpr int LV = PF < 4 ? PF : 4;            // float4s per lane of a row that is normalised in registers
-    const bool ln_regs = LN && K <= 128 * LV;
-    const bool direct = MT == 1 && (LN ? ln_regs : K <= 128 * PF);
-    float4 g[LN ? LV : 1], b[LN ? LV : 1];
-    if (ln_regs) {
+    const bool direct = MT == 1 && (LN_REGS || (FORM == ROWS_PLAIN && K <= 128 * PF));
+    float4 g[LN_REGS ? LV : 1], b[LN_REGS ? LV : 1];
+    if constexpr (LN_REGS) {
 #pragma unroll
-        for (int v = 0; v < (LN ? LV : 1); ++v) {
+        for (int v = 0; v < LV; ++v) {
             const int kk = (lane + 32 * v) * 4;
             g[v] = kk < K ? __ldg(reinterpret_cast<const float4*>(ln_g + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
             b[v] = kk < K ? __ldg(reinterpret_cast<const float4*>(ln_b + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
-    // where this thread's float4s of the first staging pass come from and go (a division per load ahead of the wait, none behind it)
-    constexpr int ST = MT == 1 ? 2 : 8;
-    int off_x[ST], off_s[ST];
-    {
-        const int vec = KS >> 2;
-        int r = threadIdx.x / vec, v = threadIdx.x - r * vec;
-#pragma unroll
-        for (int u = 0; u < ST; ++u) {
-            off_x[u] = r * ldx + v * 4;
-            off_s[u] = r < rows ? r * KS + v * 4 : -1;
-            for (v += GS_THREADS; v >= vec; v -= vec) ++r;
-        }
-    }
+    // where this thread's first float4 of a staging pass lies (the division ahead of the wait)
+    const int r_first = threadIdx.x / (KS >> 2), v_first = threadIdx.x - r_first * (KS >> 2);
     pdl_wait();
     pdl_launch_dependents();
 
@@ -191,7 +187,7 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
             const int kk = (lane + 32 * v) * 4;
             t[v] = kk < K ? __ldcg(reinterpret_cast<const float4*>(x + (size_t)m * ldx + kk)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if constexpr (LN) {
+        if constexpr (LN_REGS) {
             float sum = 0.f, q = 0.f;
 #pragma unroll
             for (int v = 0; v < V; ++v) if ((lane + 32 * v) * 4 < K) sum += (t[v].x + t[v].y) + (t[v].z + t[v].w);
@@ -212,51 +208,51 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
     };
     auto dot = [&](float& a, const float4& xv, const float4& w) { a = fmaf(xv.x, w.x, a); a = fmaf(xv.y, w.y, a); a = fmaf(xv.z, w.z, a); a = fmaf(xv.w, w.w, a); };
     if (direct) {
-        constexpr int V = LN ? LV : PF;
-        float4 t[V];
+        float4 t[PF];
         load_row(t, m0);
 #pragma unroll
-        for (int v = 0; v < V; ++v)
+        for (int v = 0; v < PF; ++v)
 #pragma unroll
             for (int c = 0; c < NC; ++c) if ((lane + 32 * v) * 4 < K) dot(acc[c], t[v], wpre[c][v]);
     } else
     for (int k0 = 0; k0 < K; k0 += GS_KC) {
         const int kc = min(GS_KC, K - k0), vec = kc >> 2;
         __syncthreads();
-        if (ln_regs) {   // (K <= 512: the only staging pass) a warp per row
-            for (int r = warp; r < rows; r += GS_WARPS) {
+        if constexpr (LN_REGS) {   // (the only staging pass) a warp per row
+            if (warp < rows) {
                 float4 t[LV];
-                load_row(t, m0 + r);
+                load_row(t, m0 + warp);
 #pragma unroll
                 for (int v = 0; v < LV; ++v)
-                    if ((lane + 32 * v) * 4 < K) *reinterpret_cast<float4*>(xs + r * KS + (lane + 32 * v) * 4) = t[v];
+                    if ((lane + 32 * v) * 4 < K) *reinterpret_cast<float4*>(xs + warp * KS + (lane + 32 * v) * 4) = t[v];
             }
-        } else if (k0 == 0 && rows * vec <= ST * GS_THREADS) {   // all of this thread's loads in flight
-            float4 t[ST];
-#pragma unroll
-            for (int u = 0; u < ST; ++u) if (off_s[u] >= 0) t[u] = __ldcg(reinterpret_cast<const float4*>(x + (size_t)m0 * ldx + off_x[u]));
-#pragma unroll
-            for (int u = 0; u < ST; ++u) if (off_s[u] >= 0) *reinterpret_cast<float4*>(xs + off_s[u]) = t[u];
-        } else {
-            for (int i = threadIdx.x; i < rows * vec; i += GS_THREADS) {
-                const int r = i / vec, v = i - r * vec;
-                *reinterpret_cast<float4*>(xs + r * KS + v * 4) = __ldcg(reinterpret_cast<const float4*>(x + (size_t)(m0 + r) * ldx + k0 + v * 4));
+        } else {   // all of this thread's copies in flight, none in registers
+            int r = r_first, v = v_first;
+            if (kc != KS) { r = threadIdx.x / vec; v = threadIdx.x - r * vec; }
+            while (r < rows) {
+                cp_async16(xs + r * KS + v * 4, x + (size_t)(m0 + r) * ldx + k0 + v * 4);
+                for (v += GS_THREADS; v >= vec; v -= vec) ++r;
             }
+            cp_async_commit();
+            cp_async_wait_all();
         }
         __syncthreads();
-        if (LN && !ln_regs) {   // one warp per row, fixed lane-strided order (biased variance, eps 1e-5)
-            for (int r = warp; r < rows; r += GS_WARPS) {
-                float* xr = xs + r * KS;
+        if constexpr (FORM == ROWS_LN_SMEM) {   // one warp per row, fixed lane-strided order (biased variance, eps 1e-5)
+            if (warp < rows) {
+                float* xr = xs + warp * KS;
                 float s = 0.f;
+#pragma unroll 4
                 for (int k = lane * 4; k < K; k += 128) { const float4 t = *reinterpret_cast<const float4*>(xr + k); s += (t.x + t.y) + (t.z + t.w); }
                 const float mu = warp_sum(s) / (float)K;
                 float q = 0.f;
+#pragma unroll 4
                 for (int k = lane * 4; k < K; k += 128) {
                     const float4 t = *reinterpret_cast<const float4*>(xr + k);
                     const float d0 = t.x - mu, d1 = t.y - mu, d2 = t.z - mu, d3 = t.w - mu;
                     q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); q = fmaf(d2, d2, q); q = fmaf(d3, d3, q);
                 }
                 const float rs = 1.0f / sqrtf(warp_sum(q) / (float)K + 1e-5f);
+#pragma unroll 4
                 for (int k = lane * 4; k < K; k += 128) {
                     float4 t = *reinterpret_cast<const float4*>(xr + k);
                     const float4 g = __ldg(reinterpret_cast<const float4*>(ln_g + k)), b = __ldg(reinterpret_cast<const float4*>(ln_b + k));
@@ -279,6 +275,7 @@ gemm_rows_kernel(const float* __restrict__ x, int ldx, int M, int K, WSegs ws, i
             }
             i = PF;
         }
+        if constexpr (LN_REGS) break;   // (a row that fits a warp's registers has had all its products)
 #pragma unroll 2
         for (int kk = (lane + 32 * i) * 4; kk < kc; kk += 128) {
             float4 w[NC];

@@ -10,6 +10,7 @@
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/tandem.h"
@@ -671,12 +672,12 @@ WSegs segs_of(const tandem_ctx& c, const Lin& l) {
 }
 
 // fp32, few rows.  ln_g / ln_b non-null: LayerNorm of the rows first (fused; K <= GS_KC, see fp32_few_rows).
-template <int MT, int NC, bool LN, int EPI>
+template <int MT, int NC, int FORM, int EPI>
 void launch_rows_as(tandem_ctx& c, const float* x, int ldx, int M, int K, const WSegs& ws, int N, const float* ln_g, const float* ln_b, const EpiArgs& e,
                     float* amax_val, int* amax_idx) {
     static std::atomic<unsigned long long> attr_done{0};
-    ensure_dyn_smem(gemm_rows_kernel<MT, NC, LN, EPI>, (size_t)MT * GS_KC * sizeof(float), attr_done);
-    launch_ex(c, true, 1, gemm_rows_kernel<MT, NC, LN, EPI>, dim3(cdiv(N, GS_WARPS * NC), cdiv(M, MT)), dim3(GS_THREADS),
+    ensure_dyn_smem(gemm_rows_kernel<MT, NC, FORM, EPI>, (size_t)MT * GS_KC * sizeof(float), attr_done);
+    launch_ex(c, true, 1, gemm_rows_kernel<MT, NC, FORM, EPI>, dim3(cdiv(N, GS_WARPS * NC), cdiv(M, MT)), dim3(GS_THREADS),
               (size_t)MT * std::min(K, GS_KC) * sizeof(float), x, ldx, M, K, ws, N, ln_g, ln_b, e, amax_val, amax_idx, c.amax_tiles);
 }
 template <bool LN, int EPI>
@@ -688,9 +689,16 @@ void launch_rows(tandem_ctx& c, const float* x, int ldx, int M, const Lin& l, co
     const float *g = static_cast<const float*>(ln_g), *b = static_cast<const float*>(ln_b);
     ProfScope ps(c, PC_GEMM_SMALLM, ((double)N * K + (double)M * K + (double)M * N) * sizeof(float));
     const bool wide = rows_columns(N) == 4;
-    if (M <= 1) { if (wide) launch_rows_as<1, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<1, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
-    else if (M <= 4) { if (wide) launch_rows_as<4, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<4, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
-    else { if (wide) launch_rows_as<8, 4, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); else launch_rows_as<8, 1, LN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai); }
+    auto go = [&](auto mt, auto nc) {
+        constexpr int MT = decltype(mt)::value, NC = decltype(nc)::value;
+        if constexpr (!LN) launch_rows_as<MT, NC, ROWS_PLAIN, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai);
+        else if (K <= rows_ln_regs_max(NC)) launch_rows_as<MT, NC, ROWS_LN_REGS, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai);
+        else launch_rows_as<MT, NC, ROWS_LN_SMEM, EPI>(c, x, ldx, M, K, ws, N, g, b, e, av, ai);
+    };
+    auto columns = [&](auto mt) { if (wide) go(mt, std::integral_constant<int, 4>()); else go(mt, std::integral_constant<int, 1>()); };
+    if (M <= 1) columns(std::integral_constant<int, 1>());
+    else if (M <= 4) columns(std::integral_constant<int, 4>());
+    else columns(std::integral_constant<int, 8>());
 }
 
 // y = x W^T with a fused epilogue for many rows: the prompt-pass kernels (tensor cores for bf16).

@@ -30,6 +30,15 @@ def test_fp32_few_row_kernels_at_their_edges(lens, gamma):
     assert _replay_compare(shape, w, prompts_for(shape, lens, seed=4), gamma, 3, TOL_FP32, 1e-6, check_kv=True) == 0
 
 
+@pytest.mark.parametrize("width", [256, 288, 512, 544])   # LayerNorm in registers up to 256 elements with four columns per warp (the heads), 512 with one
+@pytest.mark.parametrize("lens,gamma", [([6], 0), ([6], 3), ([5, 9, 3], 2)])   # one row, four, nine (eight and one)
+def test_fp32_few_row_kernel_forms(width, lens, gamma):
+    """Rows at and behind the lengths up to which a warp normalises them in its registers, in every row count's form."""
+    shape = gpu_toy_shape(large=(1, width, width // 32, 264), small=(1, width, width // 32, 136), vocab=2400, max_pos=64, layer_map=(1,))
+    w = toy_weights(shape, seed=5, std=0.03)
+    assert _replay_compare(shape, w, prompts_for(shape, lens, seed=6), gamma, 3, TOL_FP32, 1e-6, check_kv=True) == 0
+
+
 @pytest.mark.parametrize("lens", [[129],            # one row tile: K dealt to four CTAs (17 K-blocks: 4, 4, 4, 5)
                                   [130, 2, 1],      # two row tiles, the second of two rows; a prompt without processed rows
                                   [900, 385]])      # ten: two CTAs per tile, or one
