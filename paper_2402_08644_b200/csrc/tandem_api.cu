@@ -60,6 +60,7 @@ struct Layout {   // byte offsets into the arena
     // ... in one pass (bf16), see place_pass: rows in front of the products, GELU outputs, queries and the projections' buffers of the
     // large model's part; stream, rows, own keys / values, GELU outputs, queries of the small model's; the head's per-tile results
     size_t fr_x, fr_f, fr_q, fr_raw, fr_yhat, fr_a, fr_t1, fr_hs, fr_xs, fr_kv, fr_fs, fr_tiles;
+    size_t fa_yhat, fa_a, fa_t1;            // ... the projections' buffers apart from what the large model's layers write
     size_t fr_start, fr_truth;              // ... the sequences' first rows, the rows' next tokens (where a prompt pass has its staged inputs)
     size_t row_tok, row_seq, row_pos, grp_row0, grp_cnt;
     size_t stage;                                   // a prompt pass's lengths, offsets and token ids as the host staged them
@@ -72,6 +73,7 @@ struct Layout {   // byte offsets into the arena
     size_t proj_snap, proj_yhat, proj_a, proj_t1;   // per small layer: the decode projection's own buffers (it runs beside the large pass)
     size_t total;
     int max_rows, dec_rows, max_groups, n_chunks_max, vocab_tiles, score_tiles;
+    int fr_apart;                            // whether there is a second set of the projections' buffers
     int fr_rows, fr_head_rows;               // most rows of a teacher-forced pass, and of one run of its output head
     size_t kv_large_layer, kv_small_layer;   // elements per (layer, k-or-v)
 };
@@ -295,9 +297,18 @@ Layout make_layout(const tandem_config& c) {
         L.fr_head_rows = (int)std::max(few, std::min(std::min<size_t>(rows, 1024), (pass_end - L.fr_tiles) / tile_bytes));
         off = std::max(pass_end, align_up(L.fr_tiles + few * tile_bytes));
     }
-    L.logits_large = take(RD * V * 4);
-    L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
     L.dbg = take(T * dmax * 4);
+    L.logits_small = take((size_t)std::max(1, c.gamma_max) * B * V * 4);
+    if (bf) {
+        // Behind the large model's part, up to the end of the logits that only its successor writes: the projections' buffers once more, if
+        // they fit (see Rows::apart).
+        const size_t end = off, rows = L.fr_rows, t1 = c.ff_tandem_kind == TANDEM_FF_LINEAR ? 0 : rows * hidden * 4, y = rows * c.small.d_model * 4;
+        off = std::max(L.fr_q + rows * c.large.d_model * 2, L.fr_f + rows * c.large.d_ff * 4);
+        off = align_up(off);
+        if (off + align_up(t1) + 2 * align_up(y) <= end) { L.fa_t1 = take(t1); L.fa_yhat = take(y); L.fa_a = take(y); L.fr_apart = 1; }
+        off = end;
+    }
+    L.logits_large = take(RD * V * 4);
     L.forced_ids = take(B * T * 4); L.forced_len = take(B * 4); L.forced_nll = take(B * T * 4); L.forced_top = take(B * T * 4);
     L.smp_large = take(RD * 8); L.smp_small = take((size_t)std::max(1, c.gamma_max) * B * 8);
     auto take_amax = [&](int columns) {
@@ -853,6 +864,7 @@ struct Rows {
     double kv_positions;   // context positions read by one attention launch, summed over sequences (accounting only)
     bool whole_pass = false;            // a teacher-forced pass (see forced_pass)
     int plane = 0;                      // ... rows between its planes of values and of remainders
+    bool apart = false;                 // ... whose projections' buffers (but their input) lie apart from what the large model's layers write
     const int *grp = nullptr, *grp_pos = nullptr;        // ... its attention groups, see AttnArgs::pass_grp
     bf16 *own_k = nullptr, *own_v = nullptr;             // ... the small model's keys / values of its own [kv head][row of the pass][d_head], beside the large-derived ones in the cache
 };
@@ -1001,7 +1013,7 @@ void project_after(tandem_ctx& c, int n_large_layers_done, const Rows& r) {
 // waits for the last ones before the next copy is made, and for all of them at the end of the pass.  (Small pair, 99 / 511 / 1499 rows: 602 -> 567, 759 -> 731, 1279 -> 1235 us;
 // large pair, 899 rows: 1 %.)
 template <typename P>
-void prompt_project_forked(tandem_ctx& c, P project) {
+void prompt_project_forked(tandem_ctx& c, P project, bool join_all = true) {
     cudaStream_t main_stream = c.stream;
     cudaEvent_t fork = c.ev_fork[0];
     cudaEventRecord(fork, main_stream);
@@ -1009,7 +1021,7 @@ void prompt_project_forked(tandem_ctx& c, P project) {
     c.stream = c.side;
     c.next_launch_plain = true;   // first kernel after a cross-stream wait
     project();
-    cudaEventRecord(c.ev_join, c.side);
+    if (join_all) cudaEventRecord(c.ev_join, c.side);   // (else by `project`)
     c.stream = main_stream;
 }
 void prompt_project_join(tandem_ctx& c) {
@@ -1422,14 +1434,17 @@ void pass_layernorm(tandem_ctx& c, int M, int plane, const float* x, const void*
 }
 
 // FF_Tandem of a pass's rows (planes x, the large model's residual stream) for small layer j, into the small model's cache.
-void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r) {
+// read (nullable): recorded when x has been read.
+void pass_project(tandem_ctx& c, int j, const bf16* x, const Rows& r, cudaEvent_t read = nullptr) {
     const int dL = c.large.d.d_model, dS = c.small.d.d_model;
-    float* yhat = at<float>(c, c.lay.fr_yhat);
-    bf16 *a_j = at<bf16>(c, c.lay.fr_a), *t1 = at<bf16>(c, c.lay.fr_t1);
+    float* yhat = at<float>(c, r.apart ? c.lay.fa_yhat : c.lay.fr_yhat);
+    bf16 *a_j = at<bf16>(c, r.apart ? c.lay.fa_a : c.lay.fr_a), *t1 = at<bf16>(c, r.apart ? c.lay.fa_t1 : c.lay.fr_t1);
     if (c.cfg.ff_tandem_kind == TANDEM_FF_LINEAR) {
         pass_gemm<EPI_STORE_F32>(c, x, r.M, r.plane, tcw(c, wi_tandem(c, j, 0), -1, -1, dS, dL), epi_plain(yhat, dS));
+        if (read) cudaEventRecord(read, c.stream);
     } else {
         pass_gemm<EPI_GELU>(c, x, r.M, r.plane, tcw(c, wi_tandem(c, j, 0), -1, -1, c.hidden, dL), epi_plain(t1, c.hidden));
+        if (read) cudaEventRecord(read, c.stream);
         pass_gemm<EPI_STORE_F32>(c, t1, r.M, r.plane, tcw(c, wi_tandem(c, j, 1), -1, -1, dS, c.hidden), epi_plain(yhat, dS));
     }
     pass_layernorm(c, r.M, r.plane, yhat, w_layer(c, c.small, j, W_LN1G), w_layer(c, c.small, j, W_LN1B), a_j, dS);
@@ -1442,31 +1457,38 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
     const bool large = &m == &c.large, fork = large && r.M <= PROMPT_FORK_ROWS;
     bf16 *x = at<bf16>(c, large ? c.lay.fr_x : c.lay.fr_xs), *f = at<bf16>(c, large ? c.lay.fr_f : c.lay.fr_fs), *q = at<bf16>(c, large ? c.lay.fr_q : c.lay.fr_fs);
     bf16 *o = x, *raw = at<bf16>(c, c.lay.fr_raw);
-    auto project = [&](int l) {
-        for (int j = 0; j < c.small.d.n_layers; ++j)
-            if (c.layer_map[j] == l) pass_project(c, j, raw, r);
+    // Forked, the large model goes on to its FFN when the layer's projections are done, whose buffers lie under the GELU outputs; or when their
+    // input has been read, where the others lie apart (769 rows of the small pair: 1548 -> 1533 us).
+    auto project = [&](int l, bool forked) {
+        int last = 0;
+        for (int j = 0; j < c.small.d.n_layers; ++j) if (c.layer_map[j] == l) last = j;
+        for (int j = 0; j <= last; ++j)
+            if (c.layer_map[j] == l) pass_project(c, j, raw, r, forked && r.apart && j == last ? c.ev_join : nullptr);
     };
+    bool forked = false;
     for (int l = 0; l < n; ++l) {
         const bool from_here = large && projects_from(c, l);
         pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN1G), w_layer(c, m, l, W_LN1B), x, d, from_here ? raw : nullptr);
-        if (from_here) { if (fork) prompt_project_forked(c, [&] { project(l); }); else project(l); }
+        if (from_here) { if (fork) prompt_project_forked(c, [&] { project(l, true); }, !r.apart); else project(l, false); }
+        forked = forked || (from_here && fork);
         EpiArgs eq = epi_cache<bf16>(c, m, l, q);
         if (r.own_k) { eq.kcache = r.own_k; eq.vcache = r.own_v; eq.row_seq = eq.row_pos = nullptr; eq.t_max = c.lay.fr_rows; }
         pass_gemm<EPI_QKV>(c, x, r.M, r.plane, tcw3(c, wi_layer(m, l, W_WQ), wi_layer(m, l, W_WK), wi_layer(m, l, W_WV), d, m.d_kv, d), eq);
         attention_decode(c, m, l, q, o, o + (size_t)r.plane * d, r);
         pass_gemm<EPI_RESID>(c, o, r.M, r.plane, tcw(c, wi_layer(m, l, W_WO), -1, -1, d, d), epi_plain(h, d));
-        if (from_here && fork) prompt_project_join(c);   // (the GELU outputs lie over the projections' buffers)
+        if (from_here && fork) prompt_project_join(c);
         pass_layernorm(c, r.M, r.plane, h, w_layer(c, m, l, W_LN2G), w_layer(c, m, l, W_LN2B), x, d);
         pass_gemm<EPI_GELU>(c, x, r.M, r.plane, tcw(c, wi_layer(m, l, W_W1), -1, -1, dff, d), epi_plain(f, dff));
         pass_gemm<EPI_RESID>(c, f, r.M, r.plane, tcw(c, wi_layer(m, l, W_W2), -1, -1, d, dff), epi_plain(h, d));
     }
+    if (forked && r.apart) project_join(c);
     if (!large || !projects_from(c, n)) return;
     const size_t elems = (size_t)r.M * d;   // after the last layer no LayerNorm of the large model follows
     {
         ProfScope ps(c, PC_ROWS, (double)elems * 8.0);
         launch_ex(c, true, 1, cast_rows_kernel<true>, dim3((unsigned)((elems / 8 + 255) / 256)), dim3(256), 0, (const float*)h, raw, elems, (size_t)r.plane * d);
     }
-    project(n);
+    project(n, false);
 }
 
 // The rows f of a teacher-forced forward (whole blocks) through both models.  The large model reads them as one causal pass
@@ -1475,11 +1497,12 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
 // row by row in a place of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
 // is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
 // 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.51 ms like this.
-void forced_pass(tandem_ctx& c, ForcedRows f, int groups_large, int groups_small, double kv_positions) {
+void forced_pass(tandem_ctx& c, ForcedRows f, bool only, int groups_large, int groups_small, double kv_positions) {
     const Model &L = c.large, &S = c.small;
     Rows r;
     r.M = f.rows; r.decode = true; r.whole_pass = true; r.plane = c.lay.fr_rows; r.n_chunks = 1; r.kv_positions = kv_positions;
     r.grp = f.grp; r.grp_pos = f.grp_pos;
+    r.apart = only && c.lay.fr_apart != 0;   // (of several passes, an earlier one has left logits there)
     auto begin = [&](const Model& m, float* h, int last_rows) {
         ProfScope ps(c, PC_ROWS, (double)f.rows * m.d.d_model * 8.0);
         launch_ex(c, true, 1, forced_rows_kernel, dim3(f.rows + 1 + last_rows), dim3(128), 0, c.st, f, (const bf16*)w_emb(c, m), (const bf16*)w_pos(c, m), h,
@@ -2272,7 +2295,7 @@ tandem_status forced_forward(tandem_ctx* c, int gamma, int batch, const int32_t*
         }
         f.rows = end - f.v0;
         f.grp = f.top + f.v0; f.grp_pos = reinterpret_cast<int*>(f.nll) + f.v0;   // (read before the scores are written)
-        forced_pass(*c, f, groups_large, groups_small, kv);
+        forced_pass(*c, f, f.rows == rows, groups_large, groups_small, kv);
     }
     TRY(check_launch(*c));
     // scores and the error word come back behind one wait (the ids have long been copied out of the staging buffer)
