@@ -105,11 +105,24 @@ def test_bf16_prompt_layernorm_by_warps_and_blocks(width, heads, lens):
 
 @pytest.mark.parametrize("heads", [2, 1])   # head sizes 64 and 128: chunks of 64 and of 128 keys
 def test_bf16_prompt_attention_at_chunk_edges(heads):
-    """Prompts that end one query before, at and behind the end of a chunk, a tile and a group of two tiles, in one batch."""
+    """Prompts that end one query before, at and behind the end of a chunk and a tile, in one batch.  (So few heads: one tile of
+    queries per CTA.)"""
     shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, 128, heads, 128), small=(1, 64, 1, 64), max_pos=640, layer_map=(1,))
     w = _bf16_weights(shape, seed=12, std=0.1)
     prompts = prompts_for(shape, [64, 65, 66, 128, 129, 130, 256, 257, 258, 386, 514], seed=13)
     assert _replay_compare(shape, w, prompts, 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 4
+
+
+@pytest.mark.parametrize("width", [384, 768])   # six heads of 64 and of 128
+def test_bf16_prompt_attention_in_groups_of_two_tiles(width):
+    """The same ends with heads enough that a CTA takes two tiles: a second tile of one query, one that ends at and behind a chunk, a
+    group that ends at 256 and 257 queries."""
+    lens, heads = [64, 65, 66, 128, 129, 130, 256, 257, 258, 386, 514], 6
+    assert ((sum(lens) - len(lens)) // 256 + len(lens)) * heads * 2 > 148    # two tiles of queries per CTA on 148 multiprocessors
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, large=(1, width, heads, 128), small=(1, 64, 1, 64), max_pos=640, layer_map=(1,))
+    # what bf16 keys, values and activations cost grows with the logits' spread, std * sqrt(width): 2.2e-2 at 1.39, so 0.8 stays below 1.3e-2
+    w = _bf16_weights(shape, seed=12, std=0.8 / width ** 0.5)
+    assert _replay_compare(shape, w, prompts_for(shape, lens, seed=13), 1, 1, TOL_BF16, 2 * TOL_BF16, check_kv=True) <= 4
 
 
 @pytest.mark.parametrize("width,ffn", [(512, 1160), (576, 1288), (1088, 2184)])   # 8, 9 and 17 K-blocks; 9 / 10, 11 and 18 feature tiles
@@ -213,15 +226,26 @@ def test_bf16_logits_and_representations_of_the_last_blocks(lens, gamma, prefill
     t.close()
 
 
-def test_bf16_teacher_forced_pass_beyond_the_forked_rows():
-    """2100 rows keep the projections in the large model's stream and in buffers that other steps share; up to 2048 rows they run
-    beside it.  Both give a position's score within the tolerance that each has against the oracle."""
-    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, layer_map=(1, 3))
+@pytest.mark.parametrize("kw", [dict(layer_map=(1, 3)), dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3))])
+def test_bf16_teacher_forced_pass_beyond_the_forked_rows(kw):
+    """2100 rows in one pass: the projections stay in the large model's stream, before the queries and GELU outputs that share
+    their place, and the output head runs in three parts.  First, middle and last sequence against the checker."""
+    shape = gpu_toy_shape(dtype=synth.DTYPE_BF16, max_pos=200, **kw)
+    w = _bf16_weights(shape, seed=26, std=0.06)
     seqs = prompts_for(shape, [141] * 15, seed=25)
-    t = binding.Tandem(shape, _bf16_weights(shape, seed=26, std=0.06), max_batch=15, max_seq=200, gamma_max=14)
-    whole, _ = t.tandem_teacher_forced_forward(seqs, 14)
+    t = binding.Tandem(shape, w, max_batch=15, max_seq=200, gamma_max=14)
+    nll, top = t.tandem_teacher_forced_forward(seqs, 14)
+    differ = 0
+    for b in (0, 7, 14):
+        logits = O.teacher_forced_tandem_logits(shape, w, seqs[b], 14)
+        want_nll, want_top = O.next_token_scores(logits, seqs[b])
+        assert np.abs(nll[b] - want_nll).max() < 2 * TOL_BF16
+        for i in np.nonzero(top[b] != want_top)[0]:
+            assert np.max(logits[i]) - logits[i][top[b][i]] < 2 * TOL_BF16
+        differ += int((top[b] != want_top).sum())
+    assert differ <= 4
     parts = t.tandem_teacher_forced_forward(seqs[:8], 14)[0] + t.tandem_teacher_forced_forward(seqs[8:], 14)[0]
-    for got, want in zip(whole, parts):
+    for got, want in zip(nll, parts):
         assert np.abs(got - want).max() < 2 * TOL_BF16
     t.close()
 
