@@ -206,9 +206,10 @@ TANDEM_API tandem_status tandem_speculative_generate(tandem_ctx* ctx, int32_t ga
  *   ids: HOST, the sequences concatenated; lens: HOST [batch], each >= 2; max(lens) + gamma <= max_seq and max_pos.
  *   nll:  HOST [sum(lens[b] - 1)], per sequence and position 0 .. len-2 the negative log-likelihood (natural log) of
  *         the true next token under softmax of M_S's logits;  top1: HOST, same shape, M_S's arg-max (nullable).
- * Synchronous.  Replaces the context's sequences (bf16: all given tokens are rows of one pass, or of a few where they are more
- * than max_prefill_rows; fp32: an empty prompt pass and representation-only rounds whose drafts are the given tokens);
- * call tandem_prefill before decoding again. */
+ * Synchronous.  Replaces the context's sequences (bf16: all given tokens that have a next one are rows of one pass, or of a few where
+ * they are more than max_prefill_rows or the work space holds fewer rows; fp32: an empty prompt pass and representation-only rounds
+ * whose drafts are the given tokens); call tandem_prefill before decoding again.  bf16: which kernels a pass takes depends on its
+ * rows, so the last bits of a sequence's scores (1e-6) can depend on the sequences that it is scored with. */
 TANDEM_API tandem_status tandem_teacher_forced_forward(tandem_ctx* ctx, int32_t gamma, int32_t batch, const int32_t* ids,
                                                        const int32_t* lens, float* nll, int32_t* top1);
 

@@ -585,14 +585,21 @@ void launch_tc_decode(tandem_ctx& c, const TcScratch& sc, const void* x, int ldx
     }
 }
 
-// Which kernel a prompt pass's product takes, from estimated times in us.  Both are bound by their operands' way from L2 into the
-// multiprocessors, so the estimates are a start-up time, plus per K-block what a CTA's share of it takes, plus what an epilogue
-// leaves uncovered; fitted to measurements at 64-3000 rows and the widths of the three bf16 pairs, which the choice reproduces but
-// for cases within a tenth of each other.  us measured, split kernel with 1 / 2 / 4 K-slices | pair kernel:
-//    511 x 3072 x 1024         7.8  8.3 16.1 |  8.1       511 x 1024 x 4096, residual  32.1 17.5 11.3 | 17.4
-//   1023 x 1024 x 1024, resid. 17.5 10.3 11.8 |  7.2      1500 x 1024 x 4096, residual  37.3 32.1 27.7 | 20.5
-//   1023 x 4096 x 1024, GELU   12.3 20.0  -   | 16.5       511 x 4096 x 4096, residual  42.4 38.9 33.1 | 20.2
-//    255 x 12288 x 4096        32.3 37.0  -   | 28.3      2047 x 2048 x 2048, residual  40.9 56.1  -   | 18.9
+// Which kernel the product of a prompt or teacher-forced pass takes, from estimated times in us.  Both are bound by their operands' way
+// from L2 into the multiprocessors, so the estimates are a start-up time, plus per K-block what a CTA's share of it takes, plus what an
+// epilogue leaves uncovered.  They are there to choose by: single estimates are off by up to a half (residual adds of many rows), the choice is
+// within a tenth of the best kernel but for a few.  us measured, split kernel with 1 / 2 / 4 K-slices | pair kernel, * the choice:
+//   one plane
+//    511 x 3072 x 1024          7.8*  8.3  16.1 |  8.1       511 x 1024 x 4096, residual  32.1  17.5  11.3* | 17.4
+//   1023 x 1024 x 1024, resid. 17.5  10.3  11.8 |  7.2*     1500 x 1024 x 4096, residual  37.3  32.1  27.7  | 20.5*
+//   1023 x 4096 x 1024, GELU   12.3* 20.0   -   | 16.5       511 x 4096 x 4096, residual  42.4  38.9  33.1  | 20.2*
+//    255 x 12288 x 4096        32.3  37.0   -   | 28.3*     2047 x 2048 x 2048, residual  40.9  56.1   -    | 18.9*
+//   two planes (of 120 sizes, 64-3000 rows of the small and the medium pair, seven are more than a tenth off, the worst ones at the end; kernels one
+//   by one under the profiler, caches warm)
+//    256 x 3072 x 1024         13.7  11.4* 14.0 | 11.4       769 x 1024 x 4096, residual  56.3  33.5  23.4* | 26.8
+//   1500 x 4096 x 1024, GELU   39.3  43.7  69.2 | 31.3*     1023 x 1024 x 1024, residual  28.1  17.6  15.6  | 12.2*
+//   3000 x 8192 x 2048, GELU  183.4 213.7 304.1 | 132.1*     769 x 2048 x 8192, residual 108.1  83.4  67.4  | 56.9*
+//   2047 x 4096 x 1024, GELU   41.9* 57.1  88.4 | 36.2      1500 x 768 x 3072, residual   49.2  28.8  29.6* | 21.8
 struct TiledPlan { bool pair; int slices, whole, parts; };
 TiledPlan tiled_plan(int n_sms, int epi, bool planes, int tiles128, int tiles256, int KB) {
     TiledPlan best = {false, 1, 0, 1};
@@ -768,9 +775,10 @@ void launch_attn_decode_dq(tandem_ctx& c, const AttnArgs& a, int groups, int cl,
     if (pass) {
         AttnArgs w = a;
         w.units = groups * (a.n_heads / gpc);
-        // Up to four warps share a unit's keys as long as all warps run at the same time (two CTAs per multiprocessor): one sequence of 257 tokens
+        // Up to four warps share a unit's keys as long as all warps run at the same time with two CTAs per multiprocessor: one sequence of 257 tokens
         // through the small pair 1226 -> 1165 us with four (1185 with two), of 64 tokens 988 -> 967.  Beyond that the merge only
-        // adds work: eight of 400 tokens 3325 us with one, 3530 with two, 3655 with four.
+        // adds work: eight of 400 tokens 3325 us with one, 3530 with two, 3655 with four.  (128-wide heads with sixteen columns fit once: 400 / 512 rows
+        // of 8 heads a launch 36.1 / 40.0 us with two, 35.9 / 39.5 with four in two rounds, so the line is the same.)
         while (w.log_parts < 2 && w.units * 2 << w.log_parts <= 2 * ATD_WARPS * c.n_sms) ++w.log_parts;
         const dim3 warps(cdiv(w.units << w.log_parts, ATD_WARPS));
         if (narrow) launch_attn_decode_as<DH, 1, ATD_PASS>(c, w, warps, 1); else launch_attn_decode_as<DH, 2, ATD_PASS>(c, w, warps, 1);
@@ -1458,7 +1466,8 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
     bf16 *x = at<bf16>(c, large ? c.lay.fr_x : c.lay.fr_xs), *f = at<bf16>(c, large ? c.lay.fr_f : c.lay.fr_fs), *q = at<bf16>(c, large ? c.lay.fr_q : c.lay.fr_fs);
     bf16 *o = x, *raw = at<bf16>(c, c.lay.fr_raw);
     // Forked, the large model goes on to its FFN when the layer's projections are done, whose buffers lie under the GELU outputs; or when their
-    // input has been read, where the others lie apart (769 rows of the small pair: 1548 -> 1533 us).
+    // input has been read, where the others lie apart.  769 rows of the small pair, projections in the large model's stream 1580 us,
+    // forked until the FFN 1548, apart 1533; 256 rows 1180 and 1135 (the first two).
     auto project = [&](int l, bool forked) {
         int last = 0;
         for (int j = 0; j < c.small.d.n_layers; ++j) if (c.layer_map[j] == l) last = j;
@@ -1496,7 +1505,7 @@ void pass_layers(tandem_ctx& c, const Model& m, float* h, const Rows& r) {
 // are given: a row attends the large-derived keys / values of the positions before its block, and its block's own ones, which lie
 // row by row in a place of their own for the time of one layer.  Activations keep the decode passes' 16 bits (value + remainder planes), the attention
 // is theirs.  Four sequences of 129-257 tokens through the small pair: one round per block, gamma small passes and one large each,
-// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.51 ms like this.
+// 36.1 ms; the decode GEMM over groups of 64 rows 1.95 ms (a group fetches every weight tile again); 1.53 ms like this.
 void forced_pass(tandem_ctx& c, ForcedRows f, bool only, int groups_large, int groups_small, double kv_positions) {
     const Model &L = c.large, &S = c.small;
     Rows r;
