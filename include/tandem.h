@@ -274,7 +274,8 @@ TANDEM_API tandem_status tandem_large_greedy_generate(tandem_ctx* ctx, int32_t m
  *   what = 7  committed counts  int32 [batch]
  * After a representation-only iteration item 2 holds [batch][gamma] rows (then rows of earlier passes), item 0 is an earlier verify pass's.
  * After tandem_teacher_forced_forward items 1 and 2 hold the same of a last round: in a bf16 context every sequence's own last
- * block (zeros past the sequence's end), in an fp32 context the last round of the whole batch.
+ * block (zeros past the sequence's end), in an fp32 context the last round of the whole batch; and items 3-7 every sequence as far as
+ * its own length (bf16), or as the longest one of the batch, filled up with token 0 (fp32).
  * bytes must equal the size of the selected item. */
 TANDEM_API tandem_status tandem_debug_read(tandem_ctx* ctx, int32_t what, int32_t layer, int32_t seq,
                                 void* host_dst, size_t bytes);

@@ -166,6 +166,8 @@ def test_decode_attention_by_lone_ctas(batch, heads, dh, derived, own):
     ([2, 140, 23], 4, 0, dict(layer_map=(1, 3), vocab=129)),                     # one pass of 162 rows, last blocks of one to three; a head tile of one feature
     ([131, 7, 66], 3, 20, dict(layer_map=(0, 2))),                               # passes of at most 20 rows, whole blocks: a sequence over many of them
     ([190, 180], 4, 0, dict(large=(2, 128, 2, 2048), layer_map=(0, 2), max_pos=200)),   # a work space that holds fewer rows than a prompt pass's
+    ([130], 4, 130, dict(layer_map=(0, 2))),                                     # so few rows that the projections' results lie apart from the GELU outputs
+    ([128], 5, 130, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(1, 1))),   # ... and two small layers read the same representations
     ([47], 15, 0, dict(large=(2, 256, 2, 264), small=(1, 256, 2, 136), kv_heads=(1, 1), layer_map=(2,))),   # blocks of 15, 128-wide heads, shared keys / values
     ([66, 2], 1, 0, dict(kind=synth.FF_TANDEM_MLP, hidden=40, layer_map=(0, 3), small=(2, 192, 6, 136))),  # 66 blocks of one row; a small model wider than the large one
     ([141], 1, 0, dict(layer_map=(0, 3), small=(2, 192, 6, 136))),               # 840 block heads: two warps share the keys of each (four up to 592)
@@ -205,6 +207,7 @@ def test_bf16_logits_and_representations_of_the_last_blocks(lens, gamma, prefill
     t.tandem_teacher_forced_forward(seqs, gamma)
     logits = t.tandem_debug_read(binding.READ_SMALL_LOGITS, gamma)
     hidden = t.tandem_debug_read(binding.READ_LARGE_HIDDEN, gamma).reshape(-1, shape.large.d_model)
+    assert t.tandem_debug_read(binding.READ_COMMITTED).tolist() == lens
     for b, ids in enumerate(seqs):
         o = O.TandemOracle(shape, w)
         reps, _ = O.large_block_pass(o.large, o.large_cache, ids, 0)
@@ -213,6 +216,9 @@ def test_bf16_logits_and_representations_of_the_last_blocks(lens, gamma, prefill
         for p in range(first, len(ids) - 1):
             assert np.abs(logits[p - first, b] - want[p]).max() < TOL_BF16
             assert np.abs(hidden[b * gamma + p - first] - reps[-1][p]).max() < 2 * TOL_BF16
+        keys = t.tandem_debug_read(binding.READ_LARGE_K, layer=1, seq=b)
+        want = np.stack(o.large_cache.k[1][:len(ids) - 1]).reshape(len(ids) - 1, -1)
+        assert (np.abs(keys - want) < 2 * TOL_BF16 * np.maximum(1, np.abs(want))).all()
         past = (len(ids) - 2) % gamma + 1
         assert not logits[past:, b].any() and not hidden[b * gamma + past:(b + 1) * gamma].any()
     t.tandem_prefill([s[:3] for s in seqs])       # and a decode iteration's own again
